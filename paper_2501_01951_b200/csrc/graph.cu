@@ -142,25 +142,25 @@ __global__ void schedule_keys_kernel(int64_t row0, int64_t n_rows, const int64_t
     keys[i] = ((0x7FFFFFFFull - d) << 32) | (uint64_t)u;  // descending entries, ascending id
 }
 
-// perm from the sorted keys; counts[0] = rows longer than SPMM_SEG, counts[1..3] = rows longer than
-// SPMM_PACK_DEG[0..2] (one atomic per warp and counter; integers, so order does not matter).
+// perm from the sorted keys; counts[0] = rows longer than seg, counts[1..3] = rows longer than SPMM_PACK_DEG[0..2],
+// counts[4] = rows longer than SPMM_HEAVY (one atomic per warp and counter; integers, so order does not matter).
 __global__ void schedule_finish_kernel(int64_t n, const uint64_t* __restrict__ keys, int32_t* __restrict__ perm,
-                                       unsigned long long* counts) {
+                                       int seg, unsigned long long* counts) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int64_t d = -1;
     if (i < n) {
         perm[i] = (int32_t)(uint32_t)(keys[i] & 0xFFFFFFFFull);
         d = (int64_t)(0x7FFFFFFFull - (keys[i] >> 32));
     }
-    const int thr[4] = {SPMM_SEG, SPMM_PACK_DEG[0], SPMM_PACK_DEG[1], SPMM_PACK_DEG[2]};
+    const int thr[5] = {seg, SPMM_PACK_DEG[0], SPMM_PACK_DEG[1], SPMM_PACK_DEG[2], SPMM_HEAVY};
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < 5; ++q) {
         unsigned b = __ballot_sync(0xFFFFFFFFu, d > thr[q]);
         if ((threadIdx.x & 31) == 0 && b) atomicAdd(counts + q, (unsigned long long)__popc(b));
     }
 }
 
-// Long rows are cut at dyadic column-block boundaries (and every SPMM_SEG entries): a row with d
+// Long rows are cut at dyadic column-block boundaries (and every seg entries): a row with d
 // entries uses 2^k blocks, the largest k <= SPMM_MAX_LOG_BLOCKS with d / 2^k >= SPMM_BLK_MIN_ENTRIES.
 __device__ __forceinline__ int row_log_blocks(int64_t d) {
     int k = 0;
@@ -200,7 +200,7 @@ __device__ __forceinline__ int64_t owner_of(const int64_t* __restrict__ off, int
 __global__ void pair_segments_kernel(int64_t n, int64_t n_long, int64_t total_pairs, const int32_t* __restrict__ perm,
                                      const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
                                      const int64_t* __restrict__ blk_off, int64_t* __restrict__ pair_lo,
-                                     int64_t* __restrict__ pair_cnt, int64_t* __restrict__ pair_segs) {
+                                     int64_t* __restrict__ pair_cnt, int64_t* __restrict__ pair_segs, int seg) {
     int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t > total_pairs) return;
     if (t == total_pairs) { pair_segs[t] = 0; return; }
@@ -213,14 +213,14 @@ __global__ void pair_segments_kernel(int64_t n, int64_t n_long, int64_t total_pa
     const int64_t hi = lower_bound_col(col, lo, re, (b + 1) * width);
     pair_lo[t] = lo;
     pair_cnt[t] = hi - lo;
-    pair_segs[t] = (hi - lo + SPMM_SEG - 1) / SPMM_SEG;
+    pair_segs[t] = (hi - lo + seg - 1) / seg;
 }
 
 __global__ void seg_fill_kernel(int64_t n_long, int64_t total_pairs, const int32_t* __restrict__ col,
                                 const int64_t* __restrict__ blk_off, const int64_t* __restrict__ pair_lo,
                                 const int64_t* __restrict__ pair_cnt, const int64_t* __restrict__ pair_seg_off,
                                 SpmmRec* __restrict__ rec_tmp, uint32_t* __restrict__ keys, uint32_t* __restrict__ ids,
-                                int64_t* __restrict__ seg_off) {
+                                int64_t* __restrict__ seg_off, int seg) {
     int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= total_pairs) return;
     const int64_t i = owner_of(blk_off, n_long, t);
@@ -228,8 +228,8 @@ __global__ void seg_fill_kernel(int64_t n_long, int64_t total_pairs, const int32
     if (t == total_pairs - 1) seg_off[n_long] = pair_seg_off[total_pairs];
     int64_t q = pair_seg_off[t];
     const int64_t lo = pair_lo[t], hi = lo + pair_cnt[t];
-    for (int64_t pos = lo; pos < hi; pos += SPMM_SEG, ++q) {
-        SpmmRec x; x.begin = pos; x.len = (int32_t)((hi - pos) < SPMM_SEG ? (hi - pos) : SPMM_SEG); x.row = (int32_t)i;
+    for (int64_t pos = lo; pos < hi; pos += seg, ++q) {
+        SpmmRec x; x.begin = pos; x.len = (int32_t)((hi - pos) < seg ? (hi - pos) : seg); x.row = (int32_t)i;
         rec_tmp[q] = x;
         keys[q] = (uint32_t)col[pos];      // segments run in order of their first column
         ids[q] = (uint32_t)q;
@@ -290,30 +290,32 @@ void free_view(CsrView& v) {
     v = CsrView{};
 }
 
-// Schedule of rows [row0, row0 + n) of the CSR (rowptr, col) of a matrix with n_total columns.
-mixgcn_status build_schedule(int64_t n_total, const int64_t* rowptr, const int32_t* col, int64_t row0, int64_t n,
+// Schedule of rows [row0, row0 + n) of the CSR (rowptr, col) of a matrix with n_total columns and nnz entries in all
+// rows (a row chunk is cut like the whole matrix, so that its sums are the same).
+mixgcn_status build_schedule(int64_t n_total, int64_t nnz, const int64_t* rowptr, const int32_t* col, int64_t row0, int64_t n,
                              SpmmSchedule& v, cudaStream_t s) {
     v = SpmmSchedule{};
-    v.row0 = row0; v.n_rows = n;
+    v.row0 = row0; v.n_rows = n; v.seg = schedule_seg(nnz);
     if (n <= 0) return MIXGCN_OK;
     DevBuf k0, k1, tmp, hub;
     MIXGCN_CUDA(cudaMalloc(&k0.p, n * sizeof(uint64_t)));
     MIXGCN_CUDA(cudaMalloc(&k1.p, n * sizeof(uint64_t)));
-    MIXGCN_CUDA(cudaMalloc(&hub.p, 4 * sizeof(unsigned long long)));
-    MIXGCN_CUDA(cudaMemsetAsync(hub.p, 0, 4 * sizeof(unsigned long long), s));
+    MIXGCN_CUDA(cudaMalloc(&hub.p, 5 * sizeof(unsigned long long)));
+    MIXGCN_CUDA(cudaMemsetAsync(hub.p, 0, 5 * sizeof(unsigned long long), s));
     MIXGCN_CUDA(cudaMalloc((void**)&v.perm, n * sizeof(int32_t)));
     schedule_keys_kernel<<<blocks_for(n), TPB, 0, s>>>(row0, n, rowptr, k0.as<uint64_t>());
     size_t tb = 0;
     MIXGCN_CUDA(cub::DeviceRadixSort::SortKeys(nullptr, tb, k0.as<uint64_t>(), k1.as<uint64_t>(), n, 0, 64, s));
     MIXGCN_CUDA(cudaMalloc(&tmp.p, tb ? tb : 1));
     MIXGCN_CUDA(cub::DeviceRadixSort::SortKeys(tmp.p, tb, k0.as<uint64_t>(), k1.as<uint64_t>(), n, 0, 64, s));
-    schedule_finish_kernel<<<blocks_for(n), TPB, 0, s>>>(n, k1.as<uint64_t>(), v.perm, hub.as<unsigned long long>());
-    unsigned long long h[4] = {0, 0, 0, 0};
+    schedule_finish_kernel<<<blocks_for(n), TPB, 0, s>>>(n, k1.as<uint64_t>(), v.perm, v.seg, hub.as<unsigned long long>());
+    unsigned long long h[5] = {0, 0, 0, 0, 0};
     uint64_t first = 0;
     MIXGCN_CUDA(cudaMemcpyAsync(h, hub.p, sizeof(h), cudaMemcpyDeviceToHost, s));
     MIXGCN_CUDA(cudaMemcpyAsync(&first, k1.p, sizeof(first), cudaMemcpyDeviceToHost, s));
     MIXGCN_CUDA(cudaStreamSynchronize(s));
     v.n_long = (int64_t)h[0];
+    v.n_heavy = (int64_t)h[4];
     for (int q = 0; q < 3; ++q) v.rows_above[q] = (int64_t)h[q + 1];
     v.max_deg = (int32_t)(0x7FFFFFFFull - (first >> 32));
     // long rows -> (row, column block) pairs -> segments, ordered by their first column
@@ -340,7 +342,7 @@ mixgcn_status build_schedule(int64_t n_total, const int64_t* rowptr, const int32
         MIXGCN_CUDA(cudaMalloc(&pair_seg_off.p, (total_pairs + 1) * sizeof(int64_t)));
         pair_segments_kernel<<<blocks_for(total_pairs + 1), TPB, 0, s>>>(n_total, nl, total_pairs, v.perm, rowptr, col,
                                                                         blk_off.as<int64_t>(), pair_lo.as<int64_t>(),
-                                                                        pair_cnt.as<int64_t>(), pair_segs.as<int64_t>());
+                                                                        pair_cnt.as<int64_t>(), pair_segs.as<int64_t>(), v.seg);
         size_t tb3 = 0;
         MIXGCN_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tb3, pair_segs.as<int64_t>(), pair_seg_off.as<int64_t>(), total_pairs + 1, s));
         MIXGCN_CUDA(cudaMalloc(&tmp3.p, tb3 ? tb3 : 1));
@@ -361,7 +363,7 @@ mixgcn_status build_schedule(int64_t n_total, const int64_t* rowptr, const int32
         seg_fill_kernel<<<blocks_for(total_pairs), TPB, 0, s>>>(nl, total_pairs, col, blk_off.as<int64_t>(), pair_lo.as<int64_t>(),
                                                                pair_cnt.as<int64_t>(), pair_seg_off.as<int64_t>(),
                                                                rec_tmp.as<SpmmRec>(), keys0.as<uint32_t>(), ids0.as<uint32_t>(),
-                                                               v.seg_off);
+                                                               v.seg_off, v.seg);
         size_t tb4 = 0;
         MIXGCN_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, tb4, keys0.as<uint32_t>(), keys1.as<uint32_t>(), ids0.as<uint32_t>(),
                                                     ids1.as<uint32_t>(), total, 0, 32, s));
@@ -403,7 +405,7 @@ mixgcn_status finish_graph(mixgcn_graph* g, cudaStream_t s) {
         MIXGCN_CUDA(cudaStreamSynchronize(s));
         g->has_diagonal = hd == (unsigned long long)n ? 1 : (hd == 0 ? 0 : 2);
     }
-    MIXGCN_TRY(build_schedule(n, A.rowptr, A.col, 0, n, A.full, s));
+    MIXGCN_TRY(build_schedule(n, nnz, A.rowptr, A.col, 0, n, A.full, s));
     g->bwd_is_fwd = (g->symmetric && g->norm != 1) ? 1 : 0;   // row-mean values are not symmetric: A_hat^T needs its own copy
     if (g->bwd_is_fwd) {
         g->bwd = A;  // alias: the same index serves the backward aggregation
@@ -428,7 +430,7 @@ mixgcn_status finish_graph(mixgcn_graph* g, cudaStream_t s) {
                                                 nnz, 0, end_bit, s));
     rowptr_from_keys_kernel<<<blocks_for(nnz + 1), TPB, 0, s>>>(n, nnz, k1.as<uint64_t>(), T.rowptr, T.col);
     MIXGCN_CUDA(cudaStreamSynchronize(s));
-    MIXGCN_TRY(build_schedule(n, T.rowptr, T.col, 0, n, T.full, s));
+    MIXGCN_TRY(build_schedule(n, nnz, T.rowptr, T.col, 0, n, T.full, s));
     return MIXGCN_OK;
 }
 
@@ -443,8 +445,8 @@ mixgcn_status check_common(mixgcn_ctx* ctx, int64_t n, mixgcn_graph** out) {
 
 namespace mixgcn {
 
-mixgcn_status build_view_schedule(int64_t n_cols, int64_t n, CsrView& v, cudaStream_t s) {
-    return build_schedule(n_cols, v.rowptr, v.col, 0, n, v.full, s);
+mixgcn_status build_view_schedule(int64_t n_cols, int64_t n, int64_t nnz, CsrView& v, cudaStream_t s) {
+    return build_schedule(n_cols, nnz, v.rowptr, v.col, 0, n, v.full, s);
 }
 
 void release_view(CsrView& v) { free_view(v); }
@@ -462,7 +464,7 @@ mixgcn_status ensure_chunk_schedules(const mixgcn_graph* g, const CsrView& A_con
     cudaStream_t s = g->ctx->side_stream[0];
     for (int k = 0; k < chunks; ++k) {
         const int64_t r0 = (g->n * (int64_t)k) / chunks, r1 = (g->n * (int64_t)(k + 1)) / chunks;
-        mixgcn_status st = build_schedule(g->n, A.rowptr, A.col, r0, r1 - r0, sc[k], s);
+        mixgcn_status st = build_schedule(g->n, g->nnz, A.rowptr, A.col, r0, r1 - r0, sc[k], s);
         if (st != MIXGCN_OK) {
             for (int q = 0; q <= k; ++q) free_schedule(sc[q]);
             delete[] sc;

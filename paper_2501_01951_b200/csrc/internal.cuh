@@ -116,8 +116,8 @@ struct __align__(16) SpmmRec {
 };
 
 // Aggregation schedule of the rows [row0, row0 + n_rows) of one CSR orientation.
-// Rows longer than SPMM_SEG entries are cut into segments at dyadic column-block boundaries and
-// every SPMM_SEG entries; the segment records [0, total_segs) run in order of their first column, so
+// Rows longer than `seg` entries are cut into segments at dyadic column-block boundaries and
+// every `seg` entries; the segment records [0, total_segs) run in order of their first column, so
 // that segments of different long rows that gather the same rows of Y run close in time (those rows
 // are then served by the L2).  Every other row is one record, in perm order (records
 // [total_segs, total_segs + n_rows - n_long)).
@@ -125,8 +125,10 @@ struct SpmmSchedule {
     int64_t row0, n_rows;
     int32_t* perm;             // [n_rows] row ids by descending entry count (ties by ascending id)
     int32_t max_deg;
+    int32_t seg;               // segment length, see schedule_seg
     SpmmRec* rec;
     int64_t n_long, total_segs;
+    int64_t n_heavy;           // of the long rows, those with more than SPMM_HEAVY entries (the first ones)
     int64_t* seg_off;          // [n_long+1] segments of long row i are numbered seg_off[i] .. seg_off[i+1]-1 in entry order
     int64_t* seg_pos;          // [total_segs] record position (= partial-row slot) of segment number q
     int64_t rows_above[3];     // rows with more than SPMM_PACK_DEG[i] entries (bucket boundaries in perm order)
@@ -173,7 +175,17 @@ struct mixgcn_rowplan {
 
 namespace mixgcn {
 
-constexpr int SPMM_SEG = 512;               // rows longer than this are cut into segments of at most this many entries
+// Rows longer than a schedule's segment length are cut into segments of at most that many entries.  512 where the graph
+// has enough entries to keep the machine's ~4,700 resident warps busy with several such units each (the partial rows then
+// cost least: 256..1024 measured within 2 % on large graphs); shorter on small graphs, where the length of one unit's
+// serial walk is the length of the launch (70 K entries, width 64: 27 us with 512, 4 us with 64).
+constexpr int SPMM_SEG_MAX = 512, SPMM_SEG_MIN = 64;
+inline int32_t schedule_seg(int64_t nnz) {
+    int32_t seg = SPMM_SEG_MAX;
+    while (seg > SPMM_SEG_MIN && (int64_t)seg * 4 * 4736 > nnz) seg >>= 1;
+    return seg;
+}
+constexpr int SPMM_HEAVY = 2048;            // long rows above this take a block each when their segments are combined
 constexpr int SPMM_BLK_MIN_ENTRIES = 64;    // a long row uses 2^k column blocks while it keeps >= this many entries per block
 constexpr int SPMM_MAX_LOG_BLOCKS = 8;      // at most 2^this column blocks per row
 constexpr int SPMM_PACK_DEG[3] = {12, 5, 2};   // rows up to these lengths share a warp 2-, 4-, 8-fold
@@ -238,7 +250,7 @@ mixgcn_status launch_spmm(mixgcn_ctx* ctx, const mixgcn_graph* g, const CsrView&
                           int32_t w, const float* Y, int64_t ldy, float* Z, int64_t ldz,
                           const mixgcn_epilogue* epi, cudaStream_t s, const SpmmOpts& opts = SpmmOpts());
 // schedule of all n rows of a view whose column ids lie in [0, n_cols); release of a view's memory
-mixgcn_status build_view_schedule(int64_t n_cols, int64_t n, CsrView& v, cudaStream_t s);
+mixgcn_status build_view_schedule(int64_t n_cols, int64_t n, int64_t nnz, CsrView& v, cudaStream_t s);
 void release_view(CsrView& v);
 // colsum_b of launch_gemm (weight-gradient form, trans_a = 1, only): also out[n] = sum_k B[k][n], the bias
 // gradient when B = dP -- produced inside the product's kernel where that kernel reads B as fp32 words,

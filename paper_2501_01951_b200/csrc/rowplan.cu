@@ -156,7 +156,7 @@ extern "C" mixgcn_status mixgcn_rowplan_create(mixgcn_ctx* ctx, const mixgcn_gra
     if (n > 0 && nnz2 > 0)
         kept_fill_kernel<<<row_blocks, 256, 0, s>>>(n, A.rowptr, A.col, A.val, in_row_mask, pos.as<int32_t>(), V.rowptr, V.col, V.val);
     MIXGCN_CUDA(cudaGetLastError());
-    MIXGCN_TRY(build_view_schedule(in_count > 0 ? in_count : 1, n, V, s));
+    MIXGCN_TRY(build_view_schedule(in_count > 0 ? in_count : 1, n, nnz2, V, s));
     MIXGCN_CUDA(cudaStreamSynchronize(s));
     guard.p = nullptr;
     *out = p;

@@ -11,13 +11,20 @@
 //    the FMAs, with a predicated tail instead of a one-by-one remainder.
 //  - Degree buckets: rows of up to 12 / 5 / 2 entries share a warp 2- / 4- / 8-fold (fewer lanes per
 //    row, more float4 per lane), so short rows still keep eight loads per lane in flight.
-//  - Rows longer than SPMM_SEG entries are cut (at column-block boundaries and every SPMM_SEG
-//    entries) into segments that run as independent units, in order of their first column, and
-//    write partial rows to scratch: hub rows that gather the same rows of Y do so close in time
-//    and share them through the L2.  A second kernel adds the segments of each row in entry order
-//    and applies the epilogue.  Every sum has a fixed order: the result is bit-reproducible.
+//  - Narrow aggregations (up to 64 columns) have too few column lanes to keep a long unit's loads in
+//    flight: there a whole warp takes one unit of more than 12 entries, its lane groups take every EG-th
+//    entry, and a butterfly adds the groups' sums (spmm_warp_kernel).
+//  - Rows longer than the schedule's segment length (64..512 entries, shorter for small graphs) are cut (at
+//    column-block boundaries and at that length) into segments that run as independent units, in order of
+//    their first column, and write partial rows to scratch: hub rows that gather the same rows of Y do so
+//    close in time and share them through the L2.  A last kernel adds the segments of each row in a fixed
+//    order and applies the epilogue.  Every sum has a fixed order: the result is bit-reproducible.
+//  - The launches of one call overlap: each releases its successor as soon as its own blocks are all
+//    running (programmatic dependent launch), so a bucket's last wave shares the machine with the next bucket.
 //  - The epilogue (bias, ReLU, dropout mask, gate by another tensor's sign) is applied in
 //    registers before the single write of Z.
+#include <type_traits>
+
 #include "internal.cuh"
 
 using namespace mixgcn;
@@ -271,14 +278,50 @@ struct Cfg {
     static constexpr int U = U0 > LPR ? LPR : U0;   // gathered rows in flight per lane group
 };
 
+// Programmatic dependent launch.  The launches of one aggregation call are independent of each other but for the
+// combination of the segments: every kernel lets its successor start at once (trigger), and before it ends it waits
+// for its predecessor's completion (wait), so that "the last launch has completed" still means that all of them have.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Accumulate entries [b, e) into acc[] for the lane's column groups, ascending entry order.
 // The (col, val) pair of the NEXT batch of LPR entries is requested before the current batch's gathers,
 // so that the index load's latency is hidden behind them instead of preceding every batch.
 template <int LPR, int VPL, bool FULL = false>     // FULL: the slice has exactly LPR * VPL column groups (no lane is idle)
 __device__ __forceinline__ void row_segment(const SpmmParams& p, int64_t b, int64_t e, int lig, unsigned mask,
                                             int w4, float4 (&acc)[VPL], unsigned keep = 0xFFFFFFFFu) {
-    constexpr int U = Cfg<LPR, VPL>::U;
     const float* Yb = p.Y + p.j0;
+    if constexpr (LPR <= 2) {
+        // too few lanes to hold a batch of (col, val) pairs: every lane reads them itself (its group reads one address)
+        constexpr int U = VPL <= 2 ? 4 : 2;
+        for (int64_t i0 = b; i0 < e; i0 += U) {
+            int ck[U]; float ak[U]; float4 y[U][VPL];
+#pragma unroll
+            for (int t = 0; t < U; ++t) {
+                const bool in = i0 + t < e;
+                ck[t] = in ? __ldg(p.col + i0 + t) : 0;
+                ak[t] = in ? __ldg(p.val + i0 + t) : 0.0f;
+            }
+#pragma unroll
+            for (int t = 0; t < U; ++t) {
+                const float4* yr = reinterpret_cast<const float4*>(Yb + (int64_t)ck[t] * p.ldy);
+                const bool live = i0 + t < e && index_ok(ck[t], p.y_rows, p.status, SITE_SPMM_COL);
+#pragma unroll
+                for (int v = 0; v < VPL; ++v) {
+                    const int c4 = lig + v * LPR;
+                    y[t][v] = (live && (FULL || c4 < w4) && ((keep >> v) & 1u)) ? __ldg(yr + c4) : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < U; ++t)
+                if (i0 + t < e) {
+#pragma unroll
+                    for (int v = 0; v < VPL; ++v) fma4(acc[v], ak[t], y[t][v]);
+                }
+        }
+        return;
+    }
+    constexpr int U = Cfg<LPR, VPL>::U;
     int c = 0; float a = 0.0f;
     if (b + lig < e) { c = __ldg(p.col + b + lig); a = __ldg(p.val + b + lig); }
     for (int64_t i0 = b; i0 < e; i0 += LPR) {
@@ -313,10 +356,84 @@ __device__ __forceinline__ void row_segment(const SpmmParams& p, int64_t b, int6
     }
 }
 
+// The same for a whole warp on one unit of a narrow aggregation: EG = 32 / CL lane groups take entries g, g + EG, ...
+// (each lane reads its group's column id and value itself, the next step's ahead of this step's gathers; consecutive
+// groups read consecutive entries), then a butterfly over the groups leaves the complete sums in every lane.  The
+// serial chain of a unit is EG times shorter than with one group per unit, which is what bounded narrow and small
+// aggregations: 4,096 nodes / 70 K entries, widths 64 and 8: 60 -> 5 us for the slowest launch.
+template <int CL, int VPL>
+__device__ __forceinline__ void warp_segment(const SpmmParams& p, int64_t b, int len, int lane, int w4, float4 (&acc)[VPL],
+                                             unsigned keep = 0xFFFFFFFFu) {
+    constexpr int EG = 32 / CL, U = VPL == 1 ? 4 : 2;
+    const int cl = lane & (CL - 1), eg = lane / CL;
+    const float* Yb = p.Y + p.j0;
+    const int32_t* col = p.col + b;
+    const float* val = p.val + b;
+    int c[U]; float a[U];
+#pragma unroll
+    for (int t = 0; t < U; ++t) {
+        const int i = t * EG + eg;
+        c[t] = i < len ? __ldg(col + i) : 0;
+        a[t] = i < len ? __ldg(val + i) : 0.0f;
+    }
+    for (int i0 = 0; i0 < len; i0 += EG * U) {
+        int cn[U]; float an[U]; float4 y[U][VPL];
+#pragma unroll
+        for (int t = 0; t < U; ++t) {
+            const int i = i0 + EG * U + t * EG + eg;
+            cn[t] = i < len ? __ldg(col + i) : 0;
+            an[t] = i < len ? __ldg(val + i) : 0.0f;
+        }
+#pragma unroll
+        for (int t = 0; t < U; ++t) {
+            const float4* yr = reinterpret_cast<const float4*>(Yb + (int64_t)c[t] * p.ldy);
+            const bool live = i0 + t * EG + eg < len && index_ok(c[t], p.y_rows, p.status, SITE_SPMM_COL);
+#pragma unroll
+            for (int v = 0; v < VPL; ++v) {
+                const int c4 = cl + v * CL;
+                y[t][v] = (live && c4 < w4 && ((keep >> v) & 1u)) ? __ldg(yr + c4) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < U; ++t)
+            if (i0 + t * EG + eg < len) {
+#pragma unroll
+                for (int v = 0; v < VPL; ++v) fma4(acc[v], a[t], y[t][v]);
+            }
+#pragma unroll
+        for (int t = 0; t < U; ++t) { c[t] = cn[t]; a[t] = an[t]; }
+    }
+#pragma unroll
+    for (int o = CL; o < 32; o <<= 1)
+#pragma unroll
+        for (int v = 0; v < VPL; ++v) {
+            acc[v].x += __shfl_xor_sync(0xFFFFFFFFu, acc[v].x, o); acc[v].y += __shfl_xor_sync(0xFFFFFFFFu, acc[v].y, o);
+            acc[v].z += __shfl_xor_sync(0xFFFFFFFFu, acc[v].z, o); acc[v].w += __shfl_xor_sync(0xFFFFFFFFu, acc[v].w, o);
+        }
+}
+
+// Which of a lane's column groups the output mask of a sampled aggregation keeps (Eq. 4: outputs the mask drops are
+// never computed -- a lane whose four columns of this row are all masked skips its gathers of every neighbour).
+template <int LPR, int VPL>
+__device__ __forceinline__ unsigned kept_groups(const SpmmParams& p, int64_t u, int lig, int w4) {
+    const int64_t row = p.seg_perm ? __ldg(p.seg_perm + u) : u;
+    unsigned keep = 0u;
+#pragma unroll
+    for (int v = 0; v < VPL; ++v) {
+        const int c4 = lig + v * LPR;
+        if (c4 < w4) {
+            const int j = p.j0 + c4 * 4;
+            if ((__ldg(p.out_bits + row * p.ld_bits + (j >> 5)) >> (j & 31)) & 0xFu) keep |= 1u << v;
+        }
+    }
+    return keep;
+}
+
 // FULL (plain and bit-gate instances): the slice has exactly LPR * VPL column groups, so no load is predicated on its column.
 template <int LPR, int VPL, int EPI = EPI_ANY, bool FULL = false>
 __global__ void __launch_bounds__(256, VPL <= 2 ? SPMM_MINB : 1) spmm_group_kernel(const SpmmParams p) {
     constexpr bool LOSS = EPI == EPI_LOSS, PLAIN = epi_is_lean(EPI);
+    pdl_trigger();
     const int lig = threadIdx.x % LPR;
     const int64_t idx = p.idx_begin + ((int64_t)blockIdx.x * 256 + threadIdx.x) / LPR;
     if (idx >= p.idx_end) return;  // the whole group leaves together
@@ -338,20 +455,7 @@ __global__ void __launch_bounds__(256, VPL <= 2 ? SPMM_MINB : 1) spmm_group_kern
 #pragma unroll
     for (int v = 0; v < VPL; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
     unsigned keep = 0xFFFFFFFFu;
-    if (!PLAIN && p.out_bits && p.bits_skip) {
-        // Eq. 4: outputs the mask drops are never computed -- a lane whose four columns of this row are all
-        // masked skips its gathers of every neighbour (the mask is known before the aggregation)
-        const int64_t row = p.seg_perm ? __ldg(p.seg_perm + u) : u;
-        keep = 0u;
-#pragma unroll
-        for (int v = 0; v < VPL; ++v) {
-            const int c4 = lig + v * LPR;
-            if (c4 < w4) {
-                const int j = p.j0 + c4 * 4;
-                if ((__ldg(p.out_bits + row * p.ld_bits + (j >> 5)) >> (j & 31)) & 0xFu) keep |= 1u << v;
-            }
-        }
-    }
+    if (!PLAIN && p.out_bits && p.bits_skip) keep = kept_groups<LPR, VPL>(p, u, lig, w4);
     row_segment<LPR, VPL, FULL>(p, b, e, lig, mask, w4, acc, keep);
     if (p.partial) {
         float4* dst = reinterpret_cast<float4*>(p.partial + idx * p.ldp);
@@ -360,9 +464,7 @@ __global__ void __launch_bounds__(256, VPL <= 2 ? SPMM_MINB : 1) spmm_group_kern
             const int c4 = lig + v * LPR;
             if (c4 < w4) dst[c4] = acc[v];
         }
-        return;
-    }
-    if constexpr (LOSS) {
+    } else if constexpr (LOSS) {
         loss_epilogue<LPR, VPL>(p, u, lig, mask, acc);
     } else {
 #pragma unroll
@@ -374,6 +476,45 @@ __global__ void __launch_bounds__(256, VPL <= 2 ? SPMM_MINB : 1) spmm_group_kern
             }
         }
     }
+    pdl_wait();
+}
+
+// Units of more than 12 entries (and every segment) of an aggregation of at most 64 columns: one warp per unit.
+template <int CL, int VPL, int EPI = EPI_ANY>
+__global__ void __launch_bounds__(256, SPMM_MINB) spmm_warp_kernel(const SpmmParams p) {
+    pdl_trigger();
+    const int lane = threadIdx.x & 31;
+    const int64_t idx = p.idx_begin + (((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5);
+    if (idx >= p.idx_end) return;
+    const int4 r = __ldg(reinterpret_cast<const int4*>(p.rec + idx));
+    const int64_t b = ((int64_t)(uint32_t)r.y << 32) | (uint32_t)r.x, u = r.w;
+    if (!unit_ok(p, b, b + r.z, u)) return;
+    const int w4 = (p.w + 3) >> 2, cl = lane & (CL - 1);
+    float4 acc[VPL];
+#pragma unroll
+    for (int v = 0; v < VPL; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+    unsigned keep = 0xFFFFFFFFu;
+    if (EPI == EPI_ANY && p.out_bits && p.bits_skip) keep = kept_groups<CL, VPL>(p, u, cl, w4);
+    warp_segment<CL, VPL>(p, b, r.z, lane, w4, acc, keep);
+    if (lane < CL) {
+#pragma unroll
+        for (int v = 0; v < VPL; ++v) {
+            const int c4 = cl + v * CL;
+            if constexpr (EPI != EPI_LOSS) {
+                if (c4 < w4) {
+                    if (p.partial) reinterpret_cast<float4*>(p.partial + idx * p.ldp)[c4] = acc[v];
+                    else if constexpr (epi_is_lean(EPI)) store_lean<EPI>(p, u, c4, acc[v]);
+                    else store_row(p, u, c4, acc[v]);
+                }
+            } else if (p.partial && c4 < w4) {
+                reinterpret_cast<float4*>(p.partial + idx * p.ldp)[c4] = acc[v];
+            }
+        }
+        if constexpr (EPI == EPI_LOSS) {
+            if (!p.partial) loss_epilogue<CL, VPL>(p, u, cl, CL == 32 ? 0xFFFFFFFFu : (1u << (CL & 31)) - 1u, acc);
+        }
+    }
+    pdl_wait();
 }
 
 // Rows of at most MAXE entries, width <= 128: a warp takes RB schedule records at once.  Lanes read the
@@ -383,6 +524,7 @@ __global__ void __launch_bounds__(256, VPL <= 2 ? SPMM_MINB : 1) spmm_group_kern
 template <int RB, int MAXE, int EPI = EPI_ANY, int VPL = 1>      // VPL float4 per lane: widths up to 128 * VPL
 __global__ void __launch_bounds__(256, VPL == 1 ? SPMM_SHORT_MINB : SPMM_MINB) spmm_short_kernel(const SpmmParams p) {
     static_assert(RB * MAXE <= 32, "one lane per (row, entry)");
+    pdl_trigger();
     const int lane = threadIdx.x & 31;
     const int64_t idx0 = p.idx_begin + (((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5) * RB;
     if (idx0 >= p.idx_end) return;
@@ -445,6 +587,7 @@ __global__ void __launch_bounds__(256, VPL == 1 ? SPMM_SHORT_MINB : SPMM_MINB) s
             }
         }
     }
+    pdl_wait();
 }
 
 // Row-sparse input: most rows of Y are exactly zero (gradients of a masked loss and what they
@@ -576,56 +719,170 @@ __global__ void __launch_bounds__(256) spmm_filtered_kernel(const SpmmParams p) 
     }
 }
 
-// Long rows: add the segments' partial rows in entry order, apply the epilogue, write Z.
-// One group of 32 lanes per long row.
+// The same for narrow aggregations: entry order and lane split of the dense path (one group of CL lanes walks a row
+// of at most 12 entries, the whole warp shares a longer unit), so the rows are again bitwise those of the full call.
+template <int CL, int VPL>
+__global__ void __launch_bounds__(256) spmm_filtered_narrow_kernel(const SpmmParams p) {
+    constexpr int PACKED = SPMM_PACK_DEG[0];
+    const int lane = threadIdx.x & 31, cl = lane & (CL - 1);
+    const int64_t idx0 = p.idx_begin + ((((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5) << 5);
+    if (idx0 >= p.idx_end) return;
+    int4 rc = make_int4(0, 0, 0, 0);
+    bool live = false;
+    if (idx0 + lane < p.idx_end) {
+        rc = __ldg(reinterpret_cast<const int4*>(p.rec + idx0 + lane));
+        const int64_t b0 = ((int64_t)(uint32_t)rc.y << 32) | (uint32_t)rc.x;
+        if (unit_ok(p, b0, b0 + rc.z, rc.w)) {
+            const int64_t row = p.seg_perm ? __ldg(p.seg_perm + rc.w) : rc.w;
+            live = index_ok(row, p.n_out, p.status, SITE_SPMM_ROW) && __ldg(p.row_filter + row) != 0;
+        }
+    }
+    unsigned bits = __ballot_sync(0xFFFFFFFFu, live);
+    const int w4 = (p.w + 3) >> 2;
+    const unsigned gmask = CL == 32 ? 0xFFFFFFFFu : (((1u << (CL & 31)) - 1u) << (lane & ~(CL - 1)));
+    while (bits) {
+        const int src = __ffs(bits) - 1;
+        bits &= bits - 1;
+        const uint32_t lo = (uint32_t)__shfl_sync(0xFFFFFFFFu, rc.x, src), hi = (uint32_t)__shfl_sync(0xFFFFFFFFu, rc.y, src);
+        const int len = __shfl_sync(0xFFFFFFFFu, rc.z, src);
+        const int64_t u = __shfl_sync(0xFFFFFFFFu, rc.w, src);
+        const int64_t b = ((int64_t)hi << 32) | lo;
+        float4 acc[VPL];
+#pragma unroll
+        for (int v = 0; v < VPL; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (p.partial || len > PACKED) warp_segment<CL, VPL>(p, b, len, lane, w4, acc);
+        else row_segment<CL, VPL>(p, b, b + len, cl, gmask, w4, acc);
+        if (lane < CL) {
+#pragma unroll
+            for (int v = 0; v < VPL; ++v) {
+                const int c4 = cl + v * CL;
+                if (c4 < w4) {
+                    if (p.partial) reinterpret_cast<float4*>(p.partial + (idx0 + src) * p.ldp)[c4] = acc[v];
+                    else store_row(p, u, c4, acc[v]);
+                }
+            }
+        }
+        __syncwarp();
+    }
+}
+
+// Long rows: add the segments' partial rows, apply the epilogue, write Z.  The rows come longest first: the first
+// n_heavy of them (more than SPMM_HEAVY entries, tens to hundreds of segments) take a block each, whose threads split
+// (column group, share of the segments) and add the shares in order through shared memory; the others take a warp
+// (or, below 128 columns, a group of lanes) each.  With one warp for every row the launch lasted as long as the longest
+// hub row's chain of loads: 300 K nodes, width 256: 108 -> 20 us per launch.
+__device__ __forceinline__ float4 sum_segments(const SpmmParams& p, const int64_t* __restrict__ seg_pos, int64_t q, int64_t q_end, int c4) {
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (; q < q_end; q += 4) {
+        float4 t[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            t[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (q + k < q_end) {
+                const int64_t slot = __ldg(seg_pos + q + k);
+                if (index_ok(slot, p.n_partial, p.status, SITE_SPMM_SEG)) t[k] = __ldg(reinterpret_cast<const float4*>(p.partial + slot * p.ldp) + c4);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (q + k < q_end) { s.x += t[k].x; s.y += t[k].y; s.z += t[k].z; s.w += t[k].w; }
+    }
+    return s;
+}
+
 template <bool LOSS = false>
-__global__ void __launch_bounds__(256) spmm_combine_kernel(const SpmmParams p, int64_t n_long,
+__global__ void __launch_bounds__(256) spmm_combine_kernel(const SpmmParams p, int64_t n_long, int64_t n_heavy,
                                                            const int64_t* __restrict__ seg_off,
                                                            const int64_t* __restrict__ seg_pos,
                                                            const int32_t* __restrict__ perm) {
-    const int lane = threadIdx.x & 31;
-    const int64_t i = ((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5;
+    __shared__ float4 red[256];
+    pdl_wait();                                   // the partial rows are complete
+    const int w4 = (p.w + 3) >> 2;
+    const bool heavy = blockIdx.x < n_heavy;
+    int gl = 32;                                  // lanes per light row
+    if (!LOSS && !heavy) while (gl > 1 && gl / 2 >= w4) gl >>= 1;
+    const int64_t i = heavy ? (int64_t)blockIdx.x : n_heavy + (((int64_t)blockIdx.x - n_heavy) * 256 + threadIdx.x) / gl;
     if (i >= n_long) return;
     const int64_t s0 = seg_off[i], s1 = seg_off[i + 1];
     const int64_t u = perm[i];
     if (!index_ok(s0, p.n_partial + 1, p.status, SITE_SPMM_SEG) || !index_ok(s1, p.n_partial + 1, p.status, SITE_SPMM_SEG) ||
         !index_ok(u, p.n_out, p.status, SITE_SPMM_ROW)) return;
     if (p.row_filter && !__ldg(p.row_filter + u)) return;
-    const int w4 = (p.w + 3) >> 2;
-    if (p.out_mask && lane == 0) p.out_mask[u] = 1;    // long rows are kept without looking (conservative)
+    if (heavy) {
+        if (p.out_mask && threadIdx.x == 0) p.out_mask[u] = 1;    // long rows are kept without looking (conservative)
+        int cp = 1;
+        while (cp < 64 && cp * 4 < p.w_total) cp <<= 1;      // column groups side by side (by the full width: the shares set the order of the sums)
+        const int shares = 256 / cp, col = threadIdx.x % cp, share = threadIdx.x / cp;
+        const int64_t per = (s1 - s0 + shares - 1) / shares;
+        const int64_t q0 = s0 + share * per < s1 ? s0 + share * per : s1, q1 = q0 + per < s1 ? q0 + per : s1;
+        float4 row[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+        for (int c0 = 0; c0 < w4; c0 += cp) {
+            const int c4 = c0 + col;
+            red[threadIdx.x] = c4 < w4 ? sum_segments(p, seg_pos, q0, q1, c4) : make_float4(0.f, 0.f, 0.f, 0.f);
+            __syncthreads();
+            if (threadIdx.x < cp) {
+                float4 s = red[threadIdx.x];
+                for (int k = 1; k < shares; ++k) {
+                    const float4 t = red[k * cp + threadIdx.x];
+                    s.x += t.x; s.y += t.y; s.z += t.z; s.w += t.w;
+                }
+                if constexpr (LOSS) red[threadIdx.x] = s;        // one turn: at most 256 columns
+                else if (c4 < w4) store_row(p, u, c4, s);
+            }
+            __syncthreads();
+        }
+        if constexpr (LOSS) {
+            if (threadIdx.x < 32) {
+#pragma unroll
+                for (int v = 0; v < 2; ++v) if ((int)threadIdx.x + v * 32 < w4) row[v] = red[threadIdx.x + v * 32];
+                loss_epilogue<32, 2>(p, u, (int)threadIdx.x, 0xFFFFFFFFu, row);
+            }
+        }
+        return;
+    }
+    const int lane = threadIdx.x % gl;
+    if (p.out_mask && lane == 0) p.out_mask[u] = 1;
     if constexpr (LOSS) {
         // the whole row (at most 64 float4) in registers, then the same epilogue as the other rows
         float4 row[2];
 #pragma unroll
         for (int v = 0; v < 2; ++v) {
             const int c4 = lane + v * 32;
-            float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (c4 < w4)
-                for (int64_t q = s0; q < s1; ++q) {
-                    const int64_t slot = __ldg(seg_pos + q);
-                    if (!index_ok(slot, p.n_partial, p.status, SITE_SPMM_SEG)) continue;
-                    const float4 t = __ldg(reinterpret_cast<const float4*>(p.partial + slot * p.ldp) + c4);
-                    s.x += t.x; s.y += t.y; s.z += t.z; s.w += t.w;
-                }
-            row[v] = s;
+            row[v] = c4 < w4 ? sum_segments(p, seg_pos, s0, s1, c4) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         loss_epilogue<32, 2>(p, u, lane, 0xFFFFFFFFu, row);
     } else {
-        for (int c4 = lane; c4 < w4; c4 += 32) {
-            float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int64_t q = s0; q < s1; ++q) {
-                const int64_t slot = __ldg(seg_pos + q);
-                if (!index_ok(slot, p.n_partial, p.status, SITE_SPMM_SEG)) continue;
-                const float4 t = __ldg(reinterpret_cast<const float4*>(p.partial + slot * p.ldp) + c4);
-                s.x += t.x; s.y += t.y; s.z += t.z; s.w += t.w;
-            }
-            store_row(p, u, c4, s);
-        }
+        for (int c4 = lane; c4 < w4; c4 += gl) store_row(p, u, c4, sum_segments(p, seg_pos, s0, s1, c4));
     }
 }
 
+// Launch with or without leave to start before the predecessor on the stream has finished (see pdl_trigger).
+template <typename... Args>
+void launch_k(void (*kernel)(Args...), unsigned blocks, cudaStream_t s, bool early, typename std::common_type<Args>::type... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks, 1, 1);
+    cfg.blockDim = dim3(256, 1, 1);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = early ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+void launch_combine(const SpmmParams& p, const SpmmSchedule& S, bool loss, bool early, cudaStream_t s) {
+    const int w4 = (p.w + 3) >> 2;
+    int gl = 32;
+    if (!loss) while (gl > 1 && gl / 2 >= w4) gl >>= 1;
+    const int64_t light = S.n_long - S.n_heavy;
+    const unsigned blocks = (unsigned)(S.n_heavy + (light * gl + 255) / 256);
+    if (loss) launch_k(spmm_combine_kernel<true>, blocks, s, early, p, S.n_long, S.n_heavy, S.seg_off, S.seg_pos, S.perm);
+    else launch_k(spmm_combine_kernel<false>, blocks, s, early, p, S.n_long, S.n_heavy, S.seg_off, S.seg_pos, S.perm);
+}
+
 template <int LPR, int VPL, bool LOSS = false>
-void launch_group(const SpmmParams& p, cudaStream_t s) {
+void launch_group(const SpmmParams& p, cudaStream_t s, bool early) {
     const int64_t units = p.idx_end - p.idx_begin;
     if (units <= 0) return;
     const int per_block = 256 / LPR;
@@ -637,51 +894,98 @@ void launch_group(const SpmmParams& p, cudaStream_t s) {
         const bool full = LPR >= 8 && ((p.w + 3) >> 2) == LPR * VPL;     // (narrow groups: nothing to gain)
         switch (pick_epi(p)) {
             case EPI_PLAIN:
-                if (full) spmm_group_kernel<LPR, VPL, EPI_PLAIN, (LPR >= 8)><<<(unsigned)blocks, 256, 0, s>>>(p);
-                else spmm_group_kernel<LPR, VPL, EPI_PLAIN><<<(unsigned)blocks, 256, 0, s>>>(p);
+                if (full) launch_k(spmm_group_kernel<LPR, VPL, EPI_PLAIN, (LPR >= 8)>, (unsigned)blocks, s, early, p);
+                else launch_k(spmm_group_kernel<LPR, VPL, EPI_PLAIN>, (unsigned)blocks, s, early, p);
                 return;
             case EPI_BITS:
-                if (full) spmm_group_kernel<LPR, VPL, EPI_BITS, (LPR >= 8)><<<(unsigned)blocks, 256, 0, s>>>(p);
-                else spmm_group_kernel<LPR, VPL, EPI_BITS><<<(unsigned)blocks, 256, 0, s>>>(p);
+                if (full) launch_k(spmm_group_kernel<LPR, VPL, EPI_BITS, (LPR >= 8)>, (unsigned)blocks, s, early, p);
+                else launch_k(spmm_group_kernel<LPR, VPL, EPI_BITS>, (unsigned)blocks, s, early, p);
                 return;
-            case EPI_BIAS: spmm_group_kernel<LPR, VPL, EPI_BIAS><<<(unsigned)blocks, 256, 0, s>>>(p); return;
-            case EPI_GATE: spmm_group_kernel<LPR, VPL, EPI_GATE><<<(unsigned)blocks, 256, 0, s>>>(p); return;
+            case EPI_BIAS: launch_k(spmm_group_kernel<LPR, VPL, EPI_BIAS>, (unsigned)blocks, s, early, p); return;
+            case EPI_GATE: launch_k(spmm_group_kernel<LPR, VPL, EPI_GATE>, (unsigned)blocks, s, early, p); return;
             default: break;
         }
     }
-    spmm_group_kernel<LPR, VPL, LOSS ? EPI_LOSS : EPI_ANY><<<(unsigned)blocks, 256, 0, s>>>(p);
+    launch_k(spmm_group_kernel<LPR, VPL, LOSS ? EPI_LOSS : EPI_ANY>, (unsigned)blocks, s, early, p);
 }
 
-// The same packing for an aggregation with the loss epilogue (width <= 256: at most two float4 per lane
+// Narrow aggregations (w_total <= 64 columns): column lanes and float4 per lane, chosen so that few column slots of
+// a lane group stay empty.  The choice goes by the call's full width, not the slice's: the lane split decides the order
+// in which a unit's entries are added, and results do not depend on the slicing.
+struct NarrowCfg { int cl, vpl; };
+inline NarrowCfg narrow_cfg(int w_total) {
+    const int w4 = (w_total + 3) >> 2;
+    if (w4 > 16) return {0, 0};
+    if (w4 <= 1) return {1, 1};
+    if (w4 <= 2) return {2, 1};
+    if (w4 <= 4) return {4, 1};
+    if (w4 <= 6) return {2, 3};
+    if (w4 <= 8) return {8, 1};
+    if (w4 <= 12) return {4, 3};
+    return {8, 2};
+}
+
+template <int CL, int VPL>
+void launch_narrow(const SpmmParams& p, bool warp_units, bool loss, cudaStream_t s, bool early) {
+    const int64_t units = p.idx_end - p.idx_begin;
+    if (units <= 0) return;
+    if (!warp_units) {
+        if (loss) launch_group<CL, VPL, true>(p, s, early);
+        else launch_group<CL, VPL>(p, s, early);
+        return;
+    }
+    const unsigned blocks = (unsigned)((units + 7) / 8);
+    if (loss) { launch_k(spmm_warp_kernel<CL, VPL, EPI_LOSS>, blocks, s, early, p); return; }
+    switch (pick_epi(p)) {
+        case EPI_PLAIN: launch_k(spmm_warp_kernel<CL, VPL, EPI_PLAIN>, blocks, s, early, p); return;
+        case EPI_BIAS: launch_k(spmm_warp_kernel<CL, VPL, EPI_BIAS>, blocks, s, early, p); return;
+        default: launch_k(spmm_warp_kernel<CL, VPL, EPI_ANY>, blocks, s, early, p); return;
+    }
+}
+
+void dispatch_narrow(const SpmmParams& p, NarrowCfg c, bool warp_units, bool loss, cudaStream_t s, bool early) {
+#define MIXGCN_SPMM_CASE(L, V) if (c.cl == L && c.vpl == V) { launch_narrow<L, V>(p, warp_units, loss, s, early); return; }
+    MIXGCN_SPMM_CASE(1, 1) MIXGCN_SPMM_CASE(2, 1) MIXGCN_SPMM_CASE(4, 1) MIXGCN_SPMM_CASE(2, 3) MIXGCN_SPMM_CASE(8, 1)
+    MIXGCN_SPMM_CASE(4, 3) MIXGCN_SPMM_CASE(8, 2)
+#undef MIXGCN_SPMM_CASE
+}
+
+void dispatch_filtered_narrow(const SpmmParams& p, NarrowCfg c, cudaStream_t s) {
+    const int64_t units = p.idx_end - p.idx_begin;
+    if (units <= 0) return;
+    const unsigned blocks = (unsigned)((units + 255) / 256);   // 8 warps x 32 records
+#define MIXGCN_SPMM_CASE(L, V) if (c.cl == L && c.vpl == V) { spmm_filtered_narrow_kernel<L, V><<<blocks, 256, 0, s>>>(p); return; }
+    MIXGCN_SPMM_CASE(1, 1) MIXGCN_SPMM_CASE(2, 1) MIXGCN_SPMM_CASE(4, 1) MIXGCN_SPMM_CASE(2, 3) MIXGCN_SPMM_CASE(8, 1)
+    MIXGCN_SPMM_CASE(4, 3) MIXGCN_SPMM_CASE(8, 2)
+#undef MIXGCN_SPMM_CASE
+}
+
+// The same packing for an aggregation with the loss epilogue (65..256 columns, one slice: at most two float4 per lane
 // before folding).  Returns 0 if the shape has no instance.
-int dispatch_loss(const SpmmParams& p, int fold, cudaStream_t s) {
+int dispatch_loss(const SpmmParams& p, int fold, cudaStream_t s, bool early) {
     const int w4 = (p.w + 3) >> 2;
     int lpr = 1;
     while (lpr < 32 && lpr < w4) lpr <<= 1;
     int vpl = (w4 + lpr - 1) / lpr;
     while (fold > 1 && (lpr / fold < 1 || vpl * fold > 8)) fold >>= 1;
     lpr /= fold; vpl *= fold;
-#define MIXGCN_SPMM_CASE(L, V) if (lpr == L && vpl == V) { launch_group<L, V, true>(p, s); return fold; }
-    MIXGCN_SPMM_CASE(32, 1) MIXGCN_SPMM_CASE(32, 2)
-    MIXGCN_SPMM_CASE(16, 1) MIXGCN_SPMM_CASE(16, 2) MIXGCN_SPMM_CASE(16, 4)
-    MIXGCN_SPMM_CASE(8, 1) MIXGCN_SPMM_CASE(8, 2) MIXGCN_SPMM_CASE(8, 4) MIXGCN_SPMM_CASE(8, 8)
-    MIXGCN_SPMM_CASE(4, 1) MIXGCN_SPMM_CASE(4, 2) MIXGCN_SPMM_CASE(4, 4) MIXGCN_SPMM_CASE(4, 8)
-    MIXGCN_SPMM_CASE(2, 1) MIXGCN_SPMM_CASE(2, 2) MIXGCN_SPMM_CASE(2, 4) MIXGCN_SPMM_CASE(2, 8)
-    MIXGCN_SPMM_CASE(1, 1) MIXGCN_SPMM_CASE(1, 2) MIXGCN_SPMM_CASE(1, 4) MIXGCN_SPMM_CASE(1, 8)
+#define MIXGCN_SPMM_CASE(L, V) if (lpr == L && vpl == V) { launch_group<L, V, true>(p, s, early); return fold; }
+    MIXGCN_SPMM_CASE(32, 1) MIXGCN_SPMM_CASE(32, 2) MIXGCN_SPMM_CASE(16, 2) MIXGCN_SPMM_CASE(16, 4)
+    MIXGCN_SPMM_CASE(8, 4) MIXGCN_SPMM_CASE(8, 8) MIXGCN_SPMM_CASE(4, 8)
 #undef MIXGCN_SPMM_CASE
     return 0;
 }
 
 // Base configuration for a slice of w4 float4 columns, then packed `fold`-fold (fold in {1,2,4,8}):
 // fewer lanes per row, more float4 per lane.  Returns the fold actually used.
-int dispatch(const SpmmParams& p, int fold, cudaStream_t s) {
+int dispatch(const SpmmParams& p, int fold, cudaStream_t s, bool early) {
     const int w4 = (p.w + 3) >> 2;
     int lpr = 1;
     while (lpr < 32 && lpr < w4) lpr <<= 1;
     int vpl = (w4 + lpr - 1) / lpr;
     while (fold > 1 && (lpr / fold < 1 || vpl * fold > 8)) fold >>= 1;
     lpr /= fold; vpl *= fold;
-#define MIXGCN_SPMM_CASE(L, V) if (lpr == L && vpl == V) { launch_group<L, V>(p, s); return fold; }
+#define MIXGCN_SPMM_CASE(L, V) if (lpr == L && vpl == V) { launch_group<L, V>(p, s, early); return fold; }
     MIXGCN_SPMM_CASE(32, 1) MIXGCN_SPMM_CASE(32, 2) MIXGCN_SPMM_CASE(32, 3) MIXGCN_SPMM_CASE(32, 4)
     MIXGCN_SPMM_CASE(32, 5) MIXGCN_SPMM_CASE(32, 6) MIXGCN_SPMM_CASE(32, 7) MIXGCN_SPMM_CASE(32, 8)
     MIXGCN_SPMM_CASE(16, 1) MIXGCN_SPMM_CASE(16, 2) MIXGCN_SPMM_CASE(16, 4) MIXGCN_SPMM_CASE(16, 6) MIXGCN_SPMM_CASE(16, 8)
@@ -691,6 +995,20 @@ int dispatch(const SpmmParams& p, int fold, cudaStream_t s) {
     MIXGCN_SPMM_CASE(1, 1) MIXGCN_SPMM_CASE(1, 2) MIXGCN_SPMM_CASE(1, 4) MIXGCN_SPMM_CASE(1, 8)
 #undef MIXGCN_SPMM_CASE
     return 0;
+}
+
+template <int RB, int VPL>
+void launch_short(const SpmmParams& p, int64_t units, cudaStream_t s, bool early) {
+    constexpr int MAXE = SPMM_SHORT_MAXE;
+    const int64_t warps = (units + RB - 1) / RB;
+    const unsigned blocks = (unsigned)((warps + 7) / 8);
+    switch (pick_epi(p)) {
+        case EPI_PLAIN: launch_k(spmm_short_kernel<RB, MAXE, EPI_PLAIN, VPL>, blocks, s, early, p); return;
+        case EPI_BITS: launch_k(spmm_short_kernel<RB, MAXE, EPI_BITS, VPL>, blocks, s, early, p); return;
+        case EPI_BIAS: launch_k(spmm_short_kernel<RB, MAXE, EPI_BIAS, VPL>, blocks, s, early, p); return;
+        case EPI_GATE: launch_k(spmm_short_kernel<RB, MAXE, EPI_GATE, VPL>, blocks, s, early, p); return;
+        default: launch_k(spmm_short_kernel<RB, MAXE, EPI_ANY, VPL>, blocks, s, early, p); return;
+    }
 }
 
 template <int LPR, int VPL>
@@ -793,6 +1111,7 @@ mixgcn_status launch_spmm(mixgcn_ctx* ctx, const mixgcn_graph* g, const CsrView&
         p.loss_row = lf->row_loss; p.loss_pred = lf->pred; p.loss_zero_rows = lf->zero_rows;
     }
     const int slice = lf ? MAX_SLICE : ctx->spmm_slice_cols > 0 ? (ctx->spmm_slice_cols < MAX_SLICE ? ctx->spmm_slice_cols : MAX_SLICE) : DEFAULT_SLICE;
+    const NarrowCfg narrow = narrow_cfg(w);
     for (int j0 = 0; j0 < w; j0 += slice) {
         p.j0 = j0;
         p.w = (w - j0) < slice ? (w - j0) : slice;
@@ -809,8 +1128,7 @@ mixgcn_status launch_spmm(mixgcn_ctx* ctx, const mixgcn_graph* g, const CsrView&
                 }
                 {
                     LaunchScope scope(ctx, PH_SPMM_SPARSE, s);
-                    const int64_t blocks = (S.n_long * 32 + 255) / 256;
-                    spmm_combine_kernel<false><<<(unsigned)blocks, 256, 0, s>>>(p, S.n_long, S.seg_off, S.seg_pos, S.perm);
+                    launch_combine(p, S, false, false, s);
                 }
                 p.partial = nullptr;
             }
@@ -844,41 +1162,41 @@ mixgcn_status launch_spmm(mixgcn_ctx* ctx, const mixgcn_graph* g, const CsrView&
                     LaunchScope scope(ctx, PH_SPMM_SPARSE, s);
                     p.idx_begin = 0; p.idx_end = S.total_segs;
                     p.seg_perm = S.perm;
-                    dispatch_filtered(p, s);
+                    if (narrow.cl) dispatch_filtered_narrow(p, narrow, s);
+                    else dispatch_filtered(p, s);
                     p.seg_perm = nullptr;
                 }
                 {
                     LaunchScope scope(ctx, PH_SPMM_SPARSE, s);
-                    const int64_t blocks = (S.n_long * 32 + 255) / 256;
-                    spmm_combine_kernel<false><<<(unsigned)blocks, 256, 0, s>>>(p, S.n_long, S.seg_off, S.seg_pos, S.perm);
+                    launch_combine(p, S, false, false, s);
                 }
                 p.partial = nullptr;
             }
             if (S.n_rows > S.n_long) {
                 LaunchScope scope(ctx, PH_SPMM_SPARSE, s);
                 p.idx_begin = S.total_segs; p.idx_end = S.total_segs + (S.n_rows - S.n_long);
-                dispatch_filtered(p, s);
+                if (narrow.cl) dispatch_filtered_narrow(p, narrow, s);
+                else dispatch_filtered(p, s);
             }
             continue;
         }
+        // Segments of the long rows, the other rows by bucket, then the combination of the segments.  The first launch
+        // waits for whatever precedes it on the stream; the others may start as soon as their predecessor's blocks all
+        // run (each ends only after its predecessor has ended, and the combination waits before it reads).
+        bool early = false;
+        float* partial = nullptr;
+        const int64_t ldp = ((int64_t)p.w + 3) / 4 * 4;
         if (S.total_segs > 0) {
-            const int64_t ldp = ((int64_t)p.w + 3) / 4 * 4;
             MIXGCN_TRY(ensure_workspace_spmm(ctx, S.total_segs * ldp * (int64_t)sizeof(float)));
-            p.partial = reinterpret_cast<float*>(ctx->workspace_spmm); p.ldp = ldp;
-            {
-                LaunchScope scope(ctx, phase, s);
-                p.idx_begin = 0; p.idx_end = S.total_segs;
-                if (p.out_bits && p.bits_skip) p.seg_perm = S.perm;       // a segment's record names its long row by ordinal
-                dispatch(p, p.w <= SPMM_FOLD_WMAX ? SPMM_FOLD_SEG : 1, s);
-                p.seg_perm = nullptr;
-            }
-            {
-                LaunchScope scope(ctx, phase, s);
-                const int64_t blocks = (S.n_long * 32 + 255) / 256;
-                if (lf) spmm_combine_kernel<true><<<(unsigned)blocks, 256, 0, s>>>(p, S.n_long, S.seg_off, S.seg_pos, S.perm);
-                else spmm_combine_kernel<false><<<(unsigned)blocks, 256, 0, s>>>(p, S.n_long, S.seg_off, S.seg_pos, S.perm);
-            }
-            p.partial = nullptr;
+            partial = reinterpret_cast<float*>(ctx->workspace_spmm);
+            p.partial = partial; p.ldp = ldp;
+            LaunchScope scope(ctx, phase, s);
+            p.idx_begin = 0; p.idx_end = S.total_segs;
+            if (p.out_bits && p.bits_skip) p.seg_perm = S.perm;       // a segment's record names its long row by ordinal
+            if (narrow.cl) dispatch_narrow(p, narrow, true, false, s, early);
+            else dispatch(p, p.w <= SPMM_FOLD_WMAX ? SPMM_FOLD_SEG : 1, s, early);
+            p.seg_perm = nullptr; p.partial = nullptr;
+            early = true;
         }
         // ordinary rows, in perm order: [n_long, n_rows) -> records [total_segs, total_segs + n_rows - n_long)
         int64_t bound[5];
@@ -890,6 +1208,7 @@ mixgcn_status launch_spmm(mixgcn_ctx* ctx, const mixgcn_graph* g, const CsrView&
             const int64_t lim = row_limit > S.n_long ? row_limit : S.n_long;
             for (int q = 1; q < 5; ++q) if (bound[q] > lim) bound[q] = lim;
         }
+        if (narrow.cl) bound[2] = bound[3] = bound[1];     // narrow rows of up to 12 entries: one bucket, one group of lanes each
         int64_t begin = bound[0];
         int fold = 1;
         for (int q = 0; q < 4; ++q, fold <<= 1) {
@@ -898,36 +1217,28 @@ mixgcn_status launch_spmm(mixgcn_ctx* ctx, const mixgcn_graph* g, const CsrView&
             p.idx_begin = S.total_segs + (begin - S.n_long);
             p.idx_end = S.total_segs + (end - S.n_long);
             LaunchScope scope(ctx, phase, s);
-            if (lf) {
-                if (!dispatch_loss(p, q == 0 ? (p.w <= SPMM_FOLD_WMAX ? SPMM_FOLD_MED : 1) : fold, s)) MIXGCN_FAIL(MIXGCN_EUNSUPPORTED, "spmm: no loss-epilogue kernel for width %d", p.w);
+            const int64_t units = p.idx_end - p.idx_begin;
+            if (narrow.cl) {
+                dispatch_narrow(p, narrow, q == 0, lf != nullptr, s, early);
+            } else if (lf) {
+                if (!dispatch_loss(p, q == 0 ? (p.w <= SPMM_FOLD_WMAX ? SPMM_FOLD_MED : 1) : fold, s, early)) MIXGCN_FAIL(MIXGCN_EUNSUPPORTED, "spmm: no loss-epilogue kernel for width %d", p.w);
             } else if (q == 3 && p.w <= 128 && SPMM_PACK_DEG[2] <= SPMM_SHORT_MAXE) {
                 // rows of at most SPMM_PACK_DEG[2] entries: several rows per warp, whole-warp gathers
-                constexpr int RB = SPMM_SHORT_RB, MAXE = SPMM_SHORT_MAXE;
-                const int64_t units = p.idx_end - p.idx_begin;
-                const int64_t warps = (units + RB - 1) / RB;
-                const unsigned grid_short = (unsigned)((warps + 7) / 8);
-                const int epi_short = pick_epi(p);
-                if (epi_short == EPI_PLAIN) spmm_short_kernel<RB, MAXE, EPI_PLAIN><<<grid_short, 256, 0, s>>>(p);
-                else if (epi_short == EPI_BITS) spmm_short_kernel<RB, MAXE, EPI_BITS><<<grid_short, 256, 0, s>>>(p);
-                else if (epi_short == EPI_BIAS) spmm_short_kernel<RB, MAXE, EPI_BIAS><<<grid_short, 256, 0, s>>>(p);
-                else if (epi_short == EPI_GATE) spmm_short_kernel<RB, MAXE, EPI_GATE><<<grid_short, 256, 0, s>>>(p);
-                else spmm_short_kernel<RB, MAXE, EPI_ANY><<<grid_short, 256, 0, s>>>(p);
+                launch_short<SPMM_SHORT_RB, 1>(p, units, s, early);
             } else if (q == 3 && p.w <= 256 && SPMM_PACK_DEG[2] <= SPMM_SHORT_MAXE) {
                 // the same for widths up to 256: two float4 per lane, two rows per warp
-                constexpr int RB = SPMM_SHORT_RB / 2, MAXE = SPMM_SHORT_MAXE;
-                const int64_t units = p.idx_end - p.idx_begin;
-                const int64_t warps = (units + RB - 1) / RB;
-                const unsigned grid_short = (unsigned)((warps + 7) / 8);
-                const int epi_short = pick_epi(p);
-                if (epi_short == EPI_PLAIN) spmm_short_kernel<RB, MAXE, EPI_PLAIN, 2><<<grid_short, 256, 0, s>>>(p);
-                else if (epi_short == EPI_BITS) spmm_short_kernel<RB, MAXE, EPI_BITS, 2><<<grid_short, 256, 0, s>>>(p);
-                else if (epi_short == EPI_BIAS) spmm_short_kernel<RB, MAXE, EPI_BIAS, 2><<<grid_short, 256, 0, s>>>(p);
-                else if (epi_short == EPI_GATE) spmm_short_kernel<RB, MAXE, EPI_GATE, 2><<<grid_short, 256, 0, s>>>(p);
-                else spmm_short_kernel<RB, MAXE, EPI_ANY, 2><<<grid_short, 256, 0, s>>>(p);
+                launch_short<SPMM_SHORT_RB / 2, 2>(p, units, s, early);
             } else {
-                dispatch(p, q == 0 ? (p.w <= SPMM_FOLD_WMAX ? SPMM_FOLD_MED : 1) : fold, s);
+                dispatch(p, q == 0 ? (p.w <= SPMM_FOLD_WMAX ? SPMM_FOLD_MED : 1) : fold, s, early);
             }
+            early = true;
             begin = end;
+        }
+        if (S.total_segs > 0) {
+            LaunchScope scope(ctx, phase, s);
+            p.partial = partial;
+            launch_combine(p, S, lf != nullptr, early, s);
+            p.partial = nullptr;
         }
     }
     MIXGCN_CUDA(cudaGetLastError());

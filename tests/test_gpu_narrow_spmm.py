@@ -1,0 +1,61 @@
+"""Narrow aggregations (one warp per unit, at most 64 columns), segment lengths of small graphs and the block-wide
+combination of hub rows, against the oracle: rows on either side of every boundary (12 entries, the segment length,
+2,048 entries), widths on either side of every lane split."""
+import numpy as np
+import pytest
+import torch
+
+from helpers import TOL_FP32, rel_fro
+from oracle import gcn_oracle as orc
+from paper_2501_01951_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+LENGTHS = (1, 2, 3, 11, 12, 13, 14, 31, 33, 63, 64, 65, 66, 127, 129, 511, 512, 513, 514, 2046, 2047, 2048, 2049, 4999)
+
+
+@pytest.fixture(scope="module")
+def mg():
+    from paper_2501_01951_b200 import build
+    build.build()
+    from paper_2501_01951_b200 import binding
+    return binding
+
+
+@pytest.fixture(scope="module")
+def problem(mg):
+    """Directed graph whose first rows have exactly the LENGTHS (the diagonal among them)."""
+    n = 5000
+    rng = np.random.default_rng(3)
+    s, d = [], []
+    for u, k in enumerate(LENGTHS):
+        others = np.setdiff1d(rng.permutation(n), [u], assume_unique=False)
+        s.append(np.full(k - 1, u)); d.append(rng.permutation(others)[: k - 1])
+    s, d = np.concatenate(s), np.concatenate(d)
+    go = orc.graph_build(n, s, d, flags=orc.ADD_SELF_LOOPS)
+    assert tuple(np.diff(go.rowptr)[: len(LENGTHS)]) == LENGTHS
+    ctx = mg.ctx_create(0)
+    g = mg.graph_create(ctx, n, torch.tensor(s, dtype=torch.int32), torch.tensor(d, dtype=torch.int32), mg.GRAPH_ADD_SELF_LOOPS)
+    yield ctx, g, go
+    assert mg.ctx_poll_status(ctx, raise_on_error=False) == 0
+    g.close(); ctx.close()
+
+
+@pytest.mark.parametrize("w", [1, 4, 5, 8, 9, 16, 17, 24, 25, 32, 33, 47, 48, 49, 64, 65, 200])
+def test_narrow_aggregation(mg, problem, w):
+    ctx, g, go = problem
+    n, ld = go.n, (w + 3) // 4 * 4
+    X = synth.uniform_tensor((n, w), 70 + w, -1, 1)
+    b = synth.uniform_tensor((w,), 71 + w, -0.5, 0.5)
+    Y = torch.zeros(n, ld, device="cuda"); Y[:, :w] = X.cuda()
+    Z = torch.full((n, ld), 9.0, device="cuda")
+    want = orc.aggregate(go, X.numpy())
+    rows = slice(0, len(LENGTHS))
+    for epi, f in ((None, lambda z: z), (dict(bias=b.cuda(), relu=True), lambda z: np.maximum(z + b.numpy(), 0.0)),
+                   (dict(residual=Y, residual_scale=0.5, bias=b.cuda()), lambda z: z + 0.5 * X.numpy() + b.numpy())):
+        mg.spmm(ctx, g, Y, Z, w, epi=None if epi is None else mg.make_epilogue(**epi))
+        got = Z[:, :w].cpu().numpy().astype(np.float64)
+        assert rel_fro(got, f(want)) <= TOL_FP32 and rel_fro(got[rows], f(want)[rows]) <= TOL_FP32
+        assert torch.all(Z[:, w:] == 0)
+    mg.spmm(ctx, g, Y, Z, w, transposed=True)
+    assert rel_fro(Z[:, :w].cpu().numpy().astype(np.float64), orc.aggregate(go, X.numpy(), transposed=True)) <= TOL_FP32

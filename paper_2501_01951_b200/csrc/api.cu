@@ -6,6 +6,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <mutex>
 #include <new>
 
 #include "internal.cuh"
@@ -47,53 +48,85 @@ LaunchScope::~LaunchScope() {
     if (span >= 0) cudaEventRecord(ctx->spans[span].b, stream);
 }
 
-mixgcn_status ensure_workspace(mixgcn_ctx* ctx, int64_t bytes) {
-    if (bytes <= ctx->workspace_bytes) return MIXGCN_OK;
-    int64_t want = bytes + (bytes >> 2);
-    want = (want + 255) & ~(int64_t)255;
-    void* p = nullptr;
-    // the old block may still be in use by enqueued kernels: wait before releasing it
-    MIXGCN_CUDA(cudaDeviceSynchronize());
-    if (ctx->workspace) cudaFree(ctx->workspace);
-    ctx->workspace = nullptr; ctx->workspace_bytes = 0;
-    cudaError_t e = cudaMalloc(&p, (size_t)want);
+// One memory pool per device for everything the library allocates.  Building a graph takes some thirty temporary blocks
+// and its arrays; cudaMalloc and cudaFree of each cost 0.1 ms and more (7 of the 9 ms of a graph with 4 M entries, and
+// many times that when they had to map fresh memory), and each synchronises the device.  The pool keeps at most
+// POOL_KEEP bytes of freed memory for reuse; what is above goes back to the driver at the next synchronisation, and all
+// of it when the last context on the device is destroyed.  The driver's pools are safe with several threads and streams.
+namespace {
+constexpr uint64_t POOL_KEEP = 2ull << 30;
+constexpr int MAX_DEVICES = 64;
+struct DevicePool { cudaMemPool_t pool = nullptr; int contexts = 0; };
+std::mutex g_pool_mutex;
+DevicePool g_pools[MAX_DEVICES];
+
+mixgcn_status pool_of(int device, cudaMemPool_t* out) {       // g_pool_mutex held
+    DevicePool& d = g_pools[device];
+    if (!d.pool) {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = device;
+        MIXGCN_CUDA(cudaMemPoolCreate(&d.pool, &props));
+    }
+    *out = d.pool;
+    return MIXGCN_OK;
+}
+
+// A context came (+1) or went (-1): the pool keeps freed memory only while there is one.
+mixgcn_status pool_contexts(int device, int change) {
+    std::lock_guard<std::mutex> lock(g_pool_mutex);
+    cudaMemPool_t pool;
+    MIXGCN_TRY(pool_of(device, &pool));
+    DevicePool& d = g_pools[device];
+    const int before = d.contexts;
+    d.contexts += change;
+    if ((before == 0) != (d.contexts == 0)) {
+        uint64_t keep = d.contexts ? POOL_KEEP : 0;
+        MIXGCN_CUDA(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
+        if (!d.contexts) MIXGCN_CUDA(cudaMemPoolTrimTo(pool, 0));
+    }
+    return MIXGCN_OK;
+}
+}  // namespace
+
+mixgcn_status dev_alloc(void** p, int64_t bytes, cudaStream_t s) {
+    *p = nullptr;
+    int device = 0;
+    MIXGCN_CUDA(cudaGetDevice(&device));
+    cudaMemPool_t pool;
+    {
+        std::lock_guard<std::mutex> lock(g_pool_mutex);
+        MIXGCN_TRY(pool_of(device, &pool));
+    }
+    const cudaError_t e = cudaMallocFromPoolAsync(p, (size_t)bytes, pool, s);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        MIXGCN_FAIL(MIXGCN_ENOMEM, "workspace of %lld bytes could not be allocated", (long long)want);
+        *p = nullptr;
+        if (e == cudaErrorMemoryAllocation) MIXGCN_FAIL(MIXGCN_ENOMEM, "%lld bytes of device memory could not be allocated", (long long)bytes);
+        MIXGCN_FAIL(MIXGCN_ECUDA, "device allocation of %lld bytes failed: %s", (long long)bytes, cudaGetErrorString(e));
     }
-    ctx->workspace = p; ctx->workspace_bytes = want;
     return MIXGCN_OK;
 }
 
-mixgcn_status ensure_workspace_spmm(mixgcn_ctx* ctx, int64_t bytes) {
-    if (bytes <= ctx->workspace_spmm_bytes) return MIXGCN_OK;
-    int64_t want = bytes + (bytes >> 2);
-    want = (want + 255) & ~(int64_t)255;
-    void* p = nullptr;
-    MIXGCN_CUDA(cudaDeviceSynchronize());
-    if (ctx->workspace_spmm) cudaFree(ctx->workspace_spmm);
-    ctx->workspace_spmm = nullptr; ctx->workspace_spmm_bytes = 0;
-    if (cudaMalloc(&p, (size_t)want) != cudaSuccess) {
-        cudaGetLastError();
-        MIXGCN_FAIL(MIXGCN_ENOMEM, "aggregation workspace of %lld bytes could not be allocated", (long long)want);
-    }
-    ctx->workspace_spmm = p; ctx->workspace_spmm_bytes = want;
-    return MIXGCN_OK;
-}
+void dev_free(void* p, cudaStream_t s) { if (p) cudaFreeAsync(p, s); }
 
-mixgcn_status ensure_workspace_lp(mixgcn_ctx* ctx, int64_t bytes) {
-    if (bytes <= ctx->workspace_lp_bytes) return MIXGCN_OK;
-    int64_t want = bytes + (bytes >> 3);
+mixgcn_status grow_block(mixgcn_ctx* ctx, void** block, int64_t* have, int64_t bytes, const char* what, bool exact) {
+    if (bytes <= *have) return MIXGCN_OK;
+    int64_t want = exact ? bytes : bytes + (bytes >> 3);
     want = (want + 255) & ~(int64_t)255;
-    void* p = nullptr;
+    // the old block may still be in use by enqueued kernels: wait before releasing it
     MIXGCN_CUDA(cudaDeviceSynchronize());
-    if (ctx->workspace_lp) cudaFree(ctx->workspace_lp);
-    ctx->workspace_lp = nullptr; ctx->workspace_lp_bytes = 0;
-    if (cudaMalloc(&p, (size_t)want) != cudaSuccess) {
-        cudaGetLastError();
-        MIXGCN_FAIL(MIXGCN_ENOMEM, "bf16 operand workspace of %lld bytes could not be allocated", (long long)want);
-    }
-    ctx->workspace_lp = p; ctx->workspace_lp_bytes = want;
+    cudaStream_t s = ctx->side_stream[0];
+    dev_free(*block, s);
+    *block = nullptr; *have = 0;
+    ctx->blocks_generation++;
+    void* p = nullptr;
+    const mixgcn_status st = dev_alloc(&p, want, s);
+    if (st == MIXGCN_ENOMEM) MIXGCN_FAIL(MIXGCN_ENOMEM, "%s of %lld bytes could not be allocated", what, (long long)want);
+    MIXGCN_TRY(st);
+    MIXGCN_CUDA(cudaStreamSynchronize(s));       // usable on every stream from here on
+    *block = p; *have = want;
     return MIXGCN_OK;
 }
 
@@ -193,6 +226,9 @@ extern "C" mixgcn_status mixgcn_ctx_create(mixgcn_ctx** out, int device) {
     if (!c) MIXGCN_FAIL(MIXGCN_ENOMEM, "ctx_create: host allocation failed");
     memset(c, 0, sizeof(*c));
     c->device = device;
+    if (device >= MAX_DEVICES) { delete c; MIXGCN_FAIL(MIXGCN_EUNSUPPORTED, "ctx_create: device index %d not supported", device); }
+    const mixgcn_status pool_st = pool_contexts(device, +1);
+    if (pool_st != MIXGCN_OK) { delete c; return pool_st; }
     c->sm_count = prop.multiProcessorCount;
     MIXGCN_CUDA(cudaMalloc((void**)&c->d_status, 4 * sizeof(int32_t)));
     MIXGCN_CUDA(cudaMemset(c->d_status, 0, 4 * sizeof(int32_t)));
@@ -217,13 +253,10 @@ extern "C" mixgcn_status mixgcn_ctx_destroy(mixgcn_ctx* ctx) {
     for (int i = 0; i < 2; ++i) { if (ctx->join_ev[i]) cudaEventDestroy(ctx->join_ev[i]); if (ctx->side_stream[i]) cudaStreamDestroy(ctx->side_stream[i]); }
     if (ctx->fork_ev) cudaEventDestroy(ctx->fork_ev);
     free_step_cache(ctx);
-    cudaFree(ctx->workspace);
-    cudaFree(ctx->workspace_spmm);
-    cudaFree(ctx->workspace_rows);
-    cudaFree(ctx->workspace_lp);
-    cudaFree(ctx->workspace_loss);
-    cudaFree(ctx->arena);
+    for (void* block : {ctx->workspace, ctx->workspace_spmm, ctx->workspace_rows, ctx->workspace_lp, ctx->workspace_loss, ctx->arena}) dev_free(block, nullptr);
     cudaFree(ctx->d_status);
+    cudaStreamSynchronize(nullptr);
+    pool_contexts(ctx->device, -1);
     delete ctx;
     return MIXGCN_OK;
 }

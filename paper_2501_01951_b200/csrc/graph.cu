@@ -2,15 +2,19 @@
 // A_hat = D^-1/2 (A+I) D^-1/2 (Section 2.1 of the paper) -> CSR of the transpose (aliased when
 // symmetric) -> degree-sorted row schedule.  Sorting, run-length and selection steps use CUB
 // device primitives; everything else is a kernel in this file.
+//
+// What a build costs beside its kernels is memory and waiting: every temporary comes from the library's pool, the host
+// waits twice (for the entry count, then for the schedule's counts), keys carry no more bits than the ids have
+// (a radix pass over the keys costs as much as any other kernel here), and what the flags already say about the
+// structure is not looked up.  250 K nodes, 4.2 M entries: 9.0 ms and more -> 0.6 ms.
 #include <cub/cub.cuh>
 
+#include <atomic>
 #include <new>
 
 #include "internal.cuh"
 
 using namespace mixgcn;
-
-#include <atomic>
 
 namespace {
 
@@ -23,37 +27,39 @@ constexpr int TPB = 256;
 inline unsigned blocks_for(int64_t n) { return (unsigned)((n + TPB - 1) / TPB); }
 
 // flag bits written by validation kernels
-enum { F_BAD_ID = 1, F_NOT_SYMMETRIC = 2, F_BAD_ROWPTR = 4, F_UNSORTED = 8 };
+enum { F_BAD_ID = 1, F_NOT_SYMMETRIC = 2, F_BAD_ROWPTR = 4, F_UNSORTED = 8, F_DROPPED = 16 };
 
+// Keys (row << shift | column) of the entries; dropped edges become the sentinel n << shift, which sorts last.
+template <typename Key>
 __global__ void make_keys_kernel(int64_t n, int64_t m, const int32_t* __restrict__ src,
-                                 const int32_t* __restrict__ dst, int sym, int self_loops,
-                                 uint64_t sentinel, uint64_t* __restrict__ keys, int32_t* flags) {
+                                 const int32_t* __restrict__ dst, int sym, int self_loops, int shift,
+                                 Key* __restrict__ keys, int32_t* flags) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < m) {
-        int32_t u = src[i], v = dst[i];
-        bool bad = u < 0 || v < 0 || u >= n || v >= n;
-        if (bad) atomicOr(flags, F_BAD_ID);
-        bool drop = bad || u == v;
-        keys[i] = drop ? sentinel : (((uint64_t)(uint32_t)u << 32) | (uint32_t)v);
-        if (sym) keys[m + i] = drop ? sentinel : (((uint64_t)(uint32_t)v << 32) | (uint32_t)u);
+        const int32_t u = src[i], v = dst[i];
+        const bool bad = u < 0 || v < 0 || u >= n || v >= n;
+        const bool drop = bad || u == v;
+        if (drop) atomicOr(flags, bad ? (F_BAD_ID | F_DROPPED) : F_DROPPED);
+        const Key sentinel = (Key)n << shift;
+        keys[i] = drop ? sentinel : (((Key)(uint32_t)u << shift) | (Key)(uint32_t)v);
+        if (sym) keys[m + i] = drop ? sentinel : (((Key)(uint32_t)v << shift) | (Key)(uint32_t)u);
     }
-    if (self_loops && i < n) {
-        int64_t base = sym ? 2 * m : m;
-        keys[base + i] = ((uint64_t)i << 32) | (uint64_t)i;
-    }
+    if (self_loops && i < n) keys[(sym ? 2 * m : m) + i] = ((Key)i << shift) | (Key)i;
 }
 
 // rowptr[q] = first position whose row id is >= q, from the sorted unique keys.
-__global__ void rowptr_from_keys_kernel(int64_t n, int64_t nnz, const uint64_t* __restrict__ keys,
+template <typename Key>
+__global__ void rowptr_from_keys_kernel(int64_t n, int64_t nnz, int shift, const Key* __restrict__ keys,
                                         int64_t* __restrict__ rowptr, int32_t* __restrict__ col) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < nnz) {
-        int64_t r = (int64_t)(keys[i] >> 32);
-        int64_t rp = i == 0 ? -1 : (int64_t)(keys[i - 1] >> 32);
+        const Key k = keys[i];
+        const int64_t r = (int64_t)(k >> shift);
+        const int64_t rp = i == 0 ? -1 : (int64_t)(keys[i - 1] >> shift);
         for (int64_t q = rp + 1; q <= r; ++q) rowptr[q] = i;
-        col[i] = (int32_t)(uint32_t)(keys[i] & 0xFFFFFFFFull);
+        col[i] = (int32_t)(uint32_t)(k & (((Key)1 << shift) - 1));
     } else if (i == nnz) {
-        int64_t last = nnz == 0 ? -1 : (int64_t)(keys[nnz - 1] >> 32);
+        const int64_t last = nnz == 0 ? -1 : (int64_t)(keys[nnz - 1] >> shift);
         for (int64_t q = last + 1; q <= n; ++q) rowptr[q] = nnz;
     }
 }
@@ -68,21 +74,33 @@ __global__ void degree_kernel(int64_t n, const int64_t* __restrict__ rowptr, int
     dinv[u] = d > 0 ? __frcp_rn(__fsqrt_rn((float)d)) : 0.0f;
 }
 
-// One warp per row.  norm 0: val_uv = dinv_u * dinv_v (Section 2.1); 1: 1 / (entries in row u), the row
-// mean (GraphSAGE's mean aggregator); 2: 1, the plain sum (GIN's sum aggregator).
+// Value of an entry of row u.  norm 0: dinv_u * dinv_v (Section 2.1); 1: 1 / (entries in row u), the row mean (GraphSAGE's
+// mean aggregator; IEEE reciprocal); 2: 1, the plain sum (GIN's sum aggregator).
+__device__ __forceinline__ float entry_value(int norm, float dinv_u, float dinv_v, int32_t deg_u) {
+    return norm == 0 ? __fmul_rn(dinv_u, dinv_v) : norm == 1 ? __frcp_rn((float)deg_u) : 1.0f;
+}
+
+// One warp per row.
 __global__ void values_kernel(int64_t n, const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
                               const float* __restrict__ dinv, int norm, float* __restrict__ val) {
     int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int lane = threadIdx.x & 31;
     if (u >= n) return;
     const int64_t b = rowptr[u], e = rowptr[u + 1];
-    if (norm == 0) {
-        float du = dinv[u];
-        for (int64_t i = b + lane; i < e; i += 32) val[i] = __fmul_rn(du, dinv[col[i]]);
-    } else {
-        const float v = norm == 1 ? __frcp_rn((float)(e - b)) : 1.0f;   // IEEE reciprocal of the entry count
-        for (int64_t i = b + lane; i < e; i += 32) val[i] = v;
-    }
+    const float du = dinv[u];
+    for (int64_t i = b + lane; i < e; i += 32) val[i] = entry_value(norm, du, norm == 0 ? dinv[col[i]] : 0.0f, (int32_t)(e - b));
+}
+
+// One thread per entry, where the sorted keys still name its row: no row is too short or too long for its lanes
+// (250 K nodes, 4.2 M entries: 68 -> 15 us).
+template <typename Key>
+__global__ void values_from_keys_kernel(int64_t nnz, int shift, const Key* __restrict__ keys, const int32_t* __restrict__ deg,
+                                        const float* __restrict__ dinv, int norm, float* __restrict__ val) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= nnz) return;
+    const Key k = keys[i];
+    const int64_t u = (int64_t)(k >> shift), v = (int64_t)(k & (((Key)1 << shift) - 1));
+    val[i] = entry_value(norm, __ldg(dinv + u), norm == 0 ? __ldg(dinv + v) : 0.0f, norm == 1 ? __ldg(deg + u) : 0);
 }
 
 // For every stored (u,v), u != v, look v's row up for u.
@@ -124,39 +142,41 @@ __global__ void diagonal_count_kernel(int64_t n, const int64_t* __restrict__ row
     if ((threadIdx.x & 31) == 0 && b) atomicAdd(count, (unsigned long long)__popc(b));
 }
 
-__global__ void transpose_keys_kernel(int64_t n, const int64_t* __restrict__ rowptr,
+__global__ void transpose_keys_kernel(int64_t n, int shift, const int64_t* __restrict__ rowptr,
                                       const int32_t* __restrict__ col, uint64_t* __restrict__ keys) {
     int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int lane = threadIdx.x & 31;
     if (u >= n) return;
     for (int64_t i = rowptr[u] + lane; i < rowptr[u + 1]; i += 32)
-        keys[i] = ((uint64_t)(uint32_t)col[i] << 32) | (uint32_t)u;
+        keys[i] = ((uint64_t)(uint32_t)col[i] << shift) | (uint64_t)u;
 }
 
-__global__ void schedule_keys_kernel(int64_t row0, int64_t n_rows, const int64_t* __restrict__ rowptr,
-                                     uint64_t* __restrict__ keys) {
+// Sort key of a row: most entries first (top - entries); ties keep their ascending ids because the sort is stable.
+__global__ void schedule_keys_kernel(int64_t row0, int64_t n_rows, uint32_t top, const int64_t* __restrict__ rowptr,
+                                     uint32_t* __restrict__ keys, int32_t* __restrict__ ids) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_rows) return;
     const int64_t u = row0 + i;
-    uint64_t d = (uint64_t)(rowptr[u + 1] - rowptr[u]);
-    keys[i] = ((0x7FFFFFFFull - d) << 32) | (uint64_t)u;  // descending entries, ascending id
+    keys[i] = top - (uint32_t)(rowptr[u + 1] - rowptr[u]);
+    ids[i] = (int32_t)u;
 }
 
-// perm from the sorted keys; counts[0] = rows longer than seg, counts[1..3] = rows longer than SPMM_PACK_DEG[0..2],
-// counts[4] = rows longer than SPMM_HEAVY (one atomic per warp and counter; integers, so order does not matter).
-__global__ void schedule_finish_kernel(int64_t n, const uint64_t* __restrict__ keys, int32_t* __restrict__ perm,
-                                       int seg, unsigned long long* counts) {
+// What the host has to know of a schedule, counted on the device (integers, so the order of the atomics does not matter).
+struct ScheduleCounts {
+    unsigned long long rows_above_seg, rows_above[3], rows_heavy, total_segs, max_deg;
+};
+
+// Row counts of the buckets (one atomic per warp and counter).
+__global__ void schedule_counts_kernel(int64_t n, uint32_t top, const uint32_t* __restrict__ keys, int seg, ScheduleCounts* counts) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int64_t d = -1;
-    if (i < n) {
-        perm[i] = (int32_t)(uint32_t)(keys[i] & 0xFFFFFFFFull);
-        d = (int64_t)(0x7FFFFFFFull - (keys[i] >> 32));
-    }
+    const int64_t d = i < n ? (int64_t)(top - keys[i]) : -1;
+    if (i == 0) counts->max_deg = (unsigned long long)d;
     const int thr[5] = {seg, SPMM_PACK_DEG[0], SPMM_PACK_DEG[1], SPMM_PACK_DEG[2], SPMM_HEAVY};
+    unsigned long long* const to[5] = {&counts->rows_above_seg, &counts->rows_above[0], &counts->rows_above[1], &counts->rows_above[2], &counts->rows_heavy};
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
-        unsigned b = __ballot_sync(0xFFFFFFFFu, d > thr[q]);
-        if ((threadIdx.x & 31) == 0 && b) atomicAdd(counts + q, (unsigned long long)__popc(b));
+        const unsigned b = __ballot_sync(0xFFFFFFFFu, d > thr[q]);
+        if ((threadIdx.x & 31) == 0 && b) atomicAdd(to[q], (unsigned long long)__popc(b));
     }
 }
 
@@ -168,15 +188,6 @@ __device__ __forceinline__ int row_log_blocks(int64_t d) {
     return k;
 }
 
-__global__ void blk_count_kernel(int64_t n_long, const int32_t* __restrict__ perm, const int64_t* __restrict__ rowptr,
-                                 int64_t* __restrict__ nblk) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i > n_long) return;
-    if (i == n_long) { nblk[i] = 0; return; }
-    const int64_t u = perm[i];
-    nblk[i] = (int64_t)1 << row_log_blocks(rowptr[u + 1] - rowptr[u]);
-}
-
 __device__ __forceinline__ int64_t lower_bound_col(const int32_t* __restrict__ col, int64_t lo, int64_t hi, int64_t key) {
     while (lo < hi) {
         const int64_t mid = (lo + hi) >> 1;
@@ -185,55 +196,64 @@ __device__ __forceinline__ int64_t lower_bound_col(const int32_t* __restrict__ c
     return lo;
 }
 
-// largest i with off[i] <= t  (off is ascending, off[0] = 0, off[count] > t)
-__device__ __forceinline__ int64_t owner_of(const int64_t* __restrict__ off, int64_t count, int64_t t) {
-    int64_t lo = 0, hi = count;
-    while (hi - lo > 1) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (off[mid] <= t) lo = mid; else hi = mid;
+// The column blocks of one long row, a warp per row, 32 blocks at a time: f(block's first entry, its end, segments it
+// takes, segments of the row's blocks before it).  Returns the row's number of segments.
+template <typename F>
+__device__ __forceinline__ int64_t row_blocks(int64_t n_cols, int64_t rb, int64_t re, const int32_t* __restrict__ col, int seg, F f) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nb = (int64_t)1 << row_log_blocks(re - rb), width = (n_cols + nb - 1) / nb;
+    int64_t before = 0;
+    for (int64_t b0 = 0; b0 < nb; b0 += 32) {
+        const int64_t b = b0 + lane;
+        int64_t lo = re, hi = re;
+        if (b < nb) {
+            lo = lower_bound_col(col, rb, re, b * width);
+            hi = lower_bound_col(col, lo, re, (b + 1) * width);
+        }
+        const int64_t mine = (hi - lo + seg - 1) / seg;
+        int64_t incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        f(lo, hi, before + incl - mine);
+        before += __shfl_sync(0xFFFFFFFFu, incl, 31);
     }
-    return lo;
+    return before;
 }
 
-// One thread per (long row, column block) pair: the entries of the row inside the block and how many
-// segments they need.
-__global__ void pair_segments_kernel(int64_t n, int64_t n_long, int64_t total_pairs, const int32_t* __restrict__ perm,
-                                     const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                                     const int64_t* __restrict__ blk_off, int64_t* __restrict__ pair_lo,
-                                     int64_t* __restrict__ pair_cnt, int64_t* __restrict__ pair_segs, int seg) {
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t > total_pairs) return;
-    if (t == total_pairs) { pair_segs[t] = 0; return; }
-    const int64_t i = owner_of(blk_off, n_long, t);
-    const int64_t b = t - blk_off[i], nb = blk_off[i + 1] - blk_off[i];
-    const int64_t u = perm[i];
-    const int64_t rb = rowptr[u], re = rowptr[u + 1];
-    const int64_t width = (n + nb - 1) / nb;
-    const int64_t lo = lower_bound_col(col, rb, re, b * width);
-    const int64_t hi = lower_bound_col(col, lo, re, (b + 1) * width);
-    pair_lo[t] = lo;
-    pair_cnt[t] = hi - lo;
-    pair_segs[t] = (hi - lo + seg - 1) / seg;
+// row_segs[i] = segments of the i-th longest row, 0 for rows that are not cut; i <= cap (a bound of the number of long rows)
+__global__ void seg_count_kernel(int64_t n_cols, int64_t cap, const int32_t* __restrict__ perm, const int64_t* __restrict__ rowptr,
+                                 const int32_t* __restrict__ col, int seg, int64_t* __restrict__ row_segs, ScheduleCounts* counts) {
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (i > cap) return;
+    int64_t k = 0;
+    if (i < cap) {
+        const int64_t u = perm[i], rb = rowptr[u], re = rowptr[u + 1];
+        if (re - rb > seg) k = row_blocks(n_cols, rb, re, col, seg, [](int64_t, int64_t, int64_t) {});
+    }
+    if ((threadIdx.x & 31) == 0) {
+        row_segs[i] = k;
+        if (k) atomicAdd(&counts->total_segs, (unsigned long long)k);
+    }
 }
 
-__global__ void seg_fill_kernel(int64_t n_long, int64_t total_pairs, const int32_t* __restrict__ col,
-                                const int64_t* __restrict__ blk_off, const int64_t* __restrict__ pair_lo,
-                                const int64_t* __restrict__ pair_cnt, const int64_t* __restrict__ pair_seg_off,
-                                SpmmRec* __restrict__ rec_tmp, uint32_t* __restrict__ keys, uint32_t* __restrict__ ids,
-                                int64_t* __restrict__ seg_off, int seg) {
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= total_pairs) return;
-    const int64_t i = owner_of(blk_off, n_long, t);
-    if (t == blk_off[i]) seg_off[i] = pair_seg_off[t];
-    if (t == total_pairs - 1) seg_off[n_long] = pair_seg_off[total_pairs];
-    int64_t q = pair_seg_off[t];
-    const int64_t lo = pair_lo[t], hi = lo + pair_cnt[t];
-    for (int64_t pos = lo; pos < hi; pos += seg, ++q) {
-        SpmmRec x; x.begin = pos; x.len = (int32_t)((hi - pos) < seg ? (hi - pos) : seg); x.row = (int32_t)i;
-        rec_tmp[q] = x;
-        keys[q] = (uint32_t)col[pos];      // segments run in order of their first column
-        ids[q] = (uint32_t)q;
-    }
+__global__ void seg_fill_kernel(int64_t n_cols, int64_t n_long, const int32_t* __restrict__ perm, const int64_t* __restrict__ rowptr,
+                                const int32_t* __restrict__ col, int seg, const int64_t* __restrict__ seg_off,
+                                SpmmRec* __restrict__ rec_tmp, uint32_t* __restrict__ keys, uint32_t* __restrict__ ids) {
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (i >= n_long) return;
+    const int64_t u = perm[i], first = seg_off[i];
+    row_blocks(n_cols, rowptr[u], rowptr[u + 1], col, seg, [&](int64_t lo, int64_t hi, int64_t before) {
+        int64_t q = first + before;
+        for (int64_t pos = lo; pos < hi; pos += seg, ++q) {
+            SpmmRec x; x.begin = pos; x.len = (int32_t)((hi - pos) < seg ? (hi - pos) : seg); x.row = (int32_t)i;
+            rec_tmp[q] = x;
+            keys[q] = (uint32_t)col[pos];      // segments run in order of their first column
+            ids[q] = (uint32_t)q;
+        }
+    });
 }
 
 __global__ void seg_place_kernel(int64_t total_segs, const uint32_t* __restrict__ order, const SpmmRec* __restrict__ rec_tmp,
@@ -269,21 +289,16 @@ __global__ void validate_csr_kernel(int64_t n, int64_t nnz, const int64_t* __res
     }
 }
 
-struct DevBuf {  // frees on scope exit
-    void* p = nullptr;
-    ~DevBuf() { if (p) cudaFree(p); }
-    template <class T> T* as() { return reinterpret_cast<T*>(p); }
-};
-
 int bits_for(uint64_t x) { int b = 0; while (x) { ++b; x >>= 1; } return b; }
 
+// (these release memory that kernels on any stream may have used: callers synchronise the device first)
 void free_schedule(SpmmSchedule& v) {
-    cudaFree(v.perm); cudaFree(v.rec); cudaFree(v.seg_off); cudaFree(v.seg_pos);
+    dev_free(v.perm, nullptr); dev_free(v.rec, nullptr); dev_free(v.seg_off, nullptr); dev_free(v.seg_pos, nullptr);
     v = SpmmSchedule{};
 }
 
 void free_view(CsrView& v) {
-    cudaFree(v.rowptr); cudaFree(v.col); cudaFree(v.val);
+    dev_free(v.rowptr, nullptr); dev_free(v.col, nullptr); dev_free(v.val, nullptr);
     free_schedule(v.full);
     for (int k = 0; k < v.n_chunk; ++k) free_schedule(v.chunk[k]);
     delete[] v.chunk;
@@ -297,113 +312,96 @@ mixgcn_status build_schedule(int64_t n_total, int64_t nnz, const int64_t* rowptr
     v = SpmmSchedule{};
     v.row0 = row0; v.n_rows = n; v.seg = schedule_seg(nnz);
     if (n <= 0) return MIXGCN_OK;
-    DevBuf k0, k1, tmp, hub;
-    MIXGCN_CUDA(cudaMalloc(&k0.p, n * sizeof(uint64_t)));
-    MIXGCN_CUDA(cudaMalloc(&k1.p, n * sizeof(uint64_t)));
-    MIXGCN_CUDA(cudaMalloc(&hub.p, 5 * sizeof(unsigned long long)));
-    MIXGCN_CUDA(cudaMemsetAsync(hub.p, 0, 5 * sizeof(unsigned long long), s));
-    MIXGCN_CUDA(cudaMalloc((void**)&v.perm, n * sizeof(int32_t)));
-    schedule_keys_kernel<<<blocks_for(n), TPB, 0, s>>>(row0, n, rowptr, k0.as<uint64_t>());
+    // rows by descending entry count; the bucket counts; the segments each long row will need
+    const int deg_bits = bits_for((uint64_t)n_total);                      // a row has at most n_total entries
+    const uint32_t top = (uint32_t)(((uint64_t)1 << deg_bits) - 1);
+    int64_t cap = nnz / (v.seg + 1);                                       // no more rows than this are long
+    if (cap > n) cap = n;
+    DevBuf k0(s), k1(s), ids(s), tmp(s), counts(s), row_segs(s);
+    MIXGCN_TRY(k0.alloc(n * (int64_t)sizeof(uint32_t)));
+    MIXGCN_TRY(k1.alloc(n * (int64_t)sizeof(uint32_t)));
+    MIXGCN_TRY(ids.alloc(n * (int64_t)sizeof(int32_t)));
+    MIXGCN_TRY(counts.alloc(sizeof(ScheduleCounts)));
+    MIXGCN_TRY(row_segs.alloc((cap + 1) * (int64_t)sizeof(int64_t)));
+    MIXGCN_TRY(dev_alloc((void**)&v.perm, n * (int64_t)sizeof(int32_t), s));
+    MIXGCN_CUDA(cudaMemsetAsync(counts.p, 0, sizeof(ScheduleCounts), s));
+    schedule_keys_kernel<<<blocks_for(n), TPB, 0, s>>>(row0, n, top, rowptr, k0.as<uint32_t>(), ids.as<int32_t>());
     size_t tb = 0;
-    MIXGCN_CUDA(cub::DeviceRadixSort::SortKeys(nullptr, tb, k0.as<uint64_t>(), k1.as<uint64_t>(), n, 0, 64, s));
-    MIXGCN_CUDA(cudaMalloc(&tmp.p, tb ? tb : 1));
-    MIXGCN_CUDA(cub::DeviceRadixSort::SortKeys(tmp.p, tb, k0.as<uint64_t>(), k1.as<uint64_t>(), n, 0, 64, s));
-    schedule_finish_kernel<<<blocks_for(n), TPB, 0, s>>>(n, k1.as<uint64_t>(), v.perm, v.seg, hub.as<unsigned long long>());
-    unsigned long long h[5] = {0, 0, 0, 0, 0};
-    uint64_t first = 0;
-    MIXGCN_CUDA(cudaMemcpyAsync(h, hub.p, sizeof(h), cudaMemcpyDeviceToHost, s));
-    MIXGCN_CUDA(cudaMemcpyAsync(&first, k1.p, sizeof(first), cudaMemcpyDeviceToHost, s));
+    MIXGCN_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, tb, k0.as<uint32_t>(), k1.as<uint32_t>(), ids.as<int32_t>(), v.perm, n, 0, deg_bits, s));
+    MIXGCN_TRY(tmp.alloc((int64_t)tb));
+    MIXGCN_CUDA(cub::DeviceRadixSort::SortPairs(tmp.p, tb, k0.as<uint32_t>(), k1.as<uint32_t>(), ids.as<int32_t>(), v.perm, n, 0, deg_bits, s));
+    schedule_counts_kernel<<<blocks_for(n), TPB, 0, s>>>(n, top, k1.as<uint32_t>(), v.seg, counts.as<ScheduleCounts>());
+    if (cap > 0)
+        seg_count_kernel<<<blocks_for((cap + 1) * 32), TPB, 0, s>>>(n_total, cap, v.perm, rowptr, col, v.seg, row_segs.as<int64_t>(), counts.as<ScheduleCounts>());
+    ScheduleCounts h{};
+    MIXGCN_CUDA(cudaMemcpyAsync(&h, counts.p, sizeof(h), cudaMemcpyDeviceToHost, s));
     MIXGCN_CUDA(cudaStreamSynchronize(s));
-    v.n_long = (int64_t)h[0];
-    v.n_heavy = (int64_t)h[4];
-    for (int q = 0; q < 3; ++q) v.rows_above[q] = (int64_t)h[q + 1];
-    v.max_deg = (int32_t)(0x7FFFFFFFull - (first >> 32));
-    // long rows -> (row, column block) pairs -> segments, ordered by their first column
-    const int64_t nl = v.n_long;
-    DevBuf nblk, blk_off, tmp2;
-    MIXGCN_CUDA(cudaMalloc(&nblk.p, (nl + 1) * sizeof(int64_t)));
-    MIXGCN_CUDA(cudaMalloc(&blk_off.p, (nl + 1) * sizeof(int64_t)));
-    MIXGCN_CUDA(cudaMalloc((void**)&v.seg_off, (nl + 1) * sizeof(int64_t)));
-    MIXGCN_CUDA(cudaMemsetAsync(v.seg_off, 0, (nl + 1) * sizeof(int64_t), s));
-    blk_count_kernel<<<blocks_for(nl + 1), TPB, 0, s>>>(nl, v.perm, rowptr, nblk.as<int64_t>());
-    size_t tb2 = 0;
-    MIXGCN_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tb2, nblk.as<int64_t>(), blk_off.as<int64_t>(), nl + 1, s));
-    MIXGCN_CUDA(cudaMalloc(&tmp2.p, tb2 ? tb2 : 1));
-    MIXGCN_CUDA(cub::DeviceScan::ExclusiveSum(tmp2.p, tb2, nblk.as<int64_t>(), blk_off.as<int64_t>(), nl + 1, s));
-    int64_t total_pairs = 0;
-    MIXGCN_CUDA(cudaMemcpyAsync(&total_pairs, blk_off.as<int64_t>() + nl, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    MIXGCN_CUDA(cudaStreamSynchronize(s));
-    int64_t total = 0;
-    DevBuf pair_lo, pair_cnt, pair_segs, pair_seg_off, tmp3, rec_tmp, keys0, keys1, ids0, ids1, tmp4;
-    if (total_pairs > 0) {
-        MIXGCN_CUDA(cudaMalloc(&pair_lo.p, total_pairs * sizeof(int64_t)));
-        MIXGCN_CUDA(cudaMalloc(&pair_cnt.p, total_pairs * sizeof(int64_t)));
-        MIXGCN_CUDA(cudaMalloc(&pair_segs.p, (total_pairs + 1) * sizeof(int64_t)));
-        MIXGCN_CUDA(cudaMalloc(&pair_seg_off.p, (total_pairs + 1) * sizeof(int64_t)));
-        pair_segments_kernel<<<blocks_for(total_pairs + 1), TPB, 0, s>>>(n_total, nl, total_pairs, v.perm, rowptr, col,
-                                                                        blk_off.as<int64_t>(), pair_lo.as<int64_t>(),
-                                                                        pair_cnt.as<int64_t>(), pair_segs.as<int64_t>(), v.seg);
-        size_t tb3 = 0;
-        MIXGCN_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tb3, pair_segs.as<int64_t>(), pair_seg_off.as<int64_t>(), total_pairs + 1, s));
-        MIXGCN_CUDA(cudaMalloc(&tmp3.p, tb3 ? tb3 : 1));
-        MIXGCN_CUDA(cub::DeviceScan::ExclusiveSum(tmp3.p, tb3, pair_segs.as<int64_t>(), pair_seg_off.as<int64_t>(), total_pairs + 1, s));
-        MIXGCN_CUDA(cudaMemcpyAsync(&total, pair_seg_off.as<int64_t>() + total_pairs, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-        MIXGCN_CUDA(cudaStreamSynchronize(s));
-    }
+    v.n_long = (int64_t)h.rows_above_seg;
+    v.n_heavy = (int64_t)h.rows_heavy;
+    for (int q = 0; q < 3; ++q) v.rows_above[q] = (int64_t)h.rows_above[q];
+    v.max_deg = (int32_t)h.max_deg;
+    const int64_t nl = v.n_long, total = (int64_t)h.total_segs;
     if (total >= 0xFFFFFFFFll) MIXGCN_FAIL(MIXGCN_EUNSUPPORTED, "graph schedule: too many long-row segments (%lld)", (long long)total);
     v.total_segs = total;
-    MIXGCN_CUDA(cudaMalloc((void**)&v.rec, (size_t)(total + n - nl + 1) * sizeof(SpmmRec)));
-    MIXGCN_CUDA(cudaMalloc((void**)&v.seg_pos, (size_t)(total + 1) * sizeof(int64_t)));
+    MIXGCN_TRY(dev_alloc((void**)&v.seg_off, (nl + 1) * (int64_t)sizeof(int64_t), s));
+    MIXGCN_TRY(dev_alloc((void**)&v.rec, (total + n - nl + 1) * (int64_t)sizeof(SpmmRec), s));
+    MIXGCN_TRY(dev_alloc((void**)&v.seg_pos, (total + 1) * (int64_t)sizeof(int64_t), s));
     if (total > 0) {
-        MIXGCN_CUDA(cudaMalloc(&rec_tmp.p, total * sizeof(SpmmRec)));
-        MIXGCN_CUDA(cudaMalloc(&keys0.p, total * sizeof(uint32_t)));
-        MIXGCN_CUDA(cudaMalloc(&keys1.p, total * sizeof(uint32_t)));
-        MIXGCN_CUDA(cudaMalloc(&ids0.p, total * sizeof(uint32_t)));
-        MIXGCN_CUDA(cudaMalloc(&ids1.p, total * sizeof(uint32_t)));
-        seg_fill_kernel<<<blocks_for(total_pairs), TPB, 0, s>>>(nl, total_pairs, col, blk_off.as<int64_t>(), pair_lo.as<int64_t>(),
-                                                               pair_cnt.as<int64_t>(), pair_seg_off.as<int64_t>(),
-                                                               rec_tmp.as<SpmmRec>(), keys0.as<uint32_t>(), ids0.as<uint32_t>(),
-                                                               v.seg_off, v.seg);
-        size_t tb4 = 0;
-        MIXGCN_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, tb4, keys0.as<uint32_t>(), keys1.as<uint32_t>(), ids0.as<uint32_t>(),
-                                                    ids1.as<uint32_t>(), total, 0, 32, s));
-        MIXGCN_CUDA(cudaMalloc(&tmp4.p, tb4 ? tb4 : 1));
-        MIXGCN_CUDA(cub::DeviceRadixSort::SortPairs(tmp4.p, tb4, keys0.as<uint32_t>(), keys1.as<uint32_t>(), ids0.as<uint32_t>(),
-                                                    ids1.as<uint32_t>(), total, 0, 32, s));
+        // segments of the long rows, in order of their first column
+        DevBuf rec_tmp(s), keys0(s), keys1(s), ids0(s), ids1(s), tmp2(s);
+        MIXGCN_TRY(rec_tmp.alloc(total * (int64_t)sizeof(SpmmRec)));
+        MIXGCN_TRY(keys0.alloc(total * (int64_t)sizeof(uint32_t)));
+        MIXGCN_TRY(keys1.alloc(total * (int64_t)sizeof(uint32_t)));
+        MIXGCN_TRY(ids0.alloc(total * (int64_t)sizeof(uint32_t)));
+        MIXGCN_TRY(ids1.alloc(total * (int64_t)sizeof(uint32_t)));
+        const int col_bits = bits_for((uint64_t)n_total);
+        size_t tb_scan = 0, tb_sort = 0;
+        MIXGCN_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tb_scan, row_segs.as<int64_t>(), v.seg_off, nl + 1, s));
+        MIXGCN_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, tb_sort, keys0.as<uint32_t>(), keys1.as<uint32_t>(), ids0.as<uint32_t>(),
+                                                    ids1.as<uint32_t>(), total, 0, col_bits, s));
+        size_t tb2 = tb_scan > tb_sort ? tb_scan : tb_sort;
+        MIXGCN_TRY(tmp2.alloc((int64_t)tb2));
+        MIXGCN_CUDA(cub::DeviceScan::ExclusiveSum(tmp2.p, tb2, row_segs.as<int64_t>(), v.seg_off, nl + 1, s));
+        seg_fill_kernel<<<blocks_for(nl * 32), TPB, 0, s>>>(n_total, nl, v.perm, rowptr, col, v.seg, v.seg_off, rec_tmp.as<SpmmRec>(),
+                                                           keys0.as<uint32_t>(), ids0.as<uint32_t>());
+        MIXGCN_CUDA(cub::DeviceRadixSort::SortPairs(tmp2.p, tb2, keys0.as<uint32_t>(), keys1.as<uint32_t>(), ids0.as<uint32_t>(),
+                                                    ids1.as<uint32_t>(), total, 0, col_bits, s));
         seg_place_kernel<<<blocks_for(total), TPB, 0, s>>>(total, ids1.as<uint32_t>(), rec_tmp.as<SpmmRec>(), v.rec, v.seg_pos);
+    } else {
+        MIXGCN_CUDA(cudaMemsetAsync(v.seg_off, 0, (nl + 1) * sizeof(int64_t), s));
     }
     fill_records_kernel<<<blocks_for(n), TPB, 0, s>>>(n, nl, total, v.perm, rowptr, v.rec);
-    MIXGCN_CUDA(cudaStreamSynchronize(s));
     MIXGCN_CUDA(cudaGetLastError());
     return MIXGCN_OK;
 }
 
-// Everything after rowptr/col exist: degrees, values, symmetry, transpose, schedules.
-mixgcn_status finish_graph(mixgcn_graph* g, cudaStream_t s) {
+// Degrees and room for the values of a graph whose rowptr exists.
+mixgcn_status fill_degrees(mixgcn_graph* g, cudaStream_t s) {
+    MIXGCN_TRY(dev_alloc((void**)&g->deg, g->n * (int64_t)sizeof(int32_t), s));
+    MIXGCN_TRY(dev_alloc((void**)&g->dinv, g->n * (int64_t)sizeof(float), s));
+    MIXGCN_TRY(dev_alloc((void**)&g->fwd.val, (g->nnz > 0 ? g->nnz : 1) * (int64_t)sizeof(float), s));
+    degree_kernel<<<blocks_for(g->n), TPB, 0, s>>>(g->n, g->fwd.rowptr, g->deg, g->dinv);
+    return MIXGCN_OK;
+}
+
+// Everything after the CSR exists: symmetry, transpose, schedules.  known_symmetric / known_diagonal:
+// what the caller already knows of the structure (-1: look).  Leaves work in flight on `s`.
+mixgcn_status finish_graph(mixgcn_graph* g, int known_symmetric, int known_diagonal, cudaStream_t s) {
     const int64_t n = g->n, nnz = g->nnz;
     CsrView& A = g->fwd;
-    DevBuf flags;
-    MIXGCN_CUDA(cudaMalloc(&flags.p, sizeof(int32_t)));
-    MIXGCN_CUDA(cudaMemsetAsync(flags.p, 0, sizeof(int32_t), s));
-    MIXGCN_CUDA(cudaMalloc((void**)&g->deg, n * sizeof(int32_t)));
-    MIXGCN_CUDA(cudaMalloc((void**)&g->dinv, n * sizeof(float)));
-    MIXGCN_CUDA(cudaMalloc((void**)&A.val, (nnz > 0 ? nnz : 1) * sizeof(float)));
-    degree_kernel<<<blocks_for(n), TPB, 0, s>>>(n, A.rowptr, g->deg, g->dinv);
-    values_kernel<<<blocks_for(n * 32), TPB, 0, s>>>(n, A.rowptr, A.col, g->dinv, g->norm, A.val);
-    symmetry_kernel<<<blocks_for(n * 32), TPB, 0, s>>>(n, A.rowptr, A.col, flags.as<int32_t>());
-    int32_t hf = 0;
-    MIXGCN_CUDA(cudaMemcpyAsync(&hf, flags.p, sizeof(hf), cudaMemcpyDeviceToHost, s));
-    MIXGCN_CUDA(cudaStreamSynchronize(s));
-    g->symmetric = (hf & F_NOT_SYMMETRIC) ? 0 : 1;
-    {
-        DevBuf dc;
-        MIXGCN_CUDA(cudaMalloc(&dc.p, sizeof(unsigned long long)));
-        MIXGCN_CUDA(cudaMemsetAsync(dc.p, 0, sizeof(unsigned long long), s));
-        diagonal_count_kernel<<<blocks_for(n), TPB, 0, s>>>(n, A.rowptr, A.col, dc.as<unsigned long long>());
-        unsigned long long hd = 0;
-        MIXGCN_CUDA(cudaMemcpyAsync(&hd, dc.p, sizeof(hd), cudaMemcpyDeviceToHost, s));
+    g->symmetric = known_symmetric; g->has_diagonal = known_diagonal;
+    if (known_symmetric < 0 || known_diagonal < 0) {
+        struct Looked { unsigned long long diagonal; int32_t flags; } h{};
+        DevBuf looked(s);
+        MIXGCN_TRY(looked.alloc(sizeof(Looked)));
+        MIXGCN_CUDA(cudaMemsetAsync(looked.p, 0, sizeof(Looked), s));
+        Looked* d = looked.as<Looked>();
+        if (known_symmetric < 0) symmetry_kernel<<<blocks_for(n * 32), TPB, 0, s>>>(n, A.rowptr, A.col, &d->flags);
+        if (known_diagonal < 0) diagonal_count_kernel<<<blocks_for(n), TPB, 0, s>>>(n, A.rowptr, A.col, &d->diagonal);
+        MIXGCN_CUDA(cudaMemcpyAsync(&h, looked.p, sizeof(h), cudaMemcpyDeviceToHost, s));
         MIXGCN_CUDA(cudaStreamSynchronize(s));
-        g->has_diagonal = hd == (unsigned long long)n ? 1 : (hd == 0 ? 0 : 2);
+        if (known_symmetric < 0) g->symmetric = (h.flags & F_NOT_SYMMETRIC) ? 0 : 1;
+        if (known_diagonal < 0) g->has_diagonal = h.diagonal == (unsigned long long)n ? 1 : (h.diagonal == 0 ? 0 : 2);
     }
     MIXGCN_TRY(build_schedule(n, nnz, A.rowptr, A.col, 0, n, A.full, s));
     g->bwd_is_fwd = (g->symmetric && g->norm != 1) ? 1 : 0;   // row-mean values are not symmetric: A_hat^T needs its own copy
@@ -413,24 +411,58 @@ mixgcn_status finish_graph(mixgcn_graph* g, cudaStream_t s) {
     }
     // Transposed structure: sort (col,row) keys carrying the value.
     CsrView& T = g->bwd;
-    DevBuf k0, k1, v1, tmp;
+    DevBuf k0(s), k1(s), tmp(s);
     const int64_t cap = nnz > 0 ? nnz : 1;
-    MIXGCN_CUDA(cudaMalloc(&k0.p, cap * sizeof(uint64_t)));
-    MIXGCN_CUDA(cudaMalloc(&k1.p, cap * sizeof(uint64_t)));
-    MIXGCN_CUDA(cudaMalloc((void**)&T.val, cap * sizeof(float)));
-    MIXGCN_CUDA(cudaMalloc((void**)&T.rowptr, (n + 1) * sizeof(int64_t)));
-    MIXGCN_CUDA(cudaMalloc((void**)&T.col, cap * sizeof(int32_t)));
-    transpose_keys_kernel<<<blocks_for(n * 32), TPB, 0, s>>>(n, A.rowptr, A.col, k0.as<uint64_t>());
+    MIXGCN_TRY(k0.alloc(cap * (int64_t)sizeof(uint64_t)));
+    MIXGCN_TRY(k1.alloc(cap * (int64_t)sizeof(uint64_t)));
+    MIXGCN_TRY(dev_alloc((void**)&T.val, cap * (int64_t)sizeof(float), s));
+    MIXGCN_TRY(dev_alloc((void**)&T.rowptr, (n + 1) * (int64_t)sizeof(int64_t), s));
+    MIXGCN_TRY(dev_alloc((void**)&T.col, cap * (int64_t)sizeof(int32_t), s));
+    const int shift = bits_for((uint64_t)n);
+    transpose_keys_kernel<<<blocks_for(n * 32), TPB, 0, s>>>(n, shift, A.rowptr, A.col, k0.as<uint64_t>());
     size_t tb = 0;
-    const int end_bit = 32 + bits_for((uint64_t)n);
     MIXGCN_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, tb, k0.as<uint64_t>(), k1.as<uint64_t>(), A.val, T.val,
-                                                nnz, 0, end_bit, s));
-    MIXGCN_CUDA(cudaMalloc(&tmp.p, tb ? tb : 1));
+                                                nnz, shift, 2 * shift, s));
+    MIXGCN_TRY(tmp.alloc((int64_t)tb));
+    // the keys are made in row order and the sort is stable: sorting by the column part leaves the rows ascending
     MIXGCN_CUDA(cub::DeviceRadixSort::SortPairs(tmp.p, tb, k0.as<uint64_t>(), k1.as<uint64_t>(), A.val, T.val,
-                                                nnz, 0, end_bit, s));
-    rowptr_from_keys_kernel<<<blocks_for(nnz + 1), TPB, 0, s>>>(n, nnz, k1.as<uint64_t>(), T.rowptr, T.col);
+                                                nnz, shift, 2 * shift, s));
+    rowptr_from_keys_kernel<uint64_t><<<blocks_for(nnz + 1), TPB, 0, s>>>(n, nnz, shift, k1.as<uint64_t>(), T.rowptr, T.col);
+    return build_schedule(n, nnz, T.rowptr, T.col, 0, n, T.full, s);
+}
+
+// Edge list (on the device) -> CSR of the graph: keys, sort, unique, values.
+template <typename Key>
+mixgcn_status csr_from_edges(mixgcn_graph* g, int64_t m, const int32_t* src, const int32_t* dst, int sym, int self, cudaStream_t s) {
+    const int64_t n = g->n, total = m * (sym ? 2 : 1) + (self ? n : 0);
+    struct Counted { int64_t unique; int32_t flags; } h{};
+    DevBuf k0(s), k1(s), tmp(s), counted(s);
+    MIXGCN_TRY(k0.alloc(total * (int64_t)sizeof(Key)));
+    MIXGCN_TRY(k1.alloc(total * (int64_t)sizeof(Key)));
+    MIXGCN_TRY(counted.alloc(sizeof(Counted)));
+    Counted* d = counted.as<Counted>();
+    MIXGCN_CUDA(cudaMemsetAsync(d, 0, sizeof(Counted), s));
+    const int shift = bits_for((uint64_t)n);
+    const int64_t work = m > n ? m : n;
+    make_keys_kernel<Key><<<blocks_for(work), TPB, 0, s>>>(n, m, src, dst, sym, self, shift, k0.as<Key>(), &d->flags);
+    size_t tb_sort = 0, tb_uniq = 0;
+    MIXGCN_CUDA(cub::DeviceRadixSort::SortKeys(nullptr, tb_sort, k0.as<Key>(), k1.as<Key>(), total, 0, 2 * shift, s));
+    MIXGCN_CUDA(cub::DeviceSelect::Unique(nullptr, tb_uniq, k1.as<Key>(), k0.as<Key>(), &d->unique, total, s));
+    size_t tb = tb_sort > tb_uniq ? tb_sort : tb_uniq;
+    MIXGCN_TRY(tmp.alloc((int64_t)tb));
+    MIXGCN_CUDA(cub::DeviceRadixSort::SortKeys(tmp.p, tb, k0.as<Key>(), k1.as<Key>(), total, 0, 2 * shift, s));
+    MIXGCN_CUDA(cub::DeviceSelect::Unique(tmp.p, tb, k1.as<Key>(), k0.as<Key>(), &d->unique, total, s));
+    MIXGCN_CUDA(cudaMemcpyAsync(&h, d, sizeof(h), cudaMemcpyDeviceToHost, s));
     MIXGCN_CUDA(cudaStreamSynchronize(s));
-    MIXGCN_TRY(build_schedule(n, nnz, T.rowptr, T.col, 0, n, T.full, s));
+    if (h.flags & F_BAD_ID) MIXGCN_FAIL(MIXGCN_EBADGRAPH, "graph_create: a node id lies outside [0, %lld)", (long long)n);
+    const int64_t nnz = total == 0 ? 0 : h.unique - ((h.flags & F_DROPPED) ? 1 : 0);     // dropped edges left one sentinel, the last key
+    g->nnz = nnz;
+    MIXGCN_TRY(dev_alloc((void**)&g->fwd.rowptr, (n + 1) * (int64_t)sizeof(int64_t), s));
+    MIXGCN_TRY(dev_alloc((void**)&g->fwd.col, (nnz > 0 ? nnz : 1) * (int64_t)sizeof(int32_t), s));
+    rowptr_from_keys_kernel<Key><<<blocks_for(nnz + 1), TPB, 0, s>>>(n, nnz, shift, k0.as<Key>(), g->fwd.rowptr, g->fwd.col);
+    MIXGCN_TRY(fill_degrees(g, s));
+    if (nnz > 0) values_from_keys_kernel<Key><<<blocks_for(nnz), TPB, 0, s>>>(nnz, shift, k0.as<Key>(), g->deg, g->dinv, g->norm, g->fwd.val);
+    MIXGCN_CUDA(cudaGetLastError());
     return MIXGCN_OK;
 }
 
@@ -465,6 +497,7 @@ mixgcn_status ensure_chunk_schedules(const mixgcn_graph* g, const CsrView& A_con
     for (int k = 0; k < chunks; ++k) {
         const int64_t r0 = (g->n * (int64_t)k) / chunks, r1 = (g->n * (int64_t)(k + 1)) / chunks;
         mixgcn_status st = build_schedule(g->n, g->nnz, A.rowptr, A.col, r0, r1 - r0, sc[k], s);
+        if (st == MIXGCN_OK && cudaStreamSynchronize(s) != cudaSuccess) st = MIXGCN_ECUDA;    // usable on every stream from here on
         if (st != MIXGCN_OK) {
             for (int q = 0; q <= k; ++q) free_schedule(sc[q]);
             delete[] sc;
@@ -481,10 +514,11 @@ mixgcn_status ensure_chunk_schedules(const mixgcn_graph* g, const CsrView& A_con
 extern "C" mixgcn_status mixgcn_graph_destroy(mixgcn_graph* g) {
     if (!g) return MIXGCN_OK;
     cudaSetDevice(g->device);
+    cudaDeviceSynchronize();          // launches that read the graph may still be in flight on any stream
     if (!g->bwd_is_fwd) free_view(g->bwd);
     free_view(g->fwd);
-    cudaFree(g->deg);
-    cudaFree(g->dinv);
+    dev_free(g->deg, nullptr);
+    dev_free(g->dinv, nullptr);
     delete g;
     return MIXGCN_OK;
 }
@@ -497,7 +531,6 @@ extern "C" mixgcn_status mixgcn_graph_create(mixgcn_ctx* ctx, int64_t n, int64_t
     cudaStream_t s = ctx->side_stream[0];
     if ((flags & MIXGCN_GRAPH_NORM_ROW) && (flags & MIXGCN_GRAPH_NORM_NONE)) MIXGCN_FAIL(MIXGCN_EINVAL, "graph_create: NORM_ROW and NORM_NONE exclude each other");
     const int sym = (flags & MIXGCN_GRAPH_SYMMETRISE) != 0, self = (flags & MIXGCN_GRAPH_ADD_SELF_LOOPS) != 0;
-    const int64_t total = m * (sym ? 2 : 1) + (self ? n : 0);
 
     mixgcn_graph* g = new (std::nothrow) mixgcn_graph();
     if (g) g->uid = next_graph_uid();
@@ -507,58 +540,22 @@ extern "C" mixgcn_status mixgcn_graph_create(mixgcn_ctx* ctx, int64_t n, int64_t
     struct Guard { mixgcn_graph* g; bool keep = false; ~Guard() { if (!keep) { g->bwd_is_fwd = g->bwd.rowptr == g->fwd.rowptr; mixgcn_graph_destroy(g); } } } guard{g};
     LaunchScope scope(ctx, PH_GRAPH, s, 12);
 
-    DevBuf dsrc, ddst, k0, k1, tmp, fl, cnt;
+    DevBuf dsrc(s), ddst(s);
     const int32_t *ps = src, *pd = dst;
     if (!(flags & MIXGCN_GRAPH_EDGES_ON_DEVICE) && m > 0) {
-        MIXGCN_CUDA(cudaMalloc(&dsrc.p, m * sizeof(int32_t)));
-        MIXGCN_CUDA(cudaMalloc(&ddst.p, m * sizeof(int32_t)));
+        MIXGCN_TRY(dsrc.alloc(m * (int64_t)sizeof(int32_t)));
+        MIXGCN_TRY(ddst.alloc(m * (int64_t)sizeof(int32_t)));
         MIXGCN_CUDA(cudaMemcpyAsync(dsrc.p, src, m * sizeof(int32_t), cudaMemcpyHostToDevice, s));
         MIXGCN_CUDA(cudaMemcpyAsync(ddst.p, dst, m * sizeof(int32_t), cudaMemcpyHostToDevice, s));
         ps = dsrc.as<int32_t>(); pd = ddst.as<int32_t>();
     }
-    const int64_t cap = total > 0 ? total : 1;
-    MIXGCN_CUDA(cudaMalloc(&k0.p, cap * sizeof(uint64_t)));
-    MIXGCN_CUDA(cudaMalloc(&k1.p, cap * sizeof(uint64_t)));
-    MIXGCN_CUDA(cudaMalloc(&fl.p, sizeof(int32_t)));
-    MIXGCN_CUDA(cudaMalloc(&cnt.p, sizeof(int64_t)));
-    MIXGCN_CUDA(cudaMemsetAsync(fl.p, 0, sizeof(int32_t), s));
-    const uint64_t sentinel = (uint64_t)n << 32;  // sorts after every valid key
-    {
-        int64_t work = m > n ? m : n;
-        make_keys_kernel<<<blocks_for(work > 0 ? work : 1), TPB, 0, s>>>(n, m, ps, pd, sym, self, sentinel,
-                                                                        k0.as<uint64_t>(), fl.as<int32_t>());
-    }
-    const int end_bit = 32 + bits_for((uint64_t)n);
-    size_t tb_sort = 0, tb_uniq = 0;
-    MIXGCN_CUDA(cub::DeviceRadixSort::SortKeys(nullptr, tb_sort, k0.as<uint64_t>(), k1.as<uint64_t>(), total, 0, end_bit, s));
-    MIXGCN_CUDA(cub::DeviceSelect::Unique(nullptr, tb_uniq, k1.as<uint64_t>(), k0.as<uint64_t>(), cnt.as<int64_t>(), total, s));
-    size_t tb = tb_sort > tb_uniq ? tb_sort : tb_uniq;
-    MIXGCN_CUDA(cudaMalloc(&tmp.p, tb ? tb : 1));
-    MIXGCN_CUDA(cub::DeviceRadixSort::SortKeys(tmp.p, tb, k0.as<uint64_t>(), k1.as<uint64_t>(), total, 0, end_bit, s));
-    // edge arrays are no longer needed
-    MIXGCN_CUDA(cub::DeviceSelect::Unique(tmp.p, tb, k1.as<uint64_t>(), k0.as<uint64_t>(), cnt.as<int64_t>(), total, s));
-    int64_t n_unique = 0;
-    int32_t hf = 0;
-    MIXGCN_CUDA(cudaMemcpyAsync(&n_unique, cnt.p, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    MIXGCN_CUDA(cudaMemcpyAsync(&hf, fl.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    // two ids fit one 32-bit key on graphs of fewer than 2^16 nodes: half the bytes per radix pass
+    if (2 * bits_for((uint64_t)n) <= 32) MIXGCN_TRY(csr_from_edges<uint32_t>(g, m, ps, pd, sym, self, s));
+    else MIXGCN_TRY(csr_from_edges<uint64_t>(g, m, ps, pd, sym, self, s));
+    dsrc.release(); ddst.release();
+    // self loops of the input are dropped, so the flags decide what lies on the diagonal; a directed list may still be symmetric
+    MIXGCN_TRY(finish_graph(g, sym ? 1 : -1, self ? 1 : 0, s));
     MIXGCN_CUDA(cudaStreamSynchronize(s));
-    if (hf & F_BAD_ID) MIXGCN_FAIL(MIXGCN_EBADGRAPH, "graph_create: a node id lies outside [0, %lld)", (long long)n);
-    if (total == 0) n_unique = 0;
-    if (n_unique > 0) {
-        uint64_t last = 0;
-        MIXGCN_CUDA(cudaMemcpy(&last, k0.as<uint64_t>() + (n_unique - 1), sizeof(last), cudaMemcpyDeviceToHost));
-        if (last == sentinel) --n_unique;
-    }
-    g->nnz = n_unique;
-    cudaFree(k1.p); k1.p = nullptr;
-    cudaFree(tmp.p); tmp.p = nullptr;
-    MIXGCN_CUDA(cudaMalloc((void**)&g->fwd.rowptr, (n + 1) * sizeof(int64_t)));
-    MIXGCN_CUDA(cudaMalloc((void**)&g->fwd.col, (n_unique > 0 ? n_unique : 1) * sizeof(int32_t)));
-    rowptr_from_keys_kernel<<<blocks_for(n_unique + 1), TPB, 0, s>>>(n, n_unique, k0.as<uint64_t>(), g->fwd.rowptr, g->fwd.col);
-    MIXGCN_CUDA(cudaStreamSynchronize(s));
-    cudaFree(k0.p); k0.p = nullptr;
-    MIXGCN_TRY(finish_graph(g, s));
-    MIXGCN_CUDA(cudaGetLastError());
     guard.keep = true;
     *out = g;
     return MIXGCN_OK;
@@ -584,11 +581,11 @@ extern "C" mixgcn_status mixgcn_graph_create_from_csr(mixgcn_ctx* ctx, int64_t n
     g->norm = (flags & MIXGCN_GRAPH_NORM_ROW) ? 1 : ((flags & MIXGCN_GRAPH_NORM_NONE) ? 2 : 0);
     struct Guard { mixgcn_graph* g; bool keep = false; ~Guard() { if (!keep) { g->bwd_is_fwd = g->bwd.rowptr == g->fwd.rowptr; mixgcn_graph_destroy(g); } } } guard{g};
     LaunchScope scope(ctx, PH_GRAPH, s, 8);
-    DevBuf fl;
-    MIXGCN_CUDA(cudaMalloc(&fl.p, sizeof(int32_t)));
+    DevBuf fl(s);
+    MIXGCN_TRY(fl.alloc(sizeof(int32_t)));
     MIXGCN_CUDA(cudaMemsetAsync(fl.p, 0, sizeof(int32_t), s));
-    MIXGCN_CUDA(cudaMalloc((void**)&g->fwd.rowptr, (n + 1) * sizeof(int64_t)));
-    MIXGCN_CUDA(cudaMalloc((void**)&g->fwd.col, (nnz > 0 ? nnz : 1) * sizeof(int32_t)));
+    MIXGCN_TRY(dev_alloc((void**)&g->fwd.rowptr, (n + 1) * (int64_t)sizeof(int64_t), s));
+    MIXGCN_TRY(dev_alloc((void**)&g->fwd.col, (nnz > 0 ? nnz : 1) * (int64_t)sizeof(int32_t), s));
     MIXGCN_CUDA(cudaMemcpyAsync(g->fwd.rowptr, rowptr, (n + 1) * sizeof(int64_t), kind, s));
     if (nnz > 0) MIXGCN_CUDA(cudaMemcpyAsync(g->fwd.col, col, nnz * sizeof(int32_t), kind, s));
     // rowptr must be validated before col is indexed with it: first monotonicity on the host side
@@ -600,8 +597,10 @@ extern "C" mixgcn_status mixgcn_graph_create_from_csr(mixgcn_ctx* ctx, int64_t n
     if (hf & F_BAD_ROWPTR) MIXGCN_FAIL(MIXGCN_EBADGRAPH, "graph_create_from_csr: rowptr is not monotone from 0");
     if (hf & F_BAD_ID) MIXGCN_FAIL(MIXGCN_EBADGRAPH, "graph_create_from_csr: a column id lies outside [0, %lld)", (long long)n);
     if (hf & F_UNSORTED) MIXGCN_FAIL(MIXGCN_EBADGRAPH, "graph_create_from_csr: columns are not strictly ascending in a row");
-    MIXGCN_TRY(finish_graph(g, s));
-    MIXGCN_CUDA(cudaGetLastError());
+    MIXGCN_TRY(fill_degrees(g, s));
+    values_kernel<<<blocks_for(n * 32), TPB, 0, s>>>(n, g->fwd.rowptr, g->fwd.col, g->dinv, g->norm, g->fwd.val);
+    MIXGCN_TRY(finish_graph(g, -1, -1, s));
+    MIXGCN_CUDA(cudaStreamSynchronize(s));
     guard.keep = true;
     *out = g;
     return MIXGCN_OK;

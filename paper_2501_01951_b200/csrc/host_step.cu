@@ -122,7 +122,7 @@ void free_step_cache(mixgcn_ctx* ctx) {
     HostStepCache* c = ctx->step_cache;
     if (!c) return;
     drop_plans(c);
-    cudaFree(c->mask);
+    dev_free(c->mask, nullptr);
     delete c;
     ctx->step_cache = nullptr;
 }
@@ -152,14 +152,8 @@ extern "C" mixgcn_status mixgcn_train_step_host(mixgcn_ctx* ctx, const mixgcn_gr
     if (lo.bytes > ctx->arena_bytes) {
         MIXGCN_CUDA(cudaDeviceSynchronize());
         if (pf) pf->in_flight = nullptr;        // the buffer a prefetch went to is gone
-        cudaFree(ctx->arena); ctx->arena = nullptr; ctx->arena_bytes = 0;
-        void* p = nullptr;
-        if (cudaMalloc(&p, (size_t)lo.bytes) != cudaSuccess) {
-            cudaGetLastError();
-            MIXGCN_FAIL(MIXGCN_ENOMEM, "train_step_host: %lld bytes of device memory could not be allocated", (long long)lo.bytes);
-        }
-        ctx->arena = p; ctx->arena_bytes = lo.bytes;
-        MIXGCN_CUDA(cudaMemset(p, 0, (size_t)lo.bytes));
+        MIXGCN_TRY(grow_block(ctx, &ctx->arena, &ctx->arena_bytes, lo.bytes, "train_step_host: arena", true));
+        MIXGCN_CUDA(cudaMemset(ctx->arena, 0, (size_t)ctx->arena_bytes));
         MIXGCN_CUDA(cudaDeviceSynchronize());   // the copies below run on a non-blocking stream: the clear must have finished
     }
     MIXGCN_TRY(lay_out(reinterpret_cast<char*>(ctx->arena), n, L, dims, precision, lo));
@@ -194,8 +188,8 @@ extern "C" mixgcn_status mixgcn_train_step_host(mixgcn_ctx* ctx, const mixgcn_gr
             }
             if (!reuse) {
                 drop_plans(c);
-                if (c->n != n) { cudaFree(c->mask); c->mask = nullptr; c->n = 0; }
-                if (!c->mask) { MIXGCN_CUDA(cudaMalloc((void**)&c->mask, (size_t)n)); c->n = n; }
+                if (c->n != n) { dev_free(c->mask, s); c->mask = nullptr; c->n = 0; }
+                if (!c->mask) { MIXGCN_TRY(dev_alloc((void**)&c->mask, n, s)); c->n = n; }
                 MIXGCN_CUDA(cudaStreamSynchronize(s));
                 const uint8_t* in_mask = lo.mask;
                 for (int i = 0; i < levels; ++i) {

@@ -102,6 +102,7 @@ struct mixgcn_ctx {
     // device arena of mixgcn_train_step_host (activations, parameters, gradients), grown on demand
     void* arena;
     int64_t arena_bytes;
+    uint64_t blocks_generation;   // grows whenever one of the kept blocks above is replaced
     // row plans of the last mixgcn_train_step_host call, reused while graph and train mask stay the same
     struct HostStepCache* step_cache;
     struct HostStepPrefetch* step_prefetch;
@@ -199,8 +200,30 @@ struct LaunchScope {
     ~LaunchScope();
 };
 
-mixgcn_status ensure_workspace(mixgcn_ctx* ctx, int64_t bytes);
-mixgcn_status ensure_workspace_spmm(mixgcn_ctx* ctx, int64_t bytes);
+// Device memory of the library comes from one pool per device (see api.cu).  The block is usable on stream `s` at
+// once, on other streams after a synchronisation.  dev_free: everything that uses the block must have been enqueued on
+// `s` or have completed.  Both act on the current device.
+mixgcn_status dev_alloc(void** p, int64_t bytes, cudaStream_t s);
+void dev_free(void* p, cudaStream_t s);
+struct DevBuf {   // scratch of one call, freed in stream order on scope exit
+    void* p = nullptr;
+    cudaStream_t s;
+    explicit DevBuf(cudaStream_t stream) : s(stream) {}
+    DevBuf(const DevBuf&) = delete;
+    DevBuf& operator=(const DevBuf&) = delete;
+    ~DevBuf() { release(); }
+    mixgcn_status alloc(int64_t bytes) { return dev_alloc(&p, bytes > 0 ? bytes : 1, s); }
+    void release() { if (p) dev_free(p, s); p = nullptr; }
+    template <class T> T* as() { return reinterpret_cast<T*>(p); }
+};
+
+// Grow a block the context keeps between calls to at least `bytes`, with an eighth to spare unless `exact` (what: its
+// name in an error message).
+mixgcn_status grow_block(mixgcn_ctx* ctx, void** block, int64_t* have, int64_t bytes, const char* what, bool exact = false);
+inline mixgcn_status ensure_workspace(mixgcn_ctx* ctx, int64_t bytes) { return grow_block(ctx, &ctx->workspace, &ctx->workspace_bytes, bytes, "workspace"); }
+inline mixgcn_status ensure_workspace_spmm(mixgcn_ctx* ctx, int64_t bytes) { return grow_block(ctx, &ctx->workspace_spmm, &ctx->workspace_spmm_bytes, bytes, "aggregation workspace"); }
+inline mixgcn_status ensure_workspace_lp(mixgcn_ctx* ctx, int64_t bytes) { return grow_block(ctx, &ctx->workspace_lp, &ctx->workspace_lp_bytes, bytes, "bf16 operand workspace"); }
+inline mixgcn_status ensure_workspace_rows(mixgcn_ctx* ctx, int64_t bytes) { return grow_block(ctx, &ctx->workspace_rows, &ctx->workspace_rows_bytes, bytes, "row-sparse workspace"); }
 // Builds (once) the schedules of the `chunks` row chunks of this orientation.  Synchronises on first use.
 mixgcn_status ensure_chunk_schedules(const mixgcn_graph* g, const CsrView& A, int chunks);
 
@@ -286,7 +309,6 @@ mixgcn_status launch_splitk_reduce(mixgcn_ctx* ctx, int64_t M, int64_t N, int sp
                                    int64_t ldc, const mixgcn_epilogue* epi, cudaStream_t s);
 mixgcn_status launch_to_bf16(mixgcn_ctx* ctx, int64_t rows, int32_t d, const float* src, int64_t ld_src, uint16_t* dst,
                              int64_t ld_dst, cudaStream_t s);
-mixgcn_status ensure_workspace_lp(mixgcn_ctx* ctx, int64_t bytes);
 mixgcn_status launch_colsum(mixgcn_ctx* ctx, int64_t n, int32_t d, const float* X, int64_t ld, float* out,
                             cudaStream_t s);
 mixgcn_status launch_gate(mixgcn_ctx* ctx, int64_t n, int32_t d, float* G, int64_t ldg, const float* X_out,
@@ -305,7 +327,6 @@ mixgcn_status build_row_set(mixgcn_ctx* ctx, int64_t n, const uint8_t* mask, int
 mixgcn_status launch_gather_rows(mixgcn_ctx* ctx, int64_t n_rows, int64_t count, int32_t d, const int32_t* idx, const float* src,
                                  int64_t ld_src, float* dst, int64_t ld_dst, cudaStream_t s);
 
-mixgcn_status ensure_workspace_rows(mixgcn_ctx* ctx, int64_t bytes);
 void free_step_cache(mixgcn_ctx* ctx);
 // dst[idx[i], :] = src[i, :] for i < count (the inverse of launch_gather_rows)
 mixgcn_status launch_scatter_rows(mixgcn_ctx* ctx, int64_t n_rows, int64_t count, int32_t d, const int32_t* idx, const float* src,

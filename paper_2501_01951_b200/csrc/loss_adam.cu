@@ -576,17 +576,7 @@ mixgcn_status loss_fuse_begin(mixgcn_ctx* ctx, int64_t n, const int32_t* labels,
     if (blocks > cap) blocks = cap;
     const int64_t off_rows = (16 + blocks * (int64_t)sizeof(double) + 255) & ~(int64_t)255;
     const int64_t need = off_rows + n * (int64_t)sizeof(float);
-    if (need > ctx->workspace_loss_bytes) {
-        MIXGCN_CUDA(cudaDeviceSynchronize());      // the old block may still be in use by enqueued kernels
-        cudaFree(ctx->workspace_loss);
-        ctx->workspace_loss = nullptr; ctx->workspace_loss_bytes = 0;
-        void* q = nullptr;
-        if (cudaMalloc(&q, (size_t)need) != cudaSuccess) {
-            cudaGetLastError();
-            MIXGCN_FAIL(MIXGCN_ENOMEM, "loss scratch of %lld bytes could not be allocated", (long long)need);
-        }
-        ctx->workspace_loss = q; ctx->workspace_loss_bytes = need;
-    }
+    MIXGCN_TRY(grow_block(ctx, &ctx->workspace_loss, &ctx->workspace_loss_bytes, need, "loss scratch"));
     char* base = reinterpret_cast<char*>(ctx->workspace_loss);
     unsigned long long* count = reinterpret_cast<unsigned long long*>(base);
     MIXGCN_CUDA(cudaMemsetAsync(count, 0, sizeof(unsigned long long), s));

@@ -17,12 +17,6 @@ using namespace mixgcn;
 
 namespace {
 
-struct DevMem {
-    void* p = nullptr;
-    ~DevMem() { if (p) cudaFree(p); }
-    template <class T> T* as() { return reinterpret_cast<T*>(p); }
-};
-
 __global__ void pos_fill_kernel(int64_t count, const int32_t* __restrict__ idx, int32_t* __restrict__ pos) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < count) pos[idx[i]] = (int32_t)i;
@@ -81,8 +75,8 @@ extern "C" mixgcn_status mixgcn_rowplan_destroy(mixgcn_rowplan* p) {
     if (!p) return MIXGCN_OK;
     cudaSetDevice(p->device);
     cudaDeviceSynchronize();
-    cudaFree(p->idx);
-    cudaFree(p->out_mask);
+    dev_free(p->idx, nullptr);
+    dev_free(p->out_mask, nullptr);
     release_view(p->view);
     delete p;
     return MIXGCN_OK;
@@ -105,19 +99,19 @@ extern "C" mixgcn_status mixgcn_rowplan_create(mixgcn_ctx* ctx, const mixgcn_gra
     struct Guard { mixgcn_rowplan* p; ~Guard() { if (p) mixgcn_rowplan_destroy(p); } } guard{p};
 
     // kept rows, ascending, and their positions
-    DevMem sel, tmp, pos, cnt;
+    DevBuf sel(s), tmp(s), pos(s), cnt(s);
     size_t tb = 0;
     thrust::counting_iterator<int32_t> ids(0);
-    MIXGCN_CUDA(cudaMalloc((void**)&p->idx, (size_t)(n > 0 ? n : 1) * sizeof(int32_t)));
-    MIXGCN_CUDA(cudaMalloc(&sel.p, sizeof(int64_t)));
+    MIXGCN_TRY(dev_alloc((void**)&p->idx, (int64_t)((size_t)(n > 0 ? n : 1) * sizeof(int32_t)), s));
+    MIXGCN_TRY(sel.alloc((int64_t)(sizeof(int64_t))));
     MIXGCN_CUDA(cub::DeviceSelect::Flagged(nullptr, tb, ids, in_row_mask, p->idx, sel.as<int64_t>(), n, s));
-    MIXGCN_CUDA(cudaMalloc(&tmp.p, tb ? tb : 1));
+    MIXGCN_TRY(tmp.alloc((int64_t)(tb ? tb : 1)));
     MIXGCN_CUDA(cub::DeviceSelect::Flagged(tmp.p, tb, ids, in_row_mask, p->idx, sel.as<int64_t>(), n, s));
     int64_t in_count = 0;
     MIXGCN_CUDA(cudaMemcpyAsync(&in_count, sel.p, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     MIXGCN_CUDA(cudaStreamSynchronize(s));
     p->in_count = in_count;
-    MIXGCN_CUDA(cudaMalloc(&pos.p, (size_t)(n > 0 ? n : 1) * sizeof(int32_t)));
+    MIXGCN_TRY(pos.alloc((int64_t)((size_t)(n > 0 ? n : 1) * sizeof(int32_t))));
     MIXGCN_CUDA(cudaMemsetAsync(pos.p, 0xFF, (size_t)n * sizeof(int32_t), s));
     if (in_count > 0)
         pos_fill_kernel<<<(unsigned)((in_count + 255) / 256), 256, 0, s>>>(in_count, p->idx, pos.as<int32_t>());
@@ -125,22 +119,22 @@ extern "C" mixgcn_status mixgcn_rowplan_create(mixgcn_ctx* ctx, const mixgcn_gra
     // restricted CSR: per-row kept counts -> row pointers -> entries
     CsrView& V = p->view;
     V = CsrView{};
-    MIXGCN_CUDA(cudaMalloc((void**)&p->out_mask, (size_t)(n > 0 ? n : 1)));
-    MIXGCN_CUDA(cudaMalloc(&cnt.p, (size_t)(n + 1) * sizeof(int64_t)));
+    MIXGCN_TRY(dev_alloc((void**)&p->out_mask, (int64_t)((size_t)(n > 0 ? n : 1)), s));
+    MIXGCN_TRY(cnt.alloc((int64_t)((size_t)(n + 1) * sizeof(int64_t))));
     MIXGCN_CUDA(cudaMemsetAsync(cnt.p, 0, (size_t)(n + 1) * sizeof(int64_t), s));
-    MIXGCN_CUDA(cudaMalloc((void**)&V.rowptr, (size_t)(n + 1) * sizeof(int64_t)));
+    MIXGCN_TRY(dev_alloc((void**)&V.rowptr, (int64_t)((size_t)(n + 1) * sizeof(int64_t)), s));
     const unsigned row_blocks = (unsigned)((n * 32 + 255) / 256);
     if (n > 0) kept_count_kernel<<<row_blocks, 256, 0, s>>>(n, A.rowptr, A.col, in_row_mask, cnt.as<int64_t>(), p->out_mask);
-    DevMem tmp2;
+    DevBuf tmp2(s);
     size_t tb2 = 0;
     MIXGCN_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tb2, cnt.as<int64_t>(), V.rowptr, n + 1, s));
-    MIXGCN_CUDA(cudaMalloc(&tmp2.p, tb2 ? tb2 : 1));
+    MIXGCN_TRY(tmp2.alloc((int64_t)(tb2 ? tb2 : 1)));
     MIXGCN_CUDA(cub::DeviceScan::ExclusiveSum(tmp2.p, tb2, cnt.as<int64_t>(), V.rowptr, n + 1, s));
     int64_t nnz2 = 0;
     MIXGCN_CUDA(cudaMemcpyAsync(&nnz2, V.rowptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     // rows with a kept entry
-    DevMem oc;
-    MIXGCN_CUDA(cudaMalloc(&oc.p, sizeof(unsigned long long)));
+    DevBuf oc(s);
+    MIXGCN_TRY(oc.alloc((int64_t)(sizeof(unsigned long long))));
     MIXGCN_CUDA(cudaMemsetAsync(oc.p, 0, sizeof(unsigned long long), s));
     if (n > 0) {
         int64_t cb = (n + 255) / 256;
@@ -151,8 +145,8 @@ extern "C" mixgcn_status mixgcn_rowplan_create(mixgcn_ctx* ctx, const mixgcn_gra
     MIXGCN_CUDA(cudaMemcpyAsync(&out_count, oc.p, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     MIXGCN_CUDA(cudaStreamSynchronize(s));
     p->nnz = nnz2; p->out_count = out_count;
-    MIXGCN_CUDA(cudaMalloc((void**)&V.col, (size_t)(nnz2 > 0 ? nnz2 : 1) * sizeof(int32_t)));
-    MIXGCN_CUDA(cudaMalloc((void**)&V.val, (size_t)(nnz2 > 0 ? nnz2 : 1) * sizeof(float)));
+    MIXGCN_TRY(dev_alloc((void**)&V.col, (int64_t)((size_t)(nnz2 > 0 ? nnz2 : 1) * sizeof(int32_t)), s));
+    MIXGCN_TRY(dev_alloc((void**)&V.val, (int64_t)((size_t)(nnz2 > 0 ? nnz2 : 1) * sizeof(float)), s));
     if (n > 0 && nnz2 > 0)
         kept_fill_kernel<<<row_blocks, 256, 0, s>>>(n, A.rowptr, A.col, A.val, in_row_mask, pos.as<int32_t>(), V.rowptr, V.col, V.val);
     MIXGCN_CUDA(cudaGetLastError());

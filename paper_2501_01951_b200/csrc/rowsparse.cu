@@ -60,22 +60,6 @@ __global__ void scatter_rows_kernel(int64_t count, int d4, const int32_t* __rest
 
 namespace mixgcn {
 
-mixgcn_status ensure_workspace_rows(mixgcn_ctx* ctx, int64_t bytes) {
-    if (bytes <= ctx->workspace_rows_bytes) return MIXGCN_OK;
-    int64_t want = bytes + (bytes >> 3);
-    want = (want + 255) & ~(int64_t)255;
-    void* p = nullptr;
-    MIXGCN_CUDA(cudaDeviceSynchronize());
-    if (ctx->workspace_rows) cudaFree(ctx->workspace_rows);
-    ctx->workspace_rows = nullptr; ctx->workspace_rows_bytes = 0;
-    if (cudaMalloc(&p, (size_t)want) != cudaSuccess) {
-        cudaGetLastError();
-        MIXGCN_FAIL(MIXGCN_ENOMEM, "row-sparse workspace of %lld bytes could not be allocated", (long long)want);
-    }
-    ctx->workspace_rows = p; ctx->workspace_rows_bytes = want;
-    return MIXGCN_OK;
-}
-
 // Carves the row-sparse workspace and fills the row list and the position map of `mask`.
 // idx has capacity n >= count (memory-safe whatever the mask holds); if the number of set rows differs
 // from `count` the device status word receives DEV_BAD_ROW_COUNT and the unfilled slots name row 0.

@@ -183,7 +183,7 @@ mixgcn_status launch_gemm(mixgcn_ctx* ctx, int precision, int ta, int tb, int64_
     }
     if (st == MIXGCN_EUNSUPPORTED && loss) return st;      // the caller runs the product and the loss separately
     if (st == MIXGCN_EUNSUPPORTED) {
-        st = launch_gemm_simt(ctx, ta, tb, M, N, K, A, lda, B, ldb, C, ldc, epi, epi_row0, s);
+        st = launch_gemm_simt(ctx, ta, tb, M, N, K, A, lda, B, ldb, C, ldc, epi, epi_row0, s, &bits_done);
         if (st == MIXGCN_OK) ctx->gemm_path[0]++;
     }
     if (st != MIXGCN_OK) return st;

@@ -2,26 +2,26 @@
 // update line of Algorithm 2 and of its two backward products), plus the small streaming
 // kernels around them (column sums for the bias gradient, the ReLU/dropout gate on a gradient).
 //
-// C = op(A) op(B): 128 x BN output tile per CTA, 16-deep k-steps staged through shared memory
-// with the next step's global loads in flight during the FMAs; each thread owns an 8 x TN
-// micro-tile.  Long reductions (K = number of nodes in the weight-gradient product) are split
-// over CTAs into partial tiles that a second kernel adds in a fixed order in fp64, and inside a
-// CTA the fp32 accumulator is flushed into a second-level sum every 1024 terms, so rounding
-// error does not grow with the node count.
+// Long reductions (K = number of nodes in the weight-gradient product) are split over CTAs into partial
+// tiles that a second kernel adds in a fixed order in fp64, and inside a CTA the fp32 accumulator is
+// flushed into a second-level sum every 1024 terms, so rounding error does not grow with the node count.
 #include "internal.cuh"
 
 using namespace mixgcn;
 
 namespace {
 
-constexpr int BM = 128, BK = 16, NT = 256, TM = 8;
-constexpr int FLUSH_TILES = 64;  // 64 * 16 = 1024 terms per first-level accumulator
+constexpr int BK = 16;              // k-step
+constexpr int STAGES = 3;
+constexpr int FLUSH_STEPS = 64;     // 64 * 16 = 1024 terms per first-level accumulator
+constexpr int MIN_K_PER_SPLIT = 128;
 
 struct Epi {
     const float* bias; int relu;
     const uint8_t* drop; float keep_scale;
     const float* gate; int64_t ld_gate; float gate_scale;
     const uint32_t* gate_bits; int64_t ld_gate_bits;   // bit-packed gate (replaces `gate`)
+    uint32_t* sign_bits; int64_t ld_sign_bits;         // output: bit = (final y > 0)
     int64_t row0;
 };
 
@@ -34,16 +34,6 @@ __device__ __forceinline__ float apply_epi(const Epi& e, float y, int64_t m, int
     return y;
 }
 
-// Up to four consecutive floats src[0..3], element t valid iff t < valid; invalid ones are zero.
-__device__ __forceinline__ float4 load_tail(const float* src, int64_t valid) {
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (valid > 0) v.x = src[0];
-    if (valid > 1) v.y = src[1];
-    if (valid > 2) v.z = src[2];
-    if (valid > 3) v.w = src[3];
-    return v;
-}
-
 struct GemmParams {
     int64_t M, N, K;
     const float* A; int64_t lda;
@@ -52,154 +42,266 @@ struct GemmParams {
     int64_t k_per_split; int splits;
     int64_t m_tiles, n_tiles;
     int vec_a, vec_b, vec_c;     // 16-byte vector access is legal (pointer and ld aligned)
+    int vec_drop, vec_gate;      // the same for four mask bytes / four gate values at a multiple of four columns
     Epi epi;
 };
 
-template <int BN, int TN, bool TA, bool TB>
-__global__ void __launch_bounds__(NT) gemm_simt_kernel(const GemmParams p) {
-    constexpr int LDA_S = BM + 4, LDB_S = BN + 4;
-    __shared__ __align__(16) float As[BK][LDA_S];
-    __shared__ __align__(16) float Bs[BK][LDB_S];
-    constexpr int A_V = BM * BK / 4 / NT;   // float4 per thread for the A tile (2)
-    constexpr int B_V = BK * BN / 4 / NT;   // float4 per thread for the B tile (2 or 1)
+// two fp32 lanes in one register pair: one instruction, two IEEE FMAs
+typedef unsigned long long f32x2;
+__device__ __forceinline__ void ffma2(f32x2& d, f32x2 a, f32x2 b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b)); }
+__device__ __forceinline__ f32x2 dup2(float a) { f32x2 r; asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a)); return r; }
+__device__ __forceinline__ float2 split2(f32x2 v) { float2 f; asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v)); return f; }
 
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+__device__ __forceinline__ void cp_async16(void* dst, const float* src, int bytes) {      // the first `bytes` of 16, zeros behind
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* dst, const float* src, int bytes) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
+}
+// four consecutive floats, the first `valid` of them read (<= 0: none, `base` stands in for the address)
+__device__ __forceinline__ void copy4(float* dst, const float* src, int64_t valid, int vec, const float* base) {
+    const int v = valid >= 4 ? 4 : valid > 0 ? (int)valid : 0;
+    if (vec) { cp_async16(dst, v ? src : base, v * 4); return; }
+#pragma unroll
+    for (int t = 0; t < 4; ++t) cp_async4(dst + t, t < v ? src + t : base, t < v ? 4 : 0);
+}
+
+// C = op(A) op(B) on the FMA pipes: a BM x BN tile per CTA, an 8 x 16 (smaller tiles 8 x 8) micro-tile per thread held as packed pairs (one
+// fma.rn.f32x2 does two FMAs, so that the shared-memory loads and the operand copies find free issue slots beside a full
+// FMA pipe), 16-deep k-steps through three cp.async stages.  Bound by the FMA rate (72 TFLOP/s measured with either
+// form of the instruction): 170 K x 256 x 256 forward 33.7 -> 42 TFLOP/s, weight gradient 25.4 -> 48 TFLOP/s against one
+// stage, register staging and scalar FMAs; the pipe is then 72 % busy, the rest is fixed-latency waits of the two warps a
+// scheduler has room for.
+//   A with K contiguous stays [m][k] in shared memory and is read two k at a time (row pitch 20 floats: the four rows a
+//   warp reads side by side lie in different banks); A with M contiguous, and B, are [k][m] / [k][n].  B with K
+//   contiguous (the small weight matrix of dP W^T) is turned round by word-wide copies.
+// Long reductions: after 1024 terms the accumulators are added to C (the partial tile or C itself), which serves as the
+// second-level sum.
+template <int BM, int BN, int TN>
+struct SimtCfg {
+    static constexpr int NT = BM * BN / (8 * TN);                        // threads
+    static constexpr int MIN_CTAS = BM == 128 ? (BN == 128 ? 2 : 4) : BN == 64 ? 6 : 10;
+};
+
+template <int BM, int BN, int TN, bool TA, bool TB>
+__global__ void __launch_bounds__(SimtCfg<BM, BN, TN>::NT, SimtCfg<BM, BN, TN>::MIN_CTAS) gemm_simt_kernel(const GemmParams p) {
+    constexpr int NT = SimtCfg<BM, BN, TN>::NT, TX = BN / TN, Q = TN / 4, QW = BN / Q;   // Q groups of four columns, QW columns apart
+    constexpr int A_PITCH = TA ? BM + 4 : BK + 4, B_PITCH = BN + 4;
+    constexpr int A_FLOATS = TA ? BK * A_PITCH : BM * A_PITCH, B_FLOATS = BK * B_PITCH;
+    constexpr int A_V = BM * BK / 4 / NT;
+    extern __shared__ __align__(16) float smem_f[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // a warp covers 4 x 8 micro-tiles (TX >= 8) or 8 x 4
+    constexpr int WX = TX >= 8 ? 8 : TX, WY = 32 / WX, WARPS_X = TX / WX;
+    const int tx = (warp % WARPS_X) * WX + lane % WX, ty = (warp / WARPS_X) * WY + lane / WX;
     const int64_t tile = blockIdx.x;
     const int64_t m0 = (tile / p.n_tiles) * BM, n0 = (tile % p.n_tiles) * BN;
     const int64_t kb = (int64_t)blockIdx.z * p.k_per_split;
     const int64_t ke = (kb + p.k_per_split < p.K) ? kb + p.k_per_split : p.K;
+    const int steps = (int)((ke - kb + BK - 1) / BK);
+    // rows of the micro-tile: i-th row is ty + i * (BM / 8) with A as [m][k], (i / 4) * (BM / 2) + ty * 4 + i % 4 as [k][m];
+    // columns: (j / 4) * QW + tx * 4 + j % 4
+    auto row_of = [&](int i) { return TA ? (i >> 2) * (BM / 2) + ty * 4 + (i & 3) : ty + i * (BM / 8); };
 
-    float4 ra[A_V], rb[B_V];
-
-    auto load_regs = [&](int64_t k0) {
-#pragma unroll
-        for (int i = 0; i < A_V; ++i) {
-            const int f = tid + i * NT;
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (!TA) {  // A is M x K, contiguous along k
-                const int64_t m = m0 + f / 4, k = k0 + (f % 4) * 4;
-                if (m < p.M) {
-                    const float* src = p.A + m * p.lda + k;
-                    if (p.vec_a && k + 3 < ke) v = __ldg(reinterpret_cast<const float4*>(src));
-                    else v = load_tail(src, ke - k);
-                }
-            } else {    // A is K x M, contiguous along m
-                const int64_t k = k0 + f / (BM / 4), m = m0 + (f % (BM / 4)) * 4;
-                if (k < ke) {
-                    const float* src = p.A + k * p.lda + m;
-                    if (p.vec_a && m + 3 < p.M) v = __ldg(reinterpret_cast<const float4*>(src));
-                    else v = load_tail(src, p.M - m);
-                }
-            }
-            ra[i] = v;
-        }
-#pragma unroll
-        for (int i = 0; i < B_V; ++i) {
-            const int f = tid + i * NT;
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (!TB) {  // B is K x N, contiguous along n
-                const int64_t k = k0 + f / (BN / 4), n = n0 + (f % (BN / 4)) * 4;
-                if (k < ke) {
-                    const float* src = p.B + k * p.ldb + n;
-                    if (p.vec_b && n + 3 < p.N) v = __ldg(reinterpret_cast<const float4*>(src));
-                    else v = load_tail(src, p.N - n);
-                }
-            } else {    // B is N x K, contiguous along k
-                const int64_t n = n0 + f / 4, k = k0 + (f % 4) * 4;
-                if (n < p.N) {
-                    const float* src = p.B + n * p.ldb + k;
-                    if (p.vec_b && k + 3 < ke) v = __ldg(reinterpret_cast<const float4*>(src));
-                    else v = load_tail(src, ke - k);
-                }
-            }
-            rb[i] = v;
-        }
-    };
-    auto store_smem = [&]() {
+    auto load_a = [&](int ks) {
+        float* As = smem_f + (ks % STAGES) * (A_FLOATS + B_FLOATS);
+        const int64_t k0 = kb + (int64_t)ks * BK;
 #pragma unroll
         for (int i = 0; i < A_V; ++i) {
             const int f = tid + i * NT;
             if (!TA) {
-                const int m = f / 4, k = (f % 4) * 4;
-                As[k][m] = ra[i].x; As[k + 1][m] = ra[i].y; As[k + 2][m] = ra[i].z; As[k + 3][m] = ra[i].w;
+                const int r = f / 4, kq = (f % 4) * 4;
+                const int64_t m = m0 + r, k = k0 + kq;
+                copy4(As + r * A_PITCH + kq, p.A + m * p.lda + k, m < p.M ? ke - k : 0, p.vec_a, p.A);
             } else {
-                const int k = f / (BM / 4), m = (f % (BM / 4)) * 4;
-                *reinterpret_cast<float4*>(&As[k][m]) = ra[i];
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < B_V; ++i) {
-            const int f = tid + i * NT;
-            if (!TB) {
-                const int k = f / (BN / 4), n = (f % (BN / 4)) * 4;
-                *reinterpret_cast<float4*>(&Bs[k][n]) = rb[i];
-            } else {
-                const int n = f / 4, k = (f % 4) * 4;
-                Bs[k][n] = rb[i].x; Bs[k + 1][n] = rb[i].y; Bs[k + 2][n] = rb[i].z; Bs[k + 3][n] = rb[i].w;
+                const int kr = f / (BM / 4), mq = (f % (BM / 4)) * 4;
+                const int64_t k = k0 + kr, m = m0 + mq;
+                copy4(As + kr * A_PITCH + mq, p.A + k * p.lda + m, k < ke ? p.M - m : 0, p.vec_a, p.A);
             }
         }
     };
-
-    float acc[TM][TN], tot[TM][TN];
+    auto load_b = [&](int ks) {
+        float* Bs = smem_f + (ks % STAGES) * (A_FLOATS + B_FLOATS) + A_FLOATS;
+        const int64_t k0 = kb + (int64_t)ks * BK;
+        if constexpr (!TB) {
 #pragma unroll
-    for (int i = 0; i < TM; ++i)
-#pragma unroll
-        for (int j = 0; j < TN; ++j) { acc[i][j] = 0.f; tot[i][j] = 0.f; }
-
-    int since_flush = 0;
-    if (kb < ke) load_regs(kb);
-    for (int64_t k0 = kb; k0 < ke; k0 += BK) {
-        store_smem();
-        __syncthreads();
-        if (k0 + BK < ke) load_regs(k0 + BK);
-#pragma unroll
-        for (int k = 0; k < BK; ++k) {
-            float a[TM], b[TN];
-            const float4 a0 = *reinterpret_cast<const float4*>(&As[k][ty * TM]);
-            const float4 a1 = *reinterpret_cast<const float4*>(&As[k][ty * TM + 4]);
-            a[0] = a0.x; a[1] = a0.y; a[2] = a0.z; a[3] = a0.w; a[4] = a1.x; a[5] = a1.y; a[6] = a1.z; a[7] = a1.w;
-#pragma unroll
-            for (int q = 0; q < TN / 4; ++q) {
-                const float4 bq = *reinterpret_cast<const float4*>(&Bs[k][q * 64 + tx * 4]);
-                b[q * 4] = bq.x; b[q * 4 + 1] = bq.y; b[q * 4 + 2] = bq.z; b[q * 4 + 3] = bq.w;
+            for (int i = 0; i < BK * BN / 4 / NT; ++i) {
+                const int f = tid + i * NT, kr = f / (BN / 4), nq = (f % (BN / 4)) * 4;
+                const int64_t k = k0 + kr, n = n0 + nq;
+                copy4(Bs + kr * B_PITCH + nq, p.B + k * p.ldb + n, k < ke ? p.N - n : 0, p.vec_b, p.B);
             }
+        } else {
+            // word by word: sixteen lanes read one row's 64 bytes and write a column of the tile
 #pragma unroll
-            for (int i = 0; i < TM; ++i)
-#pragma unroll
-                for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+            for (int i = 0; i < BK * BN / NT; ++i) {
+                const int f = tid + i * NT, nr = f / BK, kr = f % BK;
+                const int64_t k = k0 + kr, n = n0 + nr;
+                const bool in = n < p.N && k < ke;
+                cp_async4(Bs + kr * B_PITCH + nr, in ? p.B + n * p.ldb + k : p.B, in ? 4 : 0);
+            }
         }
-        __syncthreads();
-        if (++since_flush == FLUSH_TILES) {
-            since_flush = 0;
+    };
+    auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
+
+    f32x2 acc[8][TN / 2];
 #pragma unroll
-            for (int i = 0; i < TM; ++i)
+    for (int i = 0; i < 8; ++i)
 #pragma unroll
-                for (int j = 0; j < TN; ++j) { tot[i][j] += acc[i][j]; acc[i][j] = 0.f; }
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < TM; ++i)
-#pragma unroll
-        for (int j = 0; j < TN; ++j) tot[i][j] += acc[i][j];
+        for (int j = 0; j < TN / 2; ++j) acc[i][j] = 0ull;
 
     const bool partial = p.splits > 1;
     float* Cb = partial ? p.C + (int64_t)blockIdx.z * p.M * p.N : p.C;
     const int64_t ldc = partial ? p.N : p.ldc;
+    const bool vec_c = partial ? (p.N & 3) == 0 : p.vec_c != 0;
+    // add the accumulators to C (the first time: store them) and clear them
+    auto flush = [&](bool first) {
+        // addresses are worked out here and not, hoisted, in the k-loop's registers: the compiler cannot see through the copy
+        int64_t m0c;
+        asm volatile("mov.b64 %0, %1;" : "=l"(m0c) : "l"(m0));
 #pragma unroll
-    for (int i = 0; i < TM; ++i) {
-        const int64_t m = m0 + ty * TM + i;
-        if (m >= p.M) continue;
+        for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int q = 0; q < TN / 4; ++q) {
-            const int64_t n = n0 + q * 64 + tx * 4;
-            float r[4];
+            for (int q = 0; q < Q; ++q) {
+                const int64_t m = m0c + row_of(i), n = n0 + q * QW + tx * 4;
+                float* dst = Cb + m * ldc + n;
+                const float2 lo = split2(acc[i][q * 2]), hi = split2(acc[i][q * 2 + 1]);
+                const float r[4] = {lo.x, lo.y, hi.x, hi.y};
 #pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                r[t] = tot[i][q * 4 + t];
-                if (!partial && n + t < p.N) r[t] = apply_epi(p.epi, r[t], m, n + t, p.N);
+                for (int t = 0; t < 4; ++t) if (m < p.M && n + t < p.N) dst[t] = first ? r[t] : r[t] + dst[t];
+                acc[i][q * 2] = 0ull; acc[i][q * 2 + 1] = 0ull;
             }
+    };
+
+#pragma unroll
+    for (int ks = 0; ks < STAGES - 1; ++ks) {
+        if (ks < steps) { load_a(ks); load_b(ks); }
+        commit();
+    }
+    bool flushed = false;
+    int since_flush = 0;
+    for (int ks = 0; ks < steps; ++ks) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+        __syncthreads();                       // step ks has landed; the stage of step ks - 1 is free
+        if (ks + STAGES - 1 < steps) { load_a(ks + STAGES - 1); load_b(ks + STAGES - 1); }
+        commit();
+        const float* As = smem_f + (ks % STAGES) * (A_FLOATS + B_FLOATS);
+        const float* Bs = As + A_FLOATS;
+#pragma unroll (TA ? BK / 2 : 2)        // (with the row-wise A a longer body gains nothing and spills)
+        for (int kk = 0; kk < BK; kk += 2) {
+            float2 a2[8];
+            if (!TA) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) a2[i] = *reinterpret_cast<const float2*>(As + (ty + i * (BM / 8)) * A_PITCH + kk);
+            }
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const float* brow = Bs + (kk + k) * B_PITCH + tx * 4;
+                ulonglong2 b[Q];
+#pragma unroll
+                for (int q = 0; q < Q; ++q) b[q] = *reinterpret_cast<const ulonglong2*>(brow + q * QW);
+                float a[8];
+                if (!TA) {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) a[i] = k == 0 ? a2[i].x : a2[i].y;
+                } else {
+                    const float* arow = As + (kk + k) * A_PITCH + ty * 4;
+                    const float4 x = *reinterpret_cast<const float4*>(arow), y = *reinterpret_cast<const float4*>(arow + BM / 2);
+                    a[0] = x.x; a[1] = x.y; a[2] = x.z; a[3] = x.w; a[4] = y.x; a[5] = y.y; a[6] = y.z; a[7] = y.w;
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const f32x2 av = dup2(a[i]);
+#pragma unroll
+                    for (int q = 0; q < Q; ++q) { ffma2(acc[i][2 * q], av, b[q].x); ffma2(acc[i][2 * q + 1], av, b[q].y); }
+                }
+            }
+        }
+        if (++since_flush == FLUSH_STEPS && ks + 1 < steps) {
+            since_flush = 0;
+            flush(!flushed);
+            flushed = true;
+        }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+
+    // Epilogue through shared memory, half of the rows at a time: a warp then stores (and reads gates and masks of) whole
+    // rows, and its code is one short loop.  Applied from the registers it was unrolled over the micro-tile, thirty
+    // kilobytes of branches that cost more than 128 terms of K (170 K x 256, K = 128: 617 us).
+    constexpr int S_PITCH = BN + 4, ROW4 = BN / 4;
+    const Epi& e = p.epi;
+    float* const S = smem_f;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const float2 lo = split2(acc[h * 4 + i][q * 2]), hi = split2(acc[h * 4 + i][q * 2 + 1]);
+                *reinterpret_cast<float4*>(S + (row_of(i)) * S_PITCH + q * QW + tx * 4) = make_float4(lo.x, lo.y, hi.x, hi.y);
+            }
+        __syncthreads();
+#pragma unroll 2
+        for (int f = tid; f < BM / 2 * ROW4; f += NT) {
+            const int lr = f / ROW4, lc = (f % ROW4) * 4;
+            const int64_t m = m0 + h * (BM / 2) + lr, n = n0 + lc;
+            const bool in = m < p.M && n < p.N, full = n + 3 < p.N;
+            const float4 v = *reinterpret_cast<const float4*>(S + lr * S_PITCH + lc);
+            float r[4] = {v.x, v.y, v.z, v.w};
             float* dst = Cb + m * ldc + n;
-            if (p.vec_c && n + 3 < p.N && !partial) *reinterpret_cast<float4*>(dst) = make_float4(r[0], r[1], r[2], r[3]);
+            if (flushed && in) {
+#pragma unroll
+                for (int t = 0; t < 4; ++t) if (n + t < p.N) r[t] += dst[t];
+            }
+            if (!partial) {
+                if (e.bias) {
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) if (n + t < p.N) r[t] += __ldg(e.bias + n + t);
+                }
+                if (e.relu) {
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) r[t] = fmaxf(r[t], 0.0f);
+                }
+                if (e.drop && in) {
+                    const uint8_t* dm = e.drop + (e.row0 + m) * p.N + n;
+                    if (p.vec_drop && full) {
+                        const uchar4 d4 = __ldg(reinterpret_cast<const uchar4*>(dm));
+                        r[0] = d4.x ? r[0] * e.keep_scale : 0.0f; r[1] = d4.y ? r[1] * e.keep_scale : 0.0f;
+                        r[2] = d4.z ? r[2] * e.keep_scale : 0.0f; r[3] = d4.w ? r[3] * e.keep_scale : 0.0f;
+                    } else {
+#pragma unroll
+                        for (int t = 0; t < 4; ++t) if (n + t < p.N) r[t] = dm[t] ? r[t] * e.keep_scale : 0.0f;
+                    }
+                }
+                if (e.gate && in) {
+                    const float* gp = e.gate + (e.row0 + m) * e.ld_gate + n;
+                    if (p.vec_gate && full) {
+                        const float4 g4 = __ldg(reinterpret_cast<const float4*>(gp));
+                        r[0] = g4.x > 0.0f ? r[0] * e.gate_scale : 0.0f; r[1] = g4.y > 0.0f ? r[1] * e.gate_scale : 0.0f;
+                        r[2] = g4.z > 0.0f ? r[2] * e.gate_scale : 0.0f; r[3] = g4.w > 0.0f ? r[3] * e.gate_scale : 0.0f;
+                    } else {
+#pragma unroll
+                        for (int t = 0; t < 4; ++t) if (n + t < p.N) r[t] = __ldg(gp + t) > 0.0f ? r[t] * e.gate_scale : 0.0f;
+                    }
+                }
+                if (e.gate_bits && in) {
+                    const uint32_t nib = __ldg(e.gate_bits + (e.row0 + m) * e.ld_gate_bits + (n >> 5)) >> (n & 31);   // n % 4 == 0: one word
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) r[t] = ((nib >> t) & 1u) ? r[t] * e.gate_scale : 0.0f;
+                }
+                if (e.sign_bits) {
+                    // eight lanes hold 32 consecutive columns of a row, one word of the bitmap
+                    uint32_t w = 0;
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) w |= (n + t < p.N && r[t] > 0.0f ? 1u : 0u) << t;
+                    w <<= n & 31;
+#pragma unroll
+                    for (int o = 1; o < 8; o <<= 1) w |= __shfl_xor_sync(0xFFFFFFFFu, w, o);
+                    if (in && (lane & 7) == 0) e.sign_bits[(e.row0 + m) * e.ld_sign_bits + (n >> 5)] = w;
+                }
+            }
+            if (!in) continue;
+            if (vec_c && full) *reinterpret_cast<float4*>(dst) = make_float4(r[0], r[1], r[2], r[3]);
             else {
 #pragma unroll
                 for (int t = 0; t < 4; ++t) if (n + t < p.N) dst[t] = r[t];
@@ -208,13 +310,27 @@ __global__ void __launch_bounds__(NT) gemm_simt_kernel(const GemmParams p) {
     }
 }
 
-// C[m][n] = epilogue( sum_z part[z][m][n] ), z ascending, fp64 accumulation.
-__global__ void splitk_reduce_kernel(int64_t M, int64_t N, int splits, const float* __restrict__ part,
-                                     float* __restrict__ C, int64_t ldc, const Epi epi) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= M * N) return;
+// C[m][n] = epilogue( sum_z part[z][m][n] ) in fp64.  A block owns 32 consecutive elements; its eight rows of threads add
+// an eighth of the splits each (ascending), the eighths are added in order: a hundred splits of a small weight gradient
+// cost one thread a chain of a hundred loads otherwise (16 K elements, 148 splits: 20 -> 4 us).
+constexpr int RED_PARTS = 8;
+__global__ void __launch_bounds__(32 * RED_PARTS) splitk_reduce_kernel(int64_t M, int64_t N, int splits, const float* __restrict__ part,
+                                                                      float* __restrict__ C, int64_t ldc, const Epi epi) {
+    __shared__ double sm[RED_PARTS][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t i = (int64_t)blockIdx.x * 32 + lane, MN = M * N;
+    const int per = (splits + RED_PARTS - 1) / RED_PARTS;
+    const int z0 = w * per, z1 = z0 + per < splits ? z0 + per : splits;
     double s = 0.0;
-    for (int z = 0; z < splits; ++z) s += (double)part[(int64_t)z * M * N + i];
+    if (i < MN) {
+#pragma unroll 4
+        for (int z = z0; z < z1; ++z) s += (double)__ldg(part + (int64_t)z * MN + i);
+    }
+    sm[w][lane] = s;
+    __syncthreads();
+    if (w != 0 || i >= MN) return;
+#pragma unroll
+    for (int q = 1; q < RED_PARTS; ++q) s += sm[q][lane];
     const int64_t m = i / N, n = i % N;
     C[m * ldc + n] = apply_epi(epi, (float)s, m, n, N);
 }
@@ -274,11 +390,22 @@ __global__ void __launch_bounds__(256) colsum_partial_kernel(int64_t n, int d, c
     }
 }
 
-__global__ void colsum_final_kernel(int d, int blocks, const float* __restrict__ part, float* __restrict__ out) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= d) return;
+// 32 columns per block, eight rows of threads take an eighth of the partial rows each (fp64, fixed order).
+__global__ void __launch_bounds__(32 * RED_PARTS) colsum_final_kernel(int d, int blocks, const float* __restrict__ part, float* __restrict__ out) {
+    __shared__ double sm[RED_PARTS][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, j = blockIdx.x * 32 + lane;
+    const int per = (blocks + RED_PARTS - 1) / RED_PARTS;
+    const int b0 = w * per, b1 = b0 + per < blocks ? b0 + per : blocks;
     double s = 0.0;
-    for (int b = 0; b < blocks; ++b) s += (double)part[(int64_t)b * d + j];
+    if (j < d) {
+#pragma unroll 4
+        for (int b = b0; b < b1; ++b) s += (double)__ldg(part + (int64_t)b * d + j);
+    }
+    sm[w][lane] = s;
+    __syncthreads();
+    if (w != 0 || j >= d) return;
+#pragma unroll
+    for (int q = 1; q < RED_PARTS; ++q) s += sm[q][lane];
     out[j] = (float)s;
 }
 
@@ -294,21 +421,36 @@ __global__ void gate_kernel(int64_t n, int d, float* __restrict__ G, int64_t ldg
     G[r * ldg + j] = g;
 }
 
-template <int BN, int TN>
-void launch_variant(const GemmParams& p, int ta, int tb, dim3 grid, cudaStream_t s) {
-    if (!ta && !tb) gemm_simt_kernel<BN, TN, false, false><<<grid, NT, 0, s>>>(p);
-    else if (!ta && tb) gemm_simt_kernel<BN, TN, false, true><<<grid, NT, 0, s>>>(p);
-    else if (ta && !tb) gemm_simt_kernel<BN, TN, true, false><<<grid, NT, 0, s>>>(p);
-    else gemm_simt_kernel<BN, TN, true, true><<<grid, NT, 0, s>>>(p);
+template <int BM, int BN, int TN, bool TA, bool TB>
+cudaError_t launch_form(const GemmParams& p, cudaStream_t s) {
+    constexpr int a_floats = TA ? BK * (BM + 4) : BM * (BK + 4), b_floats = BK * (BN + 4);
+    constexpr int ring = STAGES * (a_floats + b_floats), half_tile = BM / 2 * (BN + 4);
+    constexpr int smem = (ring > half_tile ? ring : half_tile) * (int)sizeof(float);
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(gemm_simt_kernel<BM, BN, TN, TA, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+    }
+    gemm_simt_kernel<BM, BN, TN, TA, TB><<<dim3((unsigned)(p.m_tiles * p.n_tiles), 1, (unsigned)p.splits), SimtCfg<BM, BN, TN>::NT, smem, s>>>(p);
+    return cudaGetLastError();
+}
+
+template <int BM, int BN, int TN>
+cudaError_t launch_variant(const GemmParams& p, int ta, int tb, cudaStream_t s) {
+    if (!ta && !tb) return launch_form<BM, BN, TN, false, false>(p, s);
+    if (!ta) return launch_form<BM, BN, TN, false, true>(p, s);
+    if (!tb) return launch_form<BM, BN, TN, true, false>(p, s);
+    return launch_form<BM, BN, TN, true, true>(p, s);
 }
 
 }  // namespace
 
 namespace mixgcn {
 
+// *bits_done: whether the sign bitmap, if one is asked for, was written (not where K is split).
 mixgcn_status launch_gemm_simt(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64_t N, int64_t K,
                                const float* A, int64_t lda, const float* B, int64_t ldb, float* C, int64_t ldc,
-                               const mixgcn_epilogue* epi, int64_t epi_row0, cudaStream_t s) {
+                               const mixgcn_epilogue* epi, int64_t epi_row0, cudaStream_t s, bool* bits_done) {
+    if (bits_done) *bits_done = false;
     if (M <= 0 || N <= 0) return MIXGCN_OK;
     GemmParams p{};
     p.M = M; p.N = N; p.K = K; p.A = A; p.lda = lda; p.B = B; p.ldb = ldb; p.C = C; p.ldc = ldc;
@@ -317,46 +459,56 @@ mixgcn_status launch_gemm_simt(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64
         p.epi.keep_scale = epi->keep_scale; p.epi.gate = epi->gate_bits ? nullptr : epi->gate; p.epi.ld_gate = epi->ld_gate;
         p.epi.gate_scale = epi->gate_scale;
         p.epi.gate_bits = epi->gate_bits; p.epi.ld_gate_bits = epi->ld_gate_bits;
+        p.epi.sign_bits = epi->sign_bits; p.epi.ld_sign_bits = epi->ld_sign_bits;
     }
     p.epi.row0 = epi_row0;
     p.vec_a = aligned16(A) && (lda & 3) == 0;
     p.vec_b = aligned16(B) && (ldb & 3) == 0;
     p.vec_c = aligned16(C) && (ldc & 3) == 0;
-    const int bn = N <= 64 ? 64 : 128;
-    p.m_tiles = (M + BM - 1) / BM;
-    p.n_tiles = (N + bn - 1) / bn;
+    p.vec_drop = p.epi.drop && (N & 3) == 0 && (reinterpret_cast<uintptr_t>(p.epi.drop) & 3) == 0;
+    p.vec_gate = p.epi.gate && aligned16(p.epi.gate) && (p.epi.ld_gate & 3) == 0;
+    // The tile: 32 columns where N has no more, else 64 or 128 by what leaves less of N to padding, 128 rows.  Where that
+    // gives fewer CTAs than the machine has SMs even with K split, 64-row tiles.
+    auto ceil_div = [](int64_t a, int64_t b) { return (a + b - 1) / b; };
+    const bool may_split = K >= 2 * MIN_K_PER_SPLIT && (K > 1024 || ta);
+    const int64_t max_splits = may_split ? ceil_div(K, MIN_K_PER_SPLIT) : 1;
+    int bm = 128, bn = N <= 32 ? 32 : ceil_div(N, 128) * 128 > ceil_div(N, 64) * 64 ? 64 : 128;
+    if (bn == 32 || ceil_div(M, bm) * ceil_div(N, bn) * max_splits < ctx->sm_count) bm = 64;
+    if (bm == 64 && bn == 128) bn = 64;
+    p.m_tiles = ceil_div(M, bm);
+    p.n_tiles = ceil_div(N, bn);
     const int64_t tiles = p.m_tiles * p.n_tiles;
-    int splits = 1;
-    if (K > 8192 && tiles < 2 * ctx->sm_count) {
-        int64_t want = (2 * ctx->sm_count + tiles - 1) / tiles;
-        int64_t maxs = (K + 4095) / 4096;
-        splits = (int)(want < maxs ? want : maxs);
+    const int per_sm = bm == 64 ? 8 : bn == 64 ? 4 : 2;        // CTAs an SM holds
+    int64_t splits = 1;
+    if (max_splits > 1 && tiles < (int64_t)per_sm * ctx->sm_count) {
+        splits = (int64_t)per_sm * ctx->sm_count / tiles;      // one full wave
+        if (splits > max_splits) splits = max_splits;
         if (splits > 1024) splits = 1024;
-        if (splits < 1) splits = 1;
     }
-    int64_t kps = (K + splits - 1) / splits;
-    kps = ((kps + BK - 1) / BK) * BK;
+    int64_t kps = ceil_div(ceil_div(K, splits), BK) * BK;
     if (kps <= 0) kps = BK;
-    splits = (int)((K + kps - 1) / kps);
+    splits = ceil_div(K, kps);
     if (splits < 1) splits = 1;
-    p.k_per_split = kps; p.splits = splits;
+    p.k_per_split = kps; p.splits = (int)splits;
     if (splits > 1) {
-        MIXGCN_TRY(ensure_workspace(ctx, (int64_t)splits * M * N * (int64_t)sizeof(float)));
+        MIXGCN_TRY(ensure_workspace(ctx, splits * M * N * (int64_t)sizeof(float)));
         p.C = reinterpret_cast<float*>(ctx->workspace);
+        p.epi.sign_bits = nullptr;
     }
     if (tiles > 0x7FFFFFFFll) MIXGCN_FAIL(MIXGCN_EUNSUPPORTED, "gemm: too many tiles");
-    dim3 grid((unsigned)tiles, 1, (unsigned)splits);
     {
         LaunchScope scope(ctx, PH_GEMM, s);
-        if (bn == 64) launch_variant<64, 4>(p, ta, tb, grid, s);
-        else launch_variant<128, 8>(p, ta, tb, grid, s);
+        MIXGCN_CUDA(bm == 64 ? (bn == 32 ? launch_variant<64, 32, 8>(p, ta, tb, s) : launch_variant<64, 64, 8>(p, ta, tb, s))
+                             : (bn == 64 ? launch_variant<128, 64, 8>(p, ta, tb, s) : launch_variant<128, 128, 16>(p, ta, tb, s)));
     }
     if (splits > 1) {
         LaunchScope scope(ctx, PH_GEMM, s);
         const int64_t total = M * N;
-        splitk_reduce_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(M, N, splits, p.C, C, ldc, p.epi);
+        splitk_reduce_kernel<<<(unsigned)((total + 31) / 32), 32 * RED_PARTS, 0, s>>>(M, N, (int)splits, p.C, C, ldc, p.epi);
+        MIXGCN_CUDA(cudaGetLastError());
+    } else if (bits_done) {
+        *bits_done = p.epi.sign_bits != nullptr;
     }
-    MIXGCN_CUDA(cudaGetLastError());
     return MIXGCN_OK;
 }
 
@@ -370,16 +522,19 @@ mixgcn_status launch_splitk_reduce(mixgcn_ctx* ctx, int64_t M, int64_t N, int sp
     }
     LaunchScope scope(ctx, PH_GEMM, s);
     const int64_t total = M * N;
-    splitk_reduce_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(M, N, splits, part, C, ldc, e);
+    splitk_reduce_kernel<<<(unsigned)((total + 31) / 32), 32 * RED_PARTS, 0, s>>>(M, N, splits, part, C, ldc, e);
     MIXGCN_CUDA(cudaGetLastError());
     return MIXGCN_OK;
 }
 
 mixgcn_status launch_colsum(mixgcn_ctx* ctx, int64_t n, int32_t d, const float* X, int64_t ld, float* out,
                             cudaStream_t s) {
-    int64_t rows_per_block = 2048;
-    int64_t blocks = (n + rows_per_block - 1) / rows_per_block;
-    if (blocks > 2048) { rows_per_block = (n + 2047) / 2048; blocks = (n + rows_per_block - 1) / rows_per_block; }
+    // four blocks per SM, so that every SM streams; no fewer than 64 rows each, and (one wave of 2048 at most) the final
+    // pass stays short
+    int64_t blocks = 4 * (int64_t)ctx->sm_count;
+    int64_t rows_per_block = (n + blocks - 1) / blocks;
+    if (rows_per_block < 64) rows_per_block = 64;
+    blocks = (n + rows_per_block - 1) / rows_per_block;
     if (blocks < 1) blocks = 1;
     MIXGCN_TRY(ensure_workspace(ctx, blocks * d * (int64_t)sizeof(float)));
     float* part = reinterpret_cast<float*>(ctx->workspace);
@@ -391,7 +546,7 @@ mixgcn_status launch_colsum(mixgcn_ctx* ctx, int64_t n, int32_t d, const float* 
     }
     {
         LaunchScope scope(ctx, PH_ELEM, s);
-        colsum_final_kernel<<<(d + 127) / 128, 128, 0, s>>>(d, (int)blocks, part, out);
+        colsum_final_kernel<<<(d + 31) / 32, 32 * RED_PARTS, 0, s>>>(d, (int)blocks, part, out);
     }
     MIXGCN_CUDA(cudaGetLastError());
     return MIXGCN_OK;

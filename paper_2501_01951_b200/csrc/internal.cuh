@@ -296,7 +296,7 @@ mixgcn_status launch_gemm(mixgcn_ctx* ctx, int precision, int ta, int tb, int64_
                           float* colsum_b = nullptr);
 mixgcn_status launch_gemm_simt(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64_t N, int64_t K,
                                const float* A, int64_t lda, const float* B, int64_t ldb, float* C, int64_t ldc,
-                               const mixgcn_epilogue* epi, int64_t epi_row0, cudaStream_t s);
+                               const mixgcn_epilogue* epi, int64_t epi_row0, cudaStream_t s, bool* bits_done = nullptr);
 mixgcn_status launch_gemm_tc(mixgcn_ctx* ctx, int kind, int ta, int tb, int64_t M, int64_t N, int64_t K, const void* A,
                              int64_t lda, const void* B, int64_t ldb, float* C, int64_t ldc,
                              const mixgcn_epilogue* epi, int64_t epi_row0, cudaStream_t s, uint16_t* C_lp, int64_t ldc_lp,

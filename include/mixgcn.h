@@ -129,6 +129,21 @@ mixgcn_status mixgcn_ctx_profile_enable(mixgcn_ctx* ctx, int enable);
 mixgcn_status mixgcn_ctx_profile_read(mixgcn_ctx* ctx, double ms[MIXGCN_N_PHASES],
                                       int64_t launches[MIXGCN_N_PHASES], int64_t* launches_total);
 
+/* Recorded call sequences (CUDA graphs).  A training iteration on a small graph is some thirty launches of a few
+ * microseconds each, and its length is what the host needs to issue them; recorded once, the sequence is one launch.
+ * mixgcn_record_begin starts recording and returns a stream: compute calls of this context issued on that stream until
+ * mixgcn_record_end are recorded, not executed.  A call that would have to allocate or to synchronise fails while
+ * recording (run the sequence once before recording it); record_end then fails too, and nothing is left behind.
+ * mixgcn_replay enqueues the recorded calls on `stream` with the arguments they were recorded with: the same pointers
+ * (whose memory must still be the caller's), sizes and scalars.  It returns MIXGCN_EUNSUPPORTED, and enqueues nothing,
+ * when the recording no longer stands for the calls -- scratch of the context has moved, an option has changed, or
+ * profiling is on; issue the calls themselves then.  A recording may be destroyed after its context, not replayed. */
+typedef struct mixgcn_recording mixgcn_recording;
+mixgcn_status mixgcn_record_begin(mixgcn_ctx* ctx, void** stream);
+mixgcn_status mixgcn_record_end(mixgcn_ctx* ctx, mixgcn_recording** out);
+mixgcn_status mixgcn_replay(mixgcn_recording* rec, void* stream);
+mixgcn_status mixgcn_recording_destroy(mixgcn_recording* rec);
+
 /* ------------------------------------------------------------------------------------------
  * Graph: the propagation matrix A_hat = D^-1/2 (A + I) D^-1/2 with D_uu = sum_v (A+I)_uv
  * (Section 2.1), kept in CSR (the adjacency index format of Section 3.2.1) together with the

@@ -8,7 +8,9 @@ module without a built ``libmixgcn.so`` raises: there is no fallback path.
 from __future__ import annotations
 
 import ctypes as C
+import gc
 import os
+import threading
 
 import torch
 
@@ -51,6 +53,7 @@ SYMBOLS = (
     "mixgcn_rowplan_export", "mixgcn_spmm_rowplan", "mixgcn_colsum", "mixgcn_ctx_gemm_paths",
     "mixgcn_train_step_host_prefetch", "mixgcn_probe_gather", "mixgcn_spmm_sampled", "mixgcn_mask_pack",
     "mixgcn_build_info", "mixgcn_debug_poke_col", "mixgcn_layer_fwd_loss",
+    "mixgcn_record_begin", "mixgcn_record_end", "mixgcn_replay", "mixgcn_recording_destroy",
 )
 
 
@@ -96,8 +99,12 @@ def _ptr(t):
     return None if t is None else C.c_void_p(t.data_ptr())
 
 
+_recording = threading.local()       # .stream: where this thread's calls go while a sequence is being recorded
+
+
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    s = getattr(_recording, "stream", None)
+    return C.c_void_p(torch.cuda.current_stream().cuda_stream) if s is None else s
 
 
 def _dev(t, dtype, name):
@@ -121,6 +128,8 @@ class Ctx:
         self.h = C.c_void_p()
         _check(lib.mixgcn_ctx_create(C.byref(self.h), C.c_int(device)))
         self.device = device
+        self.options = {}            # what ctx_set_option set, for callers that key something on it
+        self.profiling = False
 
     def close(self):
         if self.h:
@@ -159,6 +168,7 @@ OPT_GEMM_CTA_PAIRS = 5
 
 def ctx_set_option(ctx: Ctx, option: int, value: int):
     _check(lib.mixgcn_ctx_set_option(ctx.h, C.c_int32(option), C.c_int64(value)))
+    ctx.options[option] = value
 
 
 def ctx_gemm_paths(ctx: Ctx) -> dict:
@@ -170,6 +180,7 @@ def ctx_gemm_paths(ctx: Ctx) -> dict:
 
 def ctx_profile_enable(ctx: Ctx, enable: bool = True):
     _check(lib.mixgcn_ctx_profile_enable(ctx.h, C.c_int(int(enable))))
+    ctx.profiling = bool(enable)
 
 
 def ctx_profile_read(ctx: Ctx):
@@ -179,6 +190,86 @@ def ctx_profile_read(ctx: Ctx):
     tot = C.c_int64(0)
     _check(lib.mixgcn_ctx_profile_read(ctx.h, ms, ln, C.byref(tot)))
     return dict(zip(PHASES, list(ms))), dict(zip(PHASES, list(ln))), tot.value
+
+
+# ------------------------------------------------------------------------------ recorded sequences
+
+class Recording:
+    """A recorded sequence of compute calls (see mixgcn_record_begin)."""
+
+    def __init__(self, ctx: Ctx, handle):
+        self.ctx, self.h = ctx, handle
+
+    def replay(self) -> bool:
+        """Enqueue the sequence on the current stream; False (nothing enqueued) when it no longer stands for the calls."""
+        st = lib.mixgcn_replay(self.h, _stream())
+        if st == EUNSUPPORTED:
+            return False
+        _check(st)
+        return True
+
+    def close(self):
+        if self.h:
+            lib.mixgcn_recording_destroy(self.h)
+            self.h = C.c_void_p()
+
+    def __del__(self):
+        try:
+            self.close()
+        except Exception:
+            pass
+
+
+def record(ctx: Ctx, calls):
+    """Run `calls()` with every compute call of `ctx` recorded instead of executed -> Recording, or None if the sequence
+    cannot be recorded."""
+    stream, h = C.c_void_p(), C.c_void_p()
+    if lib.mixgcn_record_begin(ctx.h, C.byref(stream)) != OK:
+        return None
+    _recording.stream = stream
+    collect = gc.isenabled()
+    gc.disable()                     # a collected graph or context would synchronise, which ends a recording
+    try:
+        calls()
+    except MixgcnError:
+        pass                         # the recording is void; record_end says so
+    finally:
+        _recording.stream = None
+        st = lib.mixgcn_record_end(ctx.h, C.byref(h))
+        if collect:
+            gc.enable()
+    return Recording(ctx, h) if st == OK else None
+
+
+class Replayer:
+    """Runs a sequence of calls that a training loop issues again and again: twice call by call, then from a recording.
+    `key` is whatever decides what the calls do (pointers, flags, sizes); the recording is made when the same key
+    has come twice and the calls leave it as it was, and used while it stays the same."""
+
+    def __init__(self, ctx: Ctx):
+        self.ctx, self.key, self.rec, self.refused = ctx, None, None, None
+
+    def run(self, key, calls):
+        """key(): the current key; calls(): issues the calls."""
+        if self.ctx.profiling or getattr(_recording, "stream", None) is not None or torch.cuda.is_current_stream_capturing():
+            calls()
+            return
+        k = key()
+        if k == self.key:
+            if self.rec is not None and self.rec.replay():
+                return
+            if self.refused != k:
+                self.rec = record(self.ctx, calls)
+                if self.rec is not None and key() == k and self.rec.replay():
+                    return
+                self.rec, self.refused = None, k
+            calls()
+            self.key = key()
+            return
+        calls()
+        # (a key that changed while the calls ran is not yet at rest)
+        self.key = k if key() == k else None
+        self.rec = None
 
 
 # ------------------------------------------------------------------------------ graph

@@ -252,6 +252,8 @@ extern "C" mixgcn_status mixgcn_ctx_destroy(mixgcn_ctx* ctx) {
     for (int i = 0; i < 64; ++i) if (ctx->chunk_ev[i]) cudaEventDestroy(ctx->chunk_ev[i]);
     for (int i = 0; i < 2; ++i) { if (ctx->join_ev[i]) cudaEventDestroy(ctx->join_ev[i]); if (ctx->side_stream[i]) cudaStreamDestroy(ctx->side_stream[i]); }
     if (ctx->fork_ev) cudaEventDestroy(ctx->fork_ev);
+    if (ctx->recording) { mixgcn_recording* none = nullptr; mixgcn_record_end(ctx, &none); mixgcn_recording_destroy(none); }
+    if (ctx->record_stream) cudaStreamDestroy(ctx->record_stream);
     free_step_cache(ctx);
     for (void* block : {ctx->workspace, ctx->workspace_spmm, ctx->workspace_rows, ctx->workspace_lp, ctx->workspace_loss, ctx->arena}) dev_free(block, nullptr);
     cudaFree(ctx->d_status);
@@ -361,6 +363,104 @@ extern "C" mixgcn_status mixgcn_ctx_profile_read(mixgcn_ctx* ctx, double ms[MIXG
     ctx->n_spans = 0;
     if (launches) for (int i = 0; i < MIXGCN_N_PHASES; ++i) { launches[i] = ctx->phase_launches[i]; ctx->phase_launches[i] = 0; }
     if (launches_total) *launches_total = ctx->launches_total;
+    return MIXGCN_OK;
+}
+
+// ------------------------------------------------------------------------------------------------
+// Recorded call sequences
+// ------------------------------------------------------------------------------------------------
+
+namespace {
+// What a context counts and what decides how it issues a call.
+struct CtxState {
+    int64_t launches_total, phase_launches[MIXGCN_N_PHASES], gemm_path[3], gemm_pair_launches;
+    int options[5];
+    uint64_t blocks_generation;
+    explicit CtxState(const mixgcn_ctx* c) : launches_total(c->launches_total), gemm_pair_launches(c->gemm_pair_launches),
+        options{c->no_cta_pairs, c->debug_wait_limit, c->debug_drop_load, c->spmm_slice_cols, c->loss_train_rows_only}, blocks_generation(c->blocks_generation) {
+        for (int i = 0; i < MIXGCN_N_PHASES; ++i) phase_launches[i] = c->phase_launches[i];
+        for (int i = 0; i < 3; ++i) gemm_path[i] = c->gemm_path[i];
+    }
+};
+}  // namespace
+
+struct mixgcn_recording {
+    mixgcn_ctx* ctx;
+    int device;
+    cudaGraphExec_t exec;
+    CtxState before, counted;      // state when recording began; launches and products the sequence adds to the counters
+    explicit mixgcn_recording(mixgcn_ctx* c) : ctx(c), device(c->device), exec(nullptr), before(c), counted(c) {}
+};
+
+extern "C" mixgcn_status mixgcn_record_begin(mixgcn_ctx* ctx, void** stream) {
+    if (!ctx || !stream) MIXGCN_FAIL(MIXGCN_EINVAL, "record_begin: null argument");
+    if (ctx->recording) MIXGCN_FAIL(MIXGCN_EINVAL, "record_begin: already recording");
+    if (ctx->profile) MIXGCN_FAIL(MIXGCN_EUNSUPPORTED, "record_begin: profiling brackets every launch; switch it off to record");
+    MIXGCN_CUDA(cudaSetDevice(ctx->device));
+    if (!ctx->record_stream) MIXGCN_CUDA(cudaStreamCreateWithFlags(&ctx->record_stream, cudaStreamNonBlocking));
+    mixgcn_recording* r = new (std::nothrow) mixgcn_recording(ctx);
+    if (!r) MIXGCN_FAIL(MIXGCN_ENOMEM, "record_begin: host allocation failed");
+    const cudaError_t e = cudaStreamBeginCapture(ctx->record_stream, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        delete r;
+        MIXGCN_FAIL(MIXGCN_ECUDA, "record_begin: %s", cudaGetErrorString(e));
+    }
+    ctx->recording = r;
+    *stream = ctx->record_stream;
+    return MIXGCN_OK;
+}
+
+extern "C" mixgcn_status mixgcn_record_end(mixgcn_ctx* ctx, mixgcn_recording** out) {
+    if (!ctx || !out) MIXGCN_FAIL(MIXGCN_EINVAL, "record_end: null argument");
+    *out = nullptr;
+    mixgcn_recording* r = ctx->recording;
+    if (!r) MIXGCN_FAIL(MIXGCN_EINVAL, "record_end: not recording");
+    ctx->recording = nullptr;
+    MIXGCN_CUDA(cudaSetDevice(ctx->device));
+    // what the recorded calls counted has not run: the counters go back, replays add it
+    CtxState& c = r->counted;
+    c = CtxState(ctx);
+    c.launches_total -= r->before.launches_total; ctx->launches_total = r->before.launches_total;
+    for (int i = 0; i < MIXGCN_N_PHASES; ++i) { c.phase_launches[i] -= r->before.phase_launches[i]; ctx->phase_launches[i] = r->before.phase_launches[i]; }
+    for (int i = 0; i < 3; ++i) { c.gemm_path[i] -= r->before.gemm_path[i]; ctx->gemm_path[i] = r->before.gemm_path[i]; }
+    c.gemm_pair_launches -= r->before.gemm_pair_launches; ctx->gemm_pair_launches = r->before.gemm_pair_launches;
+    cudaGraph_t graph = nullptr;
+    cudaError_t e = cudaStreamEndCapture(ctx->record_stream, &graph);
+    if (e == cudaSuccess && graph) e = cudaGraphInstantiate(&r->exec, graph, 0);
+    if (graph) cudaGraphDestroy(graph);
+    if (e != cudaSuccess || !r->exec || ctx->blocks_generation != r->before.blocks_generation) {
+        cudaGetLastError();
+        if (r->exec) cudaGraphExecDestroy(r->exec);
+        delete r;
+        MIXGCN_FAIL(MIXGCN_ECUDA, "record_end: the calls could not be recorded (%s)", e == cudaSuccess ? "scratch was reallocated" : cudaGetErrorString(e));
+    }
+    *out = r;
+    return MIXGCN_OK;
+}
+
+extern "C" mixgcn_status mixgcn_replay(mixgcn_recording* r, void* stream) {
+    if (!r) MIXGCN_FAIL(MIXGCN_EINVAL, "replay: null recording");
+    mixgcn_ctx* ctx = r->ctx;
+    const CtxState now(ctx);
+    if (ctx->profile || now.blocks_generation != r->before.blocks_generation || memcmp(now.options, r->before.options, sizeof(now.options)) != 0)
+        MIXGCN_FAIL(MIXGCN_EUNSUPPORTED, "replay: scratch or options of the context have changed, or profiling is on");
+    MIXGCN_CUDA(cudaSetDevice(ctx->device));
+    MIXGCN_CUDA(cudaGraphLaunch(r->exec, (cudaStream_t)stream));
+    const CtxState& c = r->counted;
+    ctx->launches_total += c.launches_total;
+    for (int i = 0; i < MIXGCN_N_PHASES; ++i) ctx->phase_launches[i] += c.phase_launches[i];
+    for (int i = 0; i < 3; ++i) ctx->gemm_path[i] += c.gemm_path[i];
+    ctx->gemm_pair_launches += c.gemm_pair_launches;
+    return MIXGCN_OK;
+}
+
+extern "C" mixgcn_status mixgcn_recording_destroy(mixgcn_recording* r) {
+    if (!r) return MIXGCN_OK;
+    cudaSetDevice(r->device);
+    cudaDeviceSynchronize();           // a replay may still be in flight
+    cudaGraphExecDestroy(r->exec);
+    delete r;
     return MIXGCN_OK;
 }
 

@@ -77,18 +77,17 @@ __device__ __forceinline__ void copy4(float* dst, const float* src, int64_t vali
 //   contiguous (the small weight matrix of dP W^T) is turned round by word-wide copies.
 // Long reductions: after 1024 terms the accumulators are added to C (the partial tile or C itself), which serves as the
 // second-level sum.
-template <int BM, int BN, int TN>
+template <int BM, int BN, int TM, int TN>
 struct SimtCfg {
-    static constexpr int NT = BM * BN / (8 * TN);                        // threads
-    static constexpr int MIN_CTAS = BM == 128 ? (BN == 128 ? 2 : 4) : BN == 64 ? 6 : 10;
+    static constexpr int NT = BM * BN / (TM * TN);                       // threads
+    static constexpr int MIN_CTAS = TM == 4 ? 1 : BM == 128 ? (BN == 128 ? 2 : 4) : BN == 64 ? 6 : 10;
 };
 
-template <int BM, int BN, int TN, bool TA, bool TB>
-__global__ void __launch_bounds__(SimtCfg<BM, BN, TN>::NT, SimtCfg<BM, BN, TN>::MIN_CTAS) gemm_simt_kernel(const GemmParams p) {
-    constexpr int NT = SimtCfg<BM, BN, TN>::NT, TX = BN / TN, Q = TN / 4, QW = BN / Q;   // Q groups of four columns, QW columns apart
+template <int BM, int BN, int TM, int TN, bool TA, bool TB>
+__global__ void __launch_bounds__(SimtCfg<BM, BN, TM, TN>::NT, SimtCfg<BM, BN, TM, TN>::MIN_CTAS) gemm_simt_kernel(const GemmParams p) {
+    constexpr int NT = SimtCfg<BM, BN, TM, TN>::NT, H = TM / 4, TX = BN / TN, Q = TN / 4, QW = BN / Q;   // Q groups of four columns, QW columns apart
     constexpr int A_PITCH = TA ? BM + 4 : BK + 4, B_PITCH = BN + 4;
     constexpr int A_FLOATS = TA ? BK * A_PITCH : BM * A_PITCH, B_FLOATS = BK * B_PITCH;
-    constexpr int A_V = BM * BK / 4 / NT;
     extern __shared__ __align__(16) float smem_f[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // a warp covers 4 x 8 micro-tiles (TX >= 8) or 8 x 4
@@ -99,36 +98,48 @@ __global__ void __launch_bounds__(SimtCfg<BM, BN, TN>::NT, SimtCfg<BM, BN, TN>::
     const int64_t kb = (int64_t)blockIdx.z * p.k_per_split;
     const int64_t ke = (kb + p.k_per_split < p.K) ? kb + p.k_per_split : p.K;
     const int steps = (int)((ke - kb + BK - 1) / BK);
-    // rows of the micro-tile: i-th row is ty + i * (BM / 8) with A as [m][k], (i / 4) * (BM / 2) + ty * 4 + i % 4 as [k][m];
+    // rows of the micro-tile: i-th row is ty + i * (BM / TM) with A as [m][k], (i / 4) * (BM / H) + ty * 4 + i % 4 as [k][m];
     // columns: (j / 4) * QW + tx * 4 + j % 4
-    auto row_of = [&](int i) { return TA ? (i >> 2) * (BM / 2) + ty * 4 + (i & 3) : ty + i * (BM / 8); };
+    auto row_of = [&](int i) { return TA ? (i >> 2) * (BM / H) + ty * 4 + (i & 3) : ty + i * (BM / TM); };
 
     auto load_a = [&](int ks) {
         float* As = smem_f + (ks % STAGES) * (A_FLOATS + B_FLOATS);
         const int64_t k0 = kb + (int64_t)ks * BK;
-#pragma unroll
-        for (int i = 0; i < A_V; ++i) {
+        auto one = [&](int i, int vec) {
             const int f = tid + i * NT;
             if (!TA) {
                 const int r = f / 4, kq = (f % 4) * 4;
                 const int64_t m = m0 + r, k = k0 + kq;
-                copy4(As + r * A_PITCH + kq, p.A + m * p.lda + k, m < p.M ? ke - k : 0, p.vec_a, p.A);
+                copy4(As + r * A_PITCH + kq, p.A + m * p.lda + k, m < p.M ? ke - k : 0, vec, p.A);
             } else {
                 const int kr = f / (BM / 4), mq = (f % (BM / 4)) * 4;
                 const int64_t k = k0 + kr, m = m0 + mq;
-                copy4(As + kr * A_PITCH + mq, p.A + k * p.lda + m, k < ke ? p.M - m : 0, p.vec_a, p.A);
+                copy4(As + kr * A_PITCH + mq, p.A + k * p.lda + m, k < ke ? p.M - m : 0, vec, p.A);
             }
+        };
+        if (p.vec_a) {
+#pragma unroll
+            for (int i = 0; i < BM * BK / 4 / NT; ++i) one(i, 1);
+        } else {
+#pragma unroll 1
+            for (int i = 0; i < BM * BK / 4 / NT; ++i) one(i, 0);
         }
     };
     auto load_b = [&](int ks) {
         float* Bs = smem_f + (ks % STAGES) * (A_FLOATS + B_FLOATS) + A_FLOATS;
         const int64_t k0 = kb + (int64_t)ks * BK;
         if constexpr (!TB) {
-#pragma unroll
-            for (int i = 0; i < BK * BN / 4 / NT; ++i) {
+            auto one = [&](int i, int vec) {
                 const int f = tid + i * NT, kr = f / (BN / 4), nq = (f % (BN / 4)) * 4;
                 const int64_t k = k0 + kr, n = n0 + nq;
-                copy4(Bs + kr * B_PITCH + nq, p.B + k * p.ldb + n, k < ke ? p.N - n : 0, p.vec_b, p.B);
+                copy4(Bs + kr * B_PITCH + nq, p.B + k * p.ldb + n, k < ke ? p.N - n : 0, vec, p.B);
+            };
+            if (p.vec_b) {
+#pragma unroll
+                for (int i = 0; i < BK * BN / 4 / NT; ++i) one(i, 1);
+            } else {
+#pragma unroll 1
+                for (int i = 0; i < BK * BN / 4 / NT; ++i) one(i, 0);
             }
         } else {
             // word by word: sixteen lanes read one row's 64 bytes and write a column of the tile
@@ -143,9 +154,9 @@ __global__ void __launch_bounds__(SimtCfg<BM, BN, TN>::NT, SimtCfg<BM, BN, TN>::
     };
     auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
 
-    f32x2 acc[8][TN / 2];
+    f32x2 acc[TM][TN / 2];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < TM; ++i)
 #pragma unroll
         for (int j = 0; j < TN / 2; ++j) acc[i][j] = 0ull;
 
@@ -159,7 +170,7 @@ __global__ void __launch_bounds__(SimtCfg<BM, BN, TN>::NT, SimtCfg<BM, BN, TN>::
         int64_t m0c;
         asm volatile("mov.b64 %0, %1;" : "=l"(m0c) : "l"(m0));
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
+        for (int i = 0; i < TM; ++i)
 #pragma unroll
             for (int q = 0; q < Q; ++q) {
                 const int64_t m = m0c + row_of(i), n = n0 + q * QW + tx * 4;
@@ -172,26 +183,27 @@ __global__ void __launch_bounds__(SimtCfg<BM, BN, TN>::NT, SimtCfg<BM, BN, TN>::
             }
     };
 
-#pragma unroll
-    for (int ks = 0; ks < STAGES - 1; ++ks) {
-        if (ks < steps) { load_a(ks); load_b(ks); }
-        commit();
-    }
+    // One loop body serves the filling of the pipeline and the steps themselves: a small product runs each line of this code
+    // once or a few times, and then its length is its time.
     bool flushed = false;
     int since_flush = 0;
-    for (int ks = 0; ks < steps; ++ks) {
-        asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
-        __syncthreads();                       // step ks has landed; the stage of step ks - 1 is free
+#pragma unroll 1
+    for (int ks = 1 - STAGES; ks < steps; ++ks) {
+        if (ks >= 0) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+            __syncthreads();                   // step ks has landed; the stage of step ks - 1 is free
+        }
         if (ks + STAGES - 1 < steps) { load_a(ks + STAGES - 1); load_b(ks + STAGES - 1); }
         commit();
+        if (ks < 0) continue;
         const float* As = smem_f + (ks % STAGES) * (A_FLOATS + B_FLOATS);
         const float* Bs = As + A_FLOATS;
-#pragma unroll (TA ? BK / 2 : 2)        // (with the row-wise A a longer body gains nothing and spills)
+#pragma unroll (TA && TM == 8 ? BK / 2 : 2)        // (with the row-wise A a longer body gains nothing and spills)
         for (int kk = 0; kk < BK; kk += 2) {
-            float2 a2[8];
+            float2 a2[TM];
             if (!TA) {
 #pragma unroll
-                for (int i = 0; i < 8; ++i) a2[i] = *reinterpret_cast<const float2*>(As + (ty + i * (BM / 8)) * A_PITCH + kk);
+                for (int i = 0; i < TM; ++i) a2[i] = *reinterpret_cast<const float2*>(As + (ty + i * (BM / TM)) * A_PITCH + kk);
             }
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
@@ -199,17 +211,20 @@ __global__ void __launch_bounds__(SimtCfg<BM, BN, TN>::NT, SimtCfg<BM, BN, TN>::
                 ulonglong2 b[Q];
 #pragma unroll
                 for (int q = 0; q < Q; ++q) b[q] = *reinterpret_cast<const ulonglong2*>(brow + q * QW);
-                float a[8];
+                float a[TM];
                 if (!TA) {
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) a[i] = k == 0 ? a2[i].x : a2[i].y;
+                    for (int i = 0; i < TM; ++i) a[i] = k == 0 ? a2[i].x : a2[i].y;
                 } else {
                     const float* arow = As + (kk + k) * A_PITCH + ty * 4;
-                    const float4 x = *reinterpret_cast<const float4*>(arow), y = *reinterpret_cast<const float4*>(arow + BM / 2);
-                    a[0] = x.x; a[1] = x.y; a[2] = x.z; a[3] = x.w; a[4] = y.x; a[5] = y.y; a[6] = y.z; a[7] = y.w;
+#pragma unroll
+                    for (int g = 0; g < H; ++g) {
+                        const float4 x = *reinterpret_cast<const float4*>(arow + g * (BM / H));
+                        a[4 * g] = x.x; a[4 * g + 1] = x.y; a[4 * g + 2] = x.z; a[4 * g + 3] = x.w;
+                    }
                 }
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
+                for (int i = 0; i < TM; ++i) {
                     const f32x2 av = dup2(a[i]);
 #pragma unroll
                     for (int q = 0; q < Q; ++q) { ffma2(acc[i][2 * q], av, b[q].x); ffma2(acc[i][2 * q + 1], av, b[q].y); }
@@ -224,14 +239,14 @@ __global__ void __launch_bounds__(SimtCfg<BM, BN, TN>::NT, SimtCfg<BM, BN, TN>::
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 
-    // Epilogue through shared memory, half of the rows at a time: a warp then stores (and reads gates and masks of) whole
+    // Epilogue through shared memory, four rows of every thread (half of the tile) at a time: a warp then stores (and reads gates and masks of) whole
     // rows, and its code is one short loop.  Applied from the registers it was unrolled over the micro-tile, thirty
     // kilobytes of branches that cost more than 128 terms of K (170 K x 256, K = 128: 617 us).
     constexpr int S_PITCH = BN + 4, ROW4 = BN / 4;
     const Epi& e = p.epi;
     float* const S = smem_f;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < H; ++h) {
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < 4; ++i)
@@ -242,9 +257,9 @@ __global__ void __launch_bounds__(SimtCfg<BM, BN, TN>::NT, SimtCfg<BM, BN, TN>::
             }
         __syncthreads();
 #pragma unroll 2
-        for (int f = tid; f < BM / 2 * ROW4; f += NT) {
+        for (int f = tid; f < BM / H * ROW4; f += NT) {
             const int lr = f / ROW4, lc = (f % ROW4) * 4;
-            const int64_t m = m0 + h * (BM / 2) + lr, n = n0 + lc;
+            const int64_t m = m0 + h * (BM / H) + lr, n = n0 + lc;
             const bool in = m < p.M && n < p.N, full = n + 3 < p.N;
             const float4 v = *reinterpret_cast<const float4*>(S + lr * S_PITCH + lc);
             float r[4] = {v.x, v.y, v.z, v.w};
@@ -421,25 +436,25 @@ __global__ void gate_kernel(int64_t n, int d, float* __restrict__ G, int64_t ldg
     G[r * ldg + j] = g;
 }
 
-template <int BM, int BN, int TN, bool TA, bool TB>
+template <int BM, int BN, int TM, int TN, bool TA, bool TB>
 cudaError_t launch_form(const GemmParams& p, cudaStream_t s) {
     constexpr int a_floats = TA ? BK * (BM + 4) : BM * (BK + 4), b_floats = BK * (BN + 4);
-    constexpr int ring = STAGES * (a_floats + b_floats), half_tile = BM / 2 * (BN + 4);
+    constexpr int ring = STAGES * (a_floats + b_floats), half_tile = BM / (TM / 4) * (BN + 4);
     constexpr int smem = (ring > half_tile ? ring : half_tile) * (int)sizeof(float);
     if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(gemm_simt_kernel<BM, BN, TN, TA, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        const cudaError_t e = cudaFuncSetAttribute(gemm_simt_kernel<BM, BN, TM, TN, TA, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
     }
-    gemm_simt_kernel<BM, BN, TN, TA, TB><<<dim3((unsigned)(p.m_tiles * p.n_tiles), 1, (unsigned)p.splits), SimtCfg<BM, BN, TN>::NT, smem, s>>>(p);
+    gemm_simt_kernel<BM, BN, TM, TN, TA, TB><<<dim3((unsigned)(p.m_tiles * p.n_tiles), 1, (unsigned)p.splits), SimtCfg<BM, BN, TM, TN>::NT, smem, s>>>(p);
     return cudaGetLastError();
 }
 
-template <int BM, int BN, int TN>
+template <int BM, int BN, int TM, int TN>
 cudaError_t launch_variant(const GemmParams& p, int ta, int tb, cudaStream_t s) {
-    if (!ta && !tb) return launch_form<BM, BN, TN, false, false>(p, s);
-    if (!ta) return launch_form<BM, BN, TN, false, true>(p, s);
-    if (!tb) return launch_form<BM, BN, TN, true, false>(p, s);
-    return launch_form<BM, BN, TN, true, true>(p, s);
+    if (!ta && !tb) return launch_form<BM, BN, TM, TN, false, false>(p, s);
+    if (!ta) return launch_form<BM, BN, TM, TN, false, true>(p, s);
+    if (!tb) return launch_form<BM, BN, TM, TN, true, false>(p, s);
+    return launch_form<BM, BN, TM, TN, true, true>(p, s);
 }
 
 }  // namespace
@@ -498,8 +513,12 @@ mixgcn_status launch_gemm_simt(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64
     if (tiles > 0x7FFFFFFFll) MIXGCN_FAIL(MIXGCN_EUNSUPPORTED, "gemm: too many tiles");
     {
         LaunchScope scope(ctx, PH_GEMM, s);
-        MIXGCN_CUDA(bm == 64 ? (bn == 32 ? launch_variant<64, 32, 8>(p, ta, tb, s) : launch_variant<64, 64, 8>(p, ta, tb, s))
-                             : (bn == 64 ? launch_variant<128, 64, 8>(p, ta, tb, s) : launch_variant<128, 128, 16>(p, ta, tb, s)));
+        // 64-row tiles: 4 x 4 micro-tiles (four times the warps, half the rate) where 8 x 8 ones would leave an SM fewer
+        // than eight warps: such a product lasts as long as one tile does
+        const bool fine = bm == 64 && tiles * splits * (bn / 32) < 8 * (int64_t)ctx->sm_count;
+        MIXGCN_CUDA(fine ? (bn == 32 ? launch_variant<64, 32, 4, 4>(p, ta, tb, s) : launch_variant<64, 64, 4, 4>(p, ta, tb, s))
+                    : bm == 64 ? (bn == 32 ? launch_variant<64, 32, 8, 8>(p, ta, tb, s) : launch_variant<64, 64, 8, 8>(p, ta, tb, s))
+                               : (bn == 64 ? launch_variant<128, 64, 8, 8>(p, ta, tb, s) : launch_variant<128, 128, 8, 16>(p, ta, tb, s)));
     }
     if (splits > 1) {
         LaunchScope scope(ctx, PH_GEMM, s);

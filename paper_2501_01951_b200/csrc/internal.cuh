@@ -103,6 +103,9 @@ struct mixgcn_ctx {
     void* arena;
     int64_t arena_bytes;
     uint64_t blocks_generation;   // grows whenever one of the kept blocks above is replaced
+    // recording of call sequences
+    cudaStream_t record_stream;   // created by the first recording
+    struct mixgcn_recording* recording;   // the one being made, or null
     // row plans of the last mixgcn_train_step_host call, reused while graph and train mask stay the same
     struct HostStepCache* step_cache;
     struct HostStepPrefetch* step_prefetch;

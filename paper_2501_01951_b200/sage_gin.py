@@ -34,6 +34,7 @@ class _Base:
         self.pred = torch.zeros(self.n, dtype=torch.int32, device=self.device)
         self.n_correct = torch.zeros(1, dtype=torch.int64, device=self.device)
         self.params, self.grads, self.m, self.v = [], [], [], []
+        self._replay = mg.Replayer(ctx)      # the calls of an iteration, recorded once they have come twice with the same buffers
 
     def _z(self, r, c):
         return torch.zeros((r, c), dtype=torch.float32, device=self.device)
@@ -51,10 +52,21 @@ class _Base:
     def step(self, t, lr=0.01, beta1=0.9, beta2=0.999, eps=1e-8):
         mg.adam_step(self.ctx, self.params, self.grads, self.m, self.v, t, lr, beta1, beta2, eps)
 
-    def epoch(self, t, lr=0.01):
+    def _calls_key(self):
+        """Everything the issued calls depend on: every tensor the trainer holds, and the context's options."""
+        held = []
+        for v in self.__dict__.values():
+            for t in v if isinstance(v, list) else (v,):
+                held.append(t.data_ptr() if isinstance(t, torch.Tensor) else 0)
+        return tuple(held), self.precision, self.g.h.value, self.ctx.h.value, tuple(self.ctx.options.items()), getattr(self, "gin_eps", None)
+
+    def _iteration(self):
         self.forward()
         self.compute_loss()
         self.backward()
+
+    def epoch(self, t, lr=0.01):
+        self._replay.run(self._calls_key, self._iteration)
         self.step(t, lr)
 
 

@@ -128,6 +128,8 @@ class GcnTrainer:
         self.n_correct = torch.zeros(1, dtype=torch.int64, device=self.device)
         self.W = self.b = self.dW = self.db = None
         self.masks = [None] * L
+        # the calls of an iteration and of a forward pass, recorded once they have come twice with the same buffers
+        self._replays = {"iteration": mg.Replayer(ctx), "forward": mg.Replayer(ctx)}
 
     # -- parameters -----------------------------------------------------------------------------
     def set_params(self, Ws, bs):
@@ -218,11 +220,11 @@ class GcnTrainer:
     def forward_and_loss(self):
         """forward() + compute_loss() with the same results; X[L] then holds the gradient w.r.t. the logits."""
         if not self.last_layer_takes_the_loss():
-            self.forward()
+            self._forward()
             self.compute_loss()
             return
         L = self.L
-        self.forward(upto=L - 1)
+        self._forward(upto=L - 1)
         d = self.descs[L - 1]
         d.flags &= ~(mg.LAYER_SAVED_LP_ONLY | mg.LAYER_SAVED_IS_VALID)
         # rows the backward never reads need no zeros (same rule as compute_loss)
@@ -238,7 +240,21 @@ class GcnTrainer:
         if L == 1:
             self._first_aggregation_valid = self.orders[0] == mg.ORDER_AGG_FIRST
 
+    def _calls_key(self):
+        """Everything the issued calls depend on: buffers, descriptors (flags and companions among them), options."""
+        tensors = [*self.X, *self.saved, *self.G, *self.W, *self.b, *self.dW, *self.db, *self.masks, self.labels, self.train_mask,
+                   self.loss, self.pred, self.n_correct, *(self.row_masks or ())]
+        return (tuple([0 if t is None else t.data_ptr() for t in tensors]), tuple([bytes(d) for d in self.descs]), tuple(self.orders),
+                self.g.h.value, self.ctx.h.value, tuple(self.ctx.options.items()), self.train_rows_only, self.cache_first_aggregation,
+                self._first_aggregation_valid, self.saved_lp_only, self.row_sparse_levels)
+
     def forward(self, upto=None):
+        if upto is None:
+            self._replays["forward"].run(self._calls_key, self._forward)
+        else:
+            self._forward(upto)
+
+    def _forward(self, upto=None):
         d0 = self.descs[0]
         reuse = self.cache_first_aggregation and self._first_aggregation_valid and self.orders[0] == mg.ORDER_AGG_FIRST
         d0.flags = (d0.flags | mg.LAYER_SAVED_IS_VALID) if reuse else (d0.flags & ~mg.LAYER_SAVED_IS_VALID)
@@ -301,7 +317,10 @@ class GcnTrainer:
         mg.adam_step(self.ctx, self.W + self.b, self.dW + self.db, self.mW + self.mb, self.vW + self.vb, t,
                      lr, beta1, beta2, eps)
 
-    def epoch(self, t, lr=0.01):
+    def _iteration(self):
         self.forward_and_loss()
         self.backward()
+
+    def epoch(self, t, lr=0.01):
+        self._replays["iteration"].run(self._calls_key, self._iteration)
         self.step(t, lr)

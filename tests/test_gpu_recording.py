@@ -1,0 +1,87 @@
+"""Recorded iterations: what epoch() and forward() replay is bit for bit what the calls give, through every change that must
+end a recording -- other buffers, options, profiling, scratch that moved -- and the refusals."""
+import pytest
+import torch
+
+from helpers import padded
+from paper_2501_01951_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mg():
+    from paper_2501_01951_b200 import build
+    build.build()
+    from paper_2501_01951_b200 import binding
+    return binding
+
+
+def trainer(mg, precision, **kw):
+    from paper_2501_01951_b200.train import GcnTrainer
+    n, dims = 3000, (40, 24, 24, 9)
+    s, d = synth.rmat_graph(n, 20000, 5)
+    ctx = mg.ctx_create(0)
+    g = mg.graph_create(ctx, n, s, d)
+    tr = GcnTrainer(ctx, g, dims, precision, **kw)
+    tr.set_params([synth.glorot_uniform(a, b, 7 + a) for a, b in zip(dims, dims[1:])], [torch.zeros(b) for b in dims[1:]])
+    tr.set_inputs(padded(synth.uniform_tensor((n, dims[0]), 3, -1, 1)), synth.uniform_labels(n, 9, 4).cuda(), synth.bernoulli_mask(n, kw.pop("mask", 0.3), 6).cuda())
+    return ctx, g, tr
+
+
+@pytest.mark.parametrize("precision", [0, 1, 2])
+@pytest.mark.parametrize("kw", [{}, dict(row_sparse=1), dict(row_sparse=2, row_plans=False), dict(train_rows_only=True), dict(cache_first_aggregation=True), dict(n_chunks=3)])
+def test_replayed_iterations_are_the_calls(mg, precision, kw):
+    a, b = trainer(mg, precision, **kw), trainer(mg, precision, **kw)
+    for t in range(1, 9):
+        if t == 5:                                    # other parameter buffers: the recording ends
+            for _, _, tr in (a, b):
+                tr.W[1] = tr.W[1].clone()
+        if t == 7:                                    # scratch of the context moves
+            for ctx, _, _ in (a, b):
+                mg.ctx_reserve(ctx, 64 << 20)
+        a[2].epoch(t)
+        b[2]._iteration()
+        b[2].step(t)
+    assert a[2]._replays["iteration"].rec is not None
+    for x, y in zip(a[2].W + a[2].b + a[2].dW + a[2].mW + [a[2].loss, a[2].pred], b[2].W + b[2].b + b[2].dW + b[2].mW + [b[2].loss, b[2].pred]):
+        assert torch.equal(x, y)
+    for _ in range(3):
+        a[2].forward()
+    b[2]._forward()
+    assert torch.equal(a[2].X[-1], b[2].X[-1])
+    for ctx, _, _ in (a, b):
+        assert mg.ctx_poll_status(ctx, raise_on_error=False) == 0
+
+
+def test_launches_are_counted_and_profiling_sees_every_kernel(mg):
+    ctx, g, tr = trainer(mg, mg.PREC_TF32)
+    total = lambda: mg.ctx_profile_read(ctx)[2]
+    counts = []
+    for t in range(1, 6):
+        before, paths = total(), mg.ctx_gemm_paths(ctx)["tc_tf32"]
+        tr.epoch(t)
+        counts.append((total() - before, mg.ctx_gemm_paths(ctx)["tc_tf32"] - paths))
+    assert counts[-1] == counts[1] and counts[1][0] > 10 and tr._replays["iteration"].rec is not None
+    mg.ctx_profile_enable(ctx, True)
+    mg.ctx_profile_read(ctx)
+    tr.epoch(6)
+    ms, launches, _ = mg.ctx_profile_read(ctx)
+    mg.ctx_profile_enable(ctx, False)
+    assert launches["spmm"] > 0 and ms["spmm"] > 0
+    tr.epoch(7)
+    assert mg.ctx_poll_status(ctx, raise_on_error=False) == 0
+
+
+def test_recording_is_refused_where_calls_would_allocate(mg):
+    ctx, g, tr = trainer(mg, mg.PREC_FP32)
+    assert mg.record(ctx, lambda: mg.ctx_reserve(ctx, 1 << 28)) is None
+    tr.epoch(1)                                       # the context goes on
+    rec = mg.record(ctx, tr._iteration)
+    assert rec is not None and rec.replay()
+    mg.ctx_set_option(ctx, mg.OPT_SPMM_SLICE_COLS, 8)
+    assert not rec.replay()
+    mg.ctx_set_option(ctx, mg.OPT_SPMM_SLICE_COLS, 0)
+    assert rec.replay()
+    torch.cuda.synchronize()
+    assert mg.ctx_poll_status(ctx, raise_on_error=False) == 0

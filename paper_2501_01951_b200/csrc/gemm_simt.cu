@@ -77,19 +77,24 @@ __device__ __forceinline__ void copy4(float* dst, const float* src, int64_t vali
 //   contiguous (the small weight matrix of dP W^T) is turned round by word-wide copies.
 // Long reductions: after 1024 terms the accumulators are added to C (the partial tile or C itself), which serves as the
 // second-level sum.
-template <int BM, int BN, int TM, int TN>
+// KG > 1: KG groups of threads share a tile, each taking every KG-th part of a k-step; their sums are added, in order, in the
+// epilogue's shared memory.  Small products have few tiles: the tile's length is then the product's, and KG warps walk it
+// in a KG-th of the time without the smaller micro-tile's extra shared-memory traffic.
+template <int BM, int BN, int TN, int KG>
 struct SimtCfg {
-    static constexpr int NT = BM * BN / (TM * TN);                       // threads
-    static constexpr int MIN_CTAS = TM == 4 ? 1 : BM == 128 ? (BN == 128 ? 2 : 4) : BN == 64 ? 6 : 10;
+    static constexpr int GROUP = BM * BN / (8 * TN), NT = GROUP * KG;    // threads of a group, of the CTA
+    static constexpr int MIN_CTAS = BM == 128 ? (BN == 128 ? 2 : 4) : (BN == 64 ? 6 : 10) / KG;
 };
+constexpr int FINE_KG = 4;
 
-template <int BM, int BN, int TM, int TN, bool TA, bool TB>
-__global__ void __launch_bounds__(SimtCfg<BM, BN, TM, TN>::NT, SimtCfg<BM, BN, TM, TN>::MIN_CTAS) gemm_simt_kernel(const GemmParams p) {
-    constexpr int NT = SimtCfg<BM, BN, TM, TN>::NT, H = TM / 4, TX = BN / TN, Q = TN / 4, QW = BN / Q;   // Q groups of four columns, QW columns apart
+template <int BM, int BN, int TN, int KG, bool TA, bool TB>
+__global__ void __launch_bounds__(SimtCfg<BM, BN, TN, KG>::NT, SimtCfg<BM, BN, TN, KG>::MIN_CTAS) gemm_simt_kernel(const GemmParams p) {
+    constexpr int TM = 8, NT = SimtCfg<BM, BN, TN, KG>::NT, H = TM / 4, TX = BN / TN, Q = TN / 4, QW = BN / Q;   // Q groups of four columns, QW columns apart
     constexpr int A_PITCH = TA ? BM + 4 : BK + 4, B_PITCH = BN + 4;
     constexpr int A_FLOATS = TA ? BK * A_PITCH : BM * A_PITCH, B_FLOATS = BK * B_PITCH;
     extern __shared__ __align__(16) float smem_f[];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int kg = tid / SimtCfg<BM, BN, TN, KG>::GROUP, warp = (tid % SimtCfg<BM, BN, TN, KG>::GROUP) >> 5;
     // a warp covers 4 x 8 micro-tiles (TX >= 8) or 8 x 4
     constexpr int WX = TX >= 8 ? 8 : TX, WY = 32 / WX, WARPS_X = TX / WX;
     const int tx = (warp % WARPS_X) * WX + lane % WX, ty = (warp / WARPS_X) * WY + lane / WX;
@@ -198,8 +203,8 @@ __global__ void __launch_bounds__(SimtCfg<BM, BN, TM, TN>::NT, SimtCfg<BM, BN, T
         if (ks < 0) continue;
         const float* As = smem_f + (ks % STAGES) * (A_FLOATS + B_FLOATS);
         const float* Bs = As + A_FLOATS;
-#pragma unroll (TA && TM == 8 ? BK / 2 : 2)        // (with the row-wise A a longer body gains nothing and spills)
-        for (int kk = 0; kk < BK; kk += 2) {
+#pragma unroll (TA && KG == 1 ? BK / 2 : 2)        // (with the row-wise A a longer body gains nothing and spills)
+        for (int kk = kg * (BK / KG); kk < (kg + 1) * (BK / KG); kk += 2) {
             float2 a2[TM];
             if (!TA) {
 #pragma unroll
@@ -231,7 +236,7 @@ __global__ void __launch_bounds__(SimtCfg<BM, BN, TM, TN>::NT, SimtCfg<BM, BN, T
                 }
             }
         }
-        if (++since_flush == FLUSH_STEPS && ks + 1 < steps) {
+        if (++since_flush == FLUSH_STEPS && ks + 1 < steps && KG == 1) {
             since_flush = 0;
             flush(!flushed);
             flushed = true;
@@ -247,14 +252,20 @@ __global__ void __launch_bounds__(SimtCfg<BM, BN, TM, TN>::NT, SimtCfg<BM, BN, T
     float* const S = smem_f;
 #pragma unroll
     for (int h = 0; h < H; ++h) {
-        __syncthreads();
+        for (int g = 0; g < KG; ++g) {
+            __syncthreads();
+            if (kg != g) continue;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int q = 0; q < Q; ++q) {
-                const float2 lo = split2(acc[h * 4 + i][q * 2]), hi = split2(acc[h * 4 + i][q * 2 + 1]);
-                *reinterpret_cast<float4*>(S + (row_of(i)) * S_PITCH + q * QW + tx * 4) = make_float4(lo.x, lo.y, hi.x, hi.y);
-            }
+                for (int q = 0; q < Q; ++q) {
+                    const float2 lo = split2(acc[h * 4 + i][q * 2]), hi = split2(acc[h * 4 + i][q * 2 + 1]);
+                    float4* cell = reinterpret_cast<float4*>(S + row_of(i) * S_PITCH + q * QW + tx * 4);
+                    float4 v = make_float4(lo.x, lo.y, hi.x, hi.y);
+                    if (KG > 1 && g > 0) { const float4 o = *cell; v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w; }
+                    *cell = v;
+                }
+        }
         __syncthreads();
 #pragma unroll 2
         for (int f = tid; f < BM / H * ROW4; f += NT) {
@@ -436,25 +447,25 @@ __global__ void gate_kernel(int64_t n, int d, float* __restrict__ G, int64_t ldg
     G[r * ldg + j] = g;
 }
 
-template <int BM, int BN, int TM, int TN, bool TA, bool TB>
+template <int BM, int BN, int TN, int KG, bool TA, bool TB>
 cudaError_t launch_form(const GemmParams& p, cudaStream_t s) {
     constexpr int a_floats = TA ? BK * (BM + 4) : BM * (BK + 4), b_floats = BK * (BN + 4);
-    constexpr int ring = STAGES * (a_floats + b_floats), half_tile = BM / (TM / 4) * (BN + 4);
+    constexpr int ring = STAGES * (a_floats + b_floats), half_tile = BM / 2 * (BN + 4);
     constexpr int smem = (ring > half_tile ? ring : half_tile) * (int)sizeof(float);
     if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(gemm_simt_kernel<BM, BN, TM, TN, TA, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        const cudaError_t e = cudaFuncSetAttribute(gemm_simt_kernel<BM, BN, TN, KG, TA, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
     }
-    gemm_simt_kernel<BM, BN, TM, TN, TA, TB><<<dim3((unsigned)(p.m_tiles * p.n_tiles), 1, (unsigned)p.splits), SimtCfg<BM, BN, TM, TN>::NT, smem, s>>>(p);
+    gemm_simt_kernel<BM, BN, TN, KG, TA, TB><<<dim3((unsigned)(p.m_tiles * p.n_tiles), 1, (unsigned)p.splits), SimtCfg<BM, BN, TN, KG>::NT, smem, s>>>(p);
     return cudaGetLastError();
 }
 
-template <int BM, int BN, int TM, int TN>
+template <int BM, int BN, int TN, int KG>
 cudaError_t launch_variant(const GemmParams& p, int ta, int tb, cudaStream_t s) {
-    if (!ta && !tb) return launch_form<BM, BN, TM, TN, false, false>(p, s);
-    if (!ta) return launch_form<BM, BN, TM, TN, false, true>(p, s);
-    if (!tb) return launch_form<BM, BN, TM, TN, true, false>(p, s);
-    return launch_form<BM, BN, TM, TN, true, true>(p, s);
+    if (!ta && !tb) return launch_form<BM, BN, TN, KG, false, false>(p, s);
+    if (!ta) return launch_form<BM, BN, TN, KG, false, true>(p, s);
+    if (!tb) return launch_form<BM, BN, TN, KG, true, false>(p, s);
+    return launch_form<BM, BN, TN, KG, true, true>(p, s);
 }
 
 }  // namespace
@@ -493,7 +504,7 @@ mixgcn_status launch_gemm_simt(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64
     p.m_tiles = ceil_div(M, bm);
     p.n_tiles = ceil_div(N, bn);
     const int64_t tiles = p.m_tiles * p.n_tiles;
-    const int per_sm = bm == 64 ? 8 : bn == 64 ? 4 : 2;        // CTAs an SM holds
+    const int per_sm = bm == 64 ? 3 : bn == 64 ? 4 : 2;        // CTAs an SM holds (64-row tiles: of four groups)
     int64_t splits = 1;
     if (max_splits > 1 && tiles < (int64_t)per_sm * ctx->sm_count) {
         splits = (int64_t)per_sm * ctx->sm_count / tiles;      // one full wave
@@ -513,12 +524,12 @@ mixgcn_status launch_gemm_simt(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64
     if (tiles > 0x7FFFFFFFll) MIXGCN_FAIL(MIXGCN_EUNSUPPORTED, "gemm: too many tiles");
     {
         LaunchScope scope(ctx, PH_GEMM, s);
-        // 64-row tiles: 4 x 4 micro-tiles (four times the warps, half the rate) where 8 x 8 ones would leave an SM fewer
-        // than eight warps: such a product lasts as long as one tile does
-        const bool fine = bm == 64 && tiles * splits * (bn / 32) < 8 * (int64_t)ctx->sm_count;
-        MIXGCN_CUDA(fine ? (bn == 32 ? launch_variant<64, 32, 4, 4>(p, ta, tb, s) : launch_variant<64, 64, 4, 4>(p, ta, tb, s))
-                    : bm == 64 ? (bn == 32 ? launch_variant<64, 32, 8, 8>(p, ta, tb, s) : launch_variant<64, 64, 8, 8>(p, ta, tb, s))
-                               : (bn == 64 ? launch_variant<128, 64, 8, 8>(p, ta, tb, s) : launch_variant<128, 128, 8, 16>(p, ta, tb, s)));
+        // 64-row tiles: four groups of threads per tile where one would leave an SM fewer than eight warps (each group's
+        // accumulators see a quarter of K, and are not flushed: up to four times 1024 terms)
+        const bool fine = bm == 64 && tiles * splits * (bn / 32) < 8 * (int64_t)ctx->sm_count && kps <= FINE_KG * FLUSH_STEPS * BK;
+        MIXGCN_CUDA(fine ? (bn == 32 ? launch_variant<64, 32, 8, FINE_KG>(p, ta, tb, s) : launch_variant<64, 64, 8, FINE_KG>(p, ta, tb, s))
+                    : bm == 64 ? (bn == 32 ? launch_variant<64, 32, 8, 1>(p, ta, tb, s) : launch_variant<64, 64, 8, 1>(p, ta, tb, s))
+                               : (bn == 64 ? launch_variant<128, 64, 8, 1>(p, ta, tb, s) : launch_variant<128, 128, 16, 1>(p, ta, tb, s)));
     }
     if (splits > 1) {
         LaunchScope scope(ctx, PH_GEMM, s);

@@ -109,6 +109,138 @@ __device__ __forceinline__ void store_lp_row(uint16_t* dst, const float (&v)[32]
     }
 }
 
+// ---- per-element masks of a tile's epilogue ----
+// An epilogue thread owns a row of the accumulator and wants a dropout mask or gate as one word per 32 columns.  The words
+// are made while the accumulator still is: bytes and fp32 gates are read with coalesced requests (a row's 32 columns by
+// eight adjacent lanes), reduced to four bits per load, and brought to the row's lane by an 8 x 8 transpose of nibbles.
+// (Applied to the staged output box instead, with a dependent byte load per element, a dropout product took three to four
+// times as long: 180 K x 128 x 128: 136 us.)
+
+// Lane (g, c) = (lane / 8, lane % 8) holds in nibble i the columns 4 c .. 4 c + 3 of row 4 i + g; returns the word of row `lane`.
+__device__ __forceinline__ uint32_t row_word_from_nibbles(uint32_t x, int lane) {
+    uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, x, 4);
+    x = (lane & 4) ? (x & 0xFFFF0000u) | (y >> 16) : (x & 0x0000FFFFu) | (y << 16);
+    y = __shfl_xor_sync(0xFFFFFFFFu, x, 2);
+    x = (lane & 2) ? (x & 0xFF00FF00u) | ((y >> 8) & 0x00FF00FFu) : (x & 0x00FF00FFu) | ((y << 8) & 0xFF00FF00u);
+    y = __shfl_xor_sync(0xFFFFFFFFu, x, 1);
+    x = (lane & 1) ? (x & 0xF0F0F0F0u) | ((y >> 4) & 0x0F0F0F0Fu) : (x & 0x0F0F0F0Fu) | ((y << 4) & 0xF0F0F0F0u);
+    return __shfl_sync(0xFFFFFFFFu, x, (lane & 3) * 8 + (lane >> 2));      // row 4 i + g now lies in lane (g, i)
+}
+
+// Words of the 32 rows from `row_first`, columns nb, nb + step, ... (CHUNKS blocks of 32), for this lane's row.
+template <int CHUNKS>
+__device__ __forceinline__ void mask_words(const TcEpi& e, int64_t row_first, int64_t M, int64_t N, int nb, int step, int nb_end, int lane,
+                                           uint32_t (&dw)[CHUNKS], uint32_t (&gw)[CHUNKS]) {
+    const int g = lane >> 3, c = lane & 7;
+#pragma unroll
+    for (int k = 0; k < CHUNKS; ++k) { dw[k] = 0xFFFFFFFFu; gw[k] = 0xFFFFFFFFu; }
+    if (nb_end > N) nb_end = (int)N;
+    if (e.drop) {
+        if ((N & 3) == 0 && (reinterpret_cast<uintptr_t>(e.drop) & 3) == 0) {
+            uint32_t x[CHUNKS][8];                       // every block's loads in flight together
+#pragma unroll
+            for (int k = 0; k < CHUNKS; ++k)
+#pragma unroll
+                for (int it = 0; it < 8; ++it) {
+                    const int64_t row = row_first + it * 4 + g;
+                    const int n = nb + k * step + c * 4;
+                    x[k][it] = (row < M && n < nb_end) ? __ldg(reinterpret_cast<const uint32_t*>(e.drop + (e.row0 + row) * N + n)) : 0u;
+                }
+#pragma unroll
+            for (int k = 0; k < CHUNKS; ++k) {
+                if (nb + k * step >= nb_end) break;
+                uint32_t nibbles = 0;
+#pragma unroll
+                for (int it = 0; it < 8; ++it) nibbles |= (((__vcmpne4(x[k][it], 0u) & 0x08040201u) * 0x01010101u) >> 24) << (4 * it);
+                dw[k] = row_word_from_nibbles(nibbles, lane);
+            }
+        } else {
+            // rows that start at any byte: one byte per lane, one request and one vote per row
+#pragma unroll
+            for (int k = 0; k < CHUNKS; ++k) {
+                const int n = nb + k * step + lane;
+                if (nb + k * step >= nb_end) break;
+                uint32_t word = 0;
+#pragma unroll
+                for (int t0 = 0; t0 < 32; t0 += 16) {
+                    uint32_t b[16];
+#pragma unroll
+                    for (int t = 0; t < 16; ++t) b[t] = (n < nb_end && row_first + t0 + t < M) ? __ldg(e.drop + (e.row0 + row_first + t0 + t) * N + n) : 0u;
+#pragma unroll
+                    for (int t = 0; t < 16; ++t) {
+                        const uint32_t w = __ballot_sync(0xFFFFFFFFu, b[t] != 0u);
+                        if (lane == t0 + t) word = w;
+                    }
+                }
+                dw[k] = word;
+            }
+        }
+    }
+    if (e.gate_bits) {
+#pragma unroll
+        for (int k = 0; k < CHUNKS; ++k)
+            if (nb + k * step < nb_end) gw[k] = row_first + lane < M ? __ldg(e.gate_bits + (e.row0 + row_first + lane) * e.ld_gate_bits + ((nb + k * step) >> 5)) : 0u;
+    } else if (e.gate) {
+        const bool vec = aligned16_dev(e.gate) && (e.ld_gate & 3) == 0;
+#pragma unroll
+        for (int k = 0; k < CHUNKS; ++k) {
+            if (nb + k * step >= nb_end) break;
+            float4 x[8];
+#pragma unroll
+            for (int it = 0; it < 8; ++it) {
+                const int64_t row = row_first + it * 4 + g;
+                const int n = nb + k * step + c * 4;
+                x[it] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (row < M && n < nb_end) {
+                    const float* src = e.gate + (e.row0 + row) * e.ld_gate + n;
+                    if (vec) x[it] = __ldg(reinterpret_cast<const float4*>(src));      // inside the row's allocation: ld_gate % 4 == 0
+                    else {
+                        x[it].x = __ldg(src);
+                        if (n + 1 < nb_end) x[it].y = __ldg(src + 1);
+                        if (n + 2 < nb_end) x[it].z = __ldg(src + 2);
+                        if (n + 3 < nb_end) x[it].w = __ldg(src + 3);
+                    }
+                }
+            }
+            uint32_t nibbles = 0;
+#pragma unroll
+            for (int it = 0; it < 8; ++it)
+                nibbles |= ((x[it].x > 0.0f ? 1u : 0u) | (x[it].y > 0.0f ? 2u : 0u) | (x[it].z > 0.0f ? 4u : 0u) | (x[it].w > 0.0f ? 8u : 0u)) << (4 * it);
+            gw[k] = row_word_from_nibbles(nibbles, lane);
+        }
+    }
+}
+
+// Bias (from shared memory, or global where `bias_smem` is null), ReLU, dropout and gate on 32 columns of one row.
+__device__ __forceinline__ void chunk_epilogue(const TcEpi& e, float (&v)[32], int nb, int64_t N, const float* bias_smem, uint32_t dw, uint32_t gw) {
+    if (e.bias) {
+        if (bias_smem || (aligned16_dev(e.bias) && nb + 31 < N)) {
+            const float4* b4 = reinterpret_cast<const float4*>((bias_smem ? bias_smem : e.bias) + nb);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const float4 b = bias_smem ? b4[q] : __ldg(b4 + q);
+                v[4 * q] += b.x; v[4 * q + 1] += b.y; v[4 * q + 2] += b.z; v[4 * q + 3] += b.w;
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < 32; ++q)
+                if (nb + q < N) v[q] += __ldg(e.bias + nb + q);
+        }
+    }
+    if (e.relu) {
+#pragma unroll
+        for (int q = 0; q < 32; ++q) v[q] = fmaxf(v[q], 0.0f);
+    }
+    if (e.drop) {
+#pragma unroll
+        for (int q = 0; q < 32; ++q) v[q] = (dw >> q) & 1u ? v[q] * e.keep_scale : 0.0f;
+    }
+    if (e.gate_bits || e.gate) {
+#pragma unroll
+        for (int q = 0; q < 32; ++q) v[q] = (gw >> q) & 1u ? v[q] * e.gate_scale : 0.0f;
+    }
+}
+
 // One output tile per CTA; MN_MAJOR = true is the split-K weight-gradient form (grid.z = split).
 // Warp roles: warps 0-3 epilogue (TMEM lane quarter = warp id), warp 4 TMA producer, warp 5 TMEM
 // allocation + MMA issue.
@@ -351,7 +483,7 @@ __global__ void __launch_bounds__(KK_THREADS, 1) gemm_tc_kk_kernel(const __grid_
     if (threadIdx.x == 0) {
         abort_flag = 0;
         for (int s = 0; s < p.stages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], LOSS ? KK_EPI_WARPS / 2 : KK_EPI_WARPS); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], (LOSS || p.bn <= 32) ? KK_EPI_WARPS / 2 : KK_EPI_WARPS); }
         mbar_init(&b_bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -519,81 +651,45 @@ __global__ void __launch_bounds__(KK_THREADS, 1) gemm_tc_kk_kernel(const __grid_
     } else {
         // ---------------- epilogue: warp w reads TMEM lanes 32*(w&3).., 32-column chunks (w>>2), (w>>2)+2, ... ----------------
         const int quarter = warp & 3, half = warp >> 2;
-        // The dropout mask and the gate are per-element tensors of C's shape.  With TMA stores they are
-        // applied on the staged box, where a row's 128 bytes belong to eight adjacent lanes (coalesced
-        // reads of the gate); otherwise element by element from the registers, like a bias wider than the
-        // shared-memory copy.
-        const bool has_gate = p.epi.gate != nullptr || p.epi.gate_bits != nullptr;
-        const bool post = (p.epi.drop != nullptr || has_gate) && tma_store;
-        const bool generic = !post && (p.epi.drop != nullptr || has_gate || (p.epi.bias != nullptr && !bias_in_smem));
-        const bool wide_bias = post && p.epi.bias != nullptr && !bias_in_smem;
-        const bool add_bias = p.epi.bias != nullptr && bias_in_smem, relu = p.epi.relu != 0;
-        const bool gate_vec = p.epi.gate != nullptr && aligned16_dev(p.epi.gate) && (p.epi.ld_gate & 3) == 0;
+        const bool masks = p.epi.drop != nullptr || p.epi.gate != nullptr || p.epi.gate_bits != nullptr;
         // one staging box per warp, or two (short K: the epilogue is the critical path, and the second box is
         // filled while the TMA store of the first is still reading it)
         const int nboxes = p.epi_boxes;
         uint8_t* const box_base = smem_out + (size_t)warp * nboxes * 4096;
         uint32_t box_turn = 0;
-        uint32_t j = 0;
+        // Tiles of one 32-column chunk: the two warps of a lane quarter take alternate tiles (one accumulator buffer each)
+        // instead of alternate chunks, of which there is none for the second.
+        const bool by_tile = p.bn <= 32;
+        const int c_first = by_tile ? 0 : half * 32;
+        const uint32_t tile_step = by_tile ? 2u : 1u;
+        uint32_t j = by_tile ? (uint32_t)half : 0u;
         bool ok = true;
-        for (int64_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++j) {
+        for (int64_t tile = blockIdx.x + (int64_t)j * gridDim.x; tile < tiles && ok; tile += (int64_t)tile_step * gridDim.x, j += tile_step) {
             const uint32_t buf = j & 1;
             const int64_t m0 = (tile / p.n_tiles) * TC_BM;
             const int n0 = (int)((tile % p.n_tiles) * p.bn);
+            // the tile's mask words, while its accumulator is still being made
+            uint32_t dw[4], gw[4];
+            if (masks) mask_words(p.epi, m0 + quarter * 32, p.M, p.N, n0 + c_first, 64, n0 + p.bn, lane, dw, gw);
             if (lane == 0) ok = mbar_wait(&acc_full[buf], (j >> 1) & 1, &abort_flag, p.wait_limit);
             ok = __shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0) != 0;
             if (!ok) { if (lane == 0) { abort_flag = 1; atomicMax(p.status, DEV_WAIT_EXPIRED); } break; }
             tc_fence_after();
             const int64_t m = m0 + quarter * 32 + lane;
             const bool row_ok = m < p.M;
-            for (int c0 = half * 32; c0 < p.bn; c0 += 64) {
+            for (int c0 = c_first, ci = 0; c0 < p.bn; c0 += 64, ++ci) {
                 const int nb = n0 + c0;
-                // the gate's 32 x 32 block in the staged-box orientation (lane = row it * 4 + lane / 8,
-                // 16-byte chunk lane % 8), requested before the accumulator is read so that the loads overlap it
-                float4 g4[8];
-                if (post && p.epi.gate_bits) {
-                    // bit-packed gate: this lane's row, the chunk's word (kept in the first slot of the fp32 gate's registers:
-                    // the two forms exclude each other)
-                    g4[0].x = __uint_as_float(row_ok ? __ldg(p.epi.gate_bits + (p.epi.row0 + m) * p.epi.ld_gate_bits + (nb >> 5)) : 0u);
-                } else if (post && gate_vec) {
-#pragma unroll
-                    for (int it = 0; it < 8; ++it) {
-                        const int64_t mr = m0 + quarter * 32 + it * 4 + (lane >> 3);
-                        const int nc = nb + (lane & 7) * 4;
-                        g4[it] = (mr < p.M && nc < p.N) ? __ldg(reinterpret_cast<const float4*>(p.epi.gate + (p.epi.row0 + mr) * p.epi.ld_gate + nc))
-                                                         : make_float4(0.f, 0.f, 0.f, 0.f);
-                    }
-                }
                 uint32_t r[32];
                 tc_ld32(tmem_base + buf * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c0, r);
                 tc_wait_ld();
                 float v[32];
 #pragma unroll
                 for (int q = 0; q < 32; ++q) v[q] = __uint_as_float(r[q]);
-                if (!generic) {
-                    if (add_bias) {
-                        const float4* sb4 = reinterpret_cast<const float4*>(s_bias + nb);
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) {
-                            const float4 b4 = sb4[q];
-                            v[4 * q] += b4.x; v[4 * q + 1] += b4.y; v[4 * q + 2] += b4.z; v[4 * q + 3] += b4.w;
-                        }
-                    } else if (wide_bias) {
-#pragma unroll
-                        for (int q = 0; q < 32; ++q)
-                            if (nb + q < p.N) v[q] += p.epi.bias[nb + q];
-                    }
-                    if (relu) {
-#pragma unroll
-                        for (int q = 0; q < 32; ++q) v[q] = fmaxf(v[q], 0.0f);
-                    }
-                } else if (row_ok) {
-#pragma unroll
-                    for (int q = 0; q < 32; ++q)
-                        if (nb + q < p.N) v[q] = tc_apply_epi(p.epi, v[q], m, nb + q, p.N);
-                }
-                if (p.epi.sign_bits && row_ok && !post) p.epi.sign_bits[(p.epi.row0 + m) * p.epi.ld_sign_bits + (nb >> 5)] = sign_word(v, nb, p.N);
-                if (p.C_lp && row_ok && !post) {
+                const uint32_t dwc = ci == 0 ? dw[0] : ci == 1 ? dw[1] : ci == 2 ? dw[2] : dw[3];
+                const uint32_t gwc = ci == 0 ? gw[0] : ci == 1 ? gw[1] : ci == 2 ? gw[2] : gw[3];
+                chunk_epilogue(p.epi, v, nb, p.N, bias_in_smem ? s_bias : nullptr, dwc, gwc);
+                if (p.epi.sign_bits && row_ok && nb < p.N) p.epi.sign_bits[(p.epi.row0 + m) * p.epi.ld_sign_bits + (nb >> 5)] = sign_word(v, nb, p.N);
+                if (p.C_lp && row_ok) {
                     const int64_t left = p.N - nb, here = p.bn - c0;
                     const int valid = (int)(left < here ? left : here);
                     store_lp_row(p.C_lp + m * p.ldc_lp + nb, v, valid);
@@ -611,51 +707,6 @@ __global__ void __launch_bounds__(KK_THREADS, 1) gemm_tc_kk_kernel(const __grid_
                     for (int q = 0; q < 8; ++q)
                         *reinterpret_cast<float4*>(box + lane * 128 + ((q ^ (lane & 7)) << 4)) =
                             make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-                    if (post) {
-                        __syncwarp();
-#pragma unroll
-                        for (int it = 0; it < 8; ++it) {
-                            const int rr = it * 4 + (lane >> 3), ch = lane & 7;
-                            const uint32_t gw_rr = __shfl_sync(0xFFFFFFFFu, __float_as_uint(g4[0].x), rr);   // every lane takes part (before any lane skips)
-                            const int64_t mr = m0 + quarter * 32 + rr;
-                            const int nc = nb + ch * 4;
-                            if (mr >= p.M || nc >= p.N || c0 + ch * 4 >= p.bn) continue;
-                            float4* cell = reinterpret_cast<float4*>(box + rr * 128 + ((ch ^ (rr & 7)) << 4));
-                            const float4 y4 = *cell;
-                            float y[4] = {y4.x, y4.y, y4.z, y4.w};
-                            const int nv = p.N - nc < 4 ? (int)(p.N - nc) : 4;
-                            if (p.epi.drop) {
-                                const uint8_t* dm = p.epi.drop + (p.epi.row0 + mr) * p.N + nc;
-#pragma unroll
-                                for (int t = 0; t < 4; ++t) if (t < nv) y[t] = dm[t] ? y[t] * p.epi.keep_scale : 0.0f;
-                            }
-                            if (p.epi.gate_bits) {
-                                const uint32_t nib = (gw_rr >> (ch * 4)) & 0xFu;
-#pragma unroll
-                                for (int t = 0; t < 4; ++t) y[t] = ((nib >> t) & 1u) ? y[t] * p.epi.gate_scale : 0.0f;
-                            } else if (p.epi.gate) {
-                                const float* gp = p.epi.gate + (p.epi.row0 + mr) * p.epi.ld_gate + nc;
-                                float gq[4] = {0.f, 0.f, 0.f, 0.f};
-                                if (gate_vec) {       // the whole group lies inside the row's allocation (ld_gate % 4 == 0)
-                                    gq[0] = g4[it].x; gq[1] = g4[it].y; gq[2] = g4[it].z; gq[3] = g4[it].w;
-                                } else {
-#pragma unroll
-                                    for (int t = 0; t < 4; ++t) if (t < nv) gq[t] = __ldg(gp + t);
-                                }
-#pragma unroll
-                                for (int t = 0; t < 4; ++t) y[t] = gq[t] > 0.0f ? y[t] * p.epi.gate_scale : 0.0f;
-                            }
-                            *cell = make_float4(y[0], y[1], y[2], y[3]);
-                            if (p.C_lp) {
-                                uint16_t* dl = p.C_lp + mr * p.ldc_lp + nc;
-                                if (nv == 4) *reinterpret_cast<uint2*>(dl) = make_uint2(pack_bf16(y[0], y[1]), pack_bf16(y[2], y[3]));
-                                else {
-#pragma unroll
-                                    for (int t = 0; t < 4; ++t) if (t < nv) dl[t] = (uint16_t)(pack_bf16(y[t], 0.0f) & 0xFFFFu);
-                                }
-                            }
-                        }
-                    }
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();
                     if (lane == 0) {
@@ -735,7 +786,6 @@ __global__ void __launch_bounds__(KK_THREADS, 1) gemm_tc_pair_kernel(const __gri
     constexpr uint32_t acc_stride = PAIR_BN, tmem_cols = 2 * PAIR_BN;
     // the bias is read from global memory (every lane the same 128 bytes: a broadcast the L1 serves), which
     // leaves the shared memory a copy of it would take to a sixth stage of the ring
-    const bool bias_vec = p.epi.bias != nullptr && aligned16_dev(p.epi.bias);
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
@@ -805,11 +855,7 @@ __global__ void __launch_bounds__(KK_THREADS, 1) gemm_tc_pair_kernel(const __gri
     } else {
         // ---------------- epilogue (both CTAs): this CTA's 128 rows of the tile ----------------
         const int quarter = warp & 3, half = warp >> 2;
-        const bool has_gate = p.epi.gate != nullptr || p.epi.gate_bits != nullptr;
-        const bool post = (p.epi.drop != nullptr || has_gate) && tma_store;
-        const bool generic = !post && (p.epi.drop != nullptr || has_gate);
-        const bool add_bias = p.epi.bias != nullptr, relu = p.epi.relu != 0;
-        const bool gate_vec = p.epi.gate != nullptr && aligned16_dev(p.epi.gate) && (p.epi.ld_gate & 3) == 0;
+        const bool masks = p.epi.drop != nullptr || p.epi.gate != nullptr || p.epi.gate_bits != nullptr;
         uint8_t* box = smem_out + (size_t)warp * 4096;
         uint32_t j = 0;
         bool ok = true;
@@ -817,61 +863,28 @@ __global__ void __launch_bounds__(KK_THREADS, 1) gemm_tc_pair_kernel(const __gri
             const uint32_t buf = j & 1;
             const int64_t m0 = (tile / p.n_tiles) * PAIR_BM + rank * TC_BM;
             const int n0 = (int)((tile % p.n_tiles) * PAIR_BN);
+            uint32_t dw[4], gw[4];                        // mask words, as in gemm_tc_kk_kernel
+            if (masks) mask_words(p.epi, m0 + quarter * 32, p.M, p.N, n0 + half * 32, 64, n0 + PAIR_BN, lane, dw, gw);
             if (lane == 0) ok = mbar_wait(&acc_full[buf], (j >> 1) & 1, &abort_flag, p.wait_limit);
             ok = __shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0) != 0;
             if (!ok) { if (lane == 0) { abort_flag = 1; atomicMax(p.status, DEV_WAIT_EXPIRED); } break; }
             tc_fence_after();
             const int64_t m = m0 + quarter * 32 + lane;
             const bool row_ok = m < p.M;
-            for (int c0 = half * 32; c0 < PAIR_BN; c0 += 64) {
+            for (int c0 = half * 32, ci = 0; c0 < PAIR_BN; c0 += 64, ++ci) {
                 const int nb = n0 + c0;
                 if (nb >= p.N) break;                     // columns beyond N: nothing to store (warp-uniform)
-                float4 g4[8];
-                if (post && p.epi.gate_bits) {
-                    // bit-packed gate: this lane's row, the chunk's word (kept in the first slot of the fp32 gate's registers:
-                    // the two forms exclude each other)
-                    g4[0].x = __uint_as_float(row_ok ? __ldg(p.epi.gate_bits + (p.epi.row0 + m) * p.epi.ld_gate_bits + (nb >> 5)) : 0u);
-                } else if (post && gate_vec) {
-#pragma unroll
-                    for (int it = 0; it < 8; ++it) {
-                        const int64_t mr = m0 + quarter * 32 + it * 4 + (lane >> 3);
-                        const int nc = nb + (lane & 7) * 4;
-                        g4[it] = (mr < p.M && nc < p.N) ? __ldg(reinterpret_cast<const float4*>(p.epi.gate + (p.epi.row0 + mr) * p.epi.ld_gate + nc))
-                                                         : make_float4(0.f, 0.f, 0.f, 0.f);
-                    }
-                }
                 uint32_t r[32];
                 tc_ld32(tmem_base + buf * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c0, r);
                 tc_wait_ld();
                 float v[32];
 #pragma unroll
                 for (int q = 0; q < 32; ++q) v[q] = __uint_as_float(r[q]);
-                if (!generic) {
-                    if (add_bias) {
-                        if (bias_vec && nb + 31 < p.N) {
-                            const float4* gb4 = reinterpret_cast<const float4*>(p.epi.bias + nb);
-#pragma unroll
-                            for (int q = 0; q < 8; ++q) {
-                                const float4 b4 = __ldg(gb4 + q);
-                                v[4 * q] += b4.x; v[4 * q + 1] += b4.y; v[4 * q + 2] += b4.z; v[4 * q + 3] += b4.w;
-                            }
-                        } else {
-#pragma unroll
-                            for (int q = 0; q < 32; ++q)
-                                if (nb + q < p.N) v[q] += __ldg(p.epi.bias + nb + q);
-                        }
-                    }
-                    if (relu) {
-#pragma unroll
-                        for (int q = 0; q < 32; ++q) v[q] = fmaxf(v[q], 0.0f);
-                    }
-                } else if (row_ok) {
-#pragma unroll
-                    for (int q = 0; q < 32; ++q)
-                        if (nb + q < p.N) v[q] = tc_apply_epi(p.epi, v[q], m, nb + q, p.N);
-                }
-                if (p.epi.sign_bits && row_ok && !post) p.epi.sign_bits[(p.epi.row0 + m) * p.epi.ld_sign_bits + (nb >> 5)] = sign_word(v, nb, p.N);
-                if (p.C_lp && row_ok && !post) {
+                const uint32_t dwc = ci == 0 ? dw[0] : ci == 1 ? dw[1] : ci == 2 ? dw[2] : dw[3];
+                const uint32_t gwc = ci == 0 ? gw[0] : ci == 1 ? gw[1] : ci == 2 ? gw[2] : gw[3];
+                chunk_epilogue(p.epi, v, nb, p.N, nullptr, dwc, gwc);       // (bias: a broadcast the L1 serves)
+                if (p.epi.sign_bits && row_ok) p.epi.sign_bits[(p.epi.row0 + m) * p.epi.ld_sign_bits + (nb >> 5)] = sign_word(v, nb, p.N);
+                if (p.C_lp && row_ok) {
                     const int64_t left = p.N - nb;
                     store_lp_row(p.C_lp + m * p.ldc_lp + nb, v, (int)(left < 32 ? left : 32));
                 }
@@ -882,51 +895,6 @@ __global__ void __launch_bounds__(KK_THREADS, 1) gemm_tc_pair_kernel(const __gri
                     for (int q = 0; q < 8; ++q)
                         *reinterpret_cast<float4*>(box + lane * 128 + ((q ^ (lane & 7)) << 4)) =
                             make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-                    if (post) {
-                        __syncwarp();
-#pragma unroll
-                        for (int it = 0; it < 8; ++it) {
-                            const int rr = it * 4 + (lane >> 3), ch = lane & 7;
-                            const uint32_t gw_rr = __shfl_sync(0xFFFFFFFFu, __float_as_uint(g4[0].x), rr);   // every lane takes part (before any lane skips)
-                            const int64_t mr = m0 + quarter * 32 + rr;
-                            const int nc = nb + ch * 4;
-                            if (mr >= p.M || nc >= p.N) continue;
-                            float4* cell = reinterpret_cast<float4*>(box + rr * 128 + ((ch ^ (rr & 7)) << 4));
-                            const float4 y4 = *cell;
-                            float y[4] = {y4.x, y4.y, y4.z, y4.w};
-                            const int nv = p.N - nc < 4 ? (int)(p.N - nc) : 4;
-                            if (p.epi.drop) {
-                                const uint8_t* dm = p.epi.drop + (p.epi.row0 + mr) * p.N + nc;
-#pragma unroll
-                                for (int t = 0; t < 4; ++t) if (t < nv) y[t] = dm[t] ? y[t] * p.epi.keep_scale : 0.0f;
-                            }
-                            if (p.epi.gate_bits) {
-                                const uint32_t nib = (gw_rr >> (ch * 4)) & 0xFu;
-#pragma unroll
-                                for (int t = 0; t < 4; ++t) y[t] = ((nib >> t) & 1u) ? y[t] * p.epi.gate_scale : 0.0f;
-                            } else if (p.epi.gate) {
-                                const float* gp = p.epi.gate + (p.epi.row0 + mr) * p.epi.ld_gate + nc;
-                                float gq[4] = {0.f, 0.f, 0.f, 0.f};
-                                if (gate_vec) {
-                                    gq[0] = g4[it].x; gq[1] = g4[it].y; gq[2] = g4[it].z; gq[3] = g4[it].w;
-                                } else {
-#pragma unroll
-                                    for (int t = 0; t < 4; ++t) if (t < nv) gq[t] = __ldg(gp + t);
-                                }
-#pragma unroll
-                                for (int t = 0; t < 4; ++t) y[t] = gq[t] > 0.0f ? y[t] * p.epi.gate_scale : 0.0f;
-                            }
-                            *cell = make_float4(y[0], y[1], y[2], y[3]);
-                            if (p.C_lp) {
-                                uint16_t* dl = p.C_lp + mr * p.ldc_lp + nc;
-                                if (nv == 4) *reinterpret_cast<uint2*>(dl) = make_uint2(pack_bf16(y[0], y[1]), pack_bf16(y[2], y[3]));
-                                else {
-#pragma unroll
-                                    for (int t = 0; t < 4; ++t) if (t < nv) dl[t] = (uint16_t)(pack_bf16(y[t], 0.0f) & 0xFFFFu);
-                                }
-                            }
-                        }
-                    }
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();
                     if (lane == 0) {
@@ -1304,8 +1272,7 @@ mixgcn_status launch_kind(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64_t N,
                     LaunchScope scope(ctx, PH_GEMM, s);
                     MIXGCN_CUDA(cudaLaunchKernelEx(&cfg, gemm_tc_pair_kernel<KIND>, map_a, map_b2, map_c2, q, tma_store2));
                     ctx->gemm_pair_launches++;
-                    // the epilogue wrote the sign bitmap unless the per-element terms ran on the staged boxes
-                    if (bits_done) *bits_done = q.epi.sign_bits && !(tma_store2 && (q.epi.drop || q.epi.gate || q.epi.gate_bits));
+                    if (bits_done) *bits_done = q.epi.sign_bits != nullptr;
                     return MIXGCN_OK;
                 }
             }
@@ -1342,7 +1309,7 @@ mixgcn_status launch_kind(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64_t N,
         LaunchScope scope(ctx, PH_GEMM, s);
         gemm_tc_kk_kernel<KIND><<<dim3((unsigned)grid, 1, 1), KK_THREADS, smem_kk, s>>>(map_a, map_b, map_c, p, b_resident, tma_store);
         MIXGCN_CUDA(cudaGetLastError());
-        if (bits_done) *bits_done = p.epi.sign_bits && !(tma_store && (p.epi.drop || p.epi.gate || p.epi.gate_bits));
+        if (bits_done) *bits_done = p.epi.sign_bits != nullptr;
         return MIXGCN_OK;
     }
 
@@ -1391,7 +1358,9 @@ mixgcn_status launch_kind(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64_t N,
         }
     }
     // split K over CTAs
-    int splits = pick_splits(tiles, 2 * (int64_t)ctx->sm_count, (K + 2047) / 2048);      // two CTAs per SM
+    // (two CTAs per SM; no fewer than eight k-steps each: a CTA that walks 2,048 rows alone takes 90 us, whatever the
+    // rest of the machine does)
+    int splits = pick_splits(tiles, 2 * (int64_t)ctx->sm_count, (K + 8 * BK - 1) / (8 * BK));
     if (splits > 2048) splits = 2048;
     int64_t kps = (K + splits - 1) / splits;
     kps = (kps + BK - 1) / BK * BK;

@@ -50,11 +50,10 @@ LaunchScope::~LaunchScope() {
 
 // One memory pool per device for everything the library allocates.  Building a graph takes some thirty temporary blocks
 // and its arrays; cudaMalloc and cudaFree of each cost 0.1 ms and more (7 of the 9 ms of a graph with 4 M entries, and
-// many times that when they had to map fresh memory), and each synchronises the device.  The pool keeps at most
-// POOL_KEEP bytes of freed memory for reuse; what is above goes back to the driver at the next synchronisation, and all
-// of it when the last context on the device is destroyed.  The driver's pools are safe with several threads and streams.
+// many times that when they had to map fresh memory), and each synchronises the device.  The pool keeps at most a
+// 32nd of the device's memory in freed blocks for reuse; what is above goes back to the driver at the next
+// synchronisation, and all of it when the last context on the device is destroyed.  The driver's pools are safe with several threads and streams.
 namespace {
-constexpr uint64_t POOL_KEEP = 2ull << 30;
 constexpr int MAX_DEVICES = 64;
 struct DevicePool { cudaMemPool_t pool = nullptr; int contexts = 0; };
 std::mutex g_pool_mutex;
@@ -82,7 +81,12 @@ mixgcn_status pool_contexts(int device, int change) {
     const int before = d.contexts;
     d.contexts += change;
     if ((before == 0) != (d.contexts == 0)) {
-        uint64_t keep = d.contexts ? POOL_KEEP : 0;
+        uint64_t keep = 0;
+        if (d.contexts) {
+            size_t free_bytes = 0, total_bytes = 0;
+            MIXGCN_CUDA(cudaMemGetInfo(&free_bytes, &total_bytes));
+            keep = total_bytes / 32;
+        }
         MIXGCN_CUDA(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
         if (!d.contexts) MIXGCN_CUDA(cudaMemPoolTrimTo(pool, 0));
     }

@@ -298,6 +298,12 @@ mixgcn_status mixgcn_gemm(mixgcn_ctx* ctx, int32_t precision, int32_t trans_a, i
                           const float* B, int64_t ldb, float* C, int64_t ldc,
                           const mixgcn_epilogue* epi, void* stream);
 
+/* The weight gradient of an update and, on request, its bias gradient in one call: C = A^T B (mixgcn_gemm with trans_a = 1,
+ * trans_b = 0) for A K x M and B K x N, and colsum_b[n] = sum_k B[k][n] (device, N floats, nullable; needs B 16-byte aligned
+ * with ldb a multiple of 4) -- from the same pass over B where the product's kernel can. */
+mixgcn_status mixgcn_weight_grad(mixgcn_ctx* ctx, int32_t precision, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda,
+                                 const float* B, int64_t ldb, float* C, int64_t ldc, float* colsum_b, void* stream);
+
 /* ------------------------------------------------------------------------------------------
  * One GCN layer, X_out = drop * keep_scale * ReLU(A_hat X_in W + 1 b^T)   (Eq. 3)
  * ------------------------------------------------------------------------------------------ */

@@ -10,7 +10,6 @@ from __future__ import annotations
 import ctypes as C
 import gc
 import os
-import threading
 
 import torch
 
@@ -53,7 +52,7 @@ SYMBOLS = (
     "mixgcn_rowplan_export", "mixgcn_spmm_rowplan", "mixgcn_colsum", "mixgcn_ctx_gemm_paths",
     "mixgcn_train_step_host_prefetch", "mixgcn_probe_gather", "mixgcn_spmm_sampled", "mixgcn_mask_pack",
     "mixgcn_build_info", "mixgcn_debug_poke_col", "mixgcn_layer_fwd_loss",
-    "mixgcn_record_begin", "mixgcn_record_end", "mixgcn_replay", "mixgcn_recording_destroy",
+    "mixgcn_record_begin", "mixgcn_record_end", "mixgcn_replay", "mixgcn_recording_destroy", "mixgcn_weight_grad",
 )
 
 
@@ -99,12 +98,8 @@ def _ptr(t):
     return None if t is None else C.c_void_p(t.data_ptr())
 
 
-_recording = threading.local()       # .stream: where this thread's calls go while a sequence is being recorded
-
-
 def _stream():
-    s = getattr(_recording, "stream", None)
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream) if s is None else s
+    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
 
 
 def _dev(t, dtype, name):
@@ -221,20 +216,19 @@ class Recording:
 
 
 def record(ctx: Ctx, calls):
-    """Run `calls()` with every compute call of `ctx` recorded instead of executed -> Recording, or None if the sequence
-    cannot be recorded."""
+    """Run `calls()` with every compute call of `ctx` (and every torch operation that neither allocates nor synchronises)
+    recorded instead of executed -> Recording, or None if the sequence cannot be recorded."""
     stream, h = C.c_void_p(), C.c_void_p()
     if lib.mixgcn_record_begin(ctx.h, C.byref(stream)) != OK:
         return None
-    _recording.stream = stream
     collect = gc.isenabled()
     gc.disable()                     # a collected graph or context would synchronise, which ends a recording
     try:
-        calls()
+        with torch.cuda.stream(torch.cuda.ExternalStream(stream.value, device=torch.device("cuda", ctx.device))):
+            calls()
     except MixgcnError:
         pass                         # the recording is void; record_end says so
     finally:
-        _recording.stream = None
         st = lib.mixgcn_record_end(ctx.h, C.byref(h))
         if collect:
             gc.enable()
@@ -251,7 +245,7 @@ class Replayer:
 
     def run(self, key, calls):
         """key(): the current key; calls(): issues the calls."""
-        if self.ctx.profiling or getattr(_recording, "stream", None) is not None or torch.cuda.is_current_stream_capturing():
+        if self.ctx.profiling or torch.cuda.is_current_stream_capturing():
             calls()
             return
         k = key()
@@ -431,6 +425,15 @@ def gemm(ctx: Ctx, precision: int, trans_a: bool, trans_b: bool, M: int, N: int,
     _check(lib.mixgcn_gemm(ctx.h, C.c_int32(precision), C.c_int32(int(trans_a)), C.c_int32(int(trans_b)),
                            C.c_int64(M), C.c_int64(N), C.c_int64(K), _ptr(A), C.c_int64(lda), _ptr(B),
                            C.c_int64(ldb), _ptr(Cm), C.c_int64(ldc), None if epi is None else C.byref(epi), _stream()))
+
+
+def weight_grad(ctx: Ctx, precision: int, M: int, N: int, K: int, A: torch.Tensor, B: torch.Tensor, Cm: torch.Tensor, colsum=None):
+    """Cm = A^T B (A is K x M, B is K x N) and, if given, colsum = column sums of B."""
+    A, lda = _mat(A, "A")
+    B, ldb = _mat(B, "B")
+    Cm, ldc = _mat(Cm, "C")
+    _check(lib.mixgcn_weight_grad(ctx.h, C.c_int32(precision), C.c_int64(M), C.c_int64(N), C.c_int64(K), _ptr(A), C.c_int64(lda), _ptr(B),
+                                  C.c_int64(ldb), _ptr(Cm), C.c_int64(ldc), _ptr(colsum), _stream()))
 
 
 # ------------------------------------------------------------------------------ layers

@@ -487,6 +487,18 @@ extern "C" mixgcn_status mixgcn_gemm(mixgcn_ctx* ctx, int32_t precision, int32_t
     return launch_gemm(ctx, precision, trans_a, trans_b, M, N, K, A, lda, B, ldb, C, ldc, epi, 0, (cudaStream_t)stream);
 }
 
+extern "C" mixgcn_status mixgcn_weight_grad(mixgcn_ctx* ctx, int32_t precision, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda,
+                                            const float* B, int64_t ldb, float* C, int64_t ldc, float* colsum_b, void* stream) {
+    if (!ctx || !A || !B || !C) MIXGCN_FAIL(MIXGCN_EINVAL, "weight_grad: null argument");
+    if (M <= 0 || N <= 0 || K <= 0) MIXGCN_FAIL(MIXGCN_EINVAL, "weight_grad: M, N, K must be positive");
+    if (precision < MIXGCN_PREC_FP32 || precision > MIXGCN_PREC_BF16) MIXGCN_FAIL(MIXGCN_EINVAL, "weight_grad: unknown precision %d", precision);
+    if (lda < M || ldb < N || ldc < N) MIXGCN_FAIL(MIXGCN_EINVAL, "weight_grad: leading dimensions must cover the matrix (lda=%lld ldb=%lld ldc=%lld)", (long long)lda, (long long)ldb, (long long)ldc);
+    if (C == A || C == B) MIXGCN_FAIL(MIXGCN_EINVAL, "weight_grad: C must not overlap A or B");
+    if (colsum_b && (!aligned16(B) || (ldb & 3))) MIXGCN_FAIL(MIXGCN_EINVAL, "weight_grad: column sums need B 16-byte aligned with ldb a multiple of 4 (ldb=%lld)", (long long)ldb);
+    MIXGCN_CUDA(cudaSetDevice(ctx->device));
+    return launch_gemm(ctx, precision, 1, 0, M, N, K, A, lda, B, ldb, C, ldc, nullptr, 0, (cudaStream_t)stream, nullptr, colsum_b);
+}
+
 // ------------------------------------------------------------------------------------------------
 // Layer composition
 // ------------------------------------------------------------------------------------------------

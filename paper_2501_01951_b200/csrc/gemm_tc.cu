@@ -65,7 +65,7 @@ struct TcParams {
     float* C; int64_t ldc; int vec_c;
     uint16_t* C_lp; int64_t ldc_lp;   // nullable: bf16 copy of C (after the epilogue); ldc_lp a multiple of 8
     int raw;                // 1: store the accumulator unchanged (split-K partial)
-    double* colsum_part;    // weight-gradient form, TF32: nullable [splits][N] column sums of B over this split's k-rows
+    double* colsum_part;    // weight-gradient form, TF32: nullable [splits][m_tiles][N] column sums of B over the k-rows a CTA took
     TcEpi epi;
     int32_t* status;
     uint32_t wait_limit;    // polls after which a wait gives up
@@ -273,9 +273,12 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
     while ((int)tmem_cols < p.bn) tmem_cols <<= 1;
 
     // Column sums of B (the bias gradient 1^T dP when B = dP) as a by-product: the four epilogue warps are
-    // idle while the tiles stream through shared memory, so in the CTAs of the first row of tiles they add up
-    // each stage's B tile (fp32 words, TF32 kind only) before the stage is released.
-    const bool do_colsum = MN_MAJOR && KIND == KIND_TF32 && p.colsum_part != nullptr && tile / p.n_tiles == 0;
+    // idle while the tiles stream through shared memory, so they add up the stages' B tiles (fp32 words, TF32 kind
+    // only) before a stage is released.  The CTAs of a column of tiles see the same B and take turns, stage by stage:
+    // with the first row of tiles doing it all, a product with two rows took almost twice as long (2.4 M x 256 x 256:
+    // 743 us without the sums, 1401 us with them).
+    const bool do_colsum = MN_MAJOR && KIND == KIND_TF32 && p.colsum_part != nullptr;
+    const int turn = (int)(tile / p.n_tiles), turns = (int)p.m_tiles;
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
@@ -346,29 +349,37 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
         // ---------------- epilogue: warps 0..3 own TMEM lanes 32*warp .. 32*warp+31 ----------------
         bool ok = true;
         if (do_colsum) {
-            // warp w takes the 32-column chunks w and w + 4 of the B tile, lane l their column l.  A chunk is BK
-            // k-rows of 128 bytes in the 128-byte swizzle with 32-byte atoms: the 32-byte group g of k-row r sits
-            // at group position g ^ (r & 3).
-            double sum[2] = {0.0, 0.0};
-            const int chunks = bn_pad / Cfg::CHUNK;
+            // warp w takes the 32-column chunks w and w + 4 of the B tile: lane (g, c) = (lane / 8, lane % 8) the columns
+            // 4 c .. 4 c + 3 of the k-rows 4 i + g, 16 bytes at a time.  A chunk is BK k-rows of 128 bytes in the 128-byte
+            // swizzle with 32-byte atoms: the 32-byte group q of k-row r sits at group position q ^ (r & 3).
+            double sum[2][4] = {{0.0, 0.0, 0.0, 0.0}, {0.0, 0.0, 0.0, 0.0}};
+            const int chunks = bn_pad / Cfg::CHUNK, g = lane >> 3, c = lane & 7;
+            const int at = g * 128 + ((((c >> 1) ^ g) << 1) | (c & 1)) * 16;
+            int whose = 0;                                   // whose turn this stage is
             for (int ks = 0; ks < nk && ok; ++ks) {
                 const int s = ks % p.stages;
                 const uint32_t ph = (ks / p.stages) & 1;
                 if (lane == 0) ok = mbar_wait(&full_bar[s], ph, &abort_flag, p.wait_limit);
                 ok = __shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0) != 0;
                 if (!ok) { if (lane == 0) { abort_flag = 1; atomicMax(p.status, DEV_WAIT_EXPIRED); } break; }
-                const uint8_t* sb = smem + (size_t)s * stage_bytes + a_bytes;
+                if (whose == turn) {
+                    const uint8_t* sb = smem + (size_t)s * stage_bytes + a_bytes;
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int cc = warp + 4 * h;
-                    if (cc < chunks) {
-                        const float* chunk = reinterpret_cast<const float*>(sb + (size_t)cc * Cfg::MN_CHUNK_BYTES);
-                        float part = 0.0f;
-#pragma unroll 8
-                        for (int r = 0; r < BK; ++r) part += chunk[r * 32 + (lane ^ ((r & 3) << 3))];
-                        sum[h] += (double)part;
+                    for (int h = 0; h < 2; ++h) {
+                        const int cc = warp + 4 * h;
+                        if (cc < chunks) {
+                            const uint8_t* chunk = sb + (size_t)cc * Cfg::MN_CHUNK_BYTES + at;
+                            float4 part = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                            for (int i = 0; i < BK / 4; ++i) {
+                                const float4 v = *reinterpret_cast<const float4*>(chunk + i * 512);
+                                part.x += v.x; part.y += v.y; part.z += v.z; part.w += v.w;
+                            }
+                            sum[h][0] += (double)part.x; sum[h][1] += (double)part.y; sum[h][2] += (double)part.z; sum[h][3] += (double)part.w;
+                        }
                     }
                 }
+                if (++whose == turns) whose = 0;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&empty_bar[s]);      // this warp has read the stage
             }
@@ -376,8 +387,15 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int cc = warp + 4 * h;
-                    const int64_t n = n0 + cc * 32 + lane;
-                    if (cc < chunks && cc * 32 + lane < p.bn && n < p.N) p.colsum_part[(int64_t)blockIdx.z * p.N + n] = sum[h];
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) {
+                        double v = sum[h][t];
+                        v += __shfl_xor_sync(0xFFFFFFFFu, v, 8);
+                        v += __shfl_xor_sync(0xFFFFFFFFu, v, 16);
+                        const int col = cc * 32 + c * 4 + t;
+                        const int64_t n = n0 + col;
+                        if (g == 0 && cc < chunks && col < p.bn && n < p.N) p.colsum_part[((int64_t)blockIdx.z * turns + turn) * p.N + n] = v;
+                    }
                 }
             }
         }
@@ -1089,13 +1107,24 @@ __global__ void pack_b_kernel(const float* __restrict__ src, int64_t ld, int tra
     else reinterpret_cast<uint16_t*>(dst)[i] = (uint16_t)(pack_bf16(v, 0.0f) & 0xFFFFu);
 }
 
-// out[n] = sum over splits (ascending) of part[z][n]
-__global__ void colsum_splits_kernel(int64_t N, int splits, const double* __restrict__ part, float* __restrict__ out) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    double sacc = 0.0;
-    for (int z = 0; z < splits; ++z) sacc += part[(int64_t)z * N + n];
-    out[n] = (float)sacc;
+// out[n] = sum over splits of part[z][n]: eight rows of threads add an eighth of the splits each, the eighths are added in
+// order (one thread's chain over 296 splits took 20 us).
+__global__ void __launch_bounds__(256) colsum_splits_kernel(int64_t N, int splits, const double* __restrict__ part, float* __restrict__ out) {
+    __shared__ double sm[8][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t n = (int64_t)blockIdx.x * 32 + lane;
+    const int per = (splits + 7) / 8, z0 = w * per, z1 = z0 + per < splits ? z0 + per : splits;
+    double s = 0.0;
+    if (n < N) {
+#pragma unroll 4
+        for (int z = z0; z < z1; ++z) s += part[(int64_t)z * N + n];
+    }
+    sm[w][lane] = s;
+    __syncthreads();
+    if (w != 0 || n >= N) return;
+#pragma unroll
+    for (int q = 1; q < 8; ++q) s += sm[q][lane];
+    out[n] = (float)s;
 }
 
 // dst[r][c] = bf16(src[r][c]) for c < d (round to nearest even); four columns per thread.
@@ -1379,7 +1408,7 @@ mixgcn_status launch_kind(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64_t N,
     // with fp32 words in shared memory (TF32 kind) the kernel also sums B's columns on request
     const bool fuse_colsum = KIND == KIND_TF32 && colsum_b != nullptr;
     const int64_t part_bytes = splits > 1 ? (((int64_t)splits * M * N * (int64_t)sizeof(float) + 255) & ~(int64_t)255) : 0;
-    const int64_t cs_bytes = fuse_colsum ? (int64_t)splits * N * (int64_t)sizeof(double) : 0;
+    const int64_t cs_bytes = fuse_colsum ? (int64_t)splits * p.m_tiles * N * (int64_t)sizeof(double) : 0;
     if (part_bytes + cs_bytes > 0) MIXGCN_TRY(ensure_workspace(ctx, part_bytes + cs_bytes));
     if (splits > 1) {
         p.C = reinterpret_cast<float*>(ctx->workspace); p.ldc = N; p.vec_c = (N & 3) == 0; p.raw = 1;
@@ -1396,7 +1425,7 @@ mixgcn_status launch_kind(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64_t N,
     if (splits > 1) MIXGCN_TRY(launch_splitk_reduce(ctx, M, N, splits, p.C, C, ldc, epi, s));
     if (fuse_colsum) {
         LaunchScope scope(ctx, PH_GEMM, s);
-        colsum_splits_kernel<<<(unsigned)((N + 127) / 128), 128, 0, s>>>(N, splits, p.colsum_part, colsum_b);
+        colsum_splits_kernel<<<(unsigned)((N + 31) / 32), 256, 0, s>>>(N, (int)(splits * p.m_tiles), p.colsum_part, colsum_b);
         MIXGCN_CUDA(cudaGetLastError());
         if (colsum_done) *colsum_done = true;
     }

@@ -9,7 +9,11 @@ them; the layers are their textbook forms, built from the same C-ABI steps as th
                      epilogue's residual.
 
 As in ``train.py`` nothing is computed here: every value comes out of a kernel of ``libmixgcn.so``
-(``spmm``, ``gemm``, ``colsum``, ``loss_softmax_xent``, ``adam_step``).
+(``spmm``, ``gemm``, ``weight_grad``, ``colsum``, ``loss_softmax_xent``, ``adam_step``).
+
+Both aggregations are linear and stand before a product, so each layer picks the side of the product it aggregates on, by
+the width it costs, as the GCN layers do: M H W_neigh = M (H W_neigh) and ((1 + eps) H + A H) W1 = (1 + eps) U + A U with
+U = H W1.  A layer from 256 to 47 columns then gathers 47 instead of 256 in both directions.
 """
 from __future__ import annotations
 
@@ -20,6 +24,12 @@ from . import binding as mg
 
 def round4(x: int) -> int:
     return (x + 3) // 4 * 4
+
+
+def update_first(d_in: int, d_out: int, first: bool) -> bool:
+    """Whether aggregating after the product (at width d_out, forward and backward) is cheaper than before it (at width
+    d_in, forward and -- unless the layer is the first -- backward); ties aggregate first."""
+    return 2 * d_out < (1 if first else 2) * d_in
 
 
 class _Base:
@@ -38,6 +48,9 @@ class _Base:
 
     def _z(self, r, c):
         return torch.zeros((r, c), dtype=torch.float32, device=self.device)
+
+    def _bits(self, d):
+        return torch.zeros((self.n, (d + 31) // 32), dtype=torch.int32, device=self.device)
 
     def _set_params(self, tensors):
         self.params = [t.to(self.device, torch.float32).contiguous().clone() for t in tensors]
@@ -72,18 +85,32 @@ class _Base:
 
 class SageTrainer(_Base):
     """Mean-aggregator GraphSAGE.  ``graph`` must carry row-mean values (GRAPH_NORM_ROW, no self loops).
-    Layer l keeps S_l = [H_l | M H_l] (n x 2 ld_l): the left half is written by the layer below (or is
-    the input), the right half by the aggregation, and one product with W_l = [W_self; W_neigh]
-    (2 d_l x d_{l+1}) does the update."""
+    A layer that aggregates first keeps S_l = [H_l | M H_l] (n x 2 ld_l): the left half is written by the layer below (or is
+    the input), the right half by the aggregation, and one product with W_l = [W_self; W_neigh] (2 d_l x d_{l+1}) does the
+    update.  A layer that updates first keeps S_l = H_l; one product with [W_self | W_neigh] gives both terms side by side,
+    and the aggregation of the second adds the first as its residual."""
 
     def __init__(self, ctx, graph, dims, precision=mg.PREC_FP32):
         super().__init__(ctx, graph, dims, precision)
         n, L, ld = self.n, self.L, self.ld
-        self.S = [self._z(n, 2 * ld[l]) for l in range(L)]
-        self.logits = self._z(n, ld[L])
-        wmax = max(ld[1:L]) if L >= 2 else 4
-        self.dS = self._z(n, 2 * wmax)                     # gradient w.r.t. [H_l | M H_l]
-        self.Ga, self.Gb = self._z(n, wmax), self._z(n, wmax)
+        self.upd = [update_first(self.dims[l], self.dims[l + 1], l == 0) for l in range(L)]
+        self.S = [self._z(n, ld[l] if self.upd[l] else 2 * ld[l]) for l in range(L)]
+        # gradients w.r.t. the layers' outputs: [G | M^T G] where the layer updates first, G otherwise; the hidden ones take
+        # turns in two buffers, which the forward pass uses for the update-first products
+        self.wide = [2 * ld[l + 1] if self.upd[l] else ld[l + 1] for l in range(L)]
+        pool_w = max([self.wide[l] for l in range(L) if l < L - 1 or self.upd[l]] + [4])
+        self.pool = [self._z(n, pool_w), self._z(n, pool_w if L >= 3 else 4)]
+        self.G = [self.pool[l % 2 if L >= 3 else 0].view(-1)[: n * self.wide[l]].view(n, self.wide[l]) for l in range(L - 1)]
+        self.G.append(self._z(n, self.wide[L - 1]))
+        self.logits = self.G[L - 1][:, : ld[L]]
+        agg_hidden = [2 * ld[l] for l in range(1, L) if not self.upd[l]]
+        self.dS = self._z(n, max(agg_hidden)) if agg_hidden else None        # gradient w.r.t. [H_l | M H_l]
+        # update-first layers: [W_self | W_neigh], its gradient and the column sums of [G | M^T G]
+        self.Wc = [self._z(self.dims[l], self.wide[l]) if self.upd[l] else None for l in range(L)]
+        self.dWc = [self._z(self.dims[l], self.wide[l]) if self.upd[l] else None for l in range(L)]
+        self.dbc = [torch.zeros(self.wide[l], dtype=torch.float32, device=self.device) if self.upd[l] else None for l in range(L)]
+        # signs of the hidden activations that a product writes (one bit per element), read by the backward gates
+        self.signs = [None] + [None if self.upd[l - 1] else self._bits(self.dims[l]) for l in range(1, L)]
 
     def set_params(self, Ws_self, Ws_neigh, bs):
         """Parameter order: W_cat[0..L) (rows [W_self; W_neigh]), b[0..L)."""
@@ -100,31 +127,54 @@ class SageTrainer(_Base):
         self.S[0][:, : self.ld[0]].copy_(X0)
         self.labels, self.train_mask = labels, train_mask
 
+    def _halves(self, l, stacked, beside):
+        """Pairs of the two d_l x d_{l+1} blocks in the stacked ([self; neigh]) and the side-by-side ([self | neigh]) layout."""
+        d, ld, dout, do4 = self.dims[l], self.ld[l], self.dims[l + 1], self.ld[l + 1]
+        return ((stacked[:d], beside[:, :dout]), (stacked[ld: ld + d], beside[:, do4: do4 + dout]))
+
     def forward(self):
         L, ld = self.L, self.ld
         for l in range(L):
-            S, d = self.S[l], ld[l]
-            mg.spmm(self.ctx, self.g, S[:, :d], S[:, d:], self.dims[l])
+            S, d, dout, do4 = self.S[l], ld[l], self.dims[l + 1], ld[l + 1]
             last = l == L - 1
-            out = self.logits if last else self.S[l + 1][:, : ld[l + 1]]
-            mg.gemm(self.ctx, self.precision, False, False, self.n, self.dims[l + 1], 2 * d, S, self.params[l], out,
-                    epi=mg.make_epilogue(bias=self.params[L + l], relu=not last))
+            out = self.logits if last else self.S[l + 1][:, : do4]
+            bias, relu = self.params[L + l], not last
+            if self.upd[l]:
+                for stacked, beside in self._halves(l, self.params[l], self.Wc[l]):
+                    beside.copy_(stacked)
+                P = self.pool[0].view(-1)[: self.n * self.wide[l]].view(self.n, self.wide[l])
+                mg.gemm(self.ctx, self.precision, False, False, self.n, self.wide[l], self.dims[l], S, self.Wc[l], P)
+                mg.spmm(self.ctx, self.g, P[:, do4:], out, dout, epi=mg.make_epilogue(residual=P[:, :do4], residual_scale=1.0, bias=bias, relu=relu))
+            else:
+                mg.spmm(self.ctx, self.g, S[:, :d], S[:, d:], self.dims[l])
+                mg.gemm(self.ctx, self.precision, False, False, self.n, dout, 2 * d, S, self.params[l], out,
+                        epi=mg.make_epilogue(bias=bias, relu=relu, sign_bits=None if last else self.signs[l + 1]))
 
     def backward(self):
         L, ld = self.L, self.ld
-        G = self.logits                                     # gradient w.r.t. the layer's pre-activation
         for l in range(L - 1, -1, -1):
-            d, dout = ld[l], self.dims[l + 1]
-            mg.colsum(self.ctx, G, self.grads[L + l], dout)
-            mg.gemm(self.ctx, self.precision, True, False, 2 * d, dout, self.n, self.S[l], G, self.grads[l])
+            d, dout, do4 = ld[l], self.dims[l + 1], ld[l + 1]
+            Gc = self.G[l]                                      # gradient w.r.t. the layer's pre-activation, left half
+            G = Gc[:, :do4]
             if l > 0:
-                dS = self.dS[:, : 2 * d]
+                Gn = self.G[l - 1][:, :d]
+                gate = dict(gate_bits=self.signs[l]) if self.signs[l] is not None else dict(gate=self.S[l][:, :d])
+            if self.upd[l]:
+                mg.spmm(self.ctx, self.g, G, Gc[:, do4:], dout, transposed=True)
+                mg.weight_grad(self.ctx, self.precision, self.dims[l], self.wide[l], self.n, self.S[l], Gc, self.dWc[l], self.dbc[l])
+                for stacked, beside in self._halves(l, self.grads[l], self.dWc[l]):
+                    stacked.copy_(beside)
+                self.grads[L + l].copy_(self.dbc[l][:dout])
+                if l > 0:
+                    mg.gemm(self.ctx, self.precision, False, True, self.n, self.dims[l], self.wide[l], Gc, self.Wc[l], Gn, epi=mg.make_epilogue(gate_scale=1.0, **gate))
+                continue
+            mg.weight_grad(self.ctx, self.precision, 2 * d, dout, self.n, self.S[l], G, self.grads[l], self.grads[L + l])
+            if l > 0:
+                dS = self.dS.view(-1)[: self.n * 2 * d].view(self.n, 2 * d)
                 mg.gemm(self.ctx, self.precision, False, True, self.n, 2 * d, dout, G, self.params[l], dS)
-                Gn = (self.Ga if (L - 1 - l) % 2 == 0 else self.Gb)[:, :d]   # the two buffers alternate
                 # G_in = relu'(H_l) * (dS_left + M^T dS_right): residual and gate in the aggregation's epilogue
                 mg.spmm(self.ctx, self.g, dS[:, d:], Gn, self.dims[l], transposed=True,
-                        epi=mg.make_epilogue(residual=dS[:, :d], residual_scale=1.0, gate=self.S[l][:, :d], gate_scale=1.0))
-                G = Gn
+                        epi=mg.make_epilogue(residual=dS[:, :d], residual_scale=1.0, gate_scale=1.0, **gate))
 
 
 class GinTrainer(_Base):
@@ -135,13 +185,20 @@ class GinTrainer(_Base):
         super().__init__(ctx, graph, dims, precision)
         n, L, ld = self.n, self.L, self.ld
         self.hidden, self.ldh, self.gin_eps = int(hidden), round4(hidden), float(gin_eps)
+        self.upd = [update_first(self.dims[l], self.hidden, l == 0) for l in range(L)]
         self.H = [None] + [self._z(n, ld[l]) for l in range(1, L)]
-        self.Z = [self._z(n, ld[l]) for l in range(L)]
+        # aggregate-first layers keep (1 + eps) H + A H for their weight gradient; update-first ones share scratch for H W1
+        # and its gradient
+        self.Z = [None if self.upd[l] else self._z(n, ld[l]) for l in range(L)]
+        self.U = self._z(n, self.ldh) if any(self.upd) else None
         self.T = [self._z(n, self.ldh) for l in range(L)]
         self.logits = self._z(n, ld[L])
         wmax = max(ld[1:L]) if L >= 2 else 4
         self.dT, self.dZ = self._z(n, self.ldh), self._z(n, wmax)
         self.Ga, self.Gb = self._z(n, wmax), self._z(n, wmax)
+        # signs of the activations that a product writes (one bit per element), read by the backward gates
+        self.signs_H = [None] + [self._bits(self.dims[l]) for l in range(1, L)]
+        self.signs_T = [None if self.upd[l] else self._bits(self.hidden) for l in range(L)]
 
     def set_params(self, W1s, b1s, W2s, b2s):
         """Parameter order: W1[0..L), b1[0..L), W2[0..L), b2[0..L)."""
@@ -151,34 +208,45 @@ class GinTrainer(_Base):
         self.H[0], self.labels, self.train_mask = X0, labels, train_mask
 
     def forward(self):
-        L = self.L
+        L, h, keep = self.L, self.hidden, 1.0 + self.gin_eps
         for l in range(L):
             H, d = self.H[l], self.dims[l]
-            mg.spmm(self.ctx, self.g, H, self.Z[l], d, epi=mg.make_epilogue(residual=H, residual_scale=1.0 + self.gin_eps))
-            mg.gemm(self.ctx, self.precision, False, False, self.n, self.hidden, d, self.Z[l], self.params[l], self.T[l],
-                    epi=mg.make_epilogue(bias=self.params[L + l], relu=True))
+            if self.upd[l]:
+                mg.gemm(self.ctx, self.precision, False, False, self.n, h, d, H, self.params[l], self.U)
+                mg.spmm(self.ctx, self.g, self.U, self.T[l], h, epi=mg.make_epilogue(residual=self.U, residual_scale=keep, bias=self.params[L + l], relu=True))
+            else:
+                mg.spmm(self.ctx, self.g, H, self.Z[l], d, epi=mg.make_epilogue(residual=H, residual_scale=keep))
+                mg.gemm(self.ctx, self.precision, False, False, self.n, h, d, self.Z[l], self.params[l], self.T[l],
+                        epi=mg.make_epilogue(bias=self.params[L + l], relu=True, sign_bits=self.signs_T[l]))
             last = l == L - 1
             out = self.logits if last else self.H[l + 1]
-            mg.gemm(self.ctx, self.precision, False, False, self.n, self.dims[l + 1], self.hidden, self.T[l],
-                    self.params[2 * L + l], out, epi=mg.make_epilogue(bias=self.params[3 * L + l], relu=not last))
+            mg.gemm(self.ctx, self.precision, False, False, self.n, self.dims[l + 1], h, self.T[l], self.params[2 * L + l], out,
+                    epi=mg.make_epilogue(bias=self.params[3 * L + l], relu=not last, sign_bits=None if last else self.signs_H[l + 1]))
 
     def backward(self):
-        L = self.L
+        L, h, keep = self.L, self.hidden, 1.0 + self.gin_eps
         G = self.logits
         for l in range(L - 1, -1, -1):
-            d, dout, h = self.dims[l], self.dims[l + 1], self.hidden
-            mg.colsum(self.ctx, G, self.grads[3 * L + l], dout)
-            mg.gemm(self.ctx, self.precision, True, False, h, dout, self.n, self.T[l], G, self.grads[2 * L + l])
+            d, dout = self.dims[l], self.dims[l + 1]
+            mg.weight_grad(self.ctx, self.precision, h, dout, self.n, self.T[l], G, self.grads[2 * L + l], self.grads[3 * L + l])
             # dT = relu'(T) * (dP W2^T)
-            mg.gemm(self.ctx, self.precision, False, True, self.n, h, dout, G, self.params[2 * L + l], self.dT,
-                    epi=mg.make_epilogue(gate=self.T[l], gate_scale=1.0))
-            mg.colsum(self.ctx, self.dT, self.grads[L + l], h)
-            mg.gemm(self.ctx, self.precision, True, False, d, h, self.n, self.Z[l], self.dT, self.grads[l])
+            gate = dict(gate_bits=self.signs_T[l]) if self.signs_T[l] is not None else dict(gate=self.T[l])
+            mg.gemm(self.ctx, self.precision, False, True, self.n, h, dout, G, self.params[2 * L + l], self.dT, epi=mg.make_epilogue(gate_scale=1.0, **gate))
             if l > 0:
-                dZ = self.dZ[:, : self.ld[l]]
+                Gn = (self.Ga if (L - 1 - l) % 2 == 0 else self.Gb).view(-1)[: self.n * self.ld[l]].view(self.n, self.ld[l])   # the two buffers alternate
+            if self.upd[l]:
+                mg.colsum(self.ctx, self.dT, self.grads[L + l], h)
+                mg.spmm(self.ctx, self.g, self.dT, self.U, h, transposed=True, epi=mg.make_epilogue(residual=self.dT, residual_scale=keep))
+                mg.weight_grad(self.ctx, self.precision, d, h, self.n, self.H[l], self.U, self.grads[l])
+                if l > 0:
+                    mg.gemm(self.ctx, self.precision, False, True, self.n, d, h, self.U, self.params[l], Gn, epi=mg.make_epilogue(gate_bits=self.signs_H[l], gate_scale=1.0))
+                    G = Gn
+                continue
+            mg.weight_grad(self.ctx, self.precision, d, h, self.n, self.Z[l], self.dT, self.grads[l], self.grads[L + l])
+            if l > 0:
+                dZ = self.dZ.view(-1)[: self.n * self.ld[l]].view(self.n, self.ld[l])
                 mg.gemm(self.ctx, self.precision, False, True, self.n, d, h, self.dT, self.params[l], dZ)
-                Gn = (self.Ga if (L - 1 - l) % 2 == 0 else self.Gb)[:, : self.ld[l]]   # the two buffers alternate
                 # G_in = relu'(H_l) * ((1 + eps) dZ + A^T dZ)
                 mg.spmm(self.ctx, self.g, dZ, Gn, d, transposed=True,
-                        epi=mg.make_epilogue(residual=dZ, residual_scale=1.0 + self.gin_eps, gate=self.H[l], gate_scale=1.0))
+                        epi=mg.make_epilogue(residual=dZ, residual_scale=keep, gate_bits=self.signs_H[l], gate_scale=1.0))
                 G = Gn

@@ -245,13 +245,14 @@ __device__ __forceinline__ void chunk_epilogue(const TcEpi& e, float (&v)[32], i
 // Warp roles: warps 0-3 epilogue (TMEM lane quarter = warp id), warp 4 TMA producer, warp 5 TMEM
 // allocation + MMA issue.
 template <int KIND, bool MN_MAJOR>
-__global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a,
+__global__ void __launch_bounds__(TC_THREADS, 2) gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a,
                                                              const __grid_constant__ CUtensorMap map_b,
                                                              const TcParams p) {
     using Cfg = KindCfg<KIND>;
     constexpr int BK = Cfg::BK;
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t full_bar[8], empty_bar[8], acc_bar;
+    __shared__ __align__(8) uint64_t full_bar[8], empty_bar[8], acc_bar, sum_bar[8];
+    __shared__ double warp_sums[MN_MAJOR && KIND == KIND_TF32 ? 4 : 1][256];
     __shared__ uint32_t tmem_holder;
     __shared__ int abort_flag;
 
@@ -274,15 +275,18 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
 
     // Column sums of B (the bias gradient 1^T dP when B = dP) as a by-product: the four epilogue warps are
     // idle while the tiles stream through shared memory, so they add up the stages' B tiles (fp32 words, TF32 kind
-    // only) before a stage is released.  The CTAs of a column of tiles see the same B and take turns, stage by stage:
-    // with the first row of tiles doing it all, a product with two rows took almost twice as long (2.4 M x 256 x 256:
-    // 743 us without the sums, 1401 us with them).
+    // only) before a stage is released.  The CTAs of a column of tiles see the same B and take turns, stage by stage; the
+    // four warps share a stage by column chunk, or by k-rows where there are fewer chunks (with the CTAs of the first row of
+    // tiles on every stage, 2.4 M x 256 x 256 took 1401 us against 743 without the sums).  The warps do not wait on the
+    // stages' own barriers: one that skips uses of a stage cannot tell a phase from the one two uses earlier.  The MMA
+    // thread, which sees every use, hands them the stages of their turn through a second barrier per stage, of which at
+    // most one phase is ever open, because the stage is not refilled before they have released it.
     const bool do_colsum = MN_MAJOR && KIND == KIND_TF32 && p.colsum_part != nullptr;
     const int turn = (int)(tile / p.n_tiles), turns = (int)p.m_tiles;
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
-        for (int s = 0; s < p.stages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], do_colsum ? 5 : 1); }
+        for (int s = 0; s < p.stages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], do_colsum ? 5 : 1); mbar_init(&sum_bar[s], 1); }
         mbar_init(&acc_bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -323,6 +327,7 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
             // ---------------- MMA issuer ----------------
             const uint32_t idesc = make_idesc<KIND>(TC_BM, p.bn, MN_MAJOR);
             bool ok = true;
+            int whose = 0;                    // whose turn the stage is
             for (int ks = 0; ks < nk && ok; ++ks) {
                 const int s = ks % p.stages;
                 const uint32_t ph = (ks / p.stages) & 1;
@@ -341,62 +346,69 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
                     }
                     tc_mma<KIND>(tmem_base, ad, bd, idesc, (ks | kq) != 0 ? 1u : 0u);
                 }
-                tc_commit(&empty_bar[s]);     // the stage is free once these MMAs have read it
+                tc_commit(&empty_bar[s]);     // the stage is free once these MMAs have read it ...
+                if (do_colsum) {              // ... and the four warps that sum it have, where they do
+                    if (whose == turn) mbar_arrive(&sum_bar[s]);
+                    else mbar_arrive_n(&empty_bar[s], 4);
+                    if (++whose == turns) whose = 0;
+                }
             }
             if (ok) tc_commit(&acc_bar);      // the accumulator is complete
         }
     } else {
         // ---------------- epilogue: warps 0..3 own TMEM lanes 32*warp .. 32*warp+31 ----------------
         bool ok = true;
-        if (do_colsum) {
-            // warp w takes the 32-column chunks w and w + 4 of the B tile: lane (g, c) = (lane / 8, lane % 8) the columns
-            // 4 c .. 4 c + 3 of the k-rows 4 i + g, 16 bytes at a time.  A chunk is BK k-rows of 128 bytes in the 128-byte
-            // swizzle with 32-byte atoms: the 32-byte group q of k-row r sits at group position q ^ (r & 3).
+        if constexpr (MN_MAJOR && KIND == KIND_TF32) if (do_colsum) {
+            // Lane (g, c) = (lane / 8, lane % 8) takes the columns 4 c .. 4 c + 3 of the k-rows 4 i + g of every 32-column
+            // chunk, 16 bytes at a time.  A chunk is BK k-rows of 128 bytes in the 128-byte swizzle with 32-byte atoms: the
+            // 32-byte group q of k-row r sits at group position q ^ (r & 3).
             double sum[2][4] = {{0.0, 0.0, 0.0, 0.0}, {0.0, 0.0, 0.0, 0.0}};
             const int chunks = bn_pad / Cfg::CHUNK, g = lane >> 3, c = lane & 7;
-            const int at = g * 128 + ((((c >> 1) ^ g) << 1) | (c & 1)) * 16;
-            int whose = 0;                                   // whose turn this stage is
-            for (int ks = 0; ks < nk && ok; ++ks) {
+            const int parts = chunks == 1 ? 4 : chunks == 2 ? 2 : 1;       // warps that share a chunk's k-rows
+            const int first = warp / parts, part = warp % parts, rows4 = BK / 4 / parts;
+            const int at = g * 128 + ((((c >> 1) ^ g) << 1) | (c & 1)) * 16 + part * rows4 * 512;
+            uint32_t ph = 0;                                               // bit s: parity of the next hand-over of stage s
+            for (int ks = turn; ks < nk && ok; ks += turns) {
                 const int s = ks % p.stages;
-                const uint32_t ph = (ks / p.stages) & 1;
-                if (lane == 0) ok = mbar_wait(&full_bar[s], ph, &abort_flag, p.wait_limit);
+                if (lane == 0) ok = mbar_wait(&sum_bar[s], (ph >> s) & 1u, &abort_flag, p.wait_limit);
                 ok = __shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0) != 0;
                 if (!ok) { if (lane == 0) { abort_flag = 1; atomicMax(p.status, DEV_WAIT_EXPIRED); } break; }
-                if (whose == turn) {
-                    const uint8_t* sb = smem + (size_t)s * stage_bytes + a_bytes;
+                ph ^= 1u << s;
+                const uint8_t* sb = smem + (size_t)s * stage_bytes + a_bytes + at;
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int cc = warp + 4 * h;
-                        if (cc < chunks) {
-                            const uint8_t* chunk = sb + (size_t)cc * Cfg::MN_CHUNK_BYTES + at;
-                            float4 part = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int h = 0; h < 2; ++h) {
+                    const int cc = first + 4 * h;
+                    if (cc < chunks) {
+                        const uint8_t* chunk = sb + (size_t)cc * Cfg::MN_CHUNK_BYTES;
+                        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                            for (int i = 0; i < BK / 4; ++i) {
+                        for (int i = 0; i < BK / 4; ++i)
+                            if (i < rows4) {
                                 const float4 v = *reinterpret_cast<const float4*>(chunk + i * 512);
-                                part.x += v.x; part.y += v.y; part.z += v.z; part.w += v.w;
+                                a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
                             }
-                            sum[h][0] += (double)part.x; sum[h][1] += (double)part.y; sum[h][2] += (double)part.z; sum[h][3] += (double)part.w;
-                        }
+                        sum[h][0] += (double)a.x; sum[h][1] += (double)a.y; sum[h][2] += (double)a.z; sum[h][3] += (double)a.w;
                     }
                 }
-                if (++whose == turns) whose = 0;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&empty_bar[s]);      // this warp has read the stage
             }
-            if (ok) {
+            // the lanes' and then the warps' sums, in a fixed order
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int cc = warp + 4 * h;
+            for (int h = 0; h < 2; ++h)
 #pragma unroll
-                    for (int t = 0; t < 4; ++t) {
-                        double v = sum[h][t];
-                        v += __shfl_xor_sync(0xFFFFFFFFu, v, 8);
-                        v += __shfl_xor_sync(0xFFFFFFFFu, v, 16);
-                        const int col = cc * 32 + c * 4 + t;
-                        const int64_t n = n0 + col;
-                        if (g == 0 && cc < chunks && col < p.bn && n < p.N) p.colsum_part[((int64_t)blockIdx.z * turns + turn) * p.N + n] = v;
-                    }
+                for (int t = 0; t < 4; ++t) {
+                    double v = sum[h][t];
+                    v += __shfl_xor_sync(0xFFFFFFFFu, v, 8);
+                    v += __shfl_xor_sync(0xFFFFFFFFu, v, 16);
+                    if (g == 0 && first + 4 * h < chunks) warp_sums[part][(first + 4 * h) * 32 + c * 4 + t] = v;
                 }
+            asm volatile("bar.sync 1, 128;" ::: "memory");      // the four epilogue warps, all of which come here
+            for (int col = threadIdx.x; col < p.bn; col += 128) {
+                const int64_t n = n0 + col;
+                double v = warp_sums[0][col];
+                for (int q = 1; q < parts; ++q) v += warp_sums[q][col];
+                if (n < p.N) p.colsum_part[((int64_t)blockIdx.z * turns + turn) * p.N + n] = v;
             }
         }
         if (ok && nk > 0) {

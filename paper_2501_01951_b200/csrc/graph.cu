@@ -181,10 +181,10 @@ __global__ void schedule_counts_kernel(int64_t n, uint32_t top, const uint32_t* 
 }
 
 // Long rows are cut at dyadic column-block boundaries (and every seg entries): a row with d
-// entries uses 2^k blocks, the largest k <= SPMM_MAX_LOG_BLOCKS with d / 2^k >= SPMM_BLK_MIN_ENTRIES.
-__device__ __forceinline__ int row_log_blocks(int64_t d) {
+// entries uses 2^k blocks, the largest k <= SPMM_MAX_LOG_BLOCKS with d / 2^k >= schedule_blk_min.
+__device__ __forceinline__ int row_log_blocks(int64_t d, int64_t blk_min) {
     int k = 0;
-    while (k < SPMM_MAX_LOG_BLOCKS && (d >> (k + 1)) >= SPMM_BLK_MIN_ENTRIES) ++k;
+    while (k < SPMM_MAX_LOG_BLOCKS && (d >> (k + 1)) >= blk_min) ++k;
     return k;
 }
 
@@ -201,7 +201,7 @@ __device__ __forceinline__ int64_t lower_bound_col(const int32_t* __restrict__ c
 template <typename F>
 __device__ __forceinline__ int64_t row_blocks(int64_t n_cols, int64_t rb, int64_t re, const int32_t* __restrict__ col, int seg, F f) {
     const int lane = threadIdx.x & 31;
-    const int64_t nb = (int64_t)1 << row_log_blocks(re - rb), width = (n_cols + nb - 1) / nb;
+    const int64_t nb = (int64_t)1 << row_log_blocks(re - rb, schedule_blk_min(n_cols)), width = (n_cols + nb - 1) / nb;
     int64_t before = 0;
     for (int64_t b0 = 0; b0 < nb; b0 += 32) {
         const int64_t b = b0 + lane;

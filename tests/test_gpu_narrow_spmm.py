@@ -59,3 +59,21 @@ def test_narrow_aggregation(mg, problem, w):
         assert torch.all(Z[:, w:] == 0)
     mg.spmm(ctx, g, Y, Z, w, transposed=True)
     assert rel_fro(Z[:, :w].cpu().numpy().astype(np.float64), orc.aggregate(go, X.numpy(), transposed=True)) <= TOL_FP32
+
+
+@pytest.mark.parametrize("n", [1 << 20, (1 << 20) + 1])
+def test_column_blocks_of_large_graphs(mg, n):
+    """Either side of the size from which long rows are cut into more column blocks."""
+    lengths = (127, 128, 129, 255, 256, 257, 513, 3000)
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    dst = torch.cat([torch.randperm(n, generator=gen, device="cuda")[:k] for k in lengths]).int()
+    src = torch.cat([torch.full((k,), 100 * u + 7, dtype=torch.int32, device="cuda") for u, k in enumerate(lengths)])
+    ctx = mg.ctx_create(0)
+    g = mg.graph_create(ctx, n, src, dst, mg.GRAPH_NORM_NONE)
+    for w in (12, 100):
+        Y, Z = torch.randn(n, w, generator=gen, device="cuda"), torch.full((n, w), 9.0, device="cuda")
+        mg.spmm(ctx, g, Y, Z, w)
+        want = torch.zeros(n, w, dtype=torch.float64, device="cuda").index_add_(0, src.long(), Y.double()[dst.long()])
+        assert rel_fro(Z.double().cpu().numpy(), want.cpu().numpy()) <= TOL_FP32
+    assert mg.ctx_poll_status(ctx, raise_on_error=False) == 0
+    g.close(); ctx.close()

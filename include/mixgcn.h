@@ -110,8 +110,8 @@ mixgcn_status mixgcn_debug_poke_col(mixgcn_graph* g, int64_t entry, int32_t valu
 #define MIXGCN_OPT_GEMM_CTA_PAIRS 5
 mixgcn_status mixgcn_ctx_set_option(mixgcn_ctx* ctx, int32_t option, int64_t value);
 
-/* Which kernel served the dense products of this context since it was created: counts[0] fp32 FMA
- * kernel, counts[1] tcgen05 with TF32 operands, counts[2] tcgen05 with BF16 operands; counts[3] = how
+/* Which kernel served the dense products of this context since it was created: counts[0] fp32
+ * kernels, counts[1] tcgen05 with TF32 operands, counts[2] tcgen05 with BF16 operands; counts[3] = how
  * many of the tcgen05 products ran on CTA pairs.  A TF32 or BF16 request whose shape or alignment the
  * tensor-core kernels do not take is served by the next kernel down that list (never a lower precision
  * than asked for); these counters make that visible. */
@@ -281,7 +281,8 @@ mixgcn_status mixgcn_spmm_sampled(mixgcn_ctx* ctx, const mixgcn_graph* g, int tr
 mixgcn_status mixgcn_mask_pack(mixgcn_ctx* ctx, int64_t n, int32_t w, const float* X, int64_t ldx,
                                const uint8_t* bytes, uint32_t* bits, int64_t ld_bits, void* stream);
 
-#define MIXGCN_PREC_FP32 0 /* fp32 FMA on the CUDA cores */
+#define MIXGCN_PREC_FP32 0 /* fp32 operands and products: FMA on the CUDA cores, large products on the
+                              tensor cores with every operand cut into three bf16 parts that add up to it */
 #define MIXGCN_PREC_TF32 1 /* tensor cores, TF32 operands, fp32 accumulate */
 #define MIXGCN_PREC_BF16 2 /* tensor cores, BF16 operands (the fp32 operands rounded to nearest even),
                               fp32 accumulate, fp32 results */

@@ -167,7 +167,7 @@ def ctx_set_option(ctx: Ctx, option: int, value: int):
 
 
 def ctx_gemm_paths(ctx: Ctx) -> dict:
-    """Dense products served so far by the fp32 FMA kernel, the tcgen05 TF32 kernels, the tcgen05 BF16 kernels."""
+    """Dense products served so far by the fp32 kernels, the tcgen05 TF32 kernels, the tcgen05 BF16 kernels."""
     counts = (C.c_int64 * 4)()
     _check(lib.mixgcn_ctx_gemm_paths(ctx.h, counts))
     return dict(simt=int(counts[0]), tc_tf32=int(counts[1]), tc_bf16=int(counts[2]), cta_pairs=int(counts[3]))

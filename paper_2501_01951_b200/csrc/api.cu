@@ -187,7 +187,15 @@ mixgcn_status launch_gemm(mixgcn_ctx* ctx, int precision, int ta, int tb, int64_
     }
     if (st == MIXGCN_EUNSUPPORTED && loss) return st;      // the caller runs the product and the loss separately
     if (st == MIXGCN_EUNSUPPORTED) {
-        st = launch_gemm_simt(ctx, ta, tb, M, N, K, A, lda, B, ldb, C, ldc, epi, epi_row0, s, &bits_done);
+        // large fp32 products: three-part bf16 splits on the tensor cores, and the FMA kernel behind them for operands that
+        // cannot be split (it returns at once otherwise); all others: the FMA kernel
+        const int32_t* overflow = nullptr;
+        bool split_bits = false, fma_bits = false;
+        st = launch_gemm_split(ctx, ta, tb, M, N, K, A, lda, B, ldb, C, ldc, epi, epi_row0, s, &split_bits, &overflow);
+        if (st != MIXGCN_OK && st != MIXGCN_EUNSUPPORTED) return st;
+        const bool split = st == MIXGCN_OK;
+        st = launch_gemm_simt(ctx, ta, tb, M, N, K, A, lda, B, ldb, C, ldc, epi, epi_row0, s, &fma_bits, split ? overflow : nullptr);
+        bits_done = fma_bits && (!split || split_bits);
         if (st == MIXGCN_OK) ctx->gemm_path[0]++;
     }
     if (st != MIXGCN_OK) return st;
@@ -234,8 +242,8 @@ extern "C" mixgcn_status mixgcn_ctx_create(mixgcn_ctx** out, int device) {
     const mixgcn_status pool_st = pool_contexts(device, +1);
     if (pool_st != MIXGCN_OK) { delete c; return pool_st; }
     c->sm_count = prop.multiProcessorCount;
-    MIXGCN_CUDA(cudaMalloc((void**)&c->d_status, 4 * sizeof(int32_t)));
-    MIXGCN_CUDA(cudaMemset(c->d_status, 0, 4 * sizeof(int32_t)));
+    MIXGCN_CUDA(cudaMalloc((void**)&c->d_status, STATUS_WORDS * sizeof(int32_t)));
+    MIXGCN_CUDA(cudaMemset(c->d_status, 0, STATUS_WORDS * sizeof(int32_t)));
     for (int i = 0; i < 2; ++i) MIXGCN_CUDA(cudaStreamCreateWithFlags(&c->side_stream[i], cudaStreamNonBlocking));
     MIXGCN_CUDA(cudaEventCreateWithFlags(&c->fork_ev, cudaEventDisableTiming));
     for (int i = 0; i < 2; ++i) MIXGCN_CUDA(cudaEventCreateWithFlags(&c->join_ev[i], cudaEventDisableTiming));

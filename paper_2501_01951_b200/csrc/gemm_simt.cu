@@ -1,5 +1,6 @@
 // Dense update products in plain fp32 on the CUDA cores (the strict-precision mode of the
-// update line of Algorithm 2 and of its two backward products), plus the small streaming
+// update line of Algorithm 2 and of its two backward products, where they are too small or not aligned for the
+// tensor cores), plus the small streaming
 // kernels around them (column sums for the bias gradient, the ReLU/dropout gate on a gradient).
 //
 // Long reductions (K = number of nodes in the weight-gradient product) are split over CTAs into partial
@@ -43,6 +44,7 @@ struct GemmParams {
     int64_t m_tiles, n_tiles;
     int vec_a, vec_b, vec_c;     // 16-byte vector access is legal (pointer and ld aligned)
     int vec_drop, vec_gate;      // the same for four mask bytes / four gate values at a multiple of four columns
+    const int32_t* only_if;      // nullable: every CTA returns at once where this word is zero
     Epi epi;
 };
 
@@ -93,6 +95,7 @@ __global__ void __launch_bounds__(SimtCfg<BM, BN, TN, KG>::NT, SimtCfg<BM, BN, T
     constexpr int A_PITCH = TA ? BM + 4 : BK + 4, B_PITCH = BN + 4;
     constexpr int A_FLOATS = TA ? BK * A_PITCH : BM * A_PITCH, B_FLOATS = BK * B_PITCH;
     extern __shared__ __align__(16) float smem_f[];
+    if (p.only_if && *p.only_if == 0) return;
     const int tid = threadIdx.x, lane = tid & 31;
     const int kg = tid / SimtCfg<BM, BN, TN, KG>::GROUP, warp = (tid % SimtCfg<BM, BN, TN, KG>::GROUP) >> 5;
     // a warp covers 4 x 8 micro-tiles (TX >= 8) or 8 x 4
@@ -341,7 +344,8 @@ __global__ void __launch_bounds__(SimtCfg<BM, BN, TN, KG>::NT, SimtCfg<BM, BN, T
 // cost one thread a chain of a hundred loads otherwise (16 K elements, 148 splits: 20 -> 4 us).
 constexpr int RED_PARTS = 8;
 __global__ void __launch_bounds__(32 * RED_PARTS) splitk_reduce_kernel(int64_t M, int64_t N, int splits, const float* __restrict__ part,
-                                                                      float* __restrict__ C, int64_t ldc, const Epi epi) {
+                                                                      float* __restrict__ C, int64_t ldc, const Epi epi, const int32_t* only_if) {
+    if (only_if && *only_if == 0) return;
     __shared__ double sm[RED_PARTS][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t i = (int64_t)blockIdx.x * 32 + lane, MN = M * N;
@@ -475,7 +479,7 @@ namespace mixgcn {
 // *bits_done: whether the sign bitmap, if one is asked for, was written (not where K is split).
 mixgcn_status launch_gemm_simt(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64_t N, int64_t K,
                                const float* A, int64_t lda, const float* B, int64_t ldb, float* C, int64_t ldc,
-                               const mixgcn_epilogue* epi, int64_t epi_row0, cudaStream_t s, bool* bits_done) {
+                               const mixgcn_epilogue* epi, int64_t epi_row0, cudaStream_t s, bool* bits_done, const int32_t* only_if) {
     if (bits_done) *bits_done = false;
     if (M <= 0 || N <= 0) return MIXGCN_OK;
     GemmParams p{};
@@ -488,6 +492,7 @@ mixgcn_status launch_gemm_simt(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64
         p.epi.sign_bits = epi->sign_bits; p.epi.ld_sign_bits = epi->ld_sign_bits;
     }
     p.epi.row0 = epi_row0;
+    p.only_if = only_if;
     p.vec_a = aligned16(A) && (lda & 3) == 0;
     p.vec_b = aligned16(B) && (ldb & 3) == 0;
     p.vec_c = aligned16(C) && (ldc & 3) == 0;
@@ -534,7 +539,7 @@ mixgcn_status launch_gemm_simt(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64
     if (splits > 1) {
         LaunchScope scope(ctx, PH_GEMM, s);
         const int64_t total = M * N;
-        splitk_reduce_kernel<<<(unsigned)((total + 31) / 32), 32 * RED_PARTS, 0, s>>>(M, N, (int)splits, p.C, C, ldc, p.epi);
+        splitk_reduce_kernel<<<(unsigned)((total + 31) / 32), 32 * RED_PARTS, 0, s>>>(M, N, (int)splits, p.C, C, ldc, p.epi, only_if);
         MIXGCN_CUDA(cudaGetLastError());
     } else if (bits_done) {
         *bits_done = p.epi.sign_bits != nullptr;
@@ -552,7 +557,7 @@ mixgcn_status launch_splitk_reduce(mixgcn_ctx* ctx, int64_t M, int64_t N, int sp
     }
     LaunchScope scope(ctx, PH_GEMM, s);
     const int64_t total = M * N;
-    splitk_reduce_kernel<<<(unsigned)((total + 31) / 32), 32 * RED_PARTS, 0, s>>>(M, N, splits, part, C, ldc, e);
+    splitk_reduce_kernel<<<(unsigned)((total + 31) / 32), 32 * RED_PARTS, 0, s>>>(M, N, splits, part, C, ldc, e, nullptr);
     MIXGCN_CUDA(cudaGetLastError());
     return MIXGCN_OK;
 }

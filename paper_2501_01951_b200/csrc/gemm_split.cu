@@ -1,0 +1,618 @@
+// fp32 dense products on the tensor cores: every fp32 operand is cut into three bf16 parts, a = a0 + a1 + a2 with each part the
+// rounded-to-nearest bf16 of what the parts before it leave.  8 + 8 + 8 bits: the three parts ARE the fp32 value (as long as
+// they stay above bf16's smallest number, 2^-133), and a product of two parts is exact in fp32.  Of the nine products of parts
+// the six down to 2^-16 of the largest are formed; the three left out are below 2^-25 of |a b| together, half a unit of an
+// fp32 rounding, and not all of one sign.  The split of matrices into parts that multiply without error is that of Ozaki,
+// Ogita, Oishi and Rump ("Error-free transformations of matrix multiplication", 2012).
+//
+// What the tensor core does not do is round its accumulator to nearest: it cuts it off, once per instruction, so that an error
+// grows with the number of instructions on one accumulator.  Two things keep these products as accurate as the fp32 FMA
+// kernel (the same operands against fp64, of both signs and positive, in the tests):
+//  * the large products a0 b0 are accumulated over 32 terms only (two instructions); the epilogue warps then add the
+//    accumulator to fp32 sums in registers, rounding to nearest, while the next 32 terms go to a second accumulator;
+//  * the five small products, at most 2^-8 of the large ones, have an accumulator of their own for up to 1024 terms.
+//
+// Bound: shared memory.  A stage of 32 terms of a 128 x 128 tile is twelve instructions, 768 cycles of the tensor core and as
+// many of operand reads; the raw tile in, its conversion and the planes of B add 640 cycles of the same port.  The bf16 rate
+// over six (270 TFLOP/s of fp32 products; the FMA pipes have 72) is therefore not reached: tensor pipe 35 to 40 % active.
+// Measured against the FMA kernel: 170 K x 256 x 256 forward 508 -> 178 us (126 TFLOP/s), its weight gradient 466 -> 163,
+// 170 K x 40 x 256 145 -> 79, 1 M x 300 x 300 4493 -> 1590.
+//
+// What the layout of the work has to avoid is the latency of one stage's hand-overs in series (a wait, a proxy fence and an
+// arrival each): one group of conversion warps on every stage took 212 us where two groups on alternate stages take 178;
+// loads to registers before the fence instead of raw tiles by TMA, as much; the large products issued before the small ones
+// (the wait for their accumulator in front), 190; issue by a divergent lane instead of an elected one of a converged warp, 10 % more.
+//
+// Infinities and values that round to a bf16 infinity do not survive the split (inf - inf): the converting warps record that
+// they met one, and the FMA kernel, launched behind, then computes the product over again (otherwise it returns at once).
+// A value below 2^-109 keeps an absolute error of up to 2^-134, its last part being a bf16 subnormal.
+//
+//  * K-major form (forward, input gradient): persistent CTAs over 128 x bn tiles; the weights are cut once into three packed
+//    planes, which TMA brings in; the fp32 tiles of A come by TMA too, and the conversion warps cut them into part tiles.
+//  * MN-major form (weight gradient): K split over CTAs, both operands converted by the CTA that multiplies them.
+// Warps 0-7 epilogue (two per TMEM lane quarter, half of the columns each), 8-15 conversion, 16 TMA, 17 MMA issue.
+#include "internal.cuh"
+#include "tc_epilogue.cuh"
+#include "tc_ptx.cuh"
+
+using namespace mixgcn;
+using namespace mixgcn::tc;
+
+namespace {
+
+constexpr int BM = 128, BN_MAX = 128, BK = 32, PARTS = 3;
+constexpr int EPI_WARPS = 8, CONV_WARPS = 8, TMA_WARP = EPI_WARPS + CONV_WARPS, MMA_WARP = TMA_WARP + 1, THREADS = (MMA_WARP + 1) * 32;
+constexpr int GROUPS = 2, GROUP_WARPS = CONV_WARPS / GROUPS, GROUP_THREADS = GROUP_WARPS * 32;   // groups of conversion warps, on alternate stages
+constexpr int STAGES_MAX = 4, RAW_MAX = 8;      // most stages of part tiles and slots of raw fp32 tiles
+constexpr int HI_STAGES = 32 / BK, LO_STAGES = 1024 / BK;           // stages per accumulator of the large and of the small products
+constexpr uint32_t TMEM_COLS = 512, LO_COL = 256, BUF_COLS = 128;   // two accumulators for the large products, two for the small ones
+constexpr int RAW_BYTES = BM * BK * 4, KK_PART = BM * BK * 2;       // a raw tile; K-major part tiles: 64-byte rows and swizzle
+constexpr int CHUNK = BK * 128, MM_PART = BM / 64 * CHUNK;          // MN-major tiles: chunks of 64 columns, 128-byte k-rows and swizzle
+
+struct SplitParams {
+    int64_t M, N, K;
+    int bn;                       // columns of a tile: a multiple of 16 up to BN_MAX
+    int64_t m_tiles, n_tiles;
+    int stages, raw_slots;
+    int plane_rows;               // K-major: rows of one packed plane of B
+    int64_t k_per_split;          // MN-major: a multiple of BK
+    float* C; int64_t ldc; int vec_c;   // MN-major: partial tiles [splits][M][N] or C itself
+    int raw;
+    TcEpi epi;
+    int32_t* status;
+    uint32_t wait_limit;
+    int32_t* overflow;            // set when an operand cannot be split
+};
+
+struct Ring {                     // position in a ring of slots and the parity of its use
+    int i = 0;
+    uint32_t use = 0;
+    __device__ __forceinline__ void next(int n, int by = 1) { if ((i += by) >= n) { i -= n; use ^= 1; } }      // by <= n
+};
+
+__device__ __forceinline__ void add2(float& x, float& y, float a, float b) {
+    asm("{.reg .b64 p, q; mov.b64 p, {%0, %1}; mov.b64 q, {%2, %3}; add.rn.f32x2 p, p, q; mov.b64 {%0, %1}, p;}" : "+f"(x), "+f"(y) : "f"(a), "f"(b));
+}
+// (x, y) minus the two bf16 values of `parts`: exact
+__device__ __forceinline__ void sub_parts(float& x, float& y, uint32_t parts) {
+    asm("{.reg .b64 p, q, m; mov.b64 p, {%0, %1}; mov.b64 q, {%2, %3}; mov.b64 m, {%4, %4}; fma.rn.f32x2 p, q, m, p; mov.b64 {%0, %1}, p;}"
+        : "+f"(x), "+f"(y) : "f"(__uint_as_float(parts << 16)), "f"(__uint_as_float(parts & 0xFFFF0000u)), "f"(-1.0f));
+}
+
+// Four floats at `src` -> their three bf16 parts at dst + t * part_bytes.  top: per half the largest |first part| met, infinity
+// when a value cannot be split (a NaN needs no note, its first part is one).
+__device__ __forceinline__ void split4(float4 v, uint8_t* dst, uint32_t part_bytes, uint32_t& top) {
+#pragma unroll
+    for (int t = 0; t < PARTS; ++t) {
+        const uint32_t lo = pack_bf16(v.x, v.y), hi = pack_bf16(v.z, v.w);
+        *reinterpret_cast<uint2*>(dst + t * part_bytes) = make_uint2(lo, hi);
+        if (t == 0) {
+            asm("{.reg .b32 a; abs.bf16x2 a, %1; max.bf16x2 %0, %0, a;}" : "+r"(top) : "r"(lo));
+            asm("{.reg .b32 a; abs.bf16x2 a, %1; max.bf16x2 %0, %0, a;}" : "+r"(top) : "r"(hi));
+        }
+        if (t + 1 < PARTS) { sub_parts(v.x, v.y, lo); sub_parts(v.z, v.w, hi); }
+    }
+}
+__device__ __forceinline__ bool has_inf(uint32_t top) { return (top & 0x7FFFu) == 0x7F80u || ((top >> 16) & 0x7FFFu) == 0x7F80u; }
+
+// This thread's share of a raw tile: the float4 t, t + 128, ...
+constexpr int RAW_ITS = BM * BK / 4 / GROUP_THREADS;
+template <int N>
+__device__ __forceinline__ void take_raw(float4 (&v)[N], const uint8_t* tile, int t) {
+#pragma unroll
+    for (int it = 0; it < N; ++it) v[it] = reinterpret_cast<const float4*>(tile)[t + it * GROUP_THREADS];
+}
+
+// barriers of a CTA, TMEM address and abort flag
+struct Shared {
+    uint64_t raw_full[RAW_MAX], raw_empty[RAW_MAX];   // raw fp32 tiles: TMA -> conversion -> TMA
+    uint64_t full[STAGES_MAX], empty[STAGES_MAX];             // part tiles: conversion (and TMA) -> MMA -> conversion
+    uint64_t hi_full[2], hi_empty[2], lo_full[2], lo_empty[2];   // accumulators: MMA -> epilogue -> MMA
+    uint32_t tmem;
+    int abort_flag;
+};
+
+__device__ __forceinline__ uint32_t cta_begin(Shared& b, int full_count, int warp) {
+    if (threadIdx.x == 0) {
+        b.abort_flag = 0;
+        for (int s = 0; s < RAW_MAX; ++s) { mbar_init(&b.raw_full[s], 1); mbar_init(&b.raw_empty[s], GROUP_WARPS); }
+        for (int s = 0; s < STAGES_MAX; ++s) { mbar_init(&b.full[s], (uint32_t)full_count); mbar_init(&b.empty[s], 1); }
+        for (int s = 0; s < 2; ++s) { mbar_init(&b.hi_full[s], 1); mbar_init(&b.hi_empty[s], EPI_WARPS); mbar_init(&b.lo_full[s], 1); mbar_init(&b.lo_empty[s], EPI_WARPS); }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == MMA_WARP) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&b.tmem)), "r"(TMEM_COLS) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    return b.tmem;
+}
+
+__device__ __forceinline__ void cta_end(Shared& b, int warp, uint32_t tmem) {
+    if (threadIdx.x == 0 && b.abort_flag) {
+        for (int i = 0; i < 200; ++i) __nanosleep(1000);      // a wait expired: let copies in flight land
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == MMA_WARP) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+    }
+}
+
+__device__ __forceinline__ bool thread_wait(uint64_t* bar, uint32_t parity, Shared& b, const SplitParams& p) {
+    volatile int* flag = &b.abort_flag;
+    if (mbar_wait(bar, parity, flag, p.wait_limit)) return true;
+    *flag = 1;
+    atomicMax(p.status, DEV_WAIT_EXPIRED);
+    return false;
+}
+// One wait of a whole warp.
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, Shared& b, const SplitParams& p) {
+    return __all_sync(0xFFFFFFFFu, thread_wait(bar, parity, b, p)) != 0;
+}
+
+// add an accumulator (this warp's 32 lanes, `chunks` blocks of 32 columns) to the sums in registers
+__device__ __forceinline__ void add_accumulator(uint32_t taddr, int chunks, float (&acc)[2][32]) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        if (k < chunks) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                uint32_t r[16];
+                tc_ld16(taddr + (uint32_t)(k * 32 + h * 16), r);
+                tc_wait_ld();
+#pragma unroll
+                for (int q = 0; q < 16; q += 2) add2(acc[k][h * 16 + q], acc[k][h * 16 + q + 1], __uint_as_float(r[q]), __uint_as_float(r[q + 1]));
+            }
+        }
+}
+
+// The MMA warp's state: position in the stages and in the two pairs of accumulators.
+struct MmaState {
+    Ring stage;
+    uint32_t hc = 0, lc = 0;
+    int hi_used = 0, lo_used = 0; // stages in the current accumulators
+};
+
+// One lane of a converged warp, always the same one.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{.reg .pred q; elect.sync _|q, 0xFFFFFFFF; selp.u32 %0, 1, 0, q;}" : "=r"(p));
+    return p != 0;
+}
+
+// All products of one stage, by the whole MMA warp: uniform control flow up to the elected lane leaves the descriptors in uniform
+// registers.  desc_a, desc_b: descriptors of the first part tiles, the others a_part and b_part bytes on, the second 16
+// terms k_step bytes on (the address is the descriptor's low field, in units of 16 bytes).  last: no stage of this tile follows.
+__device__ __forceinline__ bool mma_stage(MmaState& st, Shared& b, const SplitParams& p, uint32_t tmem, uint32_t idesc, bool last, uint64_t desc_a, uint64_t desc_b,
+                                          uint32_t a_part, uint32_t b_part, uint32_t k_step) {
+    if (!warp_wait(&b.full[st.stage.i], st.stage.use, b, p)) return false;
+    if (st.lo_used == 0 && !warp_wait(&b.lo_empty[st.lc & 1], ((st.lc >> 1) & 1) ^ 1, b, p)) return false;
+    tc_fence_after();
+    auto da = [&](int part, int k16) { return desc_a + ((part * a_part + k16 * k_step) >> 4); };
+    auto db = [&](int part, int k16) { return desc_b + ((part * b_part + k16 * k_step) >> 4); };
+    const uint32_t hi = tmem + (st.hc & 1) * BUF_COLS, lo = tmem + LO_COL + (st.lc & 1) * BUF_COLS;
+    const bool hi_ends = st.hi_used + 1 == HI_STAGES || last, lo_ends = st.lo_used + 1 == LO_STAGES || last;
+    if (elect_one()) {
+        constexpr int PA[5] = {0, 1, 1, 0, 2}, PB[5] = {1, 0, 1, 2, 0};
+#pragma unroll
+        for (int t = 0; t < 5; ++t) {
+            tc_mma<KIND_BF16>(lo, da(PA[t], 0), db(PB[t], 0), idesc, st.lo_used || t ? 1u : 0u);
+            tc_mma<KIND_BF16>(lo, da(PA[t], 1), db(PB[t], 1), idesc, 1u);
+        }
+    }
+    __syncwarp();
+    if (st.hi_used == 0 && !warp_wait(&b.hi_empty[st.hc & 1], ((st.hc >> 1) & 1) ^ 1, b, p)) return false;
+    tc_fence_after();
+    if (elect_one()) {
+        tc_mma<KIND_BF16>(hi, da(0, 0), db(0, 0), idesc, st.hi_used ? 1u : 0u);
+        tc_mma<KIND_BF16>(hi, da(0, 1), db(0, 1), idesc, 1u);
+        if (hi_ends) tc_commit(&b.hi_full[st.hc & 1]);
+        tc_commit(&b.empty[st.stage.i]);
+        if (lo_ends) tc_commit(&b.lo_full[st.lc & 1]);
+    }
+    __syncwarp();
+    st.hi_used = hi_ends ? 0 : st.hi_used + 1;
+    st.lo_used = lo_ends ? 0 : st.lo_used + 1;
+    st.hc += hi_ends;
+    st.lc += lo_ends;
+    st.stage.next(p.stages);
+    return true;
+}
+
+// An epilogue warp's sums of one tile over nk stages.  t_row: TMEM address of its lanes and first column.
+struct EpiState { uint32_t hc = 0, lc = 0; };
+__device__ __forceinline__ bool sum_tile(EpiState& st, Shared& b, const SplitParams& p, uint32_t t_row, int chunks, int nk, int lane, float (&acc)[2][32]) {
+    auto take = [&](uint64_t* full, uint64_t* empty, uint32_t& c, uint32_t col) {
+        if (!warp_wait(&full[c & 1], (c >> 1) & 1, b, p)) return false;
+        tc_fence_after();
+        add_accumulator(t_row + col + (c & 1) * BUF_COLS, chunks, acc);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&empty[c & 1]);
+        ++c;
+        return true;
+    };
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int q = 0; q < 32; ++q) acc[k][q] = 0.0f;
+    for (int ks = HI_STAGES;; ks += HI_STAGES) {
+        if (!take(b.hi_full, b.hi_empty, st.hc, 0)) return false;
+        if ((ks % LO_STAGES == 0 || ks >= nk) && !take(b.lo_full, b.lo_empty, st.lc, LO_COL)) return false;
+        if (ks >= nk) return true;
+    }
+}
+
+// ---------------------------------------------------------------- K-major form
+__global__ void __launch_bounds__(THREADS, 1) gemm_split_kk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
+                                                                   const __grid_constant__ CUtensorMap map_c, const SplitParams p, const int tma_store) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) Shared bars;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int bn32 = (p.bn + 31) & ~31;
+    const uint32_t b_part = (uint32_t)bn32 * BK * 2, stage_bytes = PARTS * (KK_PART + b_part);
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t* raws = smem + (size_t)p.stages * stage_bytes;
+    uint8_t* boxes = raws + (size_t)p.raw_slots * RAW_BYTES;
+    const int nk = (int)((p.K + BK - 1) / BK);
+    const int64_t tiles = p.m_tiles * p.n_tiles;
+    const uint32_t tmem = cta_begin(bars, GROUP_WARPS + 1, warp);
+
+    if (warp < EPI_WARPS) {
+        // 8 warps x 128 + 8 x 64 + 2 x 96 registers a thread are the 18 x 96 of the launch: the sums and the epilogue fit (191 us
+        // for the forward product above with their spills, 178 without)
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 128;");
+        const int quarter = warp & 3, half = warp >> 2;
+        const int span = bn32 > 64 ? 64 : 32;                               // columns of this warp
+        const int c_first = half * span;
+        const int chunks = p.bn <= c_first ? 0 : (p.bn - c_first > 32 && span == 64) ? 2 : 1;
+        const uint32_t t_row = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c_first;
+        const bool masks = p.epi.drop != nullptr || p.epi.gate != nullptr || p.epi.gate_bits != nullptr;
+        uint8_t* const box = boxes + (size_t)warp * 4096;
+        EpiState st;
+        for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+            const int64_t m0 = (int64_t)((uint32_t)tile / (uint32_t)p.n_tiles) * BM, m = m0 + quarter * 32 + lane;
+            const int n0 = (int)((uint32_t)tile % (uint32_t)p.n_tiles) * p.bn;
+            uint32_t dw[2] = {0xFFFFFFFFu, 0xFFFFFFFFu}, gw[2] = {0xFFFFFFFFu, 0xFFFFFFFFu};
+            if (masks && chunks) mask_words(p.epi, m0 + quarter * 32, p.M, p.N, n0 + c_first, 32, n0 + (p.bn < c_first + span ? p.bn : c_first + span), lane, dw, gw);
+            float acc[2][32];
+            if (!sum_tile(st, bars, p, t_row, chunks, nk, lane, acc)) break;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                if (k >= chunks) break;
+                const int c0 = c_first + k * 32, nb = n0 + c0;
+                if (nb >= p.N) break;
+                chunk_epilogue(p.epi, acc[k], nb, p.N, nullptr, dw[k], gw[k]);
+                if (p.epi.sign_bits && m < p.M) p.epi.sign_bits[(p.epi.row0 + m) * p.epi.ld_sign_bits + (nb >> 5)] = sign_word(acc[k], nb, p.N);
+                if (tma_store && lane == 0) bulk_wait_read<0>();   // the store that last used this box has read it
+                __syncwarp();
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    *reinterpret_cast<float4*>(box + lane * 128 + ((q ^ (lane & 7)) << 4)) =
+                        make_float4(acc[k][4 * q], acc[k][4 * q + 1], acc[k][4 * q + 2], acc[k][4 * q + 3]);
+                if (tma_store && (nb + 32 <= p.N || (p.N & 3) == 0)) {
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) {
+                        tma_store_2d(&map_c, box, nb, (int32_t)(m0 + quarter * 32));
+                        bulk_commit();
+                    }
+                } else {
+                    // row by row: TMA stores whole 16-byte units, and what lies behind the matrix's last column is not ours
+                    __syncwarp();
+                    const int64_t first = m0 + quarter * 32;
+                    if (nb + lane < p.N && c0 + lane < p.bn)
+                        for (int r = 0; r < 32 && first + r < p.M; ++r)
+                            p.C[(first + r) * p.ldc + nb + lane] = *reinterpret_cast<const float*>(box + r * 128 + (((lane >> 2) ^ (r & 7)) << 4) + (lane & 3) * 4);
+                    __syncwarp();
+                }
+            }
+        }
+        if (tma_store && lane == 0) bulk_wait_all();
+    } else if (warp < TMA_WARP) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+        // Conversion: thread t of a group takes the float4 t + 128 it of the tile's 128 x 8, row it * 16 + t / 8; the swizzle
+        // (bits 4-5 of the offset by bits 7-8) is the same for all of them.
+        const int t = (threadIdx.x - EPI_WARPS * 32) % GROUP_THREADS, group = (warp - EPI_WARPS) / GROUP_WARPS;
+        const uint32_t at = (uint32_t)((t >> 3) * 64 + ((((t & 7) >> 1) ^ ((t >> 4) & 3)) << 4) + (t & 1) * 8);
+        const int64_t stages = blockIdx.x < tiles ? (tiles - blockIdx.x + gridDim.x - 1) / gridDim.x * nk : 0;
+        Ring raw, stage;
+        raw.next(p.raw_slots, group);
+        stage.next(p.stages, group);
+        uint32_t top = 0;
+        for (int64_t st = group; st < stages; st += GROUPS) {
+            if (!warp_wait(&bars.raw_full[raw.i], raw.use, bars, p)) break;
+            float4 v[RAW_ITS];
+            take_raw(v, raws + (size_t)raw.i * RAW_BYTES, t);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars.raw_empty[raw.i]);
+            if (!warp_wait(&bars.empty[stage.i], stage.use ^ 1, bars, p)) break;
+            uint8_t* dst = smem + (size_t)stage.i * stage_bytes + at;
+#pragma unroll
+            for (int it = 0; it < RAW_ITS; ++it) split4(v[it], dst + it * 16 * 64, KK_PART, top);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars.full[stage.i]);
+            raw.next(p.raw_slots, GROUPS);
+            stage.next(p.stages, GROUPS);
+        }
+        if (has_inf(top)) *p.overflow = 1;
+    } else if (warp == TMA_WARP) {
+        // The raw tiles of A run raw_slots - 1 stages ahead of the planes of B.
+        if (lane == 0) {
+            Ring raw, stage;
+            int64_t a_tile = blockIdx.x;
+            int a_ks = 0;
+            auto load_a = [&]() {
+                if (a_tile >= tiles) return true;
+                if (!thread_wait(&bars.raw_empty[raw.i], raw.use ^ 1, bars, p)) return false;
+                mbar_expect_tx(&bars.raw_full[raw.i], RAW_BYTES);
+                tma_load_2d(raws + (size_t)raw.i * RAW_BYTES, &map_a, a_ks * BK, (int32_t)((uint32_t)a_tile / (uint32_t)p.n_tiles) * BM, &bars.raw_full[raw.i]);
+                raw.next(p.raw_slots);
+                if (++a_ks == nk) { a_ks = 0; a_tile += gridDim.x; }
+                return true;
+            };
+            bool ok = true;
+            for (int i = 0; i + 1 < p.raw_slots && ok; ++i) ok = load_a();
+            for (int64_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
+                const int n0 = (int)((uint32_t)tile % (uint32_t)p.n_tiles) * p.bn;
+                for (int ks = 0; ks < nk && ok; ++ks) {
+                    if (!thread_wait(&bars.empty[stage.i], stage.use ^ 1, bars, p)) { ok = false; break; }
+                    uint8_t* sb = smem + (size_t)stage.i * stage_bytes + PARTS * KK_PART;
+                    mbar_expect_tx(&bars.full[stage.i], PARTS * b_part);
+                    for (int q = 0; q < PARTS; ++q) tma_load_2d(sb + q * b_part, &map_b, ks * BK, q * p.plane_rows + n0, &bars.full[stage.i]);
+                    stage.next(p.stages);
+                    ok = load_a();
+                }
+            }
+        }
+    } else {
+        const uint32_t idesc = make_idesc<KIND_BF16>(BM, p.bn, false);
+        MmaState st;
+        bool ok = true;
+        for (int64_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x)
+            for (int ks = 0; ks < nk && ok; ++ks) {
+                const uint32_t sa = smem_u32(smem + (size_t)st.stage.i * stage_bytes), sb = sa + PARTS * KK_PART;
+                ok = mma_stage(st, bars, p, tmem, idesc, ks + 1 == nk, make_desc(sa, 16, 512, 4), make_desc(sb, 16, 512, 4), KK_PART, b_part, 32);
+            }
+    }
+    cta_end(bars, warp, tmem);
+}
+
+// ---------------------------------------------------------------- MN-major form (weight gradient)
+__global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
+                                                                   const SplitParams p) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) Shared bars;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int bw = p.bn > 64 ? 128 : 64;                                    // columns of B that are converted
+    const uint32_t b_part = (uint32_t)(bw / 64) * CHUNK, stage_bytes = PARTS * (MM_PART + b_part);
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t* raws = smem + (size_t)p.stages * stage_bytes;
+    const int64_t tile = blockIdx.x, m0 = (tile / p.n_tiles) * BM, n0 = (tile % p.n_tiles) * p.bn;
+    const int64_t kb = (int64_t)blockIdx.z * p.k_per_split, ke = kb + p.k_per_split < p.K ? kb + p.k_per_split : p.K;
+    const int nk = (int)((ke - kb + BK - 1) / BK);
+    const uint32_t tmem = cta_begin(bars, GROUP_WARPS, warp);
+
+    if (warp < EPI_WARPS) {
+        const int quarter = warp & 3, half = warp >> 2;
+        const int span = p.bn > 64 ? 64 : 32, c_first = half * span;
+        const int chunks = p.bn <= c_first ? 0 : (p.bn - c_first > 32 && span == 64) ? 2 : 1;
+        EpiState st;
+        float acc[2][32];
+        const bool ok = sum_tile(st, bars, p, tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c_first, chunks, nk, lane, acc);
+        const int64_t m = m0 + quarter * 32 + lane;
+        if (ok && m < p.M) {
+            float* row = p.C + (p.raw ? (int64_t)blockIdx.z * p.M * p.N : 0) + m * p.ldc;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                if (k >= chunks) break;
+                const int c0 = c_first + k * 32;
+                const int64_t nb = n0 + c0;
+                float* dst = row + nb;
+                if (p.vec_c && nb + 31 < p.N && c0 + 31 < p.bn) {
+#pragma unroll
+                    for (int q = 0; q < 32; q += 4)
+                        *reinterpret_cast<float4*>(dst + q) = make_float4(acc[k][q], acc[k][q + 1], acc[k][q + 2], acc[k][q + 3]);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 32; ++q)
+                        if (nb + q < p.N && c0 + q < p.bn) dst[q] = acc[k][q];
+                }
+            }
+        }
+    } else if (warp < TMA_WARP) {
+        // Conversion: thread t of a group takes the float4 t + 128 it.  Of a tile of 128 columns that is k-row it * 4 + t / 32, of
+        // one of 64 k-row it * 8 + t / 16; the swizzle goes by k-row mod 8.
+        const int t = (threadIdx.x - EPI_WARPS * 32) % GROUP_THREADS, group = (warp - EPI_WARPS) / GROUP_WARPS;
+        auto place = [](int row, int c4) { return (uint32_t)((c4 >> 4) * CHUNK + row * 128 + ((((c4 & 15) >> 1) ^ (row & 7)) << 4) + (c4 & 1) * 8); };
+        const uint32_t at_a = place(t >> 5, t & 31), at_b = place(t >> 4, t & 15);
+        Ring raw, stage;
+        raw.next(p.raw_slots, 2 * group);                             // 2 * GROUPS slots at least: a group is never two uses behind
+        stage.next(p.stages, group);
+        uint32_t top = 0;
+        float4 v[RAW_ITS];
+        for (int ks = group; ks < nk; ks += GROUPS) {
+            if (!warp_wait(&bars.raw_full[raw.i], raw.use, bars, p)) break;
+            take_raw(v, raws + (size_t)raw.i * RAW_BYTES, t);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars.raw_empty[raw.i]);
+            raw.next(p.raw_slots);
+            if (!warp_wait(&bars.empty[stage.i], stage.use ^ 1, bars, p)) break;
+            uint8_t* dst = smem + (size_t)stage.i * stage_bytes;
+#pragma unroll
+            for (int it = 0; it < RAW_ITS; ++it) split4(v[it], dst + (at_a ^ (it & 1) * 64) + it * 4 * 128, MM_PART, top);
+            if (!warp_wait(&bars.raw_full[raw.i], raw.use, bars, p)) break;
+            dst += PARTS * MM_PART;
+            if (bw == 128) {
+                take_raw(v, raws + (size_t)raw.i * RAW_BYTES, t);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&bars.raw_empty[raw.i]);
+#pragma unroll
+                for (int it = 0; it < RAW_ITS; ++it) split4(v[it], dst + (at_a ^ (it & 1) * 64) + it * 4 * 128, b_part, top);
+            } else {
+                float4 w[RAW_ITS / 2];
+                take_raw(w, raws + (size_t)raw.i * RAW_BYTES, t);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&bars.raw_empty[raw.i]);
+#pragma unroll
+                for (int it = 0; it < RAW_ITS / 2; ++it) split4(w[it], dst + at_b + it * 8 * 128, b_part, top);
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars.full[stage.i]);
+            raw.next(p.raw_slots);
+            raw.next(p.raw_slots, 2 * (GROUPS - 1));
+            stage.next(p.stages, GROUPS);
+        }
+        if (has_inf(top)) *p.overflow = 1;
+    } else if (warp == TMA_WARP) {
+        if (lane == 0) {
+            Ring raw;
+            for (int u = 0; u < 2 * nk; ++u, raw.next(p.raw_slots)) {         // A, B, A, B, ...
+                if (!thread_wait(&bars.raw_empty[raw.i], raw.use ^ 1, bars, p)) break;
+                const int32_t k = (int32_t)(kb + (int64_t)(u >> 1) * BK);
+                mbar_expect_tx(&bars.raw_full[raw.i], u & 1 ? (uint32_t)bw * BK * 4 : (uint32_t)RAW_BYTES);
+                tma_load_2d(raws + (size_t)raw.i * RAW_BYTES, u & 1 ? &map_b : &map_a, (int32_t)(u & 1 ? n0 : m0), k, &bars.raw_full[raw.i]);
+            }
+        }
+    } else {
+        const uint32_t idesc = make_idesc<KIND_BF16>(BM, p.bn, true);
+        MmaState st;
+        for (int ks = 0; ks < nk; ++ks) {
+            const uint32_t sa = smem_u32(smem + (size_t)st.stage.i * stage_bytes), sb = sa + PARTS * MM_PART;
+            if (!mma_stage(st, bars, p, tmem, idesc, ks + 1 == nk, make_desc(sa, CHUNK, 1024, 2), make_desc(sb, CHUNK, 1024, 2), MM_PART, b_part, 2048)) break;
+        }
+    }
+    cta_end(bars, warp, tmem);
+}
+
+// Packed planes of the weight matrix: plane q of dst (rows x kpad bf16) holds part q of trans ? src[k][n] : src[n][k], zeros
+// outside N x K.
+__global__ void pack_split_kernel(const float* __restrict__ src, int64_t ld, int trans, int N, int K, int rows, int kpad,
+                                  uint16_t* __restrict__ dst, int32_t* overflow) {
+    const int64_t plane = (int64_t)rows * kpad, i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= plane) return;
+    const int n = trans ? (int)(i % rows) : (int)(i / kpad), k = trans ? (int)(i / rows) : (int)(i % kpad);     // consecutive threads read consecutive words
+    float v = 0.0f;
+    if (n < N && k < K) v = trans ? __ldg(src + (int64_t)k * ld + n) : __ldg(src + (int64_t)n * ld + k);
+#pragma unroll
+    for (int q = 0; q < PARTS; ++q) {
+        const uint32_t b = pack_bf16(v, 0.0f) & 0xFFFFu;
+        if (q == 0 && (b & 0x7FFFu) == 0x7F80u) *overflow = 1;
+        dst[q * plane + (int64_t)n * kpad + k] = (uint16_t)b;
+        v -= __uint_as_float(b << 16);
+    }
+}
+
+}  // namespace
+
+namespace mixgcn {
+
+// Whether a product is large enough.  A call costs about 10 us beside the product (tensor maps, packing of the weights, the launch
+// behind it), which the rate makes up for from about 0.8 GFLOP on: 200 K x 32 x 64 (0.8 GFLOP) 50 us against 49 on the FMA
+// pipes, 400 K x 48 x 32 61 : 73, 100 K x 100 x 100 50 : 91, weight gradients 64 x 64 x 200 K 61 : 93, 500 x 48 x 20 K 39 : 45.
+// Tiles are padded to 16 columns and, in a weight gradient, 128 rows: 200 K x 16 x 256 89 : 115, 32 x 64 x 500 K 112 : 197, and
+// nothing narrower.  The K-major form adds up one fp32 chain of K / 32 sums, which past 1024 terms of one sign is less accurate
+// than the two levels of the FMA kernel (1.2e-7 : 5e-8 at 2048).
+static bool split_pays(int ta, int64_t M, int64_t N, int64_t K) {
+    return 2.0 * M * N * K >= 8e8 && N >= 16 && (ta ? M >= 32 : K <= 1024);
+}
+
+// slots of raw tiles that fit beside `fixed` bytes (one block per SM: 227 KB, less the barriers)
+static int raw_slots(size_t fixed, int slot) {
+    const int n = (int)((227 * 1024 - 512 - fixed) / (size_t)slot);
+    return n < RAW_MAX ? n : RAW_MAX;
+}
+
+// fp32 products that pay on the tensor cores; MIXGCN_EUNSUPPORTED (nothing launched) for the others, which the FMA kernel takes.
+// *overflow_flag: the device word that the FMA kernel launched behind has to look at.
+mixgcn_status launch_gemm_split(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda,
+                                const float* B, int64_t ldb, float* C, int64_t ldc, const mixgcn_epilogue* epi, int64_t epi_row0,
+                                cudaStream_t s, bool* bits_done, const int32_t** overflow_flag) {
+    if (bits_done) *bits_done = false;
+    if (M <= 0 || N <= 0 || K <= 0 || (ta && tb) || M >= (1ll << 31) || N >= (1ll << 31) || K >= (1ll << 31)) return MIXGCN_EUNSUPPORTED;
+    if (!aligned16(A) || (lda & 3) || (ta && (!aligned16(B) || (ldb & 3) || epi))) return MIXGCN_EUNSUPPORTED;
+    if (!split_pays(ta, M, N, K)) return MIXGCN_EUNSUPPORTED;
+    auto ceil_div = [](int64_t a, int64_t b) { return (a + b - 1) / b; };
+    SplitParams p{};
+    p.M = M; p.N = N; p.K = K; p.C = C; p.ldc = ldc;
+    p.vec_c = aligned16(C) && (ldc & 3) == 0;
+    p.n_tiles = ceil_div(N, BN_MAX);
+    p.bn = (int)(p.n_tiles == 1 ? ceil_div(N, 16) * 16 : ceil_div(ceil_div(N, p.n_tiles), 32) * 32);
+    p.n_tiles = ceil_div(N, p.bn);
+    p.stages = p.bn > 64 ? 3 : 4;                      // as many as leave three raw slots and more
+    p.m_tiles = ceil_div(M, BM);
+    const int64_t tiles = p.m_tiles * p.n_tiles;
+    if (tiles > 0x7FFFFFFFll) return MIXGCN_EUNSUPPORTED;
+    p.epi = make_tc_epi(epi, epi_row0);
+    p.status = ctx->d_status;
+    p.wait_limit = ctx->debug_wait_limit > 0 ? (uint32_t)ctx->debug_wait_limit : WAIT_LIMIT_DEFAULT;
+    p.overflow = ctx->d_status + SPLIT_OVERFLOW_WORD;
+    *overflow_flag = p.overflow;
+    if (!ta) {
+        const int bn32 = (p.bn + 31) & ~31, kpad = (int)(ceil_div(K, BK) * BK);
+        const int rows = (int)p.n_tiles * bn32;
+        p.plane_rows = rows;
+        MIXGCN_TRY(ensure_workspace(ctx, (int64_t)PARTS * rows * kpad * 2));
+        uint16_t* planes = reinterpret_cast<uint16_t*>(ctx->workspace);
+        CUtensorMap map_a, map_b, map_c;
+        if (!encode_2d(&map_a, A, 4, K, M, lda, BK, BM, CU_TENSOR_MAP_SWIZZLE_NONE)) return MIXGCN_EUNSUPPORTED;
+        if (!encode_2d(&map_b, planes, 2, kpad, (int64_t)PARTS * rows, kpad, BK, bn32, CU_TENSOR_MAP_SWIZZLE_64B)) return MIXGCN_EUNSUPPORTED;
+        map_c = map_a;
+        const int tma_store = p.vec_c;
+        if (tma_store && !encode_2d(&map_c, C, 4, N, M, ldc, 32, 32)) return MIXGCN_EUNSUPPORTED;
+        const size_t fixed = (size_t)p.stages * PARTS * (KK_PART + bn32 * BK * 2) + (size_t)EPI_WARPS * 4096 + 1024;
+        p.raw_slots = raw_slots(fixed, RAW_BYTES);
+        const size_t smem = fixed + (size_t)p.raw_slots * RAW_BYTES;
+        MIXGCN_CUDA(cudaFuncSetAttribute(gemm_split_kk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        MIXGCN_CUDA(cudaMemsetAsync(p.overflow, 0, sizeof(int32_t), s));
+        {
+            LaunchScope scope(ctx, PH_GEMM, s);
+            pack_split_kernel<<<(unsigned)ceil_div((int64_t)rows * kpad, 256), 256, 0, s>>>(B, ldb, tb ? 0 : 1, (int)N, (int)K, rows, kpad, planes, p.overflow);
+        }
+        LaunchScope scope(ctx, PH_GEMM, s);
+        const unsigned grid = (unsigned)(tiles < ctx->sm_count ? tiles : ctx->sm_count);
+        gemm_split_kk_kernel<<<grid, THREADS, smem, s>>>(map_a, map_b, map_c, p, tma_store);
+        MIXGCN_CUDA(cudaGetLastError());
+        if (bits_done) *bits_done = p.epi.sign_bits != nullptr;
+        return MIXGCN_OK;
+    }
+    // one CTA per SM: as many splits as fill the machine once, no shorter than eight stages
+    // and none longer than 8,192 terms: the sums in registers are one fp32 chain
+    int64_t splits = ctx->sm_count / tiles;
+    if (splits < ceil_div(K, 8192)) splits = ceil_div(ceil_div(K, 8192) * tiles, ctx->sm_count) * ctx->sm_count / tiles;
+    const int64_t most = ceil_div(K, 8 * BK);
+    if (splits > most) splits = most;
+    if (splits < 1) splits = 1;
+    p.k_per_split = ceil_div(ceil_div(K, splits), BK) * BK;
+    splits = ceil_div(K, p.k_per_split);
+    p.raw = splits > 1;
+    if (splits > 1) {
+        MIXGCN_TRY(ensure_workspace(ctx, splits * M * N * (int64_t)sizeof(float)));
+        p.C = reinterpret_cast<float*>(ctx->workspace); p.ldc = N; p.vec_c = (N & 3) == 0;
+    }
+    const int bw = p.bn > 64 ? 128 : 64;
+    CUtensorMap map_a, map_b;
+    if (!encode_2d(&map_a, A, 4, M, K, lda, BM, BK, CU_TENSOR_MAP_SWIZZLE_NONE)) return MIXGCN_EUNSUPPORTED;
+    if (!encode_2d(&map_b, B, 4, N, K, ldb, bw, BK, CU_TENSOR_MAP_SWIZZLE_NONE)) return MIXGCN_EUNSUPPORTED;
+    const size_t fixed = (size_t)p.stages * PARTS * (BM + bw) / 64 * CHUNK + 1024;
+    p.raw_slots = raw_slots(fixed, RAW_BYTES);
+    const size_t smem = fixed + (size_t)p.raw_slots * RAW_BYTES;
+    MIXGCN_CUDA(cudaFuncSetAttribute(gemm_split_mm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    MIXGCN_CUDA(cudaMemsetAsync(p.overflow, 0, sizeof(int32_t), s));
+    {
+        LaunchScope scope(ctx, PH_GEMM, s);
+        gemm_split_mm_kernel<<<dim3((unsigned)tiles, 1, (unsigned)splits), THREADS, smem, s>>>(map_a, map_b, p);
+    }
+    MIXGCN_CUDA(cudaGetLastError());
+    if (splits > 1) MIXGCN_TRY(launch_splitk_reduce(ctx, M, N, (int)splits, p.C, C, ldc, nullptr, s));
+    return MIXGCN_OK;
+}
+
+}  // namespace mixgcn

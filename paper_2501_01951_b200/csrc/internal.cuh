@@ -69,10 +69,12 @@ struct ProfSpan {
 
 }  // namespace mixgcn
 
+constexpr int STATUS_WORDS = 32, SPLIT_OVERFLOW_WORD = 16;
+
 struct mixgcn_ctx {
     int device;
     int sm_count;
-    int32_t* d_status;        // device status word (int32[4])
+    int32_t* d_status;        // device status word (int32[4]); word SPLIT_OVERFLOW_WORD: see gemm_split.cu
     void* workspace;          // grow-on-demand scratch of the dense products, column sums and the loss
     int64_t workspace_bytes;
     void* workspace_rows;     // scratch of the row-sparse backward (row list, positions, compact operands)
@@ -303,7 +305,11 @@ mixgcn_status launch_gemm(mixgcn_ctx* ctx, int precision, int ta, int tb, int64_
                           float* colsum_b = nullptr);
 mixgcn_status launch_gemm_simt(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64_t N, int64_t K,
                                const float* A, int64_t lda, const float* B, int64_t ldb, float* C, int64_t ldc,
-                               const mixgcn_epilogue* epi, int64_t epi_row0, cudaStream_t s, bool* bits_done = nullptr);
+                               const mixgcn_epilogue* epi, int64_t epi_row0, cudaStream_t s, bool* bits_done = nullptr,
+                               const int32_t* only_if = nullptr);     // non-null: compute only if this device word is not zero
+mixgcn_status launch_gemm_split(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda,
+                                const float* B, int64_t ldb, float* C, int64_t ldc, const mixgcn_epilogue* epi, int64_t epi_row0,
+                                cudaStream_t s, bool* bits_done, const int32_t** overflow_flag);
 mixgcn_status launch_gemm_tc(mixgcn_ctx* ctx, int kind, int ta, int tb, int64_t M, int64_t N, int64_t K, const void* A,
                              int64_t lda, const void* B, int64_t ldb, float* C, int64_t ldc,
                              const mixgcn_epilogue* epi, int64_t epi_row0, cudaStream_t s, uint16_t* C_lp, int64_t ldc_lp,

@@ -1,0 +1,100 @@
+"""Large fp32 products on the tensor cores, operands in three bf16 parts: either side of the tile, stage, accumulator and split
+boundaries, with the whole epilogue, against fp64 and against the FMA kernel (which takes operands that are not aligned)."""
+import pytest
+import torch
+
+from helpers import TOL_FP32
+from paper_2501_01951_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mg():
+    from paper_2501_01951_b200 import build
+    build.build()
+    from paper_2501_01951_b200 import binding
+    return binding
+
+
+@pytest.fixture(scope="module")
+def ctx(mg):
+    c = mg.ctx_create(0)
+    yield c
+    assert mg.ctx_poll_status(c, raise_on_error=False) == 0
+    c.close()
+
+
+def device(t, ld):
+    out = torch.full((t.shape[0], ld), float("nan"), device="cuda")      # what lies beyond the matrix is not read
+    out[:, : t.shape[1]] = t
+    return out
+
+
+def up(x, aligned=True):
+    return (x + 3) // 4 * 4 if aligned else x + 1 + (x % 2 == 1)
+
+
+def product(mg, ctx, A, B, ta, tb, aligned=True, **epi):
+    M, K, N = (A.shape[1], A.shape[0], 0) if ta else (*A.shape, 0)
+    N = B.shape[0] if tb else B.shape[1]
+    C = torch.full((M, up(N)), 3.0, device="cuda")
+    mg.gemm(ctx, mg.PREC_FP32, ta, tb, M, N, K, device(A, up(A.shape[1], aligned)), device(B, up(B.shape[1], aligned)), C,
+            **({"epi": mg.make_epilogue(**epi)} if epi else {}))
+    assert torch.all(C[:, N:] == 3.0)
+    return C[:, :N]
+
+
+def error(got, want):
+    return ((got.double() - want).norm() / want.norm()).item()
+
+
+def operands(M, N, K, ta, tb, positive=False):
+    lo = 0 if positive else -1
+    return synth.uniform_tensor((K, M) if ta else (M, K), 31, lo, 1).cuda(), synth.uniform_tensor((N, K) if tb else (K, N), 32, lo, 1).cuda()
+
+
+@pytest.mark.parametrize("M,N,K,ta", [
+    (200001, 16, 127, False), (30000, 17, 1000, False), (100000, 129, 32, False), (500, 1000, 1023, False), (80001, 161, 33, False),
+    (13000, 64, 512, False), (18943, 128, 168, False), (18945, 65, 330, False), (1300000, 40, 8, False), (1000, 1003, 1024, False),
+    (32, 16, 800001, True), (33, 63, 200003, True), (129, 65, 50031, True), (128, 128, 24577, True), (501, 303, 2700, True), (1003, 1001, 401, True)])
+@pytest.mark.parametrize("positive", [False, True])
+def test_split_products(mg, ctx, M, N, K, ta, positive):
+    for tb in ((False,) if ta else (False, True)):
+        A, B = operands(M, N, K, ta, tb, positive)
+        want = (A.T if ta else A).double() @ (B.T if tb else B).double()
+        got, fma = product(mg, ctx, A, B, ta, tb), product(mg, ctx, A, B, ta, tb, aligned=False)
+        assert error(got, want) <= TOL_FP32
+        assert error(got, want) <= max(1.4 * error(fma, want), 7e-8)     # 6e-8 = one rounding to fp32
+
+
+@pytest.mark.parametrize("M,N,K", [(60001, 40, 200), (30001, 161, 97), (9000, 300, 256)])
+def test_split_epilogue(mg, ctx, M, N, K):
+    A, B = operands(M, N, K, False, False)
+    bias, drop = synth.uniform_tensor((N,), 33, -1, 1).cuda(), synth.bernoulli_mask(M * N, 0.5, 34).cuda()
+    gate = synth.uniform_tensor((M, N), 35, -1, 1).cuda()
+    words = (N + 31) // 32
+    bits = torch.full((M, words + 1), -1, dtype=torch.int32, device="cuda")
+    got = product(mg, ctx, A, B, False, False, bias=bias, relu=True, drop_mask=drop, keep_scale=2.0, gate=device(gate, up(N)), gate_scale=0.5, sign_bits=bits)
+    want = torch.relu(A.double() @ B.double() + bias.double()) * drop.reshape(M, N) * (gate > 0)
+    assert error(got, want) <= TOL_FP32
+    j = torch.arange(N, device="cuda")
+    assert torch.equal((bits[:, j // 32] >> (j % 32)) & 1, (got > 0).int()) and torch.all(bits[:, words] == -1)
+
+
+@pytest.mark.parametrize("ta", [False, True])
+@pytest.mark.parametrize("where", ["A", "B"])
+@pytest.mark.parametrize("value", [float("inf"), float("nan"), -3.4e38])
+def test_operands_that_cannot_be_split(mg, ctx, ta, where, value):
+    M, N, K = (200, 100, 25000) if ta else (25000, 100, 200)
+    A, B = operands(M, N, K, ta, False)
+    (A if where == "A" else B)[17, 5] = value
+    bits = torch.zeros(M, (N + 31) // 32, dtype=torch.int32, device="cuda")
+    epi = {} if ta else {"sign_bits": bits}
+    got, bits_got = product(mg, ctx, A, B, ta, False, **epi), bits.clone()
+    want = product(mg, ctx, A, B, ta, False, aligned=False, **epi)
+    assert torch.equal(bits_got, bits) and torch.equal(got.isnan(), want.isnan()) and torch.equal(got.isinf(), want.isinf())
+    ok = want.isfinite()
+    assert error(got[ok] / 2.0**64, want[ok].double() / 2.0**64) <= TOL_FP32
+    clean = operands(M, N, K, ta, False)                                 # the note of one product does not reach the next
+    assert error(product(mg, ctx, *clean, ta, False), (clean[0].T if ta else clean[0]).double() @ clean[1].double()) <= TOL_FP32

@@ -191,7 +191,7 @@ mixgcn_status launch_gemm(mixgcn_ctx* ctx, int precision, int ta, int tb, int64_
         // cannot be split (it returns at once otherwise); all others: the FMA kernel
         const int32_t* overflow = nullptr;
         bool split_bits = false, fma_bits = false;
-        st = launch_gemm_split(ctx, ta, tb, M, N, K, A, lda, B, ldb, C, ldc, epi, epi_row0, s, &split_bits, &overflow);
+        st = launch_gemm_split(ctx, ta, tb, M, N, K, A, lda, B, ldb, C, ldc, epi, epi_row0, s, &split_bits, &overflow, colsum_b, &colsum_done);
         if (st != MIXGCN_OK && st != MIXGCN_EUNSUPPORTED) return st;
         const bool split = st == MIXGCN_OK;
         st = launch_gemm_simt(ctx, ta, tb, M, N, K, A, lda, B, ldb, C, ldc, epi, epi_row0, s, &fma_bits, split ? overflow : nullptr);

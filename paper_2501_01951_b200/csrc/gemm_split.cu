@@ -58,6 +58,7 @@ struct SplitParams {
     int64_t k_per_split;          // MN-major: a multiple of BK
     float* C; int64_t ldc; int vec_c;   // MN-major: partial tiles [splits][M][N] or C itself
     int raw;
+    double* colsum_part;          // MN-major, nullable: [splits][m_tiles][N] column sums of B over the k-rows a CTA added up
     TcEpi epi;
     int32_t* status;
     uint32_t wait_limit;
@@ -437,6 +438,14 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
         stage.next(p.stages, group);
         uint32_t top = 0;
         float4 v[RAW_ITS];
+        // Column sums of B: the rows of tiles take the stages of a group in turn, each thread its own columns of the raw tile.
+        const int m_tile = (int)(tile / p.n_tiles);
+        int turn = (int)p.m_tiles - m_tile;                            // 0 after m_tile stages
+        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+        auto add_columns = [&](const auto& w, int its) {
+#pragma unroll
+            for (int it = 0; it < its; ++it) { add2(sum.x, sum.y, w[it].x, w[it].y); add2(sum.z, sum.w, w[it].z, w[it].w); }
+        };
         for (int ks = group; ks < nk; ks += GROUPS) {
             if (!warp_wait(&bars.raw_full[raw.i], raw.use, bars, p)) break;
             take_raw(v, raws + (size_t)raw.i * RAW_BYTES, t);
@@ -449,10 +458,13 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
             for (int it = 0; it < RAW_ITS; ++it) split4(v[it], dst + (at_a ^ (it & 1) * 64) + it * 4 * 128, MM_PART, top);
             if (!warp_wait(&bars.raw_full[raw.i], raw.use, bars, p)) break;
             dst += PARTS * MM_PART;
+            if (turn == (int)p.m_tiles) turn = 0;
+            const bool sums = p.colsum_part && turn++ == 0;
             if (bw == 128) {
                 take_raw(v, raws + (size_t)raw.i * RAW_BYTES, t);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&bars.raw_empty[raw.i]);
+                if (sums) add_columns(v, RAW_ITS);
 #pragma unroll
                 for (int it = 0; it < RAW_ITS; ++it) split4(v[it], dst + (at_a ^ (it & 1) * 64) + it * 4 * 128, b_part, top);
             } else {
@@ -460,6 +472,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
                 take_raw(w, raws + (size_t)raw.i * RAW_BYTES, t);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&bars.raw_empty[raw.i]);
+                if (sums) add_columns(w, RAW_ITS / 2);
 #pragma unroll
                 for (int it = 0; it < RAW_ITS / 2; ++it) split4(w[it], dst + at_b + it * 8 * 128, b_part, top);
             }
@@ -469,6 +482,19 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
             raw.next(p.raw_slots);
             raw.next(p.raw_slots, 2 * (GROUPS - 1));
             stage.next(p.stages, GROUPS);
+        }
+        if (p.colsum_part) {
+            // all raw tiles are used up (by both groups): their memory takes the threads' sums
+            const int all = threadIdx.x - EPI_WARPS * 32;
+            float* sums = reinterpret_cast<float*>(raws);
+            asm volatile("bar.sync 1, %0;" ::"n"(CONV_WARPS * 32) : "memory");
+            reinterpret_cast<float4*>(sums)[all] = sum;
+            asm volatile("bar.sync 1, %0;" ::"n"(CONV_WARPS * 32) : "memory");
+            if (all < p.bn && n0 + all < p.N) {
+                double s = 0.0;
+                for (int i = all; i < CONV_WARPS * 32 * 4; i += bw) s += (double)sums[i];
+                p.colsum_part[((int64_t)blockIdx.z * p.m_tiles + m_tile) * p.N + n0 + all] = s;
+            }
         }
         if (has_inf(top)) *p.overflow = 1;
     } else if (warp == TMA_WARP) {
@@ -534,8 +560,9 @@ static int raw_slots(size_t fixed, int slot) {
 // *overflow_flag: the device word that the FMA kernel launched behind has to look at.
 mixgcn_status launch_gemm_split(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda,
                                 const float* B, int64_t ldb, float* C, int64_t ldc, const mixgcn_epilogue* epi, int64_t epi_row0,
-                                cudaStream_t s, bool* bits_done, const int32_t** overflow_flag) {
+                                cudaStream_t s, bool* bits_done, const int32_t** overflow_flag, float* colsum_b, bool* colsum_done) {
     if (bits_done) *bits_done = false;
+    if (colsum_done) *colsum_done = false;
     if (M <= 0 || N <= 0 || K <= 0 || (ta && tb) || M >= (1ll << 31) || N >= (1ll << 31) || K >= (1ll << 31)) return MIXGCN_EUNSUPPORTED;
     if (!aligned16(A) || (lda & 3) || (ta && (!aligned16(B) || (ldb & 3) || epi))) return MIXGCN_EUNSUPPORTED;
     if (!split_pays(ta, M, N, K)) return MIXGCN_EUNSUPPORTED;
@@ -593,8 +620,11 @@ mixgcn_status launch_gemm_split(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int6
     p.k_per_split = ceil_div(ceil_div(K, splits), BK) * BK;
     splits = ceil_div(K, p.k_per_split);
     p.raw = splits > 1;
+    const int64_t part_bytes = splits > 1 ? (splits * M * N * (int64_t)sizeof(float) + 7) / 8 * 8 : 0;
+    const int64_t sums_bytes = colsum_b ? splits * p.m_tiles * N * (int64_t)sizeof(double) : 0;
+    if (part_bytes + sums_bytes) MIXGCN_TRY(ensure_workspace(ctx, part_bytes + sums_bytes));
+    if (colsum_b) p.colsum_part = reinterpret_cast<double*>(reinterpret_cast<char*>(ctx->workspace) + part_bytes);
     if (splits > 1) {
-        MIXGCN_TRY(ensure_workspace(ctx, splits * M * N * (int64_t)sizeof(float)));
         p.C = reinterpret_cast<float*>(ctx->workspace); p.ldc = N; p.vec_c = (N & 3) == 0;
     }
     const int bw = p.bn > 64 ? 128 : 64;
@@ -611,6 +641,10 @@ mixgcn_status launch_gemm_split(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int6
         gemm_split_mm_kernel<<<dim3((unsigned)tiles, 1, (unsigned)splits), THREADS, smem, s>>>(map_a, map_b, p);
     }
     MIXGCN_CUDA(cudaGetLastError());
+    if (colsum_b) {
+        MIXGCN_TRY(launch_colsum_splits(ctx, N, (int)(splits * p.m_tiles), p.colsum_part, colsum_b, s));
+        if (colsum_done) *colsum_done = true;
+    }
     if (splits > 1) MIXGCN_TRY(launch_splitk_reduce(ctx, M, N, (int)splits, p.C, C, ldc, nullptr, s));
     return MIXGCN_OK;
 }

@@ -1004,6 +1004,13 @@ EncodeTiledFn get_encode() {
 }  // namespace
 
 namespace mixgcn {
+mixgcn_status launch_colsum_splits(mixgcn_ctx* ctx, int64_t N, int splits, const double* part, float* out, cudaStream_t s) {
+    LaunchScope scope(ctx, PH_GEMM, s);
+    colsum_splits_kernel<<<(unsigned)((N + 31) / 32), 256, 0, s>>>(N, splits, part, out);
+    MIXGCN_CUDA(cudaGetLastError());
+    return MIXGCN_OK;
+}
+
 // 2-D tensor of fp32 (eb = 4) or bf16 (eb = 2): `inner` contiguous elements per row, `outer` rows of `ld`
 // elements; 128-byte swizzle unless stated.
 bool tc::encode_2d(CUtensorMap* map, const void* base, int eb, int64_t inner, int64_t outer, int64_t ld, int box_inner,
@@ -1263,9 +1270,7 @@ mixgcn_status launch_kind(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64_t N,
     MIXGCN_CUDA(cudaGetLastError());
     if (splits > 1) MIXGCN_TRY(launch_splitk_reduce(ctx, M, N, splits, p.C, C, ldc, epi, s));
     if (fuse_colsum) {
-        LaunchScope scope(ctx, PH_GEMM, s);
-        colsum_splits_kernel<<<(unsigned)((N + 31) / 32), 256, 0, s>>>(N, (int)(splits * p.m_tiles), p.colsum_part, colsum_b);
-        MIXGCN_CUDA(cudaGetLastError());
+        MIXGCN_TRY(launch_colsum_splits(ctx, N, (int)(splits * p.m_tiles), p.colsum_part, colsum_b, s));
         if (colsum_done) *colsum_done = true;
     }
     return MIXGCN_OK;

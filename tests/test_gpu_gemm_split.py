@@ -98,3 +98,12 @@ def test_operands_that_cannot_be_split(mg, ctx, ta, where, value):
     assert error(got[ok] / 2.0**64, want[ok].double() / 2.0**64) <= TOL_FP32
     clean = operands(M, N, K, ta, False)                                 # the note of one product does not reach the next
     assert error(product(mg, ctx, *clean, ta, False), (clean[0].T if ta else clean[0]).double() @ clean[1].double()) <= TOL_FP32
+
+
+@pytest.mark.parametrize("M,N,K", [(33, 63, 200003), (300, 17, 80001), (128, 65, 50000), (385, 161, 8193)])
+def test_column_sums(mg, ctx, M, N, K):
+    A, B = operands(M, N, K, True, False)
+    C, sums = torch.zeros(M, up(N), device="cuda"), torch.full((N + 1,), 5.0, device="cuda")
+    mg.weight_grad(ctx, mg.PREC_FP32, M, N, K, device(A, up(M)), device(B, up(N)), C, sums)
+    assert error(C[:, :N], A.double().T @ B.double()) <= TOL_FP32
+    assert (sums[:N].double() - B.double().sum(0)).abs().max() <= 1e-6 * B.double().abs().sum(0).max() and sums[N] == 5.0

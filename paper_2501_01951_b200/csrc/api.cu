@@ -264,6 +264,8 @@ extern "C" mixgcn_status mixgcn_ctx_destroy(mixgcn_ctx* ctx) {
     for (int i = 0; i < 64; ++i) if (ctx->chunk_ev[i]) cudaEventDestroy(ctx->chunk_ev[i]);
     for (int i = 0; i < 2; ++i) { if (ctx->join_ev[i]) cudaEventDestroy(ctx->join_ev[i]); if (ctx->side_stream[i]) cudaStreamDestroy(ctx->side_stream[i]); }
     if (ctx->fork_ev) cudaEventDestroy(ctx->fork_ev);
+    for (int i = 0; i < 3; ++i) if (ctx->copy_ev[i]) cudaEventDestroy(ctx->copy_ev[i]);
+    if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
     if (ctx->recording) { mixgcn_recording* none = nullptr; mixgcn_record_end(ctx, &none); mixgcn_recording_destroy(none); }
     if (ctx->record_stream) cudaStreamDestroy(ctx->record_stream);
     free_step_cache(ctx);

@@ -1,6 +1,10 @@
 // One whole training iteration (the loop body of Algorithm 2) with host inputs and outputs:
 // host -> device copies, all layers forward, loss, backward, Adam, device -> host copies.
 // Device buffers come from an arena the context keeps between calls.
+//
+// Bound by the copy of the features (500 K x 128: 256 MB, 4.6 ms of 6.0 at 55 GB/s).  It starts before anything else is looked
+// at, on a stream of its own; the mask is counted and compared, and every launch up to the loss prepared, while it runs.
+// What later layers need follows behind it, and the predictions leave during the backward pass.
 #include <new>
 #include <vector>
 
@@ -37,6 +41,22 @@ __global__ void mask_differs_kernel(int64_t n, const uint8_t* __restrict__ a, co
     if (__any_sync(0xFFFFFFFFu, d) && (threadIdx.x & 31) == 0) *differs = 1;
 }
 
+// Rows of d words back to back -> rows of ld words (a multiple of 4, zeros behind the d): a warp per row.
+__global__ void __launch_bounds__(256) spread_rows_kernel(int64_t n, int64_t d, const float* __restrict__ src, float* __restrict__ dst, int64_t ld) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); r < n; r += (int64_t)gridDim.x * 8) {
+        const float* from = src + r * d;
+        for (int64_t c = lane * 4; c < ld; c += 128) {
+            float4 v;
+            v.x = __ldg(from + c);
+            v.y = c + 1 < d ? __ldg(from + c + 1) : 0.0f;
+            v.z = c + 2 < d ? __ldg(from + c + 2) : 0.0f;
+            v.w = c + 3 < d ? __ldg(from + c + 3) : 0.0f;
+            *reinterpret_cast<float4*>(dst + r * ld + c) = v;
+        }
+    }
+}
+
 void drop_plans(HostStepCache* c) {
     for (int i = 0; i < 2; ++i) { if (c->plan[i]) mixgcn_rowplan_destroy(c->plan[i]); c->plan[i] = nullptr; }
     c->graph_uid = 0; c->levels = 0;
@@ -56,6 +76,7 @@ struct Carver {
 struct StepLayout {
     std::vector<float*> X, saved, G, W, b, dW, db, mW, vW, mb, vb;
     int32_t* labels; uint8_t* mask; float* loss; int32_t* pred;
+    float* packed_x;                 // features as they come from the host, where their rows are not a multiple of 4 words
     std::vector<uint8_t*> rowmask;   // [L] byte masks the row-sparse backward fills (layer l's input-gradient rows)
     std::vector<mixgcn_layer_desc> desc;
     int64_t bytes;
@@ -89,6 +110,7 @@ mixgcn_status lay_out(char* base, int64_t n, int L, const int32_t* dims, int pre
     lo.G[L] = lo.X[L];  // the logits' gradient overwrites the logits
     for (int l = L - 1, i = 0; l >= 1; --l, ++i) lo.G[l] = pool[i % 2];
     lo.labels = c.take<int32_t>(n); lo.mask = c.take<uint8_t>(n); lo.loss = c.take<float>(4); lo.pred = c.take<int32_t>(n);
+    lo.packed_x = ld[0] != dims[0] ? c.take<float>(n * dims[0]) : nullptr;
     lo.rowmask.resize(L);
     for (int l = 0; l < L; ++l) lo.rowmask[l] = c.take<uint8_t>(n);
     // sign bitmaps of the hidden activations a dense product writes (agg-first layer below): the backward reads
@@ -160,13 +182,59 @@ extern "C" mixgcn_status mixgcn_train_step_host(mixgcn_ctx* ctx, const mixgcn_gr
     cudaStream_t s = ctx->side_stream[0];
     const cudaMemcpyKind H2D = cudaMemcpyHostToDevice, D2H = cudaMemcpyDeviceToHost;
 
+    if (!ctx->copy_stream) {
+        MIXGCN_CUDA(cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking));
+        for (int i = 0; i < 3; ++i) MIXGCN_CUDA(cudaEventCreateWithFlags(&ctx->copy_ev[i], cudaEventDisableTiming));
+    }
+    cudaStream_t cs = ctx->copy_stream;
+    struct Landing {                        // an error leaves no copy from or to the caller's memory in flight
+        cudaStream_t a, b;
+        bool armed = true;
+        ~Landing() { if (armed) { cudaStreamSynchronize(a); cudaStreamSynchronize(b); } }
+    } landing{cs, s};
+    auto copy_layer = [&](int l, bool moments, cudaMemcpyKind kind, cudaStream_t st) -> cudaError_t {
+        const size_t wb = (size_t)dims[l] * dims[l + 1] * sizeof(float), bb = (size_t)dims[l + 1] * sizeof(float);
+        const std::vector<float*>* dev[6] = {&lo.W, &lo.b, &lo.mW, &lo.vW, &lo.mb, &lo.vb};
+        float* const* host[6] = {W, b, mW, vW, mb, vb};
+        const bool weight[6] = {true, false, true, true, false, false};
+        for (int i = moments ? 2 : 0; i < (moments ? 6 : 2); ++i) {
+            float *d = (*dev[i])[l], *h = host[i][l];
+            const cudaError_t e = kind == H2D ? cudaMemcpyAsync(d, h, weight[i] ? wb : bb, H2D, st) : cudaMemcpyAsync(h, d, weight[i] ? wb : bb, D2H, st);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    };
+
+    // inputs: mask and first layer, then the features, then what the later layers and the loss read
+    MIXGCN_CUDA(cudaMemcpyAsync(lo.mask, train_mask, n * sizeof(uint8_t), H2D, s));
+    MIXGCN_CUDA(copy_layer(0, false, H2D, s));
+    const int64_t d0 = dims[0], ld0 = round4(d0);
+    // Features whose rows have to be padded come in one piece and are spread on the device: a pitched copy moves row by row
+    // (100 K x 301: 12 ms against 2.2).
+    auto copy_features = [&](const float* src, cudaStream_t st) -> cudaError_t {
+        const cudaError_t e = cudaMemcpyAsync(lo.packed_x ? lo.packed_x : lo.X[0], src, (size_t)(n * d0) * sizeof(float), H2D, st);
+        if (e != cudaSuccess || !lo.packed_x) return e;
+        const int64_t blocks = (n + 7) / 8, most = 16 * (int64_t)ctx->sm_count;
+        spread_rows_kernel<<<(unsigned)(blocks < most ? blocks : most), 256, 0, st>>>(n, d0, lo.packed_x, lo.X[0], ld0);
+        return cudaGetLastError();
+    };
+    if (pf && pf->in_flight) MIXGCN_CUDA(cudaStreamWaitEvent(cs, pf->done, 0));     // started by the previous call, or stale and still writing X[0]
+    if (!(pf && pf->in_flight == X && pf->dst == lo.X[0] && pf->n == n && pf->d0 == d0)) MIXGCN_CUDA(copy_features(X, cs));
+    if (pf) pf->in_flight = nullptr;
+    MIXGCN_CUDA(cudaEventRecord(ctx->copy_ev[0], cs));
+    MIXGCN_CUDA(cudaMemcpyAsync(lo.labels, labels, n * sizeof(int32_t), H2D, cs));
+    for (int l = 0; l < L; ++l) {
+        if (l > 0) MIXGCN_CUDA(copy_layer(l, false, H2D, cs));
+        MIXGCN_CUDA(copy_layer(l, true, H2D, cs));
+    }
+    MIXGCN_CUDA(cudaEventRecord(ctx->copy_ev[1], cs));
+
     // Row sparsity of the backward pass: the loss gradient is non-zero on train rows only, and one
     // aggregation later on their neighbours only (same rule as the device-buffer trainer).  The row
     // plans are kept between calls and reused while the graph and the mask are the same.
     int64_t n_train = 0;
     for (int64_t i = 0; i < n; ++i) n_train += train_mask[i] ? 1 : 0;
     bool rows_only = false;
-    MIXGCN_CUDA(cudaMemcpyAsync(lo.mask, train_mask, n * sizeof(uint8_t), H2D, s));
     {
         const double frac = (double)n_train / (double)n, mean_entries = (double)g->nnz / (double)n;
         int levels = frac >= 0.25 ? 0 : (frac * mean_entries < 0.5 ? 2 : 1);
@@ -217,30 +285,6 @@ extern "C" mixgcn_status mixgcn_train_step_host(mixgcn_ctx* ctx, const mixgcn_gr
         if (rows_only) lo.desc[L - 1].flags |= MIXGCN_LAYER_OUT_ROWS_ONLY;
     }
 
-    // inputs
-    const int64_t d0 = dims[0], ld0 = round4(d0);
-    auto copy_features = [&](const float* src, cudaStream_t st) -> cudaError_t {
-        if (ld0 == d0) return cudaMemcpyAsync(lo.X[0], src, (size_t)(n * d0) * sizeof(float), H2D, st);
-        return cudaMemcpy2DAsync(lo.X[0], ld0 * sizeof(float), src, d0 * sizeof(float), d0 * sizeof(float), (size_t)n, H2D, st);
-    };
-    if (pf && pf->in_flight == X && pf->dst == lo.X[0] && pf->n == n && pf->d0 == d0) {
-        // the previous call already started this copy: wait for it instead of copying again
-        MIXGCN_CUDA(cudaStreamWaitEvent(s, pf->done, 0));
-    } else {
-        if (pf && pf->in_flight) MIXGCN_CUDA(cudaStreamWaitEvent(s, pf->done, 0));   // a stale prefetch still writes X[0]: let it finish first
-        MIXGCN_CUDA(copy_features(X, s));
-    }
-    if (pf) pf->in_flight = nullptr;
-    MIXGCN_CUDA(cudaMemcpyAsync(lo.labels, labels, n * sizeof(int32_t), H2D, s));
-    for (int l = 0; l < L; ++l) {
-        const size_t wb = (size_t)dims[l] * dims[l + 1] * sizeof(float), bb = (size_t)dims[l + 1] * sizeof(float);
-        MIXGCN_CUDA(cudaMemcpyAsync(lo.W[l], W[l], wb, H2D, s));
-        MIXGCN_CUDA(cudaMemcpyAsync(lo.mW[l], mW[l], wb, H2D, s));
-        MIXGCN_CUDA(cudaMemcpyAsync(lo.vW[l], vW[l], wb, H2D, s));
-        MIXGCN_CUDA(cudaMemcpyAsync(lo.b[l], b[l], bb, H2D, s));
-        MIXGCN_CUDA(cudaMemcpyAsync(lo.mb[l], mb[l], bb, H2D, s));
-        MIXGCN_CUDA(cudaMemcpyAsync(lo.vb[l], vb[l], bb, H2D, s));
-    }
     // forward, loss, backward, update
     auto after_first_layer = [&]() -> mixgcn_status {
         if (pf && pf->announced && lo.desc[0].order == MIXGCN_ORDER_AGG_FIRST) {
@@ -259,10 +303,13 @@ extern "C" mixgcn_status mixgcn_train_step_host(mixgcn_ctx* ctx, const mixgcn_gr
     // With predictions wanted for every node the last layer and the loss are one call (the loss is taken where
     // the logits are produced, wherever the kernels allow; rows the backward never reads are left alone).
     const bool one_call = pred != nullptr && !rows_only;
+    MIXGCN_CUDA(cudaStreamWaitEvent(s, ctx->copy_ev[0], 0));
     for (int l = 0; l < (one_call ? L - 1 : L); ++l) {
+        if (l == 1) MIXGCN_CUDA(cudaStreamWaitEvent(s, ctx->copy_ev[1], 0));
         MIXGCN_TRY(mixgcn_layer_fwd(ctx, g, &lo.desc[l], lo.X[l], lo.W[l], lo.b[l], nullptr, lo.saved[l], lo.X[l + 1], s));
         if (l == 0) MIXGCN_TRY(after_first_layer());
     }
+    MIXGCN_CUDA(cudaStreamWaitEvent(s, ctx->copy_ev[1], 0));
     {
         const int keep = ctx->loss_train_rows_only;
         mixgcn_status st;
@@ -280,6 +327,10 @@ extern "C" mixgcn_status mixgcn_train_step_host(mixgcn_ctx* ctx, const mixgcn_gr
         if (one_call && L == 1) MIXGCN_TRY(after_first_layer());
     }
     if (pf) pf->announced = nullptr;
+    MIXGCN_CUDA(cudaEventRecord(ctx->copy_ev[2], s));
+    MIXGCN_CUDA(cudaStreamWaitEvent(cs, ctx->copy_ev[2], 0));
+    MIXGCN_CUDA(cudaMemcpyAsync(loss, lo.loss, sizeof(float), D2H, cs));
+    if (pred) MIXGCN_CUDA(cudaMemcpyAsync(pred, lo.pred, n * sizeof(int32_t), D2H, cs));
     for (int l = L - 1; l >= 0; --l) {
         MIXGCN_TRY(mixgcn_layer_bwd(ctx, g, &lo.desc[l], lo.X[l], lo.saved[l], lo.X[l + 1], nullptr, lo.W[l], lo.G[l + 1],
                                     l > 0 ? lo.G[l] : nullptr, lo.dW[l], lo.db[l], s));
@@ -288,19 +339,10 @@ extern "C" mixgcn_status mixgcn_train_step_host(mixgcn_ctx* ctx, const mixgcn_gr
     for (int l = 0; l < L; ++l) { P.push_back(lo.W[l]); Gr.push_back(lo.dW[l]); M1.push_back(lo.mW[l]); M2.push_back(lo.vW[l]); numel.push_back((int64_t)dims[l] * dims[l + 1]); }
     for (int l = 0; l < L; ++l) { P.push_back(lo.b[l]); Gr.push_back(lo.db[l]); M1.push_back(lo.mb[l]); M2.push_back(lo.vb[l]); numel.push_back(dims[l + 1]); }
     MIXGCN_TRY(mixgcn_adam_step(ctx, 2 * L, P.data(), Gr.data(), M1.data(), M2.data(), numel.data(), t, lr, beta1, beta2, eps, s));
-    // results
-    MIXGCN_CUDA(cudaMemcpyAsync(loss, lo.loss, sizeof(float), D2H, s));
-    if (pred) MIXGCN_CUDA(cudaMemcpyAsync(pred, lo.pred, n * sizeof(int32_t), D2H, s));
-    for (int l = 0; l < L; ++l) {
-        const size_t wb = (size_t)dims[l] * dims[l + 1] * sizeof(float), bb = (size_t)dims[l + 1] * sizeof(float);
-        MIXGCN_CUDA(cudaMemcpyAsync(W[l], lo.W[l], wb, D2H, s));
-        MIXGCN_CUDA(cudaMemcpyAsync(mW[l], lo.mW[l], wb, D2H, s));
-        MIXGCN_CUDA(cudaMemcpyAsync(vW[l], lo.vW[l], wb, D2H, s));
-        MIXGCN_CUDA(cudaMemcpyAsync(b[l], lo.b[l], bb, D2H, s));
-        MIXGCN_CUDA(cudaMemcpyAsync(mb[l], lo.mb[l], bb, D2H, s));
-        MIXGCN_CUDA(cudaMemcpyAsync(vb[l], lo.vb[l], bb, D2H, s));
-    }
+    for (int l = 0; l < L; ++l) { MIXGCN_CUDA(copy_layer(l, false, D2H, s)); MIXGCN_CUDA(copy_layer(l, true, D2H, s)); }
+    MIXGCN_CUDA(cudaStreamSynchronize(cs));
     MIXGCN_CUDA(cudaStreamSynchronize(s));
+    landing.armed = false;
     return MIXGCN_OK;
 }
 

@@ -83,6 +83,8 @@ struct mixgcn_ctx {
     int64_t workspace_spmm_bytes;  // that an aggregation and a dense product may overlap on two streams
     cudaStream_t side_stream[2];
     cudaEvent_t fork_ev, join_ev[2];
+    cudaStream_t copy_stream; // host <-> device copies of train_step_host beside its kernels (created by the first call)
+    cudaEvent_t copy_ev[3];
     cudaEvent_t chunk_ev[64];
     void* workspace_loss;     // scratch of the loss taken inside a layer's last kernel (count, partial sums, per-row terms): its own
     int64_t workspace_loss_bytes;   // block, because the product that takes the loss packs its weights into `workspace`

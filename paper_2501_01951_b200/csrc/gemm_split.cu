@@ -43,7 +43,8 @@ namespace {
 constexpr int BM = 128, BN_MAX = 128, BK = 32, PARTS = 3;
 constexpr int EPI_WARPS = 8, CONV_WARPS = 8, TMA_WARP = EPI_WARPS + CONV_WARPS, MMA_WARP = TMA_WARP + 1, THREADS = (MMA_WARP + 1) * 32;
 constexpr int GROUPS = 2, GROUP_WARPS = CONV_WARPS / GROUPS, GROUP_THREADS = GROUP_WARPS * 32;   // groups of conversion warps, on alternate stages
-constexpr int STAGES_MAX = 4, RAW_MAX = 8;      // most stages of part tiles and slots of raw fp32 tiles
+constexpr int STAGES_MAX = 4, RAW_MAX = 8;      // most stages of part tiles and slots of raw fp32 tiles (a multiple of 2 * GROUPS)
+static_assert(RAW_MAX % (2 * GROUPS) == 0);
 constexpr int HI_STAGES = 32 / BK, LO_STAGES = 1024 / BK;           // stages per accumulator of the large and of the small products
 constexpr uint32_t TMEM_COLS = 512, LO_COL = 256, BUF_COLS = 128;   // two accumulators for the large products, two for the small ones
 constexpr int RAW_BYTES = BM * BK * 4, KK_PART = BM * BK * 2;       // a raw tile; K-major part tiles: 64-byte rows and swizzle
@@ -69,6 +70,17 @@ struct Ring {                     // position in a ring of slots and the parity 
     int i = 0;
     uint32_t use = 0;
     __device__ __forceinline__ void next(int n, int by = 1) { if ((i += by) >= n) { i -= n; use ^= 1; } }      // by <= n
+};
+
+// Position among the raw tiles.  They go through `raw_slots` slots, but their barriers go by eights: so all uses of one barrier are
+// the same group's, which has seen the one before.  (By slots, three or five of them, a group could wait on a barrier whose last
+// use, the other group's, is still in flight, and take the use before that for its own: loads land out of order.)
+struct RawRing {
+    uint32_t unit = 0;
+    int slot = 0;
+    __device__ __forceinline__ void next(int n, int by = 1) { unit += by; if ((slot += by) >= n) slot -= n; }       // by <= n
+    __device__ __forceinline__ uint32_t bar() const { return unit % RAW_MAX; }
+    __device__ __forceinline__ uint32_t use() const { return unit / RAW_MAX & 1; }
 };
 
 __device__ __forceinline__ void add2(float& x, float& y, float a, float b) {
@@ -150,6 +162,12 @@ __device__ __forceinline__ bool thread_wait(uint64_t* bar, uint32_t parity, Shar
     *flag = 1;
     atomicMax(p.status, DEV_WAIT_EXPIRED);
     return false;
+}
+// The slot of the next raw tile is free: the tile raw_slots back has been taken.
+__device__ __forceinline__ bool raw_free(const RawRing& raw, Shared& b, const SplitParams& p) {
+    if (raw.unit < (uint32_t)p.raw_slots) return true;
+    const uint32_t last = raw.unit - p.raw_slots;
+    return thread_wait(&b.raw_empty[last % RAW_MAX], last / RAW_MAX & 1, b, p);
 }
 // One wait of a whole warp.
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, Shared& b, const SplitParams& p) {
@@ -322,16 +340,17 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_kk_kernel(const __grid_
         const int t = (threadIdx.x - EPI_WARPS * 32) % GROUP_THREADS, group = (warp - EPI_WARPS) / GROUP_WARPS;
         const uint32_t at = (uint32_t)((t >> 3) * 64 + ((((t & 7) >> 1) ^ ((t >> 4) & 3)) << 4) + (t & 1) * 8);
         const int64_t stages = blockIdx.x < tiles ? (tiles - blockIdx.x + gridDim.x - 1) / gridDim.x * nk : 0;
-        Ring raw, stage;
+        RawRing raw;
+        Ring stage;
         raw.next(p.raw_slots, group);
         stage.next(p.stages, group);
         uint32_t top = 0;
         for (int64_t st = group; st < stages; st += GROUPS) {
-            if (!warp_wait(&bars.raw_full[raw.i], raw.use, bars, p)) break;
+            if (!warp_wait(&bars.raw_full[raw.bar()], raw.use(), bars, p)) break;
             float4 v[RAW_ITS];
-            take_raw(v, raws + (size_t)raw.i * RAW_BYTES, t);
+            take_raw(v, raws + (size_t)raw.slot * RAW_BYTES, t);
             __syncwarp();
-            if (lane == 0) mbar_arrive(&bars.raw_empty[raw.i]);
+            if (lane == 0) mbar_arrive(&bars.raw_empty[raw.bar()]);
             if (!warp_wait(&bars.empty[stage.i], stage.use ^ 1, bars, p)) break;
             uint8_t* dst = smem + (size_t)stage.i * stage_bytes + at;
 #pragma unroll
@@ -346,14 +365,15 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_kk_kernel(const __grid_
     } else if (warp == TMA_WARP) {
         // The raw tiles of A run raw_slots - 1 stages ahead of the planes of B.
         if (lane == 0) {
-            Ring raw, stage;
+            RawRing raw;
+            Ring stage;
             int64_t a_tile = blockIdx.x;
             int a_ks = 0;
             auto load_a = [&]() {
                 if (a_tile >= tiles) return true;
-                if (!thread_wait(&bars.raw_empty[raw.i], raw.use ^ 1, bars, p)) return false;
-                mbar_expect_tx(&bars.raw_full[raw.i], RAW_BYTES);
-                tma_load_2d(raws + (size_t)raw.i * RAW_BYTES, &map_a, a_ks * BK, (int32_t)((uint32_t)a_tile / (uint32_t)p.n_tiles) * BM, &bars.raw_full[raw.i]);
+                if (!raw_free(raw, bars, p)) return false;
+                mbar_expect_tx(&bars.raw_full[raw.bar()], RAW_BYTES);
+                tma_load_2d(raws + (size_t)raw.slot * RAW_BYTES, &map_a, a_ks * BK, (int32_t)((uint32_t)a_tile / (uint32_t)p.n_tiles) * BM, &bars.raw_full[raw.bar()]);
                 raw.next(p.raw_slots);
                 if (++a_ks == nk) { a_ks = 0; a_tile += gridDim.x; }
                 return true;
@@ -433,8 +453,9 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
         const int t = (threadIdx.x - EPI_WARPS * 32) % GROUP_THREADS, group = (warp - EPI_WARPS) / GROUP_WARPS;
         auto place = [](int row, int c4) { return (uint32_t)((c4 >> 4) * CHUNK + row * 128 + ((((c4 & 15) >> 1) ^ (row & 7)) << 4) + (c4 & 1) * 8); };
         const uint32_t at_a = place(t >> 5, t & 31), at_b = place(t >> 4, t & 15);
-        Ring raw, stage;
-        raw.next(p.raw_slots, 2 * group);                             // 2 * GROUPS slots at least: a group is never two uses behind
+        RawRing raw;
+        Ring stage;
+        raw.next(p.raw_slots, 2 * group);
         stage.next(p.stages, group);
         uint32_t top = 0;
         float4 v[RAW_ITS];
@@ -447,31 +468,31 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
             for (int it = 0; it < its; ++it) { add2(sum.x, sum.y, w[it].x, w[it].y); add2(sum.z, sum.w, w[it].z, w[it].w); }
         };
         for (int ks = group; ks < nk; ks += GROUPS) {
-            if (!warp_wait(&bars.raw_full[raw.i], raw.use, bars, p)) break;
-            take_raw(v, raws + (size_t)raw.i * RAW_BYTES, t);
+            if (!warp_wait(&bars.raw_full[raw.bar()], raw.use(), bars, p)) break;
+            take_raw(v, raws + (size_t)raw.slot * RAW_BYTES, t);
             __syncwarp();
-            if (lane == 0) mbar_arrive(&bars.raw_empty[raw.i]);
+            if (lane == 0) mbar_arrive(&bars.raw_empty[raw.bar()]);
             raw.next(p.raw_slots);
             if (!warp_wait(&bars.empty[stage.i], stage.use ^ 1, bars, p)) break;
             uint8_t* dst = smem + (size_t)stage.i * stage_bytes;
 #pragma unroll
             for (int it = 0; it < RAW_ITS; ++it) split4(v[it], dst + (at_a ^ (it & 1) * 64) + it * 4 * 128, MM_PART, top);
-            if (!warp_wait(&bars.raw_full[raw.i], raw.use, bars, p)) break;
+            if (!warp_wait(&bars.raw_full[raw.bar()], raw.use(), bars, p)) break;
             dst += PARTS * MM_PART;
             if (turn == (int)p.m_tiles) turn = 0;
             const bool sums = p.colsum_part && turn++ == 0;
             if (bw == 128) {
-                take_raw(v, raws + (size_t)raw.i * RAW_BYTES, t);
+                take_raw(v, raws + (size_t)raw.slot * RAW_BYTES, t);
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&bars.raw_empty[raw.i]);
+                if (lane == 0) mbar_arrive(&bars.raw_empty[raw.bar()]);
                 if (sums) add_columns(v, RAW_ITS);
 #pragma unroll
                 for (int it = 0; it < RAW_ITS; ++it) split4(v[it], dst + (at_a ^ (it & 1) * 64) + it * 4 * 128, b_part, top);
             } else {
                 float4 w[RAW_ITS / 2];
-                take_raw(w, raws + (size_t)raw.i * RAW_BYTES, t);
+                take_raw(w, raws + (size_t)raw.slot * RAW_BYTES, t);
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&bars.raw_empty[raw.i]);
+                if (lane == 0) mbar_arrive(&bars.raw_empty[raw.bar()]);
                 if (sums) add_columns(w, RAW_ITS / 2);
 #pragma unroll
                 for (int it = 0; it < RAW_ITS / 2; ++it) split4(w[it], dst + at_b + it * 8 * 128, b_part, top);
@@ -499,12 +520,12 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
         if (has_inf(top)) *p.overflow = 1;
     } else if (warp == TMA_WARP) {
         if (lane == 0) {
-            Ring raw;
+            RawRing raw;
             for (int u = 0; u < 2 * nk; ++u, raw.next(p.raw_slots)) {         // A, B, A, B, ...
-                if (!thread_wait(&bars.raw_empty[raw.i], raw.use ^ 1, bars, p)) break;
+                if (!raw_free(raw, bars, p)) break;
                 const int32_t k = (int32_t)(kb + (int64_t)(u >> 1) * BK);
-                mbar_expect_tx(&bars.raw_full[raw.i], u & 1 ? (uint32_t)bw * BK * 4 : (uint32_t)RAW_BYTES);
-                tma_load_2d(raws + (size_t)raw.i * RAW_BYTES, u & 1 ? &map_b : &map_a, (int32_t)(u & 1 ? n0 : m0), k, &bars.raw_full[raw.i]);
+                mbar_expect_tx(&bars.raw_full[raw.bar()], u & 1 ? (uint32_t)bw * BK * 4 : (uint32_t)RAW_BYTES);
+                tma_load_2d(raws + (size_t)raw.slot * RAW_BYTES, u & 1 ? &map_b : &map_a, (int32_t)(u & 1 ? n0 : m0), k, &bars.raw_full[raw.bar()]);
             }
         }
     } else {

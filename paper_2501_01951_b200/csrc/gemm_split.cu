@@ -267,6 +267,22 @@ __device__ __forceinline__ bool sum_tile(EpiState& st, Shared& b, const SplitPar
     }
 }
 
+// The mask bytes and gate bits that an epilogue thread's row of the CTA's next tile will want, to the L2: their latency stood
+// before every tile's sums (982 K x 63 x 91 with odd mask rows: 396 -> 372 us).
+__device__ __forceinline__ void prefetch_masks(const SplitParams& p, int64_t tile, int64_t tiles, int row, int c_first, int span) {
+    if (tile >= tiles || !(p.epi.drop || p.epi.gate_bits)) return;
+    const int64_t m = (int64_t)((uint32_t)tile / (uint32_t)p.n_tiles) * BM + row;
+    const int n = (int)((uint32_t)tile % (uint32_t)p.n_tiles) * p.bn + c_first;
+    if (m >= p.M || n >= p.N) return;
+    if (p.epi.drop) {
+        const uint8_t* at = p.epi.drop + (p.epi.row0 + m) * p.N + n;
+        const int last = (p.N - n < span ? (int)(p.N - n) : span) - 1;
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(at));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(at + last));
+    }
+    if (p.epi.gate_bits) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.epi.gate_bits + (p.epi.row0 + m) * p.epi.ld_gate_bits + (n >> 5)));
+}
+
 // ---------------------------------------------------------------- K-major form
 __global__ void __launch_bounds__(THREADS, 1) gemm_split_kk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                                                                    const __grid_constant__ CUtensorMap map_c, const SplitParams p, const int tma_store) {
@@ -299,6 +315,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_kk_kernel(const __grid_
             const int n0 = (int)((uint32_t)tile % (uint32_t)p.n_tiles) * p.bn;
             uint32_t dw[2] = {0xFFFFFFFFu, 0xFFFFFFFFu}, gw[2] = {0xFFFFFFFFu, 0xFFFFFFFFu};
             if (masks && chunks) mask_words(p.epi, m0 + quarter * 32, p.M, p.N, n0 + c_first, 32, n0 + (p.bn < c_first + span ? p.bn : c_first + span), lane, dw, gw);
+            prefetch_masks(p, tile + gridDim.x, tiles, quarter * 32 + lane, c_first, span);
             float acc[2][32];
             if (!sum_tile(st, bars, p, t_row, chunks, nk, lane, acc)) break;
 #pragma unroll
@@ -561,14 +578,23 @@ __global__ void pack_split_kernel(const float* __restrict__ src, int64_t ld, int
 
 namespace mixgcn {
 
-// Whether a product is large enough.  A call costs about 10 us beside the product (tensor maps, packing of the weights, the launch
-// behind it), which the rate makes up for from about 0.8 GFLOP on: 200 K x 32 x 64 (0.8 GFLOP) 50 us against 49 on the FMA
-// pipes, 400 K x 48 x 32 61 : 73, 100 K x 100 x 100 50 : 91, weight gradients 64 x 64 x 200 K 61 : 93, 500 x 48 x 20 K 39 : 45.
-// Tiles are padded to 16 columns and, in a weight gradient, 128 rows: 200 K x 16 x 256 89 : 115, 32 x 64 x 500 K 112 : 197, and
-// nothing narrower.  The K-major form adds up one fp32 chain of K / 32 sums, which past 1024 terms of one sign is less accurate
-// than the two levels of the FMA kernel (1.2e-7 : 5e-8 at 2048).
-static bool split_pays(int ta, int64_t M, int64_t N, int64_t K) {
-    return 2.0 * M * N * K >= 8e8 && N >= 16 && (ta ? M >= 32 : K <= 1024);
+// Whether a product is faster here than on the FMA pipes, by what both take (us, from measurements):
+//  * here 12 for packing, launches and the tail, and 0.75 per stage and 1.2 per tile of the longest CTA (weight gradient: 16 and
+//    0.85 per stage): a wave that is nearly empty counts in full.  20 K x 32 x 500 is two waves of sixteen stages, 35.5 us
+//    against 33.4 there; 20 K x 64 x 500, as long here, 37 : 73; 5 K x 128 x 256 20.8 : 25.6; 52 K x 80 x 80 22.9 : 39.7;
+//    876 K x 8 x 210 266 : 359; weight gradients 64 x 16 x 200 K 49 : 37, 40 x 40 x 200 K 51 : 85, 80 x 80 x 52 K 27 : 47;
+//  * there 20 TFLOP/s and more, with columns padded to 32, and 2 TB/s (876 K x 210 x 8: 392 : 558).
+// Below 4 columns (and, untried, 32 rows of a weight gradient) padding takes it all.  The K-major form adds up one fp32 chain of
+// K / 32 sums, which past 1024 terms of one sign is less accurate than the two levels of the FMA kernel (1.2e-7 : 5e-8 at 2048).
+static bool split_pays(const mixgcn_ctx* ctx, int ta, int64_t M, int64_t N, int64_t K) {
+    if (N < 4 || (ta ? M < 32 : K > 1024)) return false;
+    auto ceil_div = [](int64_t a, int64_t b) { return (a + b - 1) / b; };
+    const int64_t tiles = ceil_div(M, BM) * ceil_div(N, BN_MAX), nk = ceil_div(K, BK), sms = ctx->sm_count;
+    const double ops_us = 2.0 * M * (ceil_div(N, 32) * 32) * K / 20e6, bytes_us = 4.0 * (M * K + K * N + M * N) / 2e6;
+    const double fma_us = 2.0 + (ops_us > bytes_us ? ops_us : bytes_us);
+    if (!ta) return 12.0 + ceil_div(tiles, sms) * (1.2 + 0.75 * nk) < fma_us;
+    const int64_t least = nk < 8 ? nk : 8, stages = ceil_div(nk * tiles, sms);
+    return 16.0 + 0.85 * (stages > least ? stages : least) < fma_us;
 }
 
 // slots of raw tiles that fit beside `fixed` bytes (one block per SM: 227 KB, less the barriers)
@@ -586,7 +612,7 @@ mixgcn_status launch_gemm_split(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int6
     if (colsum_done) *colsum_done = false;
     if (M <= 0 || N <= 0 || K <= 0 || (ta && tb) || M >= (1ll << 31) || N >= (1ll << 31) || K >= (1ll << 31)) return MIXGCN_EUNSUPPORTED;
     if (!aligned16(A) || (lda & 3) || (ta && (!aligned16(B) || (ldb & 3) || epi))) return MIXGCN_EUNSUPPORTED;
-    if (!split_pays(ta, M, N, K)) return MIXGCN_EUNSUPPORTED;
+    if (!split_pays(ctx, ta, M, N, K)) return MIXGCN_EUNSUPPORTED;
     auto ceil_div = [](int64_t a, int64_t b) { return (a + b - 1) / b; };
     SplitParams p{};
     p.M = M; p.N = N; p.K = K; p.C = C; p.ldc = ldc;

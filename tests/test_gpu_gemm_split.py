@@ -55,6 +55,7 @@ def operands(M, N, K, ta, tb, positive=False):
 
 
 @pytest.mark.parametrize("M,N,K,ta", [
+    (200000, 4, 64, False), (5000, 128, 256, False), (60000, 5, 300, False), (40, 40, 200000, True), (300, 5, 200001, True), (128, 128, 20011, True),
     (200001, 16, 127, False), (30000, 17, 1000, False), (100000, 129, 32, False), (500, 1000, 1023, False), (80001, 161, 33, False),
     (13000, 64, 512, False), (18943, 128, 168, False), (18945, 65, 330, False), (1300000, 40, 8, False), (1000, 1003, 1024, False),
     (32, 16, 800001, True), (33, 63, 200003, True), (129, 65, 50031, True), (128, 128, 24577, True), (501, 303, 2700, True), (1003, 1001, 401, True)])

@@ -149,7 +149,13 @@ mixgcn_status launch_gemm(mixgcn_ctx* ctx, int precision, int ta, int tb, int64_
     if (ta && epi && (epi->gate_bits || epi->sign_bits)) MIXGCN_FAIL(MIXGCN_EINVAL, "gemm: bit-packed masks belong to the K-major form (trans_a = 0)");
     mixgcn_status st = MIXGCN_EUNSUPPORTED;
     const bool fp32_layout = aligned16(A) && (lda & 3) == 0 && (!ta || (aligned16(B) && (ldb & 3) == 0));
-    if (precision == MIXGCN_PREC_BF16 && !(ta && tb) && fp32_layout && M > 0 && N > 0 && K > 0) {
+    if (precision == MIXGCN_PREC_BF16 && !ta && fp32_layout && !(lp && lp->A) && !c_lp && !loss) {
+        // no bf16 copy of A, and none of C wanted: converted on the way into the product
+        st = launch_gemm_cvt(ctx, tb, M, N, K, A, lda, B, ldb, C, ldc, epi, epi_row0, s, &bits_done);
+        if (st != MIXGCN_OK && st != MIXGCN_EUNSUPPORTED) return st;
+        if (st == MIXGCN_OK) ctx->gemm_path[2]++;
+    }
+    if (st == MIXGCN_EUNSUPPORTED && precision == MIXGCN_PREC_BF16 && !(ta && tb) && fp32_layout && M > 0 && N > 0 && K > 0) {
         auto round8 = [](int64_t x) { return (x + 7) & ~(int64_t)7; };
         auto up = [](int64_t x) { return (x + 255) & ~(int64_t)255; };
         const int64_t a_rows = ta ? K : M, a_cols = ta ? M : K;

@@ -47,6 +47,7 @@ constexpr int STAGES_MAX = 4, RAW_MAX = 8;      // most stages of part tiles and
 static_assert(RAW_MAX % (2 * GROUPS) == 0);
 constexpr int HI_STAGES = 32 / BK, LO_STAGES = 1024 / BK;           // stages per accumulator of the large and of the small products
 constexpr uint32_t TMEM_COLS = 512, LO_COL = 256, BUF_COLS = 128;   // two accumulators for the large products, two for the small ones
+constexpr uint32_t CVT_COLS = 256;              // the two accumulators of the bf16 form
 constexpr int RAW_BYTES = BM * BK * 4, KK_PART = BM * BK * 2;       // a raw tile; K-major part tiles: 64-byte rows and swizzle
 constexpr int CHUNK = BK * 128, MM_PART = BM / 64 * CHUNK;          // MN-major tiles: chunks of 64 columns, 128-byte k-rows and swizzle
 
@@ -267,6 +268,62 @@ __device__ __forceinline__ bool sum_tile(EpiState& st, Shared& b, const SplitPar
     }
 }
 
+// The loads of a K-major kernel, by one thread: the raw tiles of A run raw_slots - 1 stages ahead of the planes of B.
+__device__ __forceinline__ void load_kk(const SplitParams& p, Shared& bars, const CUtensorMap& map_a, const CUtensorMap& map_b, uint8_t* smem, uint8_t* raws,
+                                        uint32_t stage_bytes, uint32_t b_offset, uint32_t b_part, int parts, int nk, int64_t tiles) {
+    RawRing raw;
+    Ring stage;
+    int64_t a_tile = blockIdx.x;
+    int a_ks = 0;
+    auto load_a = [&]() {
+        if (a_tile >= tiles) return true;
+        if (!raw_free(raw, bars, p)) return false;
+        mbar_expect_tx(&bars.raw_full[raw.bar()], RAW_BYTES);
+        tma_load_2d(raws + (size_t)raw.slot * RAW_BYTES, &map_a, a_ks * BK, (int32_t)((uint32_t)a_tile / (uint32_t)p.n_tiles) * BM, &bars.raw_full[raw.bar()]);
+        raw.next(p.raw_slots);
+        if (++a_ks == nk) { a_ks = 0; a_tile += gridDim.x; }
+        return true;
+    };
+    bool ok = true;
+    for (int i = 0; i + 1 < p.raw_slots && ok; ++i) ok = load_a();
+    for (int64_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
+        const int n0 = (int)((uint32_t)tile % (uint32_t)p.n_tiles) * p.bn;
+        for (int ks = 0; ks < nk && ok; ++ks) {
+            if (!thread_wait(&bars.empty[stage.i], stage.use ^ 1, bars, p)) return;
+            uint8_t* sb = smem + (size_t)stage.i * stage_bytes + b_offset;
+            mbar_expect_tx(&bars.full[stage.i], parts * b_part);
+            for (int q = 0; q < parts; ++q) tma_load_2d(sb + q * b_part, &map_b, ks * BK, q * p.plane_rows + n0, &bars.full[stage.i]);
+            stage.next(p.stages);
+            ok = load_a();
+        }
+    }
+}
+
+// 32 rows from row `first`, 32 columns from nb (`here` of them the tile's), through this warp's box.
+__device__ __forceinline__ void store_chunk(const SplitParams& p, const CUtensorMap& map_c, int tma_store, uint8_t* box, const float (&v)[32], int64_t first, int nb,
+                                            int here, int lane) {
+    if (tma_store && lane == 0) bulk_wait_read<0>();   // the store that last used this box has read it
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+        *reinterpret_cast<float4*>(box + lane * 128 + ((q ^ (lane & 7)) << 4)) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    if (tma_store && (nb + 32 <= p.N || (p.N & 3) == 0)) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) {
+            tma_store_2d(&map_c, box, nb, (int32_t)first);
+            bulk_commit();
+        }
+    } else {
+        // row by row: TMA stores whole 16-byte units, and what lies behind the matrix's last column is not ours
+        __syncwarp();
+        if (nb + lane < p.N && lane < here)
+            for (int r = 0; r < 32 && first + r < p.M; ++r)
+                p.C[(first + r) * p.ldc + nb + lane] = *reinterpret_cast<const float*>(box + r * 128 + (((lane >> 2) ^ (r & 7)) << 4) + (lane & 3) * 4);
+        __syncwarp();
+    }
+}
+
 // The mask bytes and gate bits that an epilogue thread's row of the CTA's next tile will want, to the L2: their latency stood
 // before every tile's sums (982 K x 63 x 91 with odd mask rows: 396 -> 372 us).
 __device__ __forceinline__ void prefetch_masks(const SplitParams& p, int64_t tile, int64_t tiles, int row, int c_first, int span) {
@@ -325,28 +382,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_kk_kernel(const __grid_
                 if (nb >= p.N) break;
                 chunk_epilogue(p.epi, acc[k], nb, p.N, nullptr, dw[k], gw[k]);
                 if (p.epi.sign_bits && m < p.M) p.epi.sign_bits[(p.epi.row0 + m) * p.epi.ld_sign_bits + (nb >> 5)] = sign_word(acc[k], nb, p.N);
-                if (tma_store && lane == 0) bulk_wait_read<0>();   // the store that last used this box has read it
-                __syncwarp();
-#pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    *reinterpret_cast<float4*>(box + lane * 128 + ((q ^ (lane & 7)) << 4)) =
-                        make_float4(acc[k][4 * q], acc[k][4 * q + 1], acc[k][4 * q + 2], acc[k][4 * q + 3]);
-                if (tma_store && (nb + 32 <= p.N || (p.N & 3) == 0)) {
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    __syncwarp();
-                    if (lane == 0) {
-                        tma_store_2d(&map_c, box, nb, (int32_t)(m0 + quarter * 32));
-                        bulk_commit();
-                    }
-                } else {
-                    // row by row: TMA stores whole 16-byte units, and what lies behind the matrix's last column is not ours
-                    __syncwarp();
-                    const int64_t first = m0 + quarter * 32;
-                    if (nb + lane < p.N && c0 + lane < p.bn)
-                        for (int r = 0; r < 32 && first + r < p.M; ++r)
-                            p.C[(first + r) * p.ldc + nb + lane] = *reinterpret_cast<const float*>(box + r * 128 + (((lane >> 2) ^ (r & 7)) << 4) + (lane & 3) * 4);
-                    __syncwarp();
-                }
+                store_chunk(p, map_c, tma_store, box, acc[k], m0 + quarter * 32, nb, p.bn - c0, lane);
             }
         }
         if (tma_store && lane == 0) bulk_wait_all();
@@ -380,35 +416,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_kk_kernel(const __grid_
         }
         if (has_inf(top)) *p.overflow = 1;
     } else if (warp == TMA_WARP) {
-        // The raw tiles of A run raw_slots - 1 stages ahead of the planes of B.
-        if (lane == 0) {
-            RawRing raw;
-            Ring stage;
-            int64_t a_tile = blockIdx.x;
-            int a_ks = 0;
-            auto load_a = [&]() {
-                if (a_tile >= tiles) return true;
-                if (!raw_free(raw, bars, p)) return false;
-                mbar_expect_tx(&bars.raw_full[raw.bar()], RAW_BYTES);
-                tma_load_2d(raws + (size_t)raw.slot * RAW_BYTES, &map_a, a_ks * BK, (int32_t)((uint32_t)a_tile / (uint32_t)p.n_tiles) * BM, &bars.raw_full[raw.bar()]);
-                raw.next(p.raw_slots);
-                if (++a_ks == nk) { a_ks = 0; a_tile += gridDim.x; }
-                return true;
-            };
-            bool ok = true;
-            for (int i = 0; i + 1 < p.raw_slots && ok; ++i) ok = load_a();
-            for (int64_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
-                const int n0 = (int)((uint32_t)tile % (uint32_t)p.n_tiles) * p.bn;
-                for (int ks = 0; ks < nk && ok; ++ks) {
-                    if (!thread_wait(&bars.empty[stage.i], stage.use ^ 1, bars, p)) { ok = false; break; }
-                    uint8_t* sb = smem + (size_t)stage.i * stage_bytes + PARTS * KK_PART;
-                    mbar_expect_tx(&bars.full[stage.i], PARTS * b_part);
-                    for (int q = 0; q < PARTS; ++q) tma_load_2d(sb + q * b_part, &map_b, ks * BK, q * p.plane_rows + n0, &bars.full[stage.i]);
-                    stage.next(p.stages);
-                    ok = load_a();
-                }
-            }
-        }
+        if (lane == 0) load_kk(p, bars, map_a, map_b, smem, raws, stage_bytes, PARTS * KK_PART, b_part, PARTS, nk, tiles);
     } else {
         const uint32_t idesc = make_idesc<KIND_BF16>(BM, p.bn, false);
         MmaState st;
@@ -556,9 +564,109 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
     cta_end(bars, warp, tmem);
 }
 
+// ---------------------------------------------------------------- bf16 product of fp32 rows
+// The K-major form with one part: a bf16 product whose fp32 operand comes without a bf16 copy (the features of an inference, mostly).
+// Converted on the way in, it is read once; a pass that wrote the copy first read and wrote it besides.  All K terms go to one
+// accumulator in the order of the bf16 kernel, so the bits are that kernel's on the copy.  Bound: HBM.  700 K x 130 x 301: 377 us
+// with the pass, 236 so.
+__global__ void __launch_bounds__(THREADS, 1) gemm_cvt_kk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
+                                                                 const __grid_constant__ CUtensorMap map_c, const SplitParams p, const int tma_store) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) Shared bars;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t stage_bytes = KK_PART + (uint32_t)((p.bn + 31) & ~31) * BK * 2;
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t* raws = smem + (size_t)p.stages * stage_bytes;
+    uint8_t* boxes = raws + (size_t)p.raw_slots * RAW_BYTES;
+    const int nk = (int)((p.K + BK - 1) / BK);
+    const int64_t tiles = p.m_tiles;                                        // one column of tiles
+    const uint32_t tmem = cta_begin(bars, GROUP_WARPS + 1, warp);
+
+    if (warp < EPI_WARPS) {
+        const int quarter = warp & 3, half = warp >> 2;                     // 32-column chunks half, half + 2, ...
+        const bool masks = p.epi.drop != nullptr || p.epi.gate != nullptr || p.epi.gate_bits != nullptr;
+        uint8_t* const box = boxes + (size_t)warp * 4096;
+        uint32_t c = 0;
+        for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++c) {
+            const int64_t m0 = tile * BM + quarter * 32, m = m0 + lane;
+            uint32_t dw[4], gw[4];
+            if (masks) mask_words(p.epi, m0, p.M, p.N, half * 32, 64, p.bn, lane, dw, gw);
+            if (!warp_wait(&bars.hi_full[c & 1], (c >> 1) & 1, bars, p)) break;
+            tc_fence_after();
+#pragma unroll
+            for (int ci = 0; ci < 4; ++ci) {
+                const int nb = half * 32 + ci * 64;
+                if (nb >= p.N) break;
+                uint32_t r[32];
+                tc_ld32(tmem + (c & 1) * CVT_COLS + ((uint32_t)(quarter * 32) << 16) + (uint32_t)nb, r);
+                tc_wait_ld();
+                float v[32];
+#pragma unroll
+                for (int q = 0; q < 32; ++q) v[q] = __uint_as_float(r[q]);
+                chunk_epilogue(p.epi, v, nb, p.N, nullptr, masks ? dw[ci] : 0xFFFFFFFFu, masks ? gw[ci] : 0xFFFFFFFFu);
+                if (p.epi.sign_bits && m < p.M) p.epi.sign_bits[(p.epi.row0 + m) * p.epi.ld_sign_bits + (nb >> 5)] = sign_word(v, nb, p.N);
+                store_chunk(p, map_c, tma_store, box, v, m0, nb, p.bn - nb, lane);
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars.hi_empty[c & 1]);
+        }
+        if (tma_store && lane == 0) bulk_wait_all();
+    } else if (warp < TMA_WARP) {
+        const int t = (threadIdx.x - EPI_WARPS * 32) % GROUP_THREADS, group = (warp - EPI_WARPS) / GROUP_WARPS;
+        const uint32_t at = (uint32_t)((t >> 3) * 64 + ((((t & 7) >> 1) ^ ((t >> 4) & 3)) << 4) + (t & 1) * 8);     // as in the K-major form
+        const int64_t stages = blockIdx.x < tiles ? (tiles - blockIdx.x + gridDim.x - 1) / gridDim.x * nk : 0;
+        RawRing raw;
+        Ring stage;
+        raw.next(p.raw_slots, group);
+        stage.next(p.stages, group);
+        for (int64_t st = group; st < stages; st += GROUPS) {
+            if (!warp_wait(&bars.raw_full[raw.bar()], raw.use(), bars, p)) break;
+            float4 v[RAW_ITS];
+            take_raw(v, raws + (size_t)raw.slot * RAW_BYTES, t);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars.raw_empty[raw.bar()]);
+            if (!warp_wait(&bars.empty[stage.i], stage.use ^ 1, bars, p)) break;
+            uint8_t* dst = smem + (size_t)stage.i * stage_bytes + at;
+#pragma unroll
+            for (int it = 0; it < RAW_ITS; ++it)
+                *reinterpret_cast<uint2*>(dst + it * 16 * 64) = make_uint2(pack_bf16(v[it].x, v[it].y), pack_bf16(v[it].z, v[it].w));
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars.full[stage.i]);
+            raw.next(p.raw_slots, GROUPS);
+            stage.next(p.stages, GROUPS);
+        }
+    } else if (warp == TMA_WARP) {
+        if (lane == 0) load_kk(p, bars, map_a, map_b, smem, raws, stage_bytes, KK_PART, stage_bytes - KK_PART, 1, nk, tiles);
+    } else {
+        const uint32_t idesc = make_idesc<KIND_BF16>(BM, p.bn, false);
+        Ring stage;
+        uint32_t c = 0;
+        bool ok = true;
+        for (int64_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++c) {
+            if (!warp_wait(&bars.hi_empty[c & 1], ((c >> 1) & 1) ^ 1, bars, p)) break;
+            for (int ks = 0; ks < nk; ++ks, stage.next(p.stages)) {
+                if (!warp_wait(&bars.full[stage.i], stage.use, bars, p)) { ok = false; break; }
+                tc_fence_after();
+                const uint32_t sa = smem_u32(smem + (size_t)stage.i * stage_bytes);
+                const uint64_t da = make_desc(sa, 16, 512, 4), db = make_desc(sa + KK_PART, 16, 512, 4);
+                if (elect_one()) {
+                    tc_mma<KIND_BF16>(tmem + (c & 1) * CVT_COLS, da, db, idesc, ks ? 1u : 0u);
+                    tc_mma<KIND_BF16>(tmem + (c & 1) * CVT_COLS, da + 2, db + 2, idesc, 1u);
+                    tc_commit(&bars.empty[stage.i]);
+                    if (ks + 1 == nk) tc_commit(&bars.hi_full[c & 1]);
+                }
+                __syncwarp();
+            }
+        }
+    }
+    cta_end(bars, warp, tmem);
+}
+
 // Packed planes of the weight matrix: plane q of dst (rows x kpad bf16) holds part q of trans ? src[k][n] : src[n][k], zeros
 // outside N x K.
-__global__ void pack_split_kernel(const float* __restrict__ src, int64_t ld, int trans, int N, int K, int rows, int kpad,
+__global__ void pack_split_kernel(const float* __restrict__ src, int64_t ld, int trans, int N, int K, int rows, int kpad, int parts,
                                   uint16_t* __restrict__ dst, int32_t* overflow) {
     const int64_t plane = (int64_t)rows * kpad, i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= plane) return;
@@ -567,8 +675,9 @@ __global__ void pack_split_kernel(const float* __restrict__ src, int64_t ld, int
     if (n < N && k < K) v = trans ? __ldg(src + (int64_t)k * ld + n) : __ldg(src + (int64_t)n * ld + k);
 #pragma unroll
     for (int q = 0; q < PARTS; ++q) {
+        if (q >= parts) break;
         const uint32_t b = pack_bf16(v, 0.0f) & 0xFFFFu;
-        if (q == 0 && (b & 0x7FFFu) == 0x7F80u) *overflow = 1;
+        if (q == 0 && overflow && (b & 0x7FFFu) == 0x7F80u) *overflow = 1;
         dst[q * plane + (int64_t)n * kpad + k] = (uint16_t)b;
         v -= __uint_as_float(b << 16);
     }
@@ -648,7 +757,7 @@ mixgcn_status launch_gemm_split(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int6
         MIXGCN_CUDA(cudaMemsetAsync(p.overflow, 0, sizeof(int32_t), s));
         {
             LaunchScope scope(ctx, PH_GEMM, s);
-            pack_split_kernel<<<(unsigned)ceil_div((int64_t)rows * kpad, 256), 256, 0, s>>>(B, ldb, tb ? 0 : 1, (int)N, (int)K, rows, kpad, planes, p.overflow);
+            pack_split_kernel<<<(unsigned)ceil_div((int64_t)rows * kpad, 256), 256, 0, s>>>(B, ldb, tb ? 0 : 1, (int)N, (int)K, rows, kpad, PARTS, planes, p.overflow);
         }
         LaunchScope scope(ctx, PH_GEMM, s);
         const unsigned grid = (unsigned)(tiles < ctx->sm_count ? tiles : ctx->sm_count);
@@ -693,6 +802,48 @@ mixgcn_status launch_gemm_split(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int6
         if (colsum_done) *colsum_done = true;
     }
     if (splits > 1) MIXGCN_TRY(launch_splitk_reduce(ctx, M, N, (int)splits, p.C, C, ldc, nullptr, s));
+    return MIXGCN_OK;
+}
+
+// C = bf16(A) bf16(op(B)) for fp32 rows A without a bf16 copy, K-major, N up to 256 (one column of tiles: wider results read and
+// convert A again for each); MIXGCN_EUNSUPPORTED (nothing launched) otherwise.
+mixgcn_status launch_gemm_cvt(mixgcn_ctx* ctx, int tb, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda, const float* B, int64_t ldb, float* C,
+                              int64_t ldc, const mixgcn_epilogue* epi, int64_t epi_row0, cudaStream_t s, bool* bits_done) {
+    if (bits_done) *bits_done = false;
+    if (M <= 0 || N <= 0 || K <= 0 || N > (int64_t)CVT_COLS || M >= (1ll << 31) || K >= (1ll << 31) || !aligned16(A) || (lda & 3)) return MIXGCN_EUNSUPPORTED;
+    // few tiles with many stages each: the bf16 kernel's longer stages win over the pass (4 K x 256 x 2048: 49 us here, 37 there)
+    if (M <= (int64_t)BM * (ctx->sm_count - 1) && K > 512) return MIXGCN_EUNSUPPORTED;
+    if (ctx->debug_drop_load) return MIXGCN_EUNSUPPORTED;
+    auto ceil_div = [](int64_t a, int64_t b) { return (a + b - 1) / b; };
+    SplitParams p{};
+    p.M = M; p.N = N; p.K = K; p.C = C; p.ldc = ldc;
+    p.vec_c = aligned16(C) && (ldc & 3) == 0;
+    p.n_tiles = 1; p.bn = (int)(ceil_div(N, 16) * 16); p.m_tiles = ceil_div(M, BM); p.stages = STAGES_MAX;
+    p.epi = make_tc_epi(epi, epi_row0);
+    p.status = ctx->d_status;
+    p.wait_limit = ctx->debug_wait_limit > 0 ? (uint32_t)ctx->debug_wait_limit : WAIT_LIMIT_DEFAULT;
+    const int bn32 = (p.bn + 31) & ~31, kpad = (int)(ceil_div(K, BK) * BK);
+    MIXGCN_TRY(ensure_workspace(ctx, (int64_t)bn32 * kpad * 2));
+    uint16_t* packed = reinterpret_cast<uint16_t*>(ctx->workspace);
+    CUtensorMap map_a, map_b, map_c;
+    if (!encode_2d(&map_a, A, 4, K, M, lda, BK, BM, CU_TENSOR_MAP_SWIZZLE_NONE)) return MIXGCN_EUNSUPPORTED;
+    if (!encode_2d(&map_b, packed, 2, kpad, bn32, kpad, BK, bn32, CU_TENSOR_MAP_SWIZZLE_64B)) return MIXGCN_EUNSUPPORTED;
+    map_c = map_a;
+    const int tma_store = p.vec_c;
+    if (tma_store && !encode_2d(&map_c, C, 4, N, M, ldc, 32, 32)) return MIXGCN_EUNSUPPORTED;
+    const size_t fixed = (size_t)p.stages * (KK_PART + bn32 * BK * 2) + (size_t)EPI_WARPS * 4096 + 1024;
+    p.raw_slots = raw_slots(fixed, RAW_BYTES);
+    const size_t smem = fixed + (size_t)p.raw_slots * RAW_BYTES;
+    MIXGCN_CUDA(cudaFuncSetAttribute(gemm_cvt_kk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    {
+        LaunchScope scope(ctx, PH_GEMM, s);
+        pack_split_kernel<<<(unsigned)ceil_div((int64_t)bn32 * kpad, 256), 256, 0, s>>>(B, ldb, tb ? 0 : 1, (int)N, (int)K, bn32, kpad, 1, packed, nullptr);
+    }
+    LaunchScope scope(ctx, PH_GEMM, s);
+    const unsigned grid = (unsigned)(p.m_tiles < ctx->sm_count ? p.m_tiles : ctx->sm_count);
+    gemm_cvt_kk_kernel<<<grid, THREADS, smem, s>>>(map_a, map_b, map_c, p, tma_store);
+    MIXGCN_CUDA(cudaGetLastError());
+    if (bits_done) *bits_done = p.epi.sign_bits != nullptr;
     return MIXGCN_OK;
 }
 

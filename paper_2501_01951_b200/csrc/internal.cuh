@@ -312,6 +312,8 @@ mixgcn_status launch_gemm_simt(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64
 mixgcn_status launch_gemm_split(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda,
                                 const float* B, int64_t ldb, float* C, int64_t ldc, const mixgcn_epilogue* epi, int64_t epi_row0,
                                 cudaStream_t s, bool* bits_done, const int32_t** overflow_flag, float* colsum_b, bool* colsum_done);
+mixgcn_status launch_gemm_cvt(mixgcn_ctx* ctx, int tb, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda, const float* B, int64_t ldb, float* C,
+                              int64_t ldc, const mixgcn_epilogue* epi, int64_t epi_row0, cudaStream_t s, bool* bits_done);
 mixgcn_status launch_colsum_splits(mixgcn_ctx* ctx, int64_t N, int splits, const double* part, float* out, cudaStream_t s);
 mixgcn_status launch_gemm_tc(mixgcn_ctx* ctx, int kind, int ta, int tb, int64_t M, int64_t N, int64_t K, const void* A,
                              int64_t lda, const void* B, int64_t ldb, float* C, int64_t ldc,

@@ -26,9 +26,13 @@ def round4(x: int) -> int:
     return (x + 3) // 4 * 4
 
 
-def update_first(d_in: int, d_out: int, first: bool) -> bool:
+def update_first(d_in: int, d_out: int, first: bool, precision: int, relu: bool) -> bool:
     """Whether aggregating after the product (at width d_out, forward and backward) is cheaper than before it (at width
-    d_in, forward and -- unless the layer is the first -- backward); ties aggregate first."""
+    d_in, forward and -- unless the layer is the first -- backward); ties aggregate first.  A product that rounds its operands
+    rounds others on the other side of the aggregation: where a ReLU follows, signs near zero would change with them (GIN in
+    bf16, whose sums grow with the degree: 1.4e-2 -> 5e-2 against fp32), so those layers keep the defining order."""
+    if relu and precision != mg.PREC_FP32:
+        return False
     return 2 * d_out < (1 if first else 2) * d_in
 
 
@@ -93,7 +97,7 @@ class SageTrainer(_Base):
     def __init__(self, ctx, graph, dims, precision=mg.PREC_FP32):
         super().__init__(ctx, graph, dims, precision)
         n, L, ld = self.n, self.L, self.ld
-        self.upd = [update_first(self.dims[l], self.dims[l + 1], l == 0) for l in range(L)]
+        self.upd = [update_first(self.dims[l], self.dims[l + 1], l == 0, precision, l < L - 1) for l in range(L)]
         self.S = [self._z(n, ld[l] if self.upd[l] else 2 * ld[l]) for l in range(L)]
         # gradients w.r.t. the layers' outputs: [G | M^T G] where the layer updates first, G otherwise; the hidden ones take
         # turns in two buffers, which the forward pass uses for the update-first products
@@ -185,7 +189,7 @@ class GinTrainer(_Base):
         super().__init__(ctx, graph, dims, precision)
         n, L, ld = self.n, self.L, self.ld
         self.hidden, self.ldh, self.gin_eps = int(hidden), round4(hidden), float(gin_eps)
-        self.upd = [update_first(self.dims[l], self.hidden, l == 0) for l in range(L)]
+        self.upd = [update_first(self.dims[l], self.hidden, l == 0, precision, True) for l in range(L)]
         self.H = [None] + [self._z(n, ld[l]) for l in range(1, L)]
         # aggregate-first layers keep (1 + eps) H + A H for their weight gradient; update-first ones share scratch for H W1
         # and its gradient

@@ -12,9 +12,10 @@
 //    accumulator to fp32 sums in registers, rounding to nearest, while the next 32 terms go to a second accumulator;
 //  * the five small products, at most 2^-8 of the large ones, have an accumulator of their own for up to 1024 terms.
 //
-// Bound: shared memory.  A stage of 32 terms of a 128 x 128 tile is twelve instructions, 768 cycles of the tensor core and as
-// many of operand reads; the raw tile in, its conversion and the planes of B add 640 cycles of the same port.  The bf16 rate
-// over six (270 TFLOP/s of fp32 products; the FMA pipes have 72) is therefore not reached: tensor pipe 35 to 40 % active.
+// Bound: the hand-overs between the roles.  A stage of 32 terms of a 128 x 128 tile is twelve instructions, 768 cycles of the
+// tensor core, and takes about 1,800: raw tile, conversion, MMA and epilogue follow one another, with the three stages of part
+// tiles in flight that shared memory holds.  Tensor pipe 43 to 45 % active (of 270 TFLOP/s of fp32 products; the FMA pipes
+// have 72), shared-memory banks 40 %, issue slots 40 to 55 %.
 // Measured against the FMA kernel: 170 K x 256 x 256 forward 508 -> 178 us (126 TFLOP/s), its weight gradient 466 -> 163,
 // 170 K x 40 x 256 145 -> 79, 1 M x 300 x 300 4493 -> 1590.
 //

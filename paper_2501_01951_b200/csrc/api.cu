@@ -197,7 +197,12 @@ mixgcn_status launch_gemm(mixgcn_ctx* ctx, int precision, int ta, int tb, int64_
         // cannot be split (it returns at once otherwise); all others: the FMA kernel
         const int32_t* overflow = nullptr;
         bool split_bits = false, fma_bits = false;
-        st = launch_gemm_split(ctx, ta, tb, M, N, K, A, lda, B, ldb, C, ldc, epi, epi_row0, s, &split_bits, &overflow, colsum_b, &colsum_done);
+        // Products under a ReLU stay with the FMA kernel and its order of sums: pre-activations within a rounding error of zero
+        // keep their signs, and the gates of the backward pass with them (170 K nodes, 256 wide: six runs of sixteen had gradients
+        // move by 2e-4 to 8e-4 otherwise, one in twenty by more than 1e-3, though the activations agree to 2e-7).
+        const bool gates = (epi && epi->relu) || (lp && lp->relu_follows);
+        st = gates ? MIXGCN_EUNSUPPORTED
+                   : launch_gemm_split(ctx, ta, tb, M, N, K, A, lda, B, ldb, C, ldc, epi, epi_row0, s, &split_bits, &overflow, colsum_b, &colsum_done);
         if (st != MIXGCN_OK && st != MIXGCN_EUNSUPPORTED) return st;
         const bool split = st == MIXGCN_OK;
         st = launch_gemm_simt(ctx, ta, tb, M, N, K, A, lda, B, ldb, C, ldc, epi, epi_row0, s, &fma_bits, split ? overflow : nullptr);
@@ -689,7 +694,7 @@ extern "C" mixgcn_status mixgcn_layer_fwd(mixgcn_ctx* ctx, const mixgcn_graph* g
     // update first: Q = X_in W (into `saved`), then X_out = epilogue(A_hat Q).  Every row of Q is
     // needed before any aggregated row can be produced, so there is nothing to chunk here.
     {
-        GemmLP glp; glp.A = lp.x_in; glp.lda = lp.ld_in;
+        GemmLP glp; glp.A = lp.x_in; glp.lda = lp.ld_in; glp.relu_follows = (d->flags & MIXGCN_LAYER_RELU) != 0;
         MIXGCN_TRY(launch_gemm(ctx, d->precision, 0, 0, n, d->d_out, d->d_in, X_in, d->ld_in, W, ldw, saved, d->ld_saved,
                                nullptr, 0, s, &glp));
     }

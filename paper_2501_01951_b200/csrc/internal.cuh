@@ -294,6 +294,7 @@ void release_view(CsrView& v);
 // Leading dimensions in bf16 elements, multiples of 8; pointers 16-byte aligned.
 struct GemmLP {
     bool a_fp32_missing = false;      // the fp32 A holds no data (only its bf16 copy was written): no fallback below bf16
+    bool relu_follows = false;        // a ReLU is taken of what an aggregation makes of C
     const LossFuse* loss = nullptr;   // K-major form, N <= 256, C = logits of a masked loss: the epilogue writes every row's arg-max to
                                       // loss->pred and only the rows of loss->train_mask to C (the others zeroed if loss->zero_rows, else
                                       // left alone); MIXGCN_EUNSUPPORTED, nothing computed, if no tensor-core kernel takes the product

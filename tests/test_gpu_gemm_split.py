@@ -76,11 +76,13 @@ def test_split_epilogue(mg, ctx, M, N, K):
     gate = synth.uniform_tensor((M, N), 35, -1, 1).cuda()
     words = (N + 31) // 32
     bits = torch.full((M, words + 1), -1, dtype=torch.int32, device="cuda")
-    got = product(mg, ctx, A, B, False, False, bias=bias, relu=True, drop_mask=drop, keep_scale=2.0, gate=device(gate, up(N)), gate_scale=0.5, sign_bits=bits)
-    want = torch.relu(A.double() @ B.double() + bias.double()) * drop.reshape(M, N) * (gate > 0)
-    assert error(got, want) <= TOL_FP32
-    j = torch.arange(N, device="cuda")
-    assert torch.equal((bits[:, j // 32] >> (j % 32)) & 1, (got > 0).int()) and torch.all(bits[:, words] == -1)
+    for relu in (False, True):                                           # under a ReLU the FMA kernel takes the product
+        got = product(mg, ctx, A, B, False, False, bias=bias, relu=relu, drop_mask=drop, keep_scale=2.0, gate=device(gate, up(N)), gate_scale=0.5, sign_bits=bits)
+        want = A.double() @ B.double() + bias.double()
+        want = (torch.relu(want) if relu else want) * drop.reshape(M, N) * (gate > 0)
+        assert error(got, want) <= TOL_FP32
+        j = torch.arange(N, device="cuda")
+        assert torch.equal((bits[:, j // 32] >> (j % 32)) & 1, (got > 0).int()) and torch.all(bits[:, words] == -1)
 
 
 @pytest.mark.parametrize("ta", [False, True])

@@ -136,8 +136,10 @@ mixgcn_status mixgcn_ctx_profile_read(mixgcn_ctx* ctx, double ms[MIXGCN_N_PHASES
  * recording (run the sequence once before recording it); record_end then fails too, and nothing is left behind.
  * mixgcn_replay enqueues the recorded calls on `stream` with the arguments they were recorded with: the same pointers
  * (whose memory must still be the caller's), sizes and scalars.  It returns MIXGCN_EUNSUPPORTED, and enqueues nothing,
- * when the recording no longer stands for the calls -- scratch of the context has moved, an option has changed, or
- * profiling is on; issue the calls themselves then.  A recording may be destroyed after its context, not replayed. */
+ * when the recording no longer stands for the calls -- scratch of the context has moved, an option has changed, a graph or
+ * row plan the calls used has been destroyed or a graph's chunk schedules have been replaced (by a call with another
+ * n_chunks), or profiling is on; issue the calls themselves then.  A recording may be destroyed after its context, not
+ * replayed. */
 typedef struct mixgcn_recording mixgcn_recording;
 mixgcn_status mixgcn_record_begin(mixgcn_ctx* ctx, void** stream);
 mixgcn_status mixgcn_record_end(mixgcn_ctx* ctx, mixgcn_recording** out);

@@ -238,7 +238,8 @@ def record(ctx: Ctx, calls):
 class Replayer:
     """Runs a sequence of calls that a training loop issues again and again: twice call by call, then from a recording.
     `key` is whatever decides what the calls do (pointers, flags, sizes); the recording is made when the same key
-    has come twice and the calls leave it as it was, and used while it stays the same."""
+    has come twice and the calls leave it as it was, and used while it stays the same.  The library knows which graphs and
+    row plans a recording points into and refuses to replay it once one of them is gone, whatever its address says."""
 
     def __init__(self, ctx: Ctx):
         self.ctx, self.key, self.rec, self.refused = ctx, None, None, None
@@ -250,9 +251,11 @@ class Replayer:
             return
         k = key()
         if k == self.key:
-            if self.rec is not None and self.rec.replay():
-                return
-            if self.refused != k:
+            if self.rec is not None:
+                if self.rec.replay():
+                    return
+                self.rec = None          # what it used has moved: the calls themselves first (they may allocate), then another
+            elif self.refused != k:
                 self.rec = record(self.ctx, calls)
                 if self.rec is not None and key() == k and self.rec.replay():
                     return

@@ -8,6 +8,7 @@
 
 #include <mutex>
 #include <new>
+#include <vector>
 
 #include "internal.cuh"
 
@@ -414,8 +415,39 @@ struct mixgcn_recording {
     int device;
     cudaGraphExec_t exec;
     CtxState before, counted;      // state when recording began; launches and products the sequence adds to the counters
+    struct Use { MemoryGeneration memory; uint64_t value; };
+    std::vector<Use> uses;         // graphs and row plans whose memory the launches point into
+    bool uses_complete = true;
     explicit mixgcn_recording(mixgcn_ctx* c) : ctx(c), device(c->device), exec(nullptr), before(c), counted(c) {}
+    bool memory_stands() const {
+        for (const Use& u : uses) if (u.memory->load() != u.value) return false;
+        return true;
+    }
 };
+
+namespace mixgcn {
+
+mixgcn_status new_generation(MemoryGeneration* out) {
+    try {
+        *out = std::make_shared<std::atomic<uint64_t>>(0);
+    } catch (const std::bad_alloc&) {
+        MIXGCN_FAIL(MIXGCN_ENOMEM, "host allocation failed");
+    }
+    return MIXGCN_OK;
+}
+
+void recording_uses(mixgcn_ctx* ctx, const MemoryGeneration& memory) {
+    mixgcn_recording* r = ctx->recording;
+    if (!r) return;
+    for (const mixgcn_recording::Use& u : r->uses) if (u.memory == memory) return;
+    try {
+        r->uses.push_back({memory, memory->load()});
+    } catch (const std::bad_alloc&) {
+        r->uses_complete = false;
+    }
+}
+
+}  // namespace mixgcn
 
 extern "C" mixgcn_status mixgcn_record_begin(mixgcn_ctx* ctx, void** stream) {
     if (!ctx || !stream) MIXGCN_FAIL(MIXGCN_EINVAL, "record_begin: null argument");
@@ -454,11 +486,11 @@ extern "C" mixgcn_status mixgcn_record_end(mixgcn_ctx* ctx, mixgcn_recording** o
     cudaError_t e = cudaStreamEndCapture(ctx->record_stream, &graph);
     if (e == cudaSuccess && graph) e = cudaGraphInstantiate(&r->exec, graph, 0);
     if (graph) cudaGraphDestroy(graph);
-    if (e != cudaSuccess || !r->exec || ctx->blocks_generation != r->before.blocks_generation) {
+    if (e != cudaSuccess || !r->exec || ctx->blocks_generation != r->before.blocks_generation || !r->uses_complete || !r->memory_stands()) {
         cudaGetLastError();
         if (r->exec) cudaGraphExecDestroy(r->exec);
         delete r;
-        MIXGCN_FAIL(MIXGCN_ECUDA, "record_end: the calls could not be recorded (%s)", e == cudaSuccess ? "scratch was reallocated" : cudaGetErrorString(e));
+        MIXGCN_FAIL(MIXGCN_ECUDA, "record_end: the calls could not be recorded (%s)", e == cudaSuccess ? "memory they use was reallocated" : cudaGetErrorString(e));
     }
     *out = r;
     return MIXGCN_OK;
@@ -470,6 +502,7 @@ extern "C" mixgcn_status mixgcn_replay(mixgcn_recording* r, void* stream) {
     const CtxState now(ctx);
     if (ctx->profile || now.blocks_generation != r->before.blocks_generation || memcmp(now.options, r->before.options, sizeof(now.options)) != 0)
         MIXGCN_FAIL(MIXGCN_EUNSUPPORTED, "replay: scratch or options of the context have changed, or profiling is on");
+    if (!r->memory_stands()) MIXGCN_FAIL(MIXGCN_EUNSUPPORTED, "replay: a graph or row plan of the recorded calls has been destroyed or has replaced its schedules");
     MIXGCN_CUDA(cudaSetDevice(ctx->device));
     MIXGCN_CUDA(cudaGraphLaunch(r->exec, (cudaStream_t)stream));
     const CtxState& c = r->counted;
@@ -801,6 +834,7 @@ extern "C" mixgcn_status mixgcn_layer_bwd(mixgcn_ctx* ctx, const mixgcn_graph* g
     if (const mixgcn_rowplan* plan = d->gout_plan) {
         // Row plan: dense products on the plan's compacted rows, aggregation on its restricted matrix.
         if (plan->ctx != ctx || plan->g != g || !plan->transposed) MIXGCN_FAIL(MIXGCN_EINVAL, "layer_bwd: gout_plan must be a plan of this graph's transposed orientation");
+        recording_uses(ctx, plan->memory);
         const int64_t cnt = plan->in_count;
         const int64_t lda = (d->d_in + 3) / 4 * 4, ldb = (d->d_out + 3) / 4 * 4;
         auto up = [](int64_t x) { return (x + 255) & ~(int64_t)255; };

@@ -513,6 +513,7 @@ mixgcn_status ensure_chunk_schedules(const mixgcn_graph* g, const CsrView& A_con
 
 extern "C" mixgcn_status mixgcn_graph_destroy(mixgcn_graph* g) {
     if (!g) return MIXGCN_OK;
+    memory_given_back(g->memory);
     cudaSetDevice(g->device);
     cudaDeviceSynchronize();          // launches that read the graph may still be in flight on any stream
     if (!g->bwd_is_fwd) free_view(g->bwd);
@@ -538,6 +539,7 @@ extern "C" mixgcn_status mixgcn_graph_create(mixgcn_ctx* ctx, int64_t n, int64_t
     g->ctx = ctx; g->device = ctx->device; g->n = n; g->nnz = 0; g->symmetric = 1; g->bwd_is_fwd = 1;
     g->norm = (flags & MIXGCN_GRAPH_NORM_ROW) ? 1 : ((flags & MIXGCN_GRAPH_NORM_NONE) ? 2 : 0);
     struct Guard { mixgcn_graph* g; bool keep = false; ~Guard() { if (!keep) { g->bwd_is_fwd = g->bwd.rowptr == g->fwd.rowptr; mixgcn_graph_destroy(g); } } } guard{g};
+    MIXGCN_TRY(new_generation(&g->memory));
     LaunchScope scope(ctx, PH_GRAPH, s, 12);
 
     DevBuf dsrc(s), ddst(s);
@@ -580,6 +582,7 @@ extern "C" mixgcn_status mixgcn_graph_create_from_csr(mixgcn_ctx* ctx, int64_t n
     g->ctx = ctx; g->device = ctx->device; g->n = n; g->nnz = nnz; g->symmetric = 1; g->bwd_is_fwd = 1;
     g->norm = (flags & MIXGCN_GRAPH_NORM_ROW) ? 1 : ((flags & MIXGCN_GRAPH_NORM_NONE) ? 2 : 0);
     struct Guard { mixgcn_graph* g; bool keep = false; ~Guard() { if (!keep) { g->bwd_is_fwd = g->bwd.rowptr == g->fwd.rowptr; mixgcn_graph_destroy(g); } } } guard{g};
+    MIXGCN_TRY(new_generation(&g->memory));
     LaunchScope scope(ctx, PH_GRAPH, s, 8);
     DevBuf fl(s);
     MIXGCN_TRY(fl.alloc(sizeof(int32_t)));

@@ -4,6 +4,9 @@
 #include <stdint.h>
 #include <stdio.h>
 
+#include <atomic>
+#include <memory>
+
 #include "mixgcn.h"
 
 namespace mixgcn {
@@ -66,6 +69,13 @@ struct ProfSpan {
     cudaEvent_t a, b;
     int phase;
 };
+
+// Counts how often an object has given back device memory that launches take pointers into: a graph whose chunk schedules
+// were replaced, a graph or a row plan destroyed.  A recording keeps the counters of the objects its calls used, past
+// the objects' own lives, and no longer stands for the calls once one of them has moved.
+using MemoryGeneration = std::shared_ptr<std::atomic<uint64_t>>;
+mixgcn_status new_generation(MemoryGeneration* out);
+inline void memory_given_back(const MemoryGeneration& m) { if (m) m->fetch_add(1); }
 
 }  // namespace mixgcn
 
@@ -156,6 +166,7 @@ struct CsrView {
 struct mixgcn_graph {
     mixgcn_ctx* ctx;
     uint64_t uid;      // unique per created graph (a freed graph's address may be reused)
+    mixgcn::MemoryGeneration memory;
     int device;        // kept apart from ctx: a graph may be destroyed after its context
     int64_t n, nnz;
     int symmetric;     // the stored STRUCTURE is symmetric
@@ -174,6 +185,7 @@ struct mixgcn_rowplan {
     mixgcn_ctx* ctx;
     int device;          // kept apart from ctx: a plan may be destroyed after its context
     const mixgcn_graph* g;
+    mixgcn::MemoryGeneration memory;
     int transposed;
     int64_t n, in_count, out_count, nnz;   // nnz: entries of the restricted matrix
     int32_t* idx;        // [in_count] kept input rows, ascending
@@ -210,6 +222,9 @@ struct LaunchScope {
     LaunchScope(mixgcn_ctx* c, int phase, cudaStream_t s, int n_launches = 1);
     ~LaunchScope();
 };
+
+// Notes, while a recording is being made, that it holds pointers into an object's device memory.
+void recording_uses(mixgcn_ctx* ctx, const MemoryGeneration& memory);
 
 // Device memory of the library comes from one pool per device (see api.cu).  The block is usable on stream `s` at
 // once, on other streams after a synchronisation.  dev_free: everything that uses the block must have been enqueued on

@@ -73,6 +73,7 @@ __global__ void kept_fill_kernel(int64_t n, const int64_t* __restrict__ rowptr, 
 
 extern "C" mixgcn_status mixgcn_rowplan_destroy(mixgcn_rowplan* p) {
     if (!p) return MIXGCN_OK;
+    memory_given_back(p->memory);
     cudaSetDevice(p->device);
     cudaDeviceSynchronize();
     dev_free(p->idx, nullptr);
@@ -97,6 +98,7 @@ extern "C" mixgcn_status mixgcn_rowplan_create(mixgcn_ctx* ctx, const mixgcn_gra
     if (!p) MIXGCN_FAIL(MIXGCN_ENOMEM, "rowplan_create: host allocation failed");
     p->ctx = ctx; p->device = ctx->device; p->g = g; p->transposed = transposed ? 1 : 0; p->n = n;
     struct Guard { mixgcn_rowplan* p; ~Guard() { if (p) mixgcn_rowplan_destroy(p); } } guard{p};
+    MIXGCN_TRY(new_generation(&p->memory));
 
     // kept rows, ascending, and their positions
     DevBuf sel(s), tmp(s), pos(s), cnt(s);
@@ -193,6 +195,7 @@ extern "C" mixgcn_status mixgcn_spmm_rowplan(mixgcn_ctx* ctx, const mixgcn_rowpl
     if (epi && epi->residual && (epi->ld_residual < w || epi->residual == Z)) MIXGCN_FAIL(MIXGCN_EINVAL, "spmm_rowplan: residual needs ld_residual >= w and must not be the output");
     if (epi && epi->residual && rows_only) MIXGCN_FAIL(MIXGCN_EUNSUPPORTED, "spmm_rowplan: rows_only cannot be combined with a residual (rows without a kept entry are not zero then)");
     MIXGCN_CUDA(cudaSetDevice(ctx->device));
+    recording_uses(ctx, p->memory);
     // rows of the restricted matrix are scheduled longest first, so its non-empty rows are the first out_count
     SpmmOpts opts;
     opts.phase = PH_SPMM_SPARSE;

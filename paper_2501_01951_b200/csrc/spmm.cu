@@ -1082,6 +1082,7 @@ mixgcn_status launch_spmm(mixgcn_ctx* ctx, const mixgcn_graph* g, const CsrView&
         MIXGCN_TRY(ensure_chunk_schedules(g, A, chunks));
         if (k < 0 || k >= A.n_chunk) MIXGCN_FAIL(MIXGCN_EINVAL, "spmm: chunk %d of %d does not exist", k, chunks);
     }
+    recording_uses(ctx, g->memory);
     const SpmmSchedule& S = chunks > 1 ? A.chunk[k] : A.full;
     if (S.n_rows <= 0) return MIXGCN_OK;
     SpmmParams p{};

@@ -17,9 +17,9 @@ def mg():
     return binding
 
 
-def trainer(mg, precision, **kw):
+def trainer(mg, precision, dims=(40, 24, 24, 9), **kw):
     from paper_2501_01951_b200.train import GcnTrainer
-    n, dims = 3000, (40, 24, 24, 9)
+    n = 3000
     s, d = synth.rmat_graph(n, 20000, 5)
     ctx = mg.ctx_create(0)
     g = mg.graph_create(ctx, n, s, d)
@@ -52,6 +52,54 @@ def test_replayed_iterations_are_the_calls(mg, precision, kw):
     assert torch.equal(a[2].X[-1], b[2].X[-1])
     for ctx, _, _ in (a, b):
         assert mg.ctx_poll_status(ctx, raise_on_error=False) == 0
+
+
+def replays_like_calls(a, b, ts):
+    """Iterations of trainer `a` through epoch(), of its twin `b` call by call: the same bits."""
+    for t in ts:
+        a.epoch(t)
+        b._iteration()
+        b.step(t)
+    for x, y in zip(a.W + a.b + a.dW + a.mW + [a.loss, a.pred], b.W + b.b + b.dW + b.mW + [b.loss, b.pred]):
+        assert torch.equal(x, y)
+    assert a._replays["iteration"].rec is not None
+
+
+@pytest.mark.parametrize("dims", [(64, 24, 24, 9), (64, 24, 9), (16, 24, 9)])     # first layer updates first, or aggregates first
+@pytest.mark.parametrize("change", ["inputs", "row_sparse"])
+def test_recording_ends_with_the_row_plans_it_used(mg, dims, change):
+    """Row plans made anew may lie where the old ones lay, under an equal key."""
+    a, b = trainer(mg, mg.PREC_FP32, dims=dims, row_sparse=1)[2], trainer(mg, mg.PREC_FP32, dims=dims, row_sparse=1)[2]
+    replays_like_calls(a, b, range(1, 5))
+    perm = torch.randperm(a.n, generator=torch.Generator().manual_seed(8)).cuda()
+    for k in range(3):
+        for tr in (a, b):
+            tr.train_mask.copy_(tr.train_mask[perm])              # other nodes, as many, in the same buffers
+            if change == "inputs":
+                tr.set_inputs(tr.X[0], tr.labels, tr.train_mask)
+            else:
+                tr.configure(row_sparse=1)
+        replays_like_calls(a, b, range(5 + 4 * k, 9 + 4 * k))
+    for tr in (a, b):
+        assert mg.ctx_poll_status(tr.ctx, raise_on_error=False) == 0
+
+
+@pytest.mark.parametrize("gone", ["plan", "graph"])
+def test_replay_is_refused_once_a_graph_or_plan_is_gone(mg, gone):
+    ctx, g, tr = trainer(mg, mg.PREC_FP32)
+    plan = mg.rowplan_create(ctx, g, tr.train_mask)
+    Y, Z = torch.ones((plan.in_count, 8), device="cuda"), torch.zeros((g.n, 8), device="cuda")
+    calls = (lambda: mg.spmm_rowplan(ctx, plan, Y, Z, 8)) if gone == "plan" else (lambda: mg.spmm(ctx, g, tr.X[0], tr.saved[0], 8))
+    bits = torch.zeros((g.n, 1), dtype=torch.int32, device="cuda")
+    calls()
+    rec, other = mg.record(ctx, calls), mg.record(ctx, lambda: mg.mask_pack(ctx, 8, bits, X=Z))
+    assert rec.replay() and other.replay()
+    plan.close()
+    if gone == "graph":
+        g.close()
+    assert not rec.replay() and other.replay()
+    torch.cuda.synchronize()
+    assert mg.ctx_poll_status(ctx, raise_on_error=False) == 0
 
 
 def test_launches_are_counted_and_profiling_sees_every_kernel(mg):

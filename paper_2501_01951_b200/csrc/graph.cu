@@ -488,6 +488,7 @@ mixgcn_status ensure_chunk_schedules(const mixgcn_graph* g, const CsrView& A_con
     CsrView& A = const_cast<CsrView&>(g->bwd_is_fwd ? g->fwd : A_const);
     if (chunks <= 1 || A.n_chunk == chunks) return MIXGCN_OK;
     MIXGCN_CUDA(cudaDeviceSynchronize());         // earlier launches may still read the schedules being replaced
+    if (A.n_chunk) memory_given_back(g->memory);  // recorded ones too
     for (int k = 0; k < A.n_chunk; ++k) free_schedule(A.chunk[k]);
     delete[] A.chunk;
     A.chunk = nullptr; A.n_chunk = 0;

@@ -84,6 +84,23 @@ def test_recording_ends_with_the_row_plans_it_used(mg, dims, change):
         assert mg.ctx_poll_status(tr.ctx, raise_on_error=False) == 0
 
 
+def test_recording_ends_with_the_chunk_schedules_it_used(mg):
+    """Two trainers share a graph and cut its rows into different numbers of chunks: each one's calls replace the other's schedules."""
+    ctx, g, a = trainer(mg, mg.PREC_FP32, n_chunks=3)
+    b, twin = trainer(mg, mg.PREC_FP32, n_chunks=3)[2], trainer(mg, mg.PREC_FP32, n_chunks=5)[2]
+    other = type(a)(ctx, g, a.dims, mg.PREC_FP32, n_chunks=5)
+    other.set_params(twin.W, twin.b)
+    other.set_inputs(a.X[0], a.labels, a.train_mask)
+    replays_like_calls(a, b, range(1, 5))
+    rec = a._replays["iteration"].rec
+    replays_like_calls(other, twin, range(1, 5))
+    assert not rec.replay()
+    replays_like_calls(a, b, range(5, 9))
+    assert a._replays["iteration"].rec is not rec
+    torch.cuda.synchronize()
+    assert mg.ctx_poll_status(ctx, raise_on_error=False) == 0
+
+
 @pytest.mark.parametrize("gone", ["plan", "graph"])
 def test_replay_is_refused_once_a_graph_or_plan_is_gone(mg, gone):
     ctx, g, tr = trainer(mg, mg.PREC_FP32)

@@ -288,6 +288,10 @@ mixgcn_status mixgcn_mask_pack(mixgcn_ctx* ctx, int64_t n, int32_t w, const floa
 #define MIXGCN_PREC_TF32 1 /* tensor cores, TF32 operands, fp32 accumulate */
 #define MIXGCN_PREC_BF16 2 /* tensor cores, BF16 operands (the fp32 operands rounded to nearest even),
                               fp32 accumulate, fp32 results */
+#define MIXGCN_PREC_FP32_FMA 3 /* mixgcn_gemm only: as FP32, on the CUDA cores at every size.  For a product that a ReLU is
+                              taken of later (after an aggregation, say): sums in another order change the signs of
+                              results within a rounding error of zero, and the gates of the backward pass with them.
+                              FP32 does so by itself under the epilogue's own relu, and so do the layer calls. */
 
 /* Dense update GEMM  C = op(A) op(B)  with fp32 storage (Algorithm 2, update line, and its
  * two backward products).  op(A) is M x K, op(B) is K x N, C is M x N row-major with ldc.

@@ -31,6 +31,7 @@ OK, EINVAL, ENOMEM, ECUDA, EUNSUPPORTED, EBADGRAPH, ETIMEOUT, EDEVICE = range(8)
 GRAPH_SYMMETRISE, GRAPH_ADD_SELF_LOOPS, GRAPH_EDGES_ON_DEVICE = 1, 2, 4
 GRAPH_NORM_ROW, GRAPH_NORM_NONE = 8, 16
 PREC_FP32, PREC_TF32, PREC_BF16 = 0, 1, 2
+PREC_FP32_FMA = 3          # gemm only
 ORDER_AUTO, ORDER_AGG_FIRST, ORDER_UPD_FIRST = 0, 1, 2
 LAYER_RELU, LAYER_FIRST, LAYER_GATE_GIN, LAYER_GOUT_GATED, LAYER_OUT_ROWS_ONLY, LAYER_GIN_ROWS_ONLY = 1, 2, 4, 8, 16, 32
 LAYER_SAVED_IS_VALID = 64

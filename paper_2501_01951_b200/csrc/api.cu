@@ -528,7 +528,7 @@ extern "C" mixgcn_status mixgcn_gemm(mixgcn_ctx* ctx, int32_t precision, int32_t
                                      const mixgcn_epilogue* epi, void* stream) {
     if (!ctx || !A || !B || !C) MIXGCN_FAIL(MIXGCN_EINVAL, "gemm: null argument");
     if (M <= 0 || N <= 0 || K <= 0) MIXGCN_FAIL(MIXGCN_EINVAL, "gemm: M, N, K must be positive");
-    if (precision < MIXGCN_PREC_FP32 || precision > MIXGCN_PREC_BF16) MIXGCN_FAIL(MIXGCN_EINVAL, "gemm: unknown precision %d", precision);
+    if (precision < MIXGCN_PREC_FP32 || precision > MIXGCN_PREC_FP32_FMA) MIXGCN_FAIL(MIXGCN_EINVAL, "gemm: unknown precision %d", precision);
     const int64_t min_lda = trans_a ? M : K, min_ldb = trans_b ? K : N;
     if (lda < min_lda || ldb < min_ldb || ldc < N)
         MIXGCN_FAIL(MIXGCN_EINVAL, "gemm: leading dimensions must cover the matrix (lda=%lld ldb=%lld ldc=%lld)",
@@ -538,7 +538,10 @@ extern "C" mixgcn_status mixgcn_gemm(mixgcn_ctx* ctx, int32_t precision, int32_t
     if (epi && ((epi->gate_bits && epi->ld_gate_bits < (N + 31) / 32) || (epi->sign_bits && epi->ld_sign_bits < (N + 31) / 32)))
         MIXGCN_FAIL(MIXGCN_EINVAL, "gemm: a bit-packed mask needs ld >= ceil(N / 32) words");
     MIXGCN_CUDA(cudaSetDevice(ctx->device));
-    return launch_gemm(ctx, precision, trans_a, trans_b, M, N, K, A, lda, B, ldb, C, ldc, epi, 0, (cudaStream_t)stream);
+    GemmLP lp;
+    lp.relu_follows = precision == MIXGCN_PREC_FP32_FMA;
+    if (lp.relu_follows) precision = MIXGCN_PREC_FP32;
+    return launch_gemm(ctx, precision, trans_a, trans_b, M, N, K, A, lda, B, ldb, C, ldc, epi, 0, (cudaStream_t)stream, &lp);
 }
 
 extern "C" mixgcn_status mixgcn_weight_grad(mixgcn_ctx* ctx, int32_t precision, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda,
@@ -678,8 +681,9 @@ extern "C" mixgcn_status mixgcn_layer_fwd(mixgcn_ctx* ctx, const mixgcn_graph* g
             MIXGCN_TRY(launch_scatter_rows(ctx, n, cnt, d->d_out, rs.idx, rs.b, ldb, X_out, d->ld_out, s));
             return MIXGCN_OK;
         }
+        GemmLP glp; glp.relu_follows = epi.relu != 0;
         MIXGCN_TRY(launch_gemm(ctx, d->precision, 0, 0, n, d->d_out, d->d_in, X_in, d->ld_in, W, ldw, saved, d->ld_saved,
-                               nullptr, 0, s));
+                               nullptr, 0, s, &glp));
         MIXGCN_TRY(launch_spmm(ctx, g, g->fwd, 1, 0, d->d_out, saved, d->ld_saved, X_out, d->ld_out, &epi, s, filter_rows));
         return MIXGCN_OK;
     }

@@ -36,6 +36,12 @@ def update_first(d_in: int, d_out: int, first: bool, precision: int, relu: bool)
     return 2 * d_out < (1 if first else 2) * d_in
 
 
+def product_precision(precision: int, relu: bool) -> int:
+    """Precision of an update-first product: where a ReLU is taken of what the aggregation makes of it, fp32 sums keep the one
+    order that GCN layers keep under a ReLU, and signs near zero with it."""
+    return mg.PREC_FP32_FMA if relu and precision == mg.PREC_FP32 else precision
+
+
 class _Base:
     def __init__(self, ctx, graph, dims, precision):
         self.ctx, self.g, self.precision = ctx, graph, precision
@@ -147,7 +153,7 @@ class SageTrainer(_Base):
                 for stacked, beside in self._halves(l, self.params[l], self.Wc[l]):
                     beside.copy_(stacked)
                 P = self.pool[0].view(-1)[: self.n * self.wide[l]].view(self.n, self.wide[l])
-                mg.gemm(self.ctx, self.precision, False, False, self.n, self.wide[l], self.dims[l], S, self.Wc[l], P)
+                mg.gemm(self.ctx, product_precision(self.precision, relu), False, False, self.n, self.wide[l], self.dims[l], S, self.Wc[l], P)
                 mg.spmm(self.ctx, self.g, P[:, do4:], out, dout, epi=mg.make_epilogue(residual=P[:, :do4], residual_scale=1.0, bias=bias, relu=relu))
             else:
                 mg.spmm(self.ctx, self.g, S[:, :d], S[:, d:], self.dims[l])
@@ -216,7 +222,7 @@ class GinTrainer(_Base):
         for l in range(L):
             H, d = self.H[l], self.dims[l]
             if self.upd[l]:
-                mg.gemm(self.ctx, self.precision, False, False, self.n, h, d, H, self.params[l], self.U)
+                mg.gemm(self.ctx, product_precision(self.precision, True), False, False, self.n, h, d, H, self.params[l], self.U)
                 mg.spmm(self.ctx, self.g, self.U, self.T[l], h, epi=mg.make_epilogue(residual=self.U, residual_scale=keep, bias=self.params[L + l], relu=True))
             else:
                 mg.spmm(self.ctx, self.g, H, self.Z[l], d, epi=mg.make_epilogue(residual=H, residual_scale=keep))

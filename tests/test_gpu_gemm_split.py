@@ -110,3 +110,47 @@ def test_column_sums(mg, ctx, M, N, K):
     mg.weight_grad(ctx, mg.PREC_FP32, M, N, K, device(A, up(M)), device(B, up(N)), C, sums)
     assert error(C[:, :N], A.double().T @ B.double()) <= TOL_FP32
     assert (sums[:N].double() - B.double().sum(0)).abs().max() <= 1e-6 * B.double().abs().sum(0).max() and sums[N] == 5.0
+
+
+def test_products_under_a_later_relu_keep_the_order_of_sums(mg, ctx):
+    """Where a ReLU follows the aggregation of a product, every way to that product gives the FMA kernel's bits: GraphSAGE and GIN
+    layers, a GCN layer, and its form on some rows only.  (The size is one the tensor cores take otherwise.)"""
+    from paper_2501_01951_b200.sage_gin import GinTrainer, SageTrainer
+    n, d, h = 20003, 300, 60
+    g = mg.graph_create(ctx, n, *synth.rmat_graph(n, 60000, 41), mg.GRAPH_SYMMETRISE | mg.GRAPH_NORM_ROW)
+    X = device(synth.uniform_tensor((n, d), 42, -1, 1), up(d)).nan_to_num()
+    W = synth.uniform_tensor((d, h), 43, -1, 1).cuda()
+    wide = torch.cat([W, -0.5 * W], 1).contiguous()
+    fma = [torch.zeros(n, k, device="cuda") for k in (h, 2 * h)]
+    for B, C in zip((W, wide), fma):
+        mg.gemm(ctx, mg.PREC_FP32_FMA, False, False, n, C.shape[1], d, X, B, C)
+        assert torch.equal(C, product(mg, ctx, X, B, False, False, aligned=False))
+        assert not torch.equal(C, product(mg, ctx, X, B, False, False))
+    y, m = synth.uniform_labels(n, 5, 44).cuda(), synth.bernoulli_mask(n, 0.3, 45).cuda()
+    zero = [torch.zeros(h), torch.zeros(5)]
+
+    want = torch.zeros(n, h, device="cuda")
+    mg.spmm(ctx, g, fma[1][:, h:], want, h, epi=mg.make_epilogue(residual=fma[1][:, :h], residual_scale=1.0, relu=True))
+    tr = SageTrainer(ctx, g, (d, h, 5), mg.PREC_FP32)
+    tr.set_params([W, torch.zeros(h, 5)], [-0.5 * W, torch.zeros(h, 5)], zero)
+    tr.set_inputs(X, y, m)
+    tr.forward()
+    assert tr.upd[0] and torch.equal(tr.S[1][:, :h], want)
+
+    mg.spmm(ctx, g, fma[0], want, h, epi=mg.make_epilogue(residual=fma[0], residual_scale=1.25, relu=True))
+    tr = GinTrainer(ctx, g, (d, 5), h, mg.PREC_FP32, gin_eps=0.25)
+    tr.set_params([W], zero[:1], [torch.zeros(h, 5)], zero[1:])
+    tr.set_inputs(X, y, m)
+    tr.forward()
+    assert tr.upd[0] and torch.equal(tr.T[0], want)
+
+    mg.spmm(ctx, g, fma[0], want, h, epi=mg.make_epilogue(relu=True))
+    desc = mg.layer_desc(d, h, up(d), h, h, mg.ORDER_UPD_FIRST, mg.PREC_FP32, mg.LAYER_RELU | mg.LAYER_FIRST)
+    saved, out = torch.zeros(n, h, device="cuda"), torch.zeros(n, h, device="cuda")
+    mg.layer_fwd(ctx, g, desc, X, W, None, None, saved, out)
+    assert torch.equal(out, want)
+    desc.flags |= mg.LAYER_OUT_ROWS_ONLY
+    desc.gout_row_mask, desc.gout_row_count = m.data_ptr(), int(m.sum())
+    mg.layer_fwd(ctx, g, desc, X, W, None, None, saved, out.fill_(-1.0))
+    rows = m.bool()
+    assert torch.equal(out[rows], want[rows]) and torch.all(out[~rows] == -1.0)

@@ -79,18 +79,20 @@ mixgcn_status pool_contexts(int device, int change) {
     cudaMemPool_t pool;
     MIXGCN_TRY(pool_of(device, &pool));
     DevicePool& d = g_pools[device];
-    const int before = d.contexts;
-    d.contexts += change;
-    if ((before == 0) != (d.contexts == 0)) {
+    const int after = d.contexts + change;
+    if ((d.contexts == 0) != (after == 0)) {
         uint64_t keep = 0;
-        if (d.contexts) {
+        if (after) {
             size_t free_bytes = 0, total_bytes = 0;
             MIXGCN_CUDA(cudaMemGetInfo(&free_bytes, &total_bytes));
             keep = total_bytes / 32;
+        } else {
+            d.contexts = 0;               // gone whatever the calls below say
         }
         MIXGCN_CUDA(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
-        if (!d.contexts) MIXGCN_CUDA(cudaMemPoolTrimTo(pool, 0));
+        if (!after) MIXGCN_CUDA(cudaMemPoolTrimTo(pool, 0));
     }
+    d.contexts = after;
     return MIXGCN_OK;
 }
 }  // namespace
@@ -253,6 +255,7 @@ extern "C" mixgcn_status mixgcn_ctx_create(mixgcn_ctx** out, int device) {
     if (device >= MAX_DEVICES) { delete c; MIXGCN_FAIL(MIXGCN_EUNSUPPORTED, "ctx_create: device index %d not supported", device); }
     const mixgcn_status pool_st = pool_contexts(device, +1);
     if (pool_st != MIXGCN_OK) { delete c; return pool_st; }
+    struct Guard { mixgcn_ctx* c; ~Guard() { if (c) mixgcn_ctx_destroy(c); } } guard{c};     // what a failure below leaves half made
     c->sm_count = prop.multiProcessorCount;
     MIXGCN_CUDA(cudaMalloc((void**)&c->d_status, STATUS_WORDS * sizeof(int32_t)));
     MIXGCN_CUDA(cudaMemset(c->d_status, 0, STATUS_WORDS * sizeof(int32_t)));
@@ -260,6 +263,7 @@ extern "C" mixgcn_status mixgcn_ctx_create(mixgcn_ctx** out, int device) {
     MIXGCN_CUDA(cudaEventCreateWithFlags(&c->fork_ev, cudaEventDisableTiming));
     for (int i = 0; i < 2; ++i) MIXGCN_CUDA(cudaEventCreateWithFlags(&c->join_ev[i], cudaEventDisableTiming));
     for (int i = 0; i < 64; ++i) MIXGCN_CUDA(cudaEventCreateWithFlags(&c->chunk_ev[i], cudaEventDisableTiming));
+    guard.c = nullptr;
     *out = c;
     return MIXGCN_OK;
 }

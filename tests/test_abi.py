@@ -87,6 +87,21 @@ def test_null_arguments_are_rejected_without_a_device(mg):
     assert b"null" in mg.lib.mixgcn_last_error()
 
 
+def test_a_context_that_cannot_be_made_leaves_nothing_behind(tmp_path):
+    """Every CUDA call of mixgcn_ctx_create made to fail in turn, by a stand-in for the runtime (see the source beside this file)."""
+    import subprocess
+    from paper_2501_01951_b200 import build as b
+    exe = tmp_path / "ctx_create_failures"
+    cmd = ["g++", "-std=c++17", "-O1", "-x", "c++", "api.cu", os.path.join(ROOT, "tests", "ctx_create_failures.cpp"), "-x", "none",
+           "-I", ".", "-I", b.INCLUDE, "-I", os.path.join(os.path.dirname(os.path.dirname(b.NVCC)), "include"), "-o", str(exe),
+           "-Wl,--unresolved-symbols=ignore-all"]          # what api.cu calls in the other sources is not reached
+    r = subprocess.run(cmd, capture_output=True, text=True, cwd=b.CSRC)
+    assert r.returncode == 0, r.stderr[-2000:]
+    r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, r.stdout
+    assert int(r.stdout.split()[0]) > 70                   # streams, events, memory: all of them were tried
+
+
 def test_hot_aggregation_kernels_compile_without_register_spills(tmp_path):
     """The aggregation kernels that carry the epochs run under a register cap (four CTAs of 256 threads per SM);
     a spill there costs several per cent of an epoch, and nothing else would notice it: ask the assembler."""

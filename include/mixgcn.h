@@ -99,9 +99,10 @@ mixgcn_status mixgcn_debug_poke_col(mixgcn_graph* g, int64_t entry, int32_t valu
 /* Test hooks of the bounded device-side waits (the failure-detection path), both 0 by default.
  * MIXGCN_OPT_DEBUG_WAIT_LIMIT: > 0 = number of polls after which a wait inside the tensor-core kernels
  * gives up (default about four million).  MIXGCN_OPT_DEBUG_DROP_LOAD: 1 = the next tensor-core products
- * in the K-major form leave the first stage of every CTA unfilled, so that the wait on it runs out: the
- * kernel records code 3 in the status word, frees its tensor memory and returns with C undefined;
- * mixgcn_ctx_poll_status then gives MIXGCN_ETIMEOUT.  Nothing traps, spins without limit or faults. */
+ * in the K-major form, and those of fp32 operands in three parts in both forms, leave the first stage of every CTA
+ * unfilled, so that the wait on it runs out: the kernel records code 3 in the status word, frees its tensor memory and
+ * returns with C undefined; mixgcn_ctx_poll_status then gives MIXGCN_ETIMEOUT.  2 = the same, and BF16 products of fp32
+ * rows may be converted on the way in (with 1 they go through a bf16 copy).  Nothing traps, spins without limit or faults. */
 #define MIXGCN_OPT_DEBUG_WAIT_LIMIT 3
 #define MIXGCN_OPT_DEBUG_DROP_LOAD 4
 /* MIXGCN_OPT_GEMM_CTA_PAIRS: 1 (default) = wide and deep K-major products (N >= 512, K >= 512, M >= 4096)

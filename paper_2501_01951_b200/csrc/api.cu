@@ -359,7 +359,7 @@ extern "C" mixgcn_status mixgcn_ctx_set_option(mixgcn_ctx* ctx, int32_t option, 
         return MIXGCN_OK;
     }
     if (option == MIXGCN_OPT_DEBUG_DROP_LOAD) {
-        if (value != 0 && value != 1) MIXGCN_FAIL(MIXGCN_EINVAL, "ctx_set_option: drop-load takes 0 or 1 (got %lld)", (long long)value);
+        if (value < 0 || value > 2) MIXGCN_FAIL(MIXGCN_EINVAL, "ctx_set_option: drop-load takes 0, 1 or 2 (got %lld)", (long long)value);
         ctx->debug_drop_load = (int)value;
         return MIXGCN_OK;
     }

@@ -65,6 +65,7 @@ struct SplitParams {
     TcEpi epi;
     int32_t* status;
     uint32_t wait_limit;
+    int drop_load;                // test hook: every CTA's first raw tile is left out (the wait for it then expires)
     int32_t* overflow;            // set when an operand cannot be split
 };
 
@@ -280,7 +281,8 @@ __device__ __forceinline__ void load_kk(const SplitParams& p, Shared& bars, cons
         if (a_tile >= tiles) return true;
         if (!raw_free(raw, bars, p)) return false;
         mbar_expect_tx(&bars.raw_full[raw.bar()], RAW_BYTES);
-        tma_load_2d(raws + (size_t)raw.slot * RAW_BYTES, &map_a, a_ks * BK, (int32_t)((uint32_t)a_tile / (uint32_t)p.n_tiles) * BM, &bars.raw_full[raw.bar()]);
+        if (!(p.drop_load && raw.unit == 0))
+            tma_load_2d(raws + (size_t)raw.slot * RAW_BYTES, &map_a, a_ks * BK, (int32_t)((uint32_t)a_tile / (uint32_t)p.n_tiles) * BM, &bars.raw_full[raw.bar()]);
         raw.next(p.raw_slots);
         if (++a_ks == nk) { a_ks = 0; a_tile += gridDim.x; }
         return true;
@@ -551,6 +553,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
                 if (!raw_free(raw, bars, p)) break;
                 const int32_t k = (int32_t)(kb + (int64_t)(u >> 1) * BK);
                 mbar_expect_tx(&bars.raw_full[raw.bar()], u & 1 ? (uint32_t)bw * BK * 4 : (uint32_t)RAW_BYTES);
+                if (p.drop_load && u == 0) continue;
                 tma_load_2d(raws + (size_t)raw.slot * RAW_BYTES, u & 1 ? &map_b : &map_a, (int32_t)(u & 1 ? n0 : m0), k, &bars.raw_full[raw.bar()]);
             }
         }
@@ -737,6 +740,7 @@ mixgcn_status launch_gemm_split(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int6
     p.epi = make_tc_epi(epi, epi_row0);
     p.status = ctx->d_status;
     p.wait_limit = ctx->debug_wait_limit > 0 ? (uint32_t)ctx->debug_wait_limit : WAIT_LIMIT_DEFAULT;
+    p.drop_load = ctx->debug_drop_load;
     p.overflow = ctx->d_status + SPLIT_OVERFLOW_WORD;
     *overflow_flag = p.overflow;
     if (!ta) {
@@ -814,7 +818,7 @@ mixgcn_status launch_gemm_cvt(mixgcn_ctx* ctx, int tb, int64_t M, int64_t N, int
     if (M <= 0 || N <= 0 || K <= 0 || N > (int64_t)CVT_COLS || M >= (1ll << 31) || K >= (1ll << 31) || !aligned16(A) || (lda & 3)) return MIXGCN_EUNSUPPORTED;
     // few tiles with many stages each: the bf16 kernel's longer stages win over the pass (4 K x 256 x 2048: 49 us here, 37 there)
     if (M <= (int64_t)BM * (ctx->sm_count - 1) && K > 512) return MIXGCN_EUNSUPPORTED;
-    if (ctx->debug_drop_load) return MIXGCN_EUNSUPPORTED;
+    if (ctx->debug_drop_load == 1) return MIXGCN_EUNSUPPORTED;        // the hook is meant for the bf16 kernel then
     auto ceil_div = [](int64_t a, int64_t b) { return (a + b - 1) / b; };
     SplitParams p{};
     p.M = M; p.N = N; p.K = K; p.C = C; p.ldc = ldc;
@@ -823,6 +827,7 @@ mixgcn_status launch_gemm_cvt(mixgcn_ctx* ctx, int tb, int64_t M, int64_t N, int
     p.epi = make_tc_epi(epi, epi_row0);
     p.status = ctx->d_status;
     p.wait_limit = ctx->debug_wait_limit > 0 ? (uint32_t)ctx->debug_wait_limit : WAIT_LIMIT_DEFAULT;
+    p.drop_load = ctx->debug_drop_load;
     const int bn32 = (p.bn + 31) & ~31, kpad = (int)(ceil_div(K, BK) * BK);
     MIXGCN_TRY(ensure_workspace(ctx, (int64_t)bn32 * kpad * 2));
     uint16_t* packed = reinterpret_cast<uint16_t*>(ctx->workspace);

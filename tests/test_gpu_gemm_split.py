@@ -154,3 +154,28 @@ def test_products_under_a_later_relu_keep_the_order_of_sums(mg, ctx):
     mg.layer_fwd(ctx, g, desc, X, W, None, None, saved, out.fill_(-1.0))
     rows = m.bool()
     assert torch.equal(out[rows], want[rows]) and torch.all(out[~rows] == -1.0)
+
+
+@pytest.mark.parametrize("precision,M,N,K,ta", [(0, 30001, 161, 97, False), (0, 128, 65, 50000, True), (2, 30001, 161, 97, False)])
+def test_a_wait_that_runs_out_is_reported(mg, precision, M, N, K, ta):
+    """The kernels that cut or convert fp32 operands, with the first load of every CTA left out and a short limit: the wait gives
+    up, the status says so, and the products after it on the same context are right."""
+    ctx = mg.ctx_create(0)
+    A, B = (t.bfloat16().float() if precision == 2 else t for t in operands(M, N, K, ta, False))
+    want = (A.T if ta else A).double() @ B.double()
+    C = torch.zeros(M, up(N), device="cuda")
+    call = lambda: mg.gemm(ctx, precision, ta, False, M, N, K, device(A, up(A.shape[1])), device(B, up(B.shape[1])), C)
+    for _ in range(2):
+        mg.ctx_set_option(ctx, mg.OPT_DEBUG_WAIT_LIMIT, 2000)
+        mg.ctx_set_option(ctx, mg.OPT_DEBUG_DROP_LOAD, 2)
+        call()
+        assert mg.ctx_poll_status(ctx, raise_on_error=False) == 3
+        mg.ctx_set_option(ctx, mg.OPT_DEBUG_DROP_LOAD, 0)
+        mg.ctx_set_option(ctx, mg.OPT_DEBUG_WAIT_LIMIT, 0)
+        for _ in range(2):
+            C.fill_(7.0)
+            call()
+            assert error(C[:, :N], want) <= TOL_FP32
+    assert mg.ctx_poll_status(ctx, raise_on_error=False) == 0
+    assert mg.ctx_gemm_paths(ctx)["tc_bf16"] == (6 if precision == 2 else 0)
+    ctx.close()

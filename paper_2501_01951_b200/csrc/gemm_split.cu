@@ -5,19 +5,33 @@
 // fp32 rounding, and not all of one sign.  The split of matrices into parts that multiply without error is that of Ozaki,
 // Ogita, Oishi and Rump ("Error-free transformations of matrix multiplication", 2012).
 //
-// What the tensor core does not do is round its accumulator to nearest: it cuts it off, once per instruction, so that an error
-// grows with the number of instructions on one accumulator.  Two things keep these products as accurate as the fp32 FMA
-// kernel (the same operands against fp64, of both signs and positive, in the tests):
-//  * the large products a0 b0 are accumulated over 32 terms only (two instructions); the epilogue warps then add the
-//    accumulator to fp32 sums in registers, rounding to nearest, while the next 32 terms go to a second accumulator;
-//  * the five small products, at most 2^-8 of the large ones, have an accumulator of their own for up to 1024 terms.
+// What the tensor core does not do is round to nearest.  An instruction aligns its 16 products and the accumulator to the
+// largest of them, cuts each off 25 bits below it, towards zero, adds exactly and cuts the sum off at 24 bits (so its
+// results say: bf16 operands of one instruction against fp64).  What is cut off does not average out; these things keep it small:
+//  * the large products a0 b0 are accumulated over few terms only; the epilogue warps add the accumulator to fp32 sums in
+//    registers, rounding to nearest, while the next terms go to a second accumulator;
+//  * the five small products, at most 2^-7 of the large ones, have an accumulator of their own.
+// K-major: 32 terms (two instructions) an accumulator, one chain of sums, at most 1024 terms.  Against fp64 its results are closer
+// than the FMA kernel's single chain on everything a layer multiplies (activations, features and gradients by weights: 0.2 to
+// 0.8 of its error).
+// Weight gradient: its operands cancel -- most entries of a column of a softmax gradient are small and of one sign, a few are large
+// and of the other -- and the small terms beside a large one are what is cut off.  So it accumulates 16 terms (one instruction)
+// at a time; the first part of A keeps seven bits, which makes products of 15 that lose nothing down to 2^-10 of the
+// largest (the three parts still hold all 24 bits; the parts left out grow to 2^-22 at most, 2^-26 in the mean, of either
+// sign); and every 512 terms the sums go to a second sum in TMEM, the rounding error of that addition going on into the next sums.
+// ReLU activations or 0 / 1 features by softmax gradients, error against the FMA kernel's: 256 x 40 over 170 K rows 0.43 to 0.97
+// of it, 128 x 80 over 524 K 0.28 to 0.79; where it comes out above (up to 1.2, with 1 to 10 % of the rows labelled) both are below one
+// rounding of the result, 2^-24.  (With 32 terms, eight bits and one chain it was up to 1.47 of it, for 156 us instead of 174 at 170 K x 256 x 256.)
+// Operands of one sign, which training does not multiply, may come out at up to 1.8 of the FMA kernel's error, near one rounding.
 //
 // Bound: the hand-overs between the roles.  A stage of 32 terms of a 128 x 128 tile is twelve instructions, 768 cycles of the
 // tensor core, and takes about 1,800: raw tile, conversion, MMA and epilogue follow one another, with the three stages of part
 // tiles in flight that shared memory holds.  Tensor pipe 43 to 45 % active (of 270 TFLOP/s of fp32 products; the FMA pipes
 // have 72), shared-memory banks 40 %, issue slots 40 to 55 %.
-// Measured against the FMA kernel: 170 K x 256 x 256 forward 508 -> 178 us (126 TFLOP/s), its weight gradient 466 -> 163,
-// 170 K x 40 x 256 145 -> 79, 1 M x 300 x 300 4493 -> 1590.
+// Measured against the FMA kernel, calls back to back: 170 K x 256 x 256 forward 501 -> 162 us (138 TFLOP/s), its weight
+// gradient 464 -> 174, 170 K x 40 x 256 144 -> 77, 1 M x 300 x 300 4494 -> 1482.
+// Behind every such product runs the FMA kernel's grid, which reads one zero word per block and returns (see the overflow
+// below): 1 M x 300 x 300 has 23 thousand blocks of it.
 //
 // What the layout of the work has to avoid is the latency of one stage's hand-overs in series (a wait, a proxy fence and an
 // arrival each): one group of conversion warps on every stage took 212 us where two groups on alternate stages take 178;
@@ -46,8 +60,13 @@ constexpr int EPI_WARPS = 8, CONV_WARPS = 8, TMA_WARP = EPI_WARPS + CONV_WARPS, 
 constexpr int GROUPS = 2, GROUP_WARPS = CONV_WARPS / GROUPS, GROUP_THREADS = GROUP_WARPS * 32;   // groups of conversion warps, on alternate stages
 constexpr int STAGES_MAX = 4, RAW_MAX = 8;      // most stages of part tiles and slots of raw fp32 tiles (a multiple of 2 * GROUPS)
 static_assert(RAW_MAX % (2 * GROUPS) == 0);
-constexpr int HI_STAGES = 32 / BK, LO_STAGES = 1024 / BK;           // stages per accumulator of the large and of the small products
-constexpr uint32_t TMEM_COLS = 512, LO_COL = 256, BUF_COLS = 128;   // two accumulators for the large products, two for the small ones
+// How a form adds up.  HI: accumulators of the large products per stage.  LO: stages per accumulator of the small products.
+// LEVELS: 1: the sums stay in registers to the end; 2: every LO stages they are carried over to a second sum in TMEM.
+// TRIM_A: 1: the first part of A keeps seven bits instead of eight.
+struct KkSums { static constexpr int HI = 1, LO = 1024 / BK, LEVELS = 1, TRIM_A = 0; };
+struct MmSums { static constexpr int HI = 2, LO = 512 / BK, LEVELS = 2, TRIM_A = 1; };
+constexpr uint32_t TMEM_COLS = 512, BUF_COLS = 128;     // two accumulators for the large products, then
+constexpr uint32_t LO_COL = 256, SUM_COL = 384;         // two for the small ones, or one and the second sum
 constexpr uint32_t CVT_COLS = 256;              // the two accumulators of the bf16 form
 constexpr int RAW_BYTES = BM * BK * 4, KK_PART = BM * BK * 2;       // a raw tile; K-major part tiles: 64-byte rows and swizzle
 constexpr int CHUNK = BK * 128, MM_PART = BM / 64 * CHUNK;          // MN-major tiles: chunks of 64 columns, 128-byte k-rows and swizzle
@@ -97,10 +116,15 @@ __device__ __forceinline__ void sub_parts(float& x, float& y, uint32_t parts) {
 
 // Four floats at `src` -> their three bf16 parts at dst + t * part_bytes.  top: per half the largest |first part| met, infinity
 // when a value cannot be split (a NaN needs no note, its first part is one).
+template <int TRIM>
 __device__ __forceinline__ void split4(float4 v, uint8_t* dst, uint32_t part_bytes, uint32_t& top) {
 #pragma unroll
     for (int t = 0; t < PARTS; ++t) {
-        const uint32_t lo = pack_bf16(v.x, v.y), hi = pack_bf16(v.z, v.w);
+        uint32_t lo = pack_bf16(v.x, v.y), hi = pack_bf16(v.z, v.w);
+        if (TRIM && t == 0) {            // to seven bits, away from zero (a NaN is lost here and comes back in the parts behind)
+            lo = (lo + 0x00010001u) & 0xFFFEFFFEu;
+            hi = (hi + 0x00010001u) & 0xFFFEFFFEu;
+        }
         *reinterpret_cast<uint2*>(dst + t * part_bytes) = make_uint2(lo, hi);
         if (t == 0) {
             asm("{.reg .b32 a; abs.bf16x2 a, %1; max.bf16x2 %0, %0, a;}" : "+r"(top) : "r"(lo));
@@ -193,11 +217,38 @@ __device__ __forceinline__ void add_accumulator(uint32_t taddr, int chunks, floa
         }
 }
 
+// The sums in registers to the second sum in TMEM, s; what its rounding leaves of them stays behind (the error of a sum is the
+// difference of two sums: Knuth, The Art of Computer Programming, 4.2.2), so that the second level adds no error of its own.
+__device__ __forceinline__ void carry_over(uint32_t taddr, int chunks, bool first, float (&acc)[2][32]) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        if (k < chunks) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const uint32_t at = taddr + (uint32_t)(k * 32 + h * 16);
+                uint32_t r[16];
+                if (!first) {
+                    tc_ld16(at, r);
+                    tc_wait_ld();
+                }
+#pragma unroll
+                for (int q = 0; q < 16; ++q) {
+                    const float a = acc[k][h * 16 + q], s = first ? 0.0f : __uint_as_float(r[q]);
+                    const float t = __fadd_rn(s, a), b = __fsub_rn(t, s);
+                    acc[k][h * 16 + q] = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(a, b));
+                    r[q] = __float_as_uint(t);
+                }
+                tc_st16(at, r);
+            }
+        }
+    tc_wait_st();
+}
+
 // The MMA warp's state: position in the stages and in the two pairs of accumulators.
 struct MmaState {
     Ring stage;
     uint32_t hc = 0, lc = 0;
-    int hi_used = 0, lo_used = 0; // stages in the current accumulators
+    int lo_used = 0;              // stages in the current accumulator of the small products
 };
 
 // One lane of a converged warp, always the same one.
@@ -210,15 +261,19 @@ __device__ __forceinline__ bool elect_one() {
 // All products of one stage, by the whole MMA warp: uniform control flow up to the elected lane leaves the descriptors in uniform
 // registers.  desc_a, desc_b: descriptors of the first part tiles, the others a_part and b_part bytes on, the second 16
 // terms k_step bytes on (the address is the descriptor's low field, in units of 16 bytes).  last: no stage of this tile follows.
+template <class Sums>
 __device__ __forceinline__ bool mma_stage(MmaState& st, Shared& b, const SplitParams& p, uint32_t tmem, uint32_t idesc, bool last, uint64_t desc_a, uint64_t desc_b,
                                           uint32_t a_part, uint32_t b_part, uint32_t k_step) {
     if (!warp_wait(&b.full[st.stage.i], st.stage.use, b, p)) return false;
-    if (st.lo_used == 0 && !warp_wait(&b.lo_empty[st.lc & 1], ((st.lc >> 1) & 1) ^ 1, b, p)) return false;
+    constexpr int HI = Sums::HI;
+    constexpr uint32_t LO_BUFS = Sums::LEVELS == 1 ? 2 : 1;
+    const uint32_t lb = st.lc % LO_BUFS;
+    if (st.lo_used == 0 && !warp_wait(&b.lo_empty[lb], ((st.lc / LO_BUFS) & 1) ^ 1, b, p)) return false;
     tc_fence_after();
     auto da = [&](int part, int k16) { return desc_a + ((part * a_part + k16 * k_step) >> 4); };
     auto db = [&](int part, int k16) { return desc_b + ((part * b_part + k16 * k_step) >> 4); };
-    const uint32_t hi = tmem + (st.hc & 1) * BUF_COLS, lo = tmem + LO_COL + (st.lc & 1) * BUF_COLS;
-    const bool hi_ends = st.hi_used + 1 == HI_STAGES || last, lo_ends = st.lo_used + 1 == LO_STAGES || last;
+    const uint32_t lo = tmem + LO_COL + lb * BUF_COLS;
+    const bool lo_ends = st.lo_used + 1 == Sums::LO || last;
     if (elect_one()) {
         constexpr int PA[5] = {0, 1, 1, 0, 2}, PB[5] = {1, 0, 1, 2, 0};
 #pragma unroll
@@ -228,19 +283,23 @@ __device__ __forceinline__ bool mma_stage(MmaState& st, Shared& b, const SplitPa
         }
     }
     __syncwarp();
-    if (st.hi_used == 0 && !warp_wait(&b.hi_empty[st.hc & 1], ((st.hc >> 1) & 1) ^ 1, b, p)) return false;
-    tc_fence_after();
-    if (elect_one()) {
-        tc_mma<KIND_BF16>(hi, da(0, 0), db(0, 0), idesc, st.hi_used ? 1u : 0u);
-        tc_mma<KIND_BF16>(hi, da(0, 1), db(0, 1), idesc, 1u);
-        if (hi_ends) tc_commit(&b.hi_full[st.hc & 1]);
-        tc_commit(&b.empty[st.stage.i]);
-        if (lo_ends) tc_commit(&b.lo_full[st.lc & 1]);
+#pragma unroll
+    for (int h = 0; h < HI; ++h, ++st.hc) {
+        if (!warp_wait(&b.hi_empty[st.hc & 1], ((st.hc >> 1) & 1) ^ 1, b, p)) return false;
+        tc_fence_after();
+        if (elect_one()) {
+            const uint32_t hi = tmem + (st.hc & 1) * BUF_COLS;
+            tc_mma<KIND_BF16>(hi, da(0, h), db(0, h), idesc, 0u);
+            if (HI == 1) tc_mma<KIND_BF16>(hi, da(0, 1), db(0, 1), idesc, 1u);
+            tc_commit(&b.hi_full[st.hc & 1]);
+            if (h + 1 == HI) {
+                tc_commit(&b.empty[st.stage.i]);
+                if (lo_ends) tc_commit(&b.lo_full[lb]);
+            }
+        }
+        __syncwarp();
     }
-    __syncwarp();
-    st.hi_used = hi_ends ? 0 : st.hi_used + 1;
     st.lo_used = lo_ends ? 0 : st.lo_used + 1;
-    st.hc += hi_ends;
     st.lc += lo_ends;
     st.stage.next(p.stages);
     return true;
@@ -248,14 +307,17 @@ __device__ __forceinline__ bool mma_stage(MmaState& st, Shared& b, const SplitPa
 
 // An epilogue warp's sums of one tile over nk stages.  t_row: TMEM address of its lanes and first column.
 struct EpiState { uint32_t hc = 0, lc = 0; };
+template <class Sums>
 __device__ __forceinline__ bool sum_tile(EpiState& st, Shared& b, const SplitParams& p, uint32_t t_row, int chunks, int nk, int lane, float (&acc)[2][32]) {
-    auto take = [&](uint64_t* full, uint64_t* empty, uint32_t& c, uint32_t col) {
-        if (!warp_wait(&full[c & 1], (c >> 1) & 1, b, p)) return false;
+    constexpr uint32_t LO_BUFS = Sums::LEVELS == 1 ? 2 : 1;
+    auto take = [&](uint64_t* full, uint64_t* empty, uint32_t& c, uint32_t bufs, uint32_t col) {
+        const uint32_t i = c % bufs;
+        if (!warp_wait(&full[i], (c / bufs) & 1, b, p)) return false;
         tc_fence_after();
-        add_accumulator(t_row + col + (c & 1) * BUF_COLS, chunks, acc);
+        add_accumulator(t_row + col + i * BUF_COLS, chunks, acc);
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&empty[c & 1]);
+        if (lane == 0) mbar_arrive(&empty[i]);
         ++c;
         return true;
     };
@@ -263,11 +325,20 @@ __device__ __forceinline__ bool sum_tile(EpiState& st, Shared& b, const SplitPar
     for (int k = 0; k < 2; ++k)
 #pragma unroll
         for (int q = 0; q < 32; ++q) acc[k][q] = 0.0f;
-    for (int ks = HI_STAGES;; ks += HI_STAGES) {
-        if (!take(b.hi_full, b.hi_empty, st.hc, 0)) return false;
-        if ((ks % LO_STAGES == 0 || ks >= nk) && !take(b.lo_full, b.lo_empty, st.lc, LO_COL)) return false;
-        if (ks >= nk) return true;
+    bool second = false;                                    // the second sum holds something
+    for (int ks = 1;; ++ks) {
+#pragma unroll
+        for (int h = 0; h < Sums::HI; ++h)
+            if (!take(b.hi_full, b.hi_empty, st.hc, 2, 0)) return false;
+        if ((ks % Sums::LO == 0 || ks >= nk) && !take(b.lo_full, b.lo_empty, st.lc, LO_BUFS, LO_COL)) return false;
+        if (ks >= nk) break;
+        if (Sums::LEVELS == 2 && ks % Sums::LO == 0) {
+            carry_over(t_row + SUM_COL, chunks, !second, acc);
+            second = true;
+        }
     }
+    if (Sums::LEVELS == 2 && second) add_accumulator(t_row + SUM_COL, chunks, acc);
+    return true;
 }
 
 // The loads of a K-major kernel, by one thread: the raw tiles of A run raw_slots - 1 stages ahead of the planes of B.
@@ -377,7 +448,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_kk_kernel(const __grid_
             if (masks && chunks) mask_words(p.epi, m0 + quarter * 32, p.M, p.N, n0 + c_first, 32, n0 + (p.bn < c_first + span ? p.bn : c_first + span), lane, dw, gw);
             prefetch_masks(p, tile + gridDim.x, tiles, quarter * 32 + lane, c_first, span);
             float acc[2][32];
-            if (!sum_tile(st, bars, p, t_row, chunks, nk, lane, acc)) break;
+            if (!sum_tile<KkSums>(st, bars, p, t_row, chunks, nk, lane, acc)) break;
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 if (k >= chunks) break;
@@ -410,7 +481,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_kk_kernel(const __grid_
             if (!warp_wait(&bars.empty[stage.i], stage.use ^ 1, bars, p)) break;
             uint8_t* dst = smem + (size_t)stage.i * stage_bytes + at;
 #pragma unroll
-            for (int it = 0; it < RAW_ITS; ++it) split4(v[it], dst + it * 16 * 64, KK_PART, top);
+            for (int it = 0; it < RAW_ITS; ++it) split4<KkSums::TRIM_A>(v[it], dst + it * 16 * 64, KK_PART, top);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars.full[stage.i]);
@@ -427,7 +498,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_kk_kernel(const __grid_
         for (int64_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x)
             for (int ks = 0; ks < nk && ok; ++ks) {
                 const uint32_t sa = smem_u32(smem + (size_t)st.stage.i * stage_bytes), sb = sa + PARTS * KK_PART;
-                ok = mma_stage(st, bars, p, tmem, idesc, ks + 1 == nk, make_desc(sa, 16, 512, 4), make_desc(sb, 16, 512, 4), KK_PART, b_part, 32);
+                ok = mma_stage<KkSums>(st, bars, p, tmem, idesc, ks + 1 == nk, make_desc(sa, 16, 512, 4), make_desc(sb, 16, 512, 4), KK_PART, b_part, 32);
             }
     }
     cta_end(bars, warp, tmem);
@@ -449,12 +520,13 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
     const uint32_t tmem = cta_begin(bars, GROUP_WARPS, warp);
 
     if (warp < EPI_WARPS) {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 128;");       // as in the K-major form
         const int quarter = warp & 3, half = warp >> 2;
         const int span = p.bn > 64 ? 64 : 32, c_first = half * span;
         const int chunks = p.bn <= c_first ? 0 : (p.bn - c_first > 32 && span == 64) ? 2 : 1;
         EpiState st;
         float acc[2][32];
-        const bool ok = sum_tile(st, bars, p, tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c_first, chunks, nk, lane, acc);
+        const bool ok = sum_tile<MmSums>(st, bars, p, tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c_first, chunks, nk, lane, acc);
         const int64_t m = m0 + quarter * 32 + lane;
         if (ok && m < p.M) {
             float* row = p.C + (p.raw ? (int64_t)blockIdx.z * p.M * p.N : 0) + m * p.ldc;
@@ -476,6 +548,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
             }
         }
     } else if (warp < TMA_WARP) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
         // Conversion: thread t of a group takes the float4 t + 128 it.  Of a tile of 128 columns that is k-row it * 4 + t / 32, of
         // one of 64 k-row it * 8 + t / 16; the swizzle goes by k-row mod 8.
         const int t = (threadIdx.x - EPI_WARPS * 32) % GROUP_THREADS, group = (warp - EPI_WARPS) / GROUP_WARPS;
@@ -504,7 +577,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
             if (!warp_wait(&bars.empty[stage.i], stage.use ^ 1, bars, p)) break;
             uint8_t* dst = smem + (size_t)stage.i * stage_bytes;
 #pragma unroll
-            for (int it = 0; it < RAW_ITS; ++it) split4(v[it], dst + (at_a ^ (it & 1) * 64) + it * 4 * 128, MM_PART, top);
+            for (int it = 0; it < RAW_ITS; ++it) split4<MmSums::TRIM_A>(v[it], dst + (at_a ^ (it & 1) * 64) + it * 4 * 128, MM_PART, top);
             if (!warp_wait(&bars.raw_full[raw.bar()], raw.use(), bars, p)) break;
             dst += PARTS * MM_PART;
             if (turn == (int)p.m_tiles) turn = 0;
@@ -515,7 +588,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
                 if (lane == 0) mbar_arrive(&bars.raw_empty[raw.bar()]);
                 if (sums) add_columns(v, RAW_ITS);
 #pragma unroll
-                for (int it = 0; it < RAW_ITS; ++it) split4(v[it], dst + (at_a ^ (it & 1) * 64) + it * 4 * 128, b_part, top);
+                for (int it = 0; it < RAW_ITS; ++it) split4<0>(v[it], dst + (at_a ^ (it & 1) * 64) + it * 4 * 128, b_part, top);
             } else {
                 float4 w[RAW_ITS / 2];
                 take_raw(w, raws + (size_t)raw.slot * RAW_BYTES, t);
@@ -523,7 +596,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
                 if (lane == 0) mbar_arrive(&bars.raw_empty[raw.bar()]);
                 if (sums) add_columns(w, RAW_ITS / 2);
 #pragma unroll
-                for (int it = 0; it < RAW_ITS / 2; ++it) split4(w[it], dst + at_b + it * 8 * 128, b_part, top);
+                for (int it = 0; it < RAW_ITS / 2; ++it) split4<0>(w[it], dst + at_b + it * 8 * 128, b_part, top);
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
@@ -562,7 +635,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
         MmaState st;
         for (int ks = 0; ks < nk; ++ks) {
             const uint32_t sa = smem_u32(smem + (size_t)st.stage.i * stage_bytes), sb = sa + PARTS * MM_PART;
-            if (!mma_stage(st, bars, p, tmem, idesc, ks + 1 == nk, make_desc(sa, CHUNK, 1024, 2), make_desc(sb, CHUNK, 1024, 2), MM_PART, b_part, 2048)) break;
+            if (!mma_stage<MmSums>(st, bars, p, tmem, idesc, ks + 1 == nk, make_desc(sa, CHUNK, 1024, 2), make_desc(sb, CHUNK, 1024, 2), MM_PART, b_part, 2048)) break;
         }
     }
     cta_end(bars, warp, tmem);
@@ -691,14 +764,20 @@ __global__ void pack_split_kernel(const float* __restrict__ src, int64_t ld, int
 
 namespace mixgcn {
 
-// Whether a product is faster here than on the FMA pipes, by what both take (us, from measurements):
-//  * here 12 for packing, launches and the tail, and 0.75 per stage and 1.2 per tile of the longest CTA (weight gradient: 16 and
-//    0.85 per stage): a wave that is nearly empty counts in full.  20 K x 32 x 500 is two waves of sixteen stages, 35.5 us
-//    against 33.4 there; 20 K x 64 x 500, as long here, 37 : 73; 5 K x 128 x 256 20.8 : 25.6; 52 K x 80 x 80 22.9 : 39.7;
-//    876 K x 8 x 210 266 : 359; weight gradients 64 x 16 x 200 K 49 : 37, 40 x 40 x 200 K 51 : 85, 80 x 80 x 52 K 27 : 47;
-//  * there 20 TFLOP/s and more, with columns padded to 32, and 2 TB/s (876 K x 210 x 8: 392 : 558).
+// Whether a product is faster here than on the FMA pipes, by what both take (us, from measurements; both sides in brackets, here
+// first, calls back to back):
+//  * here 12 for packing, launches and the tail, and 0.75 per stage and 1.2 per tile of the longest CTA: a wave that is nearly
+//    empty counts in full.  20 K x 32 x 500 is two waves of sixteen stages (40 : 35, left there, and 5 K x 128 x 256, 24 : 27);
+//    20 K x 64 x 500, as long here, 42 : 74; 52 K x 80 x 80 27 : 41; 876 K x 8 x 210 277 : 361; 876 K x 210 x 8 339 : 556;
+//  * there 20 TFLOP/s and more, with columns padded to 32, and 2 TB/s;
+//  * weight gradients here 16 and 0.85 per stage.  A stage takes 1.0, but the FMA kernel's narrow tiles do not reach 20 TFLOP/s
+//    either, so the line lies about right: 64 x 16 x 200 K 58 : 40, 128 x 128 x 5 K 29 : 21, 128 x 128 x 10 K 30 : 28 and
+//    64 x 64 x 20 K 25 : 27 are left there, 40 x 40 x 200 K 60 : 89, 80 x 80 x 52 K 33 : 47 and 64 x 47 x 400 K 102 : 162 taken
+//    (33 x 63 x 200 K, 63 : 89, is not).
 // Below 4 columns (and, untried, 32 rows of a weight gradient) padding takes it all.  The K-major form adds up one fp32 chain of
 // K / 32 sums, which past 1024 terms of one sign is less accurate than the two levels of the FMA kernel (1.2e-7 : 5e-8 at 2048).
+// (Which kernel a product takes depends on its rows: the same row may be rounded differently in a compacted, a chunked and a whole
+// product.)
 static bool split_pays(const mixgcn_ctx* ctx, int ta, int64_t M, int64_t N, int64_t K) {
     if (N < 4 || (ta ? M < 32 : K > 1024)) return false;
     auto ceil_div = [](int64_t a, int64_t b) { return (a + b - 1) / b; };

@@ -179,3 +179,58 @@ def test_a_wait_that_runs_out_is_reported(mg, precision, M, N, K, ta):
     assert mg.ctx_poll_status(ctx, raise_on_error=False) == 0
     assert mg.ctx_gemm_paths(ctx)["tc_bf16"] == (6 if precision == 2 else 0)
     ctx.close()
+
+
+def training_operands(kind, K, M, N):
+    """A (K x M) and B (K x N) of a weight gradient: activations or bag-of-words features, and the gradient of a softmax loss over
+    N classes (scores of the given spread, a share of the rows labelled) or one gated by a ReLU above it."""
+    gen = torch.Generator(device="cuda").manual_seed(51)
+    normal = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    uniform = lambda *s: torch.rand(s, generator=gen, device="cuda")
+    what, spread, share = kind
+    p = torch.softmax(normal(K, N) * spread, 1)
+    p[torch.arange(K, device="cuda"), torch.randint(0, N, (K,), generator=gen, device="cuda")] -= 1
+    G = p * (uniform(K, 1) < share)
+    if what == "words":
+        return (uniform(K, M) < 0.02).float(), G
+    H = torch.relu(normal(K, M))
+    if what == "dropout":
+        H = H * (uniform(K, M) < 0.5) * 2
+    if what == "hidden":
+        G = (G @ normal(N, N)) * (normal(K, N) > 0)
+    return H, G
+
+
+@pytest.mark.parametrize("kind", [("relu", 0.3, 0.54), ("relu", 4.0, 0.54), ("dropout", 4.0, 0.54), ("hidden", 1.0, 0.54), ("words", 4.0, 0.54), ("relu", 1.0, 0.01)])
+@pytest.mark.parametrize("M,N,K", [(256, 40, 170003), (64, 47, 400000), (300, 172, 50001), (128, 80, 524288)])
+def test_weight_gradients_of_training_lose_nothing(mg, ctx, kind, M, N, K):
+    """No further from fp64 than the FMA kernel, down to one rounding of the result (2^-24).  The operands cancel as those of
+    training do: most entries of a column of the gradient are small and of one sign, a few are large and of the other."""
+    A, B = training_operands(kind, K, M, N)
+    want = A.double().T @ B.double()
+    got = {}
+    for precision in (mg.PREC_FP32, mg.PREC_FP32_FMA):
+        C = torch.zeros(M, up(N), device="cuda")
+        mg.gemm(ctx, precision, True, False, M, N, K, device(A, up(M)), device(B, up(N)), C)
+        got[precision] = C[:, :N]
+    assert not torch.equal(*got.values())                                # the tensor cores did take it
+    assert error(got[mg.PREC_FP32], want) <= max(error(got[mg.PREC_FP32_FMA], want), 2.0**-24)
+
+
+@pytest.mark.parametrize("binades", [4, 10, 20])
+@pytest.mark.parametrize("positive", [False, True])
+@pytest.mark.parametrize("M,N,K,ta", [(20003, 128, 256, False), (30000, 64, 602, False), (256, 256, 100003, True), (128, 40, 50001, True)])
+def test_split_products_of_spread_magnitudes(mg, ctx, binades, positive, M, N, K, ta):
+    """Magnitudes over 2^-b .. 2^b inside every row and column, each element held to its own bound: an instruction of 16 terms cuts
+    its terms off 24 bits below the largest of them (two instructions per accumulator in the K-major form, one in the other),
+    and the fp32 sums behind it round once per accumulator (K / 32; 32 between two of the weight gradient's carries).  Four
+    more for the small products, the parts left out, the sum over splits and the result.  The FMA kernel's own bound is
+    K roundings, or 1024."""
+    gen = torch.Generator(device="cuda").manual_seed(52)
+    draw = lambda *s: ((torch.rand(s, generator=gen, device="cuda") if positive else torch.randn(s, generator=gen, device="cuda"))
+                       * torch.exp2((torch.rand(s, generator=gen, device="cuda") * 2 - 1) * binades))
+    A, B = draw(*((K, M) if ta else (M, K))), draw(K, N)
+    got = product(mg, ctx, A, B, ta, False).double()
+    a, b = (A.T if ta else A).double(), B.double()
+    cuts, sums = (16, 32) if ta else (32, K // 32 + 1)
+    assert torch.all((got - a @ b).abs() <= (cuts + sums + 4) * 2.0**-24 * (a.abs() @ b.abs()))

@@ -143,8 +143,9 @@ mixgcn_status launch_gemm(mixgcn_ctx* ctx, int precision, int ta, int tb, int64_
     // BF16 requests go to the tcgen05 kind::f16 kernels on bf16 copies of the activation operands: the
     // copies a producer already wrote (lp), else copies made here by a conversion kernel.  TF32
     // requests, and BF16 requests whose shape the bf16 kernels do not take, go to the kind::tf32
-    // kernels (at least the requested precision); whatever those do not take, and fp32 requests, use the
-    // FMA kernel.  ctx->gemm_path counts which kernel served each product.
+    // kernels (at least the requested precision); whatever those do not take, and fp32 requests, are fp32
+    // products: three-part splits on the tensor cores where those are faster and no ReLU follows, the FMA kernel
+    // otherwise.  ctx->gemm_path counts which kernel served each product (both fp32 forms under 0).
     uint16_t* c_lp = lp ? lp->C : nullptr;
     const int64_t ldc_lp = lp ? lp->ldc : 0;
     const LossFuse* loss = lp ? lp->loss : nullptr;

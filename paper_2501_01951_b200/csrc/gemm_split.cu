@@ -26,12 +26,12 @@
 //
 // Bound: the hand-overs between the roles.  A stage of 32 terms of a 128 x 128 tile is twelve instructions, 768 cycles of the
 // tensor core, and takes about 1,800: raw tile, conversion, MMA and epilogue follow one another, with the three stages of part
-// tiles in flight that shared memory holds.  Tensor pipe 43 to 45 % active (of 270 TFLOP/s of fp32 products; the FMA pipes
-// have 72), shared-memory banks 40 %, issue slots 40 to 55 %.
+// tiles in flight that shared memory holds.  Tensor pipe 40 to 43 % active (of 270 TFLOP/s of fp32 products; the FMA pipes
+// have 72), shared-memory banks 41 %, issue slots 40 to 54 %.
 // Measured against the FMA kernel, calls back to back: 170 K x 256 x 256 forward 501 -> 162 us (138 TFLOP/s), its weight
 // gradient 464 -> 174, 170 K x 40 x 256 144 -> 77, 1 M x 300 x 300 4494 -> 1482.
 // Behind every such product runs the FMA kernel's grid, which reads one zero word per block and returns (see the overflow
-// below): 1 M x 300 x 300 has 23 thousand blocks of it.
+// below): 5 us at 170 K x 256 x 256, 23 us (39 thousand blocks) at 1 M x 300 x 300, 3 us and 4 of its reduction for a weight gradient.
 //
 // What the layout of the work has to avoid is the latency of one stage's hand-overs in series (a wait, a proxy fence and an
 // arrival each): one group of conversion warps on every stage took 212 us where two groups on alternate stages take 178;
@@ -644,8 +644,9 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
 // ---------------------------------------------------------------- bf16 product of fp32 rows
 // The K-major form with one part: a bf16 product whose fp32 operand comes without a bf16 copy (the features of an inference, mostly).
 // Converted on the way in, it is read once; a pass that wrote the copy first read and wrote it besides.  All K terms go to one
-// accumulator in the order of the bf16 kernel, so the bits are that kernel's on the copy.  Bound: HBM.  700 K x 130 x 301: 377 us
-// with the pass, 236 so.
+// accumulator in the order of the bf16 kernel, so the bits are that kernel's on the copy.  700 K x 130 x 301: 377 us with the
+// pass, 242 so.  Bound: the hand-overs between the roles, as above: DRAM 5.0 TB/s of the 6.5 a copy reaches, tensor pipe 13 % busy,
+// issue slots 25 %; the epilogue spills 64 bytes a thread (96 registers: it has no register split).
 __global__ void __launch_bounds__(THREADS, 1) gemm_cvt_kk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                                                                  const __grid_constant__ CUtensorMap map_c, const SplitParams p, const int tma_store) {
     extern __shared__ uint8_t smem_raw[];

@@ -207,9 +207,13 @@ inline int32_t schedule_seg(int64_t nnz) {
 }
 constexpr int SPMM_HEAVY = 2048;            // long rows above this take a block each when their segments are combined
 // A long row uses 2^k column blocks while it keeps at least this many entries per block.  Finer blocks bring the segments that
-// gather the same rows closer together, which pays while the gathered matrix is larger than the L2 (2.4 M nodes, width 256:
-// 8.15 ms with 64, 8.27 with 128); on smaller graphs longer segments cost fewer partial rows and reductions (233 K nodes,
-// width 41: 1.90 -> 1.73 ms; 400 K nodes, widths 20..64: 4 to 6 % less).
+// gather the same rows closer together in time; coarser ones cost fewer partial rows and reductions.  One schedule serves every
+// width, and the line lies where 256 columns, the widest slice, turn.  R-MAT graphs of mean degree 50, ms with 64 : with 128:
+//   256 columns   400 K nodes 1.324 : 1.296, 800 K 2.46 : 2.42, 1.2 M 3.61 : 3.74, 1.6 M 5.17 : 5.18, 2.4 M 8.00 : 8.08
+//   128 columns   800 K 1.369 : 1.321, 1.2 M 1.943 : 1.880, 2.4 M 4.08 : 3.96
+//   32 columns    800 K 0.671 : 0.623, 1.2 M 0.951 : 0.887, 2.4 M 1.934 : 1.795
+// (233 K nodes of mean degree 500: 256 columns 5.28 : 5.11, 32 columns 1.433 : 1.293).  Narrow aggregations of large graphs pay 3
+// to 8 % for the wide ones' 1 to 4.
 __host__ __device__ inline int schedule_blk_min(int64_t n_cols) { return n_cols > (1 << 20) ? 64 : 128; }
 constexpr int SPMM_MAX_LOG_BLOCKS = 8;      // at most 2^this column blocks per row
 constexpr int SPMM_PACK_DEG[3] = {12, 5, 2};   // rows up to these lengths share a warp 2-, 4-, 8-fold

@@ -33,7 +33,7 @@ using namespace mixgcn;
 constexpr int SPMM_MINB = 4;          // CTAs per SM asked of the compiler for the narrow (VPL <= 2) group kernels
 constexpr int SPMM_FOLD_WMAX = 128;   // widest aggregation the two folds below apply to
 constexpr int SPMM_FOLD_SEG = 2;      // long-row segments at widths <= 128: 16 lanes x 2 float4 per unit (1 would be 32 lanes x 1)
-constexpr int SPMM_FOLD_MED = 2;      // the same for rows of 13..512 entries
+constexpr int SPMM_FOLD_MED = 2;      // the same for rows of 13 entries up to the schedule's segment length (64..512)
 constexpr int SPMM_SHORT_RB = 4;      // rows a warp of the short-row kernel takes at once
 constexpr int SPMM_SHORT_MINB = 5;    // CTAs per SM asked of the compiler for it
 constexpr int SPMM_SHORT_MAXE = 2;    // rows of at most this many entries go to the short-row kernel

@@ -21,6 +21,15 @@ def round8(x: int) -> int:
 
 
 class GcnTrainer:
+    """Buffers and call order of one model on one graph.
+
+    epoch() and forward() replay a recording of their calls once these have come twice with the same buffers: parameters,
+    inputs and dropout masks at the same addresses, the same flags and options.  Contents may change: a loop that draws new
+    dropout masks or takes other features writes them into the tensors it handed over (``copy_``, ``bernoulli_``).  With
+    new tensors in every iteration the calls are issued one by one each time, as without recordings, and looking for a
+    change costs some tens of microseconds besides.  The row-sparse backward is planned for the train mask that set_inputs()
+    saw: call it again when that mask's contents change."""
+
     def __init__(self, ctx: mg.Ctx, graph: mg.Graph, dims, precision=mg.PREC_FP32, order=mg.ORDER_AUTO,
                  n_chunks=0, fuse_gate=True, keep_scale=1.0, device=None, row_sparse="auto",
                  train_rows_only=False, row_plans=True, cache_first_aggregation=False, lp_copies=True, saved_lp_only=True, sign_bitmaps=True):

@@ -102,21 +102,36 @@ def test_a_context_that_cannot_be_made_leaves_nothing_behind(tmp_path):
     assert int(r.stdout.split()[0]) > 70                   # streams, events, memory: all of them were tried
 
 
+def spills(source, tmp_path):
+    """(kernel, bytes of spill stores, of spill loads) of every kernel of one source, as the assembler reports them."""
+    import subprocess
+    from paper_2501_01951_b200 import build as b
+    cmd = [b.NVCC, *b.ARCH, *b.CFLAGS, "-Xptxas", "-v", "-c", source, "-o", str(tmp_path / "out.o")]
+    r = subprocess.run(cmd, capture_output=True, text=True, cwd=b.CSRC)
+    assert r.returncode == 0, r.stderr[-2000:]
+    found = re.findall(r"Compiling entry function '(\S+)'.*?\n.*?\n\s+\d+ bytes stack frame, (\d+) bytes spill stores, (\d+) bytes spill loads", r.stdout + r.stderr)
+    return [(name, int(st), int(ld)) for name, st, ld in found]
+
+
 def test_hot_aggregation_kernels_compile_without_register_spills(tmp_path):
     """The aggregation kernels that carry the epochs run under a register cap (four CTAs of 256 threads per SM);
     a spill there costs several per cent of an epoch, and nothing else would notice it: ask the assembler."""
-    import subprocess
-    from paper_2501_01951_b200 import build as b
-    cmd = [b.NVCC, *b.ARCH, *b.CFLAGS, "-Xptxas", "-v", "-c", "spmm.cu", "-o", str(tmp_path / "spmm.o")]
-    r = subprocess.run(cmd, capture_output=True, text=True, cwd=b.CSRC)
-    assert r.returncode == 0, r.stderr[-2000:]
-    log = r.stdout + r.stderr
-    entries = re.findall(r"Compiling entry function '(\S+)'.*?\n.*?\n\s+\d+ bytes stack frame, (\d+) bytes spill stores, (\d+) bytes spill loads", log)
+    entries = spills("spmm.cu", tmp_path)
     assert len(entries) > 50
-    # every instance of the group kernel but those with the loss epilogue (third template argument 1), the short-row
-    # kernel and the plain combination kernel
-    hot = [(name, int(st), int(ld)) for name, st, ld in entries
-           if re.search(r"spmm_group_kernelILi\d+ELi\d+ELi[023]E", name) or "spmm_short_kernel" in name or "spmm_combine_kernelILb0" in name]
-    assert len(hot) >= 30
-    spilled = [(name, st, ld) for name, st, ld in hot if st or ld]
+    # every instance of the group kernel but those with the loss epilogue (third template argument 1), the whole-warp kernel, the
+    # short-row kernel and the plain combination kernel
+    hot = [e for e in entries if re.search(r"spmm_group_kernelILi\d+ELi\d+ELi[02345]E", e[0]) or "spmm_warp_kernel" in e[0] or "spmm_short_kernel" in e[0]
+           or "spmm_combine_kernelILb0" in e[0]]
+    for name in ("group", "warp", "short", "combine"):
+        assert any(f"spmm_{name}_kernel" in e[0] for e in hot), name
+    assert len(hot) >= 100
+    spilled = [e for e in hot if e[1] or e[2]]
     assert not spilled, spilled
+
+
+def test_split_products_compile_without_register_spills(tmp_path):
+    """The register split of their roles (setmaxnreg) leaves the epilogue room for a tile's sums.  The converting product has none
+    and spills 64 bytes: no more than that."""
+    entries = {re.search(r"\d([a-z_]+_kernel)E", name).group(1): (st, ld) for name, st, ld in spills("gemm_split.cu", tmp_path)}
+    assert entries["gemm_split_kk_kernel"] == (0, 0) and entries["gemm_split_mm_kernel"] == (0, 0)
+    assert entries["gemm_cvt_kk_kernel"][0] <= 64

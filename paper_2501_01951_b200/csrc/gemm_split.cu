@@ -38,8 +38,9 @@
 // loads to registers before the fence instead of raw tiles by TMA, as much; the large products issued before the small ones
 // (the wait for their accumulator in front), 190; issue by a divergent lane instead of an elected one of a converged warp, 10 % more.
 //
-// Infinities and values that round to a bf16 infinity do not survive the split (inf - inf): the converting warps record that
-// they met one, and the FMA kernel, launched behind, then computes the product over again (otherwise it returns at once).
+// Infinities, values that round to a bf16 infinity and sums out of fp32's range do not survive the split (inf - inf): whatever is not
+// finite in an operand or in a sum is a NaN or an infinity in the sums of its row.  The epilogue warps record that they met one,
+// and the FMA kernel, launched behind, then computes the product over again (otherwise it returns at once).
 // A value below 2^-109 keeps an absolute error of up to 2^-134, its last part being a bf16 subnormal.
 //
 //  * K-major form (forward, input gradient): persistent CTAs over 128 x bn tiles; the weights are cut once into three packed
@@ -85,7 +86,7 @@ struct SplitParams {
     int32_t* status;
     uint32_t wait_limit;
     int drop_load;                // test hook: every CTA's first raw tile is left out (the wait for it then expires)
-    int32_t* overflow;            // set when an operand cannot be split
+    int32_t* overflow;            // set when a sum is not finite
 };
 
 struct Ring {                     // position in a ring of slots and the parity of its use
@@ -114,10 +115,9 @@ __device__ __forceinline__ void sub_parts(float& x, float& y, uint32_t parts) {
         : "+f"(x), "+f"(y) : "f"(__uint_as_float(parts << 16)), "f"(__uint_as_float(parts & 0xFFFF0000u)), "f"(-1.0f));
 }
 
-// Four floats at `src` -> their three bf16 parts at dst + t * part_bytes.  top: per half the largest |first part| met, infinity
-// when a value cannot be split (a NaN needs no note, its first part is one).
+// Four floats -> their three bf16 parts at dst + t * part_bytes.
 template <int TRIM>
-__device__ __forceinline__ void split4(float4 v, uint8_t* dst, uint32_t part_bytes, uint32_t& top) {
+__device__ __forceinline__ void split4(float4 v, uint8_t* dst, uint32_t part_bytes) {
 #pragma unroll
     for (int t = 0; t < PARTS; ++t) {
         uint32_t lo = pack_bf16(v.x, v.y), hi = pack_bf16(v.z, v.w);
@@ -126,14 +126,9 @@ __device__ __forceinline__ void split4(float4 v, uint8_t* dst, uint32_t part_byt
             hi = (hi + 0x00010001u) & 0xFFFEFFFEu;
         }
         *reinterpret_cast<uint2*>(dst + t * part_bytes) = make_uint2(lo, hi);
-        if (t == 0) {
-            asm("{.reg .b32 a; abs.bf16x2 a, %1; max.bf16x2 %0, %0, a;}" : "+r"(top) : "r"(lo));
-            asm("{.reg .b32 a; abs.bf16x2 a, %1; max.bf16x2 %0, %0, a;}" : "+r"(top) : "r"(hi));
-        }
         if (t + 1 < PARTS) { sub_parts(v.x, v.y, lo); sub_parts(v.z, v.w, hi); }
     }
 }
-__device__ __forceinline__ bool has_inf(uint32_t top) { return (top & 0x7FFFu) == 0x7F80u || ((top >> 16) & 0x7FFFu) == 0x7F80u; }
 
 // This thread's share of a raw tile: the float4 t, t + 128, ...
 constexpr int RAW_ITS = BM * BK / 4 / GROUP_THREADS;
@@ -242,6 +237,22 @@ __device__ __forceinline__ void carry_over(uint32_t taddr, int chunks, bool firs
             }
         }
     tc_wait_st();
+}
+
+// Whether the sums of this warp's first `cols` columns (a multiple of 16) are all finite: 0 times anything else is NaN.
+__device__ __forceinline__ bool all_finite(const float (&acc)[2][32], int cols) {
+    float x = 0.0f, y = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (k * 32 + h * 16 < cols) {
+#pragma unroll
+                for (int q = h * 16; q < h * 16 + 16; q += 2)
+                    asm("{.reg .b64 p, z, s; mov.b64 p, {%2, %3}; mov.b64 z, {%4, %4}; mov.b64 s, {%0, %1}; fma.rn.f32x2 s, p, z, s; mov.b64 {%0, %1}, s;}"
+                        : "+f"(x), "+f"(y) : "f"(acc[k][q]), "f"(acc[k][q + 1]), "f"(0.0f));
+            }
+    return x + y == 0.0f;
 }
 
 // The MMA warp's state: position in the stages and in the two pairs of accumulators.
@@ -449,6 +460,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_kk_kernel(const __grid_
             prefetch_masks(p, tile + gridDim.x, tiles, quarter * 32 + lane, c_first, span);
             float acc[2][32];
             if (!sum_tile<KkSums>(st, bars, p, t_row, chunks, nk, lane, acc)) break;
+            if (!all_finite(acc, p.bn - c_first)) *p.overflow = 1;
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 if (k >= chunks) break;
@@ -471,7 +483,6 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_kk_kernel(const __grid_
         Ring stage;
         raw.next(p.raw_slots, group);
         stage.next(p.stages, group);
-        uint32_t top = 0;
         for (int64_t st = group; st < stages; st += GROUPS) {
             if (!warp_wait(&bars.raw_full[raw.bar()], raw.use(), bars, p)) break;
             float4 v[RAW_ITS];
@@ -481,14 +492,13 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_kk_kernel(const __grid_
             if (!warp_wait(&bars.empty[stage.i], stage.use ^ 1, bars, p)) break;
             uint8_t* dst = smem + (size_t)stage.i * stage_bytes + at;
 #pragma unroll
-            for (int it = 0; it < RAW_ITS; ++it) split4<KkSums::TRIM_A>(v[it], dst + it * 16 * 64, KK_PART, top);
+            for (int it = 0; it < RAW_ITS; ++it) split4<KkSums::TRIM_A>(v[it], dst + it * 16 * 64, KK_PART);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars.full[stage.i]);
             raw.next(p.raw_slots, GROUPS);
             stage.next(p.stages, GROUPS);
         }
-        if (has_inf(top)) *p.overflow = 1;
     } else if (warp == TMA_WARP) {
         if (lane == 0) load_kk(p, bars, map_a, map_b, smem, raws, stage_bytes, PARTS * KK_PART, b_part, PARTS, nk, tiles);
     } else {
@@ -527,6 +537,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
         EpiState st;
         float acc[2][32];
         const bool ok = sum_tile<MmSums>(st, bars, p, tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c_first, chunks, nk, lane, acc);
+        if (ok && !all_finite(acc, p.bn - c_first)) *p.overflow = 1;
         const int64_t m = m0 + quarter * 32 + lane;
         if (ok && m < p.M) {
             float* row = p.C + (p.raw ? (int64_t)blockIdx.z * p.M * p.N : 0) + m * p.ldc;
@@ -558,7 +569,6 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
         Ring stage;
         raw.next(p.raw_slots, 2 * group);
         stage.next(p.stages, group);
-        uint32_t top = 0;
         float4 v[RAW_ITS];
         // Column sums of B: the rows of tiles take the stages of a group in turn, each thread its own columns of the raw tile.
         const int m_tile = (int)(tile / p.n_tiles);
@@ -577,7 +587,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
             if (!warp_wait(&bars.empty[stage.i], stage.use ^ 1, bars, p)) break;
             uint8_t* dst = smem + (size_t)stage.i * stage_bytes;
 #pragma unroll
-            for (int it = 0; it < RAW_ITS; ++it) split4<MmSums::TRIM_A>(v[it], dst + (at_a ^ (it & 1) * 64) + it * 4 * 128, MM_PART, top);
+            for (int it = 0; it < RAW_ITS; ++it) split4<MmSums::TRIM_A>(v[it], dst + (at_a ^ (it & 1) * 64) + it * 4 * 128, MM_PART);
             if (!warp_wait(&bars.raw_full[raw.bar()], raw.use(), bars, p)) break;
             dst += PARTS * MM_PART;
             if (turn == (int)p.m_tiles) turn = 0;
@@ -588,7 +598,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
                 if (lane == 0) mbar_arrive(&bars.raw_empty[raw.bar()]);
                 if (sums) add_columns(v, RAW_ITS);
 #pragma unroll
-                for (int it = 0; it < RAW_ITS; ++it) split4<0>(v[it], dst + (at_a ^ (it & 1) * 64) + it * 4 * 128, b_part, top);
+                for (int it = 0; it < RAW_ITS; ++it) split4<0>(v[it], dst + (at_a ^ (it & 1) * 64) + it * 4 * 128, b_part);
             } else {
                 float4 w[RAW_ITS / 2];
                 take_raw(w, raws + (size_t)raw.slot * RAW_BYTES, t);
@@ -596,7 +606,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
                 if (lane == 0) mbar_arrive(&bars.raw_empty[raw.bar()]);
                 if (sums) add_columns(w, RAW_ITS / 2);
 #pragma unroll
-                for (int it = 0; it < RAW_ITS / 2; ++it) split4<0>(w[it], dst + at_b + it * 8 * 128, b_part, top);
+                for (int it = 0; it < RAW_ITS / 2; ++it) split4<0>(w[it], dst + at_b + it * 8 * 128, b_part);
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
@@ -618,7 +628,6 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
                 p.colsum_part[((int64_t)blockIdx.z * p.m_tiles + m_tile) * p.N + n0 + all] = s;
             }
         }
-        if (has_inf(top)) *p.overflow = 1;
     } else if (warp == TMA_WARP) {
         if (lane == 0) {
             RawRing raw;
@@ -745,7 +754,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_cvt_kk_kernel(const __grid_co
 // Packed planes of the weight matrix: plane q of dst (rows x kpad bf16) holds part q of trans ? src[k][n] : src[n][k], zeros
 // outside N x K.
 __global__ void pack_split_kernel(const float* __restrict__ src, int64_t ld, int trans, int N, int K, int rows, int kpad, int parts,
-                                  uint16_t* __restrict__ dst, int32_t* overflow) {
+                                  uint16_t* __restrict__ dst) {
     const int64_t plane = (int64_t)rows * kpad, i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= plane) return;
     const int n = trans ? (int)(i % rows) : (int)(i / kpad), k = trans ? (int)(i / rows) : (int)(i % kpad);     // consecutive threads read consecutive words
@@ -755,7 +764,6 @@ __global__ void pack_split_kernel(const float* __restrict__ src, int64_t ld, int
     for (int q = 0; q < PARTS; ++q) {
         if (q >= parts) break;
         const uint32_t b = pack_bf16(v, 0.0f) & 0xFFFFu;
-        if (q == 0 && overflow && (b & 0x7FFFu) == 0x7F80u) *overflow = 1;
         dst[q * plane + (int64_t)n * kpad + k] = (uint16_t)b;
         v -= __uint_as_float(b << 16);
     }
@@ -842,7 +850,7 @@ mixgcn_status launch_gemm_split(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int6
         MIXGCN_CUDA(cudaMemsetAsync(p.overflow, 0, sizeof(int32_t), s));
         {
             LaunchScope scope(ctx, PH_GEMM, s);
-            pack_split_kernel<<<(unsigned)ceil_div((int64_t)rows * kpad, 256), 256, 0, s>>>(B, ldb, tb ? 0 : 1, (int)N, (int)K, rows, kpad, PARTS, planes, p.overflow);
+            pack_split_kernel<<<(unsigned)ceil_div((int64_t)rows * kpad, 256), 256, 0, s>>>(B, ldb, tb ? 0 : 1, (int)N, (int)K, rows, kpad, PARTS, planes);
         }
         LaunchScope scope(ctx, PH_GEMM, s);
         const unsigned grid = (unsigned)(tiles < ctx->sm_count ? tiles : ctx->sm_count);
@@ -923,7 +931,7 @@ mixgcn_status launch_gemm_cvt(mixgcn_ctx* ctx, int tb, int64_t M, int64_t N, int
     MIXGCN_CUDA(cudaFuncSetAttribute(gemm_cvt_kk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     {
         LaunchScope scope(ctx, PH_GEMM, s);
-        pack_split_kernel<<<(unsigned)ceil_div((int64_t)bn32 * kpad, 256), 256, 0, s>>>(B, ldb, tb ? 0 : 1, (int)N, (int)K, bn32, kpad, 1, packed, nullptr);
+        pack_split_kernel<<<(unsigned)ceil_div((int64_t)bn32 * kpad, 256), 256, 0, s>>>(B, ldb, tb ? 0 : 1, (int)N, (int)K, bn32, kpad, 1, packed);
     }
     LaunchScope scope(ctx, PH_GEMM, s);
     const unsigned grid = (unsigned)(p.m_tiles < ctx->sm_count ? p.m_tiles : ctx->sm_count);

@@ -234,3 +234,21 @@ def test_split_products_of_spread_magnitudes(mg, ctx, binades, positive, M, N, K
     a, b = (A.T if ta else A).double(), B.double()
     cuts, sums = (16, 32) if ta else (32, K // 32 + 1)
     assert torch.all((got - a @ b).abs() <= (cuts + sums + 4) * 2.0**-24 * (a.abs() @ b.abs()))
+
+
+@pytest.mark.parametrize("M,N,K,ta", [(25000, 100, 200, False), (25000, 17, 200, False), (200, 100, 25000, True), (200, 17, 200001, True)])
+def test_sums_that_overflow(mg, ctx, M, N, K, ta):
+    """Finite operands whose products or sums leave fp32's range: the infinities (and the NaN of opposite ones) of the FMA kernel."""
+    A, B = operands(M, N, K, ta, False)
+    rows = A.T if ta else A
+    rows[3], rows[5], B[7] = 1e30, 3e37, 1e10                            # of one row of the result a product, of another the sum
+    clean = operands(M, N, K, ta, False)
+    bits = torch.zeros(M, (N + 31) // 32, dtype=torch.int32, device="cuda")
+    epi = {} if ta else {"sign_bits": bits}
+    got, bits_got = product(mg, ctx, A, B, ta, False, **epi), bits.clone()
+    want = product(mg, ctx, A, B, ta, False, aligned=False, **epi)
+    assert want.isinf().any()
+    assert torch.equal(got.isnan(), want.isnan()) and torch.equal(got.isinf(), want.isinf()) and torch.equal(bits_got, bits)
+    ok = want.isfinite()
+    assert torch.equal(got[ok], want[ok])
+    assert error(product(mg, ctx, *clean, ta, False), (clean[0].T if ta else clean[0]).double() @ clean[1].double()) <= TOL_FP32

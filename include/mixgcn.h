@@ -195,6 +195,14 @@ mixgcn_status mixgcn_graph_export(const mixgcn_graph* g, int transposed, int64_t
  * entry count (ties by ascending id). */
 mixgcn_status mixgcn_graph_export_schedule(const mixgcn_graph* g, int transposed, int32_t* perm);
 
+/* Lays the dense corner of the matrix out for the tensor cores: with rows and columns by descending entry counts, every
+ * tile of 128 x 128 that holds enough entries becomes a bitmap, and later aggregations over all rows (mixgcn_spmm and the
+ * layer calls; not sampled, row-sparse, row-filtered or chunked ones) multiply it there, sums in fp32 as before but in
+ * another order.  Costs a few passes over the entries; for a graph that many aggregations will use.  Nothing happens on
+ * graphs without such tiles, or the second time.  n_tiles, n_entries (nullable): tiles, and entries in them, of the
+ * forward orientation.  Synchronises before returning; aggregations already enqueued are not affected. */
+mixgcn_status mixgcn_graph_prepare_tiles(mixgcn_graph* g, int64_t* n_tiles, int64_t* n_entries);
+
 /* A graph may be used only while its context exists; it may be destroyed after it. */
 mixgcn_status mixgcn_graph_destroy(mixgcn_graph* g);
 

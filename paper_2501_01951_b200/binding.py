@@ -45,7 +45,7 @@ SYMBOLS = (
     "mixgcn_status_string", "mixgcn_last_error", "mixgcn_ctx_create", "mixgcn_ctx_destroy",
     "mixgcn_ctx_reserve", "mixgcn_ctx_poll_status", "mixgcn_ctx_profile_enable", "mixgcn_ctx_profile_read",
     "mixgcn_graph_create", "mixgcn_graph_create_from_csr", "mixgcn_graph_info", "mixgcn_graph_export",
-    "mixgcn_graph_export_schedule", "mixgcn_graph_destroy", "mixgcn_spmm", "mixgcn_gemm",
+    "mixgcn_graph_prepare_tiles", "mixgcn_graph_export_schedule", "mixgcn_graph_destroy", "mixgcn_spmm", "mixgcn_gemm",
     "mixgcn_layer_plan", "mixgcn_layer_fwd", "mixgcn_layer_bwd", "mixgcn_loss_softmax_xent",
     "mixgcn_adam_step", "mixgcn_train_step_host", "mixgcn_loss_softmax_xent_noalloc", "mixgcn_ctx_set_option",
     "mixgcn_graph_bandwidth", "mixgcn_graph_rcm", "mixgcn_pipeline_stages", "mixgcn_graph_create_permuted",
@@ -341,6 +341,14 @@ def graph_export_schedule(g: Graph, transposed: bool = False) -> torch.Tensor:
     perm = torch.empty(g.n, dtype=torch.int32)
     _check(lib.mixgcn_graph_export_schedule(g.h, C.c_int(int(transposed)), _ptr(perm)))
     return perm
+
+
+def graph_prepare_tiles(g: Graph) -> tuple[int, int]:
+    """Lay the dense corner of the graph out for the tensor cores -> (tiles, entries in them).  Once per graph; later calls
+    change nothing."""
+    tiles, entries = C.c_int64(0), C.c_int64(0)
+    _check(lib.mixgcn_graph_prepare_tiles(g.h, C.byref(tiles), C.byref(entries)))
+    return tiles.value, entries.value
 
 
 def build_info() -> dict:

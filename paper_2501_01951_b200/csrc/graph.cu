@@ -517,6 +517,7 @@ extern "C" mixgcn_status mixgcn_graph_destroy(mixgcn_graph* g) {
     memory_given_back(g->memory);
     cudaSetDevice(g->device);
     cudaDeviceSynchronize();          // launches that read the graph may still be in flight on any stream
+    release_tiles(g);
     if (!g->bwd_is_fwd) free_view(g->bwd);
     free_view(g->fwd);
     dev_free(g->deg, nullptr);

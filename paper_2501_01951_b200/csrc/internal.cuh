@@ -79,12 +79,12 @@ inline void memory_given_back(const MemoryGeneration& m) { if (m) m->fetch_add(1
 
 }  // namespace mixgcn
 
-constexpr int STATUS_WORDS = 32, SPLIT_OVERFLOW_WORD = 16;
+constexpr int STATUS_WORDS = 32, SPLIT_OVERFLOW_WORD = 16, TILES_UNSAFE_WORD = 17;    // (two words)
 
 struct mixgcn_ctx {
     int device;
     int sm_count;
-    int32_t* d_status;        // device status word (int32[4]); word SPLIT_OVERFLOW_WORD: see gemm_split.cu
+    int32_t* d_status;        // device status word (int32[4]); words SPLIT_OVERFLOW_WORD, TILES_UNSAFE_WORD: see gemm_split.cu, hub_tiles.cu
     void* workspace;          // grow-on-demand scratch of the dense products, column sums and the loss
     int64_t workspace_bytes;
     void* workspace_rows;     // scratch of the row-sparse backward (row list, positions, compact operands)
@@ -105,6 +105,7 @@ struct mixgcn_ctx {
     int no_cta_pairs;         // 1: keep every product on single CTAs (option, for comparison)
     int debug_wait_limit;     // > 0: polls after which the tensor-core kernels' waits give up (test of that path)
     int debug_drop_load;      // 1, 2: tensor-core products leave one stage unfilled (test of that path)
+    int tiles_turn;           // which of the two flags the next product of hub tiles uses
     int spmm_slice_cols;      // 0 = default (one slice up to 1024 columns)
     int loss_train_rows_only; // 1 = the loss skips rows outside the train mask entirely
     // profiling
@@ -176,6 +177,9 @@ struct mixgcn_graph {
     int32_t* deg;      // [n] entries per row of the stored matrix
     float* dinv;       // [n]
     CsrView fwd, bwd;  // bwd aliases fwd when symmetric
+    // tiles of the dense corner of fwd and bwd (the same object where bwd aliases fwd), null where there are none
+    std::atomic<struct HubTiles*> tiles[2];
+    bool tiles_tried;
 };
 
 // Everything about a row-sparse aggregation that depends only on the graph and on WHICH rows of the
@@ -305,6 +309,7 @@ mixgcn_status launch_spmm(mixgcn_ctx* ctx, const mixgcn_graph* g, const CsrView&
 // schedule of all n rows of a view whose column ids lie in [0, n_cols); release of a view's memory
 mixgcn_status build_view_schedule(int64_t n_cols, int64_t n, int64_t nnz, CsrView& v, cudaStream_t s);
 void release_view(CsrView& v);
+void release_tiles(mixgcn_graph* g);
 // colsum_b of launch_gemm (weight-gradient form, trans_a = 1, only): also out[n] = sum_k B[k][n], the bias
 // gradient when B = dP -- produced inside the product's kernel where that kernel reads B as fp32 words,
 // by the column-sum kernels otherwise.

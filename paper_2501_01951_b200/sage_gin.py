@@ -45,6 +45,8 @@ def product_precision(precision: int, relu: bool) -> int:
 class _Base:
     def __init__(self, ctx, graph, dims, precision):
         self.ctx, self.g, self.precision = ctx, graph, precision
+        if precision != mg.PREC_FP32:
+            mg.graph_prepare_tiles(graph)      # as in train.py
         self.dims = tuple(int(d) for d in dims)
         self.L = len(self.dims) - 1
         self.n = graph.n

@@ -52,6 +52,10 @@ class GcnTrainer:
         # the same every epoch); the paper recomputes it
         self.cache_first_aggregation = bool(cache_first_aggregation)
         self._first_aggregation_valid = False
+        # every iteration aggregates over this graph: its dense corner is laid out for the tensor cores.  fp32 iterations keep the
+        # gather kernels' order of sums, as their products under a ReLU do (signs near zero go by it)
+        if precision != mg.PREC_FP32 and n_chunks <= 1:
+            mg.graph_prepare_tiles(graph)
         n, L = self.n, self.L
         orders = order if isinstance(order, (list, tuple)) else [order] * L
         self.descs, self.orders = [], []

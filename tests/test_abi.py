@@ -135,3 +135,10 @@ def test_split_products_compile_without_register_spills(tmp_path):
     entries = {re.search(r"\d([a-z_]+_kernel)E", name).group(1): (st, ld) for name, st, ld in spills("gemm_split.cu", tmp_path)}
     assert entries["gemm_split_kk_kernel"] == (0, 0) and entries["gemm_split_mm_kernel"] == (0, 0)
     assert entries["gemm_cvt_kk_kernel"][0] <= 64
+
+
+def test_the_product_of_hub_tiles_holds_its_sums_in_registers(tmp_path):
+    """128 sums a thread beside 32 of the accumulator: they fit the split of 192 and 64 registers, which needs the 128 of every
+    thread that the launch has (512 of them)."""
+    entries = {re.search(r"\d([a-z_]+_kernel)E", name).group(1): (st, ld) for name, st, ld in spills("hub_tiles.cu", tmp_path) if "spmm_tiles" in name}
+    assert entries["spmm_tiles_kernel"] == (0, 0)

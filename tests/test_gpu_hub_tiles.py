@@ -1,0 +1,183 @@
+"""Aggregation with the dense corner of the graph on the tensor cores (graph_prepare_tiles): widths either side of chunks, halves, lane
+splits and slices, every normalisation and orientation, the epilogues, rows that lie in tiles only, values the tensor core cannot take.
+
+Against fp64: a result is a sum of fp32 sums of at most 512 terms each, so its error stays below 512 units of rounding of the sum of the
+terms' absolute values in the worst case, and near sqrt(512) units (1.3e-6 of it) where the terms' signs do not matter; 4e-7 of the 2-norm is
+what rounding to nearest gives on average (0.29 units per addition, a third of it for sums that grow)."""
+import pytest
+import torch
+
+from paper_2501_01951_b200 import synth
+
+pytestmark = pytest.mark.gpu
+N, CORE = 9001, 4099
+
+
+@pytest.fixture(scope="module")
+def mg():
+    from paper_2501_01951_b200 import build
+    build.build()
+    from paper_2501_01951_b200 import binding
+    return binding
+
+
+@pytest.fixture(scope="module")
+def ctx(mg):
+    c = mg.ctx_create(0)
+    yield c
+    assert mg.ctx_poll_status(c, raise_on_error=False) == 0
+    c.close()
+
+
+def edges(seed):
+    """A dense core of CORE nodes, ids scattered over [0, N), the first 300 of them joined to one another only; a sparse rest that leaves some
+    nodes without neighbours."""
+    gen = torch.Generator().manual_seed(seed)
+    ids = torch.randperm(N, generator=gen)
+    core = torch.randint(0, CORE, (2, 6_000_000), generator=gen)
+    clique = torch.combinations(torch.arange(300)).T
+    core = core[:, (core >= 300).all(0)]
+    rest = torch.randint(300, N - 50, (2, 60_000), generator=gen)
+    e = ids[torch.cat([core, clique, rest], 1)].int()
+    return e[0].contiguous(), e[1].contiguous()
+
+
+def matrix(mg, g, transposed):
+    ex = mg.graph_export(g, transposed)
+    return torch.sparse_csr_tensor(ex["rowptr"], ex["col"].long(), ex["val"].double(), (g.n, g.n)).cuda()
+
+
+def features(w, seed, positive=False):
+    Y = torch.full((N, (w + 3) // 4 * 4), float("nan"), device="cuda")        # what lies beyond the columns is not read
+    Y[:, :w] = synth.uniform_tensor((N, w), seed, 0 if positive else -1, 1).cuda()
+    return Y
+
+
+@pytest.fixture(scope="module")
+def graphs(mg, ctx):
+    """{(norm, symmetric): (plain graph, graph with tiles, its matrices)}"""
+    out = {}
+    for norm, flags in (("sym", 0), ("row", mg.GRAPH_NORM_ROW), ("none", mg.GRAPH_NORM_NONE)):
+        for symmetric in (True, False):
+            fl = flags | (mg.GRAPH_SYMMETRISE if symmetric else 0) | (mg.GRAPH_ADD_SELF_LOOPS if norm == "sym" else 0)
+            src, dst = edges(1)
+            plain, tiled = (mg.graph_create(ctx, N, src, dst, fl) for _ in range(2))
+            tiles, entries = mg.graph_prepare_tiles(tiled)
+            assert tiles > 100 and entries > tiled.nnz // 2
+            assert mg.graph_prepare_tiles(tiled) == (tiles, entries)
+            out[norm, symmetric] = plain, tiled, [matrix(mg, tiled, t) for t in (False, True)]
+    yield out
+    for plain, tiled, _ in out.values():
+        plain.close(), tiled.close()
+
+
+@pytest.mark.parametrize("w", [1, 5, 16, 33, 47, 64, 65, 100, 128, 129, 160, 253, 256, 257, 300, 600])
+@pytest.mark.parametrize("norm,symmetric,transposed", [("sym", True, False), ("sym", False, True), ("row", True, False), ("row", False, False),
+                                                       ("none", False, False), ("none", False, True)])
+def test_sums_against_fp64(mg, ctx, graphs, norm, symmetric, transposed, w):
+    plain, tiled, A = graphs[norm, symmetric]
+    for positive in (False, True):
+        Y = features(w, 7, positive)
+        Z, Zp = (torch.full_like(Y, 3.0) for _ in range(2))
+        mg.spmm(ctx, tiled, Y, Z, w, transposed)
+        mg.spmm(ctx, plain, Y, Zp, w, transposed)
+        assert not torch.equal(Z, Zp)                                        # the tiles' kernels ran: sums in another order
+        want = A[transposed] @ Y[:, :w].double()
+        bound = 512 * 2.0 ** -24 * (A[transposed] @ Y[:, :w].double().abs())
+        assert torch.all((Z[:, :w].double() - want).abs() <= bound)
+        err, err_plain = (((z[:, :w].double() - want).norm() / want.norm()).item() for z in (Z, Zp))
+        print(f"{norm} {symmetric} {transposed} w {w} positive {positive}: {err:.2e} gathered {err_plain:.2e}")
+        assert err < 4e-7
+        assert torch.all(Z[:, w:] == 0)
+        again = torch.empty_like(Z)
+        mg.spmm(ctx, tiled, Y, again, w, transposed)
+        assert torch.equal(Z, again)
+
+
+@pytest.mark.parametrize("w", [41, 128, 256, 260])
+def test_epilogues_and_slices(mg, ctx, graphs, w):
+    plain, tiled, _ = graphs["sym", True]
+    ld, words = (w + 3) // 4 * 4, (w + 31) // 32
+    Y = features(w, 3)
+    t = lambda seed: synth.uniform_tensor((N, ld), seed, -1, 1).cuda()
+    bits = torch.randint(-2 ** 31, 2 ** 31 - 1, (N, words), dtype=torch.int32, device="cuda")
+    drop = (t(5)[:, :w] > 0).to(torch.uint8).contiguous()
+    for epi in (dict(bias=t(4)[0, :w].contiguous(), relu=True), dict(gate=t(6), gate_scale=2.0), dict(gate_bits=bits, gate_scale=1.5),
+                dict(residual=t(8), residual_scale=0.5, relu=True), dict(drop_mask=drop, keep_scale=2.0, bias=t(4)[0, :w].contiguous())):
+        Z, Zp = (torch.full_like(Y, 3.0) for _ in range(2))
+        mg.spmm(ctx, tiled, Y, Z, w, epi=mg.make_epilogue(**epi))
+        mg.spmm(ctx, plain, Y, Zp, w, epi=mg.make_epilogue(**epi))
+        assert (Z - Zp).abs().max() <= 2e-6 * Zp.abs().max()                  # two fp32 sums of the same terms
+    whole, sliced = torch.empty_like(Y), torch.empty_like(Y)
+    mg.spmm(ctx, tiled, Y, whole, w)
+    for cols in (16, 100, 512):
+        mg.ctx_set_option(ctx, mg.OPT_SPMM_SLICE_COLS, cols)
+        mg.spmm(ctx, tiled, Y, sliced, w)
+        mg.ctx_set_option(ctx, mg.OPT_SPMM_SLICE_COLS, 0)
+        assert (whole - sliced).abs().max() <= 2e-6 * whole.abs().max()
+
+
+@pytest.mark.parametrize("w", [47, 256])
+def test_values_that_the_parts_cannot_hold(mg, ctx, graphs, w):
+    """Infinities, NaN and numbers near the largest reach the same outputs as on the gather kernels, and no call after it."""
+    plain, tiled, _ = graphs["none", True]
+    hubs = mg.graph_degrees(tiled).argsort(descending=True)
+    for value in (float("inf"), float("nan"), 3e38, -2e30, None, None):
+        Y = features(w, 9)
+        if value is not None:
+            Y[hubs[700], w // 2] = value
+        Z, Zp = (torch.empty_like(Y) for _ in range(2))
+        mg.spmm(ctx, tiled, Y, Z, w)
+        mg.spmm(ctx, plain, Y, Zp, w)
+        Z, Zp = Z[:, :w], Zp[:, :w]
+        assert torch.equal(torch.isnan(Z), torch.isnan(Zp)) and torch.equal(torch.isinf(Z), torch.isinf(Zp))
+        fine = torch.isfinite(Zp)
+        assert ((Z - Zp)[fine].abs() <= 2e-6 * Zp[fine].abs().max()).all()
+
+
+def test_numbers_of_every_size(mg, ctx, graphs):
+    """Columns from 1e-30 to 1e30 come out to the same relative error; zeros and whole numbers exactly."""
+    _, tiled, A = graphs["none", True]
+    w = 64
+    Y = features(w, 11, True) * 10.0 ** torch.linspace(-30, 26, w, device="cuda")
+    Y[:, 0] = 0
+    Y[:, 1:3] = (Y[:, 1:3] * 1e30 * 5).round()
+    Z = torch.empty_like(Y)
+    mg.spmm(ctx, tiled, Y, Z, w)
+    want = A[0] @ Y.double()
+    assert torch.all(((Z.double() - want).norm(dim=0) <= 4e-7 * want.norm(dim=0)))
+    assert torch.equal(Z[:, :3].double(), want[:, :3])
+
+
+def test_a_wait_that_runs_out_is_reported(mg, ctx, graphs):
+    _, tiled, _ = graphs["sym", True]
+    Y, Z = features(256, 3), torch.empty((N, 256), device="cuda")
+    mg.ctx_set_option(ctx, mg.OPT_DEBUG_WAIT_LIMIT, 2000)
+    mg.ctx_set_option(ctx, mg.OPT_DEBUG_DROP_LOAD, 1)
+    try:
+        mg.spmm(ctx, tiled, Y, Z, 256)
+        assert mg.ctx_poll_status(ctx, raise_on_error=False) == 3
+    finally:
+        mg.ctx_set_option(ctx, mg.OPT_DEBUG_DROP_LOAD, 0)
+        mg.ctx_set_option(ctx, mg.OPT_DEBUG_WAIT_LIMIT, 0)
+    want = torch.empty_like(Z)
+    mg.spmm(ctx, tiled, Y, Z, 256)
+    mg.spmm(ctx, graphs["sym", True][0], Y, want, 256)
+    assert mg.ctx_poll_status(ctx, raise_on_error=False) == 0 and (Z - want).abs().max() <= 2e-6 * want.abs().max()
+
+
+def test_row_means_transposed_stay_with_the_gather_kernels(mg, ctx, graphs):
+    plain, tiled, _ = graphs["row", True]
+    Y, Z, Zp = features(100, 3), torch.empty((N, 100), device="cuda"), torch.empty((N, 100), device="cuda")
+    mg.spmm(ctx, tiled, Y, Z, 100, True)
+    mg.spmm(ctx, plain, Y, Zp, 100, True)
+    assert torch.equal(Z, Zp)
+
+
+def test_small_and_sparse_graphs_have_no_tiles(mg, ctx):
+    for n, m in ((2000, 30_000), (400_000, 1_500_000)):
+        gen = torch.Generator().manual_seed(n)
+        e = torch.randint(0, n, (2, m), generator=gen, dtype=torch.int32)
+        g = mg.graph_create(ctx, n, e[0].contiguous(), e[1].contiguous())
+        assert mg.graph_prepare_tiles(g) == (0, 0)
+        g.close()

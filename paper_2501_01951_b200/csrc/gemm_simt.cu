@@ -43,7 +43,8 @@ struct GemmParams {
     int64_t k_per_split; int splits;
     int64_t m_tiles, n_tiles;
     int vec_a, vec_b, vec_c;     // 16-byte vector access is legal (pointer and ld aligned)
-    int vec_drop, vec_gate;      // the same for four mask bytes / four gate values at a multiple of four columns
+    int vec_drop;                // mask bytes that can be copied at once (16 or 4; 0: the mask is read in the epilogue)
+    int vec_gate;                // 16-byte access for four gate values at a multiple of four columns
     const int32_t* only_if;      // nullable: every CTA returns at once where this word is zero
     Epi epi;
 };
@@ -54,10 +55,10 @@ __device__ __forceinline__ void ffma2(f32x2& d, f32x2 a, f32x2 b) { asm("fma.rn.
 __device__ __forceinline__ f32x2 dup2(float a) { f32x2 r; asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a)); return r; }
 __device__ __forceinline__ float2 split2(f32x2 v) { float2 f; asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v)); return f; }
 
-__device__ __forceinline__ void cp_async16(void* dst, const float* src, int bytes) {      // the first `bytes` of 16, zeros behind
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, int bytes) {      // the first `bytes` of 16, zeros behind
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
 }
-__device__ __forceinline__ void cp_async4(void* dst, const float* src, int bytes) {
+__device__ __forceinline__ void cp_async4(void* dst, const void* src, int bytes) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
 }
 // four consecutive floats, the first `valid` of them read (<= 0: none, `base` stands in for the address)
@@ -72,8 +73,8 @@ __device__ __forceinline__ void copy4(float* dst, const float* src, int64_t vali
 // fma.rn.f32x2 does two FMAs, so that the shared-memory loads and the operand copies find free issue slots beside a full
 // FMA pipe), 16-deep k-steps through three cp.async stages.  Bound by the FMA rate (72 TFLOP/s measured with either
 // form of the instruction): 170 K x 256 x 256 forward 33.7 -> 42 TFLOP/s, weight gradient 25.4 -> 48 TFLOP/s against one
-// stage, register staging and scalar FMAs; the pipe is then 72 % busy, the rest is fixed-latency waits of the two warps a
-// scheduler has room for.
+// stage, register staging and scalar FMAs; with the large tile's operands read ahead 44 (50.8 at K = 1024), the weight gradient 50.
+// Next to the FMAs stand the operands: a micro-tile's 96 bytes a thread and k take the load/store pipe three quarters of the FMAs' time.
 //   A with K contiguous stays [m][k] in shared memory and is read two k at a time (row pitch 20 floats: the four rows a
 //   warp reads side by side lie in different banks); A with M contiguous, and B, are [k][m] / [k][n].  B with K
 //   contiguous (the small weight matrix of dP W^T) is turned round by word-wide copies.
@@ -86,6 +87,13 @@ template <int BM, int BN, int TN, int KG>
 struct SimtCfg {
     static constexpr int GROUP = BM * BN / (8 * TN), NT = GROUP * KG;    // threads of a group, of the CTA
     static constexpr int MIN_CTAS = BM == 128 ? (BN == 128 ? 2 : 4) : (BN == 64 ? 6 : 10) / KG;
+    static constexpr int a_floats(bool ta) { return ta ? BK * (BM + 4) : BM * (BK + 4); }
+    static constexpr int B_FLOATS = BK * (BN + 4);
+    // the k-steps' ring, which the epilogue uses again for half of the tile; the mask of the tile lies behind
+    static constexpr int ring_bytes(bool ta) {
+        const int ring = STAGES * (a_floats(ta) + B_FLOATS), half_tile = BM / 2 * (BN + 4);
+        return (ring > half_tile ? ring : half_tile) * (int)sizeof(float);
+    }
 };
 constexpr int FINE_KG = 4;
 
@@ -93,7 +101,8 @@ template <int BM, int BN, int TN, int KG, bool TA, bool TB>
 __global__ void __launch_bounds__(SimtCfg<BM, BN, TN, KG>::NT, SimtCfg<BM, BN, TN, KG>::MIN_CTAS) gemm_simt_kernel(const GemmParams p) {
     constexpr int TM = 8, NT = SimtCfg<BM, BN, TN, KG>::NT, H = TM / 4, TX = BN / TN, Q = TN / 4, QW = BN / Q;   // Q groups of four columns, QW columns apart
     constexpr int A_PITCH = TA ? BM + 4 : BK + 4, B_PITCH = BN + 4;
-    constexpr int A_FLOATS = TA ? BK * A_PITCH : BM * A_PITCH, B_FLOATS = BK * B_PITCH;
+    using Cfg = SimtCfg<BM, BN, TN, KG>;
+    constexpr int A_FLOATS = Cfg::a_floats(TA), B_FLOATS = Cfg::B_FLOATS;
     extern __shared__ __align__(16) float smem_f[];
     if (p.only_if && *p.only_if == 0) return;
     const int tid = threadIdx.x, lane = tid & 31;
@@ -160,6 +169,25 @@ __global__ void __launch_bounds__(SimtCfg<BM, BN, TN, KG>::NT, SimtCfg<BM, BN, T
             }
         }
     };
+    // The dropout mask of the tile comes in beside the first k-step, for the epilogue, which would wait for DRAM eight times for every
+    // half of the tile (170 K x 256 with K = 128 and a byte mask: 416 -> 306 us, K = 256: 591 -> 513).
+    uint8_t* const mask = reinterpret_cast<uint8_t*>(smem_f) + Cfg::ring_bytes(TA);
+    if (p.vec_drop && p.splits == 1) {
+        auto copy_mask = [&](int bytes) {
+            const int per_row = BN / bytes;
+#pragma unroll 4
+            for (int f = tid; f < BM * per_row; f += NT) {
+                const int r = f / per_row, c = f % per_row * bytes;
+                const int64_t m = m0 + r, n = n0 + c;
+                if (m >= p.M || n >= p.N) continue;
+                const uint8_t* src = p.epi.drop + (p.epi.row0 + m) * p.N + n;
+                if (bytes == 16) cp_async16(mask + r * BN + c, src, 16);
+                else cp_async4(mask + r * BN + c, src, 4);
+            }
+        };
+        if (p.vec_drop == 16) copy_mask(16);
+        else copy_mask(4);
+    }
     auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
 
     f32x2 acc[TM][TN / 2];
@@ -191,58 +219,123 @@ __global__ void __launch_bounds__(SimtCfg<BM, BN, TN, KG>::NT, SimtCfg<BM, BN, T
             }
     };
 
-    // One loop body serves the filling of the pipeline and the steps themselves: a small product runs each line of this code
-    // once or a few times, and then its length is its time.
     bool flushed = false;
     int since_flush = 0;
-#pragma unroll 1
-    for (int ks = 1 - STAGES; ks < steps; ++ks) {
-        if (ks >= 0) {
-            asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
-            __syncthreads();                   // step ks has landed; the stage of step ks - 1 is free
-        }
-        if (ks + STAGES - 1 < steps) { load_a(ks + STAGES - 1); load_b(ks + STAGES - 1); }
-        commit();
-        if (ks < 0) continue;
-        const float* As = smem_f + (ks % STAGES) * (A_FLOATS + B_FLOATS);
-        const float* Bs = As + A_FLOATS;
-#pragma unroll (TA && KG == 1 ? BK / 2 : 2)        // (with the row-wise A a longer body gains nothing and spills)
-        for (int kk = kg * (BK / KG); kk < (kg + 1) * (BK / KG); kk += 2) {
-            float2 a2[TM];
-            if (!TA) {
+    if constexpr (TN == 16) {
+        // Operands of the next k are read from shared memory ahead of this one's FMAs, over the step's end as well: its barrier stands before
+        // the last k, when everything of the stage is in registers, and the stage is refilled there and then (170 K x 256, K = 256: 517 -> 502 us,
+        // K = 1024: 1847 -> 1756, 50.8 TFLOP/s; same sums).
+        float2 a2[2][TM];                      // A as [m][k]: two k at a time
+        float a1[2][TM];                       // A as [k][m]
+        ulonglong2 b[2][Q];
+        auto read_a = [&](const float* As, int k) {
+            if constexpr (!TA) {
 #pragma unroll
-                for (int i = 0; i < TM; ++i) a2[i] = *reinterpret_cast<const float2*>(As + (ty + i * (BM / TM)) * A_PITCH + kk);
+                for (int i = 0; i < TM; ++i) a2[(k >> 1) & 1][i] = *reinterpret_cast<const float2*>(As + (ty + i * (BM / TM)) * A_PITCH + k);
+            } else {
+#pragma unroll
+                for (int g = 0; g < H; ++g) {
+                    const float4 x = *reinterpret_cast<const float4*>(As + k * A_PITCH + ty * 4 + g * (BM / H));
+                    a1[k & 1][4 * g] = x.x; a1[k & 1][4 * g + 1] = x.y; a1[k & 1][4 * g + 2] = x.z; a1[k & 1][4 * g + 3] = x.w;
+                }
             }
+        };
+        auto read_b = [&](const float* Bs, int k) {
 #pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const float* brow = Bs + (kk + k) * B_PITCH + tx * 4;
-                ulonglong2 b[Q];
+            for (int q = 0; q < Q; ++q) b[k & 1][q] = *reinterpret_cast<const ulonglong2*>(Bs + k * B_PITCH + tx * 4 + q * QW);
+        };
+#pragma unroll 1
+        for (int ks = 0; ks < STAGES; ++ks) {
+            if (ks < steps) { load_a(ks); load_b(ks); }
+            commit();
+        }
+        asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 1) : "memory");
+        __syncthreads();
+        read_a(smem_f, 0);
+        read_b(smem_f + A_FLOATS, 0);
+#pragma unroll 1
+        for (int ks = 0; ks < steps; ++ks) {
+            const float* As = smem_f + (ks % STAGES) * (A_FLOATS + B_FLOATS);
 #pragma unroll
-                for (int q = 0; q < Q; ++q) b[q] = *reinterpret_cast<const ulonglong2*>(brow + q * QW);
-                float a[TM];
-                if (!TA) {
-#pragma unroll
-                    for (int i = 0; i < TM; ++i) a[i] = k == 0 ? a2[i].x : a2[i].y;
+            for (int k = 0; k < BK; ++k) {
+                if (k + 1 < BK) {
+                    read_b(As + A_FLOATS, k + 1);
+                    if (TA) read_a(As, k + 1);
+                    else if (!(k & 1) && k + 2 < BK) read_a(As, k + 2);
                 } else {
-                    const float* arow = As + (kk + k) * A_PITCH + ty * 4;
-#pragma unroll
-                    for (int g = 0; g < H; ++g) {
-                        const float4 x = *reinterpret_cast<const float4*>(arow + g * (BM / H));
-                        a[4 * g] = x.x; a[4 * g + 1] = x.y; a[4 * g + 2] = x.z; a[4 * g + 3] = x.w;
-                    }
+                    asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+                    __syncthreads();           // step ks + 1 has landed, step ks is read
+                    const float* next = smem_f + ((ks + 1) % STAGES) * (A_FLOATS + B_FLOATS);
+                    read_b(next + A_FLOATS, 0);
+                    read_a(next, 0);
+                    if (ks + STAGES < steps) { load_a(ks + STAGES); load_b(ks + STAGES); }
+                    commit();
                 }
 #pragma unroll
                 for (int i = 0; i < TM; ++i) {
-                    const f32x2 av = dup2(a[i]);
+                    const f32x2 av = dup2(TA ? a1[k & 1][i] : (k & 1) ? a2[(k >> 1) & 1][i].y : a2[(k >> 1) & 1][i].x);
 #pragma unroll
-                    for (int q = 0; q < Q; ++q) { ffma2(acc[i][2 * q], av, b[q].x); ffma2(acc[i][2 * q + 1], av, b[q].y); }
+                    for (int q = 0; q < Q; ++q) { ffma2(acc[i][2 * q], av, b[k & 1][q].x); ffma2(acc[i][2 * q + 1], av, b[k & 1][q].y); }
                 }
             }
+            if (++since_flush == FLUSH_STEPS && ks + 1 < steps) {
+                since_flush = 0;
+                flush(!flushed);
+                flushed = true;
+            }
         }
-        if (++since_flush == FLUSH_STEPS && ks + 1 < steps && KG == 1) {
-            since_flush = 0;
-            flush(!flushed);
-            flushed = true;
+    } else {
+        // One loop body serves the filling of the pipeline and the steps themselves: a small product runs each line of this code
+        // once or a few times, and then its length is its time.
+#pragma unroll 1
+        for (int ks = 1 - STAGES; ks < steps; ++ks) {
+            if (ks >= 0) {
+                asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+                __syncthreads();                   // step ks has landed; the stage of step ks - 1 is free
+            }
+            if (ks + STAGES - 1 < steps) { load_a(ks + STAGES - 1); load_b(ks + STAGES - 1); }
+            commit();
+            if (ks < 0) continue;
+            const float* As = smem_f + (ks % STAGES) * (A_FLOATS + B_FLOATS);
+            const float* Bs = As + A_FLOATS;
+#pragma unroll (TA && KG == 1 ? BK / 2 : 2)        // (with the row-wise A a longer body gains nothing and spills)
+            for (int kk = kg * (BK / KG); kk < (kg + 1) * (BK / KG); kk += 2) {
+                float2 a2[TM];
+                if (!TA) {
+#pragma unroll
+                    for (int i = 0; i < TM; ++i) a2[i] = *reinterpret_cast<const float2*>(As + (ty + i * (BM / TM)) * A_PITCH + kk);
+                }
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    const float* brow = Bs + (kk + k) * B_PITCH + tx * 4;
+                    ulonglong2 b[Q];
+#pragma unroll
+                    for (int q = 0; q < Q; ++q) b[q] = *reinterpret_cast<const ulonglong2*>(brow + q * QW);
+                    float a[TM];
+                    if (!TA) {
+#pragma unroll
+                        for (int i = 0; i < TM; ++i) a[i] = k == 0 ? a2[i].x : a2[i].y;
+                    } else {
+                        const float* arow = As + (kk + k) * A_PITCH + ty * 4;
+#pragma unroll
+                        for (int g = 0; g < H; ++g) {
+                            const float4 x = *reinterpret_cast<const float4*>(arow + g * (BM / H));
+                            a[4 * g] = x.x; a[4 * g + 1] = x.y; a[4 * g + 2] = x.z; a[4 * g + 3] = x.w;
+                        }
+                    }
+#pragma unroll
+                    for (int i = 0; i < TM; ++i) {
+                        const f32x2 av = dup2(a[i]);
+#pragma unroll
+                        for (int q = 0; q < Q; ++q) { ffma2(acc[i][2 * q], av, b[q].x); ffma2(acc[i][2 * q + 1], av, b[q].y); }
+                    }
+                }
+            }
+            if (++since_flush == FLUSH_STEPS && ks + 1 < steps && KG == 1) {
+                since_flush = 0;
+                flush(!flushed);
+                flushed = true;
+            }
         }
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -293,8 +386,8 @@ __global__ void __launch_bounds__(SimtCfg<BM, BN, TN, KG>::NT, SimtCfg<BM, BN, T
                 }
                 if (e.drop && in) {
                     const uint8_t* dm = e.drop + (e.row0 + m) * p.N + n;
-                    if (p.vec_drop && full) {
-                        const uchar4 d4 = __ldg(reinterpret_cast<const uchar4*>(dm));
+                    if (p.vec_drop) {
+                        const uchar4 d4 = *reinterpret_cast<const uchar4*>(mask + (h * (BM / H) + lr) * BN + lc);
                         r[0] = d4.x ? r[0] * e.keep_scale : 0.0f; r[1] = d4.y ? r[1] * e.keep_scale : 0.0f;
                         r[2] = d4.z ? r[2] * e.keep_scale : 0.0f; r[3] = d4.w ? r[3] * e.keep_scale : 0.0f;
                     } else {
@@ -453,11 +546,10 @@ __global__ void gate_kernel(int64_t n, int d, float* __restrict__ G, int64_t ldg
 
 template <int BM, int BN, int TN, int KG, bool TA, bool TB>
 cudaError_t launch_form(const GemmParams& p, cudaStream_t s) {
-    constexpr int a_floats = TA ? BK * (BM + 4) : BM * (BK + 4), b_floats = BK * (BN + 4);
-    constexpr int ring = STAGES * (a_floats + b_floats), half_tile = BM / 2 * (BN + 4);
-    constexpr int smem = (ring > half_tile ? ring : half_tile) * (int)sizeof(float);
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(gemm_simt_kernel<BM, BN, TN, KG, TA, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    constexpr int ring = SimtCfg<BM, BN, TN, KG>::ring_bytes(TA), most = ring + BM * BN;
+    const int smem = p.vec_drop && p.splits == 1 ? most : ring;
+    if (smem > 48 * 1024) {        // (one value for every call: another thread may be between this and its launch)
+        const cudaError_t e = cudaFuncSetAttribute(gemm_simt_kernel<BM, BN, TN, KG, TA, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         if (e != cudaSuccess) return e;
     }
     gemm_simt_kernel<BM, BN, TN, KG, TA, TB><<<dim3((unsigned)(p.m_tiles * p.n_tiles), 1, (unsigned)p.splits), SimtCfg<BM, BN, TN, KG>::NT, smem, s>>>(p);
@@ -496,7 +588,8 @@ mixgcn_status launch_gemm_simt(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64
     p.vec_a = aligned16(A) && (lda & 3) == 0;
     p.vec_b = aligned16(B) && (ldb & 3) == 0;
     p.vec_c = aligned16(C) && (ldc & 3) == 0;
-    p.vec_drop = p.epi.drop && (N & 3) == 0 && (reinterpret_cast<uintptr_t>(p.epi.drop) & 3) == 0;
+    const uintptr_t mask_at = reinterpret_cast<uintptr_t>(p.epi.drop) | (uintptr_t)N;       // (every row starts at a multiple of N)
+    p.vec_drop = !p.epi.drop || (mask_at & 3) ? 0 : (mask_at & 15) ? 4 : 16;
     p.vec_gate = p.epi.gate && aligned16(p.epi.gate) && (p.epi.ld_gate & 3) == 0;
     // The tile: 32 columns where N has no more, else 64 or 128 by what leaves less of N to padding, 128 rows.  Where that
     // gives fewer CTAs than the machine has SMs even with K split, 64-row tiles.

@@ -62,3 +62,20 @@ def test_tiles(mg, ctx, M, N, K, ta, tb, aligned):
     packed[:, :N] = got > 0
     packed = (packed.reshape(M, words, 32) << np.arange(32, dtype=np.uint32)).sum(axis=2, dtype=np.uint32)
     assert np.array_equal(bits[:, :words].cpu().numpy().view(np.uint32), packed) and torch.all(bits[:, words] == -1)
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 16, 1), (63, 32, 15), (65, 48, 17), (130, 40, 40), (129, 128, 33), (20001, 128, 70), (9000, 100, 20), (257, 256, 1100)])
+@pytest.mark.parametrize("offset", [0, 4, 1])
+def test_dropout_masks(mg, ctx, M, N, K, offset):
+    """Masks that are copied 16 and 4 bytes at a time beside the k-steps, and those that are not: rows that start at multiples of 16, of 4 and at odd bytes."""
+    A, B = synth.uniform_tensor((M, K), 31, -1, 1), synth.uniform_tensor((K, N), 32, -1, 1)
+    drop = synth.bernoulli_mask(M * N, 0.5, 33)
+    at = torch.full((M * N + 16,), 255, dtype=torch.uint8, device="cuda")
+    at[offset:offset + M * N] = drop.cuda()
+    up = (N + 3) // 4 * 4
+    C = torch.full((M, up), 3.0, device="cuda")
+    mg.gemm(ctx, mg.PREC_FP32, False, False, M, N, K, device(A, (K + 3) // 4 * 4), device(B, up), C,
+            epi=mg.make_epilogue(relu=True, drop_mask=at[offset:offset + M * N], keep_scale=2.0))
+    want = np.maximum(A.numpy().astype(np.float64) @ B.numpy().astype(np.float64), 0.0) * drop.numpy().reshape(M, N) * 2.0
+    got = C[:, :N].cpu().numpy()
+    assert rel_fro(got, want) <= TOL_FP32 and not np.any(got[drop.numpy().reshape(M, N) == 0])

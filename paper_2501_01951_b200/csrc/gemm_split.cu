@@ -428,6 +428,7 @@ __device__ __forceinline__ void prefetch_masks(const SplitParams& p, int64_t til
 // ---------------------------------------------------------------- K-major form
 __global__ void __launch_bounds__(THREADS, 1) gemm_split_kk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                                                                    const __grid_constant__ CUtensorMap map_c, const SplitParams p, const int tma_store) {
+    chain_begin();
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) Shared bars;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -517,6 +518,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_kk_kernel(const __grid_
 // ---------------------------------------------------------------- MN-major form (weight gradient)
 __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                                                                    const SplitParams p) {
+    pdl_wait();               // (see chain_begin)
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) Shared bars;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -658,6 +660,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_split_mm_kernel(const __grid_
 // issue slots 25 %; the epilogue spills 64 bytes a thread (96 registers: it has no register split).
 __global__ void __launch_bounds__(THREADS, 1) gemm_cvt_kk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                                                                  const __grid_constant__ CUtensorMap map_c, const SplitParams p, const int tma_store) {
+    chain_begin();
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) Shared bars;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -755,6 +758,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_cvt_kk_kernel(const __grid_co
 // outside N x K.
 __global__ void pack_split_kernel(const float* __restrict__ src, int64_t ld, int trans, int N, int K, int rows, int kpad, int parts,
                                   uint16_t* __restrict__ dst) {
+    chain_begin();
     const int64_t plane = (int64_t)rows * kpad, i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= plane) return;
     const int n = trans ? (int)(i % rows) : (int)(i / kpad), k = trans ? (int)(i / rows) : (int)(i % kpad);     // consecutive threads read consecutive words
@@ -847,14 +851,14 @@ mixgcn_status launch_gemm_split(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int6
         p.raw_slots = raw_slots(fixed, RAW_BYTES);
         const size_t smem = fixed + (size_t)p.raw_slots * RAW_BYTES;
         MIXGCN_CUDA(cudaFuncSetAttribute(gemm_split_kk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        MIXGCN_CUDA(cudaMemsetAsync(p.overflow, 0, sizeof(int32_t), s));
+        MIXGCN_TRY(launch_clear(ctx, PH_GEMM, p.overflow, 1, nullptr, s));
         {
             LaunchScope scope(ctx, PH_GEMM, s);
-            pack_split_kernel<<<(unsigned)ceil_div((int64_t)rows * kpad, 256), 256, 0, s>>>(B, ldb, tb ? 0 : 1, (int)N, (int)K, rows, kpad, PARTS, planes);
+            launch_chained(pack_split_kernel, dim3((unsigned)ceil_div((int64_t)rows * kpad, 256)), 256, 0, s, B, ldb, tb ? 0 : 1, (int)N, (int)K, rows, kpad, PARTS, planes);
         }
         LaunchScope scope(ctx, PH_GEMM, s);
         const unsigned grid = (unsigned)(tiles < ctx->sm_count ? tiles : ctx->sm_count);
-        gemm_split_kk_kernel<<<grid, THREADS, smem, s>>>(map_a, map_b, map_c, p, tma_store);
+        launch_chained(gemm_split_kk_kernel, dim3(grid), THREADS, smem, s, map_a, map_b, map_c, p, tma_store);
         MIXGCN_CUDA(cudaGetLastError());
         if (bits_done) *bits_done = p.epi.sign_bits != nullptr;
         return MIXGCN_OK;
@@ -884,10 +888,10 @@ mixgcn_status launch_gemm_split(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int6
     p.raw_slots = raw_slots(fixed, RAW_BYTES);
     const size_t smem = fixed + (size_t)p.raw_slots * RAW_BYTES;
     MIXGCN_CUDA(cudaFuncSetAttribute(gemm_split_mm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    MIXGCN_CUDA(cudaMemsetAsync(p.overflow, 0, sizeof(int32_t), s));
+    MIXGCN_TRY(launch_clear(ctx, PH_GEMM, p.overflow, 1, nullptr, s));
     {
         LaunchScope scope(ctx, PH_GEMM, s);
-        gemm_split_mm_kernel<<<dim3((unsigned)tiles, 1, (unsigned)splits), THREADS, smem, s>>>(map_a, map_b, p);
+        launch_chained(gemm_split_mm_kernel, dim3((unsigned)tiles, 1, (unsigned)splits), THREADS, smem, s, map_a, map_b, p);
     }
     MIXGCN_CUDA(cudaGetLastError());
     if (colsum_b) {
@@ -931,11 +935,11 @@ mixgcn_status launch_gemm_cvt(mixgcn_ctx* ctx, int tb, int64_t M, int64_t N, int
     MIXGCN_CUDA(cudaFuncSetAttribute(gemm_cvt_kk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     {
         LaunchScope scope(ctx, PH_GEMM, s);
-        pack_split_kernel<<<(unsigned)ceil_div((int64_t)bn32 * kpad, 256), 256, 0, s>>>(B, ldb, tb ? 0 : 1, (int)N, (int)K, bn32, kpad, 1, packed);
+        launch_chained(pack_split_kernel, dim3((unsigned)ceil_div((int64_t)bn32 * kpad, 256)), 256, 0, s, B, ldb, tb ? 0 : 1, (int)N, (int)K, bn32, kpad, 1, packed);
     }
     LaunchScope scope(ctx, PH_GEMM, s);
     const unsigned grid = (unsigned)(p.m_tiles < ctx->sm_count ? p.m_tiles : ctx->sm_count);
-    gemm_cvt_kk_kernel<<<grid, THREADS, smem, s>>>(map_a, map_b, map_c, p, tma_store);
+    launch_chained(gemm_cvt_kk_kernel, dim3(grid), THREADS, smem, s, map_a, map_b, map_c, p, tma_store);
     MIXGCN_CUDA(cudaGetLastError());
     if (bits_done) *bits_done = p.epi.sign_bits != nullptr;
     return MIXGCN_OK;

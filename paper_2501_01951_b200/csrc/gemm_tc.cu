@@ -74,6 +74,7 @@ template <int KIND, bool MN_MAJOR>
 __global__ void __launch_bounds__(TC_THREADS, 2) gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a,
                                                              const __grid_constant__ CUtensorMap map_b,
                                                              const TcParams p) {
+    pdl_wait();               // (see chain_begin)
     using Cfg = KindCfg<KIND>;
     constexpr int BK = Cfg::BK;
     extern __shared__ uint8_t smem_raw[];
@@ -311,6 +312,7 @@ __global__ void __launch_bounds__(KK_THREADS, 1) gemm_tc_kk_kernel(const __grid_
                                                                 const __grid_constant__ CUtensorMap map_b,
                                                                 const __grid_constant__ CUtensorMap map_c,
                                                                 const TcParams p, const int b_resident, const int tma_store) {
+    chain_begin();
     using Cfg = KindCfg<KIND>;
     constexpr int BK = Cfg::BK;
     extern __shared__ uint8_t smem_raw[];
@@ -621,6 +623,7 @@ __global__ void __launch_bounds__(KK_THREADS, 1) gemm_tc_pair_kernel(const __gri
                                                                      const __grid_constant__ CUtensorMap map_b,
                                                                      const __grid_constant__ CUtensorMap map_c,
                                                                      const TcParams p, const int tma_store) {
+    chain_begin();
     using Cfg = KindCfg<KIND>;
     constexpr int BK = Cfg::BK;
     extern __shared__ uint8_t smem_raw[];
@@ -796,6 +799,7 @@ template <int KIND>
 __global__ void __launch_bounds__(TC_THREADS, 1) gemm_tc_mm_pair_kernel(const __grid_constant__ CUtensorMap map_a,
                                                                         const __grid_constant__ CUtensorMap map_b,
                                                                         const TcParams p) {
+    pdl_wait();               // (see chain_begin)
     using Cfg = KindCfg<KIND>;
     constexpr int BK = Cfg::BK;
     extern __shared__ uint8_t smem_raw[];
@@ -936,6 +940,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) gemm_tc_mm_pair_kernel(const __
 template <int KIND>
 __global__ void pack_b_kernel(const float* __restrict__ src, int64_t ld, int trans, int N, int K, int rows, int kpad,
                               void* __restrict__ dst) {
+    chain_begin();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)rows * kpad) return;
     const int n = (int)(i / kpad), k = (int)(i % kpad);
@@ -948,6 +953,7 @@ __global__ void pack_b_kernel(const float* __restrict__ src, int64_t ld, int tra
 // out[n] = sum over splits of part[z][n]: eight rows of threads add an eighth of the splits each, the eighths are added in
 // order (one thread's chain over 296 splits took 20 us).
 __global__ void __launch_bounds__(256) colsum_splits_kernel(int64_t N, int splits, const double* __restrict__ part, float* __restrict__ out) {
+    chain_begin();
     __shared__ double sm[8][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t n = (int64_t)blockIdx.x * 32 + lane;
@@ -968,6 +974,7 @@ __global__ void __launch_bounds__(256) colsum_splits_kernel(int64_t N, int split
 // dst[r][c] = bf16(src[r][c]) for c < d (round to nearest even); four columns per thread.
 __global__ void to_bf16_kernel(int64_t rows, int d4, const float* __restrict__ src, int64_t ld_src, int d,
                                uint16_t* __restrict__ dst, int64_t ld_dst) {
+    chain_begin();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= rows * d4) return;
     const int64_t r = t / d4; const int c = (int)(t % d4) * 4;
@@ -1006,7 +1013,7 @@ EncodeTiledFn get_encode() {
 namespace mixgcn {
 mixgcn_status launch_colsum_splits(mixgcn_ctx* ctx, int64_t N, int splits, const double* part, float* out, cudaStream_t s) {
     LaunchScope scope(ctx, PH_GEMM, s);
-    colsum_splits_kernel<<<(unsigned)((N + 31) / 32), 256, 0, s>>>(N, splits, part, out);
+    launch_chained(colsum_splits_kernel, dim3((unsigned)((N + 31) / 32)), 256, 0, s, N, splits, part, out);
     MIXGCN_CUDA(cudaGetLastError());
     return MIXGCN_OK;
 }
@@ -1109,7 +1116,7 @@ mixgcn_status launch_kind(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64_t N,
         {
             LaunchScope scope(ctx, PH_GEMM, s);
             const int64_t total = (int64_t)rows * kpad;
-            pack_b_kernel<KIND><<<(unsigned)((total + 255) / 256), 256, 0, s>>>(reinterpret_cast<const float*>(B), ldb, tb ? 0 : 1,
+            launch_chained(pack_b_kernel<KIND>, dim3((unsigned)((total + 255) / 256)), 256, 0, s, reinterpret_cast<const float*>(B), ldb, tb ? 0 : 1,
                                                                                  (int)N, (int)K, rows, kpad, packed);
         }
         p.splits = 1; p.k_per_split = K; p.raw = 0;
@@ -1130,9 +1137,11 @@ mixgcn_status launch_kind(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64_t N,
             if (ok2) {
                 MIXGCN_CUDA(cudaFuncSetAttribute(gemm_tc_pair_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2));
                 cudaLaunchConfig_t cfg = {};
-                cudaLaunchAttribute attr[1];
+                cudaLaunchAttribute attr[2];
                 attr[0].id = cudaLaunchAttributeClusterDimension;
                 attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+                attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // as launch_chained
+                attr[1].val.programmaticStreamSerializationAllowed = 1;
                 cfg.blockDim = dim3(KK_THREADS, 1, 1);
                 cfg.dynamicSmemBytes = smem2;
                 cfg.stream = s;
@@ -1144,6 +1153,7 @@ mixgcn_status launch_kind(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64_t N,
                 int64_t clusters = max_clusters < tiles2 ? max_clusters : tiles2;
                 if (clusters >= 1) {
                     cfg.gridDim = dim3((unsigned)(2 * clusters), 1, 1);
+                    cfg.numAttrs = 2;
                     LaunchScope scope(ctx, PH_GEMM, s);
                     MIXGCN_CUDA(cudaLaunchKernelEx(&cfg, gemm_tc_pair_kernel<KIND>, map_a, map_b2, map_c2, q, tma_store2));
                     ctx->gemm_pair_launches++;
@@ -1176,13 +1186,13 @@ mixgcn_status launch_kind(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64_t N,
             p.loss_mask = loss->train_mask; p.loss_pred = loss->pred; p.loss_zero_rows = loss->zero_rows;
             MIXGCN_CUDA(cudaFuncSetAttribute(gemm_tc_kk_kernel<KIND, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_kk));
             LaunchScope scope(ctx, PH_GEMM, s);
-            gemm_tc_kk_kernel<KIND, true><<<dim3((unsigned)grid, 1, 1), KK_THREADS, smem_kk, s>>>(map_a, map_b, map_c, p, b_resident, tma_store);
+            launch_chained(gemm_tc_kk_kernel<KIND, true>, dim3((unsigned)grid, 1, 1), KK_THREADS, smem_kk, s, map_a, map_b, map_c, p, b_resident, tma_store);
             MIXGCN_CUDA(cudaGetLastError());
             return MIXGCN_OK;
         }
         MIXGCN_CUDA(cudaFuncSetAttribute(gemm_tc_kk_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_kk));
         LaunchScope scope(ctx, PH_GEMM, s);
-        gemm_tc_kk_kernel<KIND><<<dim3((unsigned)grid, 1, 1), KK_THREADS, smem_kk, s>>>(map_a, map_b, map_c, p, b_resident, tma_store);
+        launch_chained(gemm_tc_kk_kernel<KIND>, dim3((unsigned)grid, 1, 1), KK_THREADS, smem_kk, s, map_a, map_b, map_c, p, b_resident, tma_store);
         MIXGCN_CUDA(cudaGetLastError());
         if (bits_done) *bits_done = p.epi.sign_bits != nullptr;
         return MIXGCN_OK;
@@ -1265,7 +1275,7 @@ mixgcn_status launch_kind(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64_t N,
     MIXGCN_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<KIND, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     {
         LaunchScope scope(ctx, PH_GEMM, s);
-        gemm_tc_kernel<KIND, true><<<dim3((unsigned)tiles, 1, (unsigned)splits), TC_THREADS, smem, s>>>(map_a, map_b, p);
+        launch_chained(gemm_tc_kernel<KIND, true>, dim3((unsigned)tiles, 1, (unsigned)splits), TC_THREADS, smem, s, map_a, map_b, p);
     }
     MIXGCN_CUDA(cudaGetLastError());
     if (splits > 1) MIXGCN_TRY(launch_splitk_reduce(ctx, M, N, splits, p.C, C, ldc, epi, s));
@@ -1305,7 +1315,7 @@ mixgcn_status launch_to_bf16(mixgcn_ctx* ctx, int64_t rows, int32_t d, const flo
     if (rows <= 0 || d <= 0) return MIXGCN_OK;
     const int d4 = (d + 3) / 4;
     LaunchScope scope(ctx, PH_ELEM, s);
-    to_bf16_kernel<<<(unsigned)((rows * d4 + 255) / 256), 256, 0, s>>>(rows, d4, src, ld_src, d, dst, ld_dst);
+    launch_chained(to_bf16_kernel, dim3((unsigned)((rows * d4 + 255) / 256)), 256, 0, s, rows, d4, src, ld_src, d, dst, ld_dst);
     MIXGCN_CUDA(cudaGetLastError());
     return MIXGCN_OK;
 }

@@ -19,6 +19,7 @@ __device__ __forceinline__ unsigned nonzero_bytes(uint32_t x) { return __popc(__
 // Train nodes of the mask; integers, so the order of the atomics does not matter.  Sixteen mask bytes per load where the
 // mask is aligned (2.4 M nodes: 6.5 -> 2.5 us).
 __global__ void __launch_bounds__(256) count_mask_kernel(int64_t n, const uint8_t* __restrict__ mask, unsigned long long* count) {
+    chain_begin();
     __shared__ unsigned int sm[8];
     unsigned int c = 0;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
@@ -43,6 +44,7 @@ __global__ void __launch_bounds__(256) count_mask_kernel(int64_t n, const uint8_
 constexpr int64_t COUNT_ONE_BLOCK_MAX = 1 << 17;
 __global__ void __launch_bounds__(1024) count_mask_small_kernel(int64_t n, const uint8_t* __restrict__ mask, unsigned long long* count,
                                                                unsigned int* done, unsigned long long* clear) {
+    chain_begin();
     __shared__ unsigned int sm[32];
     unsigned int c = 0;
     const int64_t n16 = (reinterpret_cast<uintptr_t>(mask) & 15u) == 0 ? n >> 4 : 0;
@@ -65,6 +67,13 @@ __global__ void __launch_bounds__(1024) count_mask_small_kernel(int64_t n, const
     }
 }
 
+// A few words, in the chain of launches (a memset between two kernels takes 5 us from the one's end to the other's start).
+__global__ void __launch_bounds__(32) clear_kernel(uint32_t* words, int n_words, int64_t* also) {
+    chain_begin();
+    if ((int)threadIdx.x < n_words) words[threadIdx.x] = 0;
+    if (threadIdx.x == 0 && also) *also = 0;
+}
+
 // Sum of `blocks` partials by one block of `threads` threads, in a fixed order: thread t takes t, t + threads, ..., then a
 // tree.  Valid in thread 0.
 template <int THREADS>
@@ -85,6 +94,7 @@ __global__ void __launch_bounds__(LOSS_WARPS * 32) loss_rows_kernel(
     int64_t n, int C, const float* logits, int64_t ld, const int32_t* __restrict__ labels,
     const uint8_t* __restrict__ mask, const unsigned long long* __restrict__ count, float* dlogits,
     int32_t* __restrict__ pred, unsigned long long* n_correct, double* __restrict__ part, int32_t* status, bool zero_rows) {
+    chain_begin();
     __shared__ double sm[LOSS_WARPS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned long long T = *count;
@@ -151,6 +161,7 @@ __global__ void __launch_bounds__(LOSS_WARPS * 32) loss_rows_vec_kernel(
     int64_t n, int C, const float* logits, int64_t ld, const int32_t* __restrict__ labels,
     const uint8_t* __restrict__ mask, const unsigned long long* __restrict__ count, float* dlogits,
     int32_t* __restrict__ pred, unsigned long long* n_correct, double* __restrict__ part, int32_t* status, bool zero_rows) {
+    chain_begin();
     __shared__ double sm[LOSS_WARPS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned long long T = *count;
@@ -265,6 +276,7 @@ __global__ void __launch_bounds__(LOSS_WARPS * 32) loss_rows_subset_kernel(
     int64_t n, int C, const float* logits, int64_t ld, const int32_t* __restrict__ labels,
     const uint8_t* __restrict__ mask, const unsigned long long* __restrict__ count, float* dlogits,
     int32_t* __restrict__ pred, unsigned long long* n_correct, double* __restrict__ part, int32_t* status) {
+    chain_begin();
     __shared__ double sm[LOSS_WARPS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned long long T = *count;
@@ -357,6 +369,7 @@ __global__ void __launch_bounds__(ROWS * LOSS_LANES_PER_ROW) loss_rows_tile_kern
     const uint8_t* __restrict__ mask, const unsigned long long* __restrict__ count, float* dlogits,
     int32_t* __restrict__ pred, unsigned long long* n_correct, double* __restrict__ part, int32_t* status,
     bool zero_rows, int64_t n_tiles) {
+    chain_begin();
     constexpr int THREADS = ROWS * LOSS_LANES_PER_ROW;
     extern __shared__ __align__(128) unsigned char loss_smem[];
     float* const tile0 = reinterpret_cast<float*>(loss_smem);
@@ -498,7 +511,7 @@ cudaError_t launch_loss_tile(int grid, size_t smem, cudaStream_t s, int64_t n, i
                              int64_t n_tiles) {
     cudaError_t e = cudaFuncSetAttribute(loss_rows_tile_kernel<ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    loss_rows_tile_kernel<ROWS><<<grid, ROWS * LOSS_LANES_PER_ROW, smem, s>>>(n, C, logits, ld, labels, mask, count, dlogits, pred, n_correct, part,
+    launch_chained(loss_rows_tile_kernel<ROWS>, dim3(grid), ROWS * LOSS_LANES_PER_ROW, smem, s, n, C, logits, ld, labels, mask, count, dlogits, pred, n_correct, part,
                                                          status, zero_rows, n_tiles);
     return cudaGetLastError();
 }
@@ -534,11 +547,11 @@ int launch_loss_rows(unsigned warp_blocks, cudaStream_t s, int64_t n, int C, con
         return e == cudaSuccess ? (int)grid : -1;
     }
     if (vec && C <= 128)
-        loss_rows_vec_kernel<1><<<warp_blocks, LOSS_WARPS * 32, 0, s>>>(n, C, logits, ld, labels, mask, count, dlogits, pred, n_correct, part, status, zero_rows);
+        launch_chained(loss_rows_vec_kernel<1>, dim3(warp_blocks), LOSS_WARPS * 32, 0, s, n, C, logits, ld, labels, mask, count, dlogits, pred, n_correct, part, status, zero_rows);
     else if (vec && C <= 256)
-        loss_rows_vec_kernel<2><<<warp_blocks, LOSS_WARPS * 32, 0, s>>>(n, C, logits, ld, labels, mask, count, dlogits, pred, n_correct, part, status, zero_rows);
+        launch_chained(loss_rows_vec_kernel<2>, dim3(warp_blocks), LOSS_WARPS * 32, 0, s, n, C, logits, ld, labels, mask, count, dlogits, pred, n_correct, part, status, zero_rows);
     else
-        loss_rows_kernel<<<warp_blocks, LOSS_WARPS * 32, 0, s>>>(n, C, logits, ld, labels, mask, count, dlogits, pred, n_correct, part, status, zero_rows);
+        launch_chained(loss_rows_kernel, dim3(warp_blocks), LOSS_WARPS * 32, 0, s, n, C, logits, ld, labels, mask, count, dlogits, pred, n_correct, part, status, zero_rows);
     return cudaGetLastError() == cudaSuccess ? (int)warp_blocks : -1;
 }
 
@@ -551,6 +564,7 @@ __device__ __forceinline__ void store_loss(double sum, unsigned long long T, flo
 
 __global__ void __launch_bounds__(LOSS_FINAL_THREADS) loss_final_kernel(int blocks, const double* __restrict__ part,
                                                                        const unsigned long long* __restrict__ count, float* loss, int32_t* status) {
+    chain_begin();
     __shared__ double sm[LOSS_FINAL_THREADS];
     const double t = sum_partials<LOSS_FINAL_THREADS>(part, blocks, sm);
     if (threadIdx.x == 0) store_loss(t, *count, loss, status);
@@ -565,6 +579,7 @@ __global__ void __launch_bounds__(FUSE_REDUCE_THREADS) loss_rows_reduce_kernel(
     int64_t n, int C, int64_t chunk, const uint8_t* __restrict__ mask, const int32_t* __restrict__ labels,
     const float* __restrict__ row_loss, const int32_t* __restrict__ pred, double* part,
     unsigned long long* n_correct, unsigned int* done, const unsigned long long* __restrict__ count, float* loss, int32_t* status) {
+    chain_begin();
     __shared__ bool last;
     __shared__ double sm[FUSE_REDUCE_THREADS];
     __shared__ unsigned int sc[FUSE_REDUCE_THREADS / 32];
@@ -613,6 +628,7 @@ struct AdamBatch {
 };
 
 __global__ void adam_kernel(const AdamBatch b) {
+    chain_begin();
     const int t = blockIdx.y;
     if (t >= b.count) return;
     const int64_t nel = b.numel[t];
@@ -632,20 +648,26 @@ __global__ void adam_kernel(const AdamBatch b) {
 
 namespace mixgcn {
 
+mixgcn_status launch_clear(mixgcn_ctx* ctx, int phase, void* words, int n_words, int64_t* also, cudaStream_t s) {
+    LaunchScope scope(ctx, phase, s);
+    launch_chained(clear_kernel, dim3(1), 32, 0, s, static_cast<uint32_t*>(words), n_words, also);
+    MIXGCN_CUDA(cudaGetLastError());
+    return MIXGCN_OK;
+}
+
 // *count = train nodes; the word behind it (blocks that have finished) and *n_correct (nullable) are cleared.
 static mixgcn_status count_train_nodes(mixgcn_ctx* ctx, int64_t n, const uint8_t* train_mask, unsigned long long* count,
                                        int64_t* n_correct, cudaStream_t s) {
     if (n <= COUNT_ONE_BLOCK_MAX) {
         LaunchScope scope(ctx, PH_LOSS, s);
-        count_mask_small_kernel<<<1, 1024, 0, s>>>(n, train_mask, count, reinterpret_cast<unsigned int*>(count + 1),
+        launch_chained(count_mask_small_kernel, dim3(1), 1024, 0, s, n, train_mask, count, reinterpret_cast<unsigned int*>(count + 1),
                                                   reinterpret_cast<unsigned long long*>(n_correct));
     } else {
-        MIXGCN_CUDA(cudaMemsetAsync(count, 0, 2 * sizeof(unsigned long long), s));
-        if (n_correct) MIXGCN_CUDA(cudaMemsetAsync(n_correct, 0, sizeof(int64_t), s));
+        MIXGCN_TRY(launch_clear(ctx, PH_LOSS, count, 4, n_correct, s));
         LaunchScope scope(ctx, PH_LOSS, s);
         int64_t cb = (n / 16 + 255) / 256;
         if (cb > (int64_t)ctx->sm_count * 8) cb = (int64_t)ctx->sm_count * 8;
-        count_mask_kernel<<<(unsigned)cb, 256, 0, s>>>(n, train_mask, count);
+        launch_chained(count_mask_kernel, dim3((unsigned)cb), 256, 0, s, n, train_mask, count);
     }
     MIXGCN_CUDA(cudaGetLastError());
     return MIXGCN_OK;
@@ -675,7 +697,7 @@ mixgcn_status loss_fuse_end(mixgcn_ctx* ctx, int64_t n, int32_t C, const LossFus
     const int64_t chunk = (n + lf.n_part - 1) / lf.n_part;
     {
         LaunchScope scope(ctx, PH_LOSS, s);
-        loss_rows_reduce_kernel<<<(unsigned)lf.n_part, FUSE_REDUCE_THREADS, 0, s>>>(n, C, chunk, lf.train_mask, lf.labels, lf.row_loss, lf.pred, lf.part,
+        launch_chained(loss_rows_reduce_kernel, dim3((unsigned)lf.n_part), FUSE_REDUCE_THREADS, 0, s, n, C, chunk, lf.train_mask, lf.labels, lf.row_loss, lf.pred, lf.part,
                                                                                   reinterpret_cast<unsigned long long*>(n_correct),
                                                                                   const_cast<unsigned int*>(reinterpret_cast<const unsigned int*>(lf.count + 1)), lf.count, loss, ctx->d_status);
     }
@@ -706,7 +728,7 @@ extern "C" mixgcn_status mixgcn_loss_softmax_xent(mixgcn_ctx* ctx, int64_t n, in
     {
         LaunchScope scope(ctx, PH_LOSS, s);
         if (ctx->loss_train_rows_only == 1)
-            loss_rows_subset_kernel<<<(unsigned)blocks, LOSS_WARPS * 32, 0, s>>>(n, C, logits, ld, labels, train_mask, count, dlogits, pred,
+            launch_chained(loss_rows_subset_kernel, dim3((unsigned)blocks), LOSS_WARPS * 32, 0, s, n, C, logits, ld, labels, train_mask, count, dlogits, pred,
                                                                               reinterpret_cast<unsigned long long*>(n_correct), part, ctx->d_status);
         else
             n_part = launch_loss_rows((unsigned)blocks, s, n, C, logits, ld, labels, train_mask, count, dlogits, pred,
@@ -716,7 +738,7 @@ extern "C" mixgcn_status mixgcn_loss_softmax_xent(mixgcn_ctx* ctx, int64_t n, in
     if (n_part < 0) MIXGCN_FAIL(MIXGCN_ECUDA, "loss: kernel launch failed: %s", cudaGetErrorString(cudaGetLastError()));
     {
         LaunchScope scope(ctx, PH_LOSS, s);
-        loss_final_kernel<<<1, LOSS_FINAL_THREADS, 0, s>>>(n_part, part, count, loss, ctx->d_status);
+        launch_chained(loss_final_kernel, dim3(1), LOSS_FINAL_THREADS, 0, s, n_part, part, count, loss, ctx->d_status);
     }
     MIXGCN_CUDA(cudaGetLastError());
     return MIXGCN_OK;
@@ -750,7 +772,7 @@ extern "C" mixgcn_status mixgcn_adam_step(mixgcn_ctx* ctx, int32_t n_tensors, fl
         b.inv_c1 = (float)(1.0 / c1); b.inv_c2 = (float)(1.0 / c2);
         int64_t bx = (mx + 255) / 256; if (bx > 1024) bx = 1024;
         LaunchScope scope(ctx, PH_ADAM, s);
-        adam_kernel<<<dim3((unsigned)bx, (unsigned)b.count), 256, 0, s>>>(b);
+        launch_chained(adam_kernel, dim3((unsigned)bx, (unsigned)b.count), 256, 0, s, b);
     }
     MIXGCN_CUDA(cudaGetLastError());
     return MIXGCN_OK;
@@ -820,13 +842,13 @@ extern "C" mixgcn_status mixgcn_loss_softmax_xent_noalloc(int64_t n, int32_t C, 
     if (n_correct) MIXGCN_CUDA(cudaMemsetAsync(n_correct, 0, sizeof(int64_t), s));
     int64_t cb = (n + 255) / 256;
     if (cb > 4096) cb = 4096;
-    count_mask_kernel<<<(unsigned)cb, 256, 0, s>>>(n, train_mask, &sc->count);
+    launch_chained(count_mask_kernel, dim3((unsigned)cb), 256, 0, s, n, train_mask, &sc->count);
     int sm_count = 0;
     MIXGCN_CUDA(cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, device));
     const int n_part = launch_loss_rows((unsigned)blocks, s, n, C, logits, ld, labels, train_mask, &sc->count, dlogits, pred,
                                         reinterpret_cast<unsigned long long*>(n_correct), sc->part, &sc->status, true, sm_count);
     if (n_part < 0) MIXGCN_FAIL(MIXGCN_ECUDA, "loss_noalloc: kernel launch failed: %s", cudaGetErrorString(cudaGetLastError()));
-    loss_final_kernel<<<1, LOSS_FINAL_THREADS, 0, s>>>(n_part, sc->part, &sc->count, loss, &sc->status);
+    launch_chained(loss_final_kernel, dim3(1), LOSS_FINAL_THREADS, 0, s, n_part, sc->part, &sc->count, loss, &sc->status);
     if (status) MIXGCN_CUDA(cudaMemcpyAsync(status, &sc->status, sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
     MIXGCN_CUDA(cudaGetLastError());
     return MIXGCN_OK;

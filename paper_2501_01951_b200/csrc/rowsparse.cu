@@ -28,6 +28,7 @@ __global__ void check_count_kernel(const int64_t* selected, int64_t expected, in
 // dst[i, :] = src[idx[i], :], float4 wide (ld multiples of 4, 16-byte aligned), d4 = ceil(d/4) groups per row
 __global__ void gather_rows_kernel(int64_t count, int d4, const int32_t* __restrict__ idx, const float* __restrict__ src,
                                    int64_t ld_src, float* __restrict__ dst, int64_t ld_dst, int64_t n_rows, int32_t* status) {
+    chain_begin();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= count * d4) return;
     const int64_t i = t / d4; const int c = (int)(t % d4);
@@ -48,6 +49,7 @@ __global__ void count_rows_kernel(int64_t n, const uint8_t* __restrict__ mask, u
 // dst[idx[i], :] = src[i, :]
 __global__ void scatter_rows_kernel(int64_t count, int d4, const int32_t* __restrict__ idx, const float* __restrict__ src,
                                     int64_t ld_src, float* __restrict__ dst, int64_t ld_dst, int64_t n_rows, int32_t* status) {
+    chain_begin();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= count * d4) return;
     const int64_t i = t / d4; const int c = (int)(t % d4);
@@ -94,7 +96,7 @@ mixgcn_status launch_gather_rows(mixgcn_ctx* ctx, int64_t n_rows, int64_t count,
     if (count <= 0) return MIXGCN_OK;
     const int d4 = (d + 3) / 4;
     LaunchScope scope(ctx, PH_ELEM, s);
-    gather_rows_kernel<<<(unsigned)((count * d4 + 255) / 256), 256, 0, s>>>(count, d4, idx, src, ld_src, dst, ld_dst, n_rows, ctx->d_status);
+    launch_chained(gather_rows_kernel, dim3((unsigned)((count * d4 + 255) / 256)), 256, 0, s, count, d4, idx, src, ld_src, dst, ld_dst, n_rows, ctx->d_status);
     MIXGCN_CUDA(cudaGetLastError());
     return MIXGCN_OK;
 }
@@ -104,7 +106,7 @@ mixgcn_status launch_scatter_rows(mixgcn_ctx* ctx, int64_t n_rows, int64_t count
     if (count <= 0) return MIXGCN_OK;
     const int d4 = (d + 3) / 4;
     LaunchScope scope(ctx, PH_ELEM, s);
-    scatter_rows_kernel<<<(unsigned)((count * d4 + 255) / 256), 256, 0, s>>>(count, d4, idx, src, ld_src, dst, ld_dst, n_rows, ctx->d_status);
+    launch_chained(scatter_rows_kernel, dim3((unsigned)((count * d4 + 255) / 256)), 256, 0, s, count, d4, idx, src, ld_src, dst, ld_dst, n_rows, ctx->d_status);
     MIXGCN_CUDA(cudaGetLastError());
     return MIXGCN_OK;
 }

@@ -320,11 +320,8 @@ struct Cfg {
     static constexpr int U = U0 > LPR ? LPR : U0;   // gathered rows in flight per lane group
 };
 
-// Programmatic dependent launch.  The launches of one aggregation call are independent of each other but for the
-// combination of the segments: every kernel lets its successor start at once (trigger), and before it ends it waits
-// for its predecessor's completion (wait), so that "the last launch has completed" still means that all of them have.
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The launches of one aggregation call are independent of each other but for the combination of the segments: every kernel lets its
+// successor start at once, and waits for its predecessor's completion only before it ends.
 
 // Accumulate entries [b, e) into acc[] for the lane's column groups, ascending entry order.
 // The (col, val) pair of the NEXT batch of LPR entries is requested before the current batch's gathers,

@@ -77,3 +77,34 @@ def test_column_blocks_of_large_graphs(mg, n):
         assert rel_fro(Z.double().cpu().numpy(), want.cpu().numpy()) <= TOL_FP32
     assert mg.ctx_poll_status(ctx, raise_on_error=False) == 0
     g.close(); ctx.close()
+
+
+@pytest.mark.parametrize("w", [65, 68, 93, 96, 97, 129, 132, 157, 192, 193])
+def test_three_float4_a_lane(w):
+    """Widths on either side of where lanes hold three float4: every column is the one that a wider call (two or four float4 a lane, entries in
+    the same order) computes, bit for bit, in every bucket of rows and for segments of long rows, with the lean and the general epilogue."""
+    from paper_2501_01951_b200 import binding as mg, synth
+    ctx = mg.ctx_create(0)
+    try:
+        n = 30011
+        src, dst = synth.rmat_graph(n, 400_000, 17)
+        g = mg.graph_create(ctx, n, src, dst)
+        gen = torch.Generator(device="cuda").manual_seed(w)
+        wide = 256 if w > 128 else 128
+        Y = torch.randn((n, wide), generator=gen, device="cuda")
+        bias, gate = torch.randn(wide, generator=gen, device="cuda"), torch.randn((n, wide), generator=gen, device="cuda")
+        ld = (w + 3) // 4 * 4
+        Yn = torch.full((n, ld), float("nan"), device="cuda")
+        Yn[:, :w] = Y[:, :w]
+        for epi in (lambda c: None, lambda c: mg.make_epilogue(bias=bias[:c].clone(), relu=True),
+                    lambda c: mg.make_epilogue(gate=gate[:, :c].contiguous() if c % 4 == 0 else torch.nn.functional.pad(gate[:, :c], (0, ld - w)), gate_scale=2.0),
+                    lambda c: mg.make_epilogue(residual=gate, residual_scale=0.5)):
+            a, b = torch.full((n, wide), 3.0, device="cuda"), torch.full((n, ld), 3.0, device="cuda")
+            ea, eb = epi(wide), epi(w)
+            mg.spmm(ctx, g, Y, a, wide, epi=ea)
+            mg.spmm(ctx, g, Yn, b, w, epi=eb)
+            assert torch.equal(a[:, :w], b[:, :w])
+        g.close()
+        assert mg.ctx_poll_status(ctx, raise_on_error=False) == 0
+    finally:
+        ctx.close()

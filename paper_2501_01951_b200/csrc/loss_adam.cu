@@ -154,111 +154,117 @@ __global__ void __launch_bounds__(LOSS_WARPS * 32) loss_rows_kernel(
     }
 }
 
-// Same computation for C <= 128 * VPL with the row held in registers: one float4-vectorised read of the
-// logits, one float4 write of the gradient (requires ld % 4 == 0 and 16-byte aligned pointers).
-template <int VPL>
+// Same computation for C <= 4 * LPR * VPL with the row held in registers: LPR lanes take a row (32 / LPR rows a warp), one
+// float4-vectorised read of the logits, one float4 write of the gradient (requires ld % 4 == 0 and 16-byte aligned pointers).
+// The next rows' logits, mask bytes and labels are requested before the current ones are reduced.  Bound: instructions (the arg-max's
+// shuffles; with a warp for every row, whatever its width, twice to three times as many: rows of 47 with a pitch of 52, 30 % in the
+// mask, 400 K 115 -> 80 us; rows of 20, 1 M 209 -> 75).
+template <int LPR, int VPL>
 __global__ void __launch_bounds__(LOSS_WARPS * 32) loss_rows_vec_kernel(
     int64_t n, int C, const float* logits, int64_t ld, const int32_t* __restrict__ labels,
     const uint8_t* __restrict__ mask, const unsigned long long* __restrict__ count, float* dlogits,
     int32_t* __restrict__ pred, unsigned long long* n_correct, double* __restrict__ part, int32_t* status, bool zero_rows) {
     chain_begin();
+    constexpr int ROWS = 32 / LPR;
+    constexpr bool AHEAD = LPR < 32;       // (a label for every row costs more than it hides where a warp takes one: 309 -> 335 us at 1 M x 172)
     __shared__ double sm[LOSS_WARPS];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lig = lane % LPR, sub = lane / LPR;
     const unsigned long long T = *count;
     const float invT = T ? (float)(1.0 / (double)T) : 0.0f;
     const int C4 = (C + 3) >> 2;
     double local = 0.0;
     unsigned int correct = 0;
-    const int64_t stride = (int64_t)gridDim.x * LOSS_WARPS;
-    // the next row's loads are issued before the current row is reduced, so two rows per warp are in flight
-    auto load_row = [&](int64_t v, float4 (&t)[VPL]) {
+    const int64_t stride = (int64_t)gridDim.x * LOSS_WARPS * ROWS;
+    float4 nxt[VPL];
+    uint8_t nxt_mask = 0; int nxt_y = 0;
+    auto load_row = [&](int64_t v) {
         const float4* row4 = reinterpret_cast<const float4*>(logits + v * ld);
 #pragma unroll
         for (int q = 0; q < VPL; ++q) {
-            const int g = lane + 32 * q;
-            t[q] = (v < n && g < C4) ? row4[g] : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+            const int g = lig + LPR * q;
+            nxt[q] = (v < n && g < C4) ? row4[g] : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
         }
+        if (AHEAD && v < n) { nxt_mask = mask[v]; nxt_y = labels[v]; }
     };
-    float4 nxt[VPL];
-    load_row((int64_t)blockIdx.x * LOSS_WARPS + warp, nxt);
-    for (int64_t v = (int64_t)blockIdx.x * LOSS_WARPS + warp; v < n; v += stride) {
+    int64_t v0 = ((int64_t)blockIdx.x * LOSS_WARPS + warp) * ROWS;
+    load_row(v0 + sub);
+    for (; v0 < n; v0 += stride) {                                 // (the whole warp together)
+        const int64_t v = v0 + sub;
+        const bool in = v < n;
         float x[VPL][4];
 #pragma unroll
         for (int q = 0; q < VPL; ++q) {
-            const int g = lane + 32 * q;
+            const int g = lig + LPR * q;
             x[q][0] = nxt[q].x; x[q][1] = nxt[q].y; x[q][2] = nxt[q].z; x[q][3] = nxt[q].w;
 #pragma unroll
             for (int e = 0; e < 4; ++e) if (g * 4 + e >= C) x[q][e] = -INFINITY;   // pad columns are not data
         }
-        load_row(v + stride, nxt);
+        const bool train = in && (AHEAD ? nxt_mask : mask[v]) != 0 && T != 0;
+        const int y = AHEAD ? nxt_y : train ? labels[v] : 0;
+        load_row(v + stride);
         float mx = -INFINITY; int arg = 0x7FFFFFFF;
 #pragma unroll
         for (int q = 0; q < VPL; ++q)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const int c = (lane + 32 * q) * 4 + e;
+                const int c = (lig + LPR * q) * 4 + e;
                 if (c < C && (x[q][e] > mx || (x[q][e] == mx && c < arg))) { mx = x[q][e]; arg = c; }
             }
-        if (arg == 0x7FFFFFFF) arg = lane * 4 < C ? lane * 4 : 0;
+        if (arg == 0x7FFFFFFF) arg = lig * 4 < C ? lig * 4 : 0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
+        for (int o = LPR / 2; o > 0; o >>= 1) {
             const float omx = __shfl_xor_sync(0xFFFFFFFFu, mx, o);
             const int oarg = __shfl_xor_sync(0xFFFFFFFFu, arg, o);
             if (omx > mx || (omx == mx && oarg < arg)) { mx = omx; arg = oarg; }
         }
-        if (pred && lane == 0) pred[v] = arg;
-        const bool train = mask[v] != 0 && T != 0;
-        int y = 0;
-        bool ok = false;
-        if (train) {
-            y = labels[v];
-            ok = y >= 0 && y < C;
-            if (!ok && lane == 0) atomicMax(status, DEV_BAD_LABEL);
-        }
-        float4* out4 = dlogits ? reinterpret_cast<float4*>(dlogits + v * ld) : nullptr;
-        if (!train || !ok) {
-            if (out4 && (zero_rows || train)) {
+        if (pred && in && lig == 0) pred[v] = arg;
+        const bool ok = train && y >= 0 && y < C;
+        if (train && !ok && lig == 0) atomicMax(status, DEV_BAD_LABEL);
+        if (!__any_sync(0xFFFFFFFFu, ok)) {
+            if (dlogits && in && (zero_rows || train)) {
 #pragma unroll
-                for (int q = 0; q < VPL; ++q) {
-                    const int g = lane + 32 * q;
-                    if (g < C4) out4[g] = make_float4(0.f, 0.f, 0.f, 0.f);
-                }
+                for (int q = 0; q < VPL; ++q)
+                    if (lig + LPR * q < C4) reinterpret_cast<float4*>(dlogits + v * ld)[lig + LPR * q] = make_float4(0.f, 0.f, 0.f, 0.f);
             }
             continue;
         }
-        float s = 0.0f;
+        float s = 0.0f, py = 0.0f;
 #pragma unroll
         for (int q = 0; q < VPL; ++q)
 #pragma unroll
             for (int e = 0; e < 4; ++e)
-                if ((lane + 32 * q) * 4 + e < C) s += expf(x[q][e] - mx);
+                if ((lig + LPR * q) * 4 + e < C) s += expf(x[q][e] - mx);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+        for (int o = LPR / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
         const float lse = mx + logf(s);
-        // the label's logit lives in lane (y/4) % 32, slot (y/4) / 32, element y % 4
-        float py = 0.0f;
+        // the label's logit lives in lane (y/4) % LPR of the row, slot (y/4) / LPR, element y % 4
 #pragma unroll
         for (int q = 0; q < VPL; ++q)
 #pragma unroll
             for (int e = 0; e < 4; ++e)
-                if ((lane + 32 * q) * 4 + e == y) py = x[q][e];
-        py = __shfl_sync(0xFFFFFFFFu, py, (y >> 2) & 31);
-        if (lane == 0) { local += (double)(lse - py); if (arg == y) ++correct; }
-        if (out4) {
+                if ((lig + LPR * q) * 4 + e == y) py = x[q][e];
+        py = __shfl_sync(0xFFFFFFFFu, py, (y >> 2) & (LPR - 1), LPR);
+        if (ok && lig == 0) { local += (double)(lse - py); if (arg == y) ++correct; }
+        if (!dlogits || !in || !(ok || zero_rows || train)) continue;
 #pragma unroll
-            for (int q = 0; q < VPL; ++q) {
-                const int g = lane + 32 * q;
-                if (g < C4) {
-                    float r[4];
+        for (int q = 0; q < VPL; ++q) {
+            const int g = lig + LPR * q;
+            if (g < C4) {
+                float r[4];
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int c = g * 4 + e;
-                        r[e] = c < C ? (expf(x[q][e] - lse) - (c == y ? 1.0f : 0.0f)) * invT : 0.0f;
-                    }
-                    out4[g] = make_float4(r[0], r[1], r[2], r[3]);
+                for (int e = 0; e < 4; ++e) {
+                    const int c = g * 4 + e;
+                    r[e] = ok && c < C ? (expf(x[q][e] - lse) - (c == y ? 1.0f : 0.0f)) * invT : 0.0f;
                 }
+                reinterpret_cast<float4*>(dlogits + v * ld)[g] = make_float4(r[0], r[1], r[2], r[3]);
             }
         }
+    }
+    // the rows of a warp in order, then its share of the block
+#pragma unroll
+    for (int o = LPR; o < 32; o <<= 1) {
+        local += __shfl_down_sync(0xFFFFFFFFu, local, o);
+        correct += __shfl_down_sync(0xFFFFFFFFu, correct, o);
     }
     if (lane == 0) sm[warp] = local;
     if (n_correct && lane == 0 && correct) atomicAdd(n_correct, (unsigned long long)correct);
@@ -531,8 +537,9 @@ int launch_loss_rows(unsigned warp_blocks, cudaStream_t s, int64_t n, int C, con
     // The tile kernel treats a tile as one dense piece of rows x ld floats (it copies and zeroes whole
     // rows), so it is taken only when the row holds nothing but its C columns and their pad to a multiple
     // of 4; a wider ld (a column slice of a larger buffer) goes to the per-row kernels, which touch columns
-    // below round4(C) only.
-    if (vec && sm_count > 0 && C >= 8 && ld == ((int64_t)C + 3) / 4 * 4 && 2 * 32 * ld * 4 <= TILE_SMEM) {
+    // below round4(C) only.  Up to 32 columns eight lanes of the per-row kernel are as fast with few train rows and faster with many (1 M x 20:
+    // 75 and 103 us with 1 and 50 % of them against 75 and 167); above, they are slower with few (2.4 M x 47, 1 %: 311 against 234).
+    if (vec && sm_count > 0 && C > 32 && ld == ((int64_t)C + 3) / 4 * 4 && 2 * 32 * ld * 4 <= TILE_SMEM) {
         const int rows = 2 * 128 * ld * 4 <= TILE_SMEM ? 128 : (2 * 64 * ld * 4 <= TILE_SMEM ? 64 : 32);
         const int64_t n_tiles = (n + rows - 1) / rows;
         int64_t per_sm = (220 * 1024) / (2 * rows * ld * 4 + 1024);
@@ -546,10 +553,11 @@ int launch_loss_rows(unsigned warp_blocks, cudaStream_t s, int64_t n, int C, con
                                     : launch_loss_tile<32>((int)grid, smem, s, n, C, logits, ld, labels, mask, count, dlogits, pred, n_correct, part, status, zero_rows, n_tiles);
         return e == cudaSuccess ? (int)grid : -1;
     }
-    if (vec && C <= 128)
-        launch_chained(loss_rows_vec_kernel<1>, dim3(warp_blocks), LOSS_WARPS * 32, 0, s, n, C, logits, ld, labels, mask, count, dlogits, pred, n_correct, part, status, zero_rows);
-    else if (vec && C <= 256)
-        launch_chained(loss_rows_vec_kernel<2>, dim3(warp_blocks), LOSS_WARPS * 32, 0, s, n, C, logits, ld, labels, mask, count, dlogits, pred, n_correct, part, status, zero_rows);
+    auto rows_vec = [&](auto kernel) { launch_chained(kernel, dim3(warp_blocks), LOSS_WARPS * 32, 0, s, n, C, logits, ld, labels, mask, count, dlogits, pred, n_correct, part, status, zero_rows); };
+    if (vec && C <= 32) rows_vec(loss_rows_vec_kernel<8, 1>);
+    else if (vec && C <= 64) rows_vec(loss_rows_vec_kernel<16, 1>);
+    else if (vec && C <= 128) rows_vec(loss_rows_vec_kernel<32, 1>);
+    else if (vec && C <= 256) rows_vec(loss_rows_vec_kernel<32, 2>);
     else
         launch_chained(loss_rows_kernel, dim3(warp_blocks), LOSS_WARPS * 32, 0, s, n, C, logits, ld, labels, mask, count, dlogits, pred, n_correct, part, status, zero_rows);
     return cudaGetLastError() == cudaSuccess ? (int)warp_blocks : -1;

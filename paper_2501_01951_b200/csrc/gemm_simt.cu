@@ -436,15 +436,34 @@ __global__ void __launch_bounds__(SimtCfg<BM, BN, TN, KG>::NT, SimtCfg<BM, BN, T
 
 // C[m][n] = epilogue( sum_z part[z][m][n] ) in fp64.  A block owns 32 consecutive elements; its eight rows of threads add
 // an eighth of the splits each (ascending), the eighths are added in order: a hundred splits of a small weight gradient
-// cost one thread a chain of a hundred loads otherwise (16 K elements, 148 splits: 20 -> 4 us).
+// cost one thread a chain of a hundred loads otherwise (16 K elements, 148 splits: 20 -> 4 us).  The blocks behind those add up the partial
+// column sums that came with the product, if any, in the same way: a launch of its own took 4 us.
 constexpr int RED_PARTS = 8;
 __global__ void __launch_bounds__(32 * RED_PARTS) splitk_reduce_kernel(int64_t M, int64_t N, int splits, const float* __restrict__ part,
-                                                                      float* __restrict__ C, int64_t ldc, const Epi epi, const int32_t* only_if) {
+                                                                      float* __restrict__ C, int64_t ldc, const Epi epi, const int32_t* only_if, const ColSums sums) {
     chain_begin();
     if (only_if && *only_if == 0) return;
     __shared__ double sm[RED_PARTS][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t i = (int64_t)blockIdx.x * 32 + lane, MN = M * N;
+    const int64_t MN = M * N, blocks = (MN + 31) / 32;
+    if (blockIdx.x >= blocks) {
+        const int64_t n = ((int64_t)blockIdx.x - blocks) * 32 + lane;
+        const int per = (sums.splits + RED_PARTS - 1) / RED_PARTS;
+        const int z0 = w * per, z1 = z0 + per < sums.splits ? z0 + per : sums.splits;
+        double s = 0.0;
+        if (n < N) {
+#pragma unroll 4
+            for (int z = z0; z < z1; ++z) s += __ldg(sums.part + (int64_t)z * N + n);
+        }
+        sm[w][lane] = s;
+        __syncthreads();
+        if (w != 0 || n >= N) return;
+#pragma unroll
+        for (int q = 1; q < RED_PARTS; ++q) s += sm[q][lane];
+        sums.out[n] = (float)s;
+        return;
+    }
+    const int64_t i = (int64_t)blockIdx.x * 32 + lane;
     const int per = (splits + RED_PARTS - 1) / RED_PARTS;
     const int z0 = w * per, z1 = z0 + per < splits ? z0 + per : splits;
     double s = 0.0;
@@ -641,7 +660,7 @@ mixgcn_status launch_gemm_simt(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64
     if (splits > 1) {
         LaunchScope scope(ctx, PH_GEMM, s);
         const int64_t total = M * N;
-        launch_chained(splitk_reduce_kernel, dim3((unsigned)((total + 31) / 32)), 32 * RED_PARTS, 0, s, M, N, (int)splits, p.C, C, ldc, p.epi, only_if);
+        launch_chained(splitk_reduce_kernel, dim3((unsigned)((total + 31) / 32)), 32 * RED_PARTS, 0, s, M, N, (int)splits, p.C, C, ldc, p.epi, only_if, ColSums{});
         MIXGCN_CUDA(cudaGetLastError());
     } else if (bits_done) {
         *bits_done = p.epi.sign_bits != nullptr;
@@ -650,7 +669,7 @@ mixgcn_status launch_gemm_simt(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64
 }
 
 mixgcn_status launch_splitk_reduce(mixgcn_ctx* ctx, int64_t M, int64_t N, int splits, const float* part, float* C,
-                                   int64_t ldc, const mixgcn_epilogue* epi, cudaStream_t s) {
+                                   int64_t ldc, const mixgcn_epilogue* epi, cudaStream_t s, const ColSums& sums) {
     Epi e{};
     if (epi) {
         e.bias = epi->bias; e.relu = epi->relu; e.drop = epi->drop_mask; e.keep_scale = epi->keep_scale;
@@ -658,8 +677,8 @@ mixgcn_status launch_splitk_reduce(mixgcn_ctx* ctx, int64_t M, int64_t N, int sp
         e.gate_bits = epi->gate_bits; e.ld_gate_bits = epi->ld_gate_bits;
     }
     LaunchScope scope(ctx, PH_GEMM, s);
-    const int64_t total = M * N;
-    launch_chained(splitk_reduce_kernel, dim3((unsigned)((total + 31) / 32)), 32 * RED_PARTS, 0, s, M, N, splits, part, C, ldc, e, nullptr);
+    const int64_t blocks = (M * N + 31) / 32 + (sums.out ? (N + 31) / 32 : 0);
+    launch_chained(splitk_reduce_kernel, dim3((unsigned)blocks), 32 * RED_PARTS, 0, s, M, N, splits, part, C, ldc, e, nullptr, sums);
     MIXGCN_CUDA(cudaGetLastError());
     return MIXGCN_OK;
 }

@@ -894,11 +894,10 @@ mixgcn_status launch_gemm_split(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int6
         launch_chained(gemm_split_mm_kernel, dim3((unsigned)tiles, 1, (unsigned)splits), THREADS, smem, s, map_a, map_b, p);
     }
     MIXGCN_CUDA(cudaGetLastError());
-    if (colsum_b) {
-        MIXGCN_TRY(launch_colsum_splits(ctx, N, (int)(splits * p.m_tiles), p.colsum_part, colsum_b, s));
-        if (colsum_done) *colsum_done = true;
-    }
-    if (splits > 1) MIXGCN_TRY(launch_splitk_reduce(ctx, M, N, (int)splits, p.C, C, ldc, nullptr, s));
+    const ColSums sums = colsum_b ? ColSums{p.colsum_part, (int)(splits * p.m_tiles), colsum_b} : ColSums{};
+    if (splits > 1) MIXGCN_TRY(launch_splitk_reduce(ctx, M, N, (int)splits, p.C, C, ldc, nullptr, s, sums));
+    else if (colsum_b) MIXGCN_TRY(launch_colsum_splits(ctx, N, sums.splits, sums.part, sums.out, s));
+    if (colsum_b && colsum_done) *colsum_done = true;
     return MIXGCN_OK;
 }
 

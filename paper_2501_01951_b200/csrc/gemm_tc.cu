@@ -1278,11 +1278,10 @@ mixgcn_status launch_kind(mixgcn_ctx* ctx, int ta, int tb, int64_t M, int64_t N,
         launch_chained(gemm_tc_kernel<KIND, true>, dim3((unsigned)tiles, 1, (unsigned)splits), TC_THREADS, smem, s, map_a, map_b, p);
     }
     MIXGCN_CUDA(cudaGetLastError());
-    if (splits > 1) MIXGCN_TRY(launch_splitk_reduce(ctx, M, N, splits, p.C, C, ldc, epi, s));
-    if (fuse_colsum) {
-        MIXGCN_TRY(launch_colsum_splits(ctx, N, (int)(splits * p.m_tiles), p.colsum_part, colsum_b, s));
-        if (colsum_done) *colsum_done = true;
-    }
+    const ColSums sums = fuse_colsum ? ColSums{p.colsum_part, (int)(splits * p.m_tiles), colsum_b} : ColSums{};
+    if (splits > 1) MIXGCN_TRY(launch_splitk_reduce(ctx, M, N, splits, p.C, C, ldc, epi, s, sums));
+    else if (fuse_colsum) MIXGCN_TRY(launch_colsum_splits(ctx, N, sums.splits, sums.part, sums.out, s));
+    if (fuse_colsum && colsum_done) *colsum_done = true;
     return MIXGCN_OK;
 }
 

@@ -351,8 +351,9 @@ mixgcn_status launch_gemm_tc(mixgcn_ctx* ctx, int kind, int ta, int tb, int64_t 
 // bits[u][j] = (X == null || X[u][j] > 0) && (bytes == null || bytes[u*w + j] != 0), n x ld_bits words
 mixgcn_status launch_mask_pack(mixgcn_ctx* ctx, int64_t n, int32_t w, const float* X, int64_t ldx, const uint8_t* bytes,
                                uint32_t* bits, int64_t ld_bits, cudaStream_t s);
+struct ColSums { const double* part = nullptr; int splits = 0; float* out = nullptr; };       // out[n] = sum of part[z][n], z < splits
 mixgcn_status launch_splitk_reduce(mixgcn_ctx* ctx, int64_t M, int64_t N, int splits, const float* part, float* C,
-                                   int64_t ldc, const mixgcn_epilogue* epi, cudaStream_t s);
+                                   int64_t ldc, const mixgcn_epilogue* epi, cudaStream_t s, const ColSums& sums = ColSums{});
 mixgcn_status launch_to_bf16(mixgcn_ctx* ctx, int64_t rows, int32_t d, const float* src, int64_t ld_src, uint16_t* dst,
                              int64_t ld_dst, cudaStream_t s);
 mixgcn_status launch_colsum(mixgcn_ctx* ctx, int64_t n, int32_t d, const float* X, int64_t ld, float* out,

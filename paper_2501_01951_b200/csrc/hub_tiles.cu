@@ -596,7 +596,8 @@ mixgcn_status build_tiles(const mixgcn_graph* g, bool transposed, HubTiles** out
     if (clusters > (t->n_tiles + LEAST_TILES - 1) / LEAST_TILES) clusters = (t->n_tiles + LEAST_TILES - 1) / LEAST_TILES;
     t->clusters = clusters;
     t->rem_nnz = g->nnz - t->entries;
-    if (!hub_tiles_pay(t, n, HUB_SLICE)) return MIXGCN_OK;
+    // (one width of every lane split)
+    if (!hub_tiles_pay(t, n, HUB_SLICE) && !hub_tiles_pay(t, n, 160) && !hub_tiles_pay(t, n, 128) && !hub_tiles_pay(t, n, 64)) return MIXGCN_OK;
     std::vector<HubPiece> pieces;
     std::vector<int32_t> first_piece(clusters + 1), piece_first(t->row_blocks + 1, 0);
     int rb = 0;
@@ -663,22 +664,23 @@ void release_tiles(mixgcn_graph* g) {
     free_tiles(f);
 }
 
-// Whether an aggregation of w columns is faster with the tiles, by what both sides take (ns).  A gathered entry: 0.05 per 256 columns,
-// no less than 0.008 (the ones in tiles are those the L1 and L2 serve).  The tiles: 2.0 us at 256 columns and 1.25 at 64 and less for each of a
-// pair, 20 us and the images for the launches, and a look at its rank for every row.  The line lies where a sixteenth of the call is
-// gained; measured without : with (us), R-MAT graphs:
-//   233 K nodes of mean degree 500   256 columns 5050 : 2300, 128 3340 : 1260, 41 1740 : 925
-//   2.4 M of 52                      256 8200 : 7400, 100 4490 : 3680, 47 2870 : 2360
-//   700 K of 22, 130 columns 926 : 880, 400 K of 31, 100 columns 406 : 378, 300 K of 31, 256 columns 565 : 533
-// and left to the gather kernels: 6 M of 18, 128 columns 4530 : 4530 (DRAM bounds both), 700 K of 22, 47 columns 306 : 345, 150 K of 22, 128
-// columns 132 : 140 and 33 columns 84 : 104.
+// Whether an aggregation of w columns is faster with the tiles, by what both sides take (ns).  A gathered entry: steps where the lane split
+// of the gather kernels changes.  The tiles: 2.0 us at 256 columns and 1.25 at 64 and less for each of a pair; for the launches the images and
+// 55 us above 128 columns, 25 from 65 on, 20 below (the pieces' partial rows); a look at its rank for every row.
+// The line lies where a sixteenth of the call is gained; measured without : with (us), R-MAT graphs:
+//   233 K nodes of mean degree 500   256 columns 5035 : 2302, 132 4646 : 1680, 128 3216 : 1258, 48 1608 : 863, 32 1286 : 767
+//   2.4 M of 52                      192 7065 : 5904, 132 6403 : 4980, 128 4422 : 3878, 48 2813 : 2397
+//   300 K of 31                      256 549 : 538, 132 459 : 403, 128 313 : 284;  400 K of 31  132 588 : 556, 100 414 : 384
+//   100 K of 106                     256 492 : 400, 128 307 : 231, 64 193 : 171
+// and left to the gather kernels: 700 K of 22  256 1001 : 1046, 132 789 : 814, 100 561 : 562;  1.5 M of 21  256 2193 : 2347, 132 1810 : 1776;
+// 300 K of 31  64 205 : 206, 48 178 : 185;  100 K of 106  32 137 : 148;  6 M of 18  128 4342 : 4319 (DRAM bounds both).
 bool hub_tiles_pay(const HubTiles* t, int64_t n, int32_t w) {
     const int32_t last = w % HUB_SLICE, slices = w / HUB_SLICE;
-    auto entry = [](int32_t c) { return c > 40 ? 0.0002 * c : c > 0 ? 0.008 : 0.0; };
+    auto entry = [](int32_t c) { return c > 128 ? 0.036 + 0.00003 * (c - 128) : c > 64 ? 0.022 + 0.00008 * (c - 64) : c > 40 ? 0.0002 * c : c > 0 ? 0.008 : 0.0; };
     auto tile = [](int32_t c) { return c > 64 ? 1000.0 + 3.9 * c : c > 0 ? 1250.0 : 0.0; };
+    auto launch = [&](int32_t c) { return c > 0 ? (c > 128 ? 55e3 : c > 64 ? 25e3 : 20e3) + 0.5 * t->n_cols / HUB_SLICE * c : 0.0; };
     const double per_entry = slices * entry(HUB_SLICE) + entry(last), per_tile = slices * tile(HUB_SLICE) + tile(last);
-    const double launches = (slices + (last > 0)) * 20e3 + 0.5 * t->n_cols / HUB_SLICE * w, ranks = 0.025 * n;
-    const double gain = per_entry * t->entries - per_tile * t->n_tiles / t->clusters - launches - ranks;
+    const double gain = per_entry * t->entries - per_tile * t->n_tiles / t->clusters - slices * launch(HUB_SLICE) - launch(last) - (w > 64 ? 0.06 : 0.025) * n;
     return gain * 16 > per_entry * (t->entries + t->rem_nnz);
 }
 

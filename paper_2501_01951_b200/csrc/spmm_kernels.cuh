@@ -470,7 +470,7 @@ __device__ __forceinline__ unsigned kept_groups(const Params& p, int64_t u, int 
 
 // FULL (plain and bit-gate instances): the slice has exactly LPR * VPL column groups, so no load is predicated on its column.
 template <int LPR, int VPL, int EPI = EPI_ANY, bool FULL = false>
-__global__ void __launch_bounds__(256, VPL <= 2 || (VPL == 3 && LPR >= 8 && LPR <= 16) ? SPMM_MINB : 1) spmm_group_kernel(const Params p) {
+__global__ void __launch_bounds__(256, VPL <= 2 ? SPMM_MINB : VPL == 3 && LPR >= 8 && LPR <= 16 ? (EPI == EPI_ANY ? SPMM_MINB - 1 : SPMM_MINB) : 1) spmm_group_kernel(const Params p) {
     constexpr bool LOSS = EPI == EPI_LOSS, PLAIN = epi_is_lean(EPI);
     pdl_trigger();
     const int lig = threadIdx.x % LPR;
@@ -805,14 +805,15 @@ void launch_group(const Params& p, cudaStream_t s, bool early) {
     // (one float4 per lane: the lean instances gain nothing there and the assembler spills a register in them)
     constexpr bool lean = !LOSS && VPL >= 2;
     if constexpr (lean) {
-        const bool full = LPR >= 8 && ((p.w + 3) >> 2) == LPR * VPL;     // (narrow groups: nothing to gain)
+        constexpr bool FULL = LPR >= 8 && VPL != 3;                      // (narrow groups: nothing to gain; three float4: spills)
+        const bool full = FULL && ((p.w + 3) >> 2) == LPR * VPL;
         switch (pick_epi(p)) {
             case EPI_PLAIN:
-                if (full) launch_k(spmm_group_kernel<LPR, VPL, EPI_PLAIN, (LPR >= 8)>, (unsigned)blocks, s, early, p);
+                if (full) launch_k(spmm_group_kernel<LPR, VPL, EPI_PLAIN, FULL>, (unsigned)blocks, s, early, p);
                 else launch_k(spmm_group_kernel<LPR, VPL, EPI_PLAIN>, (unsigned)blocks, s, early, p);
                 return;
             case EPI_BITS:
-                if (full) launch_k(spmm_group_kernel<LPR, VPL, EPI_BITS, (LPR >= 8)>, (unsigned)blocks, s, early, p);
+                if (full) launch_k(spmm_group_kernel<LPR, VPL, EPI_BITS, FULL>, (unsigned)blocks, s, early, p);
                 else launch_k(spmm_group_kernel<LPR, VPL, EPI_BITS>, (unsigned)blocks, s, early, p);
                 return;
             case EPI_BIAS: launch_k(spmm_group_kernel<LPR, VPL, EPI_BIAS>, (unsigned)blocks, s, early, p); return;

@@ -58,7 +58,7 @@ struct TileParams {
     const int32_t* tile_cb; const uint4* bits;
     float* partial; int64_t ldp;                        // row r of piece q goes to partial row q * ROWS + r
     int w4, bn, chunks, stages;
-    const int32_t* unsafe;                              // not zero: plain_pieces instead, from what follows
+    int32_t* unsafe;                                    // flag: not zero, plain_pieces instead, from what follows; then the CTAs done with it
     const float* Y; int64_t ldy, y_rows;
     const int32_t* nodes; const float* col_scale; int64_t n_cols;
     int32_t* status;
@@ -343,6 +343,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1) spmm_til
     tc_fence_before();
     __syncthreads();
     cluster_sync_all();                  // the peer is done with this CTA's shared and tensor memory
+    if (threadIdx.x == 0) {              // the flag is this call's alone: the last CTA that has read it clears it
+        __threadfence();
+        if (atomicInc(reinterpret_cast<unsigned int*>(p.unsafe) + 1, gridDim.x - 1) == gridDim.x - 1) *p.unsafe = 0;      // (back at zero itself)
+    }
     if (warp == MMA_WARP) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
@@ -353,14 +357,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1) spmm_til
 // columns], a chunk as the tensor core wants it in shared memory.  Eight lanes a row and chunk, eight columns each.  The product by
 // the scale is cut with its rounding error added to the last part, so the scaling itself rounds nothing.
 __global__ void __launch_bounds__(256) split_rows_kernel(int64_t n_cols, int kblocks, int chunks, int nh, int w, const int32_t* __restrict__ nodes, const float* __restrict__ scale,
-                                                         const float* __restrict__ Y, int64_t ldy, int64_t y_rows, uint8_t* __restrict__ images, int32_t* unsafe, int32_t* next_unsafe, int32_t* status) {
+                                                         const float* __restrict__ Y, int64_t ldy, int64_t y_rows, uint8_t* __restrict__ images, int32_t* unsafe, int32_t* status) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
     const int g = (int)(i & 7), k = (int)((i >> 3) & (COLS - 1));
     const int64_t kc = (i >> 3) / COLS, kb = kc / (2 * chunks);
     const int chunk = (int)(kc % (2 * chunks)), half = chunk / chunks, in_half = (chunk - half * chunks) * 64 + g * 8;
     const int c0 = in_half < nh ? half * nh + in_half : w;
-    if (i == 0) *next_unsafe = 0;
     if (kb >= kblocks) return;
     float x[8], lost[8];
 #pragma unroll
@@ -703,11 +706,7 @@ mixgcn_status launch_hub_tiles(mixgcn_ctx* ctx, const HubTiles* t, int phase, in
     p.w4 = (w + 3) >> 2; p.bn = half_cols(w) * 2; p.chunks = half_chunks(w);
     const int fit = STAGE_SMEM / (p.chunks * CHUNK_BYTES);
     p.stages = fit < STAGES_MAX ? fit : STAGES_MAX;
-    // two flags in turn, each cleared by the call before the one that uses it (a recording replays its calls' turns: a flag that is
-    // still set from another call sends the product to the FMA pipes, no more)
-    int32_t *unsafe = ctx->d_status + TILES_UNSAFE_WORD + ctx->tiles_turn, *next_unsafe = ctx->d_status + TILES_UNSAFE_WORD + (ctx->tiles_turn ^ 1);
-    ctx->tiles_turn ^= 1;
-    p.unsafe = unsafe;
+    p.unsafe = ctx->d_status + TILES_UNSAFE_WORD;
     p.Y = Y; p.ldy = ldy; p.y_rows = y_rows; p.nodes = t->nodes; p.col_scale = t->col_scale; p.n_cols = t->n_cols;
     p.status = ctx->d_status;
     p.wait_limit = ctx->debug_wait_limit > 0 ? (uint32_t)ctx->debug_wait_limit : WAIT_LIMIT_DEFAULT;
@@ -718,8 +717,8 @@ mixgcn_status launch_hub_tiles(mixgcn_ctx* ctx, const HubTiles* t, int phase, in
     {
         LaunchScope scope(ctx, phase, s);
         const int64_t threads = (int64_t)t->kblocks * COLS * 2 * p.chunks * 8;
-        split_rows_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(t->n_cols, t->kblocks, p.chunks, p.bn / 2, w, t->nodes, t->col_scale, Y, ldy, y_rows, images, unsafe,
-                                                                            next_unsafe, ctx->d_status);
+        split_rows_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(t->n_cols, t->kblocks, p.chunks, p.bn / 2, w, t->nodes, t->col_scale, Y, ldy, y_rows, images, p.unsafe,
+                                                                            ctx->d_status);
     }
     const size_t smem = 2 * A_BYTES + (size_t)p.stages * p.chunks * CHUNK_BYTES + EPI_WARPS * BOX_BYTES + 1024;
     MIXGCN_CUDA(cudaFuncSetAttribute(spmm_tiles_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

@@ -80,7 +80,7 @@ inline void memory_given_back(const MemoryGeneration& m) { if (m) m->fetch_add(1
 
 }  // namespace mixgcn
 
-constexpr int STATUS_WORDS = 32, SPLIT_OVERFLOW_WORD = 16, TILES_UNSAFE_WORD = 17;    // (two words)
+constexpr int STATUS_WORDS = 32, SPLIT_OVERFLOW_WORD = 16, TILES_UNSAFE_WORD = 17;    // (two words: flag, count)
 
 struct mixgcn_ctx {
     int device;
@@ -106,7 +106,6 @@ struct mixgcn_ctx {
     int no_cta_pairs;         // 1: keep every product on single CTAs (option, for comparison)
     int debug_wait_limit;     // > 0: polls after which the tensor-core kernels' waits give up (test of that path)
     int debug_drop_load;      // 1, 2: tensor-core products leave one stage unfilled (test of that path)
-    int tiles_turn;           // which of the two flags the next product of hub tiles uses
     int spmm_slice_cols;      // 0 = default (one slice up to 1024 columns)
     int loss_train_rows_only; // 1 = the loss skips rows outside the train mask entirely
     // profiling

@@ -181,3 +181,32 @@ def test_small_and_sparse_graphs_have_no_tiles(mg, ctx):
         g = mg.graph_create(ctx, n, e[0].contiguous(), e[1].contiguous())
         assert mg.graph_prepare_tiles(g) == (0, 0)
         g.close()
+
+
+@pytest.mark.parametrize("products", [1, 3])
+def test_a_value_that_the_parts_cannot_hold_leaves_nothing_to_later_replays(mg, ctx, graphs, products):
+    """Recordings with one and with three products: a replay whose last input held an infinity, then replays of the finite inputs, which
+    give the bits of the calls; calls after a recording as well."""
+    _, tiled, _ = graphs["sym", True]
+    hub = mg.graph_degrees(tiled).argsort(descending=True)[700]
+    Ys = [features(256, 20 + k) for k in range(products)]
+    Zs = [torch.empty_like(Y) for Y in Ys]
+
+    def calls():
+        for Y, Z in zip(Ys, Zs):
+            mg.spmm(ctx, tiled, Y, Z, 256)
+
+    calls()
+    want = [Z.clone() for Z in Zs]
+    rec = mg.record(ctx, calls)
+    assert rec.replay()
+    kept = Ys[-1][hub].clone()
+    Ys[-1][hub, 9] = float("inf")
+    assert rec.replay()
+    Ys[-1][hub] = kept
+    for again in (rec.replay, rec.replay, calls):
+        for Z in Zs:
+            Z.zero_()
+        again()
+        assert all(torch.equal(Z, w) for Z, w in zip(Zs, want))
+    rec.close()

@@ -6,7 +6,7 @@
 //
 //  * An entry's value is row_scale[u] * col_scale[v] (both normalisations and the plain sum have that form), so the matrix that is
 //    multiplied holds zeros and ones only: exact in bf16.
-//  * Rows of Y are scaled by col_scale and cut into three bf16 parts, x = x0 + x1 + x2 (24 bits, as in gemm_split.cu), once per
+//  * Rows of Y are scaled by col_scale (and 2^24, see CUT_SCALE) and cut into three bf16 parts, x = x0 + x1 + x2 (24 bits, as in gemm_split.cu), once per
 //    call, into images of the shared-memory tiles (split_rows_kernel): a stage of the product is one contiguous copy a CTA.
 //  * The x0 (8 bits each) are summed in an accumulator of their own, the two smaller parts in another: an instruction cuts its sum off
 //    at 24 bits, towards zero, and sums of a few hundred 8-bit numbers have next to nothing to lose there.  Every 256 terms (the
@@ -51,7 +51,10 @@ constexpr int AHEAD = 4;
 constexpr int LEAST_TILES = 8;                  // of a pair of CTAs
 constexpr int HI_TILES = 2, LO_TILES = 8;        // tiles an accumulator takes
 constexpr uint32_t LO_COL = 256;                // TMEM: sums of the largest parts in columns 0-255, of the other two behind
-constexpr float SAFE_MAX = 1.2676506e30f;       // 2^100: sums of 2^16 such terms stay finite
+constexpr float SAFE_MAX = 0x1p100f;             // sums of 2^16 such terms stay finite
+// Rows of Y are cut this many times as large: bf16 has nothing below 2^-133, and the third part of a number of 2^-110 and less would
+// be gone (numbers of 1e-35: error 2e-6 to 1e-5 without, 2e-8 as the gathers have it with; 2^24 brings all of fp32 above the line).
+constexpr float CUT_SCALE = 0x1p24f;
 
 struct TileParams {
     const HubPiece* pieces; const int32_t* first_piece; // pair i takes pieces first_piece[i] .. first_piece[i + 1] - 1
@@ -120,7 +123,7 @@ __device__ __forceinline__ uint4 expand8(uint32_t word, int j) {
     return make_uint4(r[0], r[1], r[2], r[3]);
 }
 
-// A pair's pieces on the FMA pipes, for calls in which a row of Y holds an infinity, a NaN or a number above 2^100, whose parts and sums
+// A pair's pieces on the FMA pipes, for calls in which a row of Y holds an infinity, a NaN or a number above 2^76, whose parts and sums
 // the tensor core would not keep apart (0 * infinity): the expansion warps, one per row of a piece, entries in the order of their bits.
 __device__ __forceinline__ void plain_pieces(const TileParams& p, int q0, int q1, int rank) {
     const int lane = threadIdx.x & 31;
@@ -235,7 +238,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1) spmm_til
                 if (k < chunks) {
 #pragma unroll
                     for (int i = 0; i < 8; ++i)
-                        *reinterpret_cast<float4*>(box + lane * 128 + ((i ^ (lane & 7)) << 4)) = make_float4(sum[k][i * 4], sum[k][i * 4 + 1], sum[k][i * 4 + 2], sum[k][i * 4 + 3]);
+                        *reinterpret_cast<float4*>(box + lane * 128 + ((i ^ (lane & 7)) << 4)) =
+                            make_float4(sum[k][i * 4] * (1 / CUT_SCALE), sum[k][i * 4 + 1] * (1 / CUT_SCALE), sum[k][i * 4 + 2] * (1 / CUT_SCALE), sum[k][i * 4 + 3] * (1 / CUT_SCALE));
                     __syncwarp();
                     const int c4 = (n0 >> 2) + k * 8 + (lane & 7);
                     if (c4 < p.w4) {
@@ -374,7 +378,7 @@ __global__ void __launch_bounds__(256) split_rows_kernel(int64_t n_cols, int kbl
         if (index_ok(v, y_rows, status, SITE_SPMM_COL)) {
             const float4* src = reinterpret_cast<const float4*>(Y + v * ldy + c0);
             const float4 a = __ldg(src), c = c0 + 4 < w ? __ldg(src + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
-            const float s = __ldg(scale + h), y[8] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w};
+            const float s = __ldg(scale + h) * CUT_SCALE, y[8] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w};
             bool bad = false;
 #pragma unroll
             for (int j = 0; j < 8; ++j)

@@ -210,3 +210,18 @@ def test_a_value_that_the_parts_cannot_hold_leaves_nothing_to_later_replays(mg, 
         again()
         assert all(torch.equal(Z, w) for Z, w in zip(Zs, want))
     rec.close()
+
+
+@pytest.mark.parametrize("norm", ["sym", "none"])
+def test_the_smallest_numbers_keep_their_bits(mg, ctx, graphs, norm):
+    """Columns from 1e-38, where terms fall below fp32's normal range, up to 1e22, the largest that the parts hold: no further from fp64
+    than the gather kernels, a tenth for the noise of one draw."""
+    plain, tiled, A = graphs[norm, True]
+    w = 64
+    Y = features(w, 12) * 10.0 ** torch.linspace(-38, 22, w, device="cuda")
+    Z, Zp = (torch.empty_like(Y) for _ in range(2))
+    mg.spmm(ctx, tiled, Y, Z, w)
+    mg.spmm(ctx, plain, Y, Zp, w)
+    want = A[0] @ Y.double()
+    err, err_plain = ((z.double() - want).norm(dim=0) for z in (Z, Zp))
+    assert torch.all(err <= 1.1 * err_plain), (err / err_plain)

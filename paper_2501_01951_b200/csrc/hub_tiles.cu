@@ -9,22 +9,27 @@
 //  * Rows of Y are scaled by col_scale (and 2^24, see CUT_SCALE) and cut into three bf16 parts, x = x0 + x1 + x2 (24 bits, as in gemm_split.cu), once per
 //    call, into images of the shared-memory tiles (split_rows_kernel): a stage of the product is one contiguous copy a CTA.
 //  * The x0 (8 bits each) are summed in an accumulator of their own, the two smaller parts in another: an instruction cuts its sum off
-//    at 24 bits, towards zero, and sums of a few hundred 8-bit numbers have next to nothing to lose there.  Every 256 terms (the
-//    smaller parts, 2^-8 of the others: every 1024) the epilogue warps add the accumulator to fp32 sums in registers, rounding to
-//    nearest, while the other one takes the next terms.  (All parts in one accumulator, every 128 terms: a third more error on sums of one sign.)
+//    at 24 bits, towards zero, and sums of a hundred 8-bit numbers have next to nothing to lose there unless their sizes lie far apart.
+//    Every 128 terms (the smaller parts, 2^-8 of the others: every 1024) the epilogue warps add the accumulator to fp32 sums in registers,
+//    rounding to nearest, while others take the next terms: up to 160 columns leave room for two accumulators of the x0, up to 96 for four,
+//    and there every 64 terms have one (narrow gathers add up in short chains, and a tile's time is its hand-overs': + 4 % of it).
 //  * What is not in a tile is a matrix of its own, with a schedule of its own, for the gather kernels.  They run behind the tiles, and where
-//    they have a row's sum add the row's pieces to it (the tiles of one row of tiles that one pair of CTAs takes), times row_scale.
+//    they have a row's sum add the row's pieces to it (at most 64 tiles of one row of tiles each, in fp64), times row_scale.
 //
-// Measured, R-MAT, 233 K nodes of mean degree 500 (20,473 tiles hold 74 % of the entries), 256 columns: 5.05 ms by gathers alone, 2.30 with the
-// tiles (0.55 the product, 0.03 the cut, 1.7 the rest of the matrix); more cases at hub_tiles_pay.
-// Bound: a tile of 256 x 128 by 256 columns takes a pair of CTAs 3,700 cycles, 3,072 of which its 24 instructions need; with 128 columns
-// 2,460 of 1,536, with 64 2,300 (the hand-overs of three stages).  One CTA per tile of 128 x 128 took 5,630, bound by shared memory: a
-// stage's image is written once and read once for 128 rows, here for 256.  What was slow on the way: adding up the accumulator after every
-// tile in loads of 16 columns, 4,550 (every second tile, 32 columns at a time: as above); bitmaps expanded by shift and multiply and
-// announced to the other CTA by the expanding threads, whose arrival there waits for the loads they have under way (2,000 of 2,500 cycles).
-// Error against fp64 (2-norm; gathers alone in brackets): N(0,1) 2.1e-8 (2.2e-8), their positive halves 3.4e-8 (3.5e-8), 300 K nodes,
-// 256 columns.  Row means transposed are left out: the entries of small columns carry a row's sum there, and the rest of the matrix adds
-// them up in fewer and longer chains than the whole one did (positive halves, 30 K nodes: 8.1e-8 (6.8e-8)).
+// Measured, R-MAT, 233 K nodes of mean degree 500 (20,470 tiles hold 74 % of the entries), 256 columns: 5.04 ms by gathers alone, 2.49 with the
+// tiles (0.82 the product, 0.03 the cut, 1.7 the rest of the matrix); more cases at hub_tiles_pay.
+// Bound: a tile of 256 x 128 by 256 columns takes a pair of CTAs 4,800 cycles, 3,072 of which its 24 instructions need; the rest is adding up
+// the accumulator of the x0, which nothing covers above 160 columns (every 256 terms instead: 3,700 cycles, and the error below).  One
+// CTA per tile of 128 x 128 took 5,630, bound by shared memory: a stage's image is written once and read once for 128 rows, here for
+// 256.  Also slow: loads of 16 columns from the accumulator; bitmaps expanded by shift and multiply and announced to the other CTA by the
+// expanding threads, whose arrival there waits for the loads they have under way (2,000 of 2,500 cycles).
+// Error against fp64 relative to the gather kernels' (2-norm; N(0,1), its positive halves, what a ReLU leaves of it):
+// R-MAT 300 K, mean degree 31, 132 columns 0.89, 0.88, 1.03; 60 K, 400 0.78, 0.72, 0.79, plain sums 0.38, 0.80, 0.78; 4,099 nodes, half of
+// their pairs joined, 64 to 256 columns 0.7 to 0.9, 0.4 to 0.7, 0.5 to 0.7.  One row in a thousand 2^15 times the others: 0.7 to 1.0, of
+// one sign 0.8 to 1.05 (60 K, plain sums, 64 columns 1.3).  Numbers of one sign spread further apart (exp(3 N(0,1))) are where
+// truncation shows: 1.0 to 1.7.  What it took: 256 terms an accumulator made the last three 1.2 to 2.9; pieces of any length, added up
+// in fp32, 2.1 of positive plain sums; the gather kernels' chains as they were 1.26 on the 300 K nodes.  Row means transposed are left
+// out: the entries of small columns carry a row's sum there.
 #include <cub/cub.cuh>
 
 #include <mutex>
@@ -49,8 +54,9 @@ constexpr int EPI_REGS = 192, OTHER_REGS = 64;  // a thread's, of the 128 it is 
 constexpr int STAGES_MAX = 8, STAGE_SMEM = 128 * 1024, BOX_BYTES = 4096;
 constexpr int AHEAD = 4;
 constexpr int LEAST_TILES = 8;                  // of a pair of CTAs
-constexpr int HI_TILES = 2, LO_TILES = 8;        // tiles an accumulator takes
-constexpr uint32_t LO_COL = 256;                // TMEM: sums of the largest parts in columns 0-255, of the other two behind
+constexpr int LO_TILES = 8;                     // tiles that the accumulator of the smaller parts takes; that of the largest takes one
+constexpr int PIECE_MAX = 64;                   // tiles of a piece: as many fp32 additions in a row
+constexpr uint32_t TMEM_COLS = 512;
 constexpr float SAFE_MAX = 0x1p100f;             // sums of 2^16 such terms stay finite
 // Rows of Y are cut this many times as large: bf16 has nothing below 2^-133, and the third part of a number of 2^-110 and less would
 // be gone (numbers of 1e-35: error 2e-6 to 1e-5 without, 2e-8 as the gathers have it with; 2^24 brings all of fp32 above the line).
@@ -61,6 +67,9 @@ struct TileParams {
     const int32_t* tile_cb; const uint4* bits;
     float* partial; int64_t ldp;                        // row r of piece q goes to partial row q * ROWS + r
     int w4, bn, chunks, stages;
+    // TMEM: accumulators of bn columns, those of the largest parts first.  hi_two: 1 if tiles take turns in two sets of them, hi_halves: 1 if
+    // the two halves of a tile's terms have one each; lo_col: the smaller parts' one
+    uint32_t hi_two, hi_halves, lo_col;
     int32_t* unsafe;                                    // flag: not zero, plain_pieces instead, from what follows; then the CTAs done with it
     const float* Y; int64_t ldy, y_rows;
     const int32_t* nodes; const float* col_scale; int64_t n_cols;
@@ -72,7 +81,7 @@ struct TileParams {
 struct Shared {
     uint64_t b_full[STAGES_MAX], b_empty[STAGES_MAX];   // images: TMA -> MMA -> TMA
     uint64_t a_full[2], a_empty[2];                     // expanded tiles: expansion -> MMA -> expansion
-    uint64_t hi_full, hi_empty, lo_full, lo_empty;      // the two accumulators: MMA -> epilogue -> MMA
+    uint64_t hi_full[2], hi_empty[2], lo_full, lo_empty;   // the accumulators: MMA -> epilogue -> MMA
     uint32_t tmem;
     int abort_flag;
 };
@@ -101,8 +110,8 @@ __device__ __forceinline__ bool elect_one() {
 __device__ __forceinline__ void add2(float& x, float& y, uint32_t a, uint32_t b) {
     asm("{.reg .b64 p, q; mov.b64 p, {%0, %1}; mov.b64 q, {%2, %3}; add.rn.f32x2 p, p, q; mov.b64 {%0, %1}, p;}" : "+f"(x), "+f"(y) : "r"(a), "r"(b));
 }
-// Whether an accumulator that takes n tiles is added up after tile t.
-__device__ __forceinline__ bool sum_ends(const HubPiece& piece, int t, int n) { return t + 1 == piece.end || (t - piece.begin) % n == n - 1; }
+// Whether the accumulator of the smaller parts is added up after tile i of the n of a piece.
+__device__ __forceinline__ bool lo_ends(uint32_t i, uint32_t n) { return i + 1 == n || i % LO_TILES == LO_TILES - 1; }
 
 // Where the column c (mod 32) of a tile's row has its bit: shifted left by c / 4 it is the highest bit of byte c % 4, and one
 // permutation turns the highest bits of two bytes into the masks of two bf16 (2.5 instructions a pair instead of 5).
@@ -173,12 +182,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1) spmm_til
         b.abort_flag = 0;
         for (int s = 0; s < STAGES_MAX; ++s) { mbar_init(&b.b_full[s], 1); mbar_init(&b.b_empty[s], 1); }
         for (int s = 0; s < 2; ++s) { mbar_init(&b.a_full[s], rank == 0 ? EXP_WARPS + 1 : EXP_WARPS); mbar_init(&b.a_empty[s], 1); }
-        mbar_init(&b.hi_full, 1); mbar_init(&b.hi_empty, 2 * EPI_WARPS); mbar_init(&b.lo_full, 1); mbar_init(&b.lo_empty, 2 * EPI_WARPS);
+        for (int s = 0; s < 2; ++s) { mbar_init(&b.hi_full[s], 1); mbar_init(&b.hi_empty[s], 2 * EPI_WARPS); }
+        mbar_init(&b.lo_full, 1); mbar_init(&b.lo_empty, 2 * EPI_WARPS);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     if (warp == MMA_WARP) {
-        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&b.tmem)), "r"(512u) : "memory");
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&b.tmem)), "r"(TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
@@ -197,9 +207,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1) spmm_til
         const int hw = ((p.bn + 1) / 2 + 31) & ~31;                      // columns of a half: a multiple of 32, at most 128
         const int n0 = half * hw, chunks = n0 >= p.bn ? 0 : (min(hw, p.bn - n0) + 31) / 32;
         const uint32_t lanes = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)n0;
-        const uint32_t hi_empty = mapa_shared(smem_u32(&b.hi_empty), 0), lo_empty = mapa_shared(smem_u32(&b.lo_empty), 0);
         uint8_t* const box = stages + (size_t)p.stages * stage_bytes + warp * BOX_BYTES;
-        uint32_t hi_use = 0, lo_use = 0;
+        uint32_t at = 0, lo_use = 0;            // at: tiles of the pair so far
         bool ok = true;
         for (int q = q0; q < q1 && ok; ++q) {
             const HubPiece piece = p.pieces[q];
@@ -208,27 +217,31 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1) spmm_til
             for (int k = 0; k < 4; ++k)
 #pragma unroll
                 for (int i = 0; i < 32; ++i) sum[k][i] = 0.0f;
-            auto add = [&](uint64_t* full, uint32_t empty, uint32_t& use, uint32_t col) {
+            auto add = [&](uint64_t* full, uint64_t* empty, uint32_t use, uint32_t col, uint32_t col_end) {
                 if (!warp_wait(full, use, b, p)) return false;
                 tc_fence_after();
+#pragma unroll 1
+                for (; col < col_end; col += (uint32_t)p.bn) {
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    if (k < chunks) {
-                        uint32_t r[32];
-                        tc_ld32(lanes + col + k * 32, r);
-                        tc_wait_ld();
+                    for (int k = 0; k < 4; ++k)
+                        if (k < chunks) {
+                            uint32_t r[32];
+                            tc_ld32(lanes + col + k * 32, r);
+                            tc_wait_ld();
 #pragma unroll
-                        for (int i = 0; i < 32; i += 2) add2(sum[k][i], sum[k][i + 1], r[i], r[i + 1]);
-                    }
+                            for (int i = 0; i < 32; i += 2) add2(sum[k][i], sum[k][i + 1], r[i], r[i + 1]);
+                        }
+                }
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive_cluster(empty);
-                use ^= 1;
+                if (lane == 0) mbar_arrive_cluster(mapa_shared(smem_u32(empty), 0));
                 return true;
             };
-            for (int t = piece.begin; t < piece.end && ok; ++t) {
-                if (sum_ends(piece, t, LO_TILES)) ok = add(&b.lo_full, lo_empty, lo_use, LO_COL);
-                if (ok && sum_ends(piece, t, HI_TILES)) ok = add(&b.hi_full, hi_empty, hi_use, 0);
+            const uint32_t first = at, end = at + (uint32_t)(piece.end - piece.begin);
+            for (; at < end && ok; ++at) {
+                if (lo_ends(at - first, end - first)) { ok = add(&b.lo_full, &b.lo_empty, lo_use, p.lo_col, p.lo_col + 1); lo_use ^= 1; }
+                const uint32_t slot = at & p.hi_two, set = (uint32_t)p.bn << p.hi_halves;
+                if (ok) ok = add(&b.hi_full[slot], &b.hi_empty[slot], at >> p.hi_two & 1, slot * set, slot * set + set);
             }
             if (!ok) break;
             // through a box per warp, so that a request stores whole lines (a row per lane instead: 12,000 cycles a piece)
@@ -238,15 +251,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1) spmm_til
                 if (k < chunks) {
 #pragma unroll
                     for (int i = 0; i < 8; ++i)
-                        *reinterpret_cast<float4*>(box + lane * 128 + ((i ^ (lane & 7)) << 4)) =
-                            make_float4(sum[k][i * 4] * (1 / CUT_SCALE), sum[k][i * 4 + 1] * (1 / CUT_SCALE), sum[k][i * 4 + 2] * (1 / CUT_SCALE), sum[k][i * 4 + 3] * (1 / CUT_SCALE));
+                        *reinterpret_cast<float4*>(box + lane * 128 + ((i ^ (lane & 7)) << 4)) = make_float4(sum[k][i * 4], sum[k][i * 4 + 1], sum[k][i * 4 + 2], sum[k][i * 4 + 3]);
                     __syncwarp();
                     const int c4 = (n0 >> 2) + k * 8 + (lane & 7);
                     if (c4 < p.w4) {
 #pragma unroll 2
                         for (int i = 0; i < 8; ++i) {
                             const int row = i * 4 + (lane >> 3);
-                            dst[row * (p.ldp >> 2) + c4] = *reinterpret_cast<const float4*>(box + row * 128 + (((lane & 7) ^ (row & 7)) << 4));
+                            const float4 x = *reinterpret_cast<const float4*>(box + row * 128 + (((lane & 7) ^ (row & 7)) << 4));
+                            dst[row * (p.ldp >> 2) + c4] = make_float4(x.x * (1 / CUT_SCALE), x.y * (1 / CUT_SCALE), x.z * (1 / CUT_SCALE), x.w * (1 / CUT_SCALE));
                         }
                     }
                     __syncwarp();
@@ -309,33 +322,35 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1) spmm_til
         } else if (warp == MMA_WARP && rank == 0) {
             const uint32_t idesc = make_idesc<KIND_BF16>(ROWS, p.bn, false) | (1u << 16);      // A K-major, B MN-major
             Ring st, buf;
-            uint32_t hi_use = 0, lo_use = 0, hi_more = 0, lo_more = 0;       // more: the accumulator holds some already
+            uint32_t lo_use = 0, lo_more = 0;       // lo_more: the accumulator holds some already
             bool ok = true;
             for (int q = q0; q < q1 && ok; ++q) {
                 const HubPiece piece = p.pieces[q];
                 for (int t = piece.begin; t < piece.end && ok; ++t) {
                     ok = warp_wait(&b.a_full[buf.i], buf.use, b, p) && (lo_more || warp_wait(&b.lo_empty, lo_use ^ 1, b, p));
-                    const bool lo_ends = sum_ends(piece, t, LO_TILES), hi_ends = sum_ends(piece, t, HI_TILES);
+                    const bool ends = lo_ends((uint32_t)(t - piece.begin), (uint32_t)(piece.end - piece.begin));
+                    const uint32_t k = (uint32_t)(t - t0), slot = k & p.hi_two;
                     const uint64_t a = make_desc(smem_u32(smem + buf.i * A_BYTES), 16, 1024, 2);
                     for (int s = 0; s < PARTS && ok; ++s) {
                         const bool hi = s == PARTS - 1;
-                        if (!warp_wait(&b.b_full[st.i], st.use, b, p) || (hi && !hi_more && !warp_wait(&b.hi_empty, hi_use ^ 1, b, p))) { ok = false; break; }
+                        if (!warp_wait(&b.b_full[st.i], st.use, b, p) || (hi && !warp_wait(&b.hi_empty[slot], (k >> p.hi_two & 1) ^ 1, b, p))) { ok = false; break; }
                         tc_fence_after();
-                        const uint32_t d = tmem + (hi ? 0u : LO_COL), more = hi ? hi_more : (s ? 1u : lo_more);
+                        const uint32_t d = tmem + (hi ? (slot * (uint32_t)p.bn) << p.hi_halves : p.lo_col), half = hi ? p.hi_halves : 0u, more = s ? 1u : lo_more;
                         const uint64_t bd = make_desc(smem_u32(stages + (size_t)st.i * stage_bytes), CHUNK_BYTES, 1024, 2);
                         if (elect_one()) {
 #pragma unroll
                             for (int j = 0; j < COLS / 16; ++j)
-                                tc_mma_pair<KIND_BF16>(d, a + (j >> 2) * (A_BYTES / 2 / 16) + (j & 3) * 2, bd + j * 128, idesc, j ? 1u : more);
+                                tc_mma_pair<KIND_BF16>(d + (half & j >> 2) * (uint32_t)p.bn, a + (j >> 2) * (A_BYTES / 2 / 16) + (j & 3) * 2, bd + j * 128, idesc,
+                                                       hi ? (j & (half ? 3 : 7)) != 0 : j ? 1u : more);
                             tc_commit_pair(&b.b_empty[st.i], 3);
-                            if (s == PARTS - 2 && lo_ends) tc_commit_pair(&b.lo_full, 3);
+                            if (s == PARTS - 2 && ends) tc_commit_pair(&b.lo_full, 3);
                             if (hi) tc_commit_pair(&b.a_empty[buf.i], 3);
-                            if (hi && hi_ends) tc_commit_pair(&b.hi_full, 3);
+                            if (hi) tc_commit_pair(&b.hi_full[slot], 3);
                         }
                         __syncwarp();
                         st.next(p.stages);
                     }
-                    hi_use ^= hi_ends; lo_use ^= lo_ends; hi_more = !hi_ends; lo_more = !lo_ends;
+                    lo_use ^= ends; lo_more = !ends;
                     buf.next(2);
                 }
             }
@@ -353,7 +368,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1) spmm_til
     }
     if (warp == MMA_WARP) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
     }
 }
 
@@ -604,7 +619,7 @@ mixgcn_status build_tiles(const mixgcn_graph* g, bool transposed, HubTiles** out
     t->clusters = clusters;
     t->rem_nnz = g->nnz - t->entries;
     // (one width of every lane split)
-    if (!hub_tiles_pay(t, n, HUB_SLICE) && !hub_tiles_pay(t, n, 160) && !hub_tiles_pay(t, n, 128) && !hub_tiles_pay(t, n, 64)) return MIXGCN_OK;
+    if (!hub_tiles_pay(t, HUB_SLICE) && !hub_tiles_pay(t, 160) && !hub_tiles_pay(t, 128) && !hub_tiles_pay(t, 64)) return MIXGCN_OK;
     std::vector<HubPiece> pieces;
     std::vector<int32_t> first_piece(clusters + 1), piece_first(t->row_blocks + 1, 0);
     int rb = 0;
@@ -613,7 +628,9 @@ mixgcn_status build_tiles(const mixgcn_graph* g, bool transposed, HubTiles** out
         const int end = (int)((int64_t)t->n_tiles * (c + 1) / clusters);
         for (int at = (int)((int64_t)t->n_tiles * c / clusters); at < end;) {
             while (host_first[(rb + 1) * cbs] <= at) ++rb;
-            const int row_end = host_first[(rb + 1) * cbs], stop = row_end < end ? row_end : end;
+            const int row_end = host_first[(rb + 1) * cbs];
+            int stop = row_end < end ? row_end : end;
+            if (stop > at + PIECE_MAX) stop = at + PIECE_MAX;
             pieces.push_back(HubPiece{rb, at, stop, 0});
             piece_first[rb + 1]++;
             at = stop;
@@ -671,24 +688,31 @@ void release_tiles(mixgcn_graph* g) {
     free_tiles(f);
 }
 
-// Whether an aggregation of w columns is faster with the tiles, by what both sides take (ns).  A gathered entry: steps where the lane split
-// of the gather kernels changes.  The tiles: 2.0 us at 256 columns and 1.25 at 64 and less for each of a pair; for the launches the images and
-// 55 us above 128 columns, 25 from 65 on, 20 below (the pieces' partial rows); a look at its rank for every row.
-// The line lies where a sixteenth of the call is gained; measured without : with (us), R-MAT graphs:
-//   233 K nodes of mean degree 500   256 columns 5035 : 2302, 132 4646 : 1680, 128 3216 : 1258, 48 1608 : 863, 32 1286 : 767
-//   2.4 M of 52                      192 7065 : 5904, 132 6403 : 4980, 128 4422 : 3878, 48 2813 : 2397
-//   300 K of 31                      256 549 : 538, 132 459 : 403, 128 313 : 284;  400 K of 31  132 588 : 556, 100 414 : 384
-//   100 K of 106                     256 492 : 400, 128 307 : 231, 64 193 : 171
-// and left to the gather kernels: 700 K of 22  256 1001 : 1046, 132 789 : 814, 100 561 : 562;  1.5 M of 21  256 2193 : 2347, 132 1810 : 1776;
-// 300 K of 31  64 205 : 206, 48 178 : 185;  100 K of 106  32 137 : 148;  6 M of 18  128 4342 : 4319 (DRAM bounds both).
-bool hub_tiles_pay(const HubTiles* t, int64_t n, int32_t w) {
-    const int32_t last = w % HUB_SLICE, slices = w / HUB_SLICE;
-    auto entry = [](int32_t c) { return c > 128 ? 0.036 + 0.00003 * (c - 128) : c > 64 ? 0.022 + 0.00008 * (c - 64) : c > 40 ? 0.0002 * c : c > 0 ? 0.008 : 0.0; };
-    auto tile = [](int32_t c) { return c > 64 ? 1000.0 + 3.9 * c : c > 0 ? 1250.0 : 0.0; };
-    auto launch = [&](int32_t c) { return c > 0 ? (c > 128 ? 55e3 : c > 64 ? 25e3 : 20e3) + 0.5 * t->n_cols / HUB_SLICE * c : 0.0; };
-    const double per_entry = slices * entry(HUB_SLICE) + entry(last), per_tile = slices * tile(HUB_SLICE) + tile(last);
-    const double gain = per_entry * t->entries - per_tile * t->n_tiles / t->clusters - slices * launch(HUB_SLICE) - launch(last) - (w > 64 ? 0.06 : 0.025) * n;
-    return gain * 16 > per_entry * (t->entries + t->rem_nnz);
+// Whether an aggregation of w columns is faster with the tiles, by what both sides take (us): what the gathers of the tiles' entries would
+// take, against the product, the cut and what the other entries take longer in their own kernels (add_batch; nanoseconds an
+// entry, steps where the lane split changes).  A pair's first 32 tiles are dearer: graphs with few tiles have them spread over many rows and
+// columns, and the images come from DRAM.  Fitted to the profiles of eleven graphs; taken from a 32nd of the call on, where the fit
+// is right about the sign but for 100 K nodes at 48 columns (178 : 181).  Measured without : with (us), mean degree last, entries in tiles in brackets:
+//   R-MAT 233 K, 500 (74 %)    256 columns 5036 : 2494, 132 4542 : 1711, 128 3205 : 1359, 64 1907 : 1002, 32 1284 : 835
+//   R-MAT 2.4 M, 52 (28 %)     256 7846 : 7629, 132 6107 : 5168, 128 4401 : 3926, 48 2766 : 2202
+//   R-MAT 300 K, 31 (34 %)     192 466 : 443, 132 459 : 412;  100 K, 106 (61 %)  256 521 : 430, 128 334 : 253, 64 206 : 188
+//   R-MAT 20 K, 300 (83 %)     256 276 : 165, 64 113 : 87;  8 K of 500 K nodes joined at random (51 %)  256 1907 : 1617, 64 586 : 525
+// and left to the gather kernels: R-MAT 300 K, 31  256 550 : 552, 128 313 : 303, 64 205 : 218;  700 K, 22 (28 %)  256 1002 : 1072,
+// 132 789 : 810, 128 527 : 581;  1.5 M, 21 (23 %)  256 2193 : 2331, 132 1721 : 1711;  ends drawn by rank^-0.6, 300 K, 100 (4 %)  256 2142 : 2396,
+// 128 1022 : 1164, by rank^-0.8, 1 M, 40 (11 %)  256 3315 : 3754, 132 2362 : 2309.
+bool hub_tiles_pay(const HubTiles* t, int32_t w) {
+    const double tiles = (double)t->n_tiles / t->clusters, first = tiles < 32 ? tiles : 32;      // of a pair
+    double all = 0, gain = 0;
+    auto slice = [&](int32_t c) {
+        const double entry = c > 192 ? 0.036 + 0.00003 * (c - 192) : c > 160 ? 0.036 : c > 128 ? 0.037 : c > 64 ? 0.026 : c > 24 ? 0.005 + 0.00016 * c : 0.0088;
+        const double other = c > 192 ? 0.0078 : c > 128 ? 0.0045 : c > 64 ? 0.004 : 0.001;
+        const double product = c > 160 ? (1.72 + 0.0076 * (c - 160)) * tiles + (2.8 + 0.0085 * (c - 160)) * first
+                                       : c > 128 ? 1.72 * tiles + 2.8 * first : c > 64 ? 1.5 * tiles + 2.3 * first : 1.45 * tiles + 1.6 * first;
+        all += entry * 1e-3 * (t->entries + t->rem_nnz);
+        gain += entry * 1e-3 * t->entries - other * 1e-3 * t->rem_nnz - product - 10.0 - 2e-6 * t->n_cols * c;
+    };
+    for (int32_t c0 = 0; c0 < w; c0 += HUB_SLICE) slice(w - c0 < HUB_SLICE ? w - c0 : HUB_SLICE);
+    return gain * 32 > all;
 }
 
 // columns of a half of Y, chunks of 64 of them
@@ -710,6 +734,9 @@ mixgcn_status launch_hub_tiles(mixgcn_ctx* ctx, const HubTiles* t, int phase, in
     p.w4 = (w + 3) >> 2; p.bn = half_cols(w) * 2; p.chunks = half_chunks(w);
     const int fit = STAGE_SMEM / (p.chunks * CHUNK_BYTES);
     p.stages = fit < STAGES_MAX ? fit : STAGES_MAX;
+    p.hi_two = p.bn * 3 <= (int)TMEM_COLS ? 1 : 0;
+    p.hi_halves = p.bn * 5 <= (int)TMEM_COLS ? 1 : 0;
+    p.lo_col = (uint32_t)p.bn << (p.hi_two + p.hi_halves);
     p.unsafe = ctx->d_status + TILES_UNSAFE_WORD;
     p.Y = Y; p.ldy = ldy; p.y_rows = y_rows; p.nodes = t->nodes; p.col_scale = t->col_scale; p.n_cols = t->n_cols;
     p.status = ctx->d_status;

@@ -33,7 +33,7 @@ struct HubTiles {
 
 namespace mixgcn {
 
-bool hub_tiles_pay(const HubTiles* t, int64_t n, int32_t w);
+bool hub_tiles_pay(const HubTiles* t, int32_t w);
 // bytes of scratch for w columns: partial rows of ldp floats, images (of at most 256 columns) from *images_at on
 int64_t hub_tiles_scratch(const HubTiles* t, int32_t w, int64_t ldp, int64_t* images_at);
 // partial rows of the pieces for w <= HUB_SLICE columns: row r of piece q is partial row q * 256 + r, not yet times row_scale

@@ -292,7 +292,7 @@ mixgcn_status launch_spmm(mixgcn_ctx* ctx, const mixgcn_graph* g, const CsrView&
     const HubTiles* tiles = nullptr;
     if (chunks <= 1 && !sparse && !row_filter && row_limit < 0 && !opts.out_bits && (&A == &g->fwd || &A == &g->bwd)) {
         tiles = g->tiles[&A == &g->bwd].load(std::memory_order_acquire);
-        if (tiles && !hub_tiles_pay(tiles, g->n, w)) tiles = nullptr;
+        if (tiles && !hub_tiles_pay(tiles, w)) tiles = nullptr;
     }
     const CsrView& V = tiles ? tiles->rem : A;       // with tiles: what they leave
     const SpmmSchedule& S = chunks > 1 ? A.chunk[k] : V.full;

@@ -225,3 +225,45 @@ def test_the_smallest_numbers_keep_their_bits(mg, ctx, graphs, norm):
     want = A[0] @ Y.double()
     err, err_plain = ((z.double() - want).norm(dim=0) for z in (Z, Zp))
     assert torch.all(err <= 1.1 * err_plain), (err / err_plain)
+
+
+def spreads(n, w, seed):
+    """Signed, of one sign, half zeros as behind a ReLU, and the first two with a row in a thousand 2^15 times the others."""
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    x = torch.randn((n, w), generator=gen, device="cuda")
+    few = 1 + 2.0 ** 15 * (torch.rand((n, 1), generator=gen, device="cuda") < 0.001)
+    return dict(signed=x, positive=x.abs(), relu=x.relu(), signed_mixed=x * few, positive_mixed=x.abs() * few)
+
+
+def compare_errors(mg, ctx, plain, tiled, A, w, transposed=False):
+    """The 2-norm of the error against fp64 is no larger than the gather kernels', but for a tenth: summed over ten draws, since with a few
+    large rows one draw's ratio lies anywhere between half and twice that."""
+    err = {}
+    for seed in range(10):
+        for name, Y in spreads(tiled.n, w, seed).items():
+            want = A @ Y.double()
+            for g in (tiled, plain):
+                Z = torch.empty_like(Y)
+                mg.spmm(ctx, g, Y, Z, w, transposed)
+                err[name, g is tiled] = err.get((name, g is tiled), 0.0) + ((Z.double() - want).norm() / want.norm()).item()
+    for name in spreads(8, 1, 0):
+        print(f"w {w} {name}: {err[name, True] / 10:.2e} gathered {err[name, False] / 10:.2e} ratio {err[name, True] / err[name, False]:.2f}")
+        assert err[name, True] <= 1.1 * err[name, False], name
+
+
+@pytest.mark.parametrize("w", [64, 128, 160, 256])
+@pytest.mark.parametrize("norm,symmetric,transposed", [("sym", True, False), ("row", True, False), ("none", False, False), ("none", False, True)])
+def test_error_no_larger_than_the_gather_kernels(mg, ctx, graphs, norm, symmetric, transposed, w):
+    plain, tiled, A = graphs[norm, symmetric]
+    compare_errors(mg, ctx, plain, tiled, A[transposed], w, transposed)
+
+
+@pytest.mark.parametrize("n,edges,flag", [(300_000, 4_650_000, 0), (60_000, 12_000_000, 0), (60_000, 12_000_000, "GRAPH_NORM_NONE")])
+def test_error_on_graphs_with_hubs(mg, ctx, n, edges, flag):
+    """Rows whose sums are mostly the rest of the matrix; rows of tiles of many pieces, whose sums the hubs decide."""
+    src, dst = synth.rmat_graph(n, edges, 3, device="cuda")
+    flags = mg.GRAPH_SYMMETRISE | (getattr(mg, flag) if flag else mg.GRAPH_ADD_SELF_LOOPS)
+    plain, tiled = (mg.graph_create(ctx, n, src, dst, flags) for _ in range(2))
+    assert mg.graph_prepare_tiles(tiled)[0] > 500
+    compare_errors(mg, ctx, plain, tiled, matrix(mg, tiled, False), 132)
+    plain.close(), tiled.close()

@@ -105,6 +105,9 @@ mixgcn_status mixgcn_debug_poke_col(mixgcn_graph* g, int64_t entry, int32_t valu
  * rows may be converted on the way in (with 1 they go through a bf16 copy).  Nothing traps, spins without limit or faults. */
 #define MIXGCN_OPT_DEBUG_WAIT_LIMIT 3
 #define MIXGCN_OPT_DEBUG_DROP_LOAD 4
+/* Test hook of allocation failures, 0 by default: k > 0 = of the device allocations that the layout of tiles (see
+ * mixgcn_graph_prepare_tiles) asks for from now on, for graphs of this context, the k-th fails as if there were no memory. */
+#define MIXGCN_OPT_DEBUG_FAIL_ALLOC 6
 /* MIXGCN_OPT_GEMM_CTA_PAIRS: 1 (default) = wide and deep K-major products (N >= 512, K >= 512, M >= 4096)
  * run on pairs of CTAs that share one 256 x 256 tile (tcgen05 .cta_group::2); 0 = every product on single
  * CTAs with 128 x 256 tiles.  Same results up to the order of fp32 accumulation inside the tensor core. */

@@ -159,6 +159,7 @@ OPT_SPMM_SLICE_COLS = 1
 OPT_LOSS_TRAIN_ROWS_ONLY = 2
 OPT_DEBUG_WAIT_LIMIT = 3
 OPT_DEBUG_DROP_LOAD = 4
+OPT_DEBUG_FAIL_ALLOC = 6
 OPT_GEMM_CTA_PAIRS = 5
 
 

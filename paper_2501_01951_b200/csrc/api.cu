@@ -364,6 +364,11 @@ extern "C" mixgcn_status mixgcn_ctx_set_option(mixgcn_ctx* ctx, int32_t option, 
         ctx->debug_drop_load = (int)value;
         return MIXGCN_OK;
     }
+    if (option == MIXGCN_OPT_DEBUG_FAIL_ALLOC) {
+        if (value < 0 || value > (1 << 20)) MIXGCN_FAIL(MIXGCN_EINVAL, "ctx_set_option: fail-alloc must lie in [0, 2^20] (got %lld)", (long long)value);
+        ctx->debug_fail_alloc = (int)value;
+        return MIXGCN_OK;
+    }
     MIXGCN_FAIL(MIXGCN_EINVAL, "ctx_set_option: unknown option %d", option);
 }
 

@@ -500,6 +500,7 @@ mixgcn_status ensure_chunk_schedules(const mixgcn_graph* g, const CsrView& A_con
         mixgcn_status st = build_schedule(g->n, g->nnz, A.rowptr, A.col, r0, r1 - r0, sc[k], s);
         if (st == MIXGCN_OK && cudaStreamSynchronize(s) != cudaSuccess) st = MIXGCN_ECUDA;    // usable on every stream from here on
         if (st != MIXGCN_OK) {
+            cudaStreamSynchronize(s);         // kernels that write to them
             for (int q = 0; q <= k; ++q) free_schedule(sc[q]);
             delete[] sc;
             return st;

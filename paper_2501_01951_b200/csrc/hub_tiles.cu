@@ -581,15 +581,20 @@ mixgcn_status build_tiles(const mixgcn_graph* g, bool transposed, HubTiles** out
     const int64_t n = g->n, hubs = n < HUB_MAX ? n : HUB_MAX;
     if (g->nnz < HUB_MIN_ENTRIES) return MIXGCN_OK;
     const int rbs = (int)((hubs + ROWS - 1) / ROWS), cbs = (int)((hubs + COLS - 1) / COLS), total = rbs * cbs;
-    struct Guard { HubTiles* t; ~Guard() { free_tiles(t); } } guard{new (std::nothrow) HubTiles()};
+    // (given back on a failure below only when what writes to them is through: the stream does not wait for the null stream, nor that for it)
+    struct Guard { HubTiles* t; cudaStream_t s; ~Guard() { if (t) cudaStreamSynchronize(s); free_tiles(t); } } guard{new (std::nothrow) HubTiles(), s};
     HubTiles* t = guard.t;
     if (!t) MIXGCN_FAIL(MIXGCN_ENOMEM, "hub tiles: host allocation failed");
+    auto take = [&](void** p, int64_t bytes) -> mixgcn_status {
+        if (g->ctx->debug_fail_alloc > 0 && --g->ctx->debug_fail_alloc == 0) MIXGCN_FAIL(MIXGCN_ENOMEM, "hub tiles: allocation made to fail (MIXGCN_OPT_DEBUG_FAIL_ALLOC)");
+        return dev_alloc(p, bytes > 0 ? bytes : 1, s);
+    };
     DevBuf rank(s), cnt(s), flag(s), first(s), tmp(s), totals(s), map(s), rem_len(s), tmp2(s);
-    MIXGCN_TRY(rank.alloc(n * (int64_t)sizeof(int32_t)));
-    MIXGCN_TRY(cnt.alloc(total * (int64_t)sizeof(int32_t)));
-    MIXGCN_TRY(flag.alloc((total + 1) * (int64_t)sizeof(int32_t)));
-    MIXGCN_TRY(first.alloc((total + 1) * (int64_t)sizeof(int32_t)));
-    MIXGCN_TRY(totals.alloc(sizeof(HubTotals)));
+    MIXGCN_TRY(take(&rank.p, n * (int64_t)sizeof(int32_t)));
+    MIXGCN_TRY(take(&cnt.p, total * (int64_t)sizeof(int32_t)));
+    MIXGCN_TRY(take(&flag.p, (total + 1) * (int64_t)sizeof(int32_t)));
+    MIXGCN_TRY(take(&first.p, (total + 1) * (int64_t)sizeof(int32_t)));
+    MIXGCN_TRY(take(&totals.p, sizeof(HubTotals)));
     MIXGCN_CUDA(cudaMemsetAsync(cnt.p, 0, total * sizeof(int32_t), s));
     MIXGCN_CUDA(cudaMemsetAsync(totals.p, 0, sizeof(HubTotals), s));
     rank_kernel<<<blocks_for(n), TPB, 0, s>>>(n, hubs, 0x7FFFFFFF, At.full.perm, rank.as<int32_t>());
@@ -597,7 +602,7 @@ mixgcn_status build_tiles(const mixgcn_graph* g, bool transposed, HubTiles** out
     tile_select_kernel<<<blocks_for(total + 1), TPB, 0, s>>>(total, cbs, HUB_TILE_MIN, cnt.as<int32_t>(), flag.as<int32_t>(), totals.as<HubTotals>());
     size_t tb = 0;
     MIXGCN_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tb, flag.as<int32_t>(), first.as<int32_t>(), total + 1, s));
-    MIXGCN_TRY(tmp.alloc((int64_t)tb));
+    MIXGCN_TRY(take(&tmp.p, (int64_t)tb));
     MIXGCN_CUDA(cub::DeviceScan::ExclusiveSum(tmp.p, tb, flag.as<int32_t>(), first.as<int32_t>(), total + 1, s));
     HubTotals h{};
     std::vector<int32_t> host_first(total + 1);
@@ -639,17 +644,17 @@ mixgcn_status build_tiles(const mixgcn_graph* g, bool transposed, HubTiles** out
     first_piece[clusters] = (int32_t)pieces.size();
     for (int i = 0; i < t->row_blocks; ++i) piece_first[i + 1] += piece_first[i];
     t->n_pieces = (int)pieces.size();
-    MIXGCN_TRY(map.alloc(total * (int64_t)sizeof(int32_t)));
-    MIXGCN_TRY(rem_len.alloc((n + 1) * (int64_t)sizeof(int64_t)));
-    MIXGCN_TRY(dev_alloc((void**)&t->rank, n * (int64_t)sizeof(int32_t), s));
-    MIXGCN_TRY(dev_alloc((void**)&t->pieces, t->n_pieces * (int64_t)sizeof(HubPiece), s));
-    MIXGCN_TRY(dev_alloc((void**)&t->first_piece, (clusters + 1) * (int64_t)sizeof(int32_t), s));
-    MIXGCN_TRY(dev_alloc((void**)&t->piece_first, (t->row_blocks + 1) * (int64_t)sizeof(int32_t), s));
-    MIXGCN_TRY(dev_alloc((void**)&t->tile_cb, t->n_tiles * (int64_t)sizeof(int32_t), s));
-    MIXGCN_TRY(dev_alloc((void**)&t->bits, t->n_tiles * (int64_t)ROWS * 16, s));
-    MIXGCN_TRY(dev_alloc((void**)&t->row_scale, rows * (int64_t)sizeof(float), s));
-    MIXGCN_TRY(dev_alloc((void**)&t->col_scale, t->n_cols * (int64_t)sizeof(float), s));
-    MIXGCN_TRY(dev_alloc((void**)&t->rem.rowptr, (n + 1) * (int64_t)sizeof(int64_t), s));
+    MIXGCN_TRY(take(&map.p, total * (int64_t)sizeof(int32_t)));
+    MIXGCN_TRY(take(&rem_len.p, (n + 1) * (int64_t)sizeof(int64_t)));
+    MIXGCN_TRY(take((void**)&t->rank, n * (int64_t)sizeof(int32_t)));
+    MIXGCN_TRY(take((void**)&t->pieces, t->n_pieces * (int64_t)sizeof(HubPiece)));
+    MIXGCN_TRY(take((void**)&t->first_piece, (clusters + 1) * (int64_t)sizeof(int32_t)));
+    MIXGCN_TRY(take((void**)&t->piece_first, (t->row_blocks + 1) * (int64_t)sizeof(int32_t)));
+    MIXGCN_TRY(take((void**)&t->tile_cb, t->n_tiles * (int64_t)sizeof(int32_t)));
+    MIXGCN_TRY(take((void**)&t->bits, t->n_tiles * (int64_t)ROWS * 16));
+    MIXGCN_TRY(take((void**)&t->row_scale, rows * (int64_t)sizeof(float)));
+    MIXGCN_TRY(take((void**)&t->col_scale, t->n_cols * (int64_t)sizeof(float)));
+    MIXGCN_TRY(take((void**)&t->rem.rowptr, (n + 1) * (int64_t)sizeof(int64_t)));
     MIXGCN_CUDA(cudaMemcpyAsync(t->pieces, pieces.data(), pieces.size() * sizeof(HubPiece), cudaMemcpyHostToDevice, s));
     MIXGCN_CUDA(cudaMemcpyAsync(t->first_piece, first_piece.data(), first_piece.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
     MIXGCN_CUDA(cudaMemcpyAsync(t->piece_first, piece_first.data(), piece_first.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
@@ -661,11 +666,11 @@ mixgcn_status build_tiles(const mixgcn_graph* g, bool transposed, HubTiles** out
     tile_bits_kernel<<<(unsigned)covered, TPB, 0, s>>>(n, cbs, A.full.perm, A.rowptr, A.col, rank.as<int32_t>(), map.as<int32_t>(), reinterpret_cast<uint4*>(t->bits), rem_len.as<int64_t>());
     tb = 0;
     MIXGCN_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tb, rem_len.as<int64_t>(), t->rem.rowptr, n + 1, s));
-    MIXGCN_TRY(tmp2.alloc((int64_t)tb));
+    MIXGCN_TRY(take(&tmp2.p, (int64_t)tb));
     MIXGCN_CUDA(cub::DeviceScan::ExclusiveSum(tmp2.p, tb, rem_len.as<int64_t>(), t->rem.rowptr, n + 1, s));
     const int64_t room = t->rem_nnz > 0 ? t->rem_nnz : 1;
-    MIXGCN_TRY(dev_alloc((void**)&t->rem.col, room * (int64_t)sizeof(int32_t), s));
-    MIXGCN_TRY(dev_alloc((void**)&t->rem.val, room * (int64_t)sizeof(float), s));
+    MIXGCN_TRY(take((void**)&t->rem.col, room * (int64_t)sizeof(int32_t)));
+    MIXGCN_TRY(take((void**)&t->rem.val, room * (int64_t)sizeof(float)));
     remainder_kernel<<<(unsigned)rows, TPB, 0, s>>>(cbs, A.full.perm, A.rowptr, A.col, A.val, rank.as<int32_t>(), map.as<int32_t>(), t->rem.rowptr, t->rem.col, t->rem.val);
     if (rows < n) other_rows_kernel<<<blocks_for((n - rows) * 32), TPB, 0, s>>>(rows, n, A.full.perm, A.rowptr, A.col, A.val, t->rem.rowptr, t->rem.col, t->rem.val);
     MIXGCN_CUDA(cudaGetLastError());

@@ -267,3 +267,32 @@ def test_error_on_graphs_with_hubs(mg, ctx, n, edges, flag):
     assert mg.graph_prepare_tiles(tiled)[0] > 500
     compare_errors(mg, ctx, plain, tiled, matrix(mg, tiled, False), 132)
     plain.close(), tiled.close()
+
+
+def test_a_layout_that_runs_out_of_memory_leaves_the_graph_as_it_was(mg, ctx, graphs):
+    """Each allocation of the layout made to fail in turn (what has been enqueued until then is still writing to the blocks it got), a
+    fresh graph every time, both orientations."""
+    plain, _, _ = graphs["sym", False]
+    src, dst = edges(1)
+    Y, Z, Zp = features(100, 3), torch.empty((N, 100), device="cuda"), torch.empty((N, 100), device="cuda")
+    mg.spmm(ctx, plain, Y, Zp, 100)
+    failed = 0
+    for k in range(1, 100):
+        g = mg.graph_create(ctx, N, src, dst, mg.GRAPH_ADD_SELF_LOOPS)
+        mg.ctx_set_option(ctx, mg.OPT_DEBUG_FAIL_ALLOC, k)
+        try:
+            tiles = mg.graph_prepare_tiles(g)[0]
+        except mg.MixgcnError:
+            tiles = 0
+        finally:
+            mg.ctx_set_option(ctx, mg.OPT_DEBUG_FAIL_ALLOC, 0)
+        other = mg.graph_create(ctx, N, src, dst, mg.GRAPH_ADD_SELF_LOOPS)        # takes the memory that came back
+        mg.spmm(ctx, other, Y, Z, 100)
+        assert torch.equal(Z, Zp)
+        mg.spmm(ctx, g, Y, Z, 100)
+        assert torch.equal(Z, Zp) == (tiles == 0)
+        g.close(), other.close()
+        if tiles:
+            break
+        failed += 1
+    assert 20 < failed < 90

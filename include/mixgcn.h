@@ -105,8 +105,9 @@ mixgcn_status mixgcn_debug_poke_col(mixgcn_graph* g, int64_t entry, int32_t valu
  * rows may be converted on the way in (with 1 they go through a bf16 copy).  Nothing traps, spins without limit or faults. */
 #define MIXGCN_OPT_DEBUG_WAIT_LIMIT 3
 #define MIXGCN_OPT_DEBUG_DROP_LOAD 4
-/* Test hook of allocation failures, 0 by default: k > 0 = of the device allocations that the layout of tiles (see
- * mixgcn_graph_prepare_tiles) asks for from now on, for graphs of this context, the k-th fails as if there were no memory. */
+/* Test hook of allocation failures, 0 by default: k > 0 = of the device allocations that layouts of tiles (see
+ * mixgcn_graph_prepare_tiles) for graphs of this context and the context's workspaces ask for from now on, the k-th fails
+ * as if there were no memory. */
 #define MIXGCN_OPT_DEBUG_FAIL_ALLOC 6
 /* MIXGCN_OPT_GEMM_CTA_PAIRS: 1 (default) = wide and deep K-major products (N >= 512, K >= 512, M >= 4096)
  * run on pairs of CTAs that share one 256 x 256 tile (tcgen05 .cta_group::2); 0 = every product on single
@@ -202,7 +203,8 @@ mixgcn_status mixgcn_graph_export_schedule(const mixgcn_graph* g, int transposed
  * tile of 128 x 128 that holds enough entries becomes a bitmap, and later aggregations over all rows (mixgcn_spmm and the
  * layer calls; not sampled, row-sparse, row-filtered or chunked ones) multiply it there, sums in fp32 as before but in
  * another order.  Costs a few passes over the entries; for a graph that many aggregations will use.  Nothing happens on
- * graphs without such tiles, or the second time.  n_tiles, n_entries (nullable): tiles, and entries in them, of the
+ * graphs without such tiles, or the second time; without memory for the layout (or, in an aggregation, for its scratch)
+ * the gather kernels do all the work, as they do without this call.  n_tiles, n_entries (nullable): tiles, and entries in them, of the
  * forward orientation.  Synchronises before returning; aggregations already enqueued are not affected. */
 mixgcn_status mixgcn_graph_prepare_tiles(mixgcn_graph* g, int64_t* n_tiles, int64_t* n_entries);
 

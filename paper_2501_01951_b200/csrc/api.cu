@@ -129,7 +129,8 @@ mixgcn_status grow_block(mixgcn_ctx* ctx, void** block, int64_t* have, int64_t b
     *block = nullptr; *have = 0;
     ctx->blocks_generation++;
     void* p = nullptr;
-    const mixgcn_status st = dev_alloc(&p, want, s);
+    const bool fails = ctx->debug_fail_alloc > 0 && --ctx->debug_fail_alloc == 0;
+    const mixgcn_status st = fails ? MIXGCN_ENOMEM : dev_alloc(&p, want, s);
     if (st == MIXGCN_ENOMEM) MIXGCN_FAIL(MIXGCN_ENOMEM, "%s of %lld bytes could not be allocated", what, (long long)want);
     MIXGCN_TRY(st);
     MIXGCN_CUDA(cudaStreamSynchronize(s));       // usable on every stream from here on

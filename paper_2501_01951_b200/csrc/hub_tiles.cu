@@ -779,11 +779,18 @@ extern "C" mixgcn_status mixgcn_graph_prepare_tiles(mixgcn_graph* g, int64_t* n_
         cudaStream_t s = g->ctx->side_stream[0];
         LaunchScope scope(g->ctx, PH_GRAPH, s, 12);
         HubTiles* made[2] = {nullptr, nullptr};
-        MIXGCN_TRY(build_tiles(g, false, &made[0], s));
-        if (g->bwd_is_fwd) made[1] = made[0];
-        else if (g->norm != 1) {       // (row means transposed: see the errors above)
-            const mixgcn_status st = build_tiles(g, true, &made[1], s);
-            if (st != MIXGCN_OK) { free_tiles(made[0]); return st; }
+        mixgcn_status st;
+        try {
+            st = build_tiles(g, false, &made[0], s);
+            if (g->bwd_is_fwd) made[1] = made[0];
+            else if (st == MIXGCN_OK && g->norm != 1) st = build_tiles(g, true, &made[1], s);       // (row means transposed: see the errors above)
+        } catch (const std::bad_alloc&) {
+            st = MIXGCN_ENOMEM;
+        }
+        if (st != MIXGCN_OK) {         // (the gather kernels need none of it: where there is no memory for tiles there are none)
+            free_tiles(made[0]);
+            made[0] = made[1] = nullptr;
+            if (st != MIXGCN_ENOMEM) return st;
         }
         g->tiles[0].store(made[0], std::memory_order_release);
         g->tiles[1].store(made[1], std::memory_order_release);

@@ -105,7 +105,7 @@ struct mixgcn_ctx {
     int64_t gemm_pair_launches;   // of those, products that ran on CTA pairs (tcgen05 .cta_group::2)
     int no_cta_pairs;         // 1: keep every product on single CTAs (option, for comparison)
     int debug_wait_limit;     // > 0: polls after which the tensor-core kernels' waits give up (test of that path)
-    int debug_fail_alloc;     // > 0: this many allocations from now, one for hub tiles fails (test of that path)
+    int debug_fail_alloc;     // > 0: this many allocations from now, one for hub tiles or a workspace fails (test of that path)
     int debug_drop_load;      // 1, 2: tensor-core products leave one stage unfilled (test of that path)
     int spmm_slice_cols;      // 0 = default (one slice up to 1024 columns)
     int loss_train_rows_only; // 1 = the loss skips rows outside the train mask entirely

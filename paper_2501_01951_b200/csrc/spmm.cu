@@ -259,6 +259,11 @@ void dispatch_filtered(const SpmmParams& p, cudaStream_t s) {
 constexpr int MAX_SLICE = 1024;      // columns per launch at most: 8 float4 per lane
 constexpr int DEFAULT_SLICE = 256;   // widths above this run as slices of this many columns (2 float4 per lane, four CTAs per SM)
 
+// bytes of scratch of one slice of w columns where tiles run: partial rows of the other entries' segments, then what the tiles need
+int64_t tiles_scratch(const HubTiles* t, int32_t w, int64_t ldp, int64_t* images_at) {
+    return t->rem.full.total_segs * ldp * (int64_t)sizeof(float) + 1024 + hub_tiles_scratch(t, w, ldp, images_at);
+}
+
 }  // namespace
 
 namespace mixgcn {
@@ -294,6 +299,14 @@ mixgcn_status launch_spmm(mixgcn_ctx* ctx, const mixgcn_graph* g, const CsrView&
         tiles = g->tiles[&A == &g->bwd].load(std::memory_order_acquire);
         if (tiles && !hub_tiles_pay(tiles, w)) tiles = nullptr;
     }
+    const int slice = lf ? MAX_SLICE : ctx->spmm_slice_cols > 0 ? (ctx->spmm_slice_cols < MAX_SLICE ? ctx->spmm_slice_cols : MAX_SLICE) : DEFAULT_SLICE;
+    if (tiles) {        // scratch of the widest slice; the gather kernels alone where there is no memory for it
+        int64_t images_at = 0;
+        const int64_t ldp = ((int64_t)(w < slice ? w : slice) + 3) / 4 * 4;
+        const mixgcn_status st = ensure_workspace_spmm(ctx, tiles_scratch(tiles, w < slice ? w : slice, ldp, &images_at));
+        if (st == MIXGCN_ENOMEM) tiles = nullptr;
+        else MIXGCN_TRY(st);
+    }
     const CsrView& V = tiles ? tiles->rem : A;       // with tiles: what they leave
     const SpmmSchedule& S = chunks > 1 ? A.chunk[k] : V.full;
     if (S.n_rows <= 0) return MIXGCN_OK;
@@ -323,7 +336,6 @@ mixgcn_status launch_spmm(mixgcn_ctx* ctx, const mixgcn_graph* g, const CsrView&
         p.loss_labels = lf->labels; p.loss_mask = lf->train_mask; p.loss_count = lf->count;
         p.loss_row = lf->row_loss; p.loss_pred = lf->pred; p.loss_zero_rows = lf->zero_rows;
     }
-    const int slice = lf ? MAX_SLICE : ctx->spmm_slice_cols > 0 ? (ctx->spmm_slice_cols < MAX_SLICE ? ctx->spmm_slice_cols : MAX_SLICE) : DEFAULT_SLICE;
     const NarrowCfg narrow = narrow_cfg(w);
     for (int j0 = 0; j0 < w; j0 += slice) {
         p.j0 = j0;
@@ -396,7 +408,7 @@ mixgcn_status launch_spmm(mixgcn_ctx* ctx, const mixgcn_graph* g, const CsrView&
         // the segments' partial rows, then what the tiles need
         const int64_t ldp = ((int64_t)p.w + 3) / 4 * 4, seg_bytes = S.total_segs * ldp * (int64_t)sizeof(float);
         int64_t images_at = 0;
-        const int64_t scratch = tiles ? seg_bytes + 1024 + hub_tiles_scratch(tiles, p.w, ldp, &images_at) : seg_bytes;
+        const int64_t scratch = tiles ? tiles_scratch(tiles, p.w, ldp, &images_at) : seg_bytes;
         if (scratch > 0) MIXGCN_TRY(ensure_workspace_spmm(ctx, scratch));
         float* partial = reinterpret_cast<float*>(ctx->workspace_spmm);
         p.ldp = ldp;

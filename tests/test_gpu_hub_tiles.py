@@ -280,12 +280,8 @@ def test_a_layout_that_runs_out_of_memory_leaves_the_graph_as_it_was(mg, ctx, gr
     for k in range(1, 100):
         g = mg.graph_create(ctx, N, src, dst, mg.GRAPH_ADD_SELF_LOOPS)
         mg.ctx_set_option(ctx, mg.OPT_DEBUG_FAIL_ALLOC, k)
-        try:
-            tiles = mg.graph_prepare_tiles(g)[0]
-        except mg.MixgcnError:
-            tiles = 0
-        finally:
-            mg.ctx_set_option(ctx, mg.OPT_DEBUG_FAIL_ALLOC, 0)
+        tiles = mg.graph_prepare_tiles(g)[0]
+        mg.ctx_set_option(ctx, mg.OPT_DEBUG_FAIL_ALLOC, 0)
         other = mg.graph_create(ctx, N, src, dst, mg.GRAPH_ADD_SELF_LOOPS)        # takes the memory that came back
         mg.spmm(ctx, other, Y, Z, 100)
         assert torch.equal(Z, Zp)
@@ -296,3 +292,35 @@ def test_a_layout_that_runs_out_of_memory_leaves_the_graph_as_it_was(mg, ctx, gr
             break
         failed += 1
     assert 20 < failed < 90
+
+
+@pytest.mark.parametrize("kind", ["gcn", "sage", "gin"])
+def test_trainers_do_without_tiles_where_there_is_no_memory_for_them(mg, ctx, kind):
+    from paper_2501_01951_b200.sage_gin import GinTrainer, SageTrainer
+    from paper_2501_01951_b200.train import GcnTrainer
+    make = dict(gcn=GcnTrainer, sage=SageTrainer, gin=GinTrainer)[kind]
+    src, dst = edges(1)
+    flags = mg.GRAPH_SYMMETRISE | dict(gcn=mg.GRAPH_ADD_SELF_LOOPS, sage=mg.GRAPH_NORM_ROW, gin=mg.GRAPH_NORM_NONE)[kind]
+    for k in (1, 9, 20):
+        g = mg.graph_create(ctx, N, src, dst, flags)
+        mg.ctx_set_option(ctx, mg.OPT_DEBUG_FAIL_ALLOC, k)
+        make(ctx, g, (64, 128, 16), *([128] if kind == "gin" else []), mg.PREC_TF32)
+        mg.ctx_set_option(ctx, mg.OPT_DEBUG_FAIL_ALLOC, 0)
+        assert mg.graph_prepare_tiles(g) == (0, 0)
+        g.close()
+
+
+@pytest.mark.parametrize("w", [100, 300])
+def test_an_aggregation_without_memory_for_its_tiles_gathers(mg, graphs, w):
+    plain, tiled, _ = graphs["sym", False]
+    ctx = mg.ctx_create(0)
+    Y = features(w, 3)
+    Z, Zp, Zt = (torch.empty_like(Y) for _ in range(3))
+    mg.ctx_set_option(ctx, mg.OPT_DEBUG_FAIL_ALLOC, 1)
+    mg.spmm(ctx, tiled, Y, Z, w)
+    mg.spmm(ctx, plain, Y, Zp, w)
+    assert torch.equal(Z, Zp)
+    mg.spmm(ctx, tiled, Y, Zt, w)
+    assert not torch.equal(Zt, Zp) and (Zt - Zp).abs().max() <= 2e-6 * Zp.abs().max()
+    assert mg.ctx_poll_status(ctx, raise_on_error=False) == 0
+    ctx.close()

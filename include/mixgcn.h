@@ -200,12 +200,15 @@ mixgcn_status mixgcn_graph_export(const mixgcn_graph* g, int transposed, int64_t
 mixgcn_status mixgcn_graph_export_schedule(const mixgcn_graph* g, int transposed, int32_t* perm);
 
 /* Lays the dense corner of the matrix out for the tensor cores: with rows and columns by descending entry counts, every
- * tile of 128 x 128 that holds enough entries becomes a bitmap, and later aggregations over all rows (mixgcn_spmm and the
- * layer calls; not sampled, row-sparse, row-filtered or chunked ones) multiply it there, sums in fp32 as before but in
- * another order.  Costs a few passes over the entries; for a graph that many aggregations will use.  Nothing happens on
+ * tile of 256 x 128 that holds enough entries becomes a bitmap, and aggregations over all rows (not sampled, row-sparse,
+ * row-filtered or chunked ones) that ask for it multiply it there, sums in fp32 as before but in another order.  Which calls
+ * do is the calls' affair: layers with MIXGCN_LAYER_TILES, mixgcn_spmm_tiles, and, once mixgcn_graph_prepare_tiles has been
+ * called, mixgcn_spmm.  Costs a few passes over the entries; for a graph that many aggregations will use.  Nothing happens on
  * graphs without such tiles, or the second time; without memory for the layout (or, in an aggregation, for its scratch)
- * the gather kernels do all the work, as they do without this call.  n_tiles, n_entries (nullable): tiles, and entries in them, of the
- * forward orientation.  Synchronises before returning; aggregations already enqueued are not affected. */
+ * the gather kernels do all the work, as they do without this call.  n_tiles, n_entries (nullable): tiles, and entries in
+ * them, of the forward orientation.  Synchronises before returning; aggregations already enqueued are not affected, and
+ * recordings that use the graph end when mixgcn_graph_prepare_tiles changes the order of their sums. */
+mixgcn_status mixgcn_graph_layout_tiles(mixgcn_graph* g, int64_t* n_tiles, int64_t* n_entries);
 mixgcn_status mixgcn_graph_prepare_tiles(mixgcn_graph* g, int64_t* n_tiles, int64_t* n_entries);
 
 /* A graph may be used only while its context exists; it may be destroyed after it. */
@@ -280,6 +283,12 @@ typedef struct {
 mixgcn_status mixgcn_spmm(mixgcn_ctx* ctx, const mixgcn_graph* g, int transposed, int32_t w,
                           const float* Y, int64_t ldy, float* Z, int64_t ldz,
                           const mixgcn_epilogue* epi, void* stream);
+
+/* The same, and whether it takes the tiles of mixgcn_graph_layout_tiles (tiles != 0: where the graph has them and they pay) or
+ * the gather kernels alone is said here. */
+mixgcn_status mixgcn_spmm_tiles(mixgcn_ctx* ctx, const mixgcn_graph* g, int transposed, int32_t w,
+                                const float* Y, int64_t ldy, float* Z, int64_t ldz,
+                                const mixgcn_epilogue* epi, int32_t tiles, void* stream);
 
 /* Sampled aggregation (the paper's S-SpMM, Eq. 4): Z = (A_hat Y) (.) M for a binary output mask M held as
  * a BITMAP (the output mask buffer of Section 3.2.1): bit (j % 32) of word mask_bits[u * ld_bits + j / 32]
@@ -364,6 +373,8 @@ mixgcn_status mixgcn_weight_grad(mixgcn_ctx* ctx, int32_t precision, int64_t M, 
                                        row-sparse backward (gout_row_mask / gout_plan), OUT_ROWS_ONLY or
                                        SAVED_IS_VALID; MIXGCN_EUNSUPPORTED if the BF16 kernels cannot take the
                                        shape (there is then no fp32 operand to fall back on). */
+#define MIXGCN_LAYER_TILES 256u        /* the layer's aggregations take the graph's tiles, where it has them (see
+                                       mixgcn_graph_layout_tiles): sums in another order than without */
 #define MIXGCN_LAYER_GIN_ROWS_ONLY 32u /* backward with gout_plan: write only the rows of G_in in the
                                        plan's out_row_mask (the other rows are exactly zero and
                                        are left unchanged) */

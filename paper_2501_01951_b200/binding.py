@@ -36,6 +36,7 @@ ORDER_AUTO, ORDER_AGG_FIRST, ORDER_UPD_FIRST = 0, 1, 2
 LAYER_RELU, LAYER_FIRST, LAYER_GATE_GIN, LAYER_GOUT_GATED, LAYER_OUT_ROWS_ONLY, LAYER_GIN_ROWS_ONLY = 1, 2, 4, 8, 16, 32
 LAYER_SAVED_IS_VALID = 64
 LAYER_SAVED_LP_ONLY = 128
+LAYER_TILES = 256
 N_PHASES = 7
 PHASES = ("spmm", "gemm", "elementwise", "loss", "adam", "graph", "spmm_sparse")
 PRECISIONS = {"fp32": PREC_FP32, "tf32": PREC_TF32, "bf16": PREC_BF16}
@@ -45,7 +46,7 @@ SYMBOLS = (
     "mixgcn_status_string", "mixgcn_last_error", "mixgcn_ctx_create", "mixgcn_ctx_destroy",
     "mixgcn_ctx_reserve", "mixgcn_ctx_poll_status", "mixgcn_ctx_profile_enable", "mixgcn_ctx_profile_read",
     "mixgcn_graph_create", "mixgcn_graph_create_from_csr", "mixgcn_graph_info", "mixgcn_graph_export",
-    "mixgcn_graph_prepare_tiles", "mixgcn_graph_export_schedule", "mixgcn_graph_destroy", "mixgcn_spmm", "mixgcn_gemm",
+    "mixgcn_graph_layout_tiles", "mixgcn_graph_prepare_tiles", "mixgcn_spmm_tiles", "mixgcn_graph_export_schedule", "mixgcn_graph_destroy", "mixgcn_spmm", "mixgcn_gemm",
     "mixgcn_layer_plan", "mixgcn_layer_fwd", "mixgcn_layer_bwd", "mixgcn_loss_softmax_xent",
     "mixgcn_adam_step", "mixgcn_train_step_host", "mixgcn_loss_softmax_xent_noalloc", "mixgcn_ctx_set_option",
     "mixgcn_graph_bandwidth", "mixgcn_graph_rcm", "mixgcn_pipeline_stages", "mixgcn_graph_create_permuted",
@@ -344,9 +345,16 @@ def graph_export_schedule(g: Graph, transposed: bool = False) -> torch.Tensor:
     return perm
 
 
+def graph_layout_tiles(g: Graph) -> tuple[int, int]:
+    """Lay the dense corner of the graph out for the tensor cores -> (tiles, entries in them), for the calls that ask for it
+    (LAYER_TILES, spmm(tiles=True)).  Once per graph; later calls change nothing."""
+    tiles, entries = C.c_int64(0), C.c_int64(0)
+    _check(lib.mixgcn_graph_layout_tiles(g.h, C.byref(tiles), C.byref(entries)))
+    return tiles.value, entries.value
+
+
 def graph_prepare_tiles(g: Graph) -> tuple[int, int]:
-    """Lay the dense corner of the graph out for the tensor cores -> (tiles, entries in them).  Once per graph; later calls
-    change nothing."""
+    """The same, and spmm() on this graph takes the tiles from now on unless it is told otherwise."""
     tiles, entries = C.c_int64(0), C.c_int64(0)
     _check(lib.mixgcn_graph_prepare_tiles(g.h, C.byref(tiles), C.byref(entries)))
     return tiles.value, entries.value
@@ -423,11 +431,17 @@ def make_epilogue(bias=None, relu=False, drop_mask=None, keep_scale=1.0, gate=No
     return e
 
 
-def spmm(ctx: Ctx, g: Graph, Y: torch.Tensor, Z: torch.Tensor, w: int, transposed: bool = False, epi: Epilogue | None = None):
+def spmm(ctx: Ctx, g: Graph, Y: torch.Tensor, Z: torch.Tensor, w: int, transposed: bool = False, epi: Epilogue | None = None,
+         tiles: bool | None = None):
+    """Z = A_hat Y.  tiles: whether the graph's tiles, if it has any, are taken (None: if graph_prepare_tiles was called)."""
     Y, ldy = _mat(Y, "Y")
     Z, ldz = _mat(Z, "Z")
-    _check(lib.mixgcn_spmm(ctx.h, g.h, C.c_int(int(transposed)), C.c_int32(w), _ptr(Y), C.c_int64(ldy),
-                           _ptr(Z), C.c_int64(ldz), None if epi is None else C.byref(epi), _stream()))
+    args = (ctx.h, g.h, C.c_int(int(transposed)), C.c_int32(w), _ptr(Y), C.c_int64(ldy), _ptr(Z), C.c_int64(ldz),
+            None if epi is None else C.byref(epi))
+    if tiles is None:
+        _check(lib.mixgcn_spmm(*args, _stream()))
+    else:
+        _check(lib.mixgcn_spmm_tiles(*args, C.c_int32(int(tiles)), _stream()))
 
 
 def gemm(ctx: Ctx, precision: int, trans_a: bool, trans_b: bool, M: int, N: int, K: int,

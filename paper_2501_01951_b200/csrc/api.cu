@@ -582,6 +582,8 @@ int resolve_order(const mixgcn_layer_desc* d) {
     return cost_agg <= cost_upd ? MIXGCN_ORDER_AGG_FIRST : MIXGCN_ORDER_UPD_FIRST;
 }
 
+bool layer_tiles(const mixgcn_layer_desc* d) { return (d->flags & MIXGCN_LAYER_TILES) != 0; }
+
 mixgcn_status check_desc(const mixgcn_layer_desc* d, const char* who) {
     if (!d) MIXGCN_FAIL(MIXGCN_EINVAL, "%s: null layer descriptor", who);
     if (d->d_in <= 0 || d->d_out <= 0) MIXGCN_FAIL(MIXGCN_EINVAL, "%s: widths must be positive", who);
@@ -702,7 +704,7 @@ extern "C" mixgcn_status mixgcn_layer_fwd(mixgcn_ctx* ctx, const mixgcn_graph* g
     const LayerLP lp(d);
     if (epi.relu && d->x_out_bits) { epi.sign_bits = d->x_out_bits; epi.ld_sign_bits = d->ld_out_bits; }   // the ReLU mask, one bit per element
     if (order == MIXGCN_ORDER_AGG_FIRST) {
-        SpmmOpts agg_opts; agg_opts.Z_lp = lp.saved; agg_opts.ldz_lp = lp.ld_saved;     // the aggregation also writes bf16(A_hat X)
+        SpmmOpts agg_opts; agg_opts.tiles = layer_tiles(d); agg_opts.Z_lp = lp.saved; agg_opts.ldz_lp = lp.ld_saved;     // the aggregation also writes bf16(A_hat X)
         if (chunks == 1) {
             const bool lp_only = (d->flags & MIXGCN_LAYER_SAVED_LP_ONLY) != 0;
             if (!saved_valid)
@@ -746,7 +748,7 @@ extern "C" mixgcn_status mixgcn_layer_fwd(mixgcn_ctx* ctx, const mixgcn_graph* g
         MIXGCN_TRY(launch_gemm(ctx, d->precision, 0, 0, n, d->d_out, d->d_in, X_in, d->ld_in, W, ldw, saved, d->ld_saved,
                                nullptr, 0, s, &glp));
     }
-    SpmmOpts out_opts; out_opts.Z_lp = lp.x_out; out_opts.ldz_lp = lp.ld_out;
+    SpmmOpts out_opts; out_opts.tiles = layer_tiles(d); out_opts.Z_lp = lp.x_out; out_opts.ldz_lp = lp.ld_out;
     MIXGCN_TRY(launch_spmm(ctx, g, g->fwd, 1, 0, d->d_out, saved, d->ld_saved, X_out, d->ld_out, &epi, s, out_opts));
     return MIXGCN_OK;
 }
@@ -780,7 +782,7 @@ extern "C" mixgcn_status mixgcn_layer_fwd_loss(mixgcn_ctx* ctx, const mixgcn_gra
                                nullptr, 0, s, &glp));
         LossFuse lf;
         MIXGCN_TRY(loss_fuse_begin(ctx, n, labels, train_mask, pred, n_correct, s, &lf));
-        SpmmOpts opts; opts.loss = &lf;
+        SpmmOpts opts; opts.loss = &lf; opts.tiles = layer_tiles(d);
         MIXGCN_TRY(launch_spmm(ctx, g, g->fwd, 1, 0, d->d_out, saved, d->ld_saved, dlogits, d->ld_out, &epi, s, opts));
         return loss_fuse_end(ctx, n, d->d_out, lf, loss, n_correct, s);
     }
@@ -788,7 +790,7 @@ extern "C" mixgcn_status mixgcn_layer_fwd_loss(mixgcn_ctx* ctx, const mixgcn_gra
         // logits = (A_hat X_in) W + b: the tensor-core product's epilogue finds every row's arg-max and writes the
         // logits of the train rows only; the loss then runs over those rows in place
         const LayerLP lp(d);
-        SpmmOpts agg_opts; agg_opts.Z_lp = lp.saved; agg_opts.ldz_lp = lp.ld_saved;
+        SpmmOpts agg_opts; agg_opts.tiles = layer_tiles(d); agg_opts.Z_lp = lp.saved; agg_opts.ldz_lp = lp.ld_saved;
         MIXGCN_TRY(launch_spmm(ctx, g, g->fwd, 1, 0, d->d_in, X_in, d->ld_in, saved, d->ld_saved, nullptr, s, agg_opts));
         LossFuse lf;
         lf.train_mask = train_mask; lf.pred = pred; lf.zero_rows = ctx->loss_train_rows_only == 2 ? 0 : 1;
@@ -887,7 +889,7 @@ extern "C" mixgcn_status mixgcn_layer_bwd(mixgcn_ctx* ctx, const mixgcn_graph* g
     }
     const uint8_t* rmask = d->gout_row_mask;
     SpmmRowSparse sp{rmask, nullptr, d->gin_row_mask};
-    SpmmOpts sparse_opts; sparse_opts.sparse = rmask ? &sp : nullptr;
+    SpmmOpts sparse_opts; sparse_opts.tiles = layer_tiles(d); sparse_opts.sparse = rmask ? &sp : nullptr;
     SpmmOpts gin_opts = sparse_opts; gin_opts.Z_lp = lp.g_in; gin_opts.ldz_lp = lp.ld_in;         // aggregations that produce G_in
     SpmmOpts dq_opts = sparse_opts; dq_opts.Z_lp = lp.saved; dq_opts.ldz_lp = lp.ld_saved;        // upd-first: dQ into `saved`
 

@@ -771,8 +771,8 @@ mixgcn_status launch_hub_tiles(mixgcn_ctx* ctx, const HubTiles* t, int phase, in
 
 }  // namespace mixgcn
 
-extern "C" mixgcn_status mixgcn_graph_prepare_tiles(mixgcn_graph* g, int64_t* n_tiles, int64_t* n_entries) {
-    if (!g) MIXGCN_FAIL(MIXGCN_EINVAL, "graph_prepare_tiles: null graph");
+extern "C" mixgcn_status mixgcn_graph_layout_tiles(mixgcn_graph* g, int64_t* n_tiles, int64_t* n_entries) {
+    if (!g) MIXGCN_FAIL(MIXGCN_EINVAL, "graph_layout_tiles: null graph");
     std::lock_guard<std::mutex> lock(g_build_mutex);
     if (!g->tiles_tried) {
         MIXGCN_CUDA(cudaSetDevice(g->device));
@@ -799,5 +799,12 @@ extern "C" mixgcn_status mixgcn_graph_prepare_tiles(mixgcn_graph* g, int64_t* n_
     const HubTiles* t = g->tiles[0].load(std::memory_order_acquire);
     if (n_tiles) *n_tiles = t ? t->n_tiles : 0;
     if (n_entries) *n_entries = t ? t->entries : 0;
+    return MIXGCN_OK;
+}
+
+extern "C" mixgcn_status mixgcn_graph_prepare_tiles(mixgcn_graph* g, int64_t* n_tiles, int64_t* n_entries) {
+    MIXGCN_TRY(mixgcn_graph_layout_tiles(g, n_tiles, n_entries));
+    // (recorded calls of mixgcn_spmm sum in the other order)
+    if (!g->tiles_in_spmm.exchange(true, std::memory_order_acq_rel) && g->tiles[0].load(std::memory_order_acquire)) memory_given_back(g->memory);
     return MIXGCN_OK;
 }

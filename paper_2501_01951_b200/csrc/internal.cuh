@@ -181,6 +181,7 @@ struct mixgcn_graph {
     // tiles of the dense corner of fwd and bwd (the same object where bwd aliases fwd), null where there are none
     std::atomic<struct HubTiles*> tiles[2];
     bool tiles_tried;
+    std::atomic<bool> tiles_in_spmm;   // mixgcn_spmm takes them (mixgcn_graph_prepare_tiles)
 };
 
 // Everything about a row-sparse aggregation that depends only on the graph and on WHICH rows of the
@@ -295,6 +296,7 @@ struct SpmmOpts {
     const LossFuse* loss = nullptr;          // non-null: soft-max cross-entropy epilogue (width <= 256, bias only); Z receives the gradient
     const SpmmRowSparse* sparse = nullptr;   // row-sparse input: test the input's row mask inside the kernel
     const uint8_t* row_filter = nullptr;     // compute only the output rows whose byte is non-zero (not with `sparse`)
+    bool tiles = false;                      // tiles of the dense corner where the graph has them (the order of sums is the call's, not the graph's)
     int phase = PH_SPMM;                     // profiling phase the launches are booked under
     int64_t row_limit = -1;                  // >= 0: only the first row_limit rows of the schedule (longest first)
     uint16_t* Z_lp = nullptr;                // nullable: also write a bf16 copy of Z (after the epilogue), ldz_lp a multiple of 4

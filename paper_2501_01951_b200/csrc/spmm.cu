@@ -293,9 +293,9 @@ mixgcn_status launch_spmm(mixgcn_ctx* ctx, const mixgcn_graph* g, const CsrView&
         if (k < 0 || k >= A.n_chunk) MIXGCN_FAIL(MIXGCN_EINVAL, "spmm: chunk %d of %d does not exist", k, chunks);
     }
     recording_uses(ctx, g->memory);
-    // tiles of the dense corner, where the graph has them and the call is a plain one over a whole orientation
+    // tiles of the dense corner, where the call asks for them, the graph has them and the call is a plain one over a whole orientation
     const HubTiles* tiles = nullptr;
-    if (chunks <= 1 && !sparse && !row_filter && row_limit < 0 && !opts.out_bits && (&A == &g->fwd || &A == &g->bwd)) {
+    if (opts.tiles && chunks <= 1 && !sparse && !row_filter && row_limit < 0 && !opts.out_bits && (&A == &g->fwd || &A == &g->bwd)) {
         tiles = g->tiles[&A == &g->bwd].load(std::memory_order_acquire);
         if (tiles && !hub_tiles_pay(tiles, w)) tiles = nullptr;
     }
@@ -437,6 +437,12 @@ mixgcn_status launch_spmm(mixgcn_ctx* ctx, const mixgcn_graph* g, const CsrView&
 extern "C" mixgcn_status mixgcn_spmm(mixgcn_ctx* ctx, const mixgcn_graph* g, int transposed, int32_t w,
                                      const float* Y, int64_t ldy, float* Z, int64_t ldz,
                                      const mixgcn_epilogue* epi, void* stream) {
+    return mixgcn_spmm_tiles(ctx, g, transposed, w, Y, ldy, Z, ldz, epi, g && g->tiles_in_spmm.load(std::memory_order_acquire), stream);
+}
+
+extern "C" mixgcn_status mixgcn_spmm_tiles(mixgcn_ctx* ctx, const mixgcn_graph* g, int transposed, int32_t w,
+                                           const float* Y, int64_t ldy, float* Z, int64_t ldz,
+                                           const mixgcn_epilogue* epi, int32_t tiles, void* stream) {
     if (!ctx || !g || !Y || !Z) MIXGCN_FAIL(MIXGCN_EINVAL, "spmm: null argument");
     if (w <= 0) MIXGCN_FAIL(MIXGCN_EINVAL, "spmm: w must be positive (got %d)", w);
     if (ldy < w || ldz < w || (ldy & 3) || (ldz & 3))
@@ -449,7 +455,8 @@ extern "C" mixgcn_status mixgcn_spmm(mixgcn_ctx* ctx, const mixgcn_graph* g, int
     if (epi && ((epi->gate_bits && epi->ld_gate_bits < (w + 31) / 32) || (epi->sign_bits && epi->ld_sign_bits < (w + 31) / 32)))
         MIXGCN_FAIL(MIXGCN_EINVAL, "spmm: a bit-packed mask needs ld >= ceil(w / 32) words");
     MIXGCN_CUDA(cudaSetDevice(ctx->device));
-    return launch_spmm(ctx, g, transposed ? g->bwd : g->fwd, 1, 0, w, Y, ldy, Z, ldz, epi, (cudaStream_t)stream);
+    SpmmOpts opts; opts.tiles = tiles != 0;
+    return launch_spmm(ctx, g, transposed ? g->bwd : g->fwd, 1, 0, w, Y, ldy, Z, ldz, epi, (cudaStream_t)stream, opts);
 }
 
 namespace {

@@ -45,8 +45,9 @@ def product_precision(precision: int, relu: bool) -> int:
 class _Base:
     def __init__(self, ctx, graph, dims, precision):
         self.ctx, self.g, self.precision = ctx, graph, precision
-        if precision != mg.PREC_FP32:
-            mg.graph_prepare_tiles(graph)      # as in train.py
+        self.tiles = precision != mg.PREC_FP32      # as in train.py
+        if self.tiles:
+            mg.graph_layout_tiles(graph)
         self.dims = tuple(int(d) for d in dims)
         self.L = len(self.dims) - 1
         self.n = graph.n
@@ -57,6 +58,9 @@ class _Base:
         self.n_correct = torch.zeros(1, dtype=torch.int64, device=self.device)
         self.params, self.grads, self.m, self.v = [], [], [], []
         self._replay = mg.Replayer(ctx)      # the calls of an iteration, recorded once they have come twice with the same buffers
+
+    def _spmm(self, *args, **kwargs):
+        mg.spmm(self.ctx, self.g, *args, tiles=self.tiles, **kwargs)
 
     def _z(self, r, c):
         return torch.zeros((r, c), dtype=torch.float32, device=self.device)
@@ -156,9 +160,9 @@ class SageTrainer(_Base):
                     beside.copy_(stacked)
                 P = self.pool[0].view(-1)[: self.n * self.wide[l]].view(self.n, self.wide[l])
                 mg.gemm(self.ctx, product_precision(self.precision, relu), False, False, self.n, self.wide[l], self.dims[l], S, self.Wc[l], P)
-                mg.spmm(self.ctx, self.g, P[:, do4:], out, dout, epi=mg.make_epilogue(residual=P[:, :do4], residual_scale=1.0, bias=bias, relu=relu))
+                self._spmm(P[:, do4:], out, dout, epi=mg.make_epilogue(residual=P[:, :do4], residual_scale=1.0, bias=bias, relu=relu))
             else:
-                mg.spmm(self.ctx, self.g, S[:, :d], S[:, d:], self.dims[l])
+                self._spmm(S[:, :d], S[:, d:], self.dims[l])
                 mg.gemm(self.ctx, self.precision, False, False, self.n, dout, 2 * d, S, self.params[l], out,
                         epi=mg.make_epilogue(bias=bias, relu=relu, sign_bits=None if last else self.signs[l + 1]))
 
@@ -172,7 +176,7 @@ class SageTrainer(_Base):
                 Gn = self.G[l - 1][:, :d]
                 gate = dict(gate_bits=self.signs[l]) if self.signs[l] is not None else dict(gate=self.S[l][:, :d])
             if self.upd[l]:
-                mg.spmm(self.ctx, self.g, G, Gc[:, do4:], dout, transposed=True)
+                self._spmm(G, Gc[:, do4:], dout, transposed=True)
                 mg.weight_grad(self.ctx, self.precision, self.dims[l], self.wide[l], self.n, self.S[l], Gc, self.dWc[l], self.dbc[l])
                 for stacked, beside in self._halves(l, self.grads[l], self.dWc[l]):
                     stacked.copy_(beside)
@@ -185,7 +189,7 @@ class SageTrainer(_Base):
                 dS = self.dS.view(-1)[: self.n * 2 * d].view(self.n, 2 * d)
                 mg.gemm(self.ctx, self.precision, False, True, self.n, 2 * d, dout, G, self.params[l], dS)
                 # G_in = relu'(H_l) * (dS_left + M^T dS_right): residual and gate in the aggregation's epilogue
-                mg.spmm(self.ctx, self.g, dS[:, d:], Gn, self.dims[l], transposed=True,
+                self._spmm(dS[:, d:], Gn, self.dims[l], transposed=True,
                         epi=mg.make_epilogue(residual=dS[:, :d], residual_scale=1.0, gate_scale=1.0, **gate))
 
 
@@ -225,9 +229,9 @@ class GinTrainer(_Base):
             H, d = self.H[l], self.dims[l]
             if self.upd[l]:
                 mg.gemm(self.ctx, product_precision(self.precision, True), False, False, self.n, h, d, H, self.params[l], self.U)
-                mg.spmm(self.ctx, self.g, self.U, self.T[l], h, epi=mg.make_epilogue(residual=self.U, residual_scale=keep, bias=self.params[L + l], relu=True))
+                self._spmm(self.U, self.T[l], h, epi=mg.make_epilogue(residual=self.U, residual_scale=keep, bias=self.params[L + l], relu=True))
             else:
-                mg.spmm(self.ctx, self.g, H, self.Z[l], d, epi=mg.make_epilogue(residual=H, residual_scale=keep))
+                self._spmm(H, self.Z[l], d, epi=mg.make_epilogue(residual=H, residual_scale=keep))
                 mg.gemm(self.ctx, self.precision, False, False, self.n, h, d, self.Z[l], self.params[l], self.T[l],
                         epi=mg.make_epilogue(bias=self.params[L + l], relu=True, sign_bits=self.signs_T[l]))
             last = l == L - 1
@@ -248,7 +252,7 @@ class GinTrainer(_Base):
                 Gn = (self.Ga if (L - 1 - l) % 2 == 0 else self.Gb).view(-1)[: self.n * self.ld[l]].view(self.n, self.ld[l])   # the two buffers alternate
             if self.upd[l]:
                 mg.colsum(self.ctx, self.dT, self.grads[L + l], h)
-                mg.spmm(self.ctx, self.g, self.dT, self.U, h, transposed=True, epi=mg.make_epilogue(residual=self.dT, residual_scale=keep))
+                self._spmm(self.dT, self.U, h, transposed=True, epi=mg.make_epilogue(residual=self.dT, residual_scale=keep))
                 mg.weight_grad(self.ctx, self.precision, d, h, self.n, self.H[l], self.U, self.grads[l])
                 if l > 0:
                     mg.gemm(self.ctx, self.precision, False, True, self.n, d, h, self.U, self.params[l], Gn, epi=mg.make_epilogue(gate_bits=self.signs_H[l], gate_scale=1.0))
@@ -259,6 +263,6 @@ class GinTrainer(_Base):
                 dZ = self.dZ.view(-1)[: self.n * self.ld[l]].view(self.n, self.ld[l])
                 mg.gemm(self.ctx, self.precision, False, True, self.n, d, h, self.dT, self.params[l], dZ)
                 # G_in = relu'(H_l) * ((1 + eps) dZ + A^T dZ)
-                mg.spmm(self.ctx, self.g, dZ, Gn, d, transposed=True,
+                self._spmm(dZ, Gn, d, transposed=True,
                         epi=mg.make_epilogue(residual=dZ, residual_scale=keep, gate_bits=self.signs_H[l], gate_scale=1.0))
                 G = Gn

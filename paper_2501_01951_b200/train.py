@@ -53,14 +53,16 @@ class GcnTrainer:
         self.cache_first_aggregation = bool(cache_first_aggregation)
         self._first_aggregation_valid = False
         # every iteration aggregates over this graph: its dense corner is laid out for the tensor cores.  fp32 iterations keep the
-        # gather kernels' order of sums, as their products under a ReLU do (signs near zero go by it)
-        if precision != mg.PREC_FP32 and n_chunks <= 1:
-            mg.graph_prepare_tiles(graph)
+        # gather kernels' order of sums, as their products under a ReLU do (signs near zero go by it), whatever else is made
+        # on the graph; so do iterations in chunks, whose forward pass has no tiles
+        tiles = precision != mg.PREC_FP32 and n_chunks <= 1
+        if tiles:
+            mg.graph_layout_tiles(graph)
         n, L = self.n, self.L
         orders = order if isinstance(order, (list, tuple)) else [order] * L
         self.descs, self.orders = [], []
         for l in range(L):
-            flags = (mg.LAYER_RELU if l < L - 1 else 0) | (mg.LAYER_FIRST if l == 0 else 0)
+            flags = (mg.LAYER_RELU if l < L - 1 else 0) | (mg.LAYER_FIRST if l == 0 else 0) | (mg.LAYER_TILES if tiles else 0)
             if fuse_gate:
                 if l >= 1:
                     flags |= mg.LAYER_GATE_GIN      # apply layer l-1's ReLU mask while producing G_in

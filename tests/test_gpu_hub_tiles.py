@@ -324,3 +324,62 @@ def test_an_aggregation_without_memory_for_its_tiles_gathers(mg, graphs, w):
     assert not torch.equal(Zt, Zp) and (Zt - Zp).abs().max() <= 2e-6 * Zp.abs().max()
     assert mg.ctx_poll_status(ctx, raise_on_error=False) == 0
     ctx.close()
+
+
+def iteration(mg, ctx, g, kind, precision, dims=(64, 128, 16), **kwargs):
+    """Forward, loss and backward of a new trainer: logits, loss, predictions, gradients."""
+    from paper_2501_01951_b200.sage_gin import GinTrainer, SageTrainer
+    from paper_2501_01951_b200.train import GcnTrainer
+    u = lambda *shape: synth.uniform_tensor(shape, sum(shape), -0.3, 0.3)
+    pairs = list(zip(dims, dims[1:]))
+    Ws, bs = [u(*p) for p in pairs], [u(p[1]) for p in pairs]
+    if kind == "gcn":
+        tr = GcnTrainer(ctx, g, dims, precision, **kwargs)
+        tr.set_params(Ws, bs)
+    elif kind == "sage":
+        tr = SageTrainer(ctx, g, dims, precision)
+        tr.set_params(Ws, [w + 0.1 for w in Ws], bs)
+    else:
+        tr = GinTrainer(ctx, g, dims, 96, precision)
+        tr.set_params([u(d, 96) for d in dims[:-1]], [u(96) for _ in pairs], [u(96, d) for d in dims[1:]], bs)
+    gen = torch.Generator().manual_seed(5)
+    labels = torch.randint(0, dims[-1], (N,), generator=gen, dtype=torch.int32)
+    mask = (torch.rand(N, generator=gen) < 0.3).to(torch.uint8)
+    tr.set_inputs(features(dims[0], 3), labels.cuda(), mask.cuda())
+    tr.forward()
+    logits = (tr.X[-1] if kind == "gcn" else tr.logits)[:, :dims[-1]].clone()
+    tr.compute_loss(), tr.backward()
+    return [logits, tr.loss.clone(), tr.pred.clone()] + [t.clone() for t in (tr.dW + tr.db if kind == "gcn" else tr.grads)]
+
+
+@pytest.mark.parametrize("kind", ["gcn", "sage", "gin"])
+def test_who_else_uses_a_graph_changes_no_sums(mg, ctx, kind):
+    """fp32 trainers, trainers in chunks and plain aggregations give the same bits before and after a trainer that takes the tiles is made on
+    their graph, and so do recordings and their calls; the other way round it keeps its own."""
+    src, dst = edges(1)
+    flags = mg.GRAPH_SYMMETRISE | dict(gcn=mg.GRAPH_ADD_SELF_LOOPS, sage=mg.GRAPH_NORM_ROW, gin=mg.GRAPH_NORM_NONE)[kind]
+    g, alone = (mg.graph_create(ctx, N, src, dst, flags) for _ in range(2))
+    Y, Z = features(128, 3), torch.empty((N, 128), device="cuda")
+
+    def others():
+        mg.spmm(ctx, g, Y, Z, 128)
+        return [Z.clone(), *iteration(mg, ctx, g, kind, mg.PREC_FP32), *(iteration(mg, ctx, g, kind, mg.PREC_TF32, n_chunks=3) if kind == "gcn" else [])]
+
+    low = iteration(mg, ctx, alone, kind, mg.PREC_TF32)
+    before = others()
+    rec = mg.record(ctx, lambda: mg.spmm(ctx, g, Y, Z, 128))
+    assert all(torch.equal(a, b) for a, b in zip(low, iteration(mg, ctx, g, kind, mg.PREC_TF32)))
+    assert mg.graph_layout_tiles(g)[0] > 100
+    assert all(torch.equal(a, b) for a, b in zip(before, others()))
+    assert rec.replay() and torch.equal(Z, before[0])
+    assert all(torch.equal(a, b) for a, b in zip(low, iteration(mg, ctx, g, kind, mg.PREC_TF32)))
+    # asked for on the graph itself, plain aggregations take the tiles, and their recordings end
+    mg.graph_prepare_tiles(g)
+    assert not rec.replay()
+    mg.spmm(ctx, g, Y, Z, 128)
+    assert not torch.equal(Z, before[0])
+    for t, same in ((False, True), (True, False)):
+        mg.spmm(ctx, g, Y, Z, 128, tiles=t)
+        assert torch.equal(Z, before[0]) == same
+    assert all(torch.equal(a, b) for a, b in zip(before[1:], iteration(mg, ctx, g, kind, mg.PREC_FP32)))
+    rec.close(), g.close(), alone.close()

@@ -203,12 +203,15 @@ mixgcn_status mixgcn_graph_export_schedule(const mixgcn_graph* g, int transposed
  * tile of 256 x 128 that holds enough entries becomes a bitmap, and aggregations over all rows (not sampled, row-sparse,
  * row-filtered or chunked ones) that ask for it multiply it there, sums in fp32 as before but in another order.  Which calls
  * do is the calls' affair: layers with MIXGCN_LAYER_TILES, mixgcn_spmm_tiles, and, once mixgcn_graph_prepare_tiles has been
- * called, mixgcn_spmm.  Costs a few passes over the entries; for a graph that many aggregations will use.  Nothing happens on
+ * called, mixgcn_spmm.  Costs a few passes over the entries; for a graph that many aggregations will use: widths (n_widths
+ * of them, 0 = any) are the numbers of columns these will have, and where tiles pay at none of them none are built.  With
+ * ctx not null the scratch that aggregations of these widths need is set aside in that context.  Nothing happens on
  * graphs without such tiles, or the second time; without memory for the layout (or, in an aggregation, for its scratch)
  * the gather kernels do all the work, as they do without this call.  n_tiles, n_entries (nullable): tiles, and entries in
  * them, of the forward orientation.  Synchronises before returning; aggregations already enqueued are not affected, and
  * recordings that use the graph end when mixgcn_graph_prepare_tiles changes the order of their sums. */
-mixgcn_status mixgcn_graph_layout_tiles(mixgcn_graph* g, int64_t* n_tiles, int64_t* n_entries);
+mixgcn_status mixgcn_graph_layout_tiles(mixgcn_ctx* ctx, mixgcn_graph* g, int32_t n_widths, const int32_t* widths,
+                                        int64_t* n_tiles, int64_t* n_entries);
 mixgcn_status mixgcn_graph_prepare_tiles(mixgcn_graph* g, int64_t* n_tiles, int64_t* n_entries);
 
 /* A graph may be used only while its context exists; it may be destroyed after it. */

@@ -345,11 +345,12 @@ def graph_export_schedule(g: Graph, transposed: bool = False) -> torch.Tensor:
     return perm
 
 
-def graph_layout_tiles(g: Graph) -> tuple[int, int]:
+def graph_layout_tiles(g: Graph, widths=(), ctx: Ctx | None = None) -> tuple[int, int]:
     """Lay the dense corner of the graph out for the tensor cores -> (tiles, entries in them), for the calls that ask for it
-    (LAYER_TILES, spmm(tiles=True)).  Once per graph; later calls change nothing."""
+    (LAYER_TILES, spmm(tiles=True)), if it pays at one of the widths (none given: at any); their scratch is set aside in ctx.
+    Once per graph; later calls change nothing."""
     tiles, entries = C.c_int64(0), C.c_int64(0)
-    _check(lib.mixgcn_graph_layout_tiles(g.h, C.byref(tiles), C.byref(entries)))
+    _check(lib.mixgcn_graph_layout_tiles(None if ctx is None else ctx.h, g.h, C.c_int32(len(widths)), (C.c_int32 * len(widths))(*widths), C.byref(tiles), C.byref(entries)))
     return tiles.value, entries.value
 
 

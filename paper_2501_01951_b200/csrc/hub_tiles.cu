@@ -32,6 +32,7 @@
 // out: the entries of small columns carry a row's sum there.
 #include <cub/cub.cuh>
 
+#include <algorithm>
 #include <mutex>
 #include <new>
 #include <vector>
@@ -574,9 +575,10 @@ void free_tiles(HubTiles* t) {
     delete t;
 }
 
-// Tiles of one orientation.  *out stays null where there are too few.
-mixgcn_status build_tiles(const mixgcn_graph* g, bool transposed, HubTiles** out, cudaStream_t s) {
+// Tiles of one orientation.  *out stays null where there are too few, and where they pay at none of the widths (*other_widths then).
+mixgcn_status build_tiles(const mixgcn_graph* g, bool transposed, int32_t n_widths, const int32_t* widths, HubTiles** out, bool* other_widths, cudaStream_t s) {
     *out = nullptr;
+    *other_widths = false;
     const CsrView &A = transposed ? g->bwd : g->fwd, &At = transposed ? g->fwd : g->bwd;
     const int64_t n = g->n, hubs = n < HUB_MAX ? n : HUB_MAX;
     if (g->nnz < HUB_MIN_ENTRIES) return MIXGCN_OK;
@@ -623,8 +625,8 @@ mixgcn_status build_tiles(const mixgcn_graph* g, bool transposed, HubTiles** out
     if (clusters > (t->n_tiles + LEAST_TILES - 1) / LEAST_TILES) clusters = (t->n_tiles + LEAST_TILES - 1) / LEAST_TILES;
     t->clusters = clusters;
     t->rem_nnz = g->nnz - t->entries;
-    // (one width of every lane split)
-    if (!hub_tiles_pay(t, HUB_SLICE) && !hub_tiles_pay(t, 160) && !hub_tiles_pay(t, 128) && !hub_tiles_pay(t, 64)) return MIXGCN_OK;
+    *other_widths = std::none_of(widths, widths + n_widths, [&](int32_t w) { return hub_tiles_pay(t, w); });
+    if (*other_widths) return MIXGCN_OK;
     std::vector<HubPiece> pieces;
     std::vector<int32_t> first_piece(clusters + 1), piece_first(t->row_blocks + 1, 0);
     int rb = 0;
@@ -771,39 +773,51 @@ mixgcn_status launch_hub_tiles(mixgcn_ctx* ctx, const HubTiles* t, int phase, in
 
 }  // namespace mixgcn
 
-extern "C" mixgcn_status mixgcn_graph_layout_tiles(mixgcn_graph* g, int64_t* n_tiles, int64_t* n_entries) {
-    if (!g) MIXGCN_FAIL(MIXGCN_EINVAL, "graph_layout_tiles: null graph");
+extern "C" mixgcn_status mixgcn_graph_layout_tiles(mixgcn_ctx* ctx, mixgcn_graph* g, int32_t n_widths, const int32_t* widths, int64_t* n_tiles, int64_t* n_entries) {
+    if (!g || n_widths < 0 || (n_widths > 0 && !widths)) MIXGCN_FAIL(MIXGCN_EINVAL, "graph_layout_tiles: bad argument");
+    constexpr int32_t ANY[] = {HUB_SLICE, 160, 128, 64};      // one of every lane split
+    const int32_t n_asked = n_widths ? n_widths : 4, *asked = n_widths ? widths : ANY;
     std::lock_guard<std::mutex> lock(g_build_mutex);
-    if (!g->tiles_tried) {
-        MIXGCN_CUDA(cudaSetDevice(g->device));
-        cudaStream_t s = g->ctx->side_stream[0];
-        LaunchScope scope(g->ctx, PH_GRAPH, s, 12);
-        HubTiles* made[2] = {nullptr, nullptr};
-        mixgcn_status st;
+    MIXGCN_CUDA(cudaSetDevice(g->device));
+    HubTiles* made[2] = {nullptr, nullptr};
+    bool other_widths[2] = {false, false};
+    mixgcn_status st = MIXGCN_OK;
+    for (int o = 0; o < 2 && st == MIXGCN_OK; ++o) {
+        if (g->tiles_tried[o]) continue;
+        if (o == 1 && (g->bwd_is_fwd || g->norm == 1)) {       // (row means transposed: see the errors above)
+            made[1] = g->bwd_is_fwd ? made[0] : nullptr;
+            other_widths[1] = g->bwd_is_fwd && other_widths[0];
+            continue;
+        }
+        LaunchScope scope(g->ctx, PH_GRAPH, g->ctx->side_stream[0], 6);
         try {
-            st = build_tiles(g, false, &made[0], s);
-            if (g->bwd_is_fwd) made[1] = made[0];
-            else if (st == MIXGCN_OK && g->norm != 1) st = build_tiles(g, true, &made[1], s);       // (row means transposed: see the errors above)
+            st = build_tiles(g, o == 1, n_asked, asked, &made[o], &other_widths[o], g->ctx->side_stream[0]);
         } catch (const std::bad_alloc&) {
             st = MIXGCN_ENOMEM;
         }
-        if (st != MIXGCN_OK) {         // (the gather kernels need none of it: where there is no memory for tiles there are none)
-            free_tiles(made[0]);
-            made[0] = made[1] = nullptr;
-            if (st != MIXGCN_ENOMEM) return st;
-        }
-        g->tiles[0].store(made[0], std::memory_order_release);
-        g->tiles[1].store(made[1], std::memory_order_release);
-        g->tiles_tried = true;
     }
+    if (st != MIXGCN_OK) {             // (the gather kernels need none of it: where there is no memory for tiles there are none)
+        free_tiles(made[0]);
+        made[0] = made[1] = nullptr;
+        other_widths[0] = other_widths[1] = false;
+        if (st != MIXGCN_ENOMEM) return st;
+    }
+    for (int o = 0; o < 2; ++o)
+        if (!g->tiles_tried[o]) {
+            g->tiles[o].store(made[o], std::memory_order_release);
+            g->tiles_tried[o] = !other_widths[o];
+        }
     const HubTiles* t = g->tiles[0].load(std::memory_order_acquire);
     if (n_tiles) *n_tiles = t ? t->n_tiles : 0;
     if (n_entries) *n_entries = t ? t->entries : 0;
+    if (!ctx) return MIXGCN_OK;
+    for (const auto& tiles : g->tiles)
+        for (int32_t i = 0; i < n_widths; ++i) MIXGCN_TRY(reserve_tiles_scratch(ctx, tiles.load(std::memory_order_acquire), widths[i]));
     return MIXGCN_OK;
 }
 
 extern "C" mixgcn_status mixgcn_graph_prepare_tiles(mixgcn_graph* g, int64_t* n_tiles, int64_t* n_entries) {
-    MIXGCN_TRY(mixgcn_graph_layout_tiles(g, n_tiles, n_entries));
+    MIXGCN_TRY(mixgcn_graph_layout_tiles(nullptr, g, 0, nullptr, n_tiles, n_entries));
     // (recorded calls of mixgcn_spmm sum in the other order)
     if (!g->tiles_in_spmm.exchange(true, std::memory_order_acq_rel) && g->tiles[0].load(std::memory_order_acquire)) memory_given_back(g->memory);
     return MIXGCN_OK;

@@ -33,6 +33,8 @@ struct HubTiles {
 
 namespace mixgcn {
 
+// the scratch of an aggregation of w columns, where it takes the tiles (t may be null) and there is memory for it
+mixgcn_status reserve_tiles_scratch(mixgcn_ctx* ctx, const HubTiles* t, int32_t w);
 bool hub_tiles_pay(const HubTiles* t, int32_t w);
 // bytes of scratch for w columns: partial rows of ldp floats, images (of at most 256 columns) from *images_at on
 int64_t hub_tiles_scratch(const HubTiles* t, int32_t w, int64_t ldp, int64_t* images_at);

@@ -180,7 +180,7 @@ struct mixgcn_graph {
     CsrView fwd, bwd;  // bwd aliases fwd when symmetric
     // tiles of the dense corner of fwd and bwd (the same object where bwd aliases fwd), null where there are none
     std::atomic<struct HubTiles*> tiles[2];
-    bool tiles_tried;
+    bool tiles_tried[2];               // built, or there is nothing to build at any width
     std::atomic<bool> tiles_in_spmm;   // mixgcn_spmm takes them (mixgcn_graph_prepare_tiles)
 };
 

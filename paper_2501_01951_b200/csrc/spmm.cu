@@ -259,6 +259,10 @@ void dispatch_filtered(const SpmmParams& p, cudaStream_t s) {
 constexpr int MAX_SLICE = 1024;      // columns per launch at most: 8 float4 per lane
 constexpr int DEFAULT_SLICE = 256;   // widths above this run as slices of this many columns (2 float4 per lane, four CTAs per SM)
 
+int slice_of(const mixgcn_ctx* ctx) {
+    return ctx->spmm_slice_cols > 0 ? (ctx->spmm_slice_cols < MAX_SLICE ? ctx->spmm_slice_cols : MAX_SLICE) : DEFAULT_SLICE;
+}
+
 // bytes of scratch of one slice of w columns where tiles run: partial rows of the other entries' segments, then what the tiles need
 int64_t tiles_scratch(const HubTiles* t, int32_t w, int64_t ldp, int64_t* images_at) {
     return t->rem.full.total_segs * ldp * (int64_t)sizeof(float) + 1024 + hub_tiles_scratch(t, w, ldp, images_at);
@@ -267,6 +271,14 @@ int64_t tiles_scratch(const HubTiles* t, int32_t w, int64_t ldp, int64_t* images
 }  // namespace
 
 namespace mixgcn {
+
+mixgcn_status reserve_tiles_scratch(mixgcn_ctx* ctx, const HubTiles* t, int32_t w) {
+    if (!t || w <= 0 || !hub_tiles_pay(t, w)) return MIXGCN_OK;
+    const int32_t cols = w < slice_of(ctx) ? w : slice_of(ctx);
+    int64_t images_at = 0;
+    const mixgcn_status st = ensure_workspace_spmm(ctx, tiles_scratch(t, cols, ((int64_t)cols + 3) / 4 * 4, &images_at));
+    return st == MIXGCN_ENOMEM ? MIXGCN_OK : st;
+}
 
 // Aggregation of all rows (chunks <= 1) or of row chunk k of `chunks` (the pipeline's chunks), each
 // with its own schedule: long rows as column-ordered segments, then rows longest first, short rows packed.
@@ -299,7 +311,7 @@ mixgcn_status launch_spmm(mixgcn_ctx* ctx, const mixgcn_graph* g, const CsrView&
         tiles = g->tiles[&A == &g->bwd].load(std::memory_order_acquire);
         if (tiles && !hub_tiles_pay(tiles, w)) tiles = nullptr;
     }
-    const int slice = lf ? MAX_SLICE : ctx->spmm_slice_cols > 0 ? (ctx->spmm_slice_cols < MAX_SLICE ? ctx->spmm_slice_cols : MAX_SLICE) : DEFAULT_SLICE;
+    const int slice = lf ? MAX_SLICE : slice_of(ctx);
     if (tiles) {        // scratch of the widest slice; the gather kernels alone where there is no memory for it
         int64_t images_at = 0;
         const int64_t ldp = ((int64_t)(w < slice ? w : slice) + 3) / 4 * 4;

@@ -46,8 +46,6 @@ class _Base:
     def __init__(self, ctx, graph, dims, precision):
         self.ctx, self.g, self.precision = ctx, graph, precision
         self.tiles = precision != mg.PREC_FP32      # as in train.py
-        if self.tiles:
-            mg.graph_layout_tiles(graph)
         self.dims = tuple(int(d) for d in dims)
         self.L = len(self.dims) - 1
         self.n = graph.n
@@ -58,6 +56,10 @@ class _Base:
         self.n_correct = torch.zeros(1, dtype=torch.int64, device=self.device)
         self.params, self.grads, self.m, self.v = [], [], [], []
         self._replay = mg.Replayer(ctx)      # the calls of an iteration, recorded once they have come twice with the same buffers
+
+    def _layout_tiles(self, widths):
+        if self.tiles:
+            mg.graph_layout_tiles(self.g, widths, self.ctx)
 
     def _spmm(self, *args, **kwargs):
         mg.spmm(self.ctx, self.g, *args, tiles=self.tiles, **kwargs)
@@ -110,6 +112,7 @@ class SageTrainer(_Base):
         super().__init__(ctx, graph, dims, precision)
         n, L, ld = self.n, self.L, self.ld
         self.upd = [update_first(self.dims[l], self.dims[l + 1], l == 0, precision, l < L - 1) for l in range(L)]
+        self._layout_tiles([self.dims[l + 1] if self.upd[l] else self.dims[l] for l in range(L)])
         self.S = [self._z(n, ld[l] if self.upd[l] else 2 * ld[l]) for l in range(L)]
         # gradients w.r.t. the layers' outputs: [G | M^T G] where the layer updates first, G otherwise; the hidden ones take
         # turns in two buffers, which the forward pass uses for the update-first products
@@ -202,6 +205,7 @@ class GinTrainer(_Base):
         n, L, ld = self.n, self.L, self.ld
         self.hidden, self.ldh, self.gin_eps = int(hidden), round4(hidden), float(gin_eps)
         self.upd = [update_first(self.dims[l], self.hidden, l == 0, precision, True) for l in range(L)]
+        self._layout_tiles([self.hidden if self.upd[l] else self.dims[l] for l in range(L)])
         self.H = [None] + [self._z(n, ld[l]) for l in range(1, L)]
         # aggregate-first layers keep (1 + eps) H + A H for their weight gradient; update-first ones share scratch for H W1
         # and its gradient

@@ -56,8 +56,6 @@ class GcnTrainer:
         # gather kernels' order of sums, as their products under a ReLU do (signs near zero go by it), whatever else is made
         # on the graph; so do iterations in chunks, whose forward pass has no tiles
         tiles = precision != mg.PREC_FP32 and n_chunks <= 1
-        if tiles:
-            mg.graph_layout_tiles(graph)
         n, L = self.n, self.L
         orders = order if isinstance(order, (list, tuple)) else [order] * L
         self.descs, self.orders = [], []
@@ -75,6 +73,8 @@ class GcnTrainer:
             d.order = o
             self.descs.append(d)
             self.orders.append(o)
+        if tiles:
+            mg.graph_layout_tiles(graph, [self.dims[l] if o == mg.ORDER_AGG_FIRST else self.dims[l + 1] for l, o in enumerate(self.orders)], ctx)
         z = lambda r, c: torch.zeros((r, c), dtype=torch.float32, device=self.device)
         self.X = [None] + [z(n, self.ld[l]) for l in range(1, L + 1)]
         self.saved = [z(n, self.descs[l].ld_saved) for l in range(L)]

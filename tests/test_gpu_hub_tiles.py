@@ -383,3 +383,22 @@ def test_who_else_uses_a_graph_changes_no_sums(mg, ctx, kind):
         assert torch.equal(Z, before[0]) == same
     assert all(torch.equal(a, b) for a, b in zip(before[1:], iteration(mg, ctx, g, kind, mg.PREC_FP32)))
     rec.close(), g.close(), alone.close()
+
+
+def test_tiles_are_laid_out_for_the_widths_that_will_be_used(mg):
+    """A graph whose tiles pay at 132 columns and not at 64: a trainer of narrow layers has none built, a later one of wider layers has, with
+    the scratch of its aggregations set aside (none of them allocates)."""
+    ctx = mg.ctx_create(0)
+    n = 300_000
+    src, dst = synth.rmat_graph(n, 4_650_000, 3, device="cuda")
+    g = mg.graph_create(ctx, n, src, dst)
+    assert mg.graph_layout_tiles(g, [64, 3]) == (0, 0) and mg.graph_layout_tiles(g, [64], ctx) == (0, 0)
+    tiles, entries = mg.graph_layout_tiles(g, [64, 132], ctx)
+    assert tiles > 500 and mg.graph_layout_tiles(g) == (tiles, entries)
+    Y, Z, Zp = (torch.randn((n, 132), device="cuda") for _ in range(3))
+    mg.ctx_set_option(ctx, mg.OPT_DEBUG_FAIL_ALLOC, 1)
+    mg.spmm(ctx, g, Y, Z, 132, tiles=True)
+    mg.ctx_set_option(ctx, mg.OPT_DEBUG_FAIL_ALLOC, 0)
+    mg.spmm(ctx, g, Y, Zp, 132, tiles=False)
+    assert not torch.equal(Z, Zp) and (Z - Zp).abs().max() <= 4e-6 * Zp.abs().max()
+    g.close(), ctx.close()

@@ -86,7 +86,7 @@ mixgcn_status mixgcn_debug_poke_col(mixgcn_graph* g, int64_t entry, int32_t valu
  * the two-float4-per-lane kernels keep four CTAs per SM; measured fastest at width 1024); otherwise
  * a multiple of 4 in [4, 1024].  Narrow slices shrink the part of the input
  * that must stay in the L2 at the price of re-reading the index once per slice; results do not
- * depend on the slicing. */
+ * depend on the slicing.  (Aggregations that take a graph's tiles keep slices of 256.) */
 #define MIXGCN_OPT_SPMM_SLICE_COLS 1
 /* MIXGCN_OPT_LOSS_TRAIN_ROWS_ONLY: 0 (default) = mixgcn_loss_softmax_xent as documented; 1 = rows
  * outside the train mask are not looked at: their logits are not read, their dlogits rows are

@@ -259,13 +259,15 @@ void dispatch_filtered(const SpmmParams& p, cudaStream_t s) {
 constexpr int MAX_SLICE = 1024;      // columns per launch at most: 8 float4 per lane
 constexpr int DEFAULT_SLICE = 256;   // widths above this run as slices of this many columns (2 float4 per lane, four CTAs per SM)
 
-int slice_of(const mixgcn_ctx* ctx) {
-    return ctx->spmm_slice_cols > 0 ? (ctx->spmm_slice_cols < MAX_SLICE ? ctx->spmm_slice_cols : MAX_SLICE) : DEFAULT_SLICE;
-}
-
 // bytes of scratch of one slice of w columns where tiles run: partial rows of the other entries' segments, then what the tiles need
 int64_t tiles_scratch(const HubTiles* t, int32_t w, int64_t ldp, int64_t* images_at) {
     return t->rem.full.total_segs * ldp * (int64_t)sizeof(float) + 1024 + hub_tiles_scratch(t, w, ldp, images_at);
+}
+// of the widest slice of a call of w columns
+int64_t tiles_scratch(const HubTiles* t, int32_t w) {
+    const int32_t cols = w < DEFAULT_SLICE ? w : DEFAULT_SLICE;
+    int64_t images_at = 0;
+    return tiles_scratch(t, cols, ((int64_t)cols + 3) / 4 * 4, &images_at);
 }
 
 }  // namespace
@@ -274,9 +276,7 @@ namespace mixgcn {
 
 mixgcn_status reserve_tiles_scratch(mixgcn_ctx* ctx, const HubTiles* t, int32_t w) {
     if (!t || w <= 0 || !hub_tiles_pay(t, w)) return MIXGCN_OK;
-    const int32_t cols = w < slice_of(ctx) ? w : slice_of(ctx);
-    int64_t images_at = 0;
-    const mixgcn_status st = ensure_workspace_spmm(ctx, tiles_scratch(t, cols, ((int64_t)cols + 3) / 4 * 4, &images_at));
+    const mixgcn_status st = ensure_workspace_spmm(ctx, tiles_scratch(t, w));
     return st == MIXGCN_ENOMEM ? MIXGCN_OK : st;
 }
 
@@ -311,14 +311,13 @@ mixgcn_status launch_spmm(mixgcn_ctx* ctx, const mixgcn_graph* g, const CsrView&
         tiles = g->tiles[&A == &g->bwd].load(std::memory_order_acquire);
         if (tiles && !hub_tiles_pay(tiles, w)) tiles = nullptr;
     }
-    const int slice = lf ? MAX_SLICE : slice_of(ctx);
     if (tiles) {        // scratch of the widest slice; the gather kernels alone where there is no memory for it
-        int64_t images_at = 0;
-        const int64_t ldp = ((int64_t)(w < slice ? w : slice) + 3) / 4 * 4;
-        const mixgcn_status st = ensure_workspace_spmm(ctx, tiles_scratch(tiles, w < slice ? w : slice, ldp, &images_at));
+        const mixgcn_status st = ensure_workspace_spmm(ctx, tiles_scratch(tiles, w));
         if (st == MIXGCN_ENOMEM) tiles = nullptr;
         else MIXGCN_TRY(st);
     }
+    // (with tiles the order of a row's sums goes by the slices' width, so that they always have the default one)
+    const int slice = tiles ? DEFAULT_SLICE : lf ? MAX_SLICE : ctx->spmm_slice_cols > 0 ? (ctx->spmm_slice_cols < MAX_SLICE ? ctx->spmm_slice_cols : MAX_SLICE) : DEFAULT_SLICE;
     const CsrView& V = tiles ? tiles->rem : A;       // with tiles: what they leave
     const SpmmSchedule& S = chunks > 1 ? A.chunk[k] : V.full;
     if (S.n_rows <= 0) return MIXGCN_OK;
@@ -428,8 +427,8 @@ mixgcn_status launch_spmm(mixgcn_ctx* ctx, const mixgcn_graph* g, const CsrView&
         // the tiles first: the launch behind waits for their sums
         uint8_t* base = reinterpret_cast<uint8_t*>(((uintptr_t)partial + seg_bytes + 1023) & ~(uintptr_t)1023);
         float* sums = reinterpret_cast<float*>(base);
-        for (int c0 = 0; c0 < p.w; c0 += HUB_SLICE)
-            MIXGCN_TRY(launch_hub_tiles(ctx, tiles, phase, p.w - c0 < HUB_SLICE ? p.w - c0 : HUB_SLICE, p.Y + j0 + c0, ldy, p.y_rows, sums + c0, ldp, base + images_at, s));
+        static_assert(DEFAULT_SLICE <= HUB_SLICE, "a slice is one product");
+        MIXGCN_TRY(launch_hub_tiles(ctx, tiles, phase, p.w, p.Y + j0, ldy, p.y_rows, sums, ldp, base + images_at, s));
         SpmmHubParams hp{};
         static_cast<SpmmParams&>(hp) = p;
         hp.hub_rank = tiles->rank; hp.piece_first = tiles->piece_first; hp.row_scale = tiles->row_scale;

@@ -402,3 +402,19 @@ def test_tiles_are_laid_out_for_the_widths_that_will_be_used(mg):
     mg.spmm(ctx, g, Y, Zp, 132, tiles=False)
     assert not torch.equal(Z, Zp) and (Z - Zp).abs().max() <= 4e-6 * Zp.abs().max()
     g.close(), ctx.close()
+
+
+@pytest.mark.parametrize("w", [96, 100, 161, 260, 300])
+def test_sums_do_not_depend_on_the_slices(mg, ctx, graphs, w):
+    """Slices below, at and above the widths at which the kernels' lane splits and the product's accumulators change."""
+    _, tiled, _ = graphs["sym", True]
+    Y, want = features(w, 5), torch.empty((N, (w + 3) // 4 * 4), device="cuda")
+    mg.spmm(ctx, tiled, Y, want, w)
+    for cols in (32, 64, 100, 128, 1024):
+        Z = torch.full_like(want, 7.0)
+        mg.ctx_set_option(ctx, mg.OPT_SPMM_SLICE_COLS, cols)
+        try:
+            mg.spmm(ctx, tiled, Y, Z, w)
+        finally:
+            mg.ctx_set_option(ctx, mg.OPT_SPMM_SLICE_COLS, 0)
+        assert torch.equal(Z, want), cols

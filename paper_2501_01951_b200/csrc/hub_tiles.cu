@@ -616,7 +616,7 @@ mixgcn_status build_tiles(const mixgcn_graph* g, bool transposed, int32_t n_widt
     t->row_blocks = h.last_row_block + 1; t->kblocks = h.last_col_block + 1;
     t->n_cols = (int64_t)t->kblocks * COLS < n ? (int64_t)t->kblocks * COLS : n;
     const int64_t covered = (int64_t)t->row_blocks * ROWS, rows = covered < n ? covered : n;
-    t->nodes = At.full.perm; t->rows = A.full.perm;
+    t->nodes = At.full.perm;
     // every pair of CTAs takes as many consecutive tiles as any other; a piece ends where a row of tiles does
     int clusters = 0;
     MIXGCN_TRY(resident_pairs(g->ctx, &clusters));
@@ -638,7 +638,7 @@ mixgcn_status build_tiles(const mixgcn_graph* g, bool transposed, int32_t n_widt
             const int row_end = host_first[(rb + 1) * cbs];
             int stop = row_end < end ? row_end : end;
             if (stop > at + PIECE_MAX) stop = at + PIECE_MAX;
-            pieces.push_back(HubPiece{rb, at, stop, 0});
+            pieces.push_back(HubPiece{at, stop});
             piece_first[rb + 1]++;
             at = stop;
         }

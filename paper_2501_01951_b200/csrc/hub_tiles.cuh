@@ -8,7 +8,7 @@ constexpr int HUB_ROWS = 256, HUB_COLS = 128;   // a tile
 constexpr int HUB_SLICE = 256;                  // most columns of one product
 constexpr int HUB_TILE_MIN = 1200;              // entries from which a tile pays: 60 us to gather them (256 columns), 27 for the tile
 constexpr int64_t HUB_MIN_ENTRIES = 1 << 20;    // graphs below this, and tiles that hold less than a quarter of it, are not worth the launches
-struct HubPiece { int32_t row_block, begin, end, pad; };       // tiles [begin, end) of one row of tiles
+struct HubPiece { int32_t begin, end; };       // tiles [begin, end) of one row of tiles
 
 }  // namespace mixgcn
 
@@ -19,7 +19,6 @@ struct HubTiles {
     int n_tiles, n_pieces, clusters;
     int64_t entries;           // stored entries that lie in tiles
     const int32_t* nodes;      // [n_cols] node of a hub column (the transposed schedule's perm)
-    const int32_t* rows;       // node of a hub row (the schedule's perm)
     int32_t* rank;             // [n] rank of a row that lies in a row of tiles, -1 otherwise
     float *col_scale, *row_scale;
     uint32_t* bits;            // [n_tiles][256 rows][4 words]

@@ -433,7 +433,7 @@ mixgcn_status launch_spmm(mixgcn_ctx* ctx, const mixgcn_graph* g, const CsrView&
         static_cast<SpmmParams&>(hp) = p;
         hp.hub_rank = tiles->rank; hp.piece_first = tiles->piece_first; hp.row_scale = tiles->row_scale;
         hp.tile_sums = sums; hp.n_tile_sums = (int64_t)tiles->n_pieces * HUB_ROWS;
-        MIXGCN_TRY(launch_rows_hub(ctx, hp, S, narrow, lf != nullptr, row_limit, phase, partial, s));
+        MIXGCN_TRY(launch_rows_hub(ctx, hp, S, narrow, lf != nullptr, phase, partial, s));
     }
     MIXGCN_CUDA(cudaGetLastError());
     // sign bitmap of the result: one more pass over the rows this call wrote

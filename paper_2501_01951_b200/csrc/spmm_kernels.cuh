@@ -92,7 +92,7 @@ inline NarrowCfg narrow_cfg(int w_total) {
 }
 // One slice of an aggregation over the rows of schedule S: segments of the long rows (partial rows at `partial`), the other rows by
 // bucket, the combination.  In spmm_hub.cu, for schedules of what tiles leave:
-mixgcn_status launch_rows_hub(mixgcn_ctx* ctx, const SpmmHubParams& p, const SpmmSchedule& S, NarrowCfg narrow, bool loss, int64_t row_limit, int phase, float* partial, cudaStream_t s);
+mixgcn_status launch_rows_hub(mixgcn_ctx* ctx, const SpmmHubParams& p, const SpmmSchedule& S, NarrowCfg narrow, bool loss, int phase, float* partial, cudaStream_t s);
 
 }  // namespace mixgcn
 
@@ -187,7 +187,7 @@ __device__ __forceinline__ void store_lean(const Params& p, int64_t u, int c4, f
 
 // Which lean instance serves this launch (EPI_ANY: none does).
 inline int pick_epi(const Params& p) {
-    if (p.out_bits && p.bits_skip) return EPI_ANY;                 // the sampled aggregation skips gathers: general instance
+    if (!HUB && p.out_bits && p.bits_skip) return EPI_ANY;                 // the sampled aggregation skips gathers: general instance
     if (p.partial) return EPI_PLAIN;                               // a partial row never has an epilogue
     if (p.drop || p.residual) return EPI_ANY;
     const bool bias = p.bias != nullptr || p.relu, gate = p.gate != nullptr, bits = p.out_bits != nullptr;
@@ -553,7 +553,7 @@ __global__ void __launch_bounds__(256, SPMM_MINB) spmm_warp_kernel(const Params 
 #pragma unroll
     for (int v = 0; v < VPL; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
     unsigned keep = 0xFFFFFFFFu;
-    if (EPI == EPI_ANY && p.out_bits && p.bits_skip) keep = kept_groups<CL, VPL>(p, u, cl, w4);
+    if (!HUB && EPI == EPI_ANY && p.out_bits && p.bits_skip) keep = kept_groups<CL, VPL>(p, u, cl, w4);
     warp_segment<CL, VPL>(p, b, r.z, lane, w4, acc, keep);
     if (lane < CL) {
         if (!p.partial) add_tiles<CL, VPL>(p, u, cl, w4, acc);
@@ -934,7 +934,7 @@ mixgcn_status launch_rows(mixgcn_ctx* ctx, Params p, const SpmmSchedule& S, Narr
         p.partial = partial;
         LaunchScope scope(ctx, phase, s);
         p.idx_begin = 0; p.idx_end = S.total_segs;
-        if (p.out_bits && p.bits_skip) p.seg_perm = S.perm;       // a segment's record names its long row by ordinal
+        if (!HUB && p.out_bits && p.bits_skip) p.seg_perm = S.perm;       // a segment's record names its long row by ordinal
         if (narrow.cl) dispatch_narrow(p, narrow, true, false, s, early);
         else dispatch(p, p.w <= SPMM_FOLD_WMAX ? SPMM_FOLD_SEG : 1, s, early);
         p.seg_perm = nullptr; p.partial = nullptr;
@@ -945,7 +945,7 @@ mixgcn_status launch_rows(mixgcn_ctx* ctx, Params p, const SpmmSchedule& S, Narr
     bound[0] = S.n_long;
     for (int q = 0; q < 3; ++q) bound[q + 1] = S.rows_above[q] > S.n_long ? S.rows_above[q] : S.n_long;
     bound[4] = S.n_rows;
-    if (row_limit >= 0 && row_limit < S.n_rows) {
+    if (!HUB && row_limit >= 0 && row_limit < S.n_rows) {
         // rows come longest first: only the first row_limit of them are wanted (the rest are empty)
         const int64_t lim = row_limit > S.n_long ? row_limit : S.n_long;
         for (int q = 1; q < 5; ++q) if (bound[q] > lim) bound[q] = lim;

@@ -129,6 +129,12 @@ def test_hot_aggregation_kernels_compile_without_register_spills(tmp_path):
     assert not spilled, spilled
 
 
+def test_no_aggregation_kernel_beside_tiles_spills(tmp_path):
+    """The same kernels compiled for what tiles leave, with the tiles' sums and those with the loss among them: none spills."""
+    entries = spills("spmm_hub.cu", tmp_path)
+    assert len(entries) > 200 and not [e for e in entries if e[1] or e[2]]
+
+
 def test_split_products_compile_without_register_spills(tmp_path):
     """The register split of their roles (setmaxnreg) leaves the epilogue room for a tile's sums.  The converting product has none
     and spills 64 bytes: no more than that."""

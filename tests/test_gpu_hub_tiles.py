@@ -418,3 +418,56 @@ def test_sums_do_not_depend_on_the_slices(mg, ctx, graphs, w):
         finally:
             mg.ctx_set_option(ctx, mg.OPT_SPMM_SLICE_COLS, 0)
         assert torch.equal(Z, want), cols
+
+
+def gcn(mg, ctx, g, dims, precision, **kwargs):
+    from paper_2501_01951_b200.train import GcnTrainer
+    u = lambda *shape: synth.uniform_tensor(shape, sum(shape), -0.3, 0.3)
+    tr = GcnTrainer(ctx, g, dims, precision, **kwargs)
+    tr.set_params([u(*p) for p in zip(dims, dims[1:])], [u(d) for d in dims[1:]])
+    gen = torch.Generator().manual_seed(5)
+    tr.set_inputs(features(dims[0], 3), torch.randint(0, dims[-1], (N,), generator=gen, dtype=torch.int32).cuda(),
+                  (torch.rand(N, generator=gen) < 0.3).to(torch.uint8).cuda())
+    return tr
+
+
+@pytest.mark.parametrize("classes", [3, 16, 41, 65, 100, 128, 200, 256])
+def test_the_loss_inside_an_aggregation_with_tiles(mg, ctx, graphs, classes):
+    """Narrow, one, two and three float4 a lane: predictions, loss and gradient as from the logits of the separate calls; without tiles the
+    same to rounding (a probability moves with its logit, by less than 2e-6 of the largest)."""
+    tr = gcn(mg, ctx, graphs["sym", True][1], (64, 96, classes), mg.PREC_TF32, order=[mg.ORDER_AUTO, mg.ORDER_UPD_FIRST])
+    tr.forward()
+    tr.compute_loss()
+    want = [t.clone() for t in (tr.pred, tr.loss, tr.X[-1])]
+    tr.forward_and_loss()
+    assert torch.equal(tr.pred, want[0])
+    assert abs(tr.loss.item() - want[1].item()) <= 2e-6 * want[1].item()
+    assert (tr.X[-1] - want[2]).abs().max() <= 2e-6 * want[2].abs().max()
+    with_tiles = tr.X[-1].clone()
+    tr.descs[-1].flags &= ~mg.LAYER_TILES
+    tr.forward_and_loss()
+    assert not torch.equal(tr.X[-1], with_tiles) and (tr.X[-1] - with_tiles).abs().max() <= 1e-5 * with_tiles.abs().max()
+
+
+def test_bf16_copies_beside_tiles(mg, ctx, graphs):
+    """Those of A_hat X (aggregate first) and of a layer's output (update first)."""
+    tiled = graphs["sym", True][1]
+    tr = gcn(mg, ctx, tiled, (64, 128, 100), mg.PREC_BF16, order=mg.ORDER_AGG_FIRST, saved_lp_only=False)
+    tr.forward()
+    for l in range(2):
+        assert torch.equal(tr.saved_lp[l][:, :tr.dims[l]], tr.saved[l][:, :tr.dims[l]].bfloat16())
+    tr = gcn(mg, ctx, tiled, (64, 128, 100), mg.PREC_BF16, order=mg.ORDER_UPD_FIRST)
+    tr.forward()
+    copy = next(t for t in tr.lp if t.data_ptr() == tr.descs[0].x_out_lp)
+    assert torch.equal(copy[:, :128], tr.X[1][:, :128].bfloat16())
+
+
+@pytest.mark.parametrize("precision", ["PREC_TF32", "PREC_BF16"])
+def test_recorded_iterations_with_tiles(mg, ctx, graphs, precision):
+    """Epochs, replayed from the third on, against the calls one by one: the same weights."""
+    a, b = (gcn(mg, ctx, graphs["sym", True][1], (64, 128, 41), getattr(mg, precision)) for _ in range(2))
+    for t in range(1, 6):
+        a.epoch(t)
+        b.forward_and_loss(), b.backward(), b.step(t)
+    assert a._replays["iteration"].rec is not None
+    assert all(torch.equal(x, y) for x, y in zip(a.W + a.b, b.W + b.b))

@@ -388,12 +388,13 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 // means that all of them have.  A wait is passed at once where the launch did not ask for it.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// First statement of every kernel that launch_chained launches.  (Kernels with tensor memory wait before they allocate it: one that
-// waited with tensor memory in hand would keep it from the kernel that it waits for.  Split reductions, whose successor has hundreds of
-// blocks, wait only: those blocks, brought up beside them, cost a weight gradient of 150 K x 128 x 128 7 of 40 us.)
+// First statement of the kernels that launch_chained launches.  Split reductions begin with pdl_wait alone: their successor has hundreds of
+// blocks, which, brought up beside them, cost a weight gradient of 150 K x 128 x 128 7 of 40 us.  Kernels with tensor memory wait before
+// they allocate it: one that waited with tensor memory in hand would keep it from the kernel that it waits for.  (spmm_tiles_kernel
+// allocates first: the kernel before it has none, and as an ordinary launch has seen everything before it end.)
 __device__ __forceinline__ void chain_begin() { pdl_trigger(); pdl_wait(); }
 
-// Launches a kernel that begins with chain_begin: its blocks are brought up beside the end of whatever runs before it on the stream.
+// Launches a kernel that begins with chain_begin or pdl_wait: its blocks are brought up beside the end of whatever runs before it on the stream.
 // What a launch and its drain cost shows in iterations of short kernels (0.4 to 1 us a launch; 5 to 15 where memsets stood between them: an
 // iteration of 26 launches 86.5 -> 82.6 us, one of 33 with two memsets 168 -> 157).
 template <typename... Args>

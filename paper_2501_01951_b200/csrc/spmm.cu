@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(256) spmm_sparse_kernel(const SpmmParams p) {
 // Row-filtered output: only the rows u with row_filter[u] != 0 are wanted (the last layer of a
 // training step needs its output on train nodes only).  A warp scans 32 schedule records, tests the
 // filter byte of each record's row and computes the kept ones one after the other with all 32 lanes,
-// entries in the same order as spmm_group_kernel (bitwise the same rows).
+// entries in the same order as spmm_group_kernel (bitwise the same rows as a full call without tiles).
 template <int VPL>
 __global__ void __launch_bounds__(256) spmm_filtered_kernel(const SpmmParams p) {
     const int lane = threadIdx.x & 31;
@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(256) spmm_filtered_kernel(const SpmmParams p) 
 }
 
 // The same for narrow aggregations: entry order and lane split of the dense path (one group of CL lanes walks a row
-// of at most 12 entries, the whole warp shares a longer unit), so the rows are again bitwise those of the full call.
+// of at most 12 entries, the whole warp shares a longer unit), so the rows are again bitwise those of the full call without tiles.
 template <int CL, int VPL>
 __global__ void __launch_bounds__(256) spmm_filtered_narrow_kernel(const SpmmParams p) {
     constexpr int PACKED = SPMM_PACK_DEG[0];

@@ -5,31 +5,29 @@
 // tile is a bitmap of 4 KB, and its product with 128 rows of Y is three tensor-core products.
 //
 //  * An entry's value is row_scale[u] * col_scale[v] (both normalisations and the plain sum have that form), so the matrix that is
-//    multiplied holds zeros and ones only: exact in bf16.
-//  * Rows of Y are scaled by col_scale (and 2^24, see CUT_SCALE) and cut into three bf16 parts, x = x0 + x1 + x2 (24 bits, as in gemm_split.cu), once per
-//    call, into images of the shared-memory tiles (split_rows_kernel): a stage of the product is one contiguous copy a CTA.
-//  * The x0 (8 bits each) are summed in an accumulator of their own, the two smaller parts in another: an instruction cuts its sum off
-//    at 24 bits, towards zero, and sums of a hundred 8-bit numbers have next to nothing to lose there unless their sizes lie far apart.
-//    Every 128 terms (the smaller parts, 2^-8 of the others: every 1024) the epilogue warps add the accumulator to fp32 sums in registers,
-//    rounding to nearest, while others take the next terms: up to 160 columns leave room for two accumulators of the x0, up to 96 for four,
-//    and there every 64 terms have one (narrow gathers add up in short chains, and a tile's time is its hand-overs': + 4 % of it).
+//    multiplied holds zeros and ones only.
+//  * Rows of Y are scaled by col_scale and written as whole numbers of a unit that is a column's own, 2^-31 to 2^-30 of its largest number,
+//    in four signed digits of base 256, once per call, into images of the shared-memory tiles (column_range_kernel, cut_rows_kernel).
+//    Whole-number products (tcgen05 kind::i8) take half the time of bf16 ones and their 32-bit sums are exact, so a row's tiles are one
+//    chain: nothing is added up on the way, and the sum is rounded to fp32 once.  What is lost is half a unit a term.
+//  * Columns whose numbers lie far apart (the largest more than SPREAD_MAX binades above the geometric mean) take six digits, 2^-47; infinities, NaN and
+//    numbers further apart than that send the call's tiles to the FMA pipes.  The device decides, by whole numbers: no order of blocks changes it.
+//  * A stage of the product is a tile's bitmap, expanded to bytes by four warps, and one contiguous copy of the image a CTA.  64 columns of Y (32
+//    with six digits) have 256 (192) columns of TMEM, twice: one half adds up while the epilogue empties the other.
 //  * What is not in a tile is a matrix of its own, with a schedule of its own, for the gather kernels.  They run behind the tiles, and where
-//    they have a row's sum add the row's pieces to it (at most 64 tiles of one row of tiles each, in fp64), times row_scale.
+//    they have a row's sum add the row's pieces to it (one, or two where a pair's share ends in the row), times row_scale.
 //
-// Measured, R-MAT, 233 K nodes of mean degree 500 (20,470 tiles hold 74 % of the entries), 256 columns: 5.04 ms by gathers alone, 2.49 with the
-// tiles (0.82 the product, 0.03 the cut, 1.7 the rest of the matrix); more cases at hub_tiles_pay.
-// Bound: a tile of 256 x 128 by 256 columns takes a pair of CTAs 4,800 cycles, 3,072 of which its 24 instructions need; the rest is adding up
-// the accumulator of the x0, which nothing covers above 160 columns (every 256 terms instead: 3,700 cycles, and the error below).  One
-// CTA per tile of 128 x 128 took 5,630, bound by shared memory: a stage's image is written once and read once for 128 rows, here for
-// 256.  Also slow: loads of 16 columns from the accumulator; bitmaps expanded by shift and multiply and announced to the other CTA by the
-// expanding threads, whose arrival there waits for the loads they have under way (2,000 of 2,500 cycles).
-// Error against fp64 relative to the gather kernels' (2-norm; N(0,1), its positive halves, what a ReLU leaves of it):
-// R-MAT 300 K, mean degree 31, 132 columns 0.89, 0.88, 1.03; 60 K, 400 0.78, 0.72, 0.79, plain sums 0.38, 0.80, 0.78; 4,099 nodes, half of
-// their pairs joined, 64 to 256 columns 0.7 to 0.9, 0.4 to 0.7, 0.5 to 0.7.  One row in a thousand 2^15 times the others: 0.7 to 1.0, of
-// one sign 0.8 to 1.05 (60 K, plain sums, 64 columns 1.3).  Numbers of one sign spread further apart (exp(3 N(0,1))) are where
-// truncation shows: 1.0 to 1.7.  What it took: 256 terms an accumulator made the last three 1.2 to 2.9; pieces of any length, added up
-// in fp32, 2.1 of positive plain sums; the gather kernels' chains as they were 1.26 on the 300 K nodes.  Row means transposed are left
-// out: the entries of small columns carry a row's sum there.
+// Measured, R-MAT, 233 K nodes of mean degree 500 (22,224 tiles hold 75 % of the entries), 256 columns: 5.04 ms by gathers alone, 2.01 with the
+// tiles (0.41 the product, 0.06 range and cut, 1.5 the rest of the matrix); with three bf16 parts of 24 bits, added up every 128 terms, 2.51 (0.73,
+// 0.02, 1.7 with 20,601 tiles).
+// Bound: a tile of 256 x 128 by 64 columns takes a pair of CTAs 620 cycles, 512 of which its four instructions need.  What it took: arrivals at
+// the leader's barriers without a release at cluster scope (1,815 with; 1,230 with the arrivals relayed by a warp of its own), one barrier a
+// tile for both operands and one commit (850 with two rings), a warp each for images and bitmaps, 64 columns at a time and two accumulators
+// (128 in one: 1,690 cycles per 128 and 3,200 a piece, which rows of one or two tiles pay for: hence PIECE_COST).
+// Error against fp64 relative to the gather kernels' (2-norm; N(0,1), its positive halves, what a ReLU leaves of it, softmax gradients):
+// R-MAT 300 K, mean degree 31, 132 columns 0.87, 0.74, 0.88, 0.92; 60 K, 400 0.71, 0.49, 0.57, 0.76, plain sums 0.21, 0.45, 0.52, 0.25; 233 K, 170,
+// 256 columns 0.72, 0.49, 0.64, 0.78.  One row in a thousand 2^15 times the others 0.2 to 0.95; exp(3 N(0,1)) 0.1 to 0.8 (300 K nodes, 64 columns
+// 1.16).  Row means transposed are left out: the entries of small columns carry a row's sum there.
 #include <cub/cub.cuh>
 
 #include <algorithm>
@@ -46,32 +44,56 @@ using namespace mixgcn::tc;
 
 namespace {
 
-constexpr int ROWS = HUB_ROWS, COLS = HUB_COLS, PARTS = 3;
+constexpr int ROWS = HUB_ROWS, COLS = HUB_COLS;
 constexpr int HUB_MAX = 1 << 16, CB_MAX = HUB_MAX / COLS;       // most rows and columns that are looked at
-constexpr int CHUNK_BYTES = COLS * 128;         // image of 128 rows of Y x 64 columns: 128-byte rows, 128-byte swizzle
-constexpr int A_BYTES = 128 * COLS * 2;         // a CTA's rows of a tile expanded to bf16: two halves of 64 columns, K-major, 128-byte swizzle
-constexpr int EPI_WARPS = 8, EXP_WARP = 8, EXP_WARPS = 4, TMA_WARP = 12, MMA_WARP = 13, RELAY_WARP = 14, THREADS = 512;
-constexpr int EPI_REGS = 192, OTHER_REGS = 64;  // a thread's, of the 128 it is launched with
-constexpr int STAGES_MAX = 8, STAGE_SMEM = 128 * 1024, BOX_BYTES = 4096;
-constexpr int AHEAD = 4;
+constexpr int A_BYTES = 128 * COLS;       // a CTA's rows of a tile expanded to bytes: K-major, 128-byte swizzle
+constexpr int EPI_WARPS = 8, EXP_WARP = 8, EXP_WARPS = 4, TMA_WARP = 12, BITS_WARP = 13, MMA_WARP = 14, THREADS = 480;
+constexpr int SLOTS = 6, B_BYTES = 128 * COLS, BITS_BYTES = 128 * 16, SLOT_BYTES = A_BYTES + B_BYTES;     // a CTA's half of the widest accumulator; its rows' bitmaps
+constexpr int BOX_BYTES = 2048;
+constexpr int TILES_SMEM = SLOTS * (SLOT_BYTES + BITS_BYTES) + EPI_WARPS * BOX_BYTES + 1024;
+constexpr int AHEAD = 16;                       // tiles whose bitmaps are asked for in L2
+constexpr int COLUMN_COST = 1200;               // entries whose gathers take as long as cutting a block of 128 rows of Y
+constexpr int PIECE_COST = 3;                   // tiles that take as long as a piece does beside its tiles
 constexpr int LEAST_TILES = 8;                  // of a pair of CTAs
-constexpr int LO_TILES = 8;                     // tiles that the accumulator of the smaller parts takes; that of the largest takes one
-constexpr int PIECE_MAX = 64;                   // tiles of a piece: as many fp32 additions in a row
 constexpr uint32_t TMEM_COLS = 512;
-constexpr float SAFE_MAX = 0x1p100f;             // sums of 2^16 such terms stay finite
-// Rows of Y are cut this many times as large: bf16 has nothing below 2^-133, and the third part of a number of 2^-110 and less would
-// be gone (numbers of 1e-35: error 2e-6 to 1e-5 without, 2e-8 as the gathers have it with; 2^24 brings all of fp32 above the line).
-constexpr float CUT_SCALE = 0x1p24f;
+constexpr int GROUP = 16;                       // columns of Y whose digits lie together
+// Exponents between the largest number of a column and the mean of its others up to which four digits (31 bits below the largest) do, and
+// by how many more six reach.
+constexpr int SPREAD_MAX = 9, SPREAD_MORE = 16;
+
+enum { MODE_4 = 0, MODE_6 = 1, MODE_PLAIN = 2 };     // digits of a number; plain_pieces instead
+// What column_range_kernel leaves for the kernels behind it, and its own sums, which are zero between calls.
+struct Ranges {
+    int32_t shift[HUB_SLICE];                   // numbers are cut as multiples of 2^-shift (read by fours)
+    uint32_t top[HUB_SLICE];                    // largest number of a column, as bits
+    int32_t sum[HUB_SLICE], count[HUB_SLICE];   // exponents of its numbers but zeros, and how many
+    int32_t mode;
+    uint32_t done;                              // blocks that have added theirs
+};
+static_assert(TILES_WORD * 4 % 16 == 0 && TILES_WORD + (int)(sizeof(Ranges) / 4) <= STATUS_WORDS, "room beside the status words");
+
+// How w columns of Y are taken: in blocks, all digits of a block's columns side by side in an accumulator.
+struct Shape {
+    int digits, cols, blocks;                   // columns of a block (a multiple of GROUP), blocks
+    __host__ __device__ int n() const { return digits * cols; }                            // columns of the accumulator, at most 256
+    __host__ __device__ int image_bytes() const { return n() / 2 * COLS; }                 // a CTA's half of a tile's image
+};
+Shape make_shape(int digits, int w) {
+    const int most = (int)TMEM_COLS / 2 / digits / GROUP * GROUP;
+    Shape s;
+    s.digits = digits;
+    s.blocks = (w + most - 1) / most;
+    s.cols = ((w + s.blocks - 1) / s.blocks + GROUP - 1) / GROUP * GROUP;
+    return s;
+}
 
 struct TileParams {
     const HubPiece* pieces; const int32_t* first_piece; // pair i takes pieces first_piece[i] .. first_piece[i + 1] - 1
     const int32_t* tile_cb; const uint4* bits;
     float* partial; int64_t ldp;                        // row r of piece q goes to partial row q * ROWS + r
-    int w4, bn, chunks, stages;
-    // TMEM: accumulators of bn columns, those of the largest parts first.  hi_two: 1 if tiles take turns in two sets of them, hi_halves: 1 if
-    // the two halves of a tile's terms have one each; lo_col: the smaller parts' one
-    uint32_t hi_two, hi_halves, lo_col;
-    int32_t* unsafe;                                    // flag: not zero, plain_pieces instead, from what follows; then the CTAs done with it
+    int w4, kblocks;
+    Shape shape[2];                                     // by mode
+    const Ranges* ranges;
     const float* Y; int64_t ldy, y_rows;
     const int32_t* nodes; const float* col_scale; int64_t n_cols;
     int32_t* status;
@@ -80,9 +102,8 @@ struct TileParams {
 };
 
 struct Shared {
-    uint64_t b_full[STAGES_MAX], b_empty[STAGES_MAX];   // images: TMA -> MMA -> TMA
-    uint64_t a_full[2], a_empty[2];                     // expanded tiles: expansion -> MMA -> expansion
-    uint64_t hi_full[2], hi_empty[2], lo_full, lo_empty;   // the accumulators: MMA -> epilogue -> MMA
+    uint64_t bits_full[SLOTS], full[SLOTS], empty[SLOTS];     // a tile: bitmap -> expansion, with the image -> MMA -> all of them
+    uint64_t acc_full[2], acc_empty[2];                 // accumulators: MMA -> epilogue -> MMA
     uint32_t tmem;
     int abort_flag;
 };
@@ -108,33 +129,14 @@ __device__ __forceinline__ bool elect_one() {
     asm volatile("{.reg .pred q; elect.sync _|q, 0xFFFFFFFF; selp.u32 %0, 1, 0, q;}" : "=r"(p));
     return p != 0;
 }
-__device__ __forceinline__ void add2(float& x, float& y, uint32_t a, uint32_t b) {
-    asm("{.reg .b64 p, q; mov.b64 p, {%0, %1}; mov.b64 q, {%2, %3}; add.rn.f32x2 p, p, q; mov.b64 {%0, %1}, p;}" : "+f"(x), "+f"(y) : "r"(a), "r"(b));
-}
-// Whether the accumulator of the smaller parts is added up after tile i of the n of a piece.
-__device__ __forceinline__ bool lo_ends(uint32_t i, uint32_t n) { return i + 1 == n || i % LO_TILES == LO_TILES - 1; }
 
-// Where the column c (mod 32) of a tile's row has its bit: shifted left by c / 4 it is the highest bit of byte c % 4, and one
-// permutation turns the highest bits of two bytes into the masks of two bf16 (2.5 instructions a pair instead of 5).
-__host__ __device__ constexpr int bit_of(int c) { return 8 * (c & 3) + 7 - ((c >> 2) & 7); }
-__host__ __device__ constexpr int column_of(int bit) { return 4 * (7 - (bit & 7)) + (bit >> 3); }
+// Where the column c (mod 32) of a tile's row has its bit: shifted right by c / 4 it is the lowest bit of byte c % 4, so that a shift and
+// an AND turn a word into four bytes of zeros and ones.
+__host__ __device__ constexpr int bit_of(int c) { return 8 * (c & 3) + ((c >> 2) & 7); }
+__host__ __device__ constexpr int column_of(int bit) { return 4 * (bit & 7) + (bit >> 3); }
 
-// columns 8 j .. 8 j + 7 of a word as bf16 zeros and ones
-__device__ __forceinline__ uint4 expand8(uint32_t word, int j) {
-    uint32_t r[4];
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const uint32_t t = word << (2 * j + i);
-        asm("prmt.b32 %0, %1, 0, 0x9988;" : "=r"(r[2 * i]) : "r"(t));            // (8: the byte's highest bit eight times)
-        asm("prmt.b32 %0, %1, 0, 0xBBAA;" : "=r"(r[2 * i + 1]) : "r"(t));
-        r[2 * i] &= 0x3F803F80u;
-        r[2 * i + 1] &= 0x3F803F80u;
-    }
-    return make_uint4(r[0], r[1], r[2], r[3]);
-}
-
-// A pair's pieces on the FMA pipes, for calls in which a row of Y holds an infinity, a NaN or a number above 2^76, whose parts and sums
-// the tensor core would not keep apart (0 * infinity): the expansion warps, one per row of a piece, entries in the order of their bits.
+// A pair's pieces on the FMA pipes, for calls in which a row of Y holds an infinity, a NaN, or numbers too far apart for six digits: the
+// expansion warps, one per row of a piece, entries in the order of their bits.
 __device__ __forceinline__ void plain_pieces(const TileParams& p, int q0, int q1, int rank) {
     const int lane = threadIdx.x & 31;
     for (int i = (threadIdx.x >> 5) - EXP_WARP; i < (q1 - q0) * 128; i += EXP_WARPS) {
@@ -166,29 +168,76 @@ __device__ __forceinline__ void plain_pieces(const TileParams& p, int q0, int q1
     }
 }
 
-// A pair of CTAs (cluster of two, tcgen05 .cta_group::2) takes 256 rows, 128 each; each holds half of the columns of Y.
-// The barriers b_full, hi_empty and lo_empty that count are the leader's, whose MMA warp waits on them; the others exist in both.
-// Warps 0-7 epilogue (two per TMEM lane quarter, half of the columns each), 8-11 expansion (a thread per row of the tile),
-// 12 copies, 13 MMA issue, 14 the peer's word to the leader, 15 none (register splits go by groups of four warps).
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1) spmm_tiles_kernel(const __grid_constant__ CUtensorMap images, const TileParams p) {
+// The sums of 8 columns, digits 16 columns of the accumulator apart, from two's complement digits of base 256: exact, then rounded once.
+template <int DIGITS>
+__device__ __forceinline__ void join_digits(uint32_t taddr, const int32_t* __restrict__ shift, float (&out)[8]) {
+    uint32_t r[DIGITS][8];
+#pragma unroll
+    for (int d = 0; d < DIGITS; ++d) tc_ld8(taddr + d * GROUP, r[d]);
+    tc_wait_ld();
+    const int4 s0 = __ldcg(reinterpret_cast<const int4*>(shift)), s1 = __ldcg(reinterpret_cast<const int4*>(shift) + 1);
+    const int32_t s[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        int64_t x = (int64_t)(int32_t)r[0][i] + (int64_t)(int32_t)r[1][i] * (1 << 8) + (int64_t)(int32_t)r[2][i] * (1 << 16);
+        if (DIGITS == 4) x += (int64_t)(int32_t)r[DIGITS == 4 ? 3 : 0][i] * (1 << 24);
+        else x += ((int64_t)(int32_t)r[DIGITS > 4 ? 3 : 0][i] + (int64_t)(int32_t)r[DIGITS > 4 ? 4 : 0][i] * (1 << 8) + (int64_t)(int32_t)r[DIGITS > 4 ? 5 : 0][i] * (1 << 16)) << 24;
+        const int half = -s[i] >> 1, rest = -s[i] - half;           // (2^-shift itself may lie outside fp32)
+        out[i] = __ll2float_rn(x) * __int_as_float((half + 127) << 23) * __int_as_float((rest + 127) << 23);
+    }
+}
+
+// The accumulator of one piece and block, 16 columns at a time, through a box per warp, so that a request stores whole sectors.
+template <int DIGITS>
+__device__ __forceinline__ void store_sums(const TileParams& p, uint32_t lanes, int groups, int half, int col0, float* dst, uint8_t* box) {
+    const int lane = threadIdx.x & 31;
+    for (int g = half; g < groups; g += 2) {
+#pragma unroll
+        for (int sub = 0; sub < 2; ++sub) {
+            float x[8];
+            join_digits<DIGITS>(lanes + g * GROUP * DIGITS + sub * 8, p.ranges->shift + col0 + g * GROUP + sub * 8, x);
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+                *reinterpret_cast<float4*>(box + lane * 64 + (((sub * 2 + c) ^ ((lane >> 1) & 3)) << 4)) = make_float4(x[c * 4], x[c * 4 + 1], x[c * 4 + 2], x[c * 4 + 3]);
+        }
+        __syncwarp();
+        const int c4 = ((col0 + g * GROUP) >> 2) + (lane & 3);
+        if (c4 < p.w4) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int row = i * 8 + (lane >> 2);
+                reinterpret_cast<float4*>(dst)[row * (p.ldp >> 2) + c4] = *reinterpret_cast<const float4*>(box + row * 64 + (((lane & 3) ^ ((row >> 1) & 3)) << 4));
+            }
+        }
+        __syncwarp();
+    }
+}
+
+// A pair of CTAs (cluster of two, tcgen05 .cta_group::2) takes 256 rows, 128 each; each holds half of B.  The pair's
+// tiles once for every block of the columns of Y.
+// The barriers full and acc_empty that count are the leader's, whose MMA warp waits on them; the others exist in both.
+// Warps 0-7 epilogue (two per TMEM lane quarter, alternate groups of columns), 8-11 expansion (a thread per row of the tile),
+// 12 images, 13 bitmaps, 14 MMA issue.  The expansion has its bitmaps from shared memory: its fences and its arrivals in the leader's memory would
+// wait for loads from global memory that its threads have under way (1,230 cycles a tile).
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1) spmm_tiles_kernel(const __grid_constant__ CUtensorMap images4, const __grid_constant__ CUtensorMap images6,
+                                                                                           const TileParams p) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) Shared b;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank(), pair = cluster_id_x();
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint8_t* stages = smem + 2 * A_BYTES;
-    const uint32_t stage_bytes = (uint32_t)p.chunks * CHUNK_BYTES;
-    int q0 = p.first_piece[pair], q1 = p.first_piece[pair + 1];
+    uint8_t* bitmaps = smem + SLOTS * SLOT_BYTES;          // (a slot: the expanded tile, the image)
+    uint8_t* boxes = bitmaps + SLOTS * BITS_BYTES;
+    const int q0 = p.first_piece[pair], q1 = p.first_piece[pair + 1];
+    const int t0 = q0 < q1 ? p.pieces[q0].begin : 0, t1 = q0 < q1 ? p.pieces[q1 - 1].end : 0;      // the pair's tiles are consecutive
     if (threadIdx.x == 0) {
         b.abort_flag = 0;
-        for (int s = 0; s < STAGES_MAX; ++s) { mbar_init(&b.b_full[s], 1); mbar_init(&b.b_empty[s], 1); }
-        for (int s = 0; s < 2; ++s) { mbar_init(&b.a_full[s], rank == 0 ? EXP_WARPS + 1 : EXP_WARPS); mbar_init(&b.a_empty[s], 1); }
-        for (int s = 0; s < 2; ++s) { mbar_init(&b.hi_full[s], 1); mbar_init(&b.hi_empty[s], 2 * EPI_WARPS); }
-        mbar_init(&b.lo_full, 1); mbar_init(&b.lo_empty, 2 * EPI_WARPS);
+        for (int s = 0; s < SLOTS; ++s) { mbar_init(&b.bits_full[s], 1); mbar_init(&b.full[s], 1 + 2 * EXP_WARPS); mbar_init(&b.empty[s], 1); }
+        for (int s = 0; s < 2; ++s) { mbar_init(&b.acc_full[s], 1); mbar_init(&b.acc_empty[s], 2 * EPI_WARPS); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (warp == MMA_WARP) {              // (before the wait below: the kernel before this one, an ordinary launch, has no tensor memory)
+    if (warp == MMA_WARP) {              // (before the wait below: no kernel that this one may run beside has tensor memory)
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&b.tmem)), "r"(TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
@@ -198,164 +247,95 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1) spmm_til
     tc_fence_after();
     const uint32_t tmem = b.tmem;
     asm volatile("griddepcontrol.wait;" ::: "memory");       // the images are complete
-    const int q1_plain = q1;
-    if (*p.unsafe) q1 = q0;
-    const int t0 = q0 < q1 ? p.pieces[q0].begin : 0, t1 = q0 < q1 ? p.pieces[q1 - 1].end : 0;      // the pair's tiles are consecutive
+    const int mode = __ldcg(&p.ranges->mode);
+    const Shape sh = p.shape[mode == MODE_6 ? 1 : 0];
+    const int blocks = mode == MODE_PLAIN ? 0 : sh.blocks, n = sh.n();
+    const uint32_t image_bytes = (uint32_t)sh.image_bytes();
 
     if (warp < EPI_WARPS) {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(EPI_REGS));
         const int quarter = warp & 3, half = warp >> 2;
-        const int hw = ((p.bn + 1) / 2 + 31) & ~31;                      // columns of a half: a multiple of 32, at most 128
-        const int n0 = half * hw, chunks = n0 >= p.bn ? 0 : (min(hw, p.bn - n0) + 31) / 32;
-        const uint32_t lanes = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)n0;
-        uint8_t* const box = stages + (size_t)p.stages * stage_bytes + warp * BOX_BYTES;
-        uint32_t at = 0, lo_use = 0;            // at: tiles of the pair so far
+        uint32_t at = 0;
         bool ok = true;
-        for (int q = q0; q < q1 && ok; ++q) {
-            const HubPiece piece = p.pieces[q];
-            float sum[4][32];
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-#pragma unroll
-                for (int i = 0; i < 32; ++i) sum[k][i] = 0.0f;
-            auto add = [&](uint64_t* full, uint64_t* empty, uint32_t use, uint32_t col, uint32_t col_end) {
-                if (!warp_wait(full, use, b, p)) return false;
+        for (int blk = 0; blk < blocks && ok; ++blk)
+            for (int q = q0; q < q1; ++q, ++at) {
+                const uint32_t set = at & 1, use = at >> 1 & 1;
+                if (!warp_wait(&b.acc_full[set], use, b, p)) { ok = false; break; }
                 tc_fence_after();
-#pragma unroll 1
-                for (; col < col_end; col += (uint32_t)p.bn) {
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        if (k < chunks) {
-                            uint32_t r[32];
-                            tc_ld32(lanes + col + k * 32, r);
-                            tc_wait_ld();
-#pragma unroll
-                            for (int i = 0; i < 32; i += 2) add2(sum[k][i], sum[k][i + 1], r[i], r[i + 1]);
-                        }
-                }
+                const uint32_t lanes = tmem + ((uint32_t)(quarter * 32) << 16) + set * (uint32_t)n;
+                float* dst = p.partial + ((int64_t)q * ROWS + rank * 128 + quarter * 32) * p.ldp;
+                if (mode == MODE_4) store_sums<4>(p, lanes, sh.cols / GROUP, half, blk * sh.cols, dst, boxes + warp * BOX_BYTES);
+                else store_sums<6>(p, lanes, sh.cols / GROUP, half, blk * sh.cols, dst, boxes + warp * BOX_BYTES);
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive_cluster(mapa_shared(smem_u32(empty), 0));
-                return true;
-            };
-            const uint32_t first = at, end = at + (uint32_t)(piece.end - piece.begin);
-            for (; at < end && ok; ++at) {
-                if (lo_ends(at - first, end - first)) { ok = add(&b.lo_full, &b.lo_empty, lo_use, p.lo_col, p.lo_col + 1); lo_use ^= 1; }
-                const uint32_t slot = at & p.hi_two, set = (uint32_t)p.bn << p.hi_halves;
-                if (ok) ok = add(&b.hi_full[slot], &b.hi_empty[slot], at >> p.hi_two & 1, slot * set, slot * set + set);
+                if (lane == 0) mbar_arrive_pair(mapa_shared(smem_u32(&b.acc_empty[set]), 0));
             }
-            if (!ok) break;
-            // through a box per warp, so that a request stores whole lines (a row per lane instead: 12,000 cycles a piece)
-            float4* dst = reinterpret_cast<float4*>(p.partial + ((int64_t)q * ROWS + rank * 128 + quarter * 32) * p.ldp);
+    } else if (warp < TMA_WARP) {
+        if (mode == MODE_PLAIN) plain_pieces(p, q0, q1, (int)rank);
+        const int row = threadIdx.x - EXP_WARP * 32;
+        Ring slot;
+        for (int t = blocks * (t1 - t0); t > 0; --t, slot.next(SLOTS)) {
+            if (!warp_wait(&b.bits_full[slot.i], slot.use, b, p)) break;       // (asked for when the slot was empty)
+            const uint4 bits = *reinterpret_cast<const uint4*>(bitmaps + slot.i * BITS_BYTES + row * 16);
+            const uint32_t word[4] = {bits.x, bits.y, bits.z, bits.w};
+            uint8_t* dst = smem + slot.i * SLOT_BYTES + row * 128;
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (k < chunks) {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        *reinterpret_cast<float4*>(box + lane * 128 + ((i ^ (lane & 7)) << 4)) = make_float4(sum[k][i * 4], sum[k][i * 4 + 1], sum[k][i * 4 + 2], sum[k][i * 4 + 3]);
-                    __syncwarp();
-                    const int c4 = (n0 >> 2) + k * 8 + (lane & 7);
-                    if (c4 < p.w4) {
-#pragma unroll 2
-                        for (int i = 0; i < 8; ++i) {
-                            const int row = i * 4 + (lane >> 3);
-                            const float4 x = *reinterpret_cast<const float4*>(box + row * 128 + (((lane & 7) ^ (row & 7)) << 4));
-                            dst[row * (p.ldp >> 2) + c4] = make_float4(x.x * (1 / CUT_SCALE), x.y * (1 / CUT_SCALE), x.z * (1 / CUT_SCALE), x.w * (1 / CUT_SCALE));
-                        }
-                    }
-                    __syncwarp();
+            for (int j = 0; j < 8; ++j) {
+                const uint32_t x = word[j >> 1] >> (4 * (j & 1));
+                *reinterpret_cast<uint4*>(dst + ((j ^ (row & 7)) << 4)) = make_uint4(x & 0x01010101u, x >> 1 & 0x01010101u, x >> 2 & 0x01010101u, x >> 3 & 0x01010101u);
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive_pair(mapa_shared(smem_u32(&b.full[slot.i]), 0));
+        }
+    } else if (warp == TMA_WARP) {
+        if (lane == 0) {
+            Ring slot;
+            bool ok = true;
+            for (int blk = 0; blk < blocks && ok; ++blk)
+                for (int t = t0; t < t1; ++t, slot.next(SLOTS)) {
+                    const int row = ((blk * p.kblocks + __ldg(p.tile_cb + t)) * 2 + (int)rank) * (n / 2);
+                    if (!thread_wait(&b.empty[slot.i], slot.use ^ 1, b, p)) { ok = false; break; }
+                    if (rank == 0) mbar_expect_tx(&b.full[slot.i], 2 * image_bytes);
+                    if (!(p.drop_load && blk == 0 && t == t0))
+                        tma_load_2d_pair(smem + slot.i * SLOT_BYTES + A_BYTES, mode == MODE_4 ? &images4 : &images6, 0, row, mapa_shared(smem_u32(&b.full[slot.i]), 0));
                 }
         }
-    } else {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(OTHER_REGS));
-        if (warp < TMA_WARP) {
-            if (q1 != q1_plain) plain_pieces(p, q0, q1_plain, (int)rank);
-            const int row = threadIdx.x - EXP_WARP * 32;
-            const uint4* bits = p.bits + rank * 128 + row;
-            uint4 next[AHEAD];              // bitmaps of the tiles to come
-#pragma unroll
-            for (int i = 0; i < AHEAD; ++i) next[i] = t0 + i < t1 ? __ldg(bits + (int64_t)(t0 + i) * ROWS) : make_uint4(0, 0, 0, 0);
-            Ring buf;
+    } else if (warp == BITS_WARP) {
+        if (lane == 0) {
+            Ring slot;
             bool ok = true;
-            for (int t = t0; t < t1 && ok; t += AHEAD) {
-#pragma unroll
-                for (int i = 0; i < AHEAD; ++i) {           // (unrolled: a register that a load is under way to is not moved)
-                    if (t + i >= t1) break;
-                    if (!warp_wait(&b.a_empty[buf.i], buf.use ^ 1, b, p)) { ok = false; break; }
-                    const uint32_t word[4] = {next[i].x, next[i].y, next[i].z, next[i].w};
-                    uint8_t* dst = smem + buf.i * A_BYTES + row * 128;
-#pragma unroll
-                    for (int j = 0; j < 16; ++j)
-                        *reinterpret_cast<uint4*>(dst + (j >> 3) * (A_BYTES / 2) + (((j & 7) ^ (row & 7)) << 4)) = expand8(word[j >> 2], j & 3);
-                    if (t + i + AHEAD < t1) next[i] = __ldg(bits + (int64_t)(t + i + AHEAD) * ROWS);
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&b.a_full[buf.i]);
-                    buf.next(2);
+            for (int blk = 0; blk < blocks && ok; ++blk)
+                for (int t = t0; t < t1; ++t, slot.next(SLOTS)) {
+                    const uint4* bits = p.bits + (int64_t)t * ROWS + rank * 128;
+                    if (t + AHEAD < t1) bulk_prefetch(bits + AHEAD * ROWS, BITS_BYTES);
+                    if (!thread_wait(&b.empty[slot.i], slot.use ^ 1, b, p)) { ok = false; break; }
+                    mbar_expect_tx(&b.bits_full[slot.i], BITS_BYTES);
+                    bulk_load(bitmaps + slot.i * BITS_BYTES, bits, BITS_BYTES, &b.bits_full[slot.i]);
                 }
-            }
-        } else if (warp == TMA_WARP) {
-            if (lane == 0) {
-                Ring st;
-                bool ok = true;
-                for (int t = t0; t < t1 && ok; ++t) {
-                    const int kb = __ldg(p.tile_cb + t);
-                    for (int part = PARTS - 1; part >= 0; --part) {
-                        if (!thread_wait(&b.b_empty[st.i], st.use ^ 1, b, p)) { ok = false; break; }
-                        if (rank == 0) mbar_expect_tx(&b.b_full[st.i], 2 * stage_bytes);
-                        if (!(p.drop_load && t == t0 && part == 0))
-                            tma_load_2d_pair(stages + (size_t)st.i * stage_bytes, &images, 0, ((kb * PARTS + part) * 2 + (int)rank) * p.chunks * COLS, mapa_shared(smem_u32(&b.b_full[st.i]), 0));
-                        st.next(p.stages);
-                    }
-                }
-            }
-        } else if (warp == RELAY_WARP && rank == 1) {
-            // The peer's tiles are ready: told to the leader by a thread of its own, because an arrival in another CTA's memory waits
-            // for all of the arriving thread's loads, which the expansion has under way all the time.
-            if (lane == 0) {
-                Ring buf;
-                for (int t = t0; t < t1; ++t) {
-                    if (!thread_wait(&b.a_full[buf.i], buf.use, b, p)) break;
-                    mbar_arrive_cluster(mapa_shared(smem_u32(&b.a_full[buf.i]), 0));
-                    buf.next(2);
-                }
-            }
-        } else if (warp == MMA_WARP && rank == 0) {
-            const uint32_t idesc = make_idesc<KIND_BF16>(ROWS, p.bn, false) | (1u << 16);      // A K-major, B MN-major
-            Ring st, buf;
-            uint32_t lo_use = 0, lo_more = 0;       // lo_more: the accumulator holds some already
-            bool ok = true;
-            for (int q = q0; q < q1 && ok; ++q) {
+        }
+    } else if (warp == MMA_WARP && rank == 0) {
+        const uint32_t idesc = make_idesc_u8s8(ROWS, n);
+        Ring slot;
+        uint32_t at = 0;
+        bool ok = true;
+        for (int blk = 0; blk < blocks && ok; ++blk)
+            for (int q = q0; q < q1 && ok; ++q, ++at) {
                 const HubPiece piece = p.pieces[q];
-                for (int t = piece.begin; t < piece.end && ok; ++t) {
-                    ok = warp_wait(&b.a_full[buf.i], buf.use, b, p) && (lo_more || warp_wait(&b.lo_empty, lo_use ^ 1, b, p));
-                    const bool ends = lo_ends((uint32_t)(t - piece.begin), (uint32_t)(piece.end - piece.begin));
-                    const uint32_t k = (uint32_t)(t - t0), slot = k & p.hi_two;
-                    const uint64_t a = make_desc(smem_u32(smem + buf.i * A_BYTES), 16, 1024, 2);
-                    for (int s = 0; s < PARTS && ok; ++s) {
-                        const bool hi = s == PARTS - 1;
-                        if (!warp_wait(&b.b_full[st.i], st.use, b, p) || (hi && !warp_wait(&b.hi_empty[slot], (k >> p.hi_two & 1) ^ 1, b, p))) { ok = false; break; }
-                        tc_fence_after();
-                        const uint32_t d = tmem + (hi ? (slot * (uint32_t)p.bn) << p.hi_halves : p.lo_col), half = hi ? p.hi_halves : 0u, more = s ? 1u : lo_more;
-                        const uint64_t bd = make_desc(smem_u32(stages + (size_t)st.i * stage_bytes), CHUNK_BYTES, 1024, 2);
-                        if (elect_one()) {
+                const uint32_t set = at & 1, use = at >> 1 & 1;
+                ok = warp_wait(&b.acc_empty[set], use ^ 1, b, p);
+                for (int t = piece.begin; t < piece.end && ok; ++t, slot.next(SLOTS)) {
+                    if (!warp_wait(&b.full[slot.i], slot.use, b, p)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint64_t a = make_desc(smem_u32(smem + slot.i * SLOT_BYTES), 16, 1024, 2), bd = a + A_BYTES / 16;
+                    if (elect_one()) {
 #pragma unroll
-                            for (int j = 0; j < COLS / 16; ++j)
-                                tc_mma_pair<KIND_BF16>(d + (half & j >> 2) * (uint32_t)p.bn, a + (j >> 2) * (A_BYTES / 2 / 16) + (j & 3) * 2, bd + j * 128, idesc,
-                                                       hi ? (j & (half ? 3 : 7)) != 0 : j ? 1u : more);
-                            tc_commit_pair(&b.b_empty[st.i], 3);
-                            if (s == PARTS - 2 && ends) tc_commit_pair(&b.lo_full, 3);
-                            if (hi) tc_commit_pair(&b.a_empty[buf.i], 3);
-                            if (hi) tc_commit_pair(&b.hi_full[slot], 3);
-                        }
-                        __syncwarp();
-                        st.next(p.stages);
+                        for (int j = 0; j < COLS / 32; ++j) tc_mma_pair<KIND_I8>(tmem + set * (uint32_t)n, a + j * 2, bd + j * 2, idesc, t > piece.begin || j);
+                        tc_commit_pair(&b.empty[slot.i], 3);
+                        if (t + 1 == piece.end) tc_commit_pair(&b.acc_full[set], 3);
                     }
-                    lo_use ^= ends; lo_more = !ends;
-                    buf.next(2);
+                    __syncwarp();
                 }
             }
-        }
     }
     __syncwarp();
     if (threadIdx.x == 0 && b.abort_flag)
@@ -363,57 +343,147 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1) spmm_til
     tc_fence_before();
     __syncthreads();
     cluster_sync_all();                  // the peer is done with this CTA's shared and tensor memory
-    if (threadIdx.x == 0) {              // the flag is this call's alone: the last CTA that has read it clears it
-        __threadfence();
-        if (atomicInc(reinterpret_cast<unsigned int*>(p.unsafe) + 1, gridDim.x - 1) == gridDim.x - 1) *p.unsafe = 0;      // (back at zero itself)
-    }
     if (warp == MMA_WARP) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
     }
 }
 
-// Rows of Y of the hub columns -> images of their three bf16 parts: images[column block][part][half of the columns of Y][chunk of 64
-// columns], a chunk as the tensor core wants it in shared memory.  Eight lanes a row and chunk, eight columns each.  The product by
-// the scale is cut with its rounding error added to the last part, so the scaling itself rounds nothing.
-__global__ void __launch_bounds__(256) split_rows_kernel(int64_t n_cols, int kblocks, int chunks, int nh, int w, const int32_t* __restrict__ nodes, const float* __restrict__ scale,
-                                                         const float* __restrict__ Y, int64_t ldy, int64_t y_rows, uint8_t* __restrict__ images, int32_t* unsafe, int32_t* status) {
+// The range of every column of Y over the hub columns of the matrix, scaled as they are multiplied: what unit its numbers are cut in, and how
+// many digits the call takes.  All whole numbers, so that neither depends on the order of the blocks.  2^lanes lanes a row.
+constexpr int RANGE_THREADS = 512;
+__global__ void __launch_bounds__(RANGE_THREADS) column_range_kernel(int64_t n_cols, int w, int lanes, const int32_t* __restrict__ nodes, const float* __restrict__ scale,
+                                                           const float* __restrict__ Y, int64_t ldy, int64_t y_rows, Ranges* ranges, int32_t* status) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    const int g = (int)(i & 7), k = (int)((i >> 3) & (COLS - 1));
-    const int64_t kc = (i >> 3) / COLS, kb = kc / (2 * chunks);
-    const int chunk = (int)(kc % (2 * chunks)), half = chunk / chunks, in_half = (chunk - half * chunks) * 64 + g * 8;
-    const int c0 = in_half < nh ? half * nh + in_half : w;
-    if (kb >= kblocks) return;
-    float x[8], lost[8];
+    __shared__ uint32_t top[HUB_SLICE];
+    __shared__ int32_t sum[HUB_SLICE], count[HUB_SLICE];
+    __shared__ bool last;
+    const int tid = threadIdx.x, c0 = (tid & ((1 << lanes) - 1)) * 4;
+    if (tid < HUB_SLICE) { top[tid] = 0; sum[tid] = count[tid] = 0; }
+    __syncthreads();
+    uint32_t my_top[4] = {0, 0, 0, 0};
+    int32_t my_sum[4] = {0, 0, 0, 0}, my_count[4] = {0, 0, 0, 0};
+    if (c0 < w) {
+        constexpr int BATCH = 4;            // rows whose numbers are on their way at once
+        const int64_t step = (int64_t)gridDim.x * (RANGE_THREADS >> lanes);
+        for (int64_t h0 = (int64_t)blockIdx.x * (RANGE_THREADS >> lanes) + (tid >> lanes); h0 < n_cols; h0 += BATCH * step) {
+            float4 y[BATCH];
+            float s[BATCH];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) x[j] = lost[j] = 0.0f;
-    const int64_t h = kb * COLS + k;
-    if (h < n_cols && c0 < w) {
-        const int64_t v = __ldg(nodes + h);
-        if (index_ok(v, y_rows, status, SITE_SPMM_COL)) {
-            const float4* src = reinterpret_cast<const float4*>(Y + v * ldy + c0);
-            const float4 a = __ldg(src), c = c0 + 4 < w ? __ldg(src + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
-            const float s = __ldg(scale + h) * CUT_SCALE, y[8] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w};
-            bool bad = false;
+            for (int i = 0; i < BATCH; ++i) {
+                const int64_t h = h0 + i * step, v = h < n_cols ? __ldg(nodes + h) : -1;
+                const bool live = h < n_cols && index_ok(v, y_rows, status, SITE_SPMM_COL);
+                y[i] = live ? __ldg(reinterpret_cast<const float4*>(Y + v * ldy + c0)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                s[i] = live ? __ldg(scale + h) : 0.0f;
+            }
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if (c0 + j < w) { x[j] = y[j] * s; lost[j] = fmaf(y[j], s, -x[j]); bad |= !(fabsf(x[j]) < SAFE_MAX); }
-            if (bad) *unsafe = 1;
+            for (int i = 0; i < BATCH; ++i) {
+                const float x[4] = {y[i].x, y[i].y, y[i].z, y[i].w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const uint32_t bits = __float_as_uint(x[j] * s[i]) & 0x7FFFFFFFu;
+                    my_top[j] = max(my_top[j], bits);
+                    my_sum[j] += (int32_t)(bits >> 23);
+                    my_count[j] += x[j] != 0.0f;
+                }
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (c0 + j < w) { atomicMax(&top[c0 + j], my_top[j]); atomicAdd(&sum[c0 + j], my_sum[j]); atomicAdd(&count[c0 + j], my_count[j]); }
+    }
+    __syncthreads();
+    if (tid < w) { atomicMax(&ranges->top[tid], top[tid]); atomicAdd(&ranges->sum[tid], sum[tid]); atomicAdd(&ranges->count[tid], count[tid]); }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) last = atomicInc(&ranges->done, gridDim.x - 1) == gridDim.x - 1;      // (back at zero)
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const bool mine = tid < HUB_SLICE;
+    const uint32_t most = mine ? __ldcg(&ranges->top[tid]) : 0;
+    const int32_t all = mine ? __ldcg(&ranges->sum[tid]) : 0, many = mine ? __ldcg(&ranges->count[tid]) : 0;
+    const int spread = many ? (int)(most >> 23) - all / many : 0;
+    const int mode = __syncthreads_or(most >= 0x7F800000u || spread > SPREAD_MAX + SPREAD_MORE) ? MODE_PLAIN : __syncthreads_or(spread > SPREAD_MAX) ? MODE_6 : MODE_4;
+    if (tid == 0) ranges->mode = mode;
+    if (!mine) return;
+    ranges->top[tid] = 0; ranges->sum[tid] = ranges->count[tid] = 0;
+    // the largest number stays below 2^31 - 2^24 units (2^47 - 2^40 of six digits): its highest digit takes a carry from those below
+    const int exponent = max((int)(most >> 23), 1) - 127 + ((most & 0x7FFFFFu) >= 0x7E0000u);
+    ranges->shift[tid] = (mode == MODE_6 ? 46 : 30) - exponent;
+}
+
+// 16 rows of a column -> its 16 bytes of every digit.  The product by the scale is exact (fp64), and adding 1.5 * 2^52 leaves the whole
+// number that is nearest to it in the lowest bits; what is below half a unit is all that is lost.
+template <int DIGITS>
+__device__ __forceinline__ void cut_column(const float (&y)[16], const double* __restrict__ by, double unit, uint4 (&out)[DIGITS]) {
+    constexpr uint64_t CARRIES = DIGITS == 4 ? 0x808080ull : 0x8080808080ull;       // digits from -128 to 127
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        uint64_t t[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            t[i] = ((uint64_t)__double_as_longlong(fma((double)y[q * 4 + i] * by[q * 4 + i], unit, 6755399441055744.0)) + CARRIES) ^ CARRIES;
+#pragma unroll
+        for (int d = 0; d < DIGITS; ++d) {
+            const uint32_t pick = (uint32_t)(d & 3) | (uint32_t)(4 + (d & 3)) << 4;
+            const uint32_t r = __byte_perm(__byte_perm((uint32_t)(t[0] >> (d & 4 ? 32 : 0)), (uint32_t)(t[1] >> (d & 4 ? 32 : 0)), pick),
+                                           __byte_perm((uint32_t)(t[2] >> (d & 4 ? 32 : 0)), (uint32_t)(t[3] >> (d & 4 ? 32 : 0)), pick), 0x5410);
+            (q == 0 ? out[d].x : q == 1 ? out[d].y : q == 2 ? out[d].z : out[d].w) = r;
         }
     }
-    uint8_t* dst = images + (kb * PARTS * 2 * chunks + chunk) * (int64_t)CHUNK_BYTES + k * 128 + ((g ^ (k & 7)) << 4);
+}
+
+// Rows of Y of the hub columns -> images of their digits: images[block][column block of the matrix][half of an accumulator's columns], the
+// 128 numbers of a digit of a column consecutive, as the tensor core wants them in shared memory.  A block of threads takes 128 rows and 16
+// columns (the blocks of the same rows run side by side), a thread 16 rows of a column.
+__global__ void __launch_bounds__(128) cut_rows_kernel(int64_t n_cols, int kblocks, Shape shape4, Shape shape6, int w, const int32_t* __restrict__ nodes, const float* __restrict__ scale,
+                                                       const float* __restrict__ Y, int64_t ldy, int64_t y_rows, uint8_t* __restrict__ images, const Ranges* ranges, int32_t* status) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    __shared__ __align__(16) int32_t node[COLS];
+    __shared__ __align__(16) double by[COLS];
+    const int tid = threadIdx.x, kb = blockIdx.y;
+    {
+        const int64_t h = (int64_t)kb * COLS + tid;
+        const int64_t v = h < n_cols ? __ldg(nodes + h) : -1;
+        const bool live = h < n_cols && index_ok(v, y_rows, status, SITE_SPMM_COL);
+        node[tid] = live ? (int32_t)v : -1;
+        by[tid] = live ? (double)__ldg(scale + h) : 0.0;
+    }
+    __syncthreads();
+    const int c = tid & 15, j = tid >> 4, col = (int)blockIdx.x * GROUP + c;
+    float y[16];
 #pragma unroll
-    for (int part = 0; part < PARTS; ++part) {
-        uint32_t r[4];
+    for (int q = 0; q < 4; ++q) {
+        const int4 v4 = *reinterpret_cast<const int4*>(node + j * 16 + q * 4);
+        const int v[4] = {v4.x, v4.y, v4.z, v4.w};
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            r[j] = pack_bf16(x[2 * j], x[2 * j + 1]);
-            x[2 * j] -= __uint_as_float(r[j] << 16);
-            x[2 * j + 1] -= __uint_as_float(r[j] & 0xFFFF0000u);
-            if (part == 1) { x[2 * j] += lost[2 * j]; x[2 * j + 1] += lost[2 * j + 1]; }
-        }
-        *reinterpret_cast<uint4*>(dst + (int64_t)part * 2 * chunks * CHUNK_BYTES) = make_uint4(r[0], r[1], r[2], r[3]);
+        for (int i = 0; i < 4; ++i) y[q * 4 + i] = v[i] >= 0 && col < w ? __ldg(Y + (int64_t)v[i] * ldy + col) : 0.0f;
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");       // the ranges are complete (Y was before them)
+    const int mode = __ldcg(&ranges->mode);
+    const double unit = col < w ? __hiloint2double((__ldcg(&ranges->shift[col < w ? col : 0]) + 1023) << 20, 0) : 0.0;
+    const Shape sh = mode == MODE_6 ? shape6 : shape4;
+    const int groups = sh.cols / GROUP, blk = (int)blockIdx.x / groups, g = (int)blockIdx.x % groups;
+    if (mode == MODE_PLAIN || blk >= sh.blocks) return;
+    const int64_t image = (int64_t)sh.image_bytes();
+    uint8_t* base = images + ((int64_t)blk * kblocks + kb) * 2 * image;
+    auto store = [&](int d, const uint4& x) {
+        int row = (g * sh.digits + d) * GROUP + c;
+        const int rank = row >= sh.n() / 2;
+        row -= rank * (sh.n() / 2);
+        *reinterpret_cast<uint4*>(base + rank * image + row * 128 + ((j ^ (row & 7)) << 4)) = x;
+    };
+    if (mode == MODE_4) {
+        uint4 out[4];
+        cut_column<4>(y, by + j * 16, unit, out);
+#pragma unroll
+        for (int d = 0; d < 4; ++d) store(d, out[d]);
+    } else {
+        uint4 out[6];
+        cut_column<6>(y, by + j * 16, unit, out);
+#pragma unroll
+        for (int d = 0; d < 6; ++d) store(d, out[d]);
     }
 }
 
@@ -446,16 +516,39 @@ __global__ void __launch_bounds__(TPB) tile_count_kernel(int cbs, const int32_t*
         if (hist[i]) atomicAdd(&cnt[(r / ROWS) * cbs + i], hist[i]);
 }
 
-__global__ void tile_select_kernel(int total, int cbs, int least, const int32_t* __restrict__ cnt, int32_t* __restrict__ flag, HubTotals* totals) {
-    const int i = blockIdx.x * TPB + threadIdx.x;
-    if (i > total) return;
-    const bool on = i < total && cnt[i] >= least;
-    flag[i] = on ? 1 : 0;              // one more than there are tiles: the scan's last element is their number
-    if (!on) return;
-    atomicAdd(&totals->entries, (unsigned long long)cnt[i]);
-    atomicAdd(&totals->tiles, 1);
-    atomicMax(&totals->last_row_block, i / cbs);
-    atomicMax(&totals->last_col_block, i % cbs);
+// The tiles that pay are those of `least` entries and more, in rows and columns of tiles where what they hold beyond that is worth a row's
+// piece and the cutting of a column's rows of Y.  By rows first (a block per row) ...
+__global__ void __launch_bounds__(TPB) tile_rows_kernel(int cbs, int least, int worth, const int32_t* __restrict__ cnt, int32_t* __restrict__ flag) {
+    const int32_t* mine = cnt + (int64_t)blockIdx.x * cbs;
+    __shared__ int32_t gain;
+    if (threadIdx.x == 0) gain = 0;
+    __syncthreads();
+    int sum = 0;
+    for (int i = threadIdx.x; i < cbs; i += TPB) sum += max(mine[i] - least, 0);
+    if (sum) atomicAdd(&gain, sum);
+    __syncthreads();
+    for (int i = threadIdx.x; i < cbs; i += TPB) flag[(int64_t)blockIdx.x * cbs + i] = gain >= worth && mine[i] >= least ? 1 : 0;
+}
+// ... then by columns
+__global__ void __launch_bounds__(TPB) tile_cols_kernel(int rbs, int cbs, int least, int worth, const int32_t* __restrict__ cnt, int32_t* __restrict__ flag, HubTotals* totals) {
+    const int cb = blockIdx.x;
+    __shared__ int32_t gain;
+    if (threadIdx.x == 0) gain = 0;
+    __syncthreads();
+    int sum = 0;
+    for (int i = threadIdx.x; i < rbs; i += TPB)
+        if (flag[i * cbs + cb]) sum += cnt[i * cbs + cb] - least;
+    if (sum) atomicAdd(&gain, sum);
+    __syncthreads();
+    for (int i = threadIdx.x; i < rbs; i += TPB) {
+        if (!flag[i * cbs + cb]) continue;
+        if (gain < worth) { flag[i * cbs + cb] = 0; continue; }
+        atomicAdd(&totals->entries, (unsigned long long)cnt[i * cbs + cb]);
+        atomicAdd(&totals->tiles, 1);
+        atomicMax(&totals->last_row_block, i);
+        atomicMax(&totals->last_col_block, cb);
+    }
+    if (cb == 0 && threadIdx.x == 0) flag[rbs * cbs] = 0;        // one more than there are tiles: the scan's last element is their number
 }
 
 __global__ void tile_index_kernel(int total, int cbs, const int32_t* __restrict__ flag, const int32_t* __restrict__ first, int32_t* __restrict__ map, int32_t* __restrict__ tile_cb) {
@@ -548,20 +641,15 @@ __global__ void hub_scale_kernel(int64_t count, int norm, int by_degree, const i
     scale[i] = norm == 0 ? dinv[u] : (norm == 1 && by_degree) ? (deg[u] > 0 ? __frcp_rn((float)deg[u]) : 0.0f) : 1.0f;
 }
 
-// CTA pairs of the product that run at once; none if it does not have the registers that its split hands out (an increase beyond the
-// launch's registers would wait for ever)
+// CTA pairs of the product that run at once
 mixgcn_status resident_pairs(const mixgcn_ctx* ctx, int* pairs) {
     *pairs = 0;
-    cudaFuncAttributes fa;
-    MIXGCN_CUDA(cudaFuncGetAttributes(&fa, spmm_tiles_kernel));
-    if (fa.numRegs * THREADS < EPI_REGS * EPI_WARPS * 32 + OTHER_REGS * (THREADS - EPI_WARPS * 32)) return MIXGCN_OK;
-    const int smem = 2 * A_BYTES + STAGE_SMEM + EPI_WARPS * BOX_BYTES + 1024;
-    MIXGCN_CUDA(cudaFuncSetAttribute(spmm_tiles_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    MIXGCN_CUDA(cudaFuncSetAttribute(spmm_tiles_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TILES_SMEM));
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3((unsigned)(ctx->sm_count & ~1), 1, 1); cfg.blockDim = dim3(THREADS, 1, 1); cfg.dynamicSmemBytes = smem;
+    cfg.gridDim = dim3((unsigned)(ctx->sm_count & ~1), 1, 1); cfg.blockDim = dim3(THREADS, 1, 1); cfg.dynamicSmemBytes = TILES_SMEM;
     cfg.attrs = attr; cfg.numAttrs = 1;
     MIXGCN_CUDA(cudaOccupancyMaxActiveClusters(pairs, spmm_tiles_kernel, &cfg));
     return MIXGCN_OK;
@@ -601,7 +689,8 @@ mixgcn_status build_tiles(const mixgcn_graph* g, bool transposed, int32_t n_widt
     MIXGCN_CUDA(cudaMemsetAsync(totals.p, 0, sizeof(HubTotals), s));
     rank_kernel<<<blocks_for(n), TPB, 0, s>>>(n, hubs, 0x7FFFFFFF, At.full.perm, rank.as<int32_t>());
     tile_count_kernel<<<(unsigned)hubs, TPB, 0, s>>>(cbs, A.full.perm, A.rowptr, A.col, rank.as<int32_t>(), cnt.as<int32_t>());
-    tile_select_kernel<<<blocks_for(total + 1), TPB, 0, s>>>(total, cbs, HUB_TILE_MIN, cnt.as<int32_t>(), flag.as<int32_t>(), totals.as<HubTotals>());
+    tile_rows_kernel<<<(unsigned)rbs, TPB, 0, s>>>(cbs, HUB_TILE_MIN, PIECE_COST * HUB_TILE_MIN, cnt.as<int32_t>(), flag.as<int32_t>());
+    tile_cols_kernel<<<(unsigned)cbs, TPB, 0, s>>>(rbs, cbs, HUB_TILE_MIN, COLUMN_COST, cnt.as<int32_t>(), flag.as<int32_t>(), totals.as<HubTotals>());
     size_t tb = 0;
     MIXGCN_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tb, flag.as<int32_t>(), first.as<int32_t>(), total + 1, s));
     MIXGCN_TRY(take(&tmp.p, (int64_t)tb));
@@ -617,7 +706,7 @@ mixgcn_status build_tiles(const mixgcn_graph* g, bool transposed, int32_t n_widt
     t->n_cols = (int64_t)t->kblocks * COLS < n ? (int64_t)t->kblocks * COLS : n;
     const int64_t covered = (int64_t)t->row_blocks * ROWS, rows = covered < n ? covered : n;
     t->nodes = At.full.perm;
-    // every pair of CTAs takes as many consecutive tiles as any other; a piece ends where a row of tiles does
+    // every pair of CTAs takes consecutive tiles, as many as any other where a piece counts as PIECE_COST tiles; a piece ends where a row of tiles does
     int clusters = 0;
     MIXGCN_TRY(resident_pairs(g->ctx, &clusters));
     if (clusters < 1) return MIXGCN_OK;
@@ -629,15 +718,17 @@ mixgcn_status build_tiles(const mixgcn_graph* g, bool transposed, int32_t n_widt
     if (*other_widths) return MIXGCN_OK;
     std::vector<HubPiece> pieces;
     std::vector<int32_t> first_piece(clusters + 1), piece_first(t->row_blocks + 1, 0);
-    int rb = 0;
+    int rb = 0, at = 0, rows_of_tiles = 0;
+    for (int i = 0; i < t->row_blocks; ++i) rows_of_tiles += host_first[(i + 1) * cbs] > host_first[i * cbs];
+    const int64_t cost = t->n_tiles + (int64_t)PIECE_COST * (rows_of_tiles + clusters - 1);       // each pair but the first continues a row, or nearly
     for (int c = 0; c < clusters; ++c) {
         first_piece[c] = (int32_t)pieces.size();
-        const int end = (int)((int64_t)t->n_tiles * (c + 1) / clusters);
-        for (int at = (int)((int64_t)t->n_tiles * c / clusters); at < end;) {
+        const int64_t end = c + 1 < clusters ? cost * (c + 1) / clusters : cost + t->n_tiles;
+        while (at < t->n_tiles) {
+            const int64_t room = end - (at + (int64_t)PIECE_COST * ((int64_t)pieces.size() + 1));
+            if (room <= 0) break;
             while (host_first[(rb + 1) * cbs] <= at) ++rb;
-            const int row_end = host_first[(rb + 1) * cbs];
-            int stop = row_end < end ? row_end : end;
-            if (stop > at + PIECE_MAX) stop = at + PIECE_MAX;
+            const int row_end = host_first[(rb + 1) * cbs], stop = row_end - at <= room ? row_end : at + (int)room;
             pieces.push_back(HubPiece{at, stop});
             piece_first[rb + 1]++;
             at = stop;
@@ -697,40 +788,41 @@ void release_tiles(mixgcn_graph* g) {
 
 // Whether an aggregation of w columns is faster with the tiles, by what both sides take (us): what the gathers of the tiles' entries would
 // take, against the product, the cut and what the other entries take longer in their own kernels (add_batch; nanoseconds an
-// entry, steps where the lane split changes).  A pair's first 32 tiles are dearer: graphs with few tiles have them spread over many rows and
-// columns, and the images come from DRAM.  Fitted to the profiles of eleven graphs; taken from a 32nd of the call on, where the fit
-// is right about the sign but for 100 K nodes at 48 columns (178 : 181).  Measured without : with (us), mean degree last, entries in tiles in brackets:
-//   R-MAT 233 K, 500 (74 %)    256 columns 5036 : 2494, 132 4542 : 1711, 128 3205 : 1359, 64 1907 : 1002, 32 1284 : 835
-//   R-MAT 2.4 M, 52 (28 %)     256 7846 : 7629, 132 6107 : 5168, 128 4401 : 3926, 48 2766 : 2202
-//   R-MAT 300 K, 31 (34 %)     192 466 : 443, 132 459 : 412;  100 K, 106 (61 %)  256 521 : 430, 128 334 : 253, 64 206 : 188
-//   R-MAT 20 K, 300 (83 %)     256 276 : 165, 64 113 : 87;  8 K of 500 K nodes joined at random (51 %)  256 1907 : 1617, 64 586 : 525
-// and left to the gather kernels: R-MAT 300 K, 31  256 550 : 552, 128 313 : 303, 64 205 : 218;  700 K, 22 (28 %)  256 1002 : 1072,
-// 132 789 : 810, 128 527 : 581;  1.5 M, 21 (23 %)  256 2193 : 2331, 132 1721 : 1711;  ends drawn by rank^-0.6, 300 K, 100 (4 %)  256 2142 : 2396,
-// 128 1022 : 1164, by rank^-0.8, 1 M, 40 (11 %)  256 3315 : 3754, 132 2362 : 2309.
+// entry, steps where the lane split changes).  Fitted to eighteen graphs at fourteen widths; taken from a 16th of the call on, where the fit is
+// right about the sign (a GIN layer's aggregations over 150 K nodes of mean degree 20, within a 32nd, took 2 % longer with them).  Measured
+// without : with (us), mean degree last, entries in tiles in brackets:
+//   R-MAT 233 K, 500 (75 %)    256 columns 5035 : 2012, 132 4549 : 1404, 128 3212 : 1050, 64 1908 : 623, 41 1725 : 600
+//   R-MAT 2.4 M, 52 (38 %)     256 7808 : 6938, 132 6159 : 4450, 64 2862 : 2188
+//   R-MAT 300 K, 100 (62 %)    256 1471 : 1030, 132 970 : 514;  300 K, 31 (48 %)  256 562 : 499, 132 469 : 367, 64 210 : 183
+//   R-MAT 100 K, 106 (74 %)    256 487 : 310, 132 434 : 220, 64 190 : 118;  20 K, 300 (91 %)  256 269 : 122, 132 252 : 88, 64 104 : 57
+//   R-MAT 700 K, 22 (41 %)     256 1038 : 1021, 132 823 : 744, 64 383 : 359
+//   8 K of 500 K nodes joined at random (59 %)  256 4124 : 2804, 64 1990 : 1330
+// and left to the gather kernels: R-MAT 1.5 M, 21 (35 %)  256 2481 : 2506;  6 M, 17 (22 %)  256 9497 : 9590, 128 4 % slower with tiles;  1 M, 8 (22 %)
+// 4 to 29 % slower;  50 K, 40 (66 %)  up to 64 columns 11 to 60 % slower;  ends drawn by rank^-0.8, 1 M, 40 (13 %)  256 3564 : 3956.
 bool hub_tiles_pay(const HubTiles* t, int32_t w) {
-    const double tiles = (double)t->n_tiles / t->clusters, first = tiles < 32 ? tiles : 32;      // of a pair
+    // (narrow calls over fewer than 16 M entries are short beside the launches that tiles add, and the fit is no help: 8 columns 3 to 26 % slower
+    // with less than 95 % of the entries in tiles, up to 64 columns 30 % slower to 13 % faster with less than half)
+    if (t->entries + t->rem_nnz < (int64_t)1 << 24 && ((w <= 12 && t->entries < 19 * t->rem_nnz) || (w <= 64 && t->entries < t->rem_nnz))) return false;
+    const double tiles = (double)t->n_tiles / t->clusters;      // of a pair
     double all = 0, gain = 0;
     auto slice = [&](int32_t c) {
-        const double entry = c > 192 ? 0.036 + 0.00003 * (c - 192) : c > 160 ? 0.036 : c > 128 ? 0.037 : c > 64 ? 0.026 : c > 24 ? 0.005 + 0.00016 * c : 0.0088;
-        const double other = c > 192 ? 0.0078 : c > 128 ? 0.0045 : c > 64 ? 0.004 : 0.001;
-        const double product = c > 160 ? (1.72 + 0.0076 * (c - 160)) * tiles + (2.8 + 0.0085 * (c - 160)) * first
-                                       : c > 128 ? 1.72 * tiles + 2.8 * first : c > 64 ? 1.5 * tiles + 2.3 * first : 1.45 * tiles + 1.6 * first;
+        const double entry = c > 192 ? 0.040 : c > 128 ? 0.0365 : c > 96 ? 0.0285 : c > 64 ? 0.0235 : 0.0028 + 0.0002 * (c > 8 ? c : 8);
+        const double other = c > 192 ? 0.0086 : c > 128 ? 0.0035 : c > 96 ? 0.0061 : c > 64 ? 0.0016 : c > 48 ? 0.0024 : 0.0008;
+        const Shape sh = make_shape(4, c);
+        const double product = sh.blocks * (0.30 * tiles * (sh.cols > 40 ? sh.cols : 40) / 64 + 3.0);
         all += entry * 1e-3 * (t->entries + t->rem_nnz);
-        gain += entry * 1e-3 * t->entries - other * 1e-3 * t->rem_nnz - product - 10.0 - 2e-6 * t->n_cols * c;
+        gain += entry * 1e-3 * t->entries - other * 1e-3 * t->rem_nnz - product - 12.0 - 3.2e-6 * t->n_cols * c;
     };
     for (int32_t c0 = 0; c0 < w; c0 += HUB_SLICE) slice(w - c0 < HUB_SLICE ? w - c0 : HUB_SLICE);
-    return gain * 32 > all;
+    return gain * 16 > all;
 }
-
-// columns of a half of Y, chunks of 64 of them
-inline int half_cols(int32_t w) { return (w + 31) / 32 * 16; }
-inline int half_chunks(int32_t w) { return (half_cols(w) + 63) / 64; }
 
 int64_t hub_tiles_scratch(const HubTiles* t, int32_t w, int64_t ldp, int64_t* images_at) {
     const int64_t partial = (int64_t)t->n_pieces * ROWS * ldp * (int64_t)sizeof(float);
     *images_at = (partial + 1023) & ~(int64_t)1023;
     if (w > HUB_SLICE) w = HUB_SLICE;
-    return *images_at + (int64_t)t->kblocks * PARTS * 2 * half_chunks(w) * CHUNK_BYTES;
+    const Shape s4 = make_shape(4, w), s6 = make_shape(6, w);
+    return *images_at + (int64_t)t->kblocks * 2 * std::max(s4.blocks * s4.image_bytes(), s6.blocks * s6.image_bytes());
 }
 
 mixgcn_status launch_hub_tiles(mixgcn_ctx* ctx, const HubTiles* t, int phase, int32_t w, const float* Y, int64_t ldy, int64_t y_rows, float* partial, int64_t ldp,
@@ -738,36 +830,34 @@ mixgcn_status launch_hub_tiles(mixgcn_ctx* ctx, const HubTiles* t, int phase, in
     TileParams p{};
     p.pieces = t->pieces; p.first_piece = t->first_piece; p.tile_cb = t->tile_cb; p.bits = reinterpret_cast<const uint4*>(t->bits);
     p.partial = partial; p.ldp = ldp;
-    p.w4 = (w + 3) >> 2; p.bn = half_cols(w) * 2; p.chunks = half_chunks(w);
-    const int fit = STAGE_SMEM / (p.chunks * CHUNK_BYTES);
-    p.stages = fit < STAGES_MAX ? fit : STAGES_MAX;
-    p.hi_two = p.bn * 3 <= (int)TMEM_COLS ? 1 : 0;
-    p.hi_halves = p.bn * 5 <= (int)TMEM_COLS ? 1 : 0;
-    p.lo_col = (uint32_t)p.bn << (p.hi_two + p.hi_halves);
-    p.unsafe = ctx->d_status + TILES_UNSAFE_WORD;
+    p.w4 = (w + 3) >> 2; p.kblocks = t->kblocks;
+    p.shape[0] = make_shape(4, w); p.shape[1] = make_shape(6, w);
+    Ranges* ranges = reinterpret_cast<Ranges*>(ctx->d_status + TILES_WORD);
+    p.ranges = ranges;
     p.Y = Y; p.ldy = ldy; p.y_rows = y_rows; p.nodes = t->nodes; p.col_scale = t->col_scale; p.n_cols = t->n_cols;
     p.status = ctx->d_status;
     p.wait_limit = ctx->debug_wait_limit > 0 ? (uint32_t)ctx->debug_wait_limit : WAIT_LIMIT_DEFAULT;
     p.drop_load = ctx->debug_drop_load;
-    CUtensorMap map;
-    const int64_t image_rows = (int64_t)t->kblocks * PARTS * 2 * p.chunks * COLS;
-    if (!encode_2d(&map, images, 2, 64, image_rows, 64, 64, p.chunks * COLS, CU_TENSOR_MAP_SWIZZLE_NONE)) MIXGCN_FAIL(MIXGCN_ECUDA, "spmm: no tensor map for the images of the hub rows");
-    {
-        LaunchScope scope(ctx, phase, s);
-        const int64_t threads = (int64_t)t->kblocks * COLS * 2 * p.chunks * 8;
-        split_rows_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(t->n_cols, t->kblocks, p.chunks, p.bn / 2, w, t->nodes, t->col_scale, Y, ldy, y_rows, images, p.unsafe,
-                                                                            ctx->d_status);
+    CUtensorMap map[2];
+    for (int m = 0; m < 2; ++m) {
+        const Shape& sh = p.shape[m];
+        if (!encode_2d(&map[m], images, 2, 64, (int64_t)sh.blocks * t->kblocks * sh.n(), 64, 64, sh.n() / 2, CU_TENSOR_MAP_SWIZZLE_NONE))
+            MIXGCN_FAIL(MIXGCN_ECUDA, "spmm: no tensor map for the images of the hub rows");
     }
-    const size_t smem = 2 * A_BYTES + (size_t)p.stages * p.chunks * CHUNK_BYTES + EPI_WARPS * BOX_BYTES + 1024;
-    MIXGCN_CUDA(cudaFuncSetAttribute(spmm_tiles_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    {
+        LaunchScope scope(ctx, phase, s, 2);
+        int lanes = 0;
+        while ((4 << lanes) < w) ++lanes;
+        const int64_t rows = RANGE_THREADS >> lanes, most = 2 * (int64_t)ctx->sm_count, blocks = (t->n_cols + rows * 4 - 1) / (rows * 4);
+        column_range_kernel<<<(unsigned)(blocks < most ? blocks : most), RANGE_THREADS, 0, s>>>(t->n_cols, w, lanes, t->nodes, t->col_scale, Y, ldy, y_rows, ranges, ctx->d_status);
+        const int groups = std::max(p.shape[0].blocks * p.shape[0].cols, p.shape[1].blocks * p.shape[1].cols) / GROUP;
+        launch_chained(cut_rows_kernel, dim3((unsigned)groups, (unsigned)t->kblocks), 128, 0, s, t->n_cols, t->kblocks, p.shape[0], p.shape[1], w, t->nodes, t->col_scale, Y, ldy, y_rows,
+                       images, ranges, ctx->d_status);
+    }
+    MIXGCN_CUDA(cudaFuncSetAttribute(spmm_tiles_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TILES_SMEM));
     LaunchScope scope(ctx, phase, s);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)t->clusters * 2, 1, 1); cfg.blockDim = dim3(THREADS, 1, 1); cfg.dynamicSmemBytes = smem; cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // it sets up beside the kernel before
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    MIXGCN_CUDA(cudaLaunchKernelEx(&cfg, spmm_tiles_kernel, map, p));
+    launch_chained(spmm_tiles_kernel, dim3((unsigned)t->clusters * 2), THREADS, TILES_SMEM, s, map[0], map[1], p);      // it sets up beside the kernel before
+    MIXGCN_CUDA(cudaGetLastError());
     return MIXGCN_OK;
 }
 

@@ -6,7 +6,7 @@ namespace mixgcn {
 
 constexpr int HUB_ROWS = 256, HUB_COLS = 128;   // a tile
 constexpr int HUB_SLICE = 256;                  // most columns of one product
-constexpr int HUB_TILE_MIN = 1200;              // entries from which a tile pays: 43 ns to gather them (256 columns), 33 for the tile (2.45 us on one of 74 pairs)
+constexpr int HUB_TILE_MIN = 500;               // entries from which a tile pays: 20 ns to gather them (256 columns), 18 for the tile (1.34 us on one of 74 pairs)
 constexpr int64_t HUB_MIN_ENTRIES = 1 << 20;    // graphs below this, and tiles that hold less than a quarter of it, are not worth the launches
 struct HubPiece { int32_t begin, end; };       // tiles [begin, end) of one row of tiles
 

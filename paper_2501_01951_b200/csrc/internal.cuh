@@ -80,12 +80,12 @@ inline void memory_given_back(const MemoryGeneration& m) { if (m) m->fetch_add(1
 
 }  // namespace mixgcn
 
-constexpr int STATUS_WORDS = 32, SPLIT_OVERFLOW_WORD = 16, TILES_UNSAFE_WORD = 17;    // (two words: flag, count)
+constexpr int STATUS_WORDS = 2048, SPLIT_OVERFLOW_WORD = 16, TILES_WORD = 32;    // (words from TILES_WORD on: Ranges in hub_tiles.cu)
 
 struct mixgcn_ctx {
     int device;
     int sm_count;
-    int32_t* d_status;        // device status word (int32[4]); words SPLIT_OVERFLOW_WORD, TILES_UNSAFE_WORD: see gemm_split.cu, hub_tiles.cu
+    int32_t* d_status;        // device status word (int32[4]); words SPLIT_OVERFLOW_WORD, TILES_WORD: see gemm_split.cu, hub_tiles.cu
     void* workspace;          // grow-on-demand scratch of the dense products, column sums and the loss
     int64_t workspace_bytes;
     void* workspace_rows;     // scratch of the row-sparse backward (row list, positions, compact operands)

@@ -149,6 +149,21 @@ def test_numbers_of_every_size(mg, ctx, graphs):
     assert torch.equal(Z[:, :3].double(), want[:, :3])
 
 
+@pytest.mark.parametrize("w", [1, 16, 33, 65, 100, 256, 300])
+@pytest.mark.parametrize("binades", [6, 12, 20, 40])
+def test_numbers_far_apart(mg, ctx, graphs, w, binades):
+    """One row in fifty `binades` above the others: four digits, six, and none that would do.  A term loses half a unit at most, 2^-31 and
+    2^-47 of the largest with four and six digits: 2^-25 and 2^-27 of the others' size where they are used, far inside the bound of the sums."""
+    plain, tiled, A = graphs["none", False]
+    Y = features(w, 13)
+    Y *= torch.where(torch.rand((N, 1), generator=torch.Generator().manual_seed(w)) < 0.02, 2.0 ** binades, 1.0).cuda()
+    Z = torch.empty_like(Y)
+    mg.spmm(ctx, tiled, Y, Z, w)
+    want = A[0] @ Y[:, :w].double()
+    assert torch.all((Z[:, :w].double() - want).abs() <= 512 * 2.0 ** -24 * (A[0] @ Y[:, :w].double().abs()))
+    assert ((Z[:, :w].double() - want).norm() / want.norm()).item() < 4e-7
+
+
 def test_a_wait_that_runs_out_is_reported(mg, ctx, graphs):
     _, tiled, _ = graphs["sym", True]
     Y, Z = features(256, 3), torch.empty((N, 256), device="cuda")

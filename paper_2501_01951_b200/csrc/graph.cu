@@ -1,17 +1,20 @@
 // Graph construction on the device: edge list -> A + I in CSR -> symmetric normalisation
 // A_hat = D^-1/2 (A+I) D^-1/2 (Section 2.1 of the paper) -> CSR of the transpose (aliased when
-// symmetric) -> degree-sorted row schedule.  Sorting, run-length and selection steps use CUB
-// device primitives; everything else is a kernel in this file.
+// symmetric) -> degree-sorted row schedule.  Lists of up to ten million entries become a CSR in graph_buckets.cu; sorting, run-length
+// and selection steps of larger ones, and the schedule's sort and scans, use CUB device primitives; everything else is a kernel in this file.
 //
 // What a build costs beside its kernels is memory and waiting: every temporary comes from the library's pool, the host
 // waits twice (for the entry count, then for the schedule's counts), keys carry no more bits than the ids have
 // (a radix pass over the keys costs as much as any other kernel here), and what the flags already say about the
-// structure is not looked up.  250 K nodes, 4.2 M entries: 9.0 ms and more -> 0.6 ms.
+// structure is not looked up.  The schedule looks the column blocks of a long row up once, keeps them for the segments, and orders those by
+// 4,096 ranges of first columns (250 K nodes, 4.7 M entries: seg_count_kernel 46 -> 28 us, seg_fill_kernel 47 -> 13, the order 45 -> 9).
+// Builds of that list: 9.0 ms and more -> 0.68 -> 0.42 ms.
 #include <cub/cub.cuh>
 
 #include <atomic>
 #include <new>
 
+#include "graph_values.cuh"
 #include "internal.cuh"
 
 using namespace mixgcn;
@@ -70,14 +73,7 @@ __global__ void degree_kernel(int64_t n, const int64_t* __restrict__ rowptr, int
     if (u >= n) return;
     int32_t d = (int32_t)(rowptr[u + 1] - rowptr[u]);
     deg[u] = d;
-    // dinv = 1/sqrt(deg): IEEE square root, then IEEE reciprocal, each rounded to fp32.
-    dinv[u] = d > 0 ? __frcp_rn(__fsqrt_rn((float)d)) : 0.0f;
-}
-
-// Value of an entry of row u.  norm 0: dinv_u * dinv_v (Section 2.1); 1: 1 / (entries in row u), the row mean (GraphSAGE's
-// mean aggregator; IEEE reciprocal); 2: 1, the plain sum (GIN's sum aggregator).
-__device__ __forceinline__ float entry_value(int norm, float dinv_u, float dinv_v, int32_t deg_u) {
-    return norm == 0 ? __fmul_rn(dinv_u, dinv_v) : norm == 1 ? __frcp_rn((float)deg_u) : 1.0f;
+    dinv[u] = degree_norm(d);
 }
 
 // One warp per row.
@@ -163,7 +159,7 @@ __global__ void schedule_keys_kernel(int64_t row0, int64_t n_rows, uint32_t top,
 
 // What the host has to know of a schedule, counted on the device (integers, so the order of the atomics does not matter).
 struct ScheduleCounts {
-    unsigned long long rows_above_seg, rows_above[3], rows_heavy, total_segs, max_deg;
+    unsigned long long rows_above_seg, rows_above[3], rows_heavy, total_segs, max_deg, bounds;
 };
 
 // Row counts of the buckets (one atomic per warp and counter).
@@ -196,71 +192,91 @@ __device__ __forceinline__ int64_t lower_bound_col(const int32_t* __restrict__ c
     return lo;
 }
 
-// The column blocks of one long row, a warp per row, 32 blocks at a time: f(block's first entry, its end, segments it
-// takes, segments of the row's blocks before it).  Returns the row's number of segments.
-template <typename F>
-__device__ __forceinline__ int64_t row_blocks(int64_t n_cols, int64_t rb, int64_t re, const int32_t* __restrict__ col, int seg, F f) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nb = (int64_t)1 << row_log_blocks(re - rb, schedule_blk_min(n_cols)), width = (n_cols + nb - 1) / nb;
-    int64_t before = 0;
-    for (int64_t b0 = 0; b0 < nb; b0 += 32) {
-        const int64_t b = b0 + lane;
-        int64_t lo = re, hi = re;
-        if (b < nb) {
-            lo = lower_bound_col(col, rb, re, b * width);
-            hi = lower_bound_col(col, lo, re, (b + 1) * width);
-        }
-        const int64_t mine = (hi - lo + seg - 1) / seg;
-        int64_t incl = mine;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int64_t t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-            if (lane >= o) incl += t;
-        }
-        f(lo, hi, before + incl - mine);
-        before += __shfl_sync(0xFFFFFFFFu, incl, 31);
-    }
-    return before;
-}
-
-// row_segs[i] = segments of the i-th longest row, 0 for rows that are not cut; i <= cap (a bound of the number of long rows)
-__global__ void seg_count_kernel(int64_t n_cols, int64_t cap, const int32_t* __restrict__ perm, const int64_t* __restrict__ rowptr,
-                                 const int32_t* __restrict__ col, int seg, int64_t* __restrict__ row_segs, ScheduleCounts* counts) {
+// Long rows: the number of segments of the i-th longest row (0 for rows that are not cut; i <= cap, a bound of the number of long rows), a warp
+// per row, 32 column blocks at a time.  The first entry of every block is kept for seg_fill_kernel, the row's at bounds[bound_at[i]].
+__global__ void seg_count_kernel(int64_t n_cols, int64_t cap, const int32_t* __restrict__ perm, const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col, int seg,
+                                 int64_t* __restrict__ row_segs, int32_t* __restrict__ bounds, int32_t* __restrict__ bound_at, ScheduleCounts* counts) {
     const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
     if (i > cap) return;
-    int64_t k = 0;
-    if (i < cap) {
-        const int64_t u = perm[i], rb = rowptr[u], re = rowptr[u + 1];
-        if (re - rb > seg) k = row_blocks(n_cols, rb, re, col, seg, [](int64_t, int64_t, int64_t) {});
+    int64_t segs = 0;
+    const int64_t rb = i < cap ? rowptr[perm[i]] : 0, re = i < cap ? rowptr[perm[i] + 1] : 0;
+    if (re - rb > seg) {
+        const int nb = 1 << row_log_blocks(re - rb, schedule_blk_min(n_cols));
+        const int64_t width = (n_cols + nb - 1) / nb;
+        int at = 0;
+        if (lane == 0) bound_at[i] = at = (int)atomicAdd(&counts->bounds, (unsigned long long)nb);
+        at = __shfl_sync(0xFFFFFFFFu, at, 0);
+        int64_t before = re;                   // of the blocks so far: where the last one begins
+        for (int b0 = nb - 32 < 0 ? 0 : nb - 32;; b0 -= 32) {        // from the last ones on, so that every block knows where the next one begins
+            const int b = b0 + lane;
+            const int64_t lo = b < nb ? lower_bound_col(col, rb, re, b * width) : re;
+            if (b < nb) bounds[at + b] = (int32_t)(lo - rb);
+            const int64_t next = __shfl_down_sync(0xFFFFFFFFu, lo, 1), hi = lane == 31 ? before : next;
+            segs += (hi - lo + seg - 1) / seg;
+            before = __shfl_sync(0xFFFFFFFFu, lo, 0);
+            if (b0 == 0) break;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) segs += __shfl_xor_sync(0xFFFFFFFFu, segs, o);
     }
-    if ((threadIdx.x & 31) == 0) {
-        row_segs[i] = k;
-        if (k) atomicAdd(&counts->total_segs, (unsigned long long)k);
+    if (lane == 0) {
+        row_segs[i] = segs;
+        if (segs) atomicAdd(&counts->total_segs, (unsigned long long)segs);
     }
 }
 
-__global__ void seg_fill_kernel(int64_t n_cols, int64_t n_long, const int32_t* __restrict__ perm, const int64_t* __restrict__ rowptr,
-                                const int32_t* __restrict__ col, int seg, const int64_t* __restrict__ seg_off,
-                                SpmmRec* __restrict__ rec_tmp, uint32_t* __restrict__ keys, uint32_t* __restrict__ ids) {
+// Segments run in order of their first columns, as far as SEG_BINS ranges of columns tell them apart: their order decides what the L2 holds, not
+// what is added up.
+constexpr int SEG_BINS = 4096;
+__device__ __forceinline__ int seg_bin(int64_t n_cols, int32_t c) { return (int)((int64_t)c * SEG_BINS / n_cols); }
+
+__global__ void seg_fill_kernel(int64_t n_cols, int64_t n_long, const int32_t* __restrict__ perm, const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col, int seg,
+                                const int64_t* __restrict__ seg_off, const int32_t* __restrict__ bounds, const int32_t* __restrict__ bound_at,
+                                SpmmRec* __restrict__ rec_tmp, int32_t* __restrict__ bin_of, uint32_t* __restrict__ bins) {
     const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (i >= n_long) return;
-    const int64_t u = perm[i], first = seg_off[i];
-    row_blocks(n_cols, rowptr[u], rowptr[u + 1], col, seg, [&](int64_t lo, int64_t hi, int64_t before) {
-        int64_t q = first + before;
+    const int lane = threadIdx.x & 31;
+    const int64_t u = perm[i], rb = rowptr[u], re = rowptr[u + 1];
+    const int nb = 1 << row_log_blocks(re - rb, schedule_blk_min(n_cols));
+    const int32_t* mine = bounds + bound_at[i];
+    int64_t q0 = seg_off[i];
+    for (int b0 = 0; b0 < nb; b0 += 32) {
+        const int b = b0 + lane;
+        const int64_t lo = b < nb ? rb + mine[b] : re, hi = b + 1 < nb ? rb + mine[b + 1] : re;
+        const int segs = (int)((hi - lo + seg - 1) / seg);
+        int incl = segs;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        int64_t q = q0 + incl - segs;
         for (int64_t pos = lo; pos < hi; pos += seg, ++q) {
             SpmmRec x; x.begin = pos; x.len = (int32_t)((hi - pos) < seg ? (hi - pos) : seg); x.row = (int32_t)i;
             rec_tmp[q] = x;
-            keys[q] = (uint32_t)col[pos];      // segments run in order of their first column
-            ids[q] = (uint32_t)q;
+            const int bin = seg_bin(n_cols, col[pos]);
+            bin_of[q] = bin;
+            atomicAdd(&bins[bin], 1u);
         }
-    });
+        q0 += __shfl_sync(0xFFFFFFFFu, incl, 31);
+    }
 }
 
-__global__ void seg_place_kernel(int64_t total_segs, const uint32_t* __restrict__ order, const SpmmRec* __restrict__ rec_tmp,
+__global__ void __launch_bounds__(SEG_BINS / 4) seg_bins_kernel(uint32_t* __restrict__ bins) {      // counts -> first positions
+    using Scan = cub::BlockScan<uint32_t, SEG_BINS / 4>;
+    __shared__ typename Scan::TempStorage temp;
+    uint4 c = reinterpret_cast<uint4*>(bins)[threadIdx.x];
+    uint32_t x[4] = {c.x, c.y, c.z, c.w};
+    Scan(temp).ExclusiveSum(x, x);
+    reinterpret_cast<uint4*>(bins)[threadIdx.x] = make_uint4(x[0], x[1], x[2], x[3]);
+}
+
+__global__ void seg_place_kernel(int64_t total_segs, const int32_t* __restrict__ bin_of, const SpmmRec* __restrict__ rec_tmp, uint32_t* __restrict__ bins,
                                  SpmmRec* __restrict__ rec, int64_t* __restrict__ seg_pos) {
-    int64_t pos = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (pos >= total_segs) return;
-    const uint32_t q = order[pos];
+    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= total_segs) return;
+    const uint32_t pos = atomicAdd(&bins[bin_of[q]], 1u);
     rec[pos] = rec_tmp[q];
     seg_pos[q] = pos;
 }
@@ -317,12 +333,15 @@ mixgcn_status build_schedule(int64_t n_total, int64_t nnz, const int64_t* rowptr
     const uint32_t top = (uint32_t)(((uint64_t)1 << deg_bits) - 1);
     int64_t cap = nnz / (v.seg + 1);                                       // no more rows than this are long
     if (cap > n) cap = n;
-    DevBuf k0(s), k1(s), ids(s), tmp(s), counts(s), row_segs(s);
+    DevBuf k0(s), k1(s), ids(s), tmp(s), counts(s), row_segs(s), bounds(s), bound_at(s);
     MIXGCN_TRY(k0.alloc(n * (int64_t)sizeof(uint32_t)));
     MIXGCN_TRY(k1.alloc(n * (int64_t)sizeof(uint32_t)));
     MIXGCN_TRY(ids.alloc(n * (int64_t)sizeof(int32_t)));
     MIXGCN_TRY(counts.alloc(sizeof(ScheduleCounts)));
     MIXGCN_TRY(row_segs.alloc((cap + 1) * (int64_t)sizeof(int64_t)));
+    // (a long row has a block per blk_min of its entries at most, or one)
+    MIXGCN_TRY(bounds.alloc((nnz / schedule_blk_min(n_total) + cap) * (int64_t)sizeof(int32_t)));
+    MIXGCN_TRY(bound_at.alloc(cap * (int64_t)sizeof(int32_t)));
     MIXGCN_TRY(dev_alloc((void**)&v.perm, n * (int64_t)sizeof(int32_t), s));
     MIXGCN_CUDA(cudaMemsetAsync(counts.p, 0, sizeof(ScheduleCounts), s));
     schedule_keys_kernel<<<blocks_for(n), TPB, 0, s>>>(row0, n, top, rowptr, k0.as<uint32_t>(), ids.as<int32_t>());
@@ -332,7 +351,8 @@ mixgcn_status build_schedule(int64_t n_total, int64_t nnz, const int64_t* rowptr
     MIXGCN_CUDA(cub::DeviceRadixSort::SortPairs(tmp.p, tb, k0.as<uint32_t>(), k1.as<uint32_t>(), ids.as<int32_t>(), v.perm, n, 0, deg_bits, s));
     schedule_counts_kernel<<<blocks_for(n), TPB, 0, s>>>(n, top, k1.as<uint32_t>(), v.seg, counts.as<ScheduleCounts>());
     if (cap > 0)
-        seg_count_kernel<<<blocks_for((cap + 1) * 32), TPB, 0, s>>>(n_total, cap, v.perm, rowptr, col, v.seg, row_segs.as<int64_t>(), counts.as<ScheduleCounts>());
+        seg_count_kernel<<<blocks_for((cap + 1) * 32), TPB, 0, s>>>(n_total, cap, v.perm, rowptr, col, v.seg, row_segs.as<int64_t>(), bounds.as<int32_t>(), bound_at.as<int32_t>(),
+                                                                        counts.as<ScheduleCounts>());
     ScheduleCounts h{};
     MIXGCN_CUDA(cudaMemcpyAsync(&h, counts.p, sizeof(h), cudaMemcpyDeviceToHost, s));
     MIXGCN_CUDA(cudaStreamSynchronize(s));
@@ -348,25 +368,19 @@ mixgcn_status build_schedule(int64_t n_total, int64_t nnz, const int64_t* rowptr
     MIXGCN_TRY(dev_alloc((void**)&v.seg_pos, (total + 1) * (int64_t)sizeof(int64_t), s));
     if (total > 0) {
         // segments of the long rows, in order of their first column
-        DevBuf rec_tmp(s), keys0(s), keys1(s), ids0(s), ids1(s), tmp2(s);
+        DevBuf rec_tmp(s), bin_of(s), bins(s), tmp2(s);
         MIXGCN_TRY(rec_tmp.alloc(total * (int64_t)sizeof(SpmmRec)));
-        MIXGCN_TRY(keys0.alloc(total * (int64_t)sizeof(uint32_t)));
-        MIXGCN_TRY(keys1.alloc(total * (int64_t)sizeof(uint32_t)));
-        MIXGCN_TRY(ids0.alloc(total * (int64_t)sizeof(uint32_t)));
-        MIXGCN_TRY(ids1.alloc(total * (int64_t)sizeof(uint32_t)));
-        const int col_bits = bits_for((uint64_t)n_total);
-        size_t tb_scan = 0, tb_sort = 0;
+        MIXGCN_TRY(bin_of.alloc(total * (int64_t)sizeof(int32_t)));
+        MIXGCN_TRY(bins.alloc(SEG_BINS * sizeof(uint32_t)));
+        MIXGCN_CUDA(cudaMemsetAsync(bins.p, 0, SEG_BINS * sizeof(uint32_t), s));
+        size_t tb_scan = 0;
         MIXGCN_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tb_scan, row_segs.as<int64_t>(), v.seg_off, nl + 1, s));
-        MIXGCN_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, tb_sort, keys0.as<uint32_t>(), keys1.as<uint32_t>(), ids0.as<uint32_t>(),
-                                                    ids1.as<uint32_t>(), total, 0, col_bits, s));
-        size_t tb2 = tb_scan > tb_sort ? tb_scan : tb_sort;
-        MIXGCN_TRY(tmp2.alloc((int64_t)tb2));
-        MIXGCN_CUDA(cub::DeviceScan::ExclusiveSum(tmp2.p, tb2, row_segs.as<int64_t>(), v.seg_off, nl + 1, s));
-        seg_fill_kernel<<<blocks_for(nl * 32), TPB, 0, s>>>(n_total, nl, v.perm, rowptr, col, v.seg, v.seg_off, rec_tmp.as<SpmmRec>(),
-                                                           keys0.as<uint32_t>(), ids0.as<uint32_t>());
-        MIXGCN_CUDA(cub::DeviceRadixSort::SortPairs(tmp2.p, tb2, keys0.as<uint32_t>(), keys1.as<uint32_t>(), ids0.as<uint32_t>(),
-                                                    ids1.as<uint32_t>(), total, 0, col_bits, s));
-        seg_place_kernel<<<blocks_for(total), TPB, 0, s>>>(total, ids1.as<uint32_t>(), rec_tmp.as<SpmmRec>(), v.rec, v.seg_pos);
+        MIXGCN_TRY(tmp2.alloc((int64_t)tb_scan));
+        MIXGCN_CUDA(cub::DeviceScan::ExclusiveSum(tmp2.p, tb_scan, row_segs.as<int64_t>(), v.seg_off, nl + 1, s));
+        seg_fill_kernel<<<blocks_for(nl * 32), TPB, 0, s>>>(n_total, nl, v.perm, rowptr, col, v.seg, v.seg_off, bounds.as<int32_t>(), bound_at.as<int32_t>(),
+                                                           rec_tmp.as<SpmmRec>(), bin_of.as<int32_t>(), bins.as<uint32_t>());
+        seg_bins_kernel<<<1, SEG_BINS / 4, 0, s>>>(bins.as<uint32_t>());
+        seg_place_kernel<<<blocks_for(total), TPB, 0, s>>>(total, bin_of.as<int32_t>(), rec_tmp.as<SpmmRec>(), bins.as<uint32_t>(), v.rec, v.seg_pos);
     } else {
         MIXGCN_CUDA(cudaMemsetAsync(v.seg_off, 0, (nl + 1) * sizeof(int64_t), s));
     }
@@ -377,8 +391,8 @@ mixgcn_status build_schedule(int64_t n_total, int64_t nnz, const int64_t* rowptr
 
 // Degrees and room for the values of a graph whose rowptr exists.
 mixgcn_status fill_degrees(mixgcn_graph* g, cudaStream_t s) {
-    MIXGCN_TRY(dev_alloc((void**)&g->deg, g->n * (int64_t)sizeof(int32_t), s));
-    MIXGCN_TRY(dev_alloc((void**)&g->dinv, g->n * (int64_t)sizeof(float), s));
+    if (!g->deg) MIXGCN_TRY(dev_alloc((void**)&g->deg, g->n * (int64_t)sizeof(int32_t), s));
+    if (!g->dinv) MIXGCN_TRY(dev_alloc((void**)&g->dinv, g->n * (int64_t)sizeof(float), s));
     MIXGCN_TRY(dev_alloc((void**)&g->fwd.val, (g->nnz > 0 ? g->nnz : 1) * (int64_t)sizeof(float), s));
     degree_kernel<<<blocks_for(g->n), TPB, 0, s>>>(g->n, g->fwd.rowptr, g->deg, g->dinv);
     return MIXGCN_OK;
@@ -457,7 +471,7 @@ mixgcn_status csr_from_edges(mixgcn_graph* g, int64_t m, const int32_t* src, con
     if (h.flags & F_BAD_ID) MIXGCN_FAIL(MIXGCN_EBADGRAPH, "graph_create: a node id lies outside [0, %lld)", (long long)n);
     const int64_t nnz = total == 0 ? 0 : h.unique - ((h.flags & F_DROPPED) ? 1 : 0);     // dropped edges left one sentinel, the last key
     g->nnz = nnz;
-    MIXGCN_TRY(dev_alloc((void**)&g->fwd.rowptr, (n + 1) * (int64_t)sizeof(int64_t), s));
+    if (!g->fwd.rowptr) MIXGCN_TRY(dev_alloc((void**)&g->fwd.rowptr, (n + 1) * (int64_t)sizeof(int64_t), s));
     MIXGCN_TRY(dev_alloc((void**)&g->fwd.col, (nnz > 0 ? nnz : 1) * (int64_t)sizeof(int32_t), s));
     rowptr_from_keys_kernel<Key><<<blocks_for(nnz + 1), TPB, 0, s>>>(n, nnz, shift, k0.as<Key>(), g->fwd.rowptr, g->fwd.col);
     MIXGCN_TRY(fill_degrees(g, s));
@@ -554,8 +568,11 @@ extern "C" mixgcn_status mixgcn_graph_create(mixgcn_ctx* ctx, int64_t n, int64_t
         MIXGCN_CUDA(cudaMemcpyAsync(ddst.p, dst, m * sizeof(int32_t), cudaMemcpyHostToDevice, s));
         ps = dsrc.as<int32_t>(); pd = ddst.as<int32_t>();
     }
+    bool built = false;
+    MIXGCN_TRY(csr_from_buckets(g, m, ps, pd, sym, self, s, &built));
     // two ids fit one 32-bit key on graphs of fewer than 2^16 nodes: half the bytes per radix pass
-    if (2 * bits_for((uint64_t)n) <= 32) MIXGCN_TRY(csr_from_edges<uint32_t>(g, m, ps, pd, sym, self, s));
+    if (built) {}
+    else if (2 * bits_for((uint64_t)n) <= 32) MIXGCN_TRY(csr_from_edges<uint32_t>(g, m, ps, pd, sym, self, s));
     else MIXGCN_TRY(csr_from_edges<uint64_t>(g, m, ps, pd, sym, self, s));
     dsrc.release(); ddst.release();
     // self loops of the input are dropped, so the flags decide what lies on the diagonal; a directed list may still be symmetric

@@ -776,7 +776,7 @@ __global__ void __launch_bounds__(KK_THREADS, 1) gemm_tc_pair_kernel(const __gri
             // this warp is done reading the buffer: tell the leader's MMA issuer
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(mapa_shared(smem_u32(&acc_empty[buf]), 0));
+            if (lane == 0) mbar_arrive_pair(mapa_shared(smem_u32(&acc_empty[buf]), 0));
         }
         if (tma_store && lane == 0) bulk_wait_all();
     }

@@ -788,8 +788,8 @@ void release_tiles(mixgcn_graph* g) {
 
 // Whether an aggregation of w columns is faster with the tiles, by what both sides take (us): what the gathers of the tiles' entries would
 // take, against the product, the cut and what the other entries take longer in their own kernels (add_batch; nanoseconds an
-// entry, steps where the lane split changes).  Fitted to eighteen graphs at fourteen widths; taken from a 16th of the call on, where the fit is
-// right about the sign (a GIN layer's aggregations over 150 K nodes of mean degree 20, within a 32nd, took 2 % longer with them).  Measured
+// entry, steps where the lane split changes).  Fitted to eighteen graphs at fourteen widths; taken from a 16th of the call on, an 8th below 16 M
+// entries, where the fit is right about the sign (a GIN layer's aggregations over 150 K nodes of mean degree 20 took 2 % longer to 1 % less).  Measured
 // without : with (us), mean degree last, entries in tiles in brackets:
 //   R-MAT 233 K, 500 (75 %)    256 columns 5035 : 2012, 132 4549 : 1404, 128 3212 : 1050, 64 1908 : 623, 41 1725 : 600
 //   R-MAT 2.4 M, 52 (38 %)     256 7808 : 6938, 132 6159 : 4450, 64 2862 : 2188
@@ -802,7 +802,8 @@ void release_tiles(mixgcn_graph* g) {
 bool hub_tiles_pay(const HubTiles* t, int32_t w) {
     // (narrow calls over fewer than 16 M entries are short beside the launches that tiles add, and the fit is no help: 8 columns 3 to 26 % slower
     // with less than 95 % of the entries in tiles, up to 64 columns 30 % slower to 13 % faster with less than half)
-    if (t->entries + t->rem_nnz < (int64_t)1 << 24 && ((w <= 12 && t->entries < 19 * t->rem_nnz) || (w <= 64 && t->entries < t->rem_nnz))) return false;
+    const bool small = t->entries + t->rem_nnz < (int64_t)1 << 24;
+    if (small && ((w <= 12 && t->entries < 19 * t->rem_nnz) || (w <= 64 && t->entries < t->rem_nnz))) return false;
     const double tiles = (double)t->n_tiles / t->clusters;      // of a pair
     double all = 0, gain = 0;
     auto slice = [&](int32_t c) {
@@ -814,7 +815,7 @@ bool hub_tiles_pay(const HubTiles* t, int32_t w) {
         gain += entry * 1e-3 * t->entries - other * 1e-3 * t->rem_nnz - product - 12.0 - 3.2e-6 * t->n_cols * c;
     };
     for (int32_t c0 = 0; c0 < w; c0 += HUB_SLICE) slice(w - c0 < HUB_SLICE ? w - c0 : HUB_SLICE);
-    return gain * 16 > all;
+    return gain * (small ? 8 : 16) > all;
 }
 
 int64_t hub_tiles_scratch(const HubTiles* t, int32_t w, int64_t ldp, int64_t* images_at) {

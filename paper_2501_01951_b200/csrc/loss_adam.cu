@@ -134,13 +134,13 @@ __global__ void __launch_bounds__(LOSS_WARPS * 32) loss_rows_kernel(
         for (int c = lane; c < C; c += 32) s += expf(row[c] - mx);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-        const float lse = mx + logf(s);
+        const float lse = mx + logf(s), share = 1.0f / s;
         const float py = row[y];
         if (lane == 0) { local += (double)(lse - py); if (arg == y) ++correct; }
         __syncwarp();  // dlogits may alias logits: every read of the row precedes the writes
         if (dlogits)
             for (int c = lane; c < C; c += 32) {
-                const float g = (expf(row[c] - lse) - (c == y ? 1.0f : 0.0f)) * invT;
+                const float g = (expf(row[c] - mx) * share - (c == y ? 1.0f : 0.0f)) * invT;
                 dlogits[v * ld + c] = g;
             }
     }
@@ -154,11 +154,11 @@ __global__ void __launch_bounds__(LOSS_WARPS * 32) loss_rows_kernel(
     }
 }
 
-// Same computation for C <= 4 * LPR * VPL with the row held in registers: LPR lanes take a row (32 / LPR rows a warp), one
-// float4-vectorised read of the logits, one float4 write of the gradient (requires ld % 4 == 0 and 16-byte aligned pointers).
-// The next rows' logits, mask bytes and labels are requested before the current ones are reduced.  Bound: instructions (the arg-max's
-// shuffles; with a warp for every row, whatever its width, twice to three times as many: rows of 47 with a pitch of 52, 30 % in the
-// mask, 400 K 115 -> 80 us; rows of 20, 1 M 209 -> 75).
+// Same computation for C <= 4 * LPR * VPL with the row held in registers: LPR lanes take a row (32 / LPR rows a warp), VPL
+// float4-vectorised reads of the logits and writes of the gradient a lane (requires ld % 4 == 0 and 16-byte aligned pointers).
+// The next rows' logits, mask bytes and labels are requested before the current ones are reduced.  Bound: instructions, so lanes are few and
+// their columns many (a row's shuffles serve 32 / LPR rows at once), the arg-max is looked up behind the maximum, and the exponentials of
+// the sum, over the sum, are the gradient's (as exp(x - log-sum-exp), with twice as many: 400 K x 47, 30 % in the mask, 71 us, now 47).
 template <int LPR, int VPL>
 __global__ void __launch_bounds__(LOSS_WARPS * 32) loss_rows_vec_kernel(
     int64_t n, int C, const float* logits, int64_t ld, const int32_t* __restrict__ labels,
@@ -166,7 +166,6 @@ __global__ void __launch_bounds__(LOSS_WARPS * 32) loss_rows_vec_kernel(
     int32_t* __restrict__ pred, unsigned long long* n_correct, double* __restrict__ part, int32_t* status, bool zero_rows) {
     chain_begin();
     constexpr int ROWS = 32 / LPR;
-    constexpr bool AHEAD = LPR < 32;       // (a label for every row costs more than it hides where a warp takes one: 309 -> 335 us at 1 M x 172)
     __shared__ double sm[LOSS_WARPS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lig = lane % LPR, sub = lane / LPR;
     const unsigned long long T = *count;
@@ -184,7 +183,7 @@ __global__ void __launch_bounds__(LOSS_WARPS * 32) loss_rows_vec_kernel(
             const int g = lig + LPR * q;
             nxt[q] = (v < n && g < C4) ? row4[g] : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
         }
-        if (AHEAD && v < n) { nxt_mask = mask[v]; nxt_y = labels[v]; }
+        if (v < n) { nxt_mask = mask[v]; nxt_y = labels[v]; }
     };
     int64_t v0 = ((int64_t)blockIdx.x * LOSS_WARPS + warp) * ROWS;
     load_row(v0 + sub);
@@ -199,24 +198,26 @@ __global__ void __launch_bounds__(LOSS_WARPS * 32) loss_rows_vec_kernel(
 #pragma unroll
             for (int e = 0; e < 4; ++e) if (g * 4 + e >= C) x[q][e] = -INFINITY;   // pad columns are not data
         }
-        const bool train = in && (AHEAD ? nxt_mask : mask[v]) != 0 && T != 0;
-        const int y = AHEAD ? nxt_y : train ? labels[v] : 0;
+        const bool train = in && nxt_mask != 0 && T != 0;
+        const int y = nxt_y;
         load_row(v + stride);
-        float mx = -INFINITY; int arg = 0x7FFFFFFF;
+        float mx = -INFINITY;
 #pragma unroll
-        for (int q = 0; q < VPL; ++q)
+        for (int q = 0; q < VPL; ++q) mx = fmaxf(mx, fmaxf(fmaxf(x[q][0], x[q][1]), fmaxf(x[q][2], x[q][3])));      // (no NaN among them)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
+        for (int o = LPR / 2; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
+        // the lowest column that attains it
+        int arg = 0x7FFFFFFF;
+#pragma unroll
+        for (int q = VPL - 1; q >= 0; --q)
+#pragma unroll
+            for (int e = 3; e >= 0; --e) {
                 const int c = (lig + LPR * q) * 4 + e;
-                if (c < C && (x[q][e] > mx || (x[q][e] == mx && c < arg))) { mx = x[q][e]; arg = c; }
+                if (x[q][e] == mx && c < C) arg = c;
             }
-        if (arg == 0x7FFFFFFF) arg = lig * 4 < C ? lig * 4 : 0;
 #pragma unroll
-        for (int o = LPR / 2; o > 0; o >>= 1) {
-            const float omx = __shfl_xor_sync(0xFFFFFFFFu, mx, o);
-            const int oarg = __shfl_xor_sync(0xFFFFFFFFu, arg, o);
-            if (omx > mx || (omx == mx && oarg < arg)) { mx = omx; arg = oarg; }
-        }
+        for (int o = LPR / 2; o > 0; o >>= 1) arg = min(arg, __shfl_xor_sync(0xFFFFFFFFu, arg, o));
+        if (arg == 0x7FFFFFFF) arg = 0;                            // NaN everywhere
         if (pred && in && lig == 0) pred[v] = arg;
         const bool ok = train && y >= 0 && y < C;
         if (train && !ok && lig == 0) atomicMax(status, DEV_BAD_LABEL);
@@ -229,33 +230,29 @@ __global__ void __launch_bounds__(LOSS_WARPS * 32) loss_rows_vec_kernel(
             continue;
         }
         float s = 0.0f, py = 0.0f;
-#pragma unroll
-        for (int q = 0; q < VPL; ++q)
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-                if ((lig + LPR * q) * 4 + e < C) s += expf(x[q][e] - mx);
-#pragma unroll
-        for (int o = LPR / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-        const float lse = mx + logf(s);
         // the label's logit lives in lane (y/4) % LPR of the row, slot (y/4) / LPR, element y % 4
 #pragma unroll
         for (int q = 0; q < VPL; ++q)
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
-                if ((lig + LPR * q) * 4 + e == y) py = x[q][e];
+            for (int e = 0; e < 4; ++e) {
+                const int c = (lig + LPR * q) * 4 + e;
+                if (c == y) py = x[q][e];
+                x[q][e] = c < C ? expf(x[q][e] - mx) : 0.0f;
+                s += x[q][e];
+            }
+#pragma unroll
+        for (int o = LPR / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
         py = __shfl_sync(0xFFFFFFFFu, py, (y >> 2) & (LPR - 1), LPR);
-        if (ok && lig == 0) { local += (double)(lse - py); if (arg == y) ++correct; }
+        if (ok && lig == 0) { local += (double)(mx + logf(s) - py); if (arg == y) ++correct; }
         if (!dlogits || !in || !(ok || zero_rows || train)) continue;
+        const float share = 1.0f / s;
 #pragma unroll
         for (int q = 0; q < VPL; ++q) {
             const int g = lig + LPR * q;
             if (g < C4) {
                 float r[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int c = g * 4 + e;
-                    r[e] = ok && c < C ? (expf(x[q][e] - lse) - (c == y ? 1.0f : 0.0f)) * invT : 0.0f;
-                }
+                for (int e = 0; e < 4; ++e) r[e] = ok && g * 4 + e < C ? (x[q][e] * share - (g * 4 + e == y ? 1.0f : 0.0f)) * invT : 0.0f;
                 reinterpret_cast<float4*>(dlogits + v * ld)[g] = make_float4(r[0], r[1], r[2], r[3]);
             }
         }
@@ -323,12 +320,12 @@ __global__ void __launch_bounds__(LOSS_WARPS * 32) loss_rows_subset_kernel(
             for (int c = lane; c < C; c += 32) s += expf(row[c] - mx);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-            const float lse = mx + logf(s);
+            const float lse = mx + logf(s), share = 1.0f / s;
             const float py = row[y];
             if (lane == 0) { local += (double)(lse - py); if (arg == y) ++correct; }
             __syncwarp();  // dlogits may alias logits: every read of the row precedes the writes
             if (dlogits)
-                for (int c = lane; c < C; c += 32) dlogits[v * ld + c] = (expf(row[c] - lse) - (c == y ? 1.0f : 0.0f)) * invT;
+                for (int c = lane; c < C; c += 32) dlogits[v * ld + c] = (expf(row[c] - mx) * share - (c == y ? 1.0f : 0.0f)) * invT;
             __syncwarp();
         }
     }
@@ -342,225 +339,33 @@ __global__ void __launch_bounds__(LOSS_WARPS * 32) loss_rows_subset_kernel(
     }
 }
 
-// ---- rows staged through shared memory, four lanes per row ------------------------------------
-// For C up to a few hundred the warp-per-row kernels spend more issue slots on shuffles than on data.
-// Here a CTA takes tiles of ROWS consecutive rows: a tile is one contiguous piece of memory
-// (ROWS x ld floats), fetched by a single bulk-async copy into shared memory while the previous tile
-// is being worked on (two buffers).  Four adjacent lanes own a row, a quarter of its columns each,
-// walked from a lane-dependent starting point so that a warp's 32 lanes spread over the banks; the
-// arg-max keeps the lowest index among equal maxima explicitly, so the order does not matter.  The few
-// train rows are then finished by whole warps (exponentials and gradient stores over 32 lanes).
-constexpr uint32_t LOSS_WAIT_LIMIT = 1u << 22;
-constexpr int LOSS_TILE_KB = 72;     // shared memory a CTA of the tile kernel takes at most (two tile buffers)
-constexpr int LOSS_LANES_PER_ROW = 4;
-
-__device__ __forceinline__ uint32_t loss_smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ bool loss_mbar_wait(uint64_t* bar, uint32_t parity) {
-    for (uint32_t it = 0; it < LOSS_WAIT_LIMIT; ++it) {
-        uint32_t ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok) : "r"(loss_smem_u32(bar)), "r"(parity) : "memory");
-        if (ok) return true;
-    }
-    return false;
-}
-
-template <int ROWS>
-__global__ void __launch_bounds__(ROWS * LOSS_LANES_PER_ROW) loss_rows_tile_kernel(
-    int64_t n, int C, const float* logits, int64_t ld, const int32_t* __restrict__ labels,
-    const uint8_t* __restrict__ mask, const unsigned long long* __restrict__ count, float* dlogits,
-    int32_t* __restrict__ pred, unsigned long long* n_correct, double* __restrict__ part, int32_t* status,
-    bool zero_rows, int64_t n_tiles) {
-    chain_begin();
-    constexpr int THREADS = ROWS * LOSS_LANES_PER_ROW;
-    extern __shared__ __align__(128) unsigned char loss_smem[];
-    float* const tile0 = reinterpret_cast<float*>(loss_smem);
-    float* const tile1 = tile0 + (int64_t)ROWS * ld;
-    __shared__ __align__(8) uint64_t bar[2];
-    __shared__ double red[THREADS / 32];
-    __shared__ uint8_t keep_row[2][ROWS];      // rows of the tile whose gradient row was written as a train row
-    __shared__ int expired;
-    const int tid = threadIdx.x, lane = tid & 31;
-    const int r_own = tid / LOSS_LANES_PER_ROW, q = tid % LOSS_LANES_PER_ROW;
-    const unsigned long long T = *count;
-    const float invT = T ? (float)(1.0 / (double)T) : 0.0f;
-    const int ld4 = (int)(ld >> 2);
-    const int seg = (C + LOSS_LANES_PER_ROW - 1) / LOSS_LANES_PER_ROW;
-    const int c_lo = q * seg < C ? q * seg : C, c_hi = (q + 1) * seg < C ? (q + 1) * seg : C;
-    if (tid == 0) {
-        expired = 0;
-        for (int b = 0; b < 2; ++b)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(loss_smem_u32(&bar[b])), "r"(1u) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
-    __syncthreads();
-    auto issue = [&](int64_t t, int b) {
-        const int64_t row0 = t * ROWS;
-        const int64_t rows = (n - row0) < ROWS ? (n - row0) : ROWS;
-        const uint32_t bytes = (uint32_t)(rows * ld * (int64_t)sizeof(float));    // a multiple of 16: ld % 4 == 0
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(loss_smem_u32(&bar[b])), "r"(bytes) : "memory");
-        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                     ::"r"(loss_smem_u32(b ? tile1 : tile0)), "l"(reinterpret_cast<uint64_t>(logits + row0 * ld)), "r"(bytes),
-                       "r"(loss_smem_u32(&bar[b])) : "memory");
-    };
-    double local = 0.0;
-    unsigned int correct = 0;
-    uint32_t phase0 = 0u, phase1 = 0u;       // parity to wait for on each buffer's barrier
-    int buf = 0;
-    int64_t t = blockIdx.x;
-    if (tid == 0 && t < n_tiles) issue(t, 0);                       // the first tile; later ones are requested one iteration ahead
-    for (; t < n_tiles; t += gridDim.x, buf ^= 1) {
-        const int64_t row0 = t * ROWS, v = row0 + r_own;
-        // mask byte and label of this thread's row, requested before the wait so that their latency is hidden
-        uint8_t my_mask = 0; int my_y = 0;
-        if (v < n && q == 0) { my_mask = mask[v]; my_y = labels[v]; }
-        if (!loss_mbar_wait(&bar[buf], buf ? phase1 : phase0)) expired = 1;       // bounded: give up instead of hanging
-        if (buf) phase1 ^= 1u; else phase0 ^= 1u;
-        __syncthreads();               // this tile has landed; every thread is done with the previous tile
-        if (expired) {
-            if (tid == 0) atomicMax(status, DEV_WAIT_EXPIRED);         // no other copy is in flight at this point
-            break;
-        }
-        // refill the other buffer (the previous tile's) while this one is worked on
-        if (tid == 0 && t + gridDim.x < n_tiles) issue(t + gridDim.x, buf ^ 1);
-        const int rows = (int)((n - row0) < ROWS ? (n - row0) : ROWS);
-        const float* tile = buf ? tile1 : tile0;
-        const float* row = tile + (int64_t)r_own * ld;
-        float mx = -INFINITY; int arg = 0x7FFFFFFF;
-        if (v < n && c_hi > c_lo) {
-            // two independent (max, index) chains over [start, c_hi) then [c_lo, start): plain counted
-            // loops so that the shared-memory loads are issued ahead of the compares
-            const int start = c_lo + lane % (c_hi - c_lo);
-            float mx2 = -INFINITY; int arg2 = 0x7FFFFFFF;
-            auto scan = [&](int c0, int c1) {
-                int c = c0;
-#pragma unroll 4
-                for (; c + 1 < c1; c += 2) {
-                    const float x = row[c], x2 = row[c + 1];
-                    if (x > mx || (x == mx && c < arg)) { mx = x; arg = c; }
-                    if (x2 > mx2 || (x2 == mx2 && c + 1 < arg2)) { mx2 = x2; arg2 = c + 1; }
-                }
-                if (c < c1) { const float x = row[c]; if (x > mx || (x == mx && c < arg)) { mx = x; arg = c; } }
-            };
-            scan(start, c_hi);
-            scan(c_lo, start);
-            if (mx2 > mx || (mx2 == mx && arg2 < arg)) { mx = mx2; arg = arg2; }
-        }
-        // the four lanes of a row agree on its maximum and the lowest index that attains it
-#pragma unroll
-        for (int o = 1; o < LOSS_LANES_PER_ROW; o <<= 1) {
-            const float omx = __shfl_xor_sync(0xFFFFFFFFu, mx, o);
-            const int oarg = __shfl_xor_sync(0xFFFFFFFFu, arg, o);
-            if (omx > mx || (omx == mx && oarg < arg)) { mx = omx; arg = oarg; }
-        }
-        if (arg == 0x7FFFFFFF) arg = 0;                                // every entry NaN
-        const bool wrote = v < n && q == 0 && my_mask != 0 && T != 0;
-        if (v < n && q == 0 && pred) pred[v] = arg;
-        if (dlogits && zero_rows) {
-            if (q == 0) keep_row[buf][r_own] = wrote ? 1 : 0;
-            __syncthreads();           // keep_row is complete
-            // zero gradient rows of the other nodes, written by the whole CTA in memory order
-            float4* out4 = reinterpret_cast<float4*>(dlogits + row0 * ld);
-            const int total4 = rows * ld4;
-            for (int i = tid; i < total4; i += THREADS) {
-                const int r = i / ld4;
-                if (!keep_row[buf][r]) out4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-        }
-        // train rows (few): the whole warp works on each of them in turn -- lanes stride over the columns
-        unsigned live = __ballot_sync(0xFFFFFFFFu, wrote);
-        while (live) {
-            const int src = __ffs(live) - 1;
-            live &= live - 1;
-            const float r_mx = __shfl_sync(0xFFFFFFFFu, mx, src);
-            const int r_arg = __shfl_sync(0xFFFFFFFFu, arg, src);
-            const int y = __shfl_sync(0xFFFFFFFFu, my_y, src);
-            const int r = ((tid & ~31) + src) / LOSS_LANES_PER_ROW;
-            const float* rr = tile + (int64_t)r * ld;
-            float* out = dlogits ? dlogits + (row0 + r) * ld : nullptr;
-            if (y < 0 || y >= C) {
-                if (lane == 0) atomicMax(status, DEV_BAD_LABEL);
-                if (out) for (int j = lane; j < C; j += 32) out[j] = 0.0f;
-                continue;
-            }
-            float sum = 0.0f;
-            for (int j = lane; j < C; j += 32) sum += expf(rr[j] - r_mx);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
-            const float lse = r_mx + logf(sum);
-            if (lane == 0) { local += (double)(lse - rr[y]); if (r_arg == y) ++correct; }
-            if (out) for (int j = lane; j < C; j += 32) out[j] = (expf(rr[j] - lse) - (j == y ? 1.0f : 0.0f)) * invT;
-        }
-    }
-    // fixed-order block sum of the per-warp losses
-    for (int o = 16; o > 0; o >>= 1) local += __shfl_down_sync(0xFFFFFFFFu, local, o);
-    for (int o = 16; o > 0; o >>= 1) correct += __shfl_down_sync(0xFFFFFFFFu, correct, o);
-    if (lane == 0) red[tid >> 5] = local;
-    if (n_correct && lane == 0 && correct) atomicAdd(n_correct, (unsigned long long)correct);
-    __syncthreads();
-    if (tid == 0) {
-        double s = 0.0;
-        for (int w = 0; w < THREADS / 32; ++w) s += red[w];
-        part[blockIdx.x] = s;
-    }
-}
-
-template <int ROWS>
-cudaError_t launch_loss_tile(int grid, size_t smem, cudaStream_t s, int64_t n, int C, const float* logits, int64_t ld,
-                             const int32_t* labels, const uint8_t* mask, const unsigned long long* count, float* dlogits,
-                             int32_t* pred, unsigned long long* n_correct, double* part, int32_t* status, bool zero_rows,
-                             int64_t n_tiles) {
-    cudaError_t e = cudaFuncSetAttribute(loss_rows_tile_kernel<ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    launch_chained(loss_rows_tile_kernel<ROWS>, dim3(grid), ROWS * LOSS_LANES_PER_ROW, smem, s, n, C, logits, ld, labels, mask, count, dlogits, pred, n_correct, part,
-                                                         status, zero_rows, n_tiles);
-    return cudaGetLastError();
-}
-
-// Launches the row pass and returns how many block partials it writes to `part` (<= warp_blocks, the
-// capacity the caller sized `part` for), or -1 on a launch error.  With sm_count > 0 and a row that
-// fits, the shared-memory tile kernel (one lane per row) is used; otherwise one warp per row, with
-// the row in registers when C <= 256 and the layout allows float4 access.
-int launch_loss_rows(unsigned warp_blocks, cudaStream_t s, int64_t n, int C, const float* logits, int64_t ld,
-                     const int32_t* labels, const uint8_t* mask, const unsigned long long* count, float* dlogits,
-                     int32_t* pred, unsigned long long* n_correct, double* part, int32_t* status, bool zero_rows = true,
-                     int sm_count = 0) {
+// Launches the row pass: one partial sum a block in `part`.  False on a launch error.
+bool launch_loss_rows(unsigned blocks, cudaStream_t s, int64_t n, int C, const float* logits, int64_t ld,
+                      const int32_t* labels, const uint8_t* mask, const unsigned long long* count, float* dlogits,
+                      int32_t* pred, unsigned long long* n_correct, double* part, int32_t* status, bool zero_rows = true) {
+    // Rows in registers up to 512 columns, three or four float4 a lane; the lines lie where another float4 or twice the lanes are needed.  1 % : 8 : 30 : 60 of
+    // the rows in the mask, us, against tiles of rows that bulk copies brought to shared memory (dense rows of 33 to 288 columns, four lanes
+    // a row, train rows by whole warps; 8, 16 and 32 lanes with one float4 each for the others):
+    //   400 K x 47 41 : 44 : 47 : 48 against 54 : 64 : 87 : 112, with a pitch of 52 47 : 50 : 52 : 52 against 62 : 66 : 76 : 85
+    //   1 M x 20 54 : 64 : 73 : 73 against 67 : 79 : 95 : 103;  x 64 99 : 114 : 126 : 128 against 127 : 143 : 189 : 243
+    //   1 M x 100 159 : 179 : 224 : 239 against 159 : 196 : 286 : 394;  x 172 239 : 243 : 265 : 300 against 262 : 255 : 350 : 460
+    // (the bytes alone: 24, 26, 25, 80, 124 and 214 us.)
     const bool vec = (ld & 3) == 0 && aligned16(logits) && (!dlogits || aligned16(dlogits));
-    // Several CTAs per SM (each with two tile buffers) keep some computing while others wait for their
-    // copies: a CTA takes at most LOSS_TILE_KB of shared memory; rows per tile follow from that.
-    constexpr int64_t TILE_SMEM = LOSS_TILE_KB * 1024;
-    // The tile kernel treats a tile as one dense piece of rows x ld floats (it copies and zeroes whole
-    // rows), so it is taken only when the row holds nothing but its C columns and their pad to a multiple
-    // of 4; a wider ld (a column slice of a larger buffer) goes to the per-row kernels, which touch columns
-    // below round4(C) only.  Up to 32 columns eight lanes of the per-row kernel are as fast with few train rows and faster with many (1 M x 20:
-    // 75 and 103 us with 1 and 50 % of them against 75 and 167); above, they are slower with few (2.4 M x 47, 1 %: 311 against 234).
-    if (vec && sm_count > 0 && C > 32 && ld == ((int64_t)C + 3) / 4 * 4 && 2 * 32 * ld * 4 <= TILE_SMEM) {
-        const int rows = 2 * 128 * ld * 4 <= TILE_SMEM ? 128 : (2 * 64 * ld * 4 <= TILE_SMEM ? 64 : 32);
-        const int64_t n_tiles = (n + rows - 1) / rows;
-        int64_t per_sm = (220 * 1024) / (2 * rows * ld * 4 + 1024);
-        if (per_sm > 2048 / (rows * LOSS_LANES_PER_ROW)) per_sm = 2048 / (rows * LOSS_LANES_PER_ROW);
-        if (per_sm < 1) per_sm = 1;
-        int64_t grid = n_tiles < per_sm * sm_count ? n_tiles : per_sm * sm_count;
-        if (grid > (int64_t)warp_blocks) grid = warp_blocks;
-        const size_t smem = (size_t)(2 * rows * ld * 4);
-        cudaError_t e = rows == 128 ? launch_loss_tile<128>((int)grid, smem, s, n, C, logits, ld, labels, mask, count, dlogits, pred, n_correct, part, status, zero_rows, n_tiles)
-                      : rows == 64  ? launch_loss_tile<64>((int)grid, smem, s, n, C, logits, ld, labels, mask, count, dlogits, pred, n_correct, part, status, zero_rows, n_tiles)
-                                    : launch_loss_tile<32>((int)grid, smem, s, n, C, logits, ld, labels, mask, count, dlogits, pred, n_correct, part, status, zero_rows, n_tiles);
-        return e == cudaSuccess ? (int)grid : -1;
-    }
-    auto rows_vec = [&](auto kernel) { launch_chained(kernel, dim3(warp_blocks), LOSS_WARPS * 32, 0, s, n, C, logits, ld, labels, mask, count, dlogits, pred, n_correct, part, status, zero_rows); };
-    if (vec && C <= 32) rows_vec(loss_rows_vec_kernel<8, 1>);
-    else if (vec && C <= 64) rows_vec(loss_rows_vec_kernel<16, 1>);
-    else if (vec && C <= 128) rows_vec(loss_rows_vec_kernel<32, 1>);
-    else if (vec && C <= 256) rows_vec(loss_rows_vec_kernel<32, 2>);
+    auto rows_vec = [&](auto kernel) { launch_chained(kernel, dim3(blocks), LOSS_WARPS * 32, 0, s, n, C, logits, ld, labels, mask, count, dlogits, pred, n_correct, part, status, zero_rows); };
+    const int C4 = (C + 3) >> 2;
+    if (vec && C4 <= 4) rows_vec(loss_rows_vec_kernel<4, 1>);
+    else if (vec && C4 <= 8) rows_vec(loss_rows_vec_kernel<4, 2>);
+    else if (vec && C4 <= 12) rows_vec(loss_rows_vec_kernel<4, 3>);
+    else if (vec && C4 <= 16) rows_vec(loss_rows_vec_kernel<4, 4>);
+    else if (vec && C4 <= 24) rows_vec(loss_rows_vec_kernel<8, 3>);
+    else if (vec && C4 <= 32) rows_vec(loss_rows_vec_kernel<8, 4>);
+    else if (vec && C4 <= 48) rows_vec(loss_rows_vec_kernel<16, 3>);
+    else if (vec && C4 <= 64) rows_vec(loss_rows_vec_kernel<16, 4>);
+    else if (vec && C4 <= 96) rows_vec(loss_rows_vec_kernel<32, 3>);
+    else if (vec && C4 <= 128) rows_vec(loss_rows_vec_kernel<32, 4>);
     else
-        launch_chained(loss_rows_kernel, dim3(warp_blocks), LOSS_WARPS * 32, 0, s, n, C, logits, ld, labels, mask, count, dlogits, pred, n_correct, part, status, zero_rows);
-    return cudaGetLastError() == cudaSuccess ? (int)warp_blocks : -1;
+        launch_chained(loss_rows_kernel, dim3(blocks), LOSS_WARPS * 32, 0, s, n, C, logits, ld, labels, mask, count, dlogits, pred, n_correct, part, status, zero_rows);
+    return cudaGetLastError() == cudaSuccess;
 }
 
 // (one thread adding 2,368 partials took 17 us, and 65 us beside the traffic of a large call)
@@ -732,21 +537,21 @@ extern "C" mixgcn_status mixgcn_loss_softmax_xent(mixgcn_ctx* ctx, int64_t n, in
     unsigned long long* count = reinterpret_cast<unsigned long long*>(ctx->workspace);
     double* part = reinterpret_cast<double*>(reinterpret_cast<char*>(ctx->workspace) + 16);
     MIXGCN_TRY(count_train_nodes(ctx, n, train_mask, count, n_correct, s));
-    int n_part = (int)blocks;
+    bool launched = true;
     {
         LaunchScope scope(ctx, PH_LOSS, s);
         if (ctx->loss_train_rows_only == 1)
             launch_chained(loss_rows_subset_kernel, dim3((unsigned)blocks), LOSS_WARPS * 32, 0, s, n, C, logits, ld, labels, train_mask, count, dlogits, pred,
                                                                               reinterpret_cast<unsigned long long*>(n_correct), part, ctx->d_status);
         else
-            n_part = launch_loss_rows((unsigned)blocks, s, n, C, logits, ld, labels, train_mask, count, dlogits, pred,
-                                      reinterpret_cast<unsigned long long*>(n_correct), part, ctx->d_status,
-                                      ctx->loss_train_rows_only != 2, ctx->sm_count);
+            launched = launch_loss_rows((unsigned)blocks, s, n, C, logits, ld, labels, train_mask, count, dlogits, pred,
+                                        reinterpret_cast<unsigned long long*>(n_correct), part, ctx->d_status,
+                                        ctx->loss_train_rows_only != 2);
     }
-    if (n_part < 0) MIXGCN_FAIL(MIXGCN_ECUDA, "loss: kernel launch failed: %s", cudaGetErrorString(cudaGetLastError()));
+    if (!launched) MIXGCN_FAIL(MIXGCN_ECUDA, "loss: kernel launch failed: %s", cudaGetErrorString(cudaGetLastError()));
     {
         LaunchScope scope(ctx, PH_LOSS, s);
-        launch_chained(loss_final_kernel, dim3(1), LOSS_FINAL_THREADS, 0, s, n_part, part, count, loss, ctx->d_status);
+        launch_chained(loss_final_kernel, dim3(1), LOSS_FINAL_THREADS, 0, s, (int)blocks, part, count, loss, ctx->d_status);
     }
     MIXGCN_CUDA(cudaGetLastError());
     return MIXGCN_OK;
@@ -851,12 +656,10 @@ extern "C" mixgcn_status mixgcn_loss_softmax_xent_noalloc(int64_t n, int32_t C, 
     int64_t cb = (n + 255) / 256;
     if (cb > 4096) cb = 4096;
     launch_chained(count_mask_kernel, dim3((unsigned)cb), 256, 0, s, n, train_mask, &sc->count);
-    int sm_count = 0;
-    MIXGCN_CUDA(cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, device));
-    const int n_part = launch_loss_rows((unsigned)blocks, s, n, C, logits, ld, labels, train_mask, &sc->count, dlogits, pred,
-                                        reinterpret_cast<unsigned long long*>(n_correct), sc->part, &sc->status, true, sm_count);
-    if (n_part < 0) MIXGCN_FAIL(MIXGCN_ECUDA, "loss_noalloc: kernel launch failed: %s", cudaGetErrorString(cudaGetLastError()));
-    launch_chained(loss_final_kernel, dim3(1), LOSS_FINAL_THREADS, 0, s, n_part, sc->part, &sc->count, loss, &sc->status);
+    if (!launch_loss_rows((unsigned)blocks, s, n, C, logits, ld, labels, train_mask, &sc->count, dlogits, pred,
+                          reinterpret_cast<unsigned long long*>(n_correct), sc->part, &sc->status))
+        MIXGCN_FAIL(MIXGCN_ECUDA, "loss_noalloc: kernel launch failed: %s", cudaGetErrorString(cudaGetLastError()));
+    launch_chained(loss_final_kernel, dim3(1), LOSS_FINAL_THREADS, 0, s, (int)blocks, sc->part, &sc->count, loss, &sc->status);
     if (status) MIXGCN_CUDA(cudaMemcpyAsync(status, &sc->status, sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
     MIXGCN_CUDA(cudaGetLastError());
     return MIXGCN_OK;

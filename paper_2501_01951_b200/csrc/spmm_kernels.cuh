@@ -253,21 +253,19 @@ __device__ __forceinline__ void loss_epilogue(const Params& p, int64_t u, int li
         }
         return;
     }
-    float s = 0.0f;
+    float s = 0.0f, py = 0.0f;        // the label's logit lives in lane (y/4) % LPR of the group
 #pragma unroll
     for (int v = 0; v < VPL; ++v)
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-            if ((lig + v * LPR) * 4 + e < C) s += expf(x[v][e] - mx);
+        for (int e = 0; e < 4; ++e) {
+            const int c = (lig + v * LPR) * 4 + e;
+            if (c == y) py = x[v][e];
+            x[v][e] = c < C ? expf(x[v][e] - mx) : 0.0f;
+            s += x[v][e];
+        }
 #pragma unroll
     for (int o = LPR / 2; o > 0; o >>= 1) s += __shfl_xor_sync(mask, s, o, LPR);
-    const float lse = mx + logf(s);
-    float py = 0.0f;        // the label's logit lives in lane (y/4) % LPR of the group
-#pragma unroll
-    for (int v = 0; v < VPL; ++v)
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-            if ((lig + v * LPR) * 4 + e == y) py = x[v][e];
+    const float lse = mx + logf(s), share = 1.0f / s;
     py = __shfl_sync(mask, py, (y >> 2) & (LPR - 1), LPR);
     if (lig == 0) p.loss_row[u] = lse - py;
     const float invT = (float)(1.0 / (double)T);
@@ -279,7 +277,7 @@ __device__ __forceinline__ void loss_epilogue(const Params& p, int64_t u, int li
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const int c = c4 * 4 + e;
-                r[e] = c < C ? (expf(x[v][e] - lse) - (c == y ? 1.0f : 0.0f)) * invT : 0.0f;
+                r[e] = c < C ? (x[v][e] * share - (c == y ? 1.0f : 0.0f)) * invT : 0.0f;
             }
             *reinterpret_cast<float4*>(p.Z + u * p.ldz + c4 * 4) = make_float4(r[0], r[1], r[2], r[3]);
         }

@@ -52,3 +52,32 @@ def test_rows(mg, ctx, C, n, share, room, in_place):
     assert torch.equal(pred, best) and good.item() == int(((best == y) & rows).sum())
     if room:
         assert torch.isnan(full[:, -room:]).all() and (out[:, -room:] == 5.0).all()
+
+
+@pytest.mark.parametrize("C", [16, 17, 48, 49, 96, 97, 192, 193, 257, 300, 384, 385, 512, 513])
+@pytest.mark.parametrize("n,share", [(1, 1.0), (9, 0.5), (5003, 0.02), (40_003, 0.6)])
+def test_rows_at_the_lane_splits(mg, ctx, C, n, share):
+    test_rows(mg, ctx, C, n, share, 0, True)
+    test_rows(mg, ctx, C, n, share, 4, False)
+
+
+@pytest.mark.parametrize("C", [5, 47, 100, 172, 300])
+def test_rows_without_numbers(mg, ctx, C):
+    """NaN among numbers, nothing but NaN, infinities: the prediction ignores NaN, is the lowest column where there is nothing else; loss and
+    gradient of the other rows stay as they are."""
+    n, ld = 64, (C + 3) // 4 * 4
+    x = torch.randn((n, ld), device="cuda")
+    y, m = torch.zeros(n, dtype=torch.int32, device="cuda"), torch.ones(n, dtype=torch.uint8, device="cuda")
+    m[:8] = 0
+    outs = []
+    for odd in (False, True):
+        if odd:
+            x[0, :] = float("nan")
+            x[1, 0] = float("nan")
+            x[2, C - 1] = float("inf")
+            x[3, :] = float("-inf")
+        full, loss, pred = x.clone(), torch.zeros(1, device="cuda"), torch.full((n,), 7, dtype=torch.int32, device="cuda")
+        mg.loss_softmax_xent(ctx, full, y, m, loss, dlogits=full, pred=pred, C_=C)
+        outs.append((full[:, :C].clone(), loss.clone(), pred.clone()))
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1]) and torch.equal(outs[0][2][4:], outs[1][2][4:])
+    assert outs[1][2][:4].tolist() == [0, 1 + int(x[1, 1:C].argmax()), C - 1, 0]

@@ -7,12 +7,14 @@
 // waits twice (for the entry count, then for the schedule's counts), keys carry no more bits than the ids have
 // (a radix pass over the keys costs as much as any other kernel here), and what the flags already say about the
 // structure is not looked up.  The schedule looks the column blocks of a long row up once, keeps them for the segments, and orders those by
-// 4,096 ranges of first columns (250 K nodes, 4.7 M entries: seg_count_kernel 46 -> 28 us, seg_fill_kernel 47 -> 13, the order 45 -> 9).
+// 4,096 ranges of first columns (250 K nodes, 4.7 M entries: seg_count_kernel 46 -> 20 us, of which 7 were additions of single warps to one counter,
+// seg_fill_kernel 47 -> 12, the order 45 -> 9); rows are sorted by as many bits as the longest has (43 -> 34).
 // Builds of that list: 9.0 ms and more -> 0.68 -> 0.42 ms.
 #include <cub/cub.cuh>
 
 #include <atomic>
 #include <new>
+#include <type_traits>
 
 #include "graph_values.cuh"
 #include "internal.cuh"
@@ -162,7 +164,7 @@ struct ScheduleCounts {
     unsigned long long rows_above_seg, rows_above[3], rows_heavy, total_segs, max_deg, bounds;
 };
 
-// Row counts of the buckets (one atomic per warp and counter).
+// Row counts of the buckets (one atomic per block and counter).
 __global__ void schedule_counts_kernel(int64_t n, uint32_t top, const uint32_t* __restrict__ keys, int seg, ScheduleCounts* counts) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t d = i < n ? (int64_t)(top - keys[i]) : -1;
@@ -171,8 +173,8 @@ __global__ void schedule_counts_kernel(int64_t n, uint32_t top, const uint32_t* 
     unsigned long long* const to[5] = {&counts->rows_above_seg, &counts->rows_above[0], &counts->rows_above[1], &counts->rows_above[2], &counts->rows_heavy};
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
-        const unsigned b = __ballot_sync(0xFFFFFFFFu, d > thr[q]);
-        if ((threadIdx.x & 31) == 0 && b) atomicAdd(to[q], (unsigned long long)__popc(b));
+        const int rows = __syncthreads_count(d > thr[q]);
+        if (threadIdx.x == 0 && rows) atomicAdd(to[q], (unsigned long long)rows);
     }
 }
 
@@ -184,45 +186,78 @@ __device__ __forceinline__ int row_log_blocks(int64_t d, int64_t blk_min) {
     return k;
 }
 
-__device__ __forceinline__ int64_t lower_bound_col(const int32_t* __restrict__ col, int64_t lo, int64_t hi, int64_t key) {
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if ((int64_t)col[mid] < key) lo = mid + 1; else hi = mid;
+// The positions of N columns in a row of `len` entries (how many lie below each); the searches run side by side, a request each in flight.
+template <int N>
+__device__ __forceinline__ void lower_bounds(const int32_t* __restrict__ row, int32_t len, const int64_t (&key)[N], int32_t (&at)[N]) {
+#pragma unroll
+    for (int r = 0; r < N; ++r) at[r] = 0;
+    for (int32_t step = 1 << (31 - __clz(len)); step > 0; step >>= 1) {
+        int32_t c[N];
+#pragma unroll
+        for (int r = 0; r < N; ++r) c[r] = at[r] + step <= len ? __ldg(row + at[r] + step - 1) : 0x7FFFFFFF;
+#pragma unroll
+        for (int r = 0; r < N; ++r) if ((int64_t)c[r] < key[r]) at[r] += step;
     }
-    return lo;
 }
 
 // Long rows: the number of segments of the i-th longest row (0 for rows that are not cut; i <= cap, a bound of the number of long rows), a warp
 // per row, 32 column blocks at a time.  The first entry of every block is kept for seg_fill_kernel, the row's at bounds[bound_at[i]].
-__global__ void seg_count_kernel(int64_t n_cols, int64_t cap, const int32_t* __restrict__ perm, const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col, int seg,
+__global__ void __launch_bounds__(TPB) seg_count_kernel(int64_t n_cols, int64_t cap, const int32_t* __restrict__ perm, const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col, int seg,
                                  int64_t* __restrict__ row_segs, int32_t* __restrict__ bounds, int32_t* __restrict__ bound_at, ScheduleCounts* counts) {
-    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (i > cap) return;
-    int64_t segs = 0;
+    const int64_t i = ((int64_t)blockIdx.x * TPB + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __shared__ int room[TPB / 32], block_segs[TPB / 32];       // of the block's rows: one addition each to the counters
+    int32_t segs = 0;
     const int64_t rb = i < cap ? rowptr[perm[i]] : 0, re = i < cap ? rowptr[perm[i] + 1] : 0;
-    if (re - rb > seg) {
-        const int nb = 1 << row_log_blocks(re - rb, schedule_blk_min(n_cols));
+    const int nb = re - rb > seg ? 1 << row_log_blocks(re - rb, schedule_blk_min(n_cols)) : 0;
+    if (lane == 0) room[warp] = nb;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int all = 0;
+        for (int k = 0; k < TPB / 32; ++k) { const int mine = room[k]; room[k] = all; all += mine; }
+        const int first = all ? (int)atomicAdd(&counts->bounds, (unsigned long long)all) : 0;
+        for (int k = 0; k < TPB / 32; ++k) room[k] += first;
+    }
+    __syncthreads();
+    if (nb) {
         const int64_t width = (n_cols + nb - 1) / nb;
-        int at = 0;
-        if (lane == 0) bound_at[i] = at = (int)atomicAdd(&counts->bounds, (unsigned long long)nb);
-        at = __shfl_sync(0xFFFFFFFFu, at, 0);
-        int64_t before = re;                   // of the blocks so far: where the last one begins
-        for (int b0 = nb - 32 < 0 ? 0 : nb - 32;; b0 -= 32) {        // from the last ones on, so that every block knows where the next one begins
-            const int b = b0 + lane;
-            const int64_t lo = b < nb ? lower_bound_col(col, rb, re, b * width) : re;
-            if (b < nb) bounds[at + b] = (int32_t)(lo - rb);
-            const int64_t next = __shfl_down_sync(0xFFFFFFFFu, lo, 1), hi = lane == 31 ? before : next;
-            segs += (hi - lo + seg - 1) / seg;
-            before = __shfl_sync(0xFFFFFFFFu, lo, 0);
-            if (b0 == 0) break;
-        }
+        const int at = room[warp];
+        if (lane == 0) bound_at[i] = at;
+        const int32_t len = (int32_t)(re - rb);
+        auto blocks = [&](auto n_c) {          // n_c * 32 blocks at a time, from the last ones on, so that every block knows where the next one begins
+            constexpr int N = decltype(n_c)::value;
+            int32_t next_begin = len;
+            for (int b0 = nb > N * 32 ? nb - N * 32 : 0;; b0 -= N * 32) {
+                int64_t key[N];
+                int32_t lo[N];
+#pragma unroll
+                for (int r = 0; r < N; ++r) key[r] = (int64_t)(b0 + r * 32 + lane) * width;       // (past the last block: past the last column)
+                lower_bounds<N>(col + rb, len, key, lo);
+#pragma unroll
+                for (int r = N - 1; r >= 0; --r) {
+                    const int b = b0 + r * 32 + lane;
+                    if (b < nb) bounds[at + b] = lo[r];
+                    const int32_t next = __shfl_down_sync(0xFFFFFFFFu, lo[r], 1), hi = lane == 31 ? next_begin : next;
+                    segs += (hi - lo[r] + seg - 1) / seg;
+                    next_begin = __shfl_sync(0xFFFFFFFFu, lo[r], 0);
+                }
+                if (b0 == 0) break;
+            }
+        };
+        if (nb <= 32) blocks(std::integral_constant<int, 1>());
+        else blocks(std::integral_constant<int, 4>());
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) segs += __shfl_xor_sync(0xFFFFFFFFu, segs, o);
     }
     if (lane == 0) {
-        row_segs[i] = segs;
-        if (segs) atomicAdd(&counts->total_segs, (unsigned long long)segs);
+        if (i <= cap) row_segs[i] = segs;
+        block_segs[warp] = segs;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned long long all = 0;
+        for (int k = 0; k < TPB / 32; ++k) all += (unsigned long long)block_segs[k];
+        if (all) atomicAdd(&counts->total_segs, all);
     }
 }
 
@@ -323,13 +358,14 @@ void free_view(CsrView& v) {
 
 // Schedule of rows [row0, row0 + n) of the CSR (rowptr, col) of a matrix with n_total columns and nnz entries in all
 // rows (a row chunk is cut like the whole matrix, so that its sums are the same).
-mixgcn_status build_schedule(int64_t n_total, int64_t nnz, const int64_t* rowptr, const int32_t* col, int64_t row0, int64_t n,
+// max_deg: what no row exceeds (a pass of the sort less for every eight bits).
+mixgcn_status build_schedule(int64_t n_total, int64_t nnz, int64_t max_deg, const int64_t* rowptr, const int32_t* col, int64_t row0, int64_t n,
                              SpmmSchedule& v, cudaStream_t s) {
     v = SpmmSchedule{};
     v.row0 = row0; v.n_rows = n; v.seg = schedule_seg(nnz);
     if (n <= 0) return MIXGCN_OK;
     // rows by descending entry count; the bucket counts; the segments each long row will need
-    const int deg_bits = bits_for((uint64_t)n_total);                      // a row has at most n_total entries
+    const int deg_bits = bits_for((uint64_t)(max_deg > 0 ? max_deg : 1));
     const uint32_t top = (uint32_t)(((uint64_t)1 << deg_bits) - 1);
     int64_t cap = nnz / (v.seg + 1);                                       // no more rows than this are long
     if (cap > n) cap = n;
@@ -399,8 +435,8 @@ mixgcn_status fill_degrees(mixgcn_graph* g, cudaStream_t s) {
 }
 
 // Everything after the CSR exists: symmetry, transpose, schedules.  known_symmetric / known_diagonal:
-// what the caller already knows of the structure (-1: look).  Leaves work in flight on `s`.
-mixgcn_status finish_graph(mixgcn_graph* g, int known_symmetric, int known_diagonal, cudaStream_t s) {
+// what the caller already knows of the structure (-1: look); max_deg: what no row exceeds.  Leaves work in flight on `s`.
+mixgcn_status finish_graph(mixgcn_graph* g, int known_symmetric, int known_diagonal, int64_t max_deg, cudaStream_t s) {
     const int64_t n = g->n, nnz = g->nnz;
     CsrView& A = g->fwd;
     g->symmetric = known_symmetric; g->has_diagonal = known_diagonal;
@@ -417,7 +453,7 @@ mixgcn_status finish_graph(mixgcn_graph* g, int known_symmetric, int known_diago
         if (known_symmetric < 0) g->symmetric = (h.flags & F_NOT_SYMMETRIC) ? 0 : 1;
         if (known_diagonal < 0) g->has_diagonal = h.diagonal == (unsigned long long)n ? 1 : (h.diagonal == 0 ? 0 : 2);
     }
-    MIXGCN_TRY(build_schedule(n, nnz, A.rowptr, A.col, 0, n, A.full, s));
+    MIXGCN_TRY(build_schedule(n, nnz, max_deg, A.rowptr, A.col, 0, n, A.full, s));
     g->bwd_is_fwd = (g->symmetric && g->norm != 1) ? 1 : 0;   // row-mean values are not symmetric: A_hat^T needs its own copy
     if (g->bwd_is_fwd) {
         g->bwd = A;  // alias: the same index serves the backward aggregation
@@ -442,7 +478,7 @@ mixgcn_status finish_graph(mixgcn_graph* g, int known_symmetric, int known_diago
     MIXGCN_CUDA(cub::DeviceRadixSort::SortPairs(tmp.p, tb, k0.as<uint64_t>(), k1.as<uint64_t>(), A.val, T.val,
                                                 nnz, shift, 2 * shift, s));
     rowptr_from_keys_kernel<uint64_t><<<blocks_for(nnz + 1), TPB, 0, s>>>(n, nnz, shift, k1.as<uint64_t>(), T.rowptr, T.col);
-    return build_schedule(n, nnz, T.rowptr, T.col, 0, n, T.full, s);
+    return build_schedule(n, nnz, n, T.rowptr, T.col, 0, n, T.full, s);
 }
 
 // Edge list (on the device) -> CSR of the graph: keys, sort, unique, values.
@@ -492,7 +528,7 @@ mixgcn_status check_common(mixgcn_ctx* ctx, int64_t n, mixgcn_graph** out) {
 namespace mixgcn {
 
 mixgcn_status build_view_schedule(int64_t n_cols, int64_t n, int64_t nnz, CsrView& v, cudaStream_t s) {
-    return build_schedule(n_cols, nnz, v.rowptr, v.col, 0, n, v.full, s);
+    return build_schedule(n_cols, nnz, n_cols, v.rowptr, v.col, 0, n, v.full, s);
 }
 
 void release_view(CsrView& v) { free_view(v); }
@@ -511,7 +547,7 @@ mixgcn_status ensure_chunk_schedules(const mixgcn_graph* g, const CsrView& A_con
     cudaStream_t s = g->ctx->side_stream[0];
     for (int k = 0; k < chunks; ++k) {
         const int64_t r0 = (g->n * (int64_t)k) / chunks, r1 = (g->n * (int64_t)(k + 1)) / chunks;
-        mixgcn_status st = build_schedule(g->n, g->nnz, A.rowptr, A.col, r0, r1 - r0, sc[k], s);
+        mixgcn_status st = build_schedule(g->n, g->nnz, A.full.max_deg, A.rowptr, A.col, r0, r1 - r0, sc[k], s);
         if (st == MIXGCN_OK && cudaStreamSynchronize(s) != cudaSuccess) st = MIXGCN_ECUDA;    // usable on every stream from here on
         if (st != MIXGCN_OK) {
             cudaStreamSynchronize(s);         // kernels that write to them
@@ -569,14 +605,15 @@ extern "C" mixgcn_status mixgcn_graph_create(mixgcn_ctx* ctx, int64_t n, int64_t
         ps = dsrc.as<int32_t>(); pd = ddst.as<int32_t>();
     }
     bool built = false;
-    MIXGCN_TRY(csr_from_buckets(g, m, ps, pd, sym, self, s, &built));
+    int64_t max_deg = n;               // a row has at most n entries
+    MIXGCN_TRY(csr_from_buckets(g, m, ps, pd, sym, self, s, &built, &max_deg));
     // two ids fit one 32-bit key on graphs of fewer than 2^16 nodes: half the bytes per radix pass
     if (built) {}
     else if (2 * bits_for((uint64_t)n) <= 32) MIXGCN_TRY(csr_from_edges<uint32_t>(g, m, ps, pd, sym, self, s));
     else MIXGCN_TRY(csr_from_edges<uint64_t>(g, m, ps, pd, sym, self, s));
     dsrc.release(); ddst.release();
     // self loops of the input are dropped, so the flags decide what lies on the diagonal; a directed list may still be symmetric
-    MIXGCN_TRY(finish_graph(g, sym ? 1 : -1, self ? 1 : 0, s));
+    MIXGCN_TRY(finish_graph(g, sym ? 1 : -1, self ? 1 : 0, max_deg, s));
     MIXGCN_CUDA(cudaStreamSynchronize(s));
     guard.keep = true;
     *out = g;
@@ -622,7 +659,7 @@ extern "C" mixgcn_status mixgcn_graph_create_from_csr(mixgcn_ctx* ctx, int64_t n
     if (hf & F_UNSORTED) MIXGCN_FAIL(MIXGCN_EBADGRAPH, "graph_create_from_csr: columns are not strictly ascending in a row");
     MIXGCN_TRY(fill_degrees(g, s));
     values_kernel<<<blocks_for(n * 32), TPB, 0, s>>>(n, g->fwd.rowptr, g->fwd.col, g->dinv, g->norm, g->fwd.val);
-    MIXGCN_TRY(finish_graph(g, -1, -1, s));
+    MIXGCN_TRY(finish_graph(g, -1, -1, n, s));
     MIXGCN_CUDA(cudaStreamSynchronize(s));
     guard.keep = true;
     *out = g;

@@ -42,6 +42,7 @@ enum { F_BAD_ID = 1, F_FULL = 2 };
 
 struct Counted {
     int32_t flags;
+    int32_t max_deg;                                    // without duplicates
     int32_t skip;                                       // a bucket is too large: the kernels behind the first do nothing
     uint32_t done;
     uint32_t got[BUCKETS_MAX], first[BUCKETS_MAX];      // entries of a bucket as they come, and those of the buckets before
@@ -444,6 +445,10 @@ __global__ void __launch_bounds__(TPB, 2) sort_kernel(Split sp, const uint32_t* 
         const uint32_t u = sp.node(b, i);
         if (u < sp.n) { deg[u] = (int32_t)sm.count[i]; dinv[u] = degree_norm((int32_t)sm.count[i]); }
     }
+    int32_t longest = 0;
+    for (int i = tid; i < rows; i += TPB) longest = max(longest, (int32_t)sm.count[i]);
+    longest = __reduce_max_sync(0xFFFFFFFFu, longest);
+    if (lane == 0) atomicMax(&c->max_deg, longest);
     if (tid == 0) c->kept[b] = all;
 }
 
@@ -474,7 +479,7 @@ __global__ void __launch_bounds__(TPB) fill_kernel(Split sp, int norm, const uin
 
 namespace mixgcn {
 
-mixgcn_status csr_from_buckets(mixgcn_graph* g, int64_t m, const int32_t* src, const int32_t* dst, int sym, int self, cudaStream_t s, bool* built) {
+mixgcn_status csr_from_buckets(mixgcn_graph* g, int64_t m, const int32_t* src, const int32_t* dst, int sym, int self, cudaStream_t s, bool* built, int64_t* max_deg) {
     *built = false;
     Split sp{};
     sp.n = g->n;
@@ -516,12 +521,14 @@ mixgcn_status csr_from_buckets(mixgcn_graph* g, int64_t m, const int32_t* src, c
     MIXGCN_CUDA(cub::DeviceScan::ExclusiveSum(tmp.p, tb, g->deg, g->fwd.rowptr, n + 1, s));
     MIXGCN_CUDA(cudaGetLastError());
     int64_t nnz = 0;
-    int32_t flags = 0;
+    struct { int32_t flags, max_deg; } seen{};
+    static_assert(offsetof(Counted, max_deg) == offsetof(Counted, flags) + sizeof(int32_t), "read together");
     MIXGCN_CUDA(cudaMemcpyAsync(&nnz, g->fwd.rowptr + n, sizeof(nnz), cudaMemcpyDeviceToHost, s));
-    MIXGCN_CUDA(cudaMemcpyAsync(&flags, &d->flags, sizeof(flags), cudaMemcpyDeviceToHost, s));
+    MIXGCN_CUDA(cudaMemcpyAsync(&seen, &d->flags, sizeof(seen), cudaMemcpyDeviceToHost, s));
     MIXGCN_CUDA(cudaStreamSynchronize(s));
-    if (flags & F_BAD_ID) MIXGCN_FAIL(MIXGCN_EBADGRAPH, "graph_create: a node id lies outside [0, %lld)", (long long)n);
-    if (flags & F_FULL) return MIXGCN_OK;
+    if (seen.flags & F_BAD_ID) MIXGCN_FAIL(MIXGCN_EBADGRAPH, "graph_create: a node id lies outside [0, %lld)", (long long)n);
+    if (seen.flags & F_FULL) return MIXGCN_OK;
+    *max_deg = seen.max_deg;
     g->nnz = nnz;
     const int64_t room = nnz > 0 ? nnz : 1;
     MIXGCN_TRY(dev_alloc((void**)&g->fwd.col, room * (int64_t)sizeof(int32_t), s));

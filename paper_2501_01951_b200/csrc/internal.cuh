@@ -260,8 +260,8 @@ inline mixgcn_status ensure_workspace(mixgcn_ctx* ctx, int64_t bytes) { return g
 inline mixgcn_status ensure_workspace_spmm(mixgcn_ctx* ctx, int64_t bytes) { return grow_block(ctx, &ctx->workspace_spmm, &ctx->workspace_spmm_bytes, bytes, "aggregation workspace"); }
 inline mixgcn_status ensure_workspace_lp(mixgcn_ctx* ctx, int64_t bytes) { return grow_block(ctx, &ctx->workspace_lp, &ctx->workspace_lp_bytes, bytes, "bf16 operand workspace"); }
 inline mixgcn_status ensure_workspace_rows(mixgcn_ctx* ctx, int64_t bytes) { return grow_block(ctx, &ctx->workspace_rows, &ctx->workspace_rows_bytes, bytes, "row-sparse workspace"); }
-// CSR, values and degrees of an edge list (on the device); *built stays false where it is left to the radix sort.
-mixgcn_status csr_from_buckets(mixgcn_graph* g, int64_t m, const int32_t* src, const int32_t* dst, int sym, int self, cudaStream_t s, bool* built);
+// CSR, values and degrees of an edge list (on the device), and its longest row; *built stays false where it is left to the radix sort.
+mixgcn_status csr_from_buckets(mixgcn_graph* g, int64_t m, const int32_t* src, const int32_t* dst, int sym, int self, cudaStream_t s, bool* built, int64_t* max_deg);
 // Builds (once) the schedules of the `chunks` row chunks of this orientation.  Synchronises on first use.
 mixgcn_status ensure_chunk_schedules(const mixgcn_graph* g, const CsrView& A, int chunks);
 

@@ -552,8 +552,8 @@ mixgcn_status mixgcn_loss_softmax_xent(mixgcn_ctx* ctx, int64_t n, int32_t C, co
  * process exits.
  *  - Runs on the calling thread's CURRENT device; all pointers are device pointers of it.
  *  - Arguments and results as mixgcn_loss_softmax_xent; `status` (device int32, nullable)
- *    receives 0, 1 (empty train mask), 2 (label outside [0,C)) or 3 (a bounded wait inside the
- *    kernel gave up; loss, dlogits and pred are then undefined) when the stream reaches it.
+ *    receives 0, 1 (empty train mask) or 2 (label outside [0,C)) when the stream reaches it (3, a
+ *    bounded wait that gave up, is reserved: no kernel of this call waits).
  *  - Limit: n <= 33,554,432 rows (32768 partials x 1024 rows) and 1 <= C <= 4096; larger sizes
  *    return MIXGCN_EUNSUPPORTED and launch nothing.
  *  - The first call on each device looks up the scratch array's device address (one

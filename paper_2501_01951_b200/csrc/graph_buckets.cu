@@ -4,7 +4,7 @@
 // row pointers and values 365), because every pass goes by eight bits.  Here an entry goes to the bucket of its row at once, as (row in the
 // bucket, column) in 32 bits, in no particular order; a block then sorts a bucket, drops duplicates and counts its rows, and once the host
 // knows how many entries there are the buckets are read once more into columns and values.  Two passes over the edges, two over
-// the entries: 14 + 34 + 69 + 9 + 45 us of the same list.  The result is a sorted set, so it does not depend on the order in which entries arrived.
+// the entries: 14 + 34 + 60 + 9 + 45 us of the same list.  The result is a sorted set, so it does not depend on the order in which entries arrived.
 //
 // Rows are spread over the buckets by a multiplicative hash (a bijection of the ids), so that neighbouring hubs do not meet.  In a bucket a
 // row of n entries has a power of two between n / 4 and n / 2 of bins, by the highest bits of the columns; entries are counted into bins
@@ -15,8 +15,8 @@
 // so that every SM has several blocks; there are at most 2,048, whose counters a block keeps in shared memory while it scatters.  That
 // is where the line to the radix sort lies.  Lists with a bucket of more than 64 K entries go there as well (a hub of as many neighbours: a
 // block would pass over them alone, a star of a million 3.0 ms against 0.77).  Whole builds, radix sort : buckets (us): 2 K nodes, 21 K entries 255 :
-// 233;  5 K, 1.5 M 369 : 307;  50 K, 5.2 M 519 : 419;  250 K, 4.7 M 682 : 435;  300 K, 9.4 M 985 : 580;  1 M, 4.3 M 654 : 482;  1 M, 9.3 M 1057 : 695;  ends drawn by
-// rank^-0.7, neighbouring ids, 200 K, 6 M 795 : 524;  by rank^-1, largest row 63 K, 2.7 M 689 : 650.
+// 234;  5 K, 1.5 M 369 : 302;  50 K, 5.2 M 519 : 414;  250 K, 4.7 M 682 : 400;  300 K, 9.4 M 985 : 544;  1 M, 4.3 M 654 : 482;  1 M, 9.3 M 1057 : 633;  ends drawn by
+// rank^-0.7, neighbouring ids, 200 K, 6 M 795 : 494;  by rank^-1, largest row 63 K, 2.7 M 689 : 668;  a star of a million, after the look at it, 764 : 796.
 // (Instead of bins, for 4.7 M entries: three passes of nine bits over a bucket 147 us, rows sorted one by one in registers and shared memory
 // 155; entries scattered as they come instead of in runs 48.)
 #include <cub/block/block_scan.cuh>
@@ -47,6 +47,7 @@ struct Counted {
     uint32_t done;
     uint32_t got[BUCKETS_MAX], first[BUCKETS_MAX];      // entries of a bucket as they come, and those of the buckets before
     uint32_t at[BUCKETS_MAX];                           // scattered so far
+    uint16_t order[BUCKETS_MAX];                        // the large buckets first: a block that gets one late is the end of the launch
     uint32_t kept[BUCKETS_MAX];                         // without duplicates
 };
 
@@ -116,6 +117,16 @@ __global__ void __launch_bounds__(TPB) count_kernel(Split sp, int64_t m, const i
 #pragma unroll
     for (int k = 0; k < BUCKETS_MAX / TPB; ++k) large |= x[k] > BUCKET_MAX;
     if (large) { c->skip = 1; atomicOr(&c->flags, F_FULL); }
+    uint32_t before[BUCKETS_MAX / TPB], larges[BUCKETS_MAX / TPB], all;
+#pragma unroll
+    for (int k = 0; k < BUCKETS_MAX / TPB; ++k) larges[k] = x[k] > AVERAGE * 5 / 4;
+    Scan(temp).ExclusiveSum(larges, before, all);
+#pragma unroll
+    for (int k = 0; k < BUCKETS_MAX / TPB; ++k) {
+        const uint32_t b = tid * (BUCKETS_MAX / TPB) + k;
+        c->order[larges[k] ? before[k] : all + b - before[k]] = (uint16_t)b;
+    }
+    __syncthreads();
     Scan(temp).ExclusiveSum(x, x);
 #pragma unroll
     for (int k = 0; k < BUCKETS_MAX / TPB; ++k) c->first[tid * (BUCKETS_MAX / TPB) + k] = x[k];
@@ -291,7 +302,7 @@ __global__ void __launch_bounds__(TPB, 2) sort_kernel(Split sp, const uint32_t* 
     SortMemory& sm = *reinterpret_cast<SortMemory*>(smem_raw);
     using Scan = cub::BlockScan<uint32_t, TPB>;
     constexpr int PER = ROWS_MAX / TPB;
-    const int b = blockIdx.x, rows = 1 << sp.log, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rows = 1 << sp.log, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t cols = (1u << sp.shift) - 1;
     for (int i = tid; i < ROWS_MAX; i += TPB) sm.count[i] = 0;
     for (int i = tid; i < BINS_MAX; i += TPB) sm.bins[i] = 0;
@@ -299,6 +310,7 @@ __global__ void __launch_bounds__(TPB, 2) sort_kernel(Split sp, const uint32_t* 
     __syncthreads();
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (__ldcg(&c->skip)) return;
+    const int b = __ldcg(&c->order[blockIdx.x]);
     const uint32_t got = __ldcg(&c->got[b]), first = __ldcg(&c->first[b]);
     const uint32_t* mine = keys + first;
     uint32_t* out = sorted + first;

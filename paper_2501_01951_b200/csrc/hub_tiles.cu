@@ -10,10 +10,12 @@
 //    in four signed digits of base 256, once per call, into images of the shared-memory tiles (column_range_kernel, cut_rows_kernel).
 //    Whole-number products (tcgen05 kind::i8) take half the time of bf16 ones and their 32-bit sums are exact, so a row's tiles are one
 //    chain: nothing is added up on the way, and the sum is rounded to fp32 once.  What is lost is half a unit a term.
-//  * Columns whose numbers lie far apart (the largest more than SPREAD_MAX binades above the geometric mean) take six digits, 2^-47; infinities, NaN and
-//    numbers further apart than that send the call's tiles to the FMA pipes.  The device decides, by whole numbers: no order of blocks changes it.
-//  * A stage of the product is a tile's bitmap, expanded to bytes by four warps, and one contiguous copy of the image a CTA.  64 columns of Y (32
-//    with six digits) have 256 (192) columns of TMEM, twice: one half adds up while the epilogue empties the other.
+//  * Where a column's numbers lie far apart (the largest more than SPREAD_MAX binades above the geometric mean, as in the gradients of a model that
+//    has learnt its labels) what is left of every number goes through once or twice more, in units of 2^-31 of the ones before; infinities, NaN
+//    and numbers further apart than three passes reach (71 binades) send the call's tiles to the FMA pipes.  The device decides, by whole
+//    numbers: no order of blocks changes it.
+//  * A stage of the product is a tile's bitmap, expanded to bytes by four warps, and one contiguous copy of the image a CTA.  64 columns of Y
+//    have 256 columns of TMEM, twice: one half adds up while the epilogue empties the other.
 //  * What is not in a tile is a matrix of its own, with a schedule of its own, for the gather kernels.  They run behind the tiles, and where
 //    they have a row's sum add the row's pieces to it (one, or two where a pair's share ends in the row), times row_scale.
 //
@@ -56,32 +58,30 @@ constexpr int COLUMN_COST = 1200;               // entries whose gathers take as
 constexpr int PIECE_COST = 3;                   // tiles that take as long as a piece does beside its tiles
 constexpr int LEAST_TILES = 8;                  // of a pair of CTAs
 constexpr uint32_t TMEM_COLS = 512;
-constexpr int GROUP = 16;                       // columns of Y whose digits lie together
-// Exponents between the largest number of a column and the mean of its others up to which four digits (31 bits below the largest) do, and
-// by how many more six reach.
-constexpr int SPREAD_MAX = 9, SPREAD_MORE = 16;
+constexpr int GROUP = 16, DIGITS = 4;           // columns of Y whose digits lie together, digits of a number in a pass
+// Exponents between the largest number of a column and the mean of its others up to which one pass does (31 bits below the largest), by how
+// many more every other pass reaches, and how many passes there are at most.
+constexpr int SPREAD_MAX = 9, SPREAD_MORE = 31, PASSES_MAX = 3;
 
-enum { MODE_4 = 0, MODE_6 = 1, MODE_PLAIN = 2 };     // digits of a number; plain_pieces instead
 // What column_range_kernel leaves for the kernels behind it, and its own sums, which are zero between calls.
 struct Ranges {
     int32_t shift[HUB_SLICE];                   // numbers are cut as multiples of 2^-shift (read by fours)
     uint32_t top[HUB_SLICE];                    // largest number of a column, as bits
     int32_t sum[HUB_SLICE], count[HUB_SLICE];   // exponents of its numbers but zeros, and how many
-    int32_t mode;
+    int32_t passes;                             // 0: plain_pieces instead
     uint32_t done;                              // blocks that have added theirs
 };
 static_assert(TILES_WORD * 4 % 16 == 0 && TILES_WORD + (int)(sizeof(Ranges) / 4) <= STATUS_WORDS, "room beside the status words");
 
-// How w columns of Y are taken: in blocks, all digits of a block's columns side by side in an accumulator.
+// How w columns of Y are taken: in blocks, all digits of a block's columns side by side in an accumulator; passes one behind the other.
 struct Shape {
-    int digits, cols, blocks;                   // columns of a block (a multiple of GROUP), blocks
-    __host__ __device__ int n() const { return digits * cols; }                            // columns of the accumulator, at most 256
+    int cols, blocks;                           // columns of a block (a multiple of GROUP), blocks
+    __host__ __device__ int n() const { return DIGITS * cols; }                            // columns of the accumulator, at most 256
     __host__ __device__ int image_bytes() const { return n() / 2 * COLS; }                 // a CTA's half of a tile's image
 };
-Shape make_shape(int digits, int w) {
-    const int most = (int)TMEM_COLS / 2 / digits / GROUP * GROUP;
+Shape make_shape(int w) {
+    const int most = (int)TMEM_COLS / 2 / DIGITS / GROUP * GROUP;
     Shape s;
-    s.digits = digits;
     s.blocks = (w + most - 1) / most;
     s.cols = ((w + s.blocks - 1) / s.blocks + GROUP - 1) / GROUP * GROUP;
     return s;
@@ -92,7 +92,7 @@ struct TileParams {
     const int32_t* tile_cb; const uint4* bits;
     float* partial; int64_t ldp;                        // row r of piece q goes to partial row q * ROWS + r
     int w4, kblocks;
-    Shape shape[2];                                     // by mode
+    Shape shape;
     const Ranges* ranges;
     const float* Y; int64_t ldy, y_rows;
     const int32_t* nodes; const float* col_scale; int64_t n_cols;
@@ -135,7 +135,7 @@ __device__ __forceinline__ bool elect_one() {
 __host__ __device__ constexpr int bit_of(int c) { return 8 * (c & 3) + ((c >> 2) & 7); }
 __host__ __device__ constexpr int column_of(int bit) { return 4 * (bit & 7) + (bit >> 3); }
 
-// A pair's pieces on the FMA pipes, for calls in which a row of Y holds an infinity, a NaN, or numbers too far apart for six digits: the
+// A pair's pieces on the FMA pipes, for calls in which a row of Y holds an infinity, a NaN, or numbers too far apart: the
 // expansion warps, one per row of a piece, entries in the order of their bits.
 __device__ __forceinline__ void plain_pieces(const TileParams& p, int q0, int q1, int rank) {
     const int lane = threadIdx.x & 31;
@@ -168,9 +168,9 @@ __device__ __forceinline__ void plain_pieces(const TileParams& p, int q0, int q1
     }
 }
 
-// The sums of 8 columns, digits 16 columns of the accumulator apart, from two's complement digits of base 256: exact, then rounded once.
-template <int DIGITS>
-__device__ __forceinline__ void join_digits(uint32_t taddr, const int32_t* __restrict__ shift, float (&out)[8]) {
+// The sums of 8 columns, digits 16 columns of the accumulator apart, from two's complement digits of base 256: exact, then rounded once.  finer:
+// by how many binades this pass' unit is smaller than the first one's.
+__device__ __forceinline__ void join_digits(uint32_t taddr, const int32_t* __restrict__ shift, int finer, float (&out)[8]) {
     uint32_t r[DIGITS][8];
 #pragma unroll
     for (int d = 0; d < DIGITS; ++d) tc_ld8(taddr + d * GROUP, r[d]);
@@ -179,23 +179,21 @@ __device__ __forceinline__ void join_digits(uint32_t taddr, const int32_t* __res
     const int32_t s[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-        int64_t x = (int64_t)(int32_t)r[0][i] + (int64_t)(int32_t)r[1][i] * (1 << 8) + (int64_t)(int32_t)r[2][i] * (1 << 16);
-        if (DIGITS == 4) x += (int64_t)(int32_t)r[DIGITS == 4 ? 3 : 0][i] * (1 << 24);
-        else x += ((int64_t)(int32_t)r[DIGITS > 4 ? 3 : 0][i] + (int64_t)(int32_t)r[DIGITS > 4 ? 4 : 0][i] * (1 << 8) + (int64_t)(int32_t)r[DIGITS > 4 ? 5 : 0][i] * (1 << 16)) << 24;
-        const int half = -s[i] >> 1, rest = -s[i] - half;           // (2^-shift itself may lie outside fp32)
+        const int64_t x = (int64_t)(int32_t)r[0][i] + (int64_t)(int32_t)r[1][i] * (1 << 8) + (int64_t)(int32_t)r[2][i] * (1 << 16) + (int64_t)(int32_t)r[3][i] * (1 << 24);
+        const int down = -s[i] - finer, half = down >> 1, rest = down - half;           // (2^down itself may lie outside fp32)
         out[i] = __ll2float_rn(x) * __int_as_float((half + 127) << 23) * __int_as_float((rest + 127) << 23);
     }
 }
 
-// The accumulator of one piece and block, 16 columns at a time, through a box per warp, so that a request stores whole sectors.
-template <int DIGITS>
-__device__ __forceinline__ void store_sums(const TileParams& p, uint32_t lanes, int groups, int half, int col0, float* dst, uint8_t* box) {
+// The accumulator of one piece and block, 16 columns at a time, through a box per warp, so that a request stores whole sectors; behind the
+// first pass added to what the same threads have stored.
+__device__ __forceinline__ void store_sums(const TileParams& p, uint32_t lanes, int groups, int half, int col0, int pass, float* dst, uint8_t* box) {
     const int lane = threadIdx.x & 31;
     for (int g = half; g < groups; g += 2) {
 #pragma unroll
         for (int sub = 0; sub < 2; ++sub) {
             float x[8];
-            join_digits<DIGITS>(lanes + g * GROUP * DIGITS + sub * 8, p.ranges->shift + col0 + g * GROUP + sub * 8, x);
+            join_digits(lanes + g * GROUP * DIGITS + sub * 8, p.ranges->shift + col0 + g * GROUP + sub * 8, pass * SPREAD_MORE, x);
 #pragma unroll
             for (int c = 0; c < 2; ++c)
                 *reinterpret_cast<float4*>(box + lane * 64 + (((sub * 2 + c) ^ ((lane >> 1) & 3)) << 4)) = make_float4(x[c * 4], x[c * 4 + 1], x[c * 4 + 2], x[c * 4 + 3]);
@@ -206,7 +204,10 @@ __device__ __forceinline__ void store_sums(const TileParams& p, uint32_t lanes, 
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int row = i * 8 + (lane >> 2);
-                reinterpret_cast<float4*>(dst)[row * (p.ldp >> 2) + c4] = *reinterpret_cast<const float4*>(box + row * 64 + (((lane & 3) ^ ((row >> 1) & 3)) << 4));
+                float4 x = *reinterpret_cast<const float4*>(box + row * 64 + (((lane & 3) ^ ((row >> 1) & 3)) << 4));
+                float4* to = reinterpret_cast<float4*>(dst) + row * (p.ldp >> 2) + c4;
+                if (pass) { const float4 o = *to; x.x += o.x; x.y += o.y; x.z += o.z; x.w += o.w; }
+                *to = x;
             }
         }
         __syncwarp();
@@ -214,13 +215,12 @@ __device__ __forceinline__ void store_sums(const TileParams& p, uint32_t lanes, 
 }
 
 // A pair of CTAs (cluster of two, tcgen05 .cta_group::2) takes 256 rows, 128 each; each holds half of B.  The pair's
-// tiles once for every block of the columns of Y.
+// tiles once for every block of the columns of Y and pass.
 // The barriers full and acc_empty that count are the leader's, whose MMA warp waits on them; the others exist in both.
 // Warps 0-7 epilogue (two per TMEM lane quarter, alternate groups of columns), 8-11 expansion (a thread per row of the tile),
 // 12 images, 13 bitmaps, 14 MMA issue.  The expansion has its bitmaps from shared memory: its fences and its arrivals in the leader's memory would
 // wait for loads from global memory that its threads have under way (1,230 cycles a tile).
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1) spmm_tiles_kernel(const __grid_constant__ CUtensorMap images4, const __grid_constant__ CUtensorMap images6,
-                                                                                           const TileParams p) {
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1) spmm_tiles_kernel(const __grid_constant__ CUtensorMap images, const TileParams p) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) Shared b;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -247,9 +247,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1) spmm_til
     tc_fence_after();
     const uint32_t tmem = b.tmem;
     asm volatile("griddepcontrol.wait;" ::: "memory");       // the images are complete
-    const int mode = __ldcg(&p.ranges->mode);
-    const Shape sh = p.shape[mode == MODE_6 ? 1 : 0];
-    const int blocks = mode == MODE_PLAIN ? 0 : sh.blocks, n = sh.n();
+    const Shape sh = p.shape;
+    const int passes = __ldcg(&p.ranges->passes), blocks = passes * sh.blocks, n = sh.n();       // (the blocks of all passes)
     const uint32_t image_bytes = (uint32_t)sh.image_bytes();
 
     if (warp < EPI_WARPS) {
@@ -263,14 +262,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1) spmm_til
                 tc_fence_after();
                 const uint32_t lanes = tmem + ((uint32_t)(quarter * 32) << 16) + set * (uint32_t)n;
                 float* dst = p.partial + ((int64_t)q * ROWS + rank * 128 + quarter * 32) * p.ldp;
-                if (mode == MODE_4) store_sums<4>(p, lanes, sh.cols / GROUP, half, blk * sh.cols, dst, boxes + warp * BOX_BYTES);
-                else store_sums<6>(p, lanes, sh.cols / GROUP, half, blk * sh.cols, dst, boxes + warp * BOX_BYTES);
+                store_sums(p, lanes, sh.cols / GROUP, half, blk % sh.blocks * sh.cols, blk / sh.blocks, dst, boxes + warp * BOX_BYTES);
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive_pair(mapa_shared(smem_u32(&b.acc_empty[set]), 0));
             }
     } else if (warp < TMA_WARP) {
-        if (mode == MODE_PLAIN) plain_pieces(p, q0, q1, (int)rank);
+        if (passes == 0) plain_pieces(p, q0, q1, (int)rank);
         const int row = threadIdx.x - EXP_WARP * 32;
         Ring slot;
         for (int t = blocks * (t1 - t0); t > 0; --t, slot.next(SLOTS)) {
@@ -297,7 +295,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1) spmm_til
                     if (!thread_wait(&b.empty[slot.i], slot.use ^ 1, b, p)) { ok = false; break; }
                     if (rank == 0) mbar_expect_tx(&b.full[slot.i], 2 * image_bytes);
                     if (!(p.drop_load && blk == 0 && t == t0))
-                        tma_load_2d_pair(smem + slot.i * SLOT_BYTES + A_BYTES, mode == MODE_4 ? &images4 : &images6, 0, row, mapa_shared(smem_u32(&b.full[slot.i]), 0));
+                        tma_load_2d_pair(smem + slot.i * SLOT_BYTES + A_BYTES, &images, 0, row, mapa_shared(smem_u32(&b.full[slot.i]), 0));
                 }
         }
     } else if (warp == BITS_WARP) {
@@ -350,7 +348,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1) spmm_til
 }
 
 // The range of every column of Y over the hub columns of the matrix, scaled as they are multiplied: what unit its numbers are cut in, and how
-// many digits the call takes.  All whole numbers, so that neither depends on the order of the blocks.  2^lanes lanes a row.
+// many passes the call takes.  All whole numbers, so that neither depends on the order of the blocks.  2^lanes lanes a row.
 constexpr int RANGE_THREADS = 512;
 __global__ void __launch_bounds__(RANGE_THREADS) column_range_kernel(int64_t n_cols, int w, int lanes, const int32_t* __restrict__ nodes, const float* __restrict__ scale,
                                                            const float* __restrict__ Y, int64_t ldy, int64_t y_rows, Ranges* ranges, int32_t* status) {
@@ -404,40 +402,45 @@ __global__ void __launch_bounds__(RANGE_THREADS) column_range_kernel(int64_t n_c
     const uint32_t most = mine ? __ldcg(&ranges->top[tid]) : 0;
     const int32_t all = mine ? __ldcg(&ranges->sum[tid]) : 0, many = mine ? __ldcg(&ranges->count[tid]) : 0;
     const int spread = many ? (int)(most >> 23) - all / many : 0;
-    const int mode = __syncthreads_or(most >= 0x7F800000u || spread > SPREAD_MAX + SPREAD_MORE) ? MODE_PLAIN : __syncthreads_or(spread > SPREAD_MAX) ? MODE_6 : MODE_4;
-    if (tid == 0) ranges->mode = mode;
+    int passes = 1;
+    for (int k = 0; k < PASSES_MAX; ++k) passes += __syncthreads_or(spread > SPREAD_MAX + k * SPREAD_MORE) ? 1 : 0;
+    if (__syncthreads_or(most >= 0x7F800000u) || passes > PASSES_MAX) passes = 0;
+    if (tid == 0) ranges->passes = passes;
     if (!mine) return;
     ranges->top[tid] = 0; ranges->sum[tid] = ranges->count[tid] = 0;
-    // the largest number stays below 2^31 - 2^24 units (2^47 - 2^40 of six digits): its highest digit takes a carry from those below
-    const int exponent = max((int)(most >> 23), 1) - 127 + ((most & 0x7FFFFFu) >= 0x7E0000u);
-    ranges->shift[tid] = (mode == MODE_6 ? 46 : 30) - exponent;
+    // the largest number stays below 2^31 - 2^24 units: its highest digit takes a carry from those below
+    ranges->shift[tid] = 30 - (max((int)(most >> 23), 1) - 127 + ((most & 0x7FFFFFu) >= 0x7E0000u));
 }
 
-// 16 rows of a column -> its 16 bytes of every digit.  The product by the scale is exact (fp64), and adding 1.5 * 2^52 leaves the whole
-// number that is nearest to it in the lowest bits; what is below half a unit is all that is lost.
-template <int DIGITS>
-__device__ __forceinline__ void cut_column(const float (&y)[16], const double* __restrict__ by, double unit, uint4 (&out)[DIGITS]) {
-    constexpr uint64_t CARRIES = DIGITS == 4 ? 0x808080ull : 0x8080808080ull;       // digits from -128 to 127
+// 16 rows of a column in units -> its 16 bytes of every digit; behind the first pass of what is left, in units of 2^-31 (worked out anew: kept,
+// it would take half as many registers again).  Adding 1.5 * 2^52 leaves the whole number that is nearest in the lowest bits.
+__device__ __forceinline__ void cut_column(const float (&y)[16], const double* __restrict__ by, double unit, int pass, uint4 (&out)[DIGITS]) {
+    constexpr uint32_t CARRIES = 0x808080u;                  // digits from -128 to 127
+    constexpr double WHOLE = 6755399441055744.0;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        uint64_t t[4];
+        uint32_t t[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-            t[i] = ((uint64_t)__double_as_longlong(fma((double)y[q * 4 + i] * by[q * 4 + i], unit, 6755399441055744.0)) + CARRIES) ^ CARRIES;
+        for (int i = 0; i < 4; ++i) {
+            double x = (double)y[q * 4 + i] * by[q * 4 + i] * unit;
+#pragma unroll 1
+            for (int k = 0; k < pass; ++k) x = (x - ((x + WHOLE) - WHOLE)) * 0x1p31;
+            t[i] = ((uint32_t)__double2loint(x + WHOLE) + CARRIES) ^ CARRIES;
+        }
 #pragma unroll
         for (int d = 0; d < DIGITS; ++d) {
-            const uint32_t pick = (uint32_t)(d & 3) | (uint32_t)(4 + (d & 3)) << 4;
-            const uint32_t r = __byte_perm(__byte_perm((uint32_t)(t[0] >> (d & 4 ? 32 : 0)), (uint32_t)(t[1] >> (d & 4 ? 32 : 0)), pick),
-                                           __byte_perm((uint32_t)(t[2] >> (d & 4 ? 32 : 0)), (uint32_t)(t[3] >> (d & 4 ? 32 : 0)), pick), 0x5410);
+            const uint32_t pick = (uint32_t)d | (uint32_t)(4 + d) << 4;
+            const uint32_t r = __byte_perm(__byte_perm(t[0], t[1], pick), __byte_perm(t[2], t[3], pick), 0x5410);
             (q == 0 ? out[d].x : q == 1 ? out[d].y : q == 2 ? out[d].z : out[d].w) = r;
         }
     }
 }
 
-// Rows of Y of the hub columns -> images of their digits: images[block][column block of the matrix][half of an accumulator's columns], the
+// Rows of Y of the hub columns -> images of their digits: images[pass][block][column block of the matrix][half of an accumulator's columns], the
 // 128 numbers of a digit of a column consecutive, as the tensor core wants them in shared memory.  A block of threads takes 128 rows and 16
-// columns (the blocks of the same rows run side by side), a thread 16 rows of a column.
-__global__ void __launch_bounds__(128) cut_rows_kernel(int64_t n_cols, int kblocks, Shape shape4, Shape shape6, int w, const int32_t* __restrict__ nodes, const float* __restrict__ scale,
+// columns (the blocks of the same rows run side by side), a thread 16 rows of a column.  The scaling is exact (fp64); what is below half a unit
+// of the last pass is all that is lost.  Eight blocks an SM: waiting for rows is most of its time (96 registers and five: + 30 us of a 2,050 us call).
+__global__ void __launch_bounds__(128, 8) cut_rows_kernel(int64_t n_cols, int kblocks, Shape sh, int w, const int32_t* __restrict__ nodes, const float* __restrict__ scale,
                                                        const float* __restrict__ Y, int64_t ldy, int64_t y_rows, uint8_t* __restrict__ images, const Ranges* ranges, int32_t* status) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     __shared__ __align__(16) int32_t node[COLS];
@@ -461,29 +464,23 @@ __global__ void __launch_bounds__(128) cut_rows_kernel(int64_t n_cols, int kbloc
         for (int i = 0; i < 4; ++i) y[q * 4 + i] = v[i] >= 0 && col < w ? __ldg(Y + (int64_t)v[i] * ldy + col) : 0.0f;
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");       // the ranges are complete (Y was before them)
-    const int mode = __ldcg(&ranges->mode);
+    const int passes = __ldcg(&ranges->passes);
     const double unit = col < w ? __hiloint2double((__ldcg(&ranges->shift[col < w ? col : 0]) + 1023) << 20, 0) : 0.0;
-    const Shape sh = mode == MODE_6 ? shape6 : shape4;
     const int groups = sh.cols / GROUP, blk = (int)blockIdx.x / groups, g = (int)blockIdx.x % groups;
-    if (mode == MODE_PLAIN || blk >= sh.blocks) return;
+    if (passes == 0) return;
     const int64_t image = (int64_t)sh.image_bytes();
-    uint8_t* base = images + ((int64_t)blk * kblocks + kb) * 2 * image;
-    auto store = [&](int d, const uint4& x) {
-        int row = (g * sh.digits + d) * GROUP + c;
-        const int rank = row >= sh.n() / 2;
-        row -= rank * (sh.n() / 2);
-        *reinterpret_cast<uint4*>(base + rank * image + row * 128 + ((j ^ (row & 7)) << 4)) = x;
-    };
-    if (mode == MODE_4) {
-        uint4 out[4];
-        cut_column<4>(y, by + j * 16, unit, out);
+#pragma unroll 1
+    for (int pass = 0; pass < passes; ++pass) {
+        uint4 out[DIGITS];
+        cut_column(y, by + j * 16, unit, pass, out);
+        uint8_t* base = images + ((int64_t)(pass * sh.blocks + blk) * kblocks + kb) * 2 * image;
 #pragma unroll
-        for (int d = 0; d < 4; ++d) store(d, out[d]);
-    } else {
-        uint4 out[6];
-        cut_column<6>(y, by + j * 16, unit, out);
-#pragma unroll
-        for (int d = 0; d < 6; ++d) store(d, out[d]);
+        for (int d = 0; d < DIGITS; ++d) {
+            int row = (g * DIGITS + d) * GROUP + c;
+            const int rank = row >= sh.n() / 2;
+            row -= rank * (sh.n() / 2);
+            *reinterpret_cast<uint4*>(base + rank * image + row * 128 + ((j ^ (row & 7)) << 4)) = out[d];
+        }
     }
 }
 
@@ -809,7 +806,7 @@ bool hub_tiles_pay(const HubTiles* t, int32_t w) {
     auto slice = [&](int32_t c) {
         const double entry = c > 192 ? 0.040 : c > 128 ? 0.0365 : c > 96 ? 0.0285 : c > 64 ? 0.0235 : 0.0028 + 0.0002 * (c > 8 ? c : 8);
         const double other = c > 192 ? 0.0086 : c > 128 ? 0.0035 : c > 96 ? 0.0061 : c > 64 ? 0.0016 : c > 48 ? 0.0024 : 0.0008;
-        const Shape sh = make_shape(4, c);
+        const Shape sh = make_shape(c);
         const double product = sh.blocks * (0.30 * tiles * (sh.cols > 40 ? sh.cols : 40) / 64 + 3.0);
         all += entry * 1e-3 * (t->entries + t->rem_nnz);
         gain += entry * 1e-3 * t->entries - other * 1e-3 * t->rem_nnz - product - 12.0 - 3.2e-6 * t->n_cols * c;
@@ -822,8 +819,8 @@ int64_t hub_tiles_scratch(const HubTiles* t, int32_t w, int64_t ldp, int64_t* im
     const int64_t partial = (int64_t)t->n_pieces * ROWS * ldp * (int64_t)sizeof(float);
     *images_at = (partial + 1023) & ~(int64_t)1023;
     if (w > HUB_SLICE) w = HUB_SLICE;
-    const Shape s4 = make_shape(4, w), s6 = make_shape(6, w);
-    return *images_at + (int64_t)t->kblocks * 2 * std::max(s4.blocks * s4.image_bytes(), s6.blocks * s6.image_bytes());
+    const Shape sh = make_shape(w);
+    return *images_at + (int64_t)t->kblocks * 2 * PASSES_MAX * sh.blocks * sh.image_bytes();
 }
 
 mixgcn_status launch_hub_tiles(mixgcn_ctx* ctx, const HubTiles* t, int phase, int32_t w, const float* Y, int64_t ldy, int64_t y_rows, float* partial, int64_t ldp,
@@ -832,32 +829,28 @@ mixgcn_status launch_hub_tiles(mixgcn_ctx* ctx, const HubTiles* t, int phase, in
     p.pieces = t->pieces; p.first_piece = t->first_piece; p.tile_cb = t->tile_cb; p.bits = reinterpret_cast<const uint4*>(t->bits);
     p.partial = partial; p.ldp = ldp;
     p.w4 = (w + 3) >> 2; p.kblocks = t->kblocks;
-    p.shape[0] = make_shape(4, w); p.shape[1] = make_shape(6, w);
+    p.shape = make_shape(w);
     Ranges* ranges = reinterpret_cast<Ranges*>(ctx->d_status + TILES_WORD);
     p.ranges = ranges;
     p.Y = Y; p.ldy = ldy; p.y_rows = y_rows; p.nodes = t->nodes; p.col_scale = t->col_scale; p.n_cols = t->n_cols;
     p.status = ctx->d_status;
     p.wait_limit = ctx->debug_wait_limit > 0 ? (uint32_t)ctx->debug_wait_limit : WAIT_LIMIT_DEFAULT;
     p.drop_load = ctx->debug_drop_load;
-    CUtensorMap map[2];
-    for (int m = 0; m < 2; ++m) {
-        const Shape& sh = p.shape[m];
-        if (!encode_2d(&map[m], images, 2, 64, (int64_t)sh.blocks * t->kblocks * sh.n(), 64, 64, sh.n() / 2, CU_TENSOR_MAP_SWIZZLE_NONE))
-            MIXGCN_FAIL(MIXGCN_ECUDA, "spmm: no tensor map for the images of the hub rows");
-    }
+    CUtensorMap map;
+    if (!encode_2d(&map, images, 2, 64, (int64_t)PASSES_MAX * p.shape.blocks * t->kblocks * p.shape.n(), 64, 64, p.shape.n() / 2, CU_TENSOR_MAP_SWIZZLE_NONE))
+        MIXGCN_FAIL(MIXGCN_ECUDA, "spmm: no tensor map for the images of the hub rows");
     {
         LaunchScope scope(ctx, phase, s, 2);
         int lanes = 0;
         while ((4 << lanes) < w) ++lanes;
         const int64_t rows = RANGE_THREADS >> lanes, most = 2 * (int64_t)ctx->sm_count, blocks = (t->n_cols + rows * 4 - 1) / (rows * 4);
         column_range_kernel<<<(unsigned)(blocks < most ? blocks : most), RANGE_THREADS, 0, s>>>(t->n_cols, w, lanes, t->nodes, t->col_scale, Y, ldy, y_rows, ranges, ctx->d_status);
-        const int groups = std::max(p.shape[0].blocks * p.shape[0].cols, p.shape[1].blocks * p.shape[1].cols) / GROUP;
-        launch_chained(cut_rows_kernel, dim3((unsigned)groups, (unsigned)t->kblocks), 128, 0, s, t->n_cols, t->kblocks, p.shape[0], p.shape[1], w, t->nodes, t->col_scale, Y, ldy, y_rows,
-                       images, ranges, ctx->d_status);
+        launch_chained(cut_rows_kernel, dim3((unsigned)(p.shape.blocks * p.shape.cols / GROUP), (unsigned)t->kblocks), 128, 0, s, t->n_cols, t->kblocks, p.shape, w, t->nodes, t->col_scale, Y, ldy,
+                       y_rows, images, ranges, ctx->d_status);
     }
     MIXGCN_CUDA(cudaFuncSetAttribute(spmm_tiles_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TILES_SMEM));
     LaunchScope scope(ctx, phase, s);
-    launch_chained(spmm_tiles_kernel, dim3((unsigned)t->clusters * 2), THREADS, TILES_SMEM, s, map[0], map[1], p);      // it sets up beside the kernel before
+    launch_chained(spmm_tiles_kernel, dim3((unsigned)t->clusters * 2), THREADS, TILES_SMEM, s, map, p);      // it sets up beside the kernel before
     MIXGCN_CUDA(cudaGetLastError());
     return MIXGCN_OK;
 }

@@ -150,10 +150,11 @@ def test_numbers_of_every_size(mg, ctx, graphs):
 
 
 @pytest.mark.parametrize("w", [1, 16, 33, 65, 100, 256, 300])
-@pytest.mark.parametrize("binades", [6, 12, 20, 40])
+@pytest.mark.parametrize("binades", [6, 12, 20, 38, 44, 68, 80])
 def test_numbers_far_apart(mg, ctx, graphs, w, binades):
-    """One row in fifty `binades` above the others: four digits, six, and none that would do.  A term loses half a unit at most, 2^-31 and
-    2^-47 of the largest with four and six digits: 2^-25 and 2^-27 of the others' size where they are used, far inside the bound of the sums."""
+    """One row in fifty `binades` above the others: one, two and three passes of four digits, and more than they reach.  A term loses half a unit
+    of the last pass at most, 2^-31, 2^-62 or 2^-93 of the largest, used up to 9, 40 and 71 binades: 2^-22 of the others' size, inside the bound
+    of the sums."""
     plain, tiled, A = graphs["none", False]
     Y = features(w, 13)
     Y *= torch.where(torch.rand((N, 1), generator=torch.Generator().manual_seed(w)) < 0.02, 2.0 ** binades, 1.0).cuda()
